@@ -8,7 +8,7 @@
 // chunks of 256 columns.  Warp roles:
 //   warp 0      TMA producer: K-major, 128-byte-swizzled tiles of hidden (128 x 64) and W_vocab (256 x 64) into
 //               a ring of shared-memory stages, completion on mbarriers
-//   warp 1      tcgen05.mma issuer (one elected lane): 128 x 256 x 16 bf16 MMAs into one of two 256-column fp32
+//   warp 1      tcgen05.mma issuer (the warp waits, one elected lane issues): 128 x 256 x 16 bf16 MMAs into one of two 256-column fp32
 //               accumulators in tensor memory; tcgen05.commit releases stages / publishes accumulators
 //   warps 2..5  epilogue: thread r owns token row r of the tile; tcgen05.ld of its accumulator row, running
 //               maximum and sum of 2^(z log2e - max), and the target column's logit, all in registers
@@ -274,8 +274,14 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0 && rank == 0) {
+        // The whole warp walks the loops and waits, one elected lane issues: with control flow that is uniform over the
+        // warp the descriptors and the loop state stay in uniform registers.  Under a single-thread branch around the loop
+        // every MMA's operands went through per-thread registers first, and issuing a K step's four MMAs took the thread
+        // about the 512 cycles that they run.  200,000 tokens, d = 2048, V = 61,125 (pairs): 35.6 -> 34.8 ms; 100,000,
+        // d = 4096, V = 151,936 (single blocks): 91.7 -> 90.6 ms.
+        if (rank == 0) {
             constexpr uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, BN);
+            const uint32_t a0 = smem_u32(stage_a), b0 = smem_u32(stage_b);
             uint32_t stage = 0, phase = 0;
             uint32_t acc = 0, acc_phase = 0;
             bool ok = true;
@@ -284,43 +290,48 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                 const int c0 = split * p.chunks_per_split;
                 const int c1 = min(c0 + p.chunks_per_split, total_chunks);
                 for (int c = c0; c < c1 && ok; ++c) {
-                    if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
+                    if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
                     tcgen05_fence_after();
                     const uint32_t d_tmem = tmem_base + acc * BN;
                     for (int ks = 0; ks < k_steps; ++ks) {
-                        if (!mbar_wait(&full[stage], phase, abort_flag, p.spin_limit)) { ok = false; break; }
+                        if (!mbar_wait_warp(&full[stage], phase, abort_flag, p.spin_limit)) { ok = false; break; }
                         tcgen05_fence_after();
-                        const uint64_t a_desc = make_smem_desc(smem_u32(stage_a + (size_t)stage * A_STAGE_BYTES));
-                        const uint64_t b_desc = make_smem_desc(smem_u32(stage_b + (size_t)stage * B_STAGE_BYTES));
+                        const uint64_t a_desc = make_smem_desc(a0 + stage * A_STAGE_BYTES);
+                        const uint64_t b_desc = make_smem_desc(b0 + stage * B_STAGE_BYTES);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < BK / UMMA_K; ++k) {
-                            // advancing K by 16 elements = 32 bytes inside the swizzle row: +2 in address units
-                            if constexpr (PAIR)
-                                tcgen05_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                                      (ks | k) != 0 ? 1u : 0u);
-                            else
-                                tcgen05_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                                 (ks | k) != 0 ? 1u : 0u);
+                            for (int k = 0; k < BK / UMMA_K; ++k) {
+                                // advancing K by 16 elements = 32 bytes inside the swizzle row: +2 in address units
+                                if constexpr (PAIR)
+                                    tcgen05_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
+                                                          (ks | k) != 0 ? 1u : 0u);
+                                else
+                                    tcgen05_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
+                                                     (ks | k) != 0 ? 1u : 0u);
+                            }
+                            // stage reusable (in both blocks of a pair) once these MMAs have read it; after the last K
+                            // step the accumulator is complete
+                            if constexpr (PAIR) tcgen05_commit_pair(&empty[stage], (uint16_t)3);
+                            else tcgen05_commit(&empty[stage]);
+                            if (ks + 1 == k_steps) {
+                                if constexpr (PAIR) tcgen05_commit_pair(&acc_full[acc], (uint16_t)3);
+                                else tcgen05_commit(&acc_full[acc]);
+                            }
                         }
-                        // stage reusable (in both blocks of a pair) once these MMAs have read it
-                        if constexpr (PAIR) tcgen05_commit_pair(&empty[stage], (uint16_t)3);
-                        else tcgen05_commit(&empty[stage]);
+                        __syncwarp();
                         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                    }
-                    if (ok) {                                 // accumulator complete
-                        if constexpr (PAIR) tcgen05_commit_pair(&acc_full[acc], (uint16_t)3);
-                        else tcgen05_commit(&acc_full[acc]);
                     }
                     if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
                 }
             }
-            if (!ok) {
+            if (!ok && elect_one()) {
                 // Gave up: wait (bounded) until the MMAs already issued have finished with shared and tensor memory.
                 if constexpr (PAIR) tcgen05_commit_pair(drain, (uint16_t)1);
                 else tcgen05_commit(drain);
                 for (uint32_t it = 0; it < p.spin_limit; ++it)
                     if (mbar_try_wait(drain, 0u)) break;
             }
+            __syncwarp();
         }
     } else {
         // ---------------- epilogue: one token row per thread ----------------
