@@ -375,7 +375,8 @@ def measure(w, C, K, W, local, barrier, rank, full, args):
         cyc = (st[:, 3] - st[:, 2]).astype(np.float64) * blocks_per_item
         span_ns = float(st[:, 1].max() - st[:, 0].min())
         mhz = float(cyc.sum() / ns.sum() * 1e3) / blocks_per_item
-        flops_last = 2.0 * T_last * w.d * w.V
+        # whole work items only are stamped: a (pair of) 128-row tile(s) times V / splits columns each
+        flops_last = 2.0 * len(st) * 128 * blocks_per_item * w.d * (w.V / splits)
         in_kernel = {
             "sm_mhz": mhz, "what": "sum of SM cycles / sum of nanoseconds over the work items of the region's last "
                                    "log-prob launch (clock64 and globaltimer read by the kernel; no clock control touched)",

@@ -151,11 +151,12 @@ int arrol_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* lengths, c
  * logp[t] = 0 and records ARROL_DEV_BAD_TARGET.  Rows t >= T of the outputs are not written.
  * logp float [T_max]; lse float [T_max] or NULL.  Both pointers 16-byte aligned; d % 8 == 0; inv_temperature > 0.
  * workspace: device scratch of at least arrol_token_logprob_workspace(ctx, T_max, d, V) bytes, 256-byte
- * aligned (holds per-split running maxima / sums when the vocabulary is split across thread blocks); its
+ * aligned (holds running maxima / sums over parts of the vocabulary, per token); its
  * contents need not be initialised and are undefined afterwards.  The size is monotone in T_max: a workspace sized
  * for T_max also serves calls on fewer tokens with the same d and V. */
 size_t arrol_token_logprob_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V);
-/* Number of vocabulary splits a launch on T_max tokens uses (1 = every block walks the whole vocabulary). */
+/* Number of vocabulary groups that the whole work items of a launch cover (1 = a block walks the whole vocabulary).
+ * Token tiles that would not fill a whole wave of blocks are cut finer; the results do not depend on it. */
 int32_t arrol_token_logprob_splits(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V);
 /* Form of the kernel for these sizes: 2 = pairs of thread blocks on 256-row token tiles (tcgen05 cta_group::2), 1 = one
  * block per 128-row tile.  Pairs are used wherever they need no more vocabulary splits than single blocks (hidden
@@ -176,7 +177,7 @@ int arrol_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_vocab,
  *   arrol_compact (S is clamped to S_max, T to T_max);  src_tok_off [N] int64: the array given to arrol_compact;
  *   targets [T_max] int32 in packed order (arrol_compact's dst_tokens);  logp, lse, d, V, inv_temperature as in
  *   arrol_token_logprob.  workspace: arrol_token_logprob_gathered_workspace(ctx, S_max, T_max, d, V) bytes, 256-byte
- *   aligned: the split records of arrol_token_logprob plus S_max * 128 * d * 2 bytes, into which a first small
+ *   aligned: the records of arrol_token_logprob plus S_max * 128 * d * 2 bytes, into which a first small
  *   kernel copies the token tiles that cross a survivor boundary (at most one per survivor); every other tile is
  *   read in place.
  * Results equal arrol_token_logprob on the packed rows bit for bit.  Source rows are trusted to lie inside
@@ -458,7 +459,7 @@ int64_t arrol_launch_count(arrol_ctx* ctx);
  *                                    run out after the limit above; outputs of such a call are not written.
  *   ARROL_HOOK_LOGPROB_TIMING_BUFFER value = device address of a buffer of 4 x uint64 per work item (0 = off), and
  *   ARROL_HOOK_LOGPROB_TIMING_ITEMS  value = its capacity in work items: while set, every work item (token tile x
- *                                    vocabulary split) i < capacity of an arrol_token_logprob launch records
+ *                                    vocabulary group, tiles in whole waves only) i < capacity of a launch records
  *                                    {globaltimer at start, globaltimer at end, SM clock at start, SM clock at end}
  *                                    of its epilogue, from which a benchmark derives the SM clock the kernel ran at
  *                                    (cycles / nanoseconds) without reading or setting any GPU clock control.

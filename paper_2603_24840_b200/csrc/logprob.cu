@@ -2,17 +2,25 @@
 // (Section 3: log pi_theta(o_t | o_<t); Algorithm 1 "log-probs on R'"), as a fused contraction
 // hidden[T,d] x W_vocab[V,d]^T with an online max / log-sum-exp epilogue.  The T x V logits never leave the SM.
 //
-// One thread block per SM, persistent over work items (token tile, vocabulary split).  By default the blocks work as
-// PAIRS (clusters of two, tcgen05 cta_group::2) on 256-row token tiles, see PAIR below; described first is the
-// one-block form on 128-row tiles, which the pair form extends.  Per item the block walks its vocabulary range in
-// chunks of 256 columns.  Warp roles:
+// One thread block per SM, persistent over work items.  By default the blocks work as PAIRS (clusters of two, tcgen05
+// cta_group::2) on 256-row tiles, see PAIR below; described first is the one-block form on 128-row tiles, which the
+// pair form extends.  A work item is a token tile and a range of the vocabulary, which the block walks in chunks of 256
+// columns.  Warp roles:
 //   warp 0      TMA producer: K-major, 128-byte-swizzled tiles of hidden (128 x 64) and W_vocab (256 x 64) into
 //               a ring of shared-memory stages, completion on mbarriers
-//   warp 1      tcgen05.mma issuer (the warp waits, one elected lane issues): 128 x 256 x 16 bf16 MMAs into one of two 256-column fp32
-//               accumulators in tensor memory; tcgen05.commit releases stages / publishes accumulators
-//   warps 2..5  epilogue: thread r owns token row r of the tile; tcgen05.ld of its accumulator row, running
-//               maximum and sum of 2^(z log2e - max), and the target column's logit, all in registers
+//   warp 1      tcgen05.mma issuer (the warp waits, one elected lane issues): 128 x 256 x 16 bf16 MMAs into one of two
+//               256-column fp32 accumulators in tensor memory; tcgen05.commit releases stages / publishes accumulators
+//   epilogue warps  a thread owns one token row of the tile; tcgen05.ld of its accumulator row, running maximum and sum
+//               of 2^(z log2e - max), and the target column's logit, all in registers
 // The two accumulators let the epilogue of chunk c overlap the MMAs of chunk c + 1.
+//
+// Body and tail.  Whole waves of (tile, vocabulary group) items are the body.  What is left over would keep only some of
+// the blocks busy for one more wave.  These tiles are the tail: (vocabulary segment, tile) items, as many segments as
+// SMs, dealt round robin, so that every unit gets the same number of segments give or take one (see WorkList).  A token's
+// records are merged in one order whoever computed them (see VocabPlan), so neither the token count nor the assignment of
+// work shows in the bits.  Measured as pairs at d = 2560, V = 151,936 against whole items only (with more vocabulary splits
+// while there were fewer tiles than SMs): 128 tokens 451 -> 181 us, 1,777 1,241 -> 1,051 us, 5,000 4.12 -> 2.83 ms, 9,000
+// 5.24 -> 5.08 ms, 20,000 13.6 -> 11.0 ms.
 //
 // Waves in step.  The resident blocks all stream the same W_vocab chunks; as long as they do so at about the same
 // time a chunk comes from HBM once and from L2 147 times.  Nothing in a persistent kernel keeps them together,
@@ -60,38 +68,98 @@ constexpr int PAIR_B_STAGE_BYTES = PAIR_B_ROWS * BK * 2;   // 16 KB
 constexpr int PAIR_STAGE_BYTES = A_STAGE_BYTES + PAIR_B_STAGE_BYTES;
 static_assert(PAIR_STAGES * PAIR_STAGE_BYTES == SOLO_STAGES * SOLO_STAGE_BYTES, "both variants fill the same shared memory");
 constexpr int TMEM_COLS = 512;   // two fp32 accumulators of BN columns
-constexpr int NUM_THREADS = 192;
-constexpr int EPI_THREADS = 128;
+constexpr int EPI_WARPS = 4;                 // EPI_WARPS / 4 warps per tensor-memory lane quarter share a chunk's columns
+constexpr int HALVES = EPI_WARPS / 4;
+constexpr int EPI_COLS = BN / HALVES;
+constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
+constexpr int COMBINE_BLOCKS = 16;           // blocks of segments (n_mid) that one warp merges side by side
 constexpr size_t SMEM_BYTES = (size_t)SOLO_STAGES * SOLO_STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
 
-struct PartialLse {   // per (split, token): running maximum and sum in the base-2 domain, target logit,
-    float m2, l, zy2, pad;   // pad: sum of the raw accumulators of the split (only when the confidence is asked for)
+struct PartialLse {   // of one token over some columns: running maximum and sum in the base-2 domain, target logit,
+    float m2, l, zy2, sumz;   // sum of the raw accumulators (only when the confidence is asked for)
 };
+
+// How the vocabulary is cut: total_chunks chunks of BN columns -> n_sub segments -> n_mid blocks of segments -> splits
+// groups.  A body item covers a whole group, a tail item one segment; a token's records are merged segment by segment
+// into a block, block by block into a group, then group by group, by whichever kernel holds them.
+struct VocabPlan {
+    int total_chunks, n_sub, n_mid, splits;
+    __host__ __device__ int chunk_of_sub(int i) const { return (int)((int64_t)i * total_chunks / n_sub); }
+    __host__ __device__ int sub_of_mid(int i) const { return i * n_sub / n_mid; }
+    __host__ __device__ int mid_of_group(int g) const { return g * n_mid / splits; }
+    __host__ __device__ int sub_of_group(int g) const { return sub_of_mid(mid_of_group(g)); }
+};
+
+// (M, L) <- (M, L) + (m, l): M = max, L = sum of 2^(. - M).  One rounding per operation, so that the main kernel (body)
+// and the combining kernel (tail) get the same bits.
+__device__ __forceinline__ void merge_lse(float& M, float& L, float m, float l) {
+    if (m == -INFINITY) return;                                 // no column in the record
+    const float Mn = fmaxf(M, m);
+    L = __fadd_rn(__fmul_rn(L, ex2_approx(M - Mn)), __fmul_rn(l, ex2_approx(m - Mn)));
+    M = Mn;
+}
+__device__ __forceinline__ void merge_record(PartialLse& a, const PartialLse& b) {
+    merge_lse(a.m2, a.l, b.m2, b.l);
+    a.zy2 = fmaxf(a.zy2, b.zy2);        // exactly one record holds the target column, the others hold -inf
+    a.sumz = __fadd_rn(a.sumz, b.sumz);
+}
+__device__ __forceinline__ PartialLse empty_record() { return PartialLse{-INFINITY, 0.f, -INFINITY, 0.f}; }
+
+// Work of one launch on `tiles` token tiles (128 rows, or 256 for a pair of blocks).
+struct WorkList {
+    int64_t body_tiles, body_items, tail_items, waves;   // waves: those of the body, plus one for the tail
+    int tail_tiles;                                      // at most units / splits + 1
+};
+__host__ __device__ inline WorkList make_work_list(int64_t tiles, int64_t units, const VocabPlan& v) {
+    WorkList w;
+    w.body_tiles = tiles * v.splits / units * units / v.splits;    // whole waves only
+    w.body_items = w.body_tiles * v.splits;
+    w.tail_tiles = (int)(tiles - w.body_tiles);
+    w.tail_items = (int64_t)w.tail_tiles * v.n_sub;
+    w.waves = (w.body_items + units - 1) / units + (w.tail_items > 0 ? 1 : 0);
+    return w;
+}
+struct WorkItem {
+    int64_t tile, wave;
+    int group, sub0, sub1;      // group < 0: a tail item
+};
+// k-th item of a unit; false when it has none left.  The tail walks the segments as the slow index: at any time the
+// units work on neighbouring segments of all tail tiles and share W_vocab through L2.
+__device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v, int64_t unit, int64_t units, int64_t k,
+                                          WorkItem& it) {
+    int64_t i = unit + k * units;               // body items, then tail items, in one numbering
+    it.wave = k < w.waves ? k : w.waves - 1;
+    if (i < w.body_items) {
+        it.tile = i / v.splits;
+        it.group = (int)(i - it.tile * v.splits);
+        it.sub0 = v.sub_of_group(it.group);
+        it.sub1 = v.sub_of_group(it.group + 1);
+        return true;
+    }
+    i -= w.body_items;
+    if (i >= w.tail_items) return false;
+    it.sub0 = (int)(i / w.tail_tiles);
+    it.sub1 = it.sub0 + 1;
+    it.tile = w.body_tiles + (i - (int64_t)it.sub0 * w.tail_tiles);
+    it.group = -1;
+    return true;
+}
 
 struct LogprobParams {
     const int32_t* targets;
     const int64_t* d_T;
     int64_t T_max;
     int d, V;
-    int splits;            // vocabulary splits per token tile
-    int chunks_per_split;  // chunks of BN columns per split
+    VocabPlan plan;
     float scale2;          // inv_temperature * log2(e)
-    float* logp;
-    float* lse;
-    float* conf;           // token confidence H_t = -sum_v log P_t(v) = V lse - sum_v z_v, or NULL
-    float inv_temp;
-    PartialLse* partial;   // [splits][T_max] when splits > 1
+    PartialLse* body;      // [splits][HALVES][T_max]: records of the tokens in whole waves
+    PartialLse* tail;      // [token of the tail][n_sub][HALVES]
     uint32_t spin_limit;   // tries per pipeline wait
     int mute_producer;     // test hook: the producer issues no copies
     uint32_t* d_status;
-    // gathered variant: packed token t of survivor s is source row src_tok_off[survivor_idx[s]] + (t - cu_seqlens[s])
-    const int64_t* cu_seqlens;
-    const int32_t* survivor_idx;
-    const int64_t* src_tok_off;
-    const int64_t* d_num;  // {S, T}
-    int S_max;
-    unsigned int* wave_counter;   // producers that have arrived, over all waves of this launch (zeroed before it)
-    unsigned long long* timing;   // test hook: per work item {globaltimer start, end, clock64 start, end}, or NULL
+    const int32_t* tile_row;      // gathered variant: source row of every token tile, or ~(scratch row) of a pre-packed one
+    unsigned int* wave_counter;   // producers that have arrived, over all waves of this launch (zeroed before a launch of several)
+    unsigned long long* timing;   // test hook: per body item {globaltimer start, end, clock64 start, end}, or NULL
     int64_t timing_items;
 };
 
@@ -105,6 +173,47 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
+}
+
+// Columns of chunk c that the MMA computes: BN, or what is left of the vocabulary rounded up to 32 (the granularity of
+// N for a pair of blocks, each of which brings half of the rows of W_vocab).
+__device__ __forceinline__ int chunk_columns(int V, int c) {
+    const int left = V - c * BN;
+    return left >= BN ? BN : (left + 31) & ~31;
+}
+
+// 32 columns pc0 ... of one token row into its running record.
+template <bool CONF>
+__device__ __forceinline__ void accumulate_piece(float (&v)[32], int pc0, int y, int V, float scale2, PartialLse& r) {
+    if constexpr (CONF) {                   // sum of the valid logits of the piece (before masking)
+        float ps[4] = {0.f, 0.f, 0.f, 0.f};           // four chains; only the last piece needs the mask
+        if (pc0 + 32 <= V) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) ps[j & 3] += v[j];
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) ps[j & 3] += (pc0 + j < V) ? v[j] : 0.f;
+        }
+        r.sumz += (ps[0] + ps[1]) + (ps[2] + ps[3]);
+    }
+    if (pc0 + 32 > V) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) if (pc0 + j >= V) v[j] = -INFINITY;
+    }
+    if ((unsigned)(y - pc0) < 32u) {
+        const int jy = y - pc0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) if (j == jy) r.zy2 = v[j] * scale2;
+    }
+    float bmax = v[0];
+#pragma unroll
+    for (int j = 1; j < 32; ++j) bmax = fmaxf(bmax, v[j]);
+    const float m_new = fmaxf(r.m2, bmax * scale2);
+    float sum = 0.f;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) sum += ex2_approx(fmaf(v[j], scale2, -m_new));
+    r.l = fmaf(r.l, ex2_approx(r.m2 - m_new), sum);
+    r.m2 = m_new;
 }
 
 // Survivor of packed token row t: the last s in [0, S) with cu_seqlens[s] <= t (this skips empty survivors).
@@ -151,17 +260,12 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
     const int64_t unit = PAIR ? (int64_t)(blockIdx.x >> 1) : (int64_t)blockIdx.x;
     const int64_t units = PAIR ? (int64_t)(gridDim.x >> 1) : (int64_t)gridDim.x;
 
-    int64_t T = p.T_max;
-    if (p.d_T) { const int64_t t = *p.d_T; T = t < 0 ? 0 : (t < T ? t : T); }
-    const int64_t m_tiles = (T + BM - 1) / BM;
-    const int64_t items = (PAIR ? (m_tiles + 1) / 2 : m_tiles) * p.splits;   // (pairs of) token tiles x splits
     const int k_steps = (p.d + BK - 1) / BK;
-    const int total_chunks = (p.V + BN - 1) / BN;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         // pair: the leading block's acc_empty collects the epilogue warps of both blocks
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], (PAIR ? 2 : 1) * (EPI_THREADS / 32)); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], (PAIR ? 2 : 1) * EPI_WARPS); }
         mbar_init(drain, 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -184,6 +288,12 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
         lead_full0 = map_to_cta(smem_u32(&full[0]), 0u);
         lead_acc_empty0 = map_to_cta(smem_u32(&acc_empty[0]), 0u);
     }
+    pdl_launch_dependents();       // the combining kernel may be set up while this one runs
+    pdl_wait();                    // the set-up above overlaps the end of the preceding kernel
+    int64_t T = p.T_max;
+    if (p.d_T) { const int64_t t = *pdl_acquire(p.d_T); T = t < 0 ? 0 : (t < T ? t : T); }
+    const int64_t m_tiles = (T + BM - 1) / BM;
+    const WorkList work = make_work_list(PAIR ? (m_tiles + 1) / 2 : m_tiles, units, p.plan);
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -191,52 +301,43 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
             uint32_t stage = 0, phase = 0;
             uint32_t issued = 0;
             bool ok = true;
-            int S = 0;
-            if constexpr (GATHER) {
-                const int64_t s64 = p.d_num[0];
-                S = (int)(s64 < 0 ? 0 : (s64 > (int64_t)p.S_max ? (int64_t)p.S_max : s64));
-            }
-            const int64_t waves = (items + units - 1) / units;
-            unsigned int wave = 0;
-            for (int64_t item = unit; ok && !p.mute_producer; item += units, ++wave) {
-                if (wave > 0 && wave < waves) {
-                    // hold the blocks in step: arrive for this wave (one arrival per unit), then wait for everybody (a
-                    // unit without a work item in the last, partial wave arrives as well and leaves)
-                    if (rank == 0) {
-                        __threadfence();
-                        atomicAdd(p.wave_counter, 1u);
+            const int32_t* tile_row = pdl_acquire(p.tile_row);
+            // first of the 128 source rows of this block's tile (gathered variant; requested one item ahead)
+            auto source_row = [&](const WorkItem& it) {
+                return tile_row[PAIR ? 2 * it.tile + (int64_t)rank : it.tile];
+            };
+            WorkItem it, next;
+            bool have = !p.mute_producer && work_item(work, p.plan, unit, units, 0, it);
+            int row = 0;
+            if constexpr (GATHER) if (have) row = source_row(it);
+            int64_t arrived = 0, waited = 0;        // waves
+            for (int64_t k = 0; !p.mute_producer; ++k) {
+                // hold the blocks in step: arrive for the item's wave (one arrival per unit and wave), then wait for
+                // everybody; a unit without an item in a partial wave arrives as well
+                const int64_t wave = have ? it.wave : work.waves - 1;
+                for (; arrived < wave; ++arrived)
+                    if (rank == 0) { __threadfence(); atomicAdd(p.wave_counter, 1u); }
+                if (!have) break;
+                if (wave > waited) {
+                    const unsigned int target = (unsigned int)wave * (unsigned int)units;
+                    uint32_t spin = 0;
+                    while (ld_acquire_u32(p.wave_counter) < target) {
+                        __nanosleep(64);
+                        if (++spin >= p.spin_limit || ((spin & 1023u) == 1023u && *abort_flag)) { ok = false; break; }
                     }
-                    if (item < items) {
-                        const unsigned int target = wave * (unsigned int)units;
-                        uint32_t it = 0;
-                        while (ld_acquire_u32(p.wave_counter) < target) {
-                            __nanosleep(64);
-                            if (++it >= p.spin_limit || ((it & 1023u) == 1023u && *abort_flag)) { ok = false; break; }
-                        }
-                        if (!ok) { *abort_flag = 1u; break; }
-                    }
+                    if (!ok) { *abort_flag = 1u; break; }
+                    waited = wave;
                 }
-                if (item >= items) break;
-                const int tile_unit = (int)(item / p.splits), split = (int)(item % p.splits);
-                const int m_tile = PAIR ? 2 * tile_unit + (int)rank : tile_unit;      // this block's 128 rows
-                const int c0 = split * p.chunks_per_split;
-                const int c1 = min(c0 + p.chunks_per_split, total_chunks);
+                const bool have_next = work_item(work, p.plan, unit, units, k + 1, next);
+                int row_next = 0;
+                if constexpr (GATHER) if (have_next) row_next = source_row(next);
+                const int c0 = p.plan.chunk_of_sub(it.sub0), c1 = p.plan.chunk_of_sub(it.sub1);
                 // where the tile's 128 rows come from: the packed rows, a run of source rows, or a scratch slot
                 const CUtensorMap* a_map = &map_h;
-                int a_row = m_tile * BM;
+                int a_row = (int)(PAIR ? 2 * it.tile + (int64_t)rank : it.tile) * BM;
                 if constexpr (GATHER) {
-                    const int64_t t0 = (int64_t)m_tile * BM;
-                    a_row = 0;                              // a pair's second tile may lie past T: any rows will do
-                    if (t0 < T) {
-                        const int s0 = survivor_of_row(p.cu_seqlens, S, t0);
-                        const int64_t s_end = p.cu_seqlens[s0 + 1];
-                        if (s_end < t0 + BM && s_end < T) {     // the tile runs on into the next survivor: pre-packed
-                            a_map = &map_s;
-                            a_row = s0 * BM;
-                        } else {
-                            a_row = (int)(p.src_tok_off[p.survivor_idx[s0]] + (t0 - p.cu_seqlens[s0]));
-                        }
-                    }
+                    a_row = row;
+                    if (row < 0) { a_map = &map_s; a_row = ~row; }
                 }
                 for (int c = c0; c < c1 && ok; ++c) {
                     for (int ks = 0; ks < k_steps; ++ks) {
@@ -247,7 +348,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                             if (rank == 0) mbar_expect_tx(&full[stage], 2 * STAGE_BYTES);
                             tma_load_2d_pair(stage_a + (size_t)stage * A_STAGE_BYTES, a_map, ks * BK, a_row, bar);
                             tma_load_2d_pair(stage_b + (size_t)stage * B_STAGE_BYTES, &map_w, ks * BK,
-                                             c * BN + (int)rank * PAIR_B_ROWS, bar);
+                                             c * BN + (int)rank * (chunk_columns(p.V, c) / 2), bar);
                         } else {
                             mbar_expect_tx(&full[stage], STAGE_BYTES);
                             tma_load_2d(stage_a + (size_t)stage * A_STAGE_BYTES, a_map, ks * BK, a_row, &full[stage]);
@@ -257,6 +358,10 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                     }
                 }
+                if (!ok) break;
+                it = next;
+                have = have_next;
+                row = row_next;
             }
             if (!ok && rank == 0) {
                 // Gave up: let the copies already issued land before the block's shared memory goes away.
@@ -280,16 +385,16 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
         // about the 512 cycles that they run.  200,000 tokens, d = 2048, V = 61,125 (pairs): 35.6 -> 34.8 ms; 100,000,
         // d = 4096, V = 151,936 (single blocks): 91.7 -> 90.6 ms.
         if (rank == 0) {
-            constexpr uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, BN);
+            const int k_last = (p.d - (k_steps - 1) * BK + UMMA_K - 1) / UMMA_K;     // K slices of the last K step
             const uint32_t a0 = smem_u32(stage_a), b0 = smem_u32(stage_b);
             uint32_t stage = 0, phase = 0;
             uint32_t acc = 0, acc_phase = 0;
             bool ok = true;
-            for (int64_t item = unit; item < items && ok; item += units) {
-                const int split = (int)(item % p.splits);
-                const int c0 = split * p.chunks_per_split;
-                const int c1 = min(c0 + p.chunks_per_split, total_chunks);
+            WorkItem it;
+            for (int64_t k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
+                const int c0 = p.plan.chunk_of_sub(it.sub0), c1 = p.plan.chunk_of_sub(it.sub1);
                 for (int c = c0; c < c1 && ok; ++c) {
+                    const uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, chunk_columns(p.V, c));
                     if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
                     tcgen05_fence_after();
                     const uint32_t d_tmem = tmem_base + acc * BN;
@@ -299,15 +404,20 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                         const uint64_t a_desc = make_smem_desc(a0 + stage * A_STAGE_BYTES);
                         const uint64_t b_desc = make_smem_desc(b0 + stage * B_STAGE_BYTES);
                         if (elect_one()) {
-#pragma unroll
-                            for (int k = 0; k < BK / UMMA_K; ++k) {
-                                // advancing K by 16 elements = 32 bytes inside the swizzle row: +2 in address units
+                            // advancing K by 16 elements = 32 bytes inside the swizzle row: +2 in address units
+                            auto mma = [&](int j) {
                                 if constexpr (PAIR)
-                                    tcgen05_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                                          (ks | k) != 0 ? 1u : 0u);
+                                    tcgen05_mma_bf16_pair(d_tmem, a_desc + (uint64_t)(2 * j), b_desc + (uint64_t)(2 * j), idesc,
+                                                          (ks | j) != 0 ? 1u : 0u);
                                 else
-                                    tcgen05_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                                     (ks | k) != 0 ? 1u : 0u);
+                                    tcgen05_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * j), b_desc + (uint64_t)(2 * j), idesc,
+                                                     (ks | j) != 0 ? 1u : 0u);
+                            };
+                            if (ks + 1 < k_steps || k_last == BK / UMMA_K) {
+#pragma unroll
+                                for (int j = 0; j < BK / UMMA_K; ++j) mma(j);
+                            } else {
+                                for (int j = 0; j < k_last; ++j) mma(j);     // slices past d are zeros
                             }
                             // stage reusable (in both blocks of a pair) once these MMAs have read it; after the last K
                             // step the accumulator is complete
@@ -334,91 +444,69 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
             __syncwarp();
         }
     } else {
-        // ---------------- epilogue: one token row per thread ----------------
+        // ---------------- epilogue: one token row (and its share of the columns) per thread ----------------
         const int quarter = warp & 3;                       // TMEM lanes 32*quarter .. 32*quarter+31
+        const int half = (warp - 2) >> 2;                   // columns EPI_COLS * half ... of every chunk
         const int row_in_tile = quarter * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+        const int32_t* targets = pdl_acquire(p.targets);
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int64_t item = unit; item < items && ok; item += units) {
-            const int tile_unit = (int)(item / p.splits), split = (int)(item % p.splits);
-            const int m_tile = PAIR ? 2 * tile_unit + (int)rank : tile_unit;
-            const int c0 = split * p.chunks_per_split;
-            const int c1 = min(c0 + p.chunks_per_split, total_chunks);
-            const int64_t t = (int64_t)m_tile * BM + row_in_tile;
-            const int y = (t < T) ? p.targets[t] : -1;
-            float m2 = -INFINITY, l = 0.f, zy2 = -INFINITY, sumz = 0.f;
-            const bool stamp = p.timing != nullptr && threadIdx.x == 64 && rank == 0 && item < p.timing_items;
-            if (stamp) { p.timing[4 * item] = global_timer_ns(); p.timing[4 * item + 2] = (unsigned long long)clock64(); }
-            for (int c = c0; c < c1 && ok; ++c) {
-                ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit);
-                ok = __all_sync(0xffffffffu, ok) != 0;     // keep the warp converged for the aligned tensor-memory loads
-                if (!ok) break;
-                tcgen05_fence_after();
-                const int col0 = c * BN;
+        WorkItem it;
+        for (int64_t k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
+            const int64_t t = (PAIR ? 2 * it.tile + (int64_t)rank : it.tile) * BM + row_in_tile;
+            const int y = (t < T) ? targets[t] : -1;
+            PartialLse sub = empty_record(), mid = empty_record(), group = empty_record();
+            const int64_t stamp_at = it.tile * p.plan.splits + it.group;
+            const bool stamp = p.timing != nullptr && threadIdx.x == 64 && rank == 0 && it.group >= 0 && stamp_at < p.timing_items;
+            if (stamp) { p.timing[4 * stamp_at] = global_timer_ns(); p.timing[4 * stamp_at + 2] = (unsigned long long)clock64(); }
+            int mid_i = it.group >= 0 ? p.plan.mid_of_group(it.group) : 0;
+            int mid_end = p.plan.sub_of_mid(mid_i + 1);
+            for (int s = it.sub0; s < it.sub1 && ok; ++s) {
+                const int c1 = p.plan.chunk_of_sub(s + 1);
+                for (int c = p.plan.chunk_of_sub(s); c < c1 && ok; ++c) {
+                    ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit);
+                    ok = __all_sync(0xffffffffu, ok) != 0;     // keep the warp converged for the aligned tensor-memory loads
+                    if (!ok) break;
+                    tcgen05_fence_after();
+                    const int col0 = c * BN + half * EPI_COLS;
 #pragma unroll 1
-                for (int piece = 0; piece < BN / 32; ++piece) {
-                    const int pc0 = col0 + piece * 32;
-                    if (pc0 >= p.V) break;                  // columns past the vocabulary (zero-filled by TMA)
-                    float v[32];
-                    tcgen05_ld_32x32(tmem_base + lane_addr + acc * BN + piece * 32, v);
-                    if constexpr (CONF) {                   // sum of the valid logits of the piece (before masking)
-                        float ps[4] = {0.f, 0.f, 0.f, 0.f};           // four chains; only the last piece needs the mask
-                        if (pc0 + 32 <= p.V) {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) ps[j & 3] += v[j];
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) ps[j & 3] += (pc0 + j < p.V) ? v[j] : 0.f;
-                        }
-                        sumz += (ps[0] + ps[1]) + (ps[2] + ps[3]);
+                    for (int piece = 0; piece < EPI_COLS / 32; ++piece) {
+                        const int pc0 = col0 + piece * 32;
+                        if (pc0 >= p.V) break;                  // columns past the vocabulary
+                        float v[32];
+                        tcgen05_ld_32x32(tmem_base + lane_addr + acc * BN + half * EPI_COLS + piece * 32, v);
+                        accumulate_piece<CONF>(v, pc0, y, p.V, p.scale2, sub);
                     }
-                    if (pc0 + 32 > p.V) {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) if (pc0 + j >= p.V) v[j] = -INFINITY;
+                    tcgen05_fence_before();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(lead_acc_empty0 + acc * (uint32_t)sizeof(uint64_t));
+                        else mbar_arrive(&acc_empty[acc]);
                     }
-                    if ((unsigned)(y - pc0) < 32u) {
-                        const int jy = y - pc0;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) if (j == jy) zy2 = v[j] * p.scale2;
-                    }
-                    float bmax = v[0];
-#pragma unroll
-                    for (int j = 1; j < 32; ++j) bmax = fmaxf(bmax, v[j]);
-                    const float m_new = fmaxf(m2, bmax * p.scale2);
-                    float sum = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) sum += ex2_approx(fmaf(v[j], p.scale2, -m_new));
-                    l = fmaf(l, ex2_approx(m2 - m_new), sum);
-                    m2 = m_new;
+                    if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
                 }
-                tcgen05_fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    if constexpr (PAIR) mbar_arrive_cluster(lead_acc_empty0 + acc * (uint32_t)sizeof(uint64_t));
-                    else mbar_arrive(&acc_empty[acc]);
+                if (it.group >= 0) {                           // the segment is complete: segment -> block -> group
+                    merge_record(mid, sub);
+                    sub = empty_record();
+                    if (s + 1 == mid_end) {
+                        merge_record(group, mid);
+                        mid = empty_record();
+                        mid_end = p.plan.sub_of_mid(++mid_i + 1);
+                    }
                 }
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
             }
-            if (stamp) { p.timing[4 * item + 1] = global_timer_ns(); p.timing[4 * item + 3] = (unsigned long long)clock64(); }
+            if (stamp) { p.timing[4 * stamp_at + 1] = global_timer_ns(); p.timing[4 * stamp_at + 3] = (unsigned long long)clock64(); }
             if (ok && t < T) {
-                if (p.splits == 1) {
-                    const float lse2 = m2 + log2f(l);
-                    const float ln2 = 0.69314718055994530942f;
-                    float out = 0.f;
-                    if (y >= 0) {
-                        if (y < p.V) out = (zy2 - lse2) * ln2;
-                        else atomicOr(p.d_status, ARROL_DEV_BAD_TARGET);
-                    }
-                    p.logp[t] = out;
-                    if (p.lse) p.lse[t] = lse2 * ln2;
-                    if constexpr (CONF) p.conf[t] = (float)p.V * (lse2 * ln2) - sumz * p.inv_temp;
+                const PartialLse& r = it.group >= 0 ? group : sub;
+                PartialLse* dst;
+                if (it.group >= 0) {
+                    dst = p.body + ((int64_t)it.group * HALVES + half) * p.T_max + t;
                 } else {
-                    PartialLse pr;
-                    pr.m2 = m2; pr.l = l; pr.zy2 = zy2; pr.pad = sumz;
-                    *reinterpret_cast<float4*>(&p.partial[(int64_t)split * p.T_max + t]) =
-                        make_float4(pr.m2, pr.l, pr.zy2, pr.pad);
+                    const int64_t tail_row = t - work.body_tiles * ((PAIR ? 2 : 1) * BM);
+                    dst = p.tail + (tail_row * p.plan.n_sub + it.sub0) * HALVES + half;
                 }
+                *reinterpret_cast<float4*>(dst) = make_float4(r.m2, r.l, r.zy2, r.sumz);
             }
         }
     }
@@ -442,7 +530,7 @@ __global__ void __launch_bounds__(PACK_THREADS)
 pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __restrict__ cu_seqlens,
                            const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off,
                            const int64_t* __restrict__ d_num, int S_max, int64_t T_max, int vec_per_row,
-                           uint4* __restrict__ scratch) {
+                           uint4* __restrict__ scratch, int32_t* __restrict__ tile_row) {
     __shared__ int64_t src_row_of[BM];
     pdl_launch_dependents();
     pdl_wait();
@@ -451,6 +539,20 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
     int64_t S64 = d_num[0], T = d_num[1];
     const int S = (int)(S64 < 0 ? 0 : (S64 > (int64_t)S_max ? (int64_t)S_max : S64));
     T = T < 0 ? 0 : (T < T_max ? T : T_max);
+    // where every token tile's rows come from (an even number of entries: a pair's second tile may lie past T)
+    const int64_t tiles = ((T + BM - 1) / BM + 1) / 2 * 2;
+    for (int64_t i = blockIdx.x * (int64_t)PACK_THREADS + threadIdx.x; i < tiles; i += (int64_t)gridDim.x * PACK_THREADS) {
+        const int64_t t0 = i * BM;
+        int32_t row = 0;
+        if (t0 < T) {
+            const int s0 = survivor_of_row(cu_seqlens, S, t0);
+            const int64_t s_end = cu_seqlens[s0 + 1];
+            // the tile runs on into the next survivor: its pre-packed copy
+            if (s_end < t0 + BM && s_end < T) row = ~(s0 * BM);
+            else row = (int32_t)(src_tok_off[survivor_idx[s0]] + (t0 - cu_seqlens[s0]));
+        }
+        tile_row[i] = row;
+    }
     for (int s0 = blockIdx.x; s0 < S; s0 += gridDim.x) {
         const int64_t begin = cu_seqlens[s0], end = cu_seqlens[s0 + 1];
         if (end <= begin || end >= T) continue;                 // empty, or nothing follows
@@ -486,46 +588,89 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
     }
 }
 
-// Merge of the per-split (max, sum, target logit) triples: M = max m_s, L = sum l_s 2^(m_s - M).
-__global__ void combine_splits_kernel(const PartialLse* __restrict__ partial, const int32_t* __restrict__ targets,
-                                      const int64_t* __restrict__ d_T, int64_t T_max, int V, int splits,
-                                      float* __restrict__ logp, float* __restrict__ lse, float* __restrict__ conf,
-                                      float inv_temp, uint32_t* d_status) {
+// Merges every token's records.  Tokens of the body: one thread each, splits x HALVES records.  Tokens of the tail: one
+// warp each; lane (block of segments, column half) merges its segments, then all lanes walk the blocks in order.
+constexpr int COMBINE_THREADS = 256;
+__global__ void __launch_bounds__(COMBINE_THREADS)
+combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
+                      int64_t T_max, int V, VocabPlan plan, int tile_rows, int64_t units, float* __restrict__ logp,
+                      float* __restrict__ lse, float* __restrict__ conf, float inv_temp, uint32_t* d_status) {
+    pdl_wait();
+    body = pdl_acquire(body); tail = pdl_acquire(tail); targets = pdl_acquire(targets); d_T = pdl_acquire(d_T);
     int64_t T = T_max;
     if (d_T) { const int64_t t = *d_T; T = t < 0 ? 0 : (t < T ? t : T); }
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T; t += (int64_t)gridDim.x * blockDim.x) {
-        float M = -INFINITY, zy2 = -INFINITY;
-        for (int s = 0; s < splits; ++s) {
-            const float4 pr = *reinterpret_cast<const float4*>(&partial[(int64_t)s * T_max + t]);
-            M = fmaxf(M, pr.x);
-            zy2 = fmaxf(zy2, pr.z);          // exactly one split holds the target column; the others hold -inf
-        }
-        float L = 0.f, sumz = 0.f;
-        for (int s = 0; s < splits; ++s) {
-            const float4 pr = *reinterpret_cast<const float4*>(&partial[(int64_t)s * T_max + t]);
-            L += pr.y * exp2f(pr.x - M);
-            sumz += pr.w;
-        }
-        const float lse2 = M + log2f(L);
+    const WorkList work = make_work_list((T + tile_rows - 1) / tile_rows, units, plan);
+    const int64_t body_rows = min(T, work.body_tiles * tile_rows);
+    auto load = [](const PartialLse* p) {
+        const float4 r = *reinterpret_cast<const float4*>(p);
+        return PartialLse{r.x, r.y, r.z, r.w};
+    };
+    auto finish = [&](int64_t t, const PartialLse (&halves)[HALVES]) {
+        PartialLse r = halves[0];
+#pragma unroll
+        for (int h = 1; h < HALVES; ++h) merge_record(r, halves[h]);
+        const float lse2 = r.m2 + log2f(r.l);
         const float ln2 = 0.69314718055994530942f;
         const int y = targets[t];
         float out = 0.f;
         if (y >= 0) {
-            if (y < V) out = (zy2 - lse2) * ln2;
+            if (y < V) out = (r.zy2 - lse2) * ln2;
             else atomicOr(d_status, ARROL_DEV_BAD_TARGET);
         }
         logp[t] = out;
         if (lse) lse[t] = lse2 * ln2;
-        if (conf) conf[t] = (float)V * (lse2 * ln2) - sumz * inv_temp;
+        if (conf) conf[t] = (float)V * (lse2 * ln2) - r.sumz * inv_temp;
+    };
+    const int64_t thread = blockIdx.x * (int64_t)COMBINE_THREADS + threadIdx.x;
+    const int64_t threads = (int64_t)gridDim.x * COMBINE_THREADS;
+    for (int64_t t = thread; t < body_rows; t += threads) {
+        PartialLse total[HALVES];
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) total[h] = empty_record();
+        for (int g = 0; g < plan.splits; ++g)
+#pragma unroll
+            for (int h = 0; h < HALVES; ++h) merge_record(total[h], load(body + ((int64_t)g * HALVES + h) * T_max + t));
+        finish(t, total);
+    }
+    const int lane = threadIdx.x & 31;
+    for (int64_t t = body_rows + (thread >> 5); t < T; t += threads >> 5) {
+        const PartialLse* rec = tail + (t - body_rows) * plan.n_sub * HALVES;
+        PartialLse total[HALVES], group[HALVES];
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) total[h] = group[h] = empty_record();
+        int g = 0;
+        for (int base = 0; base < plan.n_mid; base += COMBINE_BLOCKS) {
+            const int b = base + lane / HALVES;
+            PartialLse mine = empty_record();
+            if (b < plan.n_mid && lane < COMBINE_BLOCKS * HALVES) {
+                const int s1 = plan.sub_of_mid(b + 1);
+#pragma unroll 4
+                for (int s = plan.sub_of_mid(b); s < s1; ++s) merge_record(mine, load(rec + s * HALVES + lane % HALVES));
+            }
+            const int in_base = min(COMBINE_BLOCKS, plan.n_mid - base);
+            for (int j = 0; j < in_base; ++j) {
+#pragma unroll
+                for (int h = 0; h < HALVES; ++h) {
+                    const int from = j * HALVES + h;
+                    merge_record(group[h], PartialLse{__shfl_sync(0xffffffffu, mine.m2, from), __shfl_sync(0xffffffffu, mine.l, from),
+                                                      __shfl_sync(0xffffffffu, mine.zy2, from), __shfl_sync(0xffffffffu, mine.sumz, from)});
+                }
+                if (base + j + 1 == plan.mid_of_group(g + 1)) {
+#pragma unroll
+                    for (int h = 0; h < HALVES; ++h) { merge_record(total[h], group[h]); group[h] = empty_record(); }
+                    ++g;
+                }
+            }
+        }
+        if (lane == 0) finish(t, total);
     }
 }
 
 // How many vocabulary splits per token tile.  With one split every resident block streams a different token
 // tile (128 x d x 2 bytes each) against the same W chunks; when those tiles together outgrow about half of L2
 // the tiles are re-fetched from HBM once per chunk, so the vocabulary is split until they fit.
-int splits_for(const arrol_ctx* ctx, int64_t T_max, int d, int V, bool pair) {
+int splits_for(const arrol_ctx* ctx, int d, int V, bool pair) {
     const int total_chunks = (V + BN - 1) / BN;
-    const int64_t m_tiles = (T_max + BM - 1) / BM;
     // Measured with the blocks in step (TFLOP/s, packed rows / rows read in place by the gathered variant):
     //   d = 2048: 1 split (148 resident tiles, 74 MB) 1,380 / 1,200;  2 splits (74 tiles, 37 MB) 1,377 / 1,378
     //   d = 2560: 1 split (95 MB) 1,041 / 1,070;  2 splits (47 MB) 1,392 / 1,391;  4 splits (24 MB) 1,362 / 1,362
@@ -535,7 +680,7 @@ int splits_for(const arrol_ctx* ctx, int64_t T_max, int d, int V, bool pair) {
     //   d = 2560: 2 splits 1,428 / 1,413;  4 splits 1,403 / 1,396
     //   d = 4096: 2 splits (74 MB) 1,235 / 1,232;  4 splits (37 MB) 1,392 / 1,371;  8 splits 1,357 / 1,352
     // Token tiles beyond what L2 keeps are re-fetched from HBM once per chunk; every split beyond that streams
-    // W_vocab from HBM once more per wave.  So: two splits whenever there is a full wave of tiles (tiles read in place
+    // W_vocab from HBM once more per wave.  So: two splits (tiles read in place
     // are scattered over the source buffer and 148 of them do not stay resident even at 74 MB), more only while the
     // resident tiles exceed 80 MB (one block per tile) or 50 MB (pairs).  The packed and the in-place variant follow
     // the same rule, so their results are bit-identical.
@@ -544,52 +689,64 @@ int splits_for(const arrol_ctx* ctx, int64_t T_max, int d, int V, bool pair) {
     // seconds-long run under the 1 kW cap the SM clock settles 4 % lower (1,195 against 1,250 MHz, read by the kernel)
     // and the step is 2 % SLOWER (1,369 against 1,392-1,396 TFLOP/s).  So pairs only where they need no more splits.
     if (ctx->logprob_splits > 0) return ctx->logprob_splits < total_chunks ? ctx->logprob_splits : total_chunks;
-    int splits = m_tiles >= ctx->sm_count ? 2 : 1;
+    int splits = 2;
     const double l2_budget = (pair ? 50.0 : 80.0) * 1024 * 1024;
     const double tile_bytes = (double)BM * d * 2;
     while (splits < 8 && (ctx->sm_count / splits) * tile_bytes > l2_budget) splits *= 2;
-    // few token tiles: split so that every SM has work
-    while (splits < 16 && m_tiles * splits < ctx->sm_count && splits * 2 <= total_chunks) splits *= 2;
-    if (splits > total_chunks) splits = total_chunks;
-    return splits < 1 ? 1 : splits;
+    return splits < total_chunks ? splits : total_chunks;
 }
 
 // The form of the kernel for these sizes: pairs of blocks unless switched off, forced, or costlier in splits.
-bool pair_for(const arrol_ctx* ctx, int64_t T_max, int d, int V) {
+bool pair_for(const arrol_ctx* ctx, int d, int V) {
     if (ctx->sm_count < 2 || ctx->logprob_pair == 0) return false;
     if (ctx->logprob_pair == 1) return true;
-    return splits_for(ctx, T_max, d, V, true) <= splits_for(ctx, T_max, d, V, false);
+    return splits_for(ctx, d, V, true) <= splits_for(ctx, d, V, false);
 }
 
-int choose_splits(const arrol_ctx* ctx, int64_t T_max, int d, int V) {
-    return splits_for(ctx, T_max, d, V, pair_for(ctx, T_max, d, V));
+VocabPlan plan_for(const arrol_ctx* ctx, int d, int V) {
+    VocabPlan v;
+    v.total_chunks = (V + BN - 1) / BN;
+    v.splits = splits_for(ctx, d, V, pair_for(ctx, d, V));
+    // one segment per SM: then the tail's items fill the units (SMs, or half as many pairs) a whole number of times
+    v.n_sub = v.total_chunks < ctx->sm_count ? v.total_chunks : ctx->sm_count;
+    if (v.n_sub < v.splits) v.splits = v.n_sub;
+    const int per_group = COMBINE_BLOCKS / v.splits > 1 ? COMBINE_BLOCKS / v.splits : 1;
+    v.n_mid = v.splits * per_group < v.n_sub ? v.splits * per_group : v.n_sub;
+    return v;
+}
+
+// Workspace: wave counter, body records, tail records, source rows of the token tiles (gathered variant).  Every part
+// grows with T_max alone, so a workspace sized for T_max serves any call on fewer tokens with the same d and V.
+struct WorkspaceLayout { size_t body, tail, tile_row, total; };
+WorkspaceLayout workspace_layout(const arrol_ctx* ctx, int64_t T_max, int d, int V) {
+    const VocabPlan v = plan_for(ctx, d, V);
+    WorkspaceLayout L;
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    L.body = 256;
+    L.tail = L.body + up((size_t)v.splits * HALVES * (size_t)T_max * sizeof(PartialLse));
+    // tail tiles: at most units / splits + 1 tiles of 256 rows for pairs, of 128 rows for twice as many single blocks
+    const int64_t most = ((int64_t)(ctx->sm_count / 2) / v.splits + 1) * 2 * BM;
+    const int64_t rows = (T_max + 2 * BM - 1) / (2 * BM) * (2 * BM);
+    L.tile_row = L.tail + up((size_t)(rows < most ? rows : most) * v.n_sub * HALVES * sizeof(PartialLse));
+    L.total = L.tile_row + up((size_t)(rows / BM) * sizeof(int32_t));
+    return L;
 }
 
 }  // namespace
 
 extern "C" size_t arrol_token_logprob_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    // splits x tokens partial records.  Few token tiles get more splits (to fill the SMs) but then splits x tokens stays
-    // below two waves of tiles, so flooring the count there makes the size monotone in T_max: a workspace sized for
-    // T_max also serves any call on fewer tokens with the same d and V.
-    const int splits = choose_splits(ctx, T_max, d, V);
-    const size_t floor_records = (size_t)2 * ctx->sm_count * BM;
-    size_t records = (size_t)(splits > 1 ? splits : 0) * (size_t)T_max;
-    if (records < floor_records) records = floor_records;
-    return records * sizeof(PartialLse) + 256;
+    return workspace_layout(ctx, T_max, d, V).total;
 }
 
 extern "C" int32_t arrol_token_logprob_form(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    return pair_for(ctx, T_max, d, V) ? 2 : 1;
+    return pair_for(ctx, d, V) ? 2 : 1;
 }
 
 extern "C" int32_t arrol_token_logprob_splits(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    const int total_chunks = (V + BN - 1) / BN;
-    int splits = choose_splits(ctx, T_max, d, V);
-    const int chunks_per_split = (total_chunks + splits - 1) / splits;
-    return (total_chunks + chunks_per_split - 1) / chunks_per_split;
+    return plan_for(ctx, d, V).splits;
 }
 
 // Gather description of the gathered variant: the token rows come from `hidden` = the source buffer of
@@ -616,7 +773,8 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     if (d % 8 != 0) return ARROL_ERR_UNSUPPORTED;
     if (!arrol_aligned(hidden, 16) || !arrol_aligned(W_vocab, 16)) return ARROL_ERR_INVALID_ARG;
     if (T_max > (int64_t)INT32_MAX - BM) return ARROL_ERR_UNSUPPORTED;   // TMA coordinates are 32-bit
-    const size_t split_bytes = arrol_token_logprob_workspace(ctx, T_max, d, V);
+    const WorkspaceLayout L = workspace_layout(ctx, T_max, d, V);
+    const size_t split_bytes = L.total;
     const size_t need = split_bytes + (ga ? boundary_scratch_bytes(ga->S_max, d) : 0);
     if (!workspace || workspace_bytes < need || !arrol_aligned(workspace, 256)) return ARROL_ERR_WORKSPACE;
 
@@ -625,7 +783,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     cudaStream_t s = (cudaStream_t)stream;
 
     CUtensorMap map_h, map_s, map_w;
-    void* scratch = static_cast<uint8_t*>(workspace) + split_bytes;      // split_bytes is a multiple of 16 (256-aligned + records)
+    void* scratch = static_cast<uint8_t*>(workspace) + split_bytes;      // a multiple of 256 bytes
     if (make_map(ctx, &map_h, hidden, (uint64_t)(ga ? ga->source_rows : T_max), (uint64_t)d, BM) != ARROL_OK)
         return ARROL_ERR_CUDA;
     if (ga) {
@@ -634,7 +792,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         map_s = map_h;
     }
     // pair variant (clusters of two blocks): every block loads half of a chunk's W_vocab rows
-    const bool pair = pair_for(ctx, T_max, d, V);
+    const bool pair = pair_for(ctx, d, V);
     if (make_map(ctx, &map_w, W_vocab, (uint64_t)V, (uint64_t)d, pair ? PAIR_B_ROWS : BN) != ARROL_OK) return ARROL_ERR_CUDA;
 
     LogprobParams p;
@@ -643,40 +801,32 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     p.T_max = T_max;
     p.d = d;
     p.V = V;
-    p.splits = choose_splits(ctx, T_max, d, V);
-    const int total_chunks = (V + BN - 1) / BN;
-    p.chunks_per_split = (total_chunks + p.splits - 1) / p.splits;
-    p.splits = (total_chunks + p.chunks_per_split - 1) / p.chunks_per_split;   // no empty split
+    p.plan = plan_for(ctx, d, V);
     p.scale2 = inv_temperature * 1.44269504088896340736f;
-    p.logp = logp;
-    p.lse = lse;
-    p.conf = conf;
-    p.inv_temp = inv_temperature;
-    p.partial = static_cast<PartialLse*>(workspace);
+    uint8_t* ws = static_cast<uint8_t*>(workspace);
+    p.body = reinterpret_cast<PartialLse*>(ws + L.body);
+    p.tail = reinterpret_cast<PartialLse*>(ws + L.tail);
+    int32_t* tile_row = reinterpret_cast<int32_t*>(ws + L.tile_row);
     p.d_status = ctx->d_status;
     p.spin_limit = ctx->test_spin_limit ? ctx->test_spin_limit : SPIN_LIMIT;
     p.mute_producer = ctx->test_mute_producer;
-    p.cu_seqlens = ga ? ga->cu_seqlens : nullptr;
-    p.survivor_idx = ga ? ga->survivor_idx : nullptr;
-    p.src_tok_off = ga ? ga->src_tok_off : nullptr;
-    p.d_num = ga ? ga->d_num : nullptr;
-    p.S_max = ga ? ga->S_max : 0;
-    p.wave_counter = ctx->d_tile_counters + ARROL_TILE_COUNTERS - 1;   // last word of the page: not a scoring counter
+    p.tile_row = tile_row;
+    p.wave_counter = reinterpret_cast<unsigned int*>(ws);      // in the call's own workspace: calls on several streams do not share it
     p.timing = ctx->logprob_timing;
     p.timing_items = ctx->logprob_timing_items;
 
-    ARROL_CUDA_OK(cudaFuncSetAttribute(token_logprob_kernel<false, false, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(token_logprob_kernel<true, false, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(token_logprob_kernel<false, true, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(token_logprob_kernel<false, false, true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(token_logprob_kernel<false, true, true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(token_logprob_kernel<true, false, true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    if (!ctx->logprob_smem_set) {
+        const void* variants[] = {
+            reinterpret_cast<const void*>(token_logprob_kernel<false, false, false>),
+            reinterpret_cast<const void*>(token_logprob_kernel<true, false, false>),
+            reinterpret_cast<const void*>(token_logprob_kernel<false, true, false>),
+            reinterpret_cast<const void*>(token_logprob_kernel<false, false, true>),
+            reinterpret_cast<const void*>(token_logprob_kernel<true, false, true>),
+            reinterpret_cast<const void*>(token_logprob_kernel<false, true, true>)};
+        for (const void* f : variants)
+            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        ctx->logprob_smem_set = true;
+    }
     const int64_t m_tiles = (T_max + BM - 1) / BM;
     typedef void (*KernelFn)(CUtensorMap, CUtensorMap, CUtensorMap, LogprobParams);
     const int variant = ga ? 2 : (conf ? 1 : 0);
@@ -685,14 +835,14 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
                                                                          : token_logprob_kernel<false, false, true>);
     else fn = ga ? token_logprob_kernel<false, true, false> : (conf ? token_logprob_kernel<true, false, false>
                                                                      : token_logprob_kernel<false, false, false>);
-    // work items and the units that take them: blocks, or pairs of blocks on 256 rows
-    const int64_t items_max = (pair ? (m_tiles + 1) / 2 : m_tiles) * p.splits;
+    // the units that take the work items: blocks, or pairs of blocks on 256 rows
+    const int64_t tiles_max = pair ? (m_tiles + 1) / 2 : m_tiles;
     int64_t units = pair ? ctx->sm_count / 2 : ctx->sm_count;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(NUM_THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = s;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     int n_attr = 0;
     if (pair) {
         attr[n_attr].id = cudaLaunchAttributeClusterDimension;
@@ -716,15 +866,18 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         }
         if (units > ctx->pair_max_clusters[variant]) units = ctx->pair_max_clusters[variant];
     }
-    if (units > items_max) units = items_max;
+    if (units > tiles_max * p.plan.n_sub) units = tiles_max * p.plan.n_sub;
     const int64_t grid = pair ? 2 * units : units;
-    // more than one wave: the blocks wait for one another, so they must all be resident (single blocks: cooperative
-    // launch)
-    const bool several_waves = items_max > units;
+    // more than one wave: the blocks wait for one another, so they must all be resident (single blocks: cooperative launch)
+    const bool several_waves = make_work_list(tiles_max, units, p.plan).waves > 1;
     if (several_waves) ARROL_CUDA_OK(cudaMemsetAsync(p.wave_counter, 0, sizeof(unsigned int), s));
     if (several_waves && !pair) {
         attr[n_attr].id = cudaLaunchAttributeCooperative;
         attr[n_attr].val.cooperative = 1;
+        ++n_attr;
+    } else {
+        attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
         ++n_attr;
     }
     cfg.gridDim = dim3((unsigned)grid);
@@ -734,20 +887,23 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         int blocks = ga->S_max < ctx->sm_count * 4 ? ga->S_max : ctx->sm_count * 4;
         ARROL_CUDA_OK(arrol_launch_pdl(pack_boundary_tiles_kernel, dim3((unsigned)blocks), dim3(PACK_THREADS), 0, s,
                                        static_cast<const uint4*>(hidden), ga->cu_seqlens, ga->survivor_idx,
-                                       ga->src_tok_off, ga->d_num, ga->S_max, T_max, d / 8, static_cast<uint4*>(scratch)));
+                                       ga->src_tok_off, ga->d_num, ga->S_max, T_max, d / 8, static_cast<uint4*>(scratch), tile_row));
         ctx->launches += 1;
     }
     ARROL_CUDA_OK(cudaLaunchKernelEx(&cfg, fn, map_h, map_s, map_w, p));
     ctx->launches += 1;
     ARROL_CUDA_OK(cudaGetLastError());
-    if (p.splits > 1) {
-        int64_t blocks = (T_max + 255) / 256;
-        if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
-        combine_splits_kernel<<<(unsigned)blocks, 256, 0, s>>>(p.partial, targets, d_T, T_max, V, p.splits, logp,
-                                                              lse, conf, inv_temperature, ctx->d_status);
-        ctx->launches += 1;
-        ARROL_CUDA_OK(cudaGetLastError());
-    }
+    // one thread per token of the body, one warp per token of the tail
+    const int64_t tile_rows = (pair ? 2 : 1) * BM;
+    const int64_t tail_rows = (tiles_max < units / p.plan.splits + 1 ? tiles_max : units / p.plan.splits + 1) * tile_rows;
+    int64_t blocks = (T_max + COMBINE_THREADS - 1) / COMBINE_THREADS;
+    const int64_t tail_blocks = (tail_rows * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
+    if (blocks < tail_blocks) blocks = tail_blocks;
+    if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
+    ARROL_CUDA_OK(arrol_launch_pdl(combine_splits_kernel, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
+                                   static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
+                                   T_max, V, p.plan, (int)tile_rows, units, logp, lse, conf, inv_temperature, ctx->d_status));
+    ctx->launches += 1;
     return ARROL_OK;
 }
 

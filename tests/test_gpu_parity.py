@@ -545,3 +545,35 @@ def test_logprob_device_side_count_below_a_capacity_of_several_waves(T_live):
         assert np.abs(lp.cpu().numpy()[rows] - ref).max() <= 2e-3
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("pair", [0, 1])
+@pytest.mark.parametrize("V", [37, 300, 5000, 40000])            # one chunk; fewer segments than SMs; 157 chunks in 148 segments
+def test_logprob_bits_do_not_depend_on_the_token_count(V, pair):
+    """Whole waves of token tiles take one path, the rest (cut into vocabulary segments) another, merged by another kernel:
+    on both sides of every wave edge the rows a launch shares with a longer one get the same bits, and match the oracle."""
+    ctx = B.Context(0)
+    B.arrol_test_hook(ctx, B.HOOK_LOGPROB_PAIR, pair)
+    g = np.random.default_rng(V)
+    wave = 148 * 128 // 2                                        # tokens per wave with two vocabulary groups
+    T_max, d = 3 * wave + 700, 72
+    H = torch.from_numpy(g.normal(size=(T_max, d)).astype(np.float32)).to(torch.bfloat16)
+    W = torch.from_numpy(g.normal(0, 0.1, size=(V, d)).astype(np.float32)).to(torch.bfloat16)
+    y = g.integers(0, V, size=T_max).astype(np.int32)
+    Hd, Wd, yd = H.cuda(), W.cuda(), dev(y)
+    full = None
+    for T in (T_max, 3 * wave, 2 * wave + 1, 2 * wave - 1, wave + 129, wave + 1, wave, wave - 1, 257, 256, 128, 1):
+        ws = torch.empty(B.arrol_token_logprob_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+        lp, lse = torch.full((T,), 7.0, device="cuda"), torch.full((T,), 7.0, device="cuda")
+        B.arrol_token_logprob(ctx, Hd, Wd, yd, T, d, V, lp, ws, lse=lse)
+        torch.cuda.synchronize()
+        if full is None:
+            full = (lp, lse)
+        assert torch.equal(lp, full[0][:T]) and torch.equal(lse, full[1][:T])
+    rows = np.unique(np.concatenate([[0, wave - 1, wave, 2 * wave - 1, 2 * wave, 3 * wave - 1, 3 * wave, T_max - 1],
+                                     g.integers(0, T_max, size=24)])).astype(np.int64)
+    lp_ref, lse_ref = oracle.token_logprob(synth.as_oracle_array(H), synth.as_oracle_array(W), y, rows=rows)
+    assert np.abs(full[0].cpu().numpy()[rows] - lp_ref).max() <= LOGP_TOL
+    assert np.abs(full[1].cpu().numpy()[rows] - lse_ref).max() <= LOGP_TOL
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    ctx.close()
