@@ -442,7 +442,7 @@ def measure(w, C, K, W, local, barrier, rank, full, args):
             print("e2e leg skipped: %s" % str(exc).splitlines()[0], file=sys.stderr)
 
     # ---- the log-prob call with the kernel's OTHER form.  The library runs the kernel as pairs of blocks on 256-row
-    # tiles (tcgen05 cta_group::2) where pairs need no more vocabulary splits than single blocks, else as one block per
+    # tiles (tcgen05 cta_group::2) for hidden widths above 512, else as one block per
     # 128-row tile (see include/arrol.h, ARROL_HOOK_LOGPROB_PAIR); this leg forces the form the step did not use ----
     other_kernel = None
     kernel_form = int(B.arrol_token_logprob_form(ctx, views[0].cap, w.d, w.V))

@@ -51,7 +51,8 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
     ctx->test_spin_limit = 0;
     ctx->test_mute_producer = 0;
     ctx->logprob_pair = 2;
-    for (int i = 0; i < 3; ++i) ctx->pair_max_clusters[i] = 0;
+    for (auto& width : ctx->pair_max_clusters)
+        for (int& n : width) n = 0;
     ctx->logprob_splits = 0;
     ctx->logprob_timing = nullptr;
     ctx->logprob_timing_items = 0;

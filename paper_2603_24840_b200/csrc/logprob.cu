@@ -68,10 +68,7 @@ constexpr int PAIR_B_STAGE_BYTES = PAIR_B_ROWS * BK * 2;   // 16 KB
 constexpr int PAIR_STAGE_BYTES = A_STAGE_BYTES + PAIR_B_STAGE_BYTES;
 static_assert(PAIR_STAGES * PAIR_STAGE_BYTES == SOLO_STAGES * SOLO_STAGE_BYTES, "both variants fill the same shared memory");
 constexpr int TMEM_COLS = 512;   // two fp32 accumulators of BN columns
-constexpr int EPI_WARPS = 4;                 // EPI_WARPS / 4 warps per tensor-memory lane quarter share a chunk's columns
-constexpr int HALVES = EPI_WARPS / 4;
-constexpr int EPI_COLS = BN / HALVES;
-constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
+constexpr int num_threads(int halves) { return 64 + 128 * halves; }     // producer, issuer, four epilogue warps per column half
 constexpr int COMBINE_BLOCKS = 16;           // blocks of segments (n_mid) that one warp merges side by side
 constexpr size_t SMEM_BYTES = (size_t)SOLO_STAGES * SOLO_STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
 
@@ -152,8 +149,8 @@ struct LogprobParams {
     int d, V;
     VocabPlan plan;
     float scale2;          // inv_temperature * log2(e)
-    PartialLse* body;      // [splits][HALVES][T_max]: records of the tokens in whole waves
-    PartialLse* tail;      // [token of the tail][n_sub][HALVES]
+    PartialLse* body;      // [splits][column halves][T_max]: records of the tokens in whole waves
+    PartialLse* tail;      // [token of the tail][n_sub][column halves]
     uint32_t spin_limit;   // tries per pipeline wait
     int mute_producer;     // test hook: the producer issues no copies
     uint32_t* d_status;
@@ -233,13 +230,15 @@ __device__ __forceinline__ int survivor_of_row(const int64_t* __restrict__ cu_se
 // blocks' tensor memory, every block loads its own 128 rows of A and its own 128 of the chunk's 256 W_vocab rows and
 // runs the epilogue of its own rows.  Per block and K step 32 KB come in from L2 instead of 48 KB and the tensor
 // core reads 8 KB of operands per MMA from shared memory instead of 12 KB.
-template <bool CONF, bool GATHER, bool PAIR>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+// HALVES: epilogue warps per tensor-memory lane quarter; two share a chunk's columns between them.
+template <bool CONF, bool GATHER, bool PAIR, int HALVES>
+__global__ void __launch_bounds__(num_threads(HALVES), 1)
 token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_s,
                      const __grid_constant__ CUtensorMap map_w, const LogprobParams p) {
     constexpr int STAGES = PAIR ? PAIR_STAGES : SOLO_STAGES;
     constexpr int B_STAGE_BYTES = PAIR ? PAIR_B_STAGE_BYTES : SOLO_B_STAGE_BYTES;
     constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
+    constexpr int EPI_WARPS = 4 * HALVES, EPI_COLS = BN / HALVES;
     extern __shared__ uint8_t smem_raw[];
     // stage buffers need 1024-byte alignment for the 128-byte swizzle pattern
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -591,6 +590,7 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
 // Merges every token's records.  Tokens of the body: one thread each, splits x HALVES records.  Tokens of the tail: one
 // warp each; lane (block of segments, column half) merges its segments, then all lanes walk the blocks in order.
 constexpr int COMBINE_THREADS = 256;
+template <int HALVES>
 __global__ void __launch_bounds__(COMBINE_THREADS)
 combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
                       int64_t T_max, int V, VocabPlan plan, int tile_rows, int64_t units, float* __restrict__ logp,
@@ -680,14 +680,9 @@ int splits_for(const arrol_ctx* ctx, int d, int V, bool pair) {
     //   d = 2560: 2 splits 1,428 / 1,413;  4 splits 1,403 / 1,396
     //   d = 4096: 2 splits (74 MB) 1,235 / 1,232;  4 splits (37 MB) 1,392 / 1,371;  8 splits 1,357 / 1,352
     // Token tiles beyond what L2 keeps are re-fetched from HBM once per chunk; every split beyond that streams
-    // W_vocab from HBM once more per wave.  So: two splits (tiles read in place
-    // are scattered over the source buffer and 148 of them do not stay resident even at 74 MB), more only while the
-    // resident tiles exceed 80 MB (one block per tile) or 50 MB (pairs).  The packed and the in-place variant follow
+    // W_vocab from HBM once more per wave.  So: two splits (tiles read in place are scattered over the source buffer and
+    // 148 of them do not stay resident even at 74 MB), more only while the resident tiles exceed 80 MB (one block per tile) or 50 MB (pairs).  The packed and the in-place variant follow
     // the same rule, so their results are bit-identical.
-    // Which form: pairs are 1.5-3 % faster at equal split counts; where they need more splits than single blocks
-    // (d = 4096: four against two) the extra W_vocab streams and the busier tensor pipe draw more power, and in a
-    // seconds-long run under the 1 kW cap the SM clock settles 4 % lower (1,195 against 1,250 MHz, read by the kernel)
-    // and the step is 2 % SLOWER (1,369 against 1,392-1,396 TFLOP/s).  So pairs only where they need no more splits.
     if (ctx->logprob_splits > 0) return ctx->logprob_splits < total_chunks ? ctx->logprob_splits : total_chunks;
     int splits = 2;
     const double l2_budget = (pair ? 50.0 : 80.0) * 1024 * 1024;
@@ -696,17 +691,27 @@ int splits_for(const arrol_ctx* ctx, int d, int V, bool pair) {
     return splits < total_chunks ? splits : total_chunks;
 }
 
-// The form of the kernel for these sizes: pairs of blocks unless switched off, forced, or costlier in splits.
-bool pair_for(const arrol_ctx* ctx, int d, int V) {
+// The form of the kernel for these sizes (V = 61,125, 100,000 tokens; us as single blocks with 4 / 8 epilogue warps and as
+// pairs with 4 / 8):
+//   d = 256   3,676 / 3,090   3,935 / 3,514        d = 640    6,006 / 6,120    6,297 / 5,877
+//   d = 384   4,393 / 3,879   4,616 / 4,385        d = 768    7,140 / 7,242    6,954 / 6,653
+//   d = 512   5,077 / 5,000   5,595 / 5,168        d = 1,024  9,376 / 9,445    8,798 / 8,854
+//   d = 4,096 (V = 151,936, 287,000 tokens): single blocks with two splits 250.6 ms, pairs with four 247.9 ms
+// A chunk's 128 x 256 exponentials take an SM's special-function units 2,048 cycles, its MMAs 8 d: at small d the epilogue
+// sets the pace.  Two warps per scheduler then hide the latency of one another's tensor-memory loads, and single blocks
+// hand an accumulator back without waiting for a peer's epilogue.  At large d the tensor pipe and the power cap set it:
+// pairs move fewer operand bytes, and the fewer epilogue warps draw less power.
+constexpr int PAIR_MIN_WIDTH = 513, EIGHT_WARPS_MAX_WIDTH = 896;
+bool pair_for(const arrol_ctx* ctx, int d) {
     if (ctx->sm_count < 2 || ctx->logprob_pair == 0) return false;
-    if (ctx->logprob_pair == 1) return true;
-    return splits_for(ctx, d, V, true) <= splits_for(ctx, d, V, false);
+    return ctx->logprob_pair == 1 || d >= PAIR_MIN_WIDTH;
 }
+int halves_for(int d) { return d <= EIGHT_WARPS_MAX_WIDTH ? 2 : 1; }
 
 VocabPlan plan_for(const arrol_ctx* ctx, int d, int V) {
     VocabPlan v;
     v.total_chunks = (V + BN - 1) / BN;
-    v.splits = splits_for(ctx, d, V, pair_for(ctx, d, V));
+    v.splits = splits_for(ctx, d, V, pair_for(ctx, d));
     // one segment per SM: then the tail's items fill the units (SMs, or half as many pairs) a whole number of times
     v.n_sub = v.total_chunks < ctx->sm_count ? v.total_chunks : ctx->sm_count;
     if (v.n_sub < v.splits) v.splits = v.n_sub;
@@ -721,13 +726,14 @@ struct WorkspaceLayout { size_t body, tail, tile_row, total; };
 WorkspaceLayout workspace_layout(const arrol_ctx* ctx, int64_t T_max, int d, int V) {
     const VocabPlan v = plan_for(ctx, d, V);
     WorkspaceLayout L;
+    const int halves = halves_for(d);
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     L.body = 256;
-    L.tail = L.body + up((size_t)v.splits * HALVES * (size_t)T_max * sizeof(PartialLse));
+    L.tail = L.body + up((size_t)v.splits * halves * (size_t)T_max * sizeof(PartialLse));
     // tail tiles: at most units / splits + 1 tiles of 256 rows for pairs, of 128 rows for twice as many single blocks
     const int64_t most = ((int64_t)(ctx->sm_count / 2) / v.splits + 1) * 2 * BM;
     const int64_t rows = (T_max + 2 * BM - 1) / (2 * BM) * (2 * BM);
-    L.tile_row = L.tail + up((size_t)(rows < most ? rows : most) * v.n_sub * HALVES * sizeof(PartialLse));
+    L.tile_row = L.tail + up((size_t)(rows < most ? rows : most) * v.n_sub * halves * sizeof(PartialLse));
     L.total = L.tile_row + up((size_t)(rows / BM) * sizeof(int32_t));
     return L;
 }
@@ -741,7 +747,7 @@ extern "C" size_t arrol_token_logprob_workspace(arrol_ctx* ctx, int64_t T_max, i
 
 extern "C" int32_t arrol_token_logprob_form(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    return pair_for(ctx, d, V) ? 2 : 1;
+    return pair_for(ctx, d) ? 2 : 1;
 }
 
 extern "C" int32_t arrol_token_logprob_splits(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
@@ -792,7 +798,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         map_s = map_h;
     }
     // pair variant (clusters of two blocks): every block loads half of a chunk's W_vocab rows
-    const bool pair = pair_for(ctx, d, V);
+    const bool pair = pair_for(ctx, d);
     if (make_map(ctx, &map_w, W_vocab, (uint64_t)V, (uint64_t)d, pair ? PAIR_B_ROWS : BN) != ARROL_OK) return ARROL_ERR_CUDA;
 
     LogprobParams p;
@@ -815,31 +821,29 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     p.timing = ctx->logprob_timing;
     p.timing_items = ctx->logprob_timing_items;
 
-    if (!ctx->logprob_smem_set) {
-        const void* variants[] = {
-            reinterpret_cast<const void*>(token_logprob_kernel<false, false, false>),
-            reinterpret_cast<const void*>(token_logprob_kernel<true, false, false>),
-            reinterpret_cast<const void*>(token_logprob_kernel<false, true, false>),
-            reinterpret_cast<const void*>(token_logprob_kernel<false, false, true>),
-            reinterpret_cast<const void*>(token_logprob_kernel<true, false, true>),
-            reinterpret_cast<const void*>(token_logprob_kernel<false, true, true>)};
-        for (const void* f : variants)
-            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-        ctx->logprob_smem_set = true;
-    }
     const int64_t m_tiles = (T_max + BM - 1) / BM;
     typedef void (*KernelFn)(CUtensorMap, CUtensorMap, CUtensorMap, LogprobParams);
+    // [pair][two column halves][plain, with confidence, rows in place]
+    static const KernelFn kernels[2][2][3] = {
+        {{token_logprob_kernel<false, false, false, 1>, token_logprob_kernel<true, false, false, 1>, token_logprob_kernel<false, true, false, 1>},
+         {token_logprob_kernel<false, false, false, 2>, token_logprob_kernel<true, false, false, 2>, token_logprob_kernel<false, true, false, 2>}},
+        {{token_logprob_kernel<false, false, true, 1>, token_logprob_kernel<true, false, true, 1>, token_logprob_kernel<false, true, true, 1>},
+         {token_logprob_kernel<false, false, true, 2>, token_logprob_kernel<true, false, true, 2>, token_logprob_kernel<false, true, true, 2>}}};
+    if (!ctx->logprob_smem_set) {
+        for (const auto& form : kernels)
+            for (const auto& width : form)
+                for (const KernelFn f : width)
+                    ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+        ctx->logprob_smem_set = true;
+    }
+    const int halves = halves_for(d);
     const int variant = ga ? 2 : (conf ? 1 : 0);
-    KernelFn fn;
-    if (pair) fn = ga ? token_logprob_kernel<false, true, true> : (conf ? token_logprob_kernel<true, false, true>
-                                                                         : token_logprob_kernel<false, false, true>);
-    else fn = ga ? token_logprob_kernel<false, true, false> : (conf ? token_logprob_kernel<true, false, false>
-                                                                     : token_logprob_kernel<false, false, false>);
+    const KernelFn fn = kernels[pair ? 1 : 0][halves - 1][variant];
     // the units that take the work items: blocks, or pairs of blocks on 256 rows
     const int64_t tiles_max = pair ? (m_tiles + 1) / 2 : m_tiles;
     int64_t units = pair ? ctx->sm_count / 2 : ctx->sm_count;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(NUM_THREADS);
+    cfg.blockDim = dim3(num_threads(halves));
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = s;
     cudaLaunchAttribute attr[3];
@@ -855,16 +859,16 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         // ("LaunchFailed"; the same grid without the attribute profiles), so the check is made here instead: never
         // more pairs than the occupancy query says fit at once (asked once per context and kernel variant).  The
         // waits themselves are bounded either way.
-        if (ctx->pair_max_clusters[variant] == 0) {
+        if (ctx->pair_max_clusters[halves - 1][variant] == 0) {
             cfg.gridDim = dim3((unsigned)(2 * units));
             cfg.attrs = attr;
             cfg.numAttrs = n_attr;
             int fit = 0;
             ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&fit, fn, &cfg));
             if (fit < 1) return ARROL_ERR_CUDA;
-            ctx->pair_max_clusters[variant] = fit;
+            ctx->pair_max_clusters[halves - 1][variant] = fit;
         }
-        if (units > ctx->pair_max_clusters[variant]) units = ctx->pair_max_clusters[variant];
+        if (units > ctx->pair_max_clusters[halves - 1][variant]) units = ctx->pair_max_clusters[halves - 1][variant];
     }
     if (units > tiles_max * p.plan.n_sub) units = tiles_max * p.plan.n_sub;
     const int64_t grid = pair ? 2 * units : units;
@@ -900,7 +904,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     const int64_t tail_blocks = (tail_rows * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
     if (blocks < tail_blocks) blocks = tail_blocks;
     if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
-    ARROL_CUDA_OK(arrol_launch_pdl(combine_splits_kernel, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
+    ARROL_CUDA_OK(arrol_launch_pdl(halves == 2 ? combine_splits_kernel<2> : combine_splits_kernel<1>, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
                                    static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
                                    T_max, V, p.plan, (int)tile_rows, units, logp, lse, conf, inv_temperature, ctx->d_status));
     ctx->launches += 1;

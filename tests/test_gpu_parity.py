@@ -548,17 +548,18 @@ def test_logprob_device_side_count_below_a_capacity_of_several_waves(T_live):
 
 
 @pytest.mark.parametrize("pair", [0, 1])
-@pytest.mark.parametrize("V", [37, 300, 5000, 40000])            # one chunk; fewer segments than SMs; 157 chunks in 148 segments
-def test_logprob_bits_do_not_depend_on_the_token_count(V, pair):
+@pytest.mark.parametrize("V,d", [(37, 72), (300, 512), (40000, 72),            # one chunk; two; 157 chunks in 148 segments
+                                 (5000, 520), (700, 896), (700, 904)])         # both sides of the widths where the form changes
+def test_logprob_bits_do_not_depend_on_the_token_count(V, d, pair):
     """Whole waves of token tiles take one path, the rest (cut into vocabulary segments) another, merged by another kernel:
     on both sides of every wave edge the rows a launch shares with a longer one get the same bits, and match the oracle."""
     ctx = B.Context(0)
     B.arrol_test_hook(ctx, B.HOOK_LOGPROB_PAIR, pair)
     g = np.random.default_rng(V)
     wave = 148 * 128 // 2                                        # tokens per wave with two vocabulary groups
-    T_max, d = 3 * wave + 700, 72
+    T_max = 3 * wave + 700
     H = torch.from_numpy(g.normal(size=(T_max, d)).astype(np.float32)).to(torch.bfloat16)
-    W = torch.from_numpy(g.normal(0, 0.1, size=(V, d)).astype(np.float32)).to(torch.bfloat16)
+    W = torch.from_numpy(g.normal(0, 0.8 / d ** 0.5, size=(V, d)).astype(np.float32)).to(torch.bfloat16)
     y = g.integers(0, V, size=T_max).astype(np.int32)
     Hd, Wd, yd = H.cuda(), W.cuda(), dev(y)
     full = None
