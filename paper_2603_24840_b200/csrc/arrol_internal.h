@@ -19,6 +19,7 @@ struct arrol_ctx {
     uint32_t* d_tile_counters; // MLP head on the tensor cores: finished blocks per row tile, zero between calls
     unsigned long long* d_chain;   // fused prune step: finished blocks, index-check flag, per-block totals; zero between calls
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
+    bool backward_smem_set;    // likewise for the lm_head backward
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
     uint32_t test_spin_limit;  // arrol_test_hook: tries per pipeline wait of the log-prob kernel, 0 = the normal limit

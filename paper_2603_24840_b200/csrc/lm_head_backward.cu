@@ -9,19 +9,29 @@
 //   dz_kernel     recomputes the chunk's logits tile by tile and turns each accumulator tile into dz (bf16),
 //                 written once as dZ [TC, V]
 //   gemm_kernel   dH[chunk] = dZ . W       A = dZ K-major (K = V contiguous), B = W MN-major (N = d contiguous)
-//   gemm_kernel   dW       += dZ^T . H     A = dZ MN-major (M = V contiguous), B = H chunk MN-major
+//   gemm_kernel   dW       (+)= dZ^T . H   A = dZ MN-major (M = V contiguous), B = H chunk MN-major
 // The MN-major operands are read by the tensor core straight from their row-major storage (transpose bits in the
 // instruction descriptor, MN-major shared-memory descriptors), so nothing is transposed in memory and the T x V
 // matrix exists only one chunk at a time, once, in the workspace.
+//
+// All three work as PAIRS of blocks (clusters of two, tcgen05 cta_group::2) on 256 x 256 tiles: block r of a pair owns
+// the tile's rows 128 r ..., brings them and half of the tile's 256 columns of B, and runs the epilogue of its rows;
+// block 0 issues the MMAs for both.  Per block and K step 32 KB come in from L2 instead of the 48 KB of a 128 x 256 tile of
+// its own.  These kernels are bound by the board's power cap and by the SM-to-L2 path, which their results share with
+// the operands, not by the issue of MMAs (a warp-uniform issuer alone changed nothing), so fewer operand bytes are what
+// helps.  Whole call against single blocks (which also walked the dead tiles of a partly live chunk): 47,360 tokens,
+// d = 2048, V = 128,256 59.0 -> 56.8 ms; 28,000, d = 4096, V = 151,936 85.8 -> 78.6 ms; 3,000, d = 2048 6.78 -> 3.92 ms; 600,
+// d = 1024, V = 30,000 689 -> 221 us.
 #include "arrol_internal.h"
 #include "tc_common.cuh"
 
 namespace {
 
-constexpr int BM = 128, BN = 256;
-constexpr int STAGES = 4;
+constexpr int BM = 128, BN = 256;        // rows of a block, columns of a tile
+constexpr int TILE_ROWS = 2 * BM;        // rows of a pair's tile
+constexpr int STAGES = 6;
 constexpr int A_STAGE_BYTES = BM * BK * 2;
-constexpr int B_STAGE_BYTES = BN * BK * 2;
+constexpr int B_STAGE_BYTES = BN / 2 * BK * 2;
 constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr int MN_BLOCK_BYTES = BK * 128;   // one 64-element MN block of an MN-major stage: BK rows of 128 bytes
 constexpr int TMEM_COLS = 512;
@@ -33,7 +43,7 @@ constexpr int EPI_PIECES = BN / 32 / (EPI_WARPS / 4);   // 32-column pieces per 
 constexpr int EPI_STAGE_TILE = 32 * 128;
 constexpr size_t EPI_STAGE_OFFSET = (size_t)STAGES * STAGE_BYTES + 1024;
 constexpr size_t SMEM_BYTES = EPI_STAGE_OFFSET + (size_t)EPI_WARPS * EPI_STAGE_TILE + 1024;
-constexpr int TC = 74 * BM;      // tokens per chunk: 74 token tiles, so that TC/128 x d/256 tiles fill 148 SMs evenly
+constexpr int TC = 37 * TILE_ROWS;      // tokens per chunk: 37 tiles of a pair, so that TC/256 x d/256 tiles fill 74 pairs evenly
 
 struct PipeSmem {
     uint8_t* stage_a;
@@ -41,9 +51,14 @@ struct PipeSmem {
     uint64_t *full, *empty, *acc_full, *acc_empty, *drain;
     uint32_t* tmem_slot;
     volatile uint32_t* abort_flag;
+    uint32_t rank;                           // of this block in its pair (0 leads)
+    uint32_t tmem_base;
+    uint32_t lead_full, lead_acc_empty;      // shared::cluster addresses in the leading block
 };
 
-__device__ __forceinline__ PipeSmem carve_smem(uint8_t* smem_raw) {
+// Common prologue: barriers, tensor-memory allocation, then the wait for the preceding kernel (everything before it
+// overlaps that kernel's end).
+__device__ __forceinline__ PipeSmem pipe_setup(uint8_t* smem_raw, const CUtensorMap* ma, const CUtensorMap* mb) {
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     PipeSmem ps;
     ps.stage_a = smem;
@@ -56,72 +71,78 @@ __device__ __forceinline__ PipeSmem carve_smem(uint8_t* smem_raw) {
     ps.drain = ps.acc_empty + 2;
     ps.tmem_slot = reinterpret_cast<uint32_t*>(ps.drain + 1);
     ps.abort_flag = ps.tmem_slot + 1;
-    return ps;
-}
-
-// Common prologue: barriers, tensor-memory allocation.  Returns the tensor-memory base address.
-__device__ __forceinline__ uint32_t pipe_setup(const PipeSmem& ps, const CUtensorMap* ma, const CUtensorMap* mb) {
-    const int warp = threadIdx.x >> 5;
+    ps.rank = cluster_cta_rank();
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&ps.full[s], 1); mbar_init(&ps.empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&ps.acc_full[b], 1); mbar_init(&ps.acc_empty[b], EPI_WARPS); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&ps.acc_full[b], 1); mbar_init(&ps.acc_empty[b], 2 * EPI_WARPS); }
         mbar_init(ps.drain, 1);
         *ps.abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(ma) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(mb) : "memory");
     }
-    if (warp == 1) {
-        tcgen05_alloc(ps.tmem_slot, TMEM_COLS);
-        tcgen05_relinquish();
+    if ((threadIdx.x >> 5) == 1) {
+        tcgen05_alloc_pair(ps.tmem_slot, TMEM_COLS);
+        tcgen05_relinquish_pair();
     }
     tcgen05_fence_before();
     __syncthreads();
+    cluster_sync_all();                      // the peer's barriers exist before anything arrives on them
     tcgen05_fence_after();
-    return *ps.tmem_slot;
+    ps.tmem_base = *ps.tmem_slot;
+    ps.lead_full = map_to_cta(smem_u32(&ps.full[0]), 0u);
+    ps.lead_acc_empty = map_to_cta(smem_u32(&ps.acc_empty[0]), 0u);
+    pdl_launch_dependents();
+    pdl_wait();
+    return ps;
 }
 
-__device__ __forceinline__ void pipe_teardown(const PipeSmem& ps, uint32_t tmem_base, uint32_t* d_status) {
+__device__ __forceinline__ void pipe_teardown(const PipeSmem& ps, uint32_t* d_status) {
     tcgen05_fence_before();
     __syncthreads();
+    cluster_sync_all();                      // neither block's shared or tensor memory goes away under the other
     if (threadIdx.x == 0 && *ps.abort_flag) atomicOr(d_status, ARROL_DEV_WAIT_EXPIRED);
     if ((threadIdx.x >> 5) == 1) {
         tcgen05_fence_after();
-        tcgen05_dealloc(tmem_base, TMEM_COLS);
+        tcgen05_dealloc_pair(ps.tmem_base, TMEM_COLS);
     }
 }
 
-// Producer role (one thread).  For every accumulator tile `coords(it, a_mn0, b_mn0)` gives the operands' MN
-// origins (it returns false when the tile list is exhausted); for every K step the stage receives
-//   K-major operand:  one box  [MN rows x 64 K columns]           at (x = k, y = mn0)
-//   MN-major operand: MN/64 blocks [64 K rows x 64 MN columns], BK*128 bytes apart: one three-dimensional box
-//                     (64 elements, 64 K rows, MN/64 blocks) at (0, k, mn0/64) when the map is of that kind
+// One accumulator tile's operands: origin of the tile's rows (A) and columns (B), and the columns that the MMA computes.
+struct TileAt { int a0, b0, n; };
+
+// Producer role (one thread of each block).  For every accumulator tile `coords(it, tile)` gives the operands' MN origins
+// (false when the list is exhausted); this block loads rows a0 + 128 rank ... of A and b0 + (n / 2) rank ... of B.  Per K step
+//   K-major operand:  one box  [128 MN rows x 64 K columns]      at (x = k, y = mn0)
+//   MN-major operand: 2 blocks [64 K rows x 64 MN columns], BK*128 bytes apart: one three-dimensional box
+//                     (64 elements, 64 K rows, 2 blocks) at (0, k, mn0/64) when the map is of that kind
 //                     (a3d / b3d), else one two-dimensional box per block at (x = mn0 + 64 b, y = k).
-// Issuing a copy costs the thread about 60 cycles, and a stage's MMAs last 512: with one copy per operand the
-// producer keeps ahead of the tensor pipe, with six it does not.
+// Both blocks' bytes are counted on the leading block's barrier.
 template <bool A_MN, bool B_MN, typename Coords>
 __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensorMap* ma, const CUtensorMap* mb,
                                               int k_steps, Coords coords, bool a3d = false, bool b3d = false,
                                               const CUtensorMap* mb_tail = nullptr, int tail_ks = -1) {
     uint32_t stage = 0, phase = 0, issued = 0;
     bool ok = true;
-    int ay, by;
-    for (int64_t it = 0; ok && coords(it, ay, by); ++it) {
+    TileAt tile;
+    for (int64_t it = 0; ok && coords(it, tile); ++it) {
+        const int ay = tile.a0 + (int)ps.rank * BM, by = tile.b0 + (int)ps.rank * (tile.n / 2);
         for (int ks = 0; ks < k_steps; ++ks) {
             if (!mbar_wait(&ps.empty[stage], phase ^ 1u, ps.abort_flag)) { ok = false; break; }
-            mbar_expect_tx(&ps.full[stage], STAGE_BYTES);
+            const uint32_t bar = ps.lead_full + stage * (uint32_t)sizeof(uint64_t);
+            if (ps.rank == 0) mbar_expect_tx(&ps.full[stage], 2 * STAGE_BYTES);
             uint8_t* sa = ps.stage_a + (size_t)stage * A_STAGE_BYTES;
             uint8_t* sb = ps.stage_b + (size_t)stage * B_STAGE_BYTES;
             if constexpr (A_MN) {
                 if (a3d) {
-                    tma_load_3d(sa, ma, 0, ks * BK, ay >> 6, &ps.full[stage]);
+                    tma_load_3d_pair(sa, ma, 0, ks * BK, ay >> 6, bar);
                 } else {
 #pragma unroll
                     for (int b = 0; b < BM / 64; ++b)
-                        tma_load_2d(sa + b * MN_BLOCK_BYTES, ma, ay + 64 * b, ks * BK, &ps.full[stage]);
+                        tma_load_2d_pair(sa + b * MN_BLOCK_BYTES, ma, ay + 64 * b, ks * BK, bar);
                 }
             } else {
-                tma_load_2d(sa, ma, ks * BK, ay, &ps.full[stage]);
+                tma_load_2d_pair(sa, ma, ks * BK, ay, bar);
             }
             if constexpr (B_MN) {
                 // the K step that holds the last, partly live block of rows is read from its zero-padded copy
@@ -129,20 +150,22 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
                 const CUtensorMap* m = tail ? mb_tail : mb;
                 const int ky = tail ? 0 : ks * BK;
                 if (b3d) {
-                    tma_load_3d(sb, m, 0, ky, by >> 6, &ps.full[stage]);
+                    tma_load_3d_pair(sb, m, 0, ky, by >> 6, bar);
                 } else {
 #pragma unroll
-                    for (int b = 0; b < BN / 64; ++b)
-                        tma_load_2d(sb + b * MN_BLOCK_BYTES, m, by + 64 * b, ky, &ps.full[stage]);
+                    for (int b = 0; b < BN / 2 / 64; ++b)
+                        tma_load_2d_pair(sb + b * MN_BLOCK_BYTES, m, by + 64 * b, ky, bar);
                 }
             } else {
-                tma_load_2d(sb, mb, ks * BK, by, &ps.full[stage]);
+                tma_load_2d_pair(sb, mb, ks * BK, by, bar);
             }
             ++issued;
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
     }
-    if (!ok) {   // gave up: let the copies already issued land before shared memory goes away (bounded)
+    if (!ok && ps.rank == 0) {
+        // gave up: let the copies already issued land before shared memory goes away (bounded); the peer's copies are
+        // counted here too, and the cluster barrier at the end keeps its shared memory alive until then
         const uint32_t pending = issued < (uint32_t)STAGES ? issued : (uint32_t)STAGES;
         uint32_t s = stage, ph = phase;
         for (uint32_t i = 0; i < pending; ++i) {
@@ -153,50 +176,66 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
     }
 }
 
-// MMA role (one thread): n_items accumulator tiles of k_steps K steps each, alternating the two accumulators.
+// MMA role (one warp of the leading block): the accumulator tiles that `columns(it)` lists (their MMA columns, 0 = no
+// more), k_steps K steps each (the last one of k_last slices of 16), alternating the two accumulators.  The whole warp
+// walks the loops and waits, one elected lane issues.
 // Inside a stage the four K = 16 slices are 32 bytes apart for a K-major operand (columns of the swizzled row) and
 // 16 rows = 2048 bytes apart for an MN-major one.
-template <bool A_MN, bool B_MN>
-__device__ __forceinline__ void mma_loop(const PipeSmem& ps, uint32_t tmem_base, int64_t n_items, int k_steps) {
-    constexpr uint32_t idesc = make_idesc(BM, BN, A_MN, B_MN);
+template <bool A_MN, bool B_MN, typename Columns>
+__device__ __forceinline__ void mma_loop(const PipeSmem& ps, int k_steps, int k_last, Columns columns) {
     constexpr uint64_t a_step = A_MN ? (UMMA_K * 128) >> 4 : (UMMA_K * 2) >> 4;
     constexpr uint64_t b_step = B_MN ? (UMMA_K * 128) >> 4 : (UMMA_K * 2) >> 4;
+    const uint32_t a0 = smem_u32(ps.stage_a), b0 = smem_u32(ps.stage_b);
     uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
     bool ok = true;
-    for (int64_t it = 0; it < n_items && ok; ++it) {
-        if (!mbar_wait(&ps.acc_empty[acc], acc_phase ^ 1u, ps.abort_flag)) { ok = false; break; }
+    for (int64_t it = 0; ok; ++it) {
+        const int n = columns(it);
+        if (n == 0) break;
+        const uint32_t idesc = make_idesc(TILE_ROWS, n, A_MN, B_MN);
+        if (!mbar_wait_warp(&ps.acc_empty[acc], acc_phase ^ 1u, ps.abort_flag)) { ok = false; break; }
         tcgen05_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
+        const uint32_t d_tmem = ps.tmem_base + acc * BN;
         for (int ks = 0; ks < k_steps; ++ks) {
-            if (!mbar_wait(&ps.full[stage], phase, ps.abort_flag)) { ok = false; break; }
+            if (!mbar_wait_warp(&ps.full[stage], phase, ps.abort_flag)) { ok = false; break; }
             tcgen05_fence_after();
-            const uint32_t sa = smem_u32(ps.stage_a + (size_t)stage * A_STAGE_BYTES);
-            const uint32_t sb = smem_u32(ps.stage_b + (size_t)stage * B_STAGE_BYTES);
+            const uint32_t sa = a0 + stage * A_STAGE_BYTES, sb = b0 + stage * B_STAGE_BYTES;
             const uint64_t a_desc = A_MN ? make_smem_desc_mn(sa, BK) : make_smem_desc(sa);
             const uint64_t b_desc = B_MN ? make_smem_desc_mn(sb, BK) : make_smem_desc(sb);
+            if (elect_one()) {
+                if (ks + 1 < k_steps || k_last == BK / UMMA_K) {
 #pragma unroll
-            for (int k = 0; k < BK / UMMA_K; ++k)
-                tcgen05_mma_bf16(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, (ks | k) != 0 ? 1u : 0u);
-            tcgen05_commit(&ps.empty[stage]);
+                    for (int k = 0; k < BK / UMMA_K; ++k)
+                        tcgen05_mma_bf16_pair(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, (ks | k) != 0 ? 1u : 0u);
+                } else {
+                    for (int k = 0; k < k_last; ++k)         // slices past the end of K are zeros
+                        tcgen05_mma_bf16_pair(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, (ks | k) != 0 ? 1u : 0u);
+                }
+                tcgen05_commit_pair(&ps.empty[stage], (uint16_t)3);
+                if (ks + 1 == k_steps) tcgen05_commit_pair(&ps.acc_full[acc], (uint16_t)3);
+            }
+            __syncwarp();
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (ok) tcgen05_commit(&ps.acc_full[acc]);
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
-    if (!ok) {
-        tcgen05_commit(ps.drain);
+    if (!ok && elect_one()) {
+        tcgen05_commit_pair(ps.drain, (uint16_t)1);
         for (uint32_t spin = 0; spin < SPIN_LIMIT; ++spin)
             if (mbar_try_wait(ps.drain, 0u)) break;
     }
+    __syncwarp();
 }
 
 __device__ __forceinline__ int64_t live_tokens(const int64_t* d_T, int64_t T_max) {
     int64_t T = T_max;
-    if (d_T) { const int64_t t = *d_T; T = t < 0 ? 0 : (t < T ? t : T); }
+    if (d_T) { const int64_t t = *pdl_acquire(d_T); T = t < 0 ? 0 : (t < T ? t : T); }
     return T;
 }
 
 // ---- dz: recompute logits, write the softmax gradient of one token chunk --------------------------------------
+// Work item = (vocabulary chunk of 256 columns, token tile), the chunk as the slow index: the pairs share W_vocab chunks and
+// token tiles through L2, and a chunk with few live tiles still spreads evenly.  When the token tiles of the whole chunk
+// outgrow L2's share (50 MB, as in the forward kernel), they go in groups of `group_tiles`, each with its own pass over W_vocab.
 struct DzParams {
     const int32_t* targets;
     const float* grad_logp;
@@ -204,170 +243,201 @@ struct DzParams {
     const int64_t* d_T;
     int64_t T_max, t0;        // chunk = tokens [t0, t0 + TC)
     int d, V;
-    int64_t ldz;              // row pitch of dZ (V rounded up to 8)
-    int splits, chunks_per_split;
+    int group_tiles;
     float scale2, inv_temp;
-    __nv_bfloat16* dZ;        // [TC, ldz]
+    const uint16_t* hidden;
+    uint16_t* tail;           // [64, d]: the last, partly live 64-row block of the chunk's hidden rows, zero-padded
     uint32_t* d_status;
 };
+
+__device__ __forceinline__ bool dz_item(int64_t i, int m_tiles, int total_chunks, int group_tiles, int& m, int& c) {
+    const int64_t per_group = (int64_t)group_tiles * total_chunks;
+    const int64_t g = i / per_group;
+    const int first = (int)g * group_tiles;
+    if (first >= m_tiles) return false;
+    const int size = min(group_tiles, m_tiles - first);
+    i -= g * per_group;
+    if (i >= (int64_t)size * total_chunks) return false;
+    c = (int)(i / size);
+    m = first + (int)(i - (int64_t)c * size);
+    return true;
+}
+
+// Columns of vocabulary chunk c that the MMA computes: a multiple of 32 (the granularity of N for a pair).
+__device__ __forceinline__ int chunk_columns(int V, int c) {
+    const int left = V - c * BN;
+    return left >= BN ? BN : (left + 31) & ~31;
+}
 
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w,
           const __grid_constant__ CUtensorMap map_dz, const DzParams p) {
     extern __shared__ uint8_t smem_raw[];
-    const PipeSmem ps = carve_smem(smem_raw);
+    const PipeSmem ps = pipe_setup(smem_raw, &map_h, &map_w);
     uint8_t* dz_stage = ps.stage_a + EPI_STAGE_OFFSET;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t T = live_tokens(p.d_T, p.T_max);
-    if (p.t0 >= T) return;                                  // chunk past the live tokens (uniform for the grid)
-    const int64_t items = (int64_t)(TC / BM) * p.splits;
+    const int live = (int)max((int64_t)0, min((int64_t)TC, T - p.t0));     // 0: chunk past the live tokens, nothing to do
+    const int m_tiles = (live + TILE_ROWS - 1) / TILE_ROWS;
     const int k_steps = (p.d + BK - 1) / BK;
+    const int k_last = (p.d - (k_steps - 1) * BK + UMMA_K - 1) / UMMA_K;
     const int total_chunks = (p.V + BN - 1) / BN;
-    const uint32_t tmem_base = pipe_setup(ps, &map_h, &map_w);
-
-    // work item -> (token tile, vocabulary range); the accumulator tiles of one item are its vocabulary chunks
-    auto item_range = [&](int64_t item, int& m_tile, int& c0, int& c1) {
-        m_tile = (int)(item / p.splits);
-        const int split = (int)(item % p.splits);
-        c0 = split * p.chunks_per_split;
-        c1 = min(c0 + p.chunks_per_split, total_chunks);
-    };
+    const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
 
     if (warp == 0) {
         if (lane == 0) {
-            int64_t item = blockIdx.x;
-            int m_tile = 0, c = 0, c1 = 0;
-            bool have = false;
-            producer_loop<false, false>(ps, &map_h, &map_w, k_steps, [&](int64_t, int& ay, int& by) {
-                while (!have || c >= c1) {
-                    if (have) item += gridDim.x;
-                    if (item >= items) return false;
-                    item_range(item, m_tile, c, c1);
-                    have = true;
-                }
-                ay = (int)(p.t0 + (int64_t)m_tile * BM);
-                by = c * BN;
-                ++c;
+            producer_loop<false, false>(ps, &map_h, &map_w, k_steps, [&](int64_t it, TileAt& t) {
+                int m, c;
+                if (!dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c)) return false;
+                t.a0 = (int)p.t0 + m * TILE_ROWS;
+                t.b0 = c * BN;
+                t.n = chunk_columns(p.V, c);
                 return true;
             });
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int64_t n_tiles = 0;
-            for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-                int m_tile, c0, c1;
-                item_range(item, m_tile, c0, c1);
-                n_tiles += max(c1 - c0, 0);
-            }
-            mma_loop<false, false>(ps, tmem_base, n_tiles, k_steps);
-        }
+        if (ps.rank == 0)
+            mma_loop<false, false>(ps, k_steps, k_last, [&](int64_t it) {
+                int m, c;
+                return dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c) ? chunk_columns(p.V, c) : 0;
+            });
     } else {
+        // The last, partly live 64-row block of the chunk's hidden rows, padded with zeros, for the dW contraction: rows past
+        // the live tokens (caller memory that may hold anything) never reach the tensor core.
+        if (live % BK != 0) {
+            const int r0 = live / BK * BK, vec_per_row = p.d / 8;
+            const uint16_t* hidden = pdl_acquire(p.hidden);
+            for (int i = (int)blockIdx.x * 32 * EPI_WARPS + (int)threadIdx.x - 64; i < BK * vec_per_row; i += (int)gridDim.x * 32 * EPI_WARPS) {
+                const int r = i / vec_per_row, v = i - r * vec_per_row;
+                uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                if (r0 + r < live) x = *reinterpret_cast<const uint4*>(hidden + (p.t0 + r0 + r) * p.d + v * 8);
+                *reinterpret_cast<uint4*>(p.tail + (int64_t)r * p.d + v * 8) = x;
+            }
+        }
+        const int32_t* targets = pdl_acquire(p.targets);
+        const float* grad_logp = pdl_acquire(p.grad_logp);
+        const float* lse = pdl_acquire(p.lse);
         const int quarter = warp & 3;
         const int col_half = (warp - 2) >> 2;           // 0 or 1: which half of the accumulator's columns
-        const int row_in_tile = quarter * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+        // dz leaves through shared memory: the warp's 32 rows x 64 columns (two pieces, 128 bytes per row, 128-byte
+        // swizzle) are staged and written by one TMA tile store, i.e. in whole 128-byte lines; columns past V are
+        // clipped by the copy.  (16-byte stores straight from the registers touch 32 lines per instruction and
+        // cost the kernel 14 %.)
+        uint8_t* stg = dz_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        for (int64_t item = blockIdx.x; item < items && ok; item += gridDim.x) {
-            int m_tile, c0, c1;
-            item_range(item, m_tile, c0, c1);
-            const int row_in_chunk = m_tile * BM + row_in_tile;
-            const int64_t t = p.t0 + row_in_chunk;
+        int m, c;
+        for (int64_t item = unit; ok && dz_item(item, m_tiles, total_chunks, p.group_tiles, m, c); item += units) {
+            const int row0 = m * TILE_ROWS + (int)ps.rank * BM + quarter * 32;
+            const int64_t t = p.t0 + row0 + lane;
             int y = -1;
             float coef = 0.f, lse2 = 0.f;
             if (t < T) {
-                y = p.targets[t];
+                y = targets[t];
                 if (y >= 0 && y < p.V) {
-                    coef = p.grad_logp[t] * p.inv_temp;
-                    lse2 = p.lse[t] * 1.44269504088896340736f;
+                    coef = grad_logp[t] * p.inv_temp;
+                    lse2 = lse[t] * 1.44269504088896340736f;
                 } else {
                     y = -1;
                 }
             }
-            // dz leaves through shared memory: the warp's 32 rows x 64 columns (two pieces, 128 bytes per row, 128-byte
-            // swizzle) are staged and written by one TMA tile store, i.e. in whole 128-byte lines; columns past V are
-            // clipped by the copy.  (16-byte stores straight from the registers touch 32 lines per instruction and
-            // cost the kernel 14 %.)
-            uint8_t* stg = dz_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
-            const int row0 = m_tile * BM + quarter * 32;
-            for (int c = c0; c < c1 && ok; ++c) {
-                ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
-                ok = __all_sync(0xffffffffu, ok) != 0;
-                if (!ok) break;
-                tcgen05_fence_after();
-                // Two register buffers: the tensor-memory load of piece i + 1 is in flight while piece i is turned
-                // into dz and staged.
-                const uint32_t tacc = tmem_base + lane_addr + acc * BN;
-                auto to_dz = [&](const uint32_t (&raw)[32], int piece, uint32_t (&packed)[16]) {
-                    const int pc0 = c * BN + piece * 32;
+            ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
+            ok = __all_sync(0xffffffffu, ok) != 0;
+            if (!ok) break;
+            tcgen05_fence_after();
+            // Two register buffers: the tensor-memory load of piece i + 1 is in flight while piece i is turned
+            // into dz and staged.
+            const uint32_t tacc = ps.tmem_base + lane_addr + acc * BN;
+            auto to_dz = [&](const uint32_t (&raw)[32], int piece, uint32_t (&packed)[16]) {
+                const int pc0 = c * BN + piece * 32;
 #pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        // dz = coef ([v = y] - 2^(z log2e - lse log2e)); coef = 0 for rows that carry no gradient
-                        float d0 = -coef * ex2_approx(fmaf(__uint_as_float(raw[j]), p.scale2, -lse2));
-                        float d1 = -coef * ex2_approx(fmaf(__uint_as_float(raw[j + 1]), p.scale2, -lse2));
-                        if (pc0 + j == y) d0 += coef;
-                        if (pc0 + j + 1 == y) d1 += coef;
-                        if (coef == 0.f) { d0 = 0.f; d1 = 0.f; }      // also guards 0 * inf from stale lse values
-                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(d0, d1);
-                        packed[j >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
-                    }
-                };
-                auto stage_piece = [&](const uint32_t (&packed)[16], int piece) {
-                    const int chunk0 = (piece & 1) * 4;               // 16-byte chunks of the 128-byte staging row
-#pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4)
-                        *reinterpret_cast<uint4*>(stg + lane * 128 + (((chunk0 + q4) ^ (lane & 7)) << 4)) =
-                            make_uint4(packed[4 * q4], packed[4 * q4 + 1], packed[4 * q4 + 2], packed[4 * q4 + 3]);
-                };
-                uint32_t ra[32], rb[32];
-                const int p0 = col_half * EPI_PIECES, p1 = p0 + EPI_PIECES;   // this warp's pieces of the accumulator
-                tcgen05_ld_32x32_issue(tacc + p0 * 32, ra);
-#pragma unroll 1
-                for (int piece = p0; piece < p1; piece += 2) {
-                    tcgen05_ld_wait(ra);
-                    tcgen05_ld_32x32_issue(tacc + (piece + 1) * 32, rb);
-                    uint32_t pa[16], pb[16];
-                    to_dz(ra, piece, pa);
-                    tcgen05_ld_wait(rb);
-                    if (piece + 2 < p1) tcgen05_ld_32x32_issue(tacc + (piece + 2) * 32, ra);
-                    to_dz(rb, piece + 1, pb);
-                    if (lane == 0) bulk_wait_read_all();          // the previous tile store has read the staging tile
-                    __syncwarp();
-                    stage_piece(pa, piece);
-                    stage_piece(pb, piece + 1);
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    const int col0 = c * BN + piece * 32;
-                    if (lane == 0 && col0 < p.V) {
-                        tma_store_2d(&map_dz, col0, row0, stg);
-                        bulk_commit_group();
-                    }
+                for (int j = 0; j < 32; j += 2) {
+                    // dz = coef ([v = y] - 2^(z log2e - lse log2e)); coef = 0 for rows that carry no gradient
+                    float d0 = -coef * ex2_approx(fmaf(__uint_as_float(raw[j]), p.scale2, -lse2));
+                    float d1 = -coef * ex2_approx(fmaf(__uint_as_float(raw[j + 1]), p.scale2, -lse2));
+                    if (pc0 + j == y) d0 += coef;
+                    if (pc0 + j + 1 == y) d1 += coef;
+                    if (coef == 0.f) { d0 = 0.f; d1 = 0.f; }      // also guards 0 * inf from stale lse values
+                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(d0, d1);
+                    packed[j >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
                 }
-                tcgen05_fence_before();
+            };
+            auto stage_piece = [&](const uint32_t (&packed)[16], int piece) {
+                const int chunk0 = (piece & 1) * 4;               // 16-byte chunks of the 128-byte staging row
+#pragma unroll
+                for (int q4 = 0; q4 < 4; ++q4)
+                    *reinterpret_cast<uint4*>(stg + lane * 128 + (((chunk0 + q4) ^ (lane & 7)) << 4)) =
+                        make_uint4(packed[4 * q4], packed[4 * q4 + 1], packed[4 * q4 + 2], packed[4 * q4 + 3]);
+            };
+            uint32_t ra[32], rb[32];
+            const int p0 = col_half * EPI_PIECES, p1 = p0 + EPI_PIECES;   // this warp's pieces of the accumulator
+            tcgen05_ld_32x32_issue(tacc + p0 * 32, ra);
+#pragma unroll 1
+            for (int piece = p0; piece < p1; piece += 2) {
+                tcgen05_ld_wait(ra);
+                tcgen05_ld_32x32_issue(tacc + (piece + 1) * 32, rb);
+                uint32_t pa[16], pb[16];
+                to_dz(ra, piece, pa);
+                tcgen05_ld_wait(rb);
+                if (piece + 2 < p1) tcgen05_ld_32x32_issue(tacc + (piece + 2) * 32, ra);
+                to_dz(rb, piece + 1, pb);
+                if (lane == 0) bulk_wait_read_all();          // the previous tile store has read the staging tile
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ps.acc_empty[acc]);
-                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+                stage_piece(pa, piece);
+                stage_piece(pb, piece + 1);
+                fence_proxy_async_smem();
+                __syncwarp();
+                const int col0 = c * BN + piece * 32;
+                if (lane == 0 && col0 < p.V) {
+                    tma_store_2d(&map_dz, col0, row0, stg);
+                    bulk_commit_group();
+                }
             }
+            tcgen05_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait_all();       // the tile stores have completed before the block's shared memory goes
     }
-    pipe_teardown(ps, tmem_base, p.d_status);
+    pipe_teardown(ps, p.d_status);
 }
 
 // ---- C[M,N] (+)= op(A) op(B): bf16 operands in either orientation, fp32 result ------------------------------------
 //   A_MN = false: A stored [M, K] row-major;  A_MN = true: A stored [K, M] row-major (used as its transpose)
 //   B_MN = false: B stored [N, K] row-major;  B_MN = true: B stored [K, N] row-major
+// Tiles of 256 x 256, dealt to the pairs in groups of `group_n` column tiles: within a group consecutive pairs share the
+// A panel and walk the B panels.  group_n keeps the B panels of a group (for dW a whole chunk of hidden rows) in L2 and the
+// wave of 74 tiles near square, which is what it reads least bytes per K step with.
 struct GemmParams {
     int M, N, K;
-    float* C;
-    int64_t ldc;
+    int group_n;
     int accumulate;           // 1: C += ..., 0: C = ...
-    int k_is_tokens;          // 1: K counts the chunk's tokens: only the live ones (T - t0) are contracted
+    // rows of M (dH) or extent of K (dW) that count the chunk's tokens: only the live ones (T - t0) are contracted; dead rows
+    // of C are written as zeros
+    int m_is_tokens, k_is_tokens;
+    int zero_if_dead;         // chunk without a live token: C = 0 instead of leaving it alone
     int a3d, b3d;             // the MN-major operand's maps are three-dimensional (one copy per stage)
-    const int64_t* d_T;       // the launch is skipped when t0 >= live tokens
+    const int64_t* d_T;
     int64_t T_max, t0;
     uint32_t* d_status;
 };
+
+struct GemmTile { int m, n; };
+__device__ __forceinline__ bool gemm_item(int64_t i, int m_tiles, int n_tiles, int group_n, GemmTile& t) {
+    const int64_t per_group = (int64_t)m_tiles * group_n;
+    if (per_group == 0) return false;
+    const int64_t g = i / per_group;
+    const int first = (int)g * group_n;
+    if (first >= n_tiles) return false;
+    const int size = min(group_n, n_tiles - first);
+    i -= g * per_group;
+    t.m = (int)(i / size);
+    if (t.m >= m_tiles) return false;
+    t.n = first + (int)(i - (int64_t)t.m * size);
+    return true;
+}
 
 template <bool A_MN, bool B_MN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -375,56 +445,61 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const __grid_constant__ CUtensorMap map_b_tail, const __grid_constant__ CUtensorMap map_c,
             const GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
-    const PipeSmem ps = carve_smem(smem_raw);
+    const PipeSmem ps = pipe_setup(smem_raw, &map_a, &map_b);
     uint8_t* c_stage = ps.stage_a + EPI_STAGE_OFFSET;      // one 32 x 32 fp32 staging tile per epilogue warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t T_live = live_tokens(p.d_T, p.T_max);
-    if (p.t0 >= T_live) return;
-    const int m_tiles = (p.M + BM - 1) / BM, n_tiles = (p.N + BN - 1) / BN;
-    const int64_t items = (int64_t)m_tiles * n_tiles;
-    const int K = p.k_is_tokens ? (int)min((int64_t)p.K, T_live - p.t0) : p.K;
+    const int64_t live = max((int64_t)0, live_tokens(p.d_T, p.T_max) - p.t0);
+    const int n_tiles = (p.N + BN - 1) / BN;
+    const int all_m_tiles = (p.M + TILE_ROWS - 1) / TILE_ROWS;
+    const int K = p.k_is_tokens ? (int)min((int64_t)p.K, live) : p.K;
     const int k_steps = (K + BK - 1) / BK;
-    const uint32_t tmem_base = pipe_setup(ps, &map_a, &map_b);
+    const int k_last = (K - (k_steps - 1) * BK + UMMA_K - 1) / UMMA_K;
+    // tiles that are contracted; the rest (rows of tokens that do not live) is written as zeros
+    const int m_tiles = K == 0 ? 0 : p.m_is_tokens ? (int)min((int64_t)all_m_tiles, (live + TILE_ROWS - 1) / TILE_ROWS) : all_m_tiles;
+    const int zero_m_tiles = live > 0 || p.zero_if_dead ? all_m_tiles - m_tiles : 0;
+    const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
+    // 64 columns per block at least: the granularity of an MN-major B tile's blocks
+    auto columns = [&](int n) { const int left = p.N - n * BN; return left > BN / 2 ? BN : BN / 2; };
 
     if (warp == 0) {
         if (lane == 0) {
             const int tail_ks = (p.k_is_tokens && (K % BK) != 0) ? k_steps - 1 : -1;
-            producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, k_steps, [&](int64_t it, int& ay, int& by) {
-                const int64_t item = blockIdx.x + it * gridDim.x;
-                if (item >= items) return false;
-                ay = (int)(item / n_tiles) * BM;       // consecutive blocks share the A panel, walk the B panels
-                by = (int)(item % n_tiles) * BN;
+            producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, k_steps, [&](int64_t it, TileAt& t) {
+                GemmTile g;
+                if (!gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g)) return false;
+                t.a0 = g.m * TILE_ROWS;
+                t.b0 = g.n * BN;
+                t.n = columns(g.n);
                 return true;
             }, p.a3d != 0, p.b3d != 0, &map_b_tail, tail_ks);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const int64_t mine = items > blockIdx.x ? (items - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-            mma_loop<A_MN, B_MN>(ps, tmem_base, mine, k_steps);
-        }
+        if (ps.rank == 0)
+            mma_loop<A_MN, B_MN>(ps, k_steps, k_last, [&](int64_t it) {
+                GemmTile g;
+                return gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g) ? columns(g.n) : 0;
+            });
     } else {
         const int quarter = warp & 3;
         const int col_half = (warp - 2) >> 2;           // 0 or 1: which half of the accumulator's columns
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        uint32_t acc = 0, acc_phase = 0;
-        bool ok = true;
-        for (int64_t item = blockIdx.x; item < items && ok; item += gridDim.x) {
-            const int col0 = (int)(item % n_tiles) * BN;
-            ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
-            ok = __all_sync(0xffffffffu, ok) != 0;
-            if (!ok) break;
-            tcgen05_fence_after();
-            // The warp's 32 rows x 32 columns leave through shared memory (128-byte swizzle) as one TMA tile store, or
-            // as one TMA reduction (global += tile) when the result is accumulated: whole 128-byte lines, no read of C by
-            // the SM, and rows / columns past M / N are clipped by the copy.
-            uint8_t* stg = c_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
-            const int row0 = (int)(item / n_tiles) * BM + quarter * 32;
+        // The warp's 32 rows x 32 columns leave through shared memory (128-byte swizzle) as one TMA tile store, or
+        // as one TMA reduction (global += tile) when the result is accumulated: whole 128-byte lines, no read of C by
+        // the SM, and rows / columns past M / N are clipped by the copy.
+        uint8_t* stg = c_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
+        auto store_tile = [&](const GemmTile& g, bool zero, uint32_t tacc) {
+            const int row0 = g.m * TILE_ROWS + (int)ps.rank * BM + quarter * 32;
 #pragma unroll 1
             for (int piece = col_half * EPI_PIECES; piece < (col_half + 1) * EPI_PIECES; ++piece) {
-                const int pc0 = col0 + piece * 32;
+                const int pc0 = g.n * BN + piece * 32;
                 if (pc0 >= p.N) break;
                 float v[32];
-                tcgen05_ld_32x32(tmem_base + lane_addr + acc * BN + piece * 32, v);
+                if (zero) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = 0.f;
+                } else {
+                    tcgen05_ld_32x32(tacc + piece * 32, v);
+                }
                 if (lane == 0) bulk_wait_read_all();          // the previous tile copy has read the staging tile
                 __syncwarp();
 #pragma unroll
@@ -439,28 +514,63 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     bulk_commit_group();
                 }
             }
+        };
+        uint32_t acc = 0, acc_phase = 0;
+        bool ok = true;
+        GemmTile g;
+        for (int64_t item = unit; ok && gemm_item(item, m_tiles, n_tiles, p.group_n, g); item += units) {
+            ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
+            ok = __all_sync(0xffffffffu, ok) != 0;
+            if (!ok) break;
+            tcgen05_fence_after();
+            store_tile(g, false, ps.tmem_base + lane_addr + acc * BN);
             tcgen05_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&ps.acc_empty[acc]);
+            if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
+        if (!p.accumulate)
+            for (int64_t item = unit; gemm_item(item, zero_m_tiles, n_tiles, p.group_n, g); item += units) {
+                g.m += m_tiles;
+                store_tile(g, true, 0u);
+            }
         if (lane == 0) bulk_wait_all();       // the tile copies have completed before the block's shared memory goes
     }
-    pipe_teardown(ps, tmem_base, p.d_status);
+    pipe_teardown(ps, p.d_status);
 }
 
-// Copies the last, partly live 64-row block of the chunk's hidden rows into `tail` [64, d] and pads it with zeros,
-// so that rows past the live tokens (caller memory that may hold anything) never reach the tensor core.
-__global__ void tail_block_kernel(const uint16_t* __restrict__ hidden, int d, const int64_t* d_T, int64_t T_max,
-                                  int64_t t0, uint16_t* __restrict__ tail) {
-    const int64_t T = live_tokens(d_T, T_max);
-    if (t0 >= T) return;
-    const int64_t live = min((int64_t)TC, T - t0);
-    const int64_t r0 = live / BK * BK;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)BK * d; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / d, c = i - r * d;
-        tail[i] = (r0 + r < live) ? hidden[(t0 + r0 + r) * d + c] : (uint16_t)0;
-    }
+int group_columns(int n_tiles) {          // column tiles per group: at most 10 (48 MB of B panels for K = 9,472), evenly
+    const int groups = (n_tiles + 9) / 10;
+    return (n_tiles + groups - 1) / groups;
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pairs(arrol_ctx* ctx, void (*kernel)(KArgs...), int64_t items, cudaStream_t s, Args&&... args) {
+    const int64_t pairs = items < 1 ? 1 : (items < ctx->sm_count / 2 ? items : ctx->sm_count / 2);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.blockDim = dim3(NUM_THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+int raise_smem_limits(arrol_ctx* ctx) {
+    if (ctx->backward_smem_set) return ARROL_OK;
+    ARROL_CUDA_OK(cudaFuncSetAttribute(dz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    ARROL_CUDA_OK(cudaFuncSetAttribute(gemm_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    ARROL_CUDA_OK(cudaFuncSetAttribute(gemm_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    ctx->backward_smem_set = true;
+    return ARROL_OK;
 }
 
 struct BackwardLayout {
@@ -482,22 +592,22 @@ BackwardLayout backward_layout(int d, int V) {
 int arrol_internal_gemm_tn(arrol_ctx* ctx, const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N, int K,
                            float* C, int64_t ldc, int accumulate, cudaStream_t s) {
     if (M <= 0 || N <= 0 || K <= 0 || lda % 8 != 0 || ldb % 8 != 0) return ARROL_ERR_UNSUPPORTED;
-    ARROL_CUDA_OK(cudaFuncSetAttribute(gemm_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+    if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
     CUtensorMap map_a, map_b, map_c;
     if (make_map_f32_tile(ctx, &map_c, C, (uint64_t)M, (uint64_t)N, (uint64_t)ldc) != ARROL_OK) return ARROL_ERR_CUDA;
     bool a3 = M % 64 == 0, b3 = N % 64 == 0;
     if (a3 && make_map_mn3d(ctx, &map_a, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM / 64) != ARROL_OK) a3 = false;
-    if (b3 && make_map_mn3d(ctx, &map_b, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BN / 64) != ARROL_OK) b3 = false;
+    if (b3 && make_map_mn3d(ctx, &map_b, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BN / 2 / 64) != ARROL_OK) b3 = false;
     if (!a3 && make_map_ld(ctx, &map_a, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK) != ARROL_OK) return ARROL_ERR_CUDA;
     if (!b3 && make_map_ld(ctx, &map_b, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BK) != ARROL_OK) return ARROL_ERR_CUDA;
-    GemmParams g;
-    g.M = M; g.N = N; g.K = K; g.C = C; g.ldc = ldc; g.accumulate = accumulate; g.k_is_tokens = 0;
-    g.a3d = a3; g.b3d = b3; g.d_T = nullptr; g.T_max = 1; g.t0 = 0; g.d_status = ctx->d_status;
-    const int64_t items = (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
-    gemm_kernel<true, true><<<(unsigned)(items < ctx->sm_count ? items : ctx->sm_count), NUM_THREADS, SMEM_BYTES, s>>>(
-        map_a, map_b, map_b, map_c, g);
+    GemmParams g = {};
+    g.M = M; g.N = N; g.K = K; g.accumulate = accumulate;
+    g.a3d = a3; g.b3d = b3; g.T_max = 1; g.d_status = ctx->d_status;
+    const int n_tiles = (N + BN - 1) / BN;
+    g.group_n = group_columns(n_tiles);
+    const int64_t items = (int64_t)((M + TILE_ROWS - 1) / TILE_ROWS) * n_tiles;
+    ARROL_CUDA_OK(launch_pairs(ctx, gemm_kernel<true, true>, items, s, map_a, map_b, map_b, map_c, g));
     ctx->launches += 1;
-    ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;
 }
 
@@ -517,8 +627,10 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     ArrolDeviceGuard guard(ctx->device);
     if (!guard.ok) return ARROL_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    ARROL_CUDA_OK(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)V * d, s));
-    if (T_max == 0) return ARROL_OK;
+    if (T_max == 0) {
+        ARROL_CUDA_OK(cudaMemsetAsync(dW, 0, sizeof(float) * (size_t)V * d, s));
+        return ARROL_OK;
+    }
     if (!hidden || !W_vocab || !targets || !grad_logp || !lse || !dH) return ARROL_ERR_INVALID_ARG;
     if (!arrol_aligned(hidden, 16) || !arrol_aligned(W_vocab, 16) || !arrol_aligned(dH, 16) || !arrol_aligned(dW, 16))
         return ARROL_ERR_INVALID_ARG;
@@ -526,24 +638,21 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     if (!workspace || workspace_bytes < L.total || !arrol_aligned(workspace, 256)) return ARROL_ERR_WORKSPACE;
     __nv_bfloat16* dZ = reinterpret_cast<__nv_bfloat16*>(static_cast<uint8_t*>(workspace) + L.dz);
     uint16_t* Htail = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + L.tail);
+    if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
 
-    ARROL_CUDA_OK(cudaFuncSetAttribute(dz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(gemm_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    ARROL_CUDA_OK(cudaFuncSetAttribute(gemm_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-
-    // tensor maps: K-major operands are fetched as [MN rows x 64 K columns] boxes; MN-major ones (the same row-major
+    // tensor maps: K-major operands are fetched as [128 MN rows x 64 K columns] boxes; MN-major ones (the same row-major
     // storage read the other way) as one three-dimensional box per stage when the MN extent is a whole number of
     // 64-element blocks, else as one [64 K rows x 64 MN columns] box per block
     CUtensorMap map_h_k, map_w_k, map_dz_k, map_dz_st, map_w_mn, map_dz_mn, map_h_mn, map_h_tail;
     if (make_map(ctx, &map_h_k, hidden, (uint64_t)T_max, (uint64_t)d, BM) != ARROL_OK) return ARROL_ERR_CUDA;
-    if (make_map(ctx, &map_w_k, W_vocab, (uint64_t)V, (uint64_t)d, BN) != ARROL_OK) return ARROL_ERR_CUDA;
+    if (make_map(ctx, &map_w_k, W_vocab, (uint64_t)V, (uint64_t)d, BN / 2) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map_ld(ctx, &map_dz_k, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BM) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map_ld(ctx, &map_dz_st, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, 32) != ARROL_OK) return ARROL_ERR_CUDA;   // store tiles
     CUtensorMap map_dw;
     if (make_map_f32_tile(ctx, &map_dw, dW, (uint64_t)V, (uint64_t)d, (uint64_t)d) != ARROL_OK) return ARROL_ERR_CUDA;
     bool d3 = d % 64 == 0, v3 = V % 64 == 0;
-    if (d3 && (make_map_mn3d(ctx, &map_w_mn, W_vocab, (uint64_t)V, (uint64_t)d, (uint64_t)d, BN / 64) != ARROL_OK ||
-               make_map_mn3d(ctx, &map_h_tail, Htail, (uint64_t)BK, (uint64_t)d, (uint64_t)d, BN / 64) != ARROL_OK))
+    if (d3 && (make_map_mn3d(ctx, &map_w_mn, W_vocab, (uint64_t)V, (uint64_t)d, (uint64_t)d, BN / 2 / 64) != ARROL_OK ||
+               make_map_mn3d(ctx, &map_h_tail, Htail, (uint64_t)BK, (uint64_t)d, (uint64_t)d, BN / 2 / 64) != ARROL_OK))
         d3 = false;
     if (v3 && make_map_mn3d(ctx, &map_dz_mn, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BM / 64) != ARROL_OK) v3 = false;
     if (!d3) {
@@ -552,47 +661,42 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     }
     if (!v3 && make_map_ld(ctx, &map_dz_mn, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BK) != ARROL_OK) return ARROL_ERR_CUDA;
 
-    const int total_chunks = (V + BN - 1) / BN;
-    int splits = 1;
-    while ((TC / BM) * splits < ctx->sm_count && splits * 2 <= total_chunks) splits *= 2;
-    const int chunks_per_split = (total_chunks + splits - 1) / splits;
-    splits = (total_chunks + chunks_per_split - 1) / chunks_per_split;
+    const int total_chunks = (V + BN - 1) / BN, n_tiles = (d + BN - 1) / BN;
+    int m_groups = 1;
+    while ((double)TC / m_groups * d * 2 > 50.0 * 1024 * 1024) ++m_groups;
 
     for (int64_t t0 = 0; t0 < T_max; t0 += TC) {
         const int64_t rows = (T_max - t0) < TC ? (T_max - t0) : (int64_t)TC;
+        const int m_tiles = (int)((rows + TILE_ROWS - 1) / TILE_ROWS);
         // the chunk of hidden as an MN-major B operand: [rows (K), d (N)]; rows past T_max read as zero
         const void* h_chunk = static_cast<const uint8_t*>(hidden) + (size_t)t0 * d * 2;
-        if ((d3 ? make_map_mn3d(ctx, &map_h_mn, h_chunk, (uint64_t)rows, (uint64_t)d, (uint64_t)d, BN / 64)
+        if ((d3 ? make_map_mn3d(ctx, &map_h_mn, h_chunk, (uint64_t)rows, (uint64_t)d, (uint64_t)d, BN / 2 / 64)
                 : make_map(ctx, &map_h_mn, h_chunk, (uint64_t)rows, (uint64_t)d, BK)) != ARROL_OK)
             return ARROL_ERR_CUDA;
 
         DzParams zp;
         zp.targets = targets; zp.grad_logp = grad_logp; zp.lse = lse; zp.d_T = d_T; zp.T_max = T_max; zp.t0 = t0;
-        zp.d = d; zp.V = V; zp.ldz = L.ldz; zp.splits = splits; zp.chunks_per_split = chunks_per_split;
+        zp.d = d; zp.V = V; zp.group_tiles = (TC / TILE_ROWS + m_groups - 1) / m_groups;
         zp.scale2 = inv_temperature * 1.44269504088896340736f; zp.inv_temp = inv_temperature;
-        zp.dZ = dZ; zp.d_status = ctx->d_status;
-        int64_t grid = (int64_t)(TC / BM) * splits;
-        if (grid > ctx->sm_count) grid = ctx->sm_count;
-        dz_kernel<<<(unsigned)grid, NUM_THREADS, SMEM_BYTES, s>>>(map_h_k, map_w_k, map_dz_st, zp);
+        zp.hidden = static_cast<const uint16_t*>(hidden); zp.tail = Htail; zp.d_status = ctx->d_status;
+        ARROL_CUDA_OK(launch_pairs(ctx, dz_kernel, (int64_t)m_tiles * total_chunks, s, map_h_k, map_w_k, map_dz_st, zp));
 
-        GemmParams gh;    // dH[chunk] = dZ . W
-        gh.M = (int)rows; gh.N = d; gh.K = V; gh.C = dH + t0 * d; gh.ldc = d; gh.accumulate = 0; gh.k_is_tokens = 0; gh.a3d = 0; gh.b3d = d3;
+        GemmParams gh = {};    // dH[chunk] = dZ . W
+        gh.M = (int)rows; gh.N = d; gh.K = V; gh.group_n = group_columns(n_tiles);
+        gh.m_is_tokens = 1; gh.b3d = d3;
         gh.d_T = d_T; gh.T_max = T_max; gh.t0 = t0; gh.d_status = ctx->d_status;
-        const int64_t gh_items = (int64_t)((rows + BM - 1) / BM) * ((d + BN - 1) / BN);
         CUtensorMap map_dh;      // this chunk's rows of dH: rows past the chunk are clipped by the tile stores
         if (make_map_f32_tile(ctx, &map_dh, dH + t0 * d, (uint64_t)rows, (uint64_t)d, (uint64_t)d) != ARROL_OK)
             return ARROL_ERR_CUDA;
-        gemm_kernel<false, true><<<(unsigned)(gh_items < ctx->sm_count ? gh_items : ctx->sm_count), NUM_THREADS,
-                                   SMEM_BYTES, s>>>(map_dz_k, map_w_mn, map_w_mn, map_dh, gh);
-        tail_block_kernel<<<64, 256, 0, s>>>(static_cast<const uint16_t*>(hidden), d, d_T, T_max, t0, Htail);
-        GemmParams gw;    // dW += dZ^T . H[chunk]
-        gw.M = V; gw.N = d; gw.K = (int)rows; gw.C = dW; gw.ldc = d; gw.accumulate = 1; gw.k_is_tokens = 1; gw.a3d = v3; gw.b3d = d3;
+        ARROL_CUDA_OK(launch_pairs(ctx, gemm_kernel<false, true>, (int64_t)m_tiles * n_tiles, s, map_dz_k, map_w_mn, map_w_mn,
+                                   map_dh, gh));
+        GemmParams gw = {};    // dW (+)= dZ^T . H[chunk]; the first chunk writes dW, zeros where no token lives
+        gw.M = V; gw.N = d; gw.K = (int)rows; gw.group_n = group_columns(n_tiles);
+        gw.accumulate = t0 > 0; gw.k_is_tokens = 1; gw.zero_if_dead = t0 == 0; gw.a3d = v3; gw.b3d = d3;
         gw.d_T = d_T; gw.T_max = T_max; gw.t0 = t0; gw.d_status = ctx->d_status;
-        const int64_t gw_items = (int64_t)((V + BM - 1) / BM) * ((d + BN - 1) / BN);
-        gemm_kernel<true, true><<<(unsigned)(gw_items < ctx->sm_count ? gw_items : ctx->sm_count), NUM_THREADS,
-                                  SMEM_BYTES, s>>>(map_dz_mn, map_h_mn, map_h_tail, map_dw, gw);
-        ctx->launches += 4;
-        ARROL_CUDA_OK(cudaGetLastError());
+        ARROL_CUDA_OK(launch_pairs(ctx, gemm_kernel<true, true>, (int64_t)((V + TILE_ROWS - 1) / TILE_ROWS) * n_tiles, s,
+                                   map_dz_mn, map_h_mn, map_h_tail, map_dw, gw));
+        ctx->launches += 3;
     }
     return ARROL_OK;
 }

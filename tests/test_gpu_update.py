@@ -102,6 +102,28 @@ def test_lm_head_backward_many_chunks_temperature_and_device_T(ctx):
     _backward_case(ctx, 9700, 64, 512, seed=5, T_live=9500)    # the partly live block is in the second chunk
 
 
+# edges of the pairs' 256 x 256 tiles: a full tile and one row more, one vocabulary column in the last chunk, a last column tile
+# of 8 (half a tile for the MMA) and of 136, a chunk of 37 tiles and one row more, dead rows in whole tiles of their own
+@pytest.mark.parametrize("T,d,V,T_live", [(256, 64, 256, None), (257, 264, 2305, None), (129, 392, 640, None),
+                                          (9473, 72, 300, None), (1100, 136, 520, 257), (9472, 64, 257, 9471)])
+def test_lm_head_backward_at_the_edges_of_a_pairs_tile(ctx, T, d, V, T_live):
+    dH, n = _backward_case(ctx, T, d, V, seed=T + d, T_live=T_live)
+    assert np.all(dH[n:] == 0.0)
+
+
+def test_lm_head_backward_without_a_live_token(ctx):
+    T, d, V = 300, 136, 700
+    Z = torch.full((T, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    W = torch.zeros((V, d), device="cuda", dtype=torch.bfloat16)
+    f = torch.zeros(T, device="cuda")
+    dH, dW = torch.full((T, d), 9.0, device="cuda"), torch.full((V, d), 9.0, device="cuda")
+    ws = torch.empty(U.arrol_lm_head_backward_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+    U.arrol_lm_head_backward(ctx, Z, W, torch.zeros(T, dtype=torch.int32, device="cuda"), f, f, T, d, V, dH, dW, ws,
+                             d_T=torch.zeros(1, dtype=torch.int64, device="cuda"))
+    torch.cuda.synchronize()
+    assert torch.all(dW == 0.0) and torch.all((dH == 0.0) | (dH == 9.0))
+
+
 def test_update_argument_errors(ctx):
     z = torch.zeros(8, device="cuda")
     with pytest.raises(B.ArrolError) as e:
