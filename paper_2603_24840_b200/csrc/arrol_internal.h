@@ -19,6 +19,7 @@ struct arrol_ctx {
     uint32_t* d_tile_counters; // MLP head on the tensor cores: finished blocks per row tile, zero between calls
     unsigned long long* d_chain;   // fused prune step: finished blocks, index-check flag, per-block totals; zero between calls
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
+    int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
     bool backward_smem_set;    // likewise for the lm_head backward
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
@@ -43,7 +44,7 @@ constexpr int ARROL_MLP_TH = 64;             // hidden units per MLP thread-bloc
 constexpr int ARROL_MAX_H = 4096;
 constexpr size_t ARROL_SCRATCH_FLOATS = (size_t)ARROL_MAX_MLP_N * (ARROL_MAX_H / ARROL_MLP_TH);
 constexpr size_t ARROL_PACK_BYTES = (size_t)64 << 20;
-constexpr int ARROL_TILE_COUNTERS = 1024;   // row tiles of the MLP head
+constexpr int ARROL_TILE_COUNTERS = 1024;   // [0, 1020) row tiles of the MLP head, then 16 bytes for the head training step's contractions
 constexpr int ARROL_SCORE_ROW_TILES = 1020;
 constexpr int ARROL_CHAIN_BLOCKS = 510;      // blocks of the fused prune step's chained scan (2 + 2 * 510 words = 8 KB)
 

@@ -51,6 +51,7 @@ struct PipeSmem {
     uint64_t *full, *empty, *acc_full, *acc_empty, *drain;
     uint32_t* tmem_slot;
     volatile uint32_t* abort_flag;
+    volatile uint32_t* lock_seen;            // copy of the lock-step counter, 16 bytes
     uint32_t rank;                           // of this block in its pair (0 leads)
     uint32_t tmem_base;
     uint32_t lead_full, lead_acc_empty;      // shared::cluster addresses in the leading block
@@ -71,6 +72,7 @@ __device__ __forceinline__ PipeSmem pipe_setup(uint8_t* smem_raw, const CUtensor
     ps.drain = ps.acc_empty + 2;
     ps.tmem_slot = reinterpret_cast<uint32_t*>(ps.drain + 1);
     ps.abort_flag = ps.tmem_slot + 1;
+    ps.lock_seen = reinterpret_cast<uint32_t*>(smem + (size_t)STAGES * STAGE_BYTES + 512);
     ps.rank = cluster_cta_rank();
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&ps.full[s], 1); mbar_init(&ps.empty[s], 1); }
@@ -108,10 +110,55 @@ __device__ __forceinline__ void pipe_teardown(const PipeSmem& ps, uint32_t* d_st
     }
 }
 
+// Pairs in step.  The pairs of a launch share operand panels through L2, but only while they read them at about the same
+// time, and nothing in a persistent kernel keeps them together: measured at d = 4,096, the dH contraction of a chunk read 33 GB
+// from HBM where 11 would do and ran at 1.09 GHz under the power cap, the dz kernel beside it, with its little traffic, at 1.27.
+// So about every EPOCH K steps the leading producer of a pair reports on a counter in global memory and waits until all
+// pairs have reported two epochs ago; none gets further ahead of the others than that.  The counter is fetched an epoch
+// ahead by an asynchronous copy into shared memory, so a pair that is not ahead does not wait for memory either.
+// (A plain load of the counter by one thread at every epoch cost the tensor pipe 6-14 % of the cycles.)  One chunk alone, without
+// and with it: d = 2,048, V = 128,256 HBM reads of dH 12.0 -> 6.8 GB, of dW 8.9 -> 6.1, the three kernels 10.4 -> 10.0 ms; d = 4,096,
+// V = 151,936 34 -> 17 and 25 -> 15.5 GB, 25.7 -> 24.0 ms.  Over seconds, where the power cap evens it out, an update of a
+// DAPO-shaped micro-batch takes 70.3 -> 69.4 ms.  Epochs of 8 steps reach the least traffic (4.9 and 4.7 GB, 11.7 and 11.2) but
+// gain nothing more over seconds.  All pairs must be resident: no more are launched than the occupancy query allows, and the wait is bounded
+// like every other.
+constexpr int EPOCH = 16;
+constexpr size_t LOCK_BYTES = 16;      // per counter
+struct Lockstep {
+    unsigned int* counter;      // zero before the launch, 16-byte aligned
+    uint32_t units, epochs;     // epochs of the pair with the most work
+    int items_per_epoch;        // > 1 when a tile has few K steps
+};
+__device__ __forceinline__ Lockstep lockstep_for(unsigned int* counter, int64_t units, int64_t items, int k_steps) {
+    Lockstep l;
+    l.counter = counter;
+    l.units = (uint32_t)units;
+    l.items_per_epoch = k_steps >= EPOCH ? 1 : EPOCH / max(k_steps, 1);
+    const int64_t most = (items + units - 1) / units;
+    l.epochs = (uint32_t)(k_steps >= EPOCH ? most * ((k_steps + EPOCH - 1) / EPOCH)
+                                           : (most + l.items_per_epoch - 1) / l.items_per_epoch);
+    return l;
+}
+// One thread, at the beginning of its pair's epoch `epoch`.  False: the wait ran out.
+__device__ __forceinline__ bool begin_epoch(const Lockstep& lock, volatile uint32_t* seen, uint32_t epoch,
+                                            volatile uint32_t* abort_flag) {
+    atomicAdd(lock.counter, 1u);
+    cp_async_wait_all();
+    const uint32_t target = epoch < 2 ? 0u : (epoch - 1) * lock.units;       // everybody has begun epoch - 2
+    if (target != 0u && *seen < target) {
+        for (uint32_t spin = 0; ld_relaxed_u32(lock.counter) < target; ++spin) {
+            __nanosleep(32);
+            if (spin >= SPIN_LIMIT || ((spin & 1023u) == 1023u && *abort_flag)) { *abort_flag = 1u; return false; }
+        }
+    }
+    cp_async_16(seen, lock.counter);                                          // looked at when the next epoch begins
+    return true;
+}
+
 // One accumulator tile's operands: origin of the tile's rows (A) and columns (B), and the columns that the MMA computes.
 struct TileAt { int a0, b0, n; };
 
-// Producer role (one thread of each block).  For every accumulator tile `coords(it, tile)` gives the operands' MN origins
+// Producer role (one warp of each block; the warp walks the loops and waits, one elected lane issues).  For every accumulator tile `coords(it, tile)` gives the operands' MN origins
 // (false when the list is exhausted); this block loads rows a0 + 128 rank ... of A and b0 + (n / 2) rank ... of B.  Per K step
 //   K-major operand:  one box  [128 MN rows x 64 K columns]      at (x = k, y = mn0)
 //   MN-major operand: 2 blocks [64 K rows x 64 MN columns], BK*128 bytes apart: one three-dimensional box
@@ -120,50 +167,71 @@ struct TileAt { int a0, b0, n; };
 // Both blocks' bytes are counted on the leading block's barrier.
 template <bool A_MN, bool B_MN, typename Coords>
 __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensorMap* ma, const CUtensorMap* mb,
-                                              int k_steps, Coords coords, bool a3d = false, bool b3d = false,
+                                              int k_steps, const Lockstep& lock, Coords coords, bool a3d = false, bool b3d = false,
                                               const CUtensorMap* mb_tail = nullptr, int tail_ks = -1) {
-    uint32_t stage = 0, phase = 0, issued = 0;
+    const uint32_t a0 = smem_u32(ps.stage_a), b0 = smem_u32(ps.stage_b);
+    uint32_t stage = 0, phase = 0, issued = 0, epoch = 0;
     bool ok = true;
     TileAt tile;
+    int to_epoch = 0;                     // items until the next epoch
     for (int64_t it = 0; ok && coords(it, tile); ++it) {
         const int ay = tile.a0 + (int)ps.rank * BM, by = tile.b0 + (int)ps.rank * (tile.n / 2);
-        for (int ks = 0; ks < k_steps; ++ks) {
-            if (!mbar_wait(&ps.empty[stage], phase ^ 1u, ps.abort_flag)) { ok = false; break; }
-            const uint32_t bar = ps.lead_full + stage * (uint32_t)sizeof(uint64_t);
-            if (ps.rank == 0) mbar_expect_tx(&ps.full[stage], 2 * STAGE_BYTES);
-            uint8_t* sa = ps.stage_a + (size_t)stage * A_STAGE_BYTES;
-            uint8_t* sb = ps.stage_b + (size_t)stage * B_STAGE_BYTES;
-            if constexpr (A_MN) {
-                if (a3d) {
-                    tma_load_3d_pair(sa, ma, 0, ks * BK, ay >> 6, bar);
-                } else {
-#pragma unroll
-                    for (int b = 0; b < BM / 64; ++b)
-                        tma_load_2d_pair(sa + b * MN_BLOCK_BYTES, ma, ay + 64 * b, ks * BK, bar);
+        for (int ks0 = 0; ks0 < k_steps && ok; ks0 += EPOCH) {
+            if (ks0 > 0 || to_epoch == 0) {
+                if (ps.rank == 0) {
+                    if (elect_one()) ok = begin_epoch(lock, ps.lock_seen, epoch, ps.abort_flag);
+                    ok = __all_sync(0xffffffffu, ok) != 0;
+                    if (!ok) break;
                 }
-            } else {
-                tma_load_2d_pair(sa, ma, ks * BK, ay, bar);
+                ++epoch;
+                if (ks0 == 0) to_epoch = lock.items_per_epoch;
             }
-            if constexpr (B_MN) {
-                // the K step that holds the last, partly live block of rows is read from its zero-padded copy
-                const bool tail = ks == tail_ks;
-                const CUtensorMap* m = tail ? mb_tail : mb;
-                const int ky = tail ? 0 : ks * BK;
-                if (b3d) {
-                    tma_load_3d_pair(sb, m, 0, ky, by >> 6, bar);
-                } else {
+            const int ks1 = min(ks0 + EPOCH, k_steps);
+            for (int ks = ks0; ks < ks1; ++ks) {
+                if (!mbar_wait_warp(&ps.empty[stage], phase ^ 1u, ps.abort_flag)) { ok = false; break; }
+                if (elect_one()) {
+                    const uint32_t bar = ps.lead_full + stage * (uint32_t)sizeof(uint64_t);
+                    if (ps.rank == 0) mbar_expect_tx(&ps.full[stage], 2 * STAGE_BYTES);
+                    const uint32_t sa = a0 + stage * A_STAGE_BYTES, sb = b0 + stage * B_STAGE_BYTES;
+                    if constexpr (A_MN) {
+                        if (a3d) {
+                            tma_load_3d_pair(sa, ma, 0, ks * BK, ay >> 6, bar);
+                        } else {
 #pragma unroll
-                    for (int b = 0; b < BN / 2 / 64; ++b)
-                        tma_load_2d_pair(sb + b * MN_BLOCK_BYTES, m, by + 64 * b, ky, bar);
+                            for (int b = 0; b < BM / 64; ++b)
+                                tma_load_2d_pair(sa + b * MN_BLOCK_BYTES, ma, ay + 64 * b, ks * BK, bar);
+                        }
+                    } else {
+                        tma_load_2d_pair(sa, ma, ks * BK, ay, bar);
+                    }
+                    if constexpr (B_MN) {
+                        // the K step that holds the last, partly live block of rows is read from its zero-padded copy
+                        const bool tail = ks == tail_ks;
+                        const CUtensorMap* m = tail ? mb_tail : mb;
+                        const int ky = tail ? 0 : ks * BK;
+                        if (b3d) {
+                            tma_load_3d_pair(sb, m, 0, ky, by >> 6, bar);
+                        } else {
+#pragma unroll
+                            for (int b = 0; b < BN / 2 / 64; ++b)
+                                tma_load_2d_pair(sb + b * MN_BLOCK_BYTES, m, by + 64 * b, ky, bar);
+                        }
+                    } else {
+                        tma_load_2d_pair(sb, mb, ks * BK, by, bar);
+                    }
                 }
-            } else {
-                tma_load_2d_pair(sb, mb, ks * BK, by, bar);
+                __syncwarp();
+                ++issued;
+                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
-            ++issued;
-            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
+        --to_epoch;
     }
-    if (!ok && ps.rank == 0) {
+    if (ps.rank == 0 && elect_one()) {
+        cp_async_wait_all();
+        if (epoch < lock.epochs) atomicAdd(lock.counter, lock.epochs - epoch);   // done: nobody waits for this pair
+    }
+    if (!ok && ps.rank == 0 && elect_one()) {
         // gave up: let the copies already issued land before shared memory goes away (bounded); the peer's copies are
         // counted here too, and the cluster barrier at the end keeps its shared memory alive until then
         const uint32_t pending = issued < (uint32_t)STAGES ? issued : (uint32_t)STAGES;
@@ -174,6 +242,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
                 if (mbar_try_wait(&ps.full[s], ph)) break;
         }
     }
+    __syncwarp();
 }
 
 // MMA role (one warp of the leading block): the accumulator tiles that `columns(it)` lists (their MMA columns, 0 = no
@@ -246,6 +315,7 @@ struct DzParams {
     int group_tiles;
     float scale2, inv_temp;
     const uint16_t* hidden;
+    unsigned int* lock_counter;
     uint16_t* tail;           // [64, d]: the last, partly live 64-row block of the chunk's hidden rows, zero-padded
     uint32_t* d_status;
 };
@@ -285,16 +355,15 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
     const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
 
     if (warp == 0) {
-        if (lane == 0) {
-            producer_loop<false, false>(ps, &map_h, &map_w, k_steps, [&](int64_t it, TileAt& t) {
-                int m, c;
-                if (!dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c)) return false;
-                t.a0 = (int)p.t0 + m * TILE_ROWS;
-                t.b0 = c * BN;
-                t.n = chunk_columns(p.V, c);
-                return true;
-            });
-        }
+        const Lockstep lock = lockstep_for(p.lock_counter, units, (int64_t)m_tiles * total_chunks, k_steps);
+        producer_loop<false, false>(ps, &map_h, &map_w, k_steps, lock, [&](int64_t it, TileAt& t) {
+            int m, c;
+            if (!dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c)) return false;
+            t.a0 = (int)p.t0 + m * TILE_ROWS;
+            t.b0 = c * BN;
+            t.n = chunk_columns(p.V, c);
+            return true;
+        });
     } else if (warp == 1) {
         if (ps.rank == 0)
             mma_loop<false, false>(ps, k_steps, k_last, [&](int64_t it) {
@@ -421,6 +490,7 @@ struct GemmParams {
     int a3d, b3d;             // the MN-major operand's maps are three-dimensional (one copy per stage)
     const int64_t* d_T;
     int64_t T_max, t0;
+    unsigned int* lock_counter;
     uint32_t* d_status;
 };
 
@@ -462,17 +532,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     auto columns = [&](int n) { const int left = p.N - n * BN; return left > BN / 2 ? BN : BN / 2; };
 
     if (warp == 0) {
-        if (lane == 0) {
-            const int tail_ks = (p.k_is_tokens && (K % BK) != 0) ? k_steps - 1 : -1;
-            producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, k_steps, [&](int64_t it, TileAt& t) {
-                GemmTile g;
-                if (!gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g)) return false;
-                t.a0 = g.m * TILE_ROWS;
-                t.b0 = g.n * BN;
-                t.n = columns(g.n);
-                return true;
-            }, p.a3d != 0, p.b3d != 0, &map_b_tail, tail_ks);
-        }
+        const int tail_ks = (p.k_is_tokens && (K % BK) != 0) ? k_steps - 1 : -1;
+        const Lockstep lock = lockstep_for(p.lock_counter, units, (int64_t)m_tiles * n_tiles, k_steps);
+        producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, k_steps, lock, [&](int64_t it, TileAt& t) {
+            GemmTile g;
+            if (!gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g)) return false;
+            t.a0 = g.m * TILE_ROWS;
+            t.b0 = g.n * BN;
+            t.n = columns(g.n);
+            return true;
+        }, p.a3d != 0, p.b3d != 0, &map_b_tail, tail_ks);
     } else if (warp == 1) {
         if (ps.rank == 0)
             mma_loop<A_MN, B_MN>(ps, k_steps, k_last, [&](int64_t it) {
@@ -545,10 +614,9 @@ int group_columns(int n_tiles) {          // column tiles per group: at most 10 
 }
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pairs(arrol_ctx* ctx, void (*kernel)(KArgs...), int64_t items, cudaStream_t s, Args&&... args) {
-    const int64_t pairs = items < 1 ? 1 : (items < ctx->sm_count / 2 ? items : ctx->sm_count / 2);
+cudaError_t launch_pairs(arrol_ctx* ctx, int which, void (*kernel)(KArgs...), int64_t items, cudaStream_t s, Args&&... args) {
+    int64_t pairs = items < 1 ? 1 : (items < ctx->sm_count / 2 ? items : ctx->sm_count / 2);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(2 * pairs));
     cfg.blockDim = dim3(NUM_THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = s;
@@ -560,6 +628,19 @@ cudaError_t launch_pairs(arrol_ctx* ctx, void (*kernel)(KArgs...), int64_t items
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
+    // the pairs wait for one another: never more of them than are resident at once (asked once per context and kernel)
+    if (ctx->backward_max_pairs[which] == 0) {
+        int fit = 0;
+        cudaLaunchConfig_t ask = cfg;
+        ask.gridDim = dim3((unsigned)(ctx->sm_count / 2 * 2));
+        ask.numAttrs = 1;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, kernel, &ask);
+        if (e != cudaSuccess) return e;
+        if (fit < 1) return cudaErrorInvalidConfiguration;
+        ctx->backward_max_pairs[which] = fit;
+    }
+    if (pairs > ctx->backward_max_pairs[which]) pairs = ctx->backward_max_pairs[which];
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
@@ -575,15 +656,16 @@ int raise_smem_limits(arrol_ctx* ctx) {
 
 struct BackwardLayout {
     int64_t ldz;       // V rounded up to 8
-    size_t dz, tail, total;
+    size_t dz, tail, counters, total;
 };
 
-BackwardLayout backward_layout(int d, int V) {
+BackwardLayout backward_layout(int64_t T_max, int d, int V) {
     BackwardLayout L;
     L.ldz = ((int64_t)V + 7) & ~(int64_t)7;
     L.dz = 0;
     L.tail = (((size_t)TC * L.ldz * 2) + 255) & ~(size_t)255;
-    L.total = L.tail + (((size_t)BK * d * 2 + 255) & ~(size_t)255);
+    L.counters = L.tail + (((size_t)BK * d * 2 + 255) & ~(size_t)255);
+    L.total = L.counters + (((size_t)((T_max + TC - 1) / TC) * 3 * LOCK_BYTES + 255) & ~(size_t)255);   // one per kernel
     return L;
 }
 
@@ -602,18 +684,21 @@ int arrol_internal_gemm_tn(arrol_ctx* ctx, const void* A, int64_t lda, const voi
     if (!b3 && make_map_ld(ctx, &map_b, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BK) != ARROL_OK) return ARROL_ERR_CUDA;
     GemmParams g = {};
     g.M = M; g.N = N; g.K = K; g.accumulate = accumulate;
+    // the last words of ctx->d_tile_counters: zeroed before every launch (calls on a context's buffers are ordered by the caller)
+    g.lock_counter = ctx->d_tile_counters + ARROL_SCORE_ROW_TILES;
+    ARROL_CUDA_OK(cudaMemsetAsync(g.lock_counter, 0, sizeof(unsigned int), s));
     g.a3d = a3; g.b3d = b3; g.T_max = 1; g.d_status = ctx->d_status;
     const int n_tiles = (N + BN - 1) / BN;
     g.group_n = group_columns(n_tiles);
     const int64_t items = (int64_t)((M + TILE_ROWS - 1) / TILE_ROWS) * n_tiles;
-    ARROL_CUDA_OK(launch_pairs(ctx, gemm_kernel<true, true>, items, s, map_a, map_b, map_b, map_c, g));
+    ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, items, s, map_a, map_b, map_b, map_c, g));
     ctx->launches += 1;
     return ARROL_OK;
 }
 
 extern "C" size_t arrol_lm_head_backward_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    return backward_layout(d, V).total;
+    return backward_layout(T_max, d, V).total;
 }
 
 extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const void* W_vocab, const int32_t* targets,
@@ -634,10 +719,12 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     if (!hidden || !W_vocab || !targets || !grad_logp || !lse || !dH) return ARROL_ERR_INVALID_ARG;
     if (!arrol_aligned(hidden, 16) || !arrol_aligned(W_vocab, 16) || !arrol_aligned(dH, 16) || !arrol_aligned(dW, 16))
         return ARROL_ERR_INVALID_ARG;
-    const BackwardLayout L = backward_layout(d, V);
+    const BackwardLayout L = backward_layout(T_max, d, V);
     if (!workspace || workspace_bytes < L.total || !arrol_aligned(workspace, 256)) return ARROL_ERR_WORKSPACE;
     __nv_bfloat16* dZ = reinterpret_cast<__nv_bfloat16*>(static_cast<uint8_t*>(workspace) + L.dz);
     uint16_t* Htail = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + L.tail);
+    unsigned int* counters = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + L.counters);
+    ARROL_CUDA_OK(cudaMemsetAsync(counters, 0, L.total - L.counters, s));
     if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
 
     // tensor maps: K-major operands are fetched as [128 MN rows x 64 K columns] boxes; MN-major ones (the same row-major
@@ -678,23 +765,25 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         zp.targets = targets; zp.grad_logp = grad_logp; zp.lse = lse; zp.d_T = d_T; zp.T_max = T_max; zp.t0 = t0;
         zp.d = d; zp.V = V; zp.group_tiles = (TC / TILE_ROWS + m_groups - 1) / m_groups;
         zp.scale2 = inv_temperature * 1.44269504088896340736f; zp.inv_temp = inv_temperature;
+        zp.lock_counter = counters; counters += LOCK_BYTES / sizeof(unsigned int);
         zp.hidden = static_cast<const uint16_t*>(hidden); zp.tail = Htail; zp.d_status = ctx->d_status;
-        ARROL_CUDA_OK(launch_pairs(ctx, dz_kernel, (int64_t)m_tiles * total_chunks, s, map_h_k, map_w_k, map_dz_st, zp));
+        ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, (int64_t)m_tiles * total_chunks, s, map_h_k, map_w_k, map_dz_st, zp));
 
         GemmParams gh = {};    // dH[chunk] = dZ . W
         gh.M = (int)rows; gh.N = d; gh.K = V; gh.group_n = group_columns(n_tiles);
-        gh.m_is_tokens = 1; gh.b3d = d3;
+        gh.m_is_tokens = 1; gh.b3d = d3; gh.lock_counter = counters; counters += LOCK_BYTES / sizeof(unsigned int);
         gh.d_T = d_T; gh.T_max = T_max; gh.t0 = t0; gh.d_status = ctx->d_status;
         CUtensorMap map_dh;      // this chunk's rows of dH: rows past the chunk are clipped by the tile stores
         if (make_map_f32_tile(ctx, &map_dh, dH + t0 * d, (uint64_t)rows, (uint64_t)d, (uint64_t)d) != ARROL_OK)
             return ARROL_ERR_CUDA;
-        ARROL_CUDA_OK(launch_pairs(ctx, gemm_kernel<false, true>, (int64_t)m_tiles * n_tiles, s, map_dz_k, map_w_mn, map_w_mn,
+        ARROL_CUDA_OK(launch_pairs(ctx, 1, gemm_kernel<false, true>, (int64_t)m_tiles * n_tiles, s, map_dz_k, map_w_mn, map_w_mn,
                                    map_dh, gh));
         GemmParams gw = {};    // dW (+)= dZ^T . H[chunk]; the first chunk writes dW, zeros where no token lives
         gw.M = V; gw.N = d; gw.K = (int)rows; gw.group_n = group_columns(n_tiles);
         gw.accumulate = t0 > 0; gw.k_is_tokens = 1; gw.zero_if_dead = t0 == 0; gw.a3d = v3; gw.b3d = d3;
+        gw.lock_counter = counters; counters += LOCK_BYTES / sizeof(unsigned int);
         gw.d_T = d_T; gw.T_max = T_max; gw.t0 = t0; gw.d_status = ctx->d_status;
-        ARROL_CUDA_OK(launch_pairs(ctx, gemm_kernel<true, true>, (int64_t)((V + TILE_ROWS - 1) / TILE_ROWS) * n_tiles, s,
+        ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, (int64_t)((V + TILE_ROWS - 1) / TILE_ROWS) * n_tiles, s,
                                    map_dz_mn, map_h_mn, map_h_tail, map_dw, gw));
         ctx->launches += 3;
     }

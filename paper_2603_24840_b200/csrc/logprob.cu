@@ -345,8 +345,8 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                             // both blocks' bytes are counted on the leading block's barrier
                             const uint32_t bar = lead_full0 + stage * (uint32_t)sizeof(uint64_t);
                             if (rank == 0) mbar_expect_tx(&full[stage], 2 * STAGE_BYTES);
-                            tma_load_2d_pair(stage_a + (size_t)stage * A_STAGE_BYTES, a_map, ks * BK, a_row, bar);
-                            tma_load_2d_pair(stage_b + (size_t)stage * B_STAGE_BYTES, &map_w, ks * BK,
+                            tma_load_2d_pair(smem_u32(stage_a) + stage * A_STAGE_BYTES, a_map, ks * BK, a_row, bar);
+                            tma_load_2d_pair(smem_u32(stage_b) + stage * B_STAGE_BYTES, &map_w, ks * BK,
                                              c * BN + (int)rank * (chunk_columns(p.V, c) / 2), bar);
                         } else {
                             mbar_expect_tx(&full[stage], STAGE_BYTES);
