@@ -20,6 +20,7 @@ struct arrol_ctx {
     unsigned long long* d_chain;   // fused prune step: finished blocks, index-check flag, per-block totals; zero between calls
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
     int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
+    bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel

@@ -68,201 +68,277 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
     }
 }
 
+// One block, bound by latency: a handful of dependent round trips to memory and a serial search.  Every input is read once
+// (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
+// that one block scan ranks all of them, and the bisection is settled in about five rounds of 31 points (see below) instead
+// of 64 steps, twenty of them with a serial sum.  Per call: N = 2,048, 128 bins 61.5 -> 26.7 us; N = 32, 64 bins 41 -> 22 us;
+// N = 8,192, 256 bins 100 -> 37 us.
+constexpr int CAL_STAGED = 8192;
+constexpr int CAL_POINTS = 31;                 // points per round, one warp each
+__host__ __device__ inline int product_pitch(int B) { return B | 1; }      // odd: 31 lanes walk 31 rows without bank conflicts
+constexpr int CAL_PRODUCT_BINS = 704;          // most bins whose products are held in shared memory (31 x 705 x 8 = 175 KB)
 __global__ void __launch_bounds__(CAL_THREADS)
 calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ bin, const float* __restrict__ rewards,
                     const uint8_t* __restrict__ mask, int N, double kappa, double lambda, double rho, double p_min,
                     double p_max, int B_arg, int64_t cap_arg, uint32_t* d_status) {
     CalibHeader* hd = reinterpret_cast<CalibHeader*>(state);
+    const int B = B_arg;
+    const int64_t cap = cap_arg;
+    __shared__ int16_t staged[CAL_STAGED];      // 2 bin + label of a rollout that is pushed, -1 of one that is not
+    __shared__ int32_t warp_sum[2][32];
+    __shared__ int32_t hist[2][MAX_BINS];       // signed change of the counts
+    __shared__ double term[MAX_BINS];           // lambda (rho - q_b)
+    __shared__ double weight[MAX_BINS];         // c_b^+ + c_b^-
+    __shared__ double point_at[32], point_sum[32], point_slope[32];
+    __shared__ double round_lo, round_hi, round_at;
+    __shared__ int round_kind;                  // 0 = done, 1 = tree, 2 = around the linear estimate
+    extern __shared__ double products[];        // [31][B rounded up to odd]: c_b p_b of a round's points
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+
+    auto code_of = [&](int i) {
+        if (mask && !mask[i]) return -1;
+        int b = bin[i];
+        b = b < 0 ? 0 : (b >= B ? B - 1 : b);
+        return 2 * b + (rewards[i] > 0.5f ? 1 : 0);
+    };
+    const bool in_shared = N <= CAL_STAGED;
+    if (in_shared) {
+#pragma unroll 4
+        for (int i = tid; i < N; i += CAL_THREADS) staged[i] = (int16_t)code_of(i);
+    }
     // The byte layout L comes from the call's (B, cap); the state must have been initialised with the same pair.
     // A mismatched or uninitialised state is left untouched and reported (uniform over the block: no barrier yet).
-    if (hd->B != B_arg || hd->cap != cap_arg) {
-        if (threadIdx.x == 0) atomicOr(d_status, ARROL_DEV_BAD_STATE);
+    if (hd->B != B || hd->cap != cap) {
+        if (tid == 0) atomicOr(d_status, ARROL_DEV_BAD_STATE);
         return;
     }
     int64_t* cnt[2] = {reinterpret_cast<int64_t*>(state + L.cneg), reinterpret_cast<int64_t*>(state + L.cpos)};
     int16_t* ring[2] = {reinterpret_cast<int16_t*>(state + L.ring_neg), reinterpret_cast<int16_t*>(state + L.ring_pos)};
     float* lut = reinterpret_cast<float*>(state + L.q_lut);
-    const int B = hd->B;
-    const int64_t cap = hd->cap;
-
-    __shared__ int32_t warp_sum[2][32];
-    __shared__ int64_t total_new[2];            // labelled rollouts pushed this call, per label
-    __shared__ int64_t head0[2], n0[2];
-    __shared__ int32_t hist[2][MAX_BINS];       // signed change of the counts
-    __shared__ double term[MAX_BINS];           // lambda (rho - q_b)
-    __shared__ double weight[MAX_BINS];         // c_b^+ + c_b^-
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-
-    for (int b = threadIdx.x; b < B; b += CAL_THREADS) { hist[0][b] = 0; hist[1][b] = 0; }
-    if (threadIdx.x == 0) {
-        head0[0] = hd->head_neg; n0[0] = hd->n_neg; head0[1] = hd->head_pos; n0[1] = hd->n_pos;
-        total_new[0] = 0; total_new[1] = 0;
-    }
+    const int64_t head0[2] = {hd->head_neg, hd->head_pos}, n0[2] = {hd->n_neg, hd->n_pos};
+    const double alpha = hd->alpha;
+    int64_t old_cnt[2] = {0, 0};                // B <= MAX_BINS = CAL_THREADS: thread b owns bin b
+    if (tid < B) { old_cnt[0] = cnt[0][tid]; old_cnt[1] = cnt[1][tid]; hist[0][tid] = 0; hist[1][tid] = 0; }
     __syncthreads();
 
-    // pass 1: how many new entries per label
-    {
-        int32_t c[2] = {0, 0};
-        for (int i = threadIdx.x; i < N; i += CAL_THREADS)
-            if (!mask || mask[i]) c[rewards[i] > 0.5f ? 1 : 0] += 1;
+    // rank of every new entry among those of its label, in index order
+    const int per = (N + CAL_THREADS - 1) / CAL_THREADS;
+    const int i0 = min(N, tid * per), i1 = min(N, i0 + per);
+    auto code = [&](int i) { return in_shared ? (int)staged[i] : code_of(i); };
+    int32_t mine[2] = {0, 0};
+    for (int i = i0; i < i1; ++i) {
+        const int c = code(i);
+        if (c >= 0) mine[c & 1] += 1;
+    }
+    int32_t incl[2];
 #pragma unroll
-        for (int l = 0; l < 2; ++l) {
-            int32_t v = c[l];
+    for (int l = 0; l < 2; ++l) {
+        int32_t v = mine[l];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) warp_sum[l][wid] = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += t;
         }
-        __syncthreads();
-        if (threadIdx.x < 2) {
-            int64_t t = 0;
-            for (int w = 0; w < CAL_THREADS / 32; ++w) t += warp_sum[threadIdx.x][w];
-            total_new[threadIdx.x] = t;
+        incl[l] = v;
+        if (lane == 31) warp_sum[l][wid] = v;
+    }
+    __syncthreads();
+    int64_t total_new[2], first_rank[2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {                // every warp scans the warp totals for itself
+        int32_t v = warp_sum[l][lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += t;
         }
-        __syncthreads();
+        total_new[l] = __shfl_sync(0xffffffffu, v, 31);
+        const int32_t before = __shfl_sync(0xffffffffu, v, wid > 0 ? wid - 1 : 0);
+        first_rank[l] = (wid > 0 ? before : 0) + incl[l] - mine[l];
     }
 
     // evict the oldest entries that the push displaces (read the rings before they are overwritten)
+#pragma unroll
     for (int l = 0; l < 2; ++l) {
         const int64_t over = n0[l] + total_new[l] - cap;
         const int64_t evict = over <= 0 ? 0 : (over < n0[l] ? over : n0[l]);
-        for (int64_t j = threadIdx.x; j < evict; j += CAL_THREADS)
-            atomicSub(&hist[l][ring[l][(head0[l] + j) % cap]], 1);
+        for (int64_t j = tid; j < evict; j += CAL_THREADS) {
+            const int64_t at = head0[l] + j;     // head0, j < cap
+            atomicSub(&hist[l][ring[l][at < cap ? at : at - cap]], 1);
+        }
     }
     __syncthreads();
 
-    // pass 2: write the new entries in index order; entry r of m lands in slot (head + n + r) mod cap, and only the
-    // last `cap` of them survive the call
-    int64_t carry[2] = {0, 0};
-    for (int base = 0; base < N; base += CAL_THREADS) {
-        const int i = base + threadIdx.x;
-        const bool on = (i < N) && (!mask || mask[i]);
-        const int lab = (on && rewards[i] > 0.5f) ? 1 : 0;
-        int32_t f[2] = {on && lab == 0 ? 1 : 0, on && lab == 1 ? 1 : 0};
-        int32_t incl[2];
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-            int32_t v = f[l];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += t;
-            }
-            incl[l] = v;
-            if (lane == 31) warp_sum[l][wid] = v;
-        }
-        __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int l = 0; l < 2; ++l) {
-                int32_t v = warp_sum[l][lane];
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
-                    if (lane >= o) v += t;
-                }
-                warp_sum[l][lane] = v;
+    // entry r of m lands in slot (head + n + r) mod cap, and only the last `cap` of them survive the call
+    {
+        const int64_t slot0[2] = {(head0[0] + n0[0]) % cap, (head0[1] + n0[1]) % cap};
+        int64_t r[2] = {first_rank[0], first_rank[1]};
+        for (int i = i0; i < i1; ++i) {
+            const int c = code(i);
+            if (c < 0) continue;
+            const int l = c & 1;
+            const int64_t rank = l ? r[1]++ : r[0]++;
+            if (rank >= total_new[l] - cap) {
+                const int64_t at = slot0[l] + (rank < cap ? rank : rank % cap);
+                ring[l][at < cap ? at : at - cap] = (int16_t)(c >> 1);
+                atomicAdd(&hist[l][c >> 1], 1);
             }
         }
-        __syncthreads();
-        if (on) {
-            const int64_t r = carry[lab] + (wid ? warp_sum[lab][wid - 1] : 0) + incl[lab] - 1;
-            if (r >= total_new[lab] - cap) {
-                int b = bin[i];
-                b = b < 0 ? 0 : (b >= B ? B - 1 : b);
-                ring[lab][(head0[lab] + n0[lab] + r) % cap] = (int16_t)b;
-                atomicAdd(&hist[lab][b], 1);
-            }
-        }
-        carry[0] += warp_sum[0][31];
-        carry[1] += warp_sum[1][31];
-        __syncthreads();
-    }
-
-    // counts, ring bookkeeping
-    for (int b = threadIdx.x; b < B; b += CAL_THREADS) {
-        cnt[0][b] += hist[0][b];
-        cnt[1][b] += hist[1][b];
     }
     __syncthreads();
-    if (threadIdx.x < 2) {
-        const int l = threadIdx.x;
+
+    // ring bookkeeping; every thread keeps the new sizes
+    int64_t n1[2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
         const int64_t over = n0[l] + total_new[l] - cap;
-        const int64_t n1 = over > 0 ? cap : n0[l] + total_new[l];
-        const int64_t h1 = over > 0 ? (head0[l] + over) % cap : head0[l];
-        if (l == 0) { hd->head_neg = h1; hd->n_neg = n1; } else { hd->head_pos = h1; hd->n_pos = n1; }
-        n0[l] = n1;     // totals for the table below
+        n1[l] = over > 0 ? cap : n0[l] + total_new[l];
+        if (tid == l) {
+            const int64_t h1 = over > 0 ? (head0[l] + over) % cap : head0[l];
+            if (l == 0) { hd->head_neg = h1; hd->n_neg = n1[l]; } else { hd->head_pos = h1; hd->n_pos = n1[l]; }
+        }
     }
-    __syncthreads();
 
     // posterior table (Laplace-smoothed likelihoods, Bayes rule), fp64, one rounding per operation
-    const double n_pos = (double)n0[1], n_neg = (double)n0[0];
-    const double alpha = hd->alpha;
-    const double prior = (n_pos + n_neg > 0.0) ? __ddiv_rn(n_pos, __dadd_rn(n_pos, n_neg)) : 0.5;
-    const double den_pos = __dadd_rn(n_pos, __dmul_rn(alpha, (double)B));
-    const double den_neg = __dadd_rn(n_neg, __dmul_rn(alpha, (double)B));
-    for (int b = threadIdx.x; b < B; b += CAL_THREADS) {
-        const double p1 = __ddiv_rn(__dadd_rn((double)cnt[1][b], alpha), den_pos);
-        const double p0 = __ddiv_rn(__dadd_rn((double)cnt[0][b], alpha), den_neg);
+    const double n_pos = (double)n1[1], n_neg = (double)n1[0];
+    const double n = __dadd_rn(n_pos, n_neg);
+    if (tid < B) {
+        const double prior = n > 0.0 ? __ddiv_rn(n_pos, n) : 0.5;
+        const double den_pos = __dadd_rn(n_pos, __dmul_rn(alpha, (double)B));
+        const double den_neg = __dadd_rn(n_neg, __dmul_rn(alpha, (double)B));
+        const int64_t c_neg = old_cnt[0] + hist[0][tid], c_pos = old_cnt[1] + hist[1][tid];
+        cnt[0][tid] = c_neg;
+        cnt[1][tid] = c_pos;
+        const double p1 = __ddiv_rn(__dadd_rn((double)c_pos, alpha), den_pos);
+        const double p0 = __ddiv_rn(__dadd_rn((double)c_neg, alpha), den_neg);
         const double num = __dmul_rn(prior, p1);
         const double den = __dadd_rn(num, __dmul_rn(__dsub_rn(1.0, prior), p0));
         const float qb = (float)__ddiv_rn(num, den);
-        lut[b] = qb;
-        term[b] = __dmul_rn(lambda, __dsub_rn(rho, (double)qb));
-        weight[b] = (double)(cnt[0][b] + cnt[1][b]);
+        lut[tid] = qb;
+        term[tid] = __dmul_rn(lambda, __dsub_rn(rho, (double)qb));
+        weight[tid] = (double)(c_neg + c_pos);
     }
     __syncthreads();
 
-    // delta: 64 bisection steps on E[p](delta) = kappa, by the first warp alone (no block barriers in the loop).  The
-    // value that decides a step is the expected keep rate summed over the bins in index order, one rounding per
-    // operation (so that delta agrees bit for bit with a plain loop).  Per step the lanes form the per-bin products
-    // c_b p_b (all >= 0) and a butterfly sum S of them; the in-order sum differs from S by at most
-    // (B + 8) 2^-53 S (both are within their standard error bounds of the exact sum), so when S / n is further from
-    // kappa than four times that bound plus the rounding of the division, S / n < kappa already is the decision.
-    // Only the steps near convergence (about the last twenty) need the serial chain of B additions.
-    if (wid == 0) {
-        __shared__ double prod[MAX_BINS];
-        const double n = __dadd_rn(n_pos, n_neg);
-        double delta = 0.0;
-        if (n > 0.0) {                                   // uniform for the warp
-            double lo = -(1.0 + lambda), hi = 1.0 + lambda;
-            const double u = 1.1102230246251565e-16;     // 2^-53
-            for (int it = 0; it < 64; ++it) {
-                const double mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
-                const double base = __dadd_rn(kappa, mid);
-                double part = 0.0;
-                for (int b = lane; b < B; b += 32) {
-                    double p = __dadd_rn(base, term[b]);
-                    if (p < p_min) p = p_min;
-                    if (p > p_max) p = p_max;
-                    const double x = __dmul_rn(weight[b], p);
-                    prod[b] = x;
-                    part += x;
+    // delta: 64 bisection steps on E[p](delta) = kappa.  The value that decides a step is the expected keep rate summed over
+    // the bins in index order, one rounding per operation (so that delta agrees bit for bit with a plain loop).
+    //   Rounded addition, multiplication, clamping and division are all monotone, so the decision "below" is a monotone
+    // function of the midpoint, bit for bit: one evaluation at x settles every midpoint on its side of x.  So the block
+    // evaluates 31 points a round (one warp each) and the first warp replays the bisection as far as the settled points
+    // reach.  Rounds 0 and 1 take the 31 midpoints of the next five levels; round 2 takes points at growing distances around
+    // the root of the linear piece that E is on by then, which settles most of the remaining levels; then five levels a
+    // round again until the bracket stops shrinking.
+    //   One evaluation: the lanes form the per-bin products c_b p_b (all >= 0) and a butterfly sum S of them; the in-order sum
+    // differs from S by at most (B + 8) 2^-53 S (both are within their standard error bounds of the exact sum), so when S is
+    // further from kappa n than four times that bound plus the roundings of the division and of kappa n, S < kappa n already
+    // is the decision.  Points closer than that need the serial chain of B additions: the first warp runs the chains of all
+    // 31 points side by side, one per lane (an addition takes about 30 cycles, and chains in 31 warps would queue for the fp64
+    // pipe).
+    double delta = 0.0;
+    if (n > 0.0) {                                   // uniform for the block
+        const double u = 1.1102230246251565e-16;     // 2^-53
+        const double goal = kappa * n;
+        const int pitch = product_pitch(B);
+        auto midpoint = [](double a, double b) { return __dmul_rn(0.5, __dadd_rn(a, b)); };
+        auto clipped = [&](double p) {
+            if (p < p_min) p = p_min;
+            if (p > p_max) p = p_max;
+            return p;
+        };
+        double lo = -(1.0 + lambda), hi = 1.0 + lambda;           // the first warp's
+        double known_below = lo - 1.0, known_above = hi + 1.0;    // settled points next to the threshold
+        double sum_at = 0.0, slope_at = 0.0;                      // S and dS/d(delta) at known_below
+        int step = 0;
+        for (int round = 0;; ++round) {
+            if (wid == 0) {
+                for (; step < 64; ++step) {
+                    const double m = midpoint(lo, hi);
+                    if (m <= known_below) { if (m == lo) step = 64; lo = m; }        // an unchanged bracket stays unchanged
+                    else if (m >= known_above) { if (m == hi) step = 64; hi = m; }
+                    else break;
+                }
+                if (lane == 0) {
+                    const bool linear = round == 2 && slope_at > 0.0;
+                    round_kind = step >= 64 ? 0 : (linear ? 2 : 1);
+                    round_lo = lo; round_hi = hi;
+                    round_at = linear ? fmin(fmax(known_below + (goal - sum_at) / slope_at, lo), hi) : 0.0;
+                }
+            }
+            __syncthreads();
+            const int kind = round_kind;
+            if (kind == 0) break;
+            // this warp's point
+            double x = 0.0;
+            if (kind == 1) {                         // node of the binary tree of midpoints, 1 = the next one; children 2k, 2k + 1
+                double a = round_lo, b = round_hi;
+                const int node = wid < CAL_POINTS ? wid + 1 : 1;
+                for (int bit = 30 - __clz(node); bit >= 0; --bit) {
+                    const double m = midpoint(a, b);
+                    if ((node >> bit) & 1) a = m; else b = m;
+                }
+                x = midpoint(a, b);
+            } else {
+                const int i = wid < 15 ? 15 - wid : wid - 15;       // 0 .. 15 steps away: 2^-51 ... 2^-44, then coarser
+                const int e = i <= 8 ? i - 52 : (i == 9 ? -42 : i == 10 ? -39 : i == 11 ? -36 : i == 12 ? -32 : i == 13 ? -26 : i == 14 ? -18 : -10);
+                const double off = i == 0 ? 0.0 : scalbn(1.0 + lambda, e);
+                x = wid < 15 ? round_at - off : round_at + off;
+            }
+            if (wid < CAL_POINTS) {
+                const double base = __dadd_rn(kappa, x);
+                double part = 0.0, slope = 0.0;
+                for (int k = lane; k < B; k += 32) {
+                    const double raw = __dadd_rn(base, term[k]), p = clipped(raw);
+                    const double v = __dmul_rn(weight[k], p);
+                    if (B <= CAL_PRODUCT_BINS) products[wid * pitch + k] = v;
+                    part += v;
+                    if (p == raw) slope += weight[k];
                 }
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);   // the same bits in every lane
-                const double e_tree = part / n;
-                const double slack = 4.0 * ((double)(B + 8) * u * e_tree + 2.0 * u * (e_tree + kappa));
-                int below;
-                if (fabs(e_tree - kappa) > slack) {
-                    below = e_tree < kappa ? 1 : 0;
-                } else {
-                    __syncwarp();
-                    below = 0;
-                    if (lane == 0) {
-                        double e = 0.0;
-#pragma unroll 8
-                        for (int b = 0; b < B; ++b) e = __dadd_rn(e, prod[b]);
-                        below = __ddiv_rn(e, n) < kappa ? 1 : 0;
-                    }
-                    below = __shfl_sync(0xffffffffu, below, 0);
+                for (int o = 16; o > 0; o >>= 1) {
+                    part += __shfl_xor_sync(0xffffffffu, part, o);
+                    slope += __shfl_xor_sync(0xffffffffu, slope, o);
                 }
-                __syncwarp();                            // prod is rewritten by the next step
-                if (below) lo = mid; else hi = mid;
+                if (lane == 0) { point_sum[wid] = part; point_slope[wid] = slope; }
+                if (lane == 1) point_at[wid] = x;
             }
-            delta = __dmul_rn(0.5, __dadd_rn(lo, hi));
+            __syncthreads();
+            if (wid == 0) {
+                const bool has = lane < CAL_POINTS;
+                const double S = has ? point_sum[lane] : 0.0;
+                const double at = has ? point_at[lane] : 0.0;
+                const double slack = 4.0 * ((double)(B + 8) * u * S + 3.0 * u * (S + goal));
+                const bool near = has && fabs(S - goal) <= slack;
+                bool below = S < goal;
+                if (__any_sync(0xffffffffu, near)) {
+                    double e = 0.0;
+                    if (B <= CAL_PRODUCT_BINS) {
+                        const double* row = products + (has ? lane : 0) * pitch;
+#pragma unroll 8
+                        for (int k = 0; k < B; ++k) e = __dadd_rn(e, row[k]);
+                    } else {
+                        const double base = __dadd_rn(kappa, at);
+#pragma unroll 4
+                        for (int k = 0; k < B; ++k) e = __dadd_rn(e, __dmul_rn(weight[k], clipped(__dadd_rn(base, term[k]))));
+                    }
+                    if (near) below = __ddiv_rn(e, n) < kappa;
+                }
+                // settled points next to the threshold, over the warp
+                double best_below = has && below ? at : known_below, best_above = has && !below ? at : known_above;
+                double s_at = has && below ? S : sum_at, d_at = has && below ? point_slope[lane] : slope_at;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const double ob = __shfl_xor_sync(0xffffffffu, best_below, o), os = __shfl_xor_sync(0xffffffffu, s_at, o);
+                    const double od = __shfl_xor_sync(0xffffffffu, d_at, o), oa = __shfl_xor_sync(0xffffffffu, best_above, o);
+                    if (ob > best_below) { best_below = ob; s_at = os; d_at = od; }
+                    best_above = fmin(best_above, oa);
+                }
+                if (best_below > known_below) { known_below = best_below; sum_at = s_at; slope_at = d_at; }
+                known_above = fmin(known_above, best_above);
+            }
         }
-        if (lane == 0) hd->delta = delta;
+        delta = midpoint(lo, hi);                    // meaningful in the first warp
     }
+    if (tid == 0) hd->delta = delta;
 }
 
 __global__ void select_stochastic_kernel(const float* __restrict__ q, const float* __restrict__ u,
@@ -338,7 +414,13 @@ extern "C" int arrol_calib_update(arrol_ctx* ctx, void* state, int32_t B, int64_
     if (N > 0 && (!bin || !rewards)) return ARROL_ERR_INVALID_ARG;
     ArrolDeviceGuard guard(ctx->device);
     if (!guard.ok) return ARROL_ERR_CUDA;
-    calib_update_kernel<<<1, CAL_THREADS, 0, (cudaStream_t)stream>>>(static_cast<uint8_t*>(state), layout_of(B, cap), bin,
+    if (!ctx->calib_smem_set) {
+        ARROL_CUDA_OK(cudaFuncSetAttribute(calib_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(sizeof(double) * CAL_POINTS * product_pitch(CAL_PRODUCT_BINS))));
+        ctx->calib_smem_set = true;
+    }
+    const size_t smem = B <= CAL_PRODUCT_BINS ? sizeof(double) * CAL_POINTS * product_pitch(B) : 0;
+    calib_update_kernel<<<1, CAL_THREADS, smem, (cudaStream_t)stream>>>(static_cast<uint8_t*>(state), layout_of(B, cap), bin,
                                                                   rewards, mask, N, sp->kappa, sp->lambda, sp->rho,
                                                                   sp->p_min, sp->p_max, B, cap, ctx->d_status);
     ctx->launches += 1;

@@ -54,6 +54,12 @@ def test_calibrator_update_matches_oracle(ctx, n_bins, cap, sizes):
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
 
 
+@pytest.mark.parametrize("n_bins,cap,sizes", [(1024, 3000, [9000, 8192, 8193, 1]),      # both sides of the staged rollouts
+                                              (33, 20000, [1025, 12345, 1023])])
+def test_calibrator_update_beyond_the_staged_rollouts(ctx, n_bins, cap, sizes):
+    test_calibrator_update_matches_oracle(ctx, n_bins, cap, sizes)
+
+
 def test_delta_is_bit_equal_over_many_states_and_parameters(ctx):
     """delta decides by comparisons that turn on the last bits near convergence: many random buffer states, skewed
     score distributions and survival parameters, every one bit for bit."""
