@@ -15,11 +15,13 @@ struct arrol_ctx {
     uint32_t* d_status;        // device status word (bits ARROL_DEV_*)
     uint32_t* h_status;        // pinned host mirror used by arrol_poll_status
     float* d_scratch;          // MLP-head partial sums: [ARROL_SCRATCH_FLOATS]
-    void* d_pack;              // MLP head on the tensor cores: the scored rows packed as bf16 [N][d], ARROL_PACK_BYTES
     uint32_t* d_tile_counters; // MLP head on the tensor cores: finished blocks per row tile, zero between calls
+    void* d_pack;              // MLP head on the tensor cores: the scored rows packed as bf16 [N][d], ARROL_PACK_BYTES
+    uint32_t* d_head_counters; // head training step: finished runs per column tile, zero between calls
     unsigned long long* d_chain;   // fused prune step: finished blocks, index-check flag, per-block totals; zero between calls
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
     int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
+    bool head_dw1_smem_set[2]; // likewise for the head training step's contraction (column tiles of 64, 128)
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
@@ -45,7 +47,8 @@ constexpr int ARROL_MLP_TH = 64;             // hidden units per MLP thread-bloc
 constexpr int ARROL_MAX_H = 4096;
 constexpr size_t ARROL_SCRATCH_FLOATS = (size_t)ARROL_MAX_MLP_N * (ARROL_MAX_H / ARROL_MLP_TH);
 constexpr size_t ARROL_PACK_BYTES = (size_t)64 << 20;
-constexpr int ARROL_TILE_COUNTERS = 1024;   // [0, 1020) row tiles of the MLP head, then 16 bytes for the head training step's contractions
+constexpr int ARROL_TILE_COUNTERS = 1024;   // [0, 1020) row tiles of the MLP head
+constexpr int ARROL_HEAD_COUNTERS = ARROL_MAX_H / 32;   // column tiles of the head training step
 constexpr int ARROL_SCORE_ROW_TILES = 1020;
 constexpr int ARROL_CHAIN_BLOCKS = 510;      // blocks of the fused prune step's chained scan (2 + 2 * 510 words = 8 KB)
 
@@ -145,7 +148,6 @@ int arrol_internal_gather_rows_bulk(arrol_ctx* ctx, const int64_t* d_num, const 
                                     const int32_t* survivor_idx, const int64_t* src_tok_off, const void* src_rows,
                                     int64_t row_bytes, int64_t capacity, void* dst_rows, cudaStream_t s);
 
-// lm_head_backward.cu: C[M,N] (+)= A^T B on the tensor cores, A stored [K, M] and B stored [K, N] row-major bf16
-// (rows lda / ldb elements apart, multiples of 8), C fp32 with rows ldc apart.  Rows past K read as zero.
-int arrol_internal_gemm_tn(arrol_ctx* ctx, const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N, int K,
-                           float* C, int64_t ldc, int accumulate, cudaStream_t s);
+// head_grad_tc.cu: dW1[h, d] = (du_hi + du_lo)^T X on the tensor cores, du planes [N, h] bf16, X [N, d] bf16 with rows ldx apart.
+int arrol_internal_head_dw1(arrol_ctx* ctx, const void* du_hi, const void* du_lo, const void* X, int64_t ldx, int N, int d,
+                            int h, float* dW1, cudaStream_t s);

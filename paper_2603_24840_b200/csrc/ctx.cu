@@ -43,6 +43,8 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
     ctx->h_status = nullptr;
     ctx->d_scratch = nullptr;
     ctx->d_pack = nullptr;
+    ctx->d_head_counters = nullptr;
+    ctx->head_dw1_smem_set[0] = ctx->head_dw1_smem_set[1] = false;
     ctx->d_tile_counters = nullptr;
     ctx->d_chain = nullptr;
     ctx->logprob_smem_set = false;
@@ -71,6 +73,8 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
               cudaMallocHost(&ctx->h_status, 64) == cudaSuccess &&
               cudaMalloc(&ctx->d_scratch, ARROL_SCRATCH_FLOATS * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&ctx->d_pack, ARROL_PACK_BYTES) == cudaSuccess &&
+              cudaMalloc(&ctx->d_head_counters, ARROL_HEAD_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
+              cudaMemset(ctx->d_head_counters, 0, ARROL_HEAD_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_tile_counters, ARROL_TILE_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMemset(ctx->d_tile_counters, 0, ARROL_TILE_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_chain, (2 + 2 * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
@@ -103,6 +107,7 @@ extern "C" int arrol_destroy(arrol_ctx* ctx) {
     if (ctx->h_status) (void)cudaFreeHost(ctx->h_status);
     if (ctx->d_scratch) (void)cudaFree(ctx->d_scratch);
     if (ctx->d_pack) (void)cudaFree(ctx->d_pack);
+    if (ctx->d_head_counters) (void)cudaFree(ctx->d_head_counters);
     if (ctx->d_tile_counters) (void)cudaFree(ctx->d_tile_counters);
     if (ctx->d_chain) (void)cudaFree(ctx->d_chain);
     if (ctx->h_keep) (void)cudaFreeHost(ctx->h_keep);

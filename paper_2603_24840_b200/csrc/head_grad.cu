@@ -12,7 +12,7 @@
 namespace {
 
 constexpr int DS_THREADS = 1024;
-constexpr int DU_RUNS = 32;          // row runs of the du kernel on the tensor-core path
+constexpr int DU_RUNS = 32;          // runs of rollouts of head_du_kernel
 
 __device__ __forceinline__ double block_sum(double v, double* sh /* [32] */) {
 #pragma unroll
@@ -25,18 +25,11 @@ __device__ __forceinline__ double block_sum(double v, double* sh /* [32] */) {
     return t;
 }
 
-// s_i (given, or assembled from the MLP tile partials), ds_i, loss, sum of ds.  One block.
-template <typename T>
+// Linear head: ds_i, loss, sum of ds.  One block.
 __global__ void __launch_bounds__(DS_THREADS)
-head_ds_kernel(const float* __restrict__ score, const float* __restrict__ partial, int h_tiles,
-               const T* __restrict__ b2_ptr, int N,
-               const float* __restrict__ rewards, const uint8_t* __restrict__ mask, float* __restrict__ ds,
+head_ds_kernel(const float* __restrict__ score, int N, const float* __restrict__ rewards, const uint8_t* __restrict__ mask, float* __restrict__ ds,
                double* __restrict__ loss, float* __restrict__ dbias) {
     __shared__ double sh[32];
-    float b2 = 0.f;
-    if (b2_ptr) {
-        if constexpr (sizeof(T) == 2) b2 = __bfloat162float(b2_ptr[0]); else b2 = b2_ptr[0];
-    }
     double cnt = 0.0;
     for (int i = threadIdx.x; i < N; i += DS_THREADS) cnt += (!mask || mask[i]) ? 1.0 : 0.0;
     const double n = block_sum(cnt, sh);
@@ -44,13 +37,7 @@ head_ds_kernel(const float* __restrict__ score, const float* __restrict__ partia
     for (int i = threadIdx.x; i < N; i += DS_THREADS) {
         float v = 0.f;
         if (!mask || mask[i]) {
-            float s;
-            if (score) s = score[i];
-            else {
-                s = 0.f;
-                for (int t = 0; t < h_tiles; ++t) s += partial[(int64_t)t * N + i];
-                s += b2;
-            }
+            const float s = score[i];
             const float y = rewards[i] > 0.5f ? 1.f : 0.f;
             const float softplus = s > 0.f ? s + log1pf(expf(-s)) : log1pf(expf(s));
             l += (double)(softplus - y * s);
@@ -67,6 +54,8 @@ head_ds_kernel(const float* __restrict__ score, const float* __restrict__ partia
     }
 }
 
+__device__ __forceinline__ float widen(__nv_bfloat16 x) { return __bfloat162float(x); }
+__device__ __forceinline__ float widen(float x) { return x; }
 __device__ __forceinline__ void widen8(const __nv_bfloat16* p, float (&o)[8]) {
     const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -110,48 +99,148 @@ __global__ void column_sum_kernel(const float* __restrict__ partial, int chunks,
     out[k] = s;
 }
 
-// MLP head: du_ij, and per hidden unit j the sums dw2_j = sum_i ds_i gelu(u_ij), db1_j = sum_i du_ij.
-// Block = 32 hidden units x 8 row lanes; rows are walked in a fixed order.
+// MLP head: everything between the forward and the dW1 contraction in one launch: ds_i, the loss, du_ij, and per hidden unit
+// the sums dw2_j = sum_i ds_i gelu(u_ij), db1_j = sum_i du_ij.  (It was four launches: ds by one block, du, two column sums,
+// 22 us at N = 2,048, h = 256 against 9 now.)  Block (x, y): 32 hidden units, a run of rollouts.  Every block counts the labelled rollouts itself and forms the
+// ds of its own run; the last block of a column tile to arrive (a counter per tile, reset by that block) adds the runs' sums in
+// index order, the one of tile 0 the loss and db2 as well.  The score is given, or the sum of the forward's tile partials + b2.
+// du goes out as float (SIMT contraction) or as the sum of two bf16 planes (error 2^-17 relative: the tensor-core operand).
+template <int THREADS>
+__device__ __forceinline__ int count_labelled(const uint8_t* mask, int N) {
+    if (!mask) return N;
+    int c = 0;
+    const int vec = (reinterpret_cast<uintptr_t>(mask) & 15) == 0 ? N / 16 : 0;
+    for (int i = threadIdx.x; i < vec; i += THREADS) {
+        const uint4 v = reinterpret_cast<const uint4*>(mask)[i];
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c += __popc(__vcmpne4(w[k], 0u)) >> 3;
+    }
+    for (int i = vec * 16 + threadIdx.x; i < N; i += THREADS) c += mask[i] ? 1 : 0;
+    return c;
+}
+
+constexpr int DU_THREADS = 256;
 template <typename T>
-__global__ void __launch_bounds__(256)
-mlp_du_kernel(const float* __restrict__ u, const float* __restrict__ ds, const T* __restrict__ w2, int N, int h,
-              float* __restrict__ du, __nv_bfloat16* __restrict__ du_hi, __nv_bfloat16* __restrict__ du_lo,
-              float* __restrict__ dw2, float* __restrict__ db1, int rows_per_block) {
-    __shared__ float sh_w2[8][33], sh_b1[8][33];
+__global__ void __launch_bounds__(DU_THREADS)
+head_du_kernel(const float* u, const float* score, const float* partial, int h_tiles, const T* b2, const float* rewards,
+               const uint8_t* mask, const T* w2, int N, int h, int rows_per_run, float* __restrict__ du,
+               __nv_bfloat16* __restrict__ du_hi, __nv_bfloat16* __restrict__ du_lo, float* run_sums /* [2][runs][h] */,
+               double* run_loss /* [2][runs] */, uint32_t* counters, float* __restrict__ dw2, float* __restrict__ db1,
+               double* __restrict__ loss, float* __restrict__ db2) {
+    extern __shared__ float ds_s[];            // [rows_per_run]; NaN-free: 0 for rollouts that do not count
+    __shared__ float sums[2][8][33];
+    __shared__ double warp_d[2][DU_THREADS / 32];
+    __shared__ int warp_n[DU_THREADS / 32], is_last;
+    pdl_launch_dependents();
+    pdl_wait();
+    u = pdl_acquire(u); score = pdl_acquire(score); rewards = pdl_acquire(rewards); mask = pdl_acquire(mask);
+    w2 = pdl_acquire(w2); partial = pdl_acquire(partial); b2 = pdl_acquire(b2);
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int runs = gridDim.y, run = blockIdx.y;
+    const int i0 = run * rows_per_run, i1 = min(N, i0 + rows_per_run);
     const int j = blockIdx.x * 32 + tx;
+    // everything that depends on nothing is requested first: the first pre-activations, then the labels to count
+    constexpr int AHEAD = 8;
+    float ahead[AHEAD];
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) {
+        const int i = i0 + ty + 8 * k;
+        ahead[k] = j < h && i < i1 ? u[(int64_t)i * h + j] : 0.f;
+    }
+    const float wj = j < h ? widen(w2[j]) : 0.f;
+    {
+        int c = count_labelled<DU_THREADS>(mask, N);
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (tx == 0) warp_n[ty] = mask ? c : 0;
+    }
+    __syncthreads();
+    int n = mask ? 0 : N;
+#pragma unroll
+    for (int w = 0; w < DU_THREADS / 32; ++w) n += warp_n[w];
+    double l = 0.0, sd = 0.0;
+    for (int i = i0 + threadIdx.x; i < i1; i += DU_THREADS) {
+        float v = 0.f;
+        if (!mask || mask[i]) {
+            float s = 0.f;
+            if (score) {
+                s = score[i];
+            } else {
+                for (int t = 0; t < h_tiles; ++t) s += partial[(int64_t)t * N + i];
+                if (b2) s += widen(b2[0]);
+            }
+            const float y = rewards[i] > 0.5f ? 1.f : 0.f;
+            const float softplus = s > 0.f ? s + log1pf(expf(-s)) : log1pf(expf(s));
+            l += (double)(softplus - y * s);
+            v = (1.0f / (1.0f + expf(-s)) - y) / (float)n;
+            sd += (double)v;
+        }
+        ds_s[i - i0] = v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        l += __shfl_xor_sync(0xffffffffu, l, o);
+        sd += __shfl_xor_sync(0xffffffffu, sd, o);
+    }
+    if (tx == 0) { warp_d[0][ty] = l; warp_d[1][ty] = sd; }
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x < 2) {
+        double t = 0.0;
+        for (int w = 0; w < DU_THREADS / 32; ++w) t += warp_d[threadIdx.x][w];
+        run_loss[threadIdx.x * runs + run] = t;
+    }
     float a_w2 = 0.f, a_b1 = 0.f;
     if (j < h) {
-        float wj;
-        if constexpr (sizeof(T) == 2) wj = __bfloat162float(w2[j]); else wj = w2[j];
-        // blockIdx.y picks a run of rows; its sums go to row blockIdx.y of dw2 / db1 ([gridDim.y][h]), added up in
-        // index order by column_sum_kernel when there is more than one run
-        const int i_begin = blockIdx.y * rows_per_block, i_end = min(N, i_begin + rows_per_block);
-        for (int i = i_begin + ty; i < i_end; i += 8) {
-            const float g = ds[i];
-            const float a = u[(int64_t)i * h + j];
+        auto one = [&](int i, float a) {
+            const float g = ds_s[i - i0];
             const float cdf = 0.5f * (1.0f + erff(a * 0.70710678118654752440f));
             const float pdf = expf(-0.5f * a * a) * 0.39894228040143267794f;
             const float d_u = g * wj * (cdf + a * pdf);
-            if (du_hi) {       // du as the sum of two bf16 numbers (error 2^-17 relative): the tensor-core operand
+            if (du) {
+                du[(int64_t)i * h + j] = d_u;
+            } else {
                 const __nv_bfloat16 hi = __float2bfloat16_rn(d_u);
                 du_hi[(int64_t)i * h + j] = hi;
                 du_lo[(int64_t)i * h + j] = __float2bfloat16_rn(d_u - __bfloat162float(hi));
-            } else {
-                du[(int64_t)i * h + j] = d_u;
             }
             a_w2 = fmaf(g, a * cdf, a_w2);
             a_b1 += d_u;
-        }
+        };
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k)
+            if (i0 + ty + 8 * k < i1) one(i0 + ty + 8 * k, ahead[k]);
+#pragma unroll 4
+        for (int i = i0 + ty + 8 * AHEAD; i < i1; i += 8) one(i, u[(int64_t)i * h + j]);
     }
-    sh_w2[ty][tx] = a_w2;
-    sh_b1[ty][tx] = a_b1;
+    sums[0][ty][tx] = a_w2;
+    sums[1][ty][tx] = a_b1;
     __syncthreads();
-    if (ty == 0 && j < h) {
-        float s1 = 0.f, s2 = 0.f;
-        for (int r = 0; r < 8; ++r) { s1 += sh_w2[r][tx]; s2 += sh_b1[r][tx]; }
-        dw2[(int64_t)blockIdx.y * h + j] = s1;
-        db1[(int64_t)blockIdx.y * h + j] = s2;
+    if (ty < 2 && j < h) {
+        float t = 0.f;
+        for (int r = 0; r < 8; ++r) t += sums[ty][r][tx];
+        run_sums[((int64_t)ty * runs + run) * h + j] = t;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        is_last = atomicAdd(&counters[blockIdx.x], 1u) == (uint32_t)runs - 1u ? 1 : 0;
+        if (is_last) counters[blockIdx.x] = 0u;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    if (ty < 2 && j < h) {
+        float t = 0.f;
+#pragma unroll 8
+        for (int r = 0; r < runs; ++r) t += __ldcg(&run_sums[((int64_t)ty * runs + r) * h + j]);
+        (ty == 0 ? dw2 : db1)[j] = t;
+    }
+    if (blockIdx.x == 0 && threadIdx.x >= 64 && threadIdx.x < 66) {
+        const int which = threadIdx.x - 64;
+        double t = 0.0;
+        for (int r = 0; r < runs; ++r) t += __ldcg(&run_loss[which * runs + r]);
+        if (which == 0) *loss = n > 0 ? t / (double)n : 0.0;
+        else *db2 = (float)t;
     }
 }
 
@@ -215,7 +304,7 @@ mlp_dw1_kernel(const float* __restrict__ du, const T* __restrict__ hidden, int64
 }
 
 struct GradLayout {
-    size_t tmp3, ds, u, du, partial, total;   // byte offsets
+    size_t tmp3, ds, u, du, run_loss, run_sums, partial, total;   // byte offsets
     size_t du_plane;                          // bytes of one bf16 plane of du (hi at du, lo at du + du_plane)
 };
 GradLayout grad_layout(int N, int d, int h) {
@@ -232,7 +321,8 @@ GradLayout grad_layout(int N, int d, int h) {
     const size_t chunks = ((size_t)N + LIN_ROWS - 1) / LIN_ROWS;
     const size_t tiles = (size_t)((h > 0 ? h : 0) + ARROL_MLP_TH - 1) / ARROL_MLP_TH;
     size_t part = h > 0 ? tiles * (size_t)N : chunks * (size_t)d;
-    if (h > 0 && part < 2 * (size_t)DU_RUNS * (size_t)h) part = 2 * (size_t)DU_RUNS * (size_t)h;   // dw2 / db1 per row run
+    L.run_loss = o; o = up(o + sizeof(double) * 2 * DU_RUNS);                                       // loss / db2 per run
+    L.run_sums = o; o = up(o + sizeof(float) * 2 * (size_t)DU_RUNS * (size_t)(h > 0 ? h : 0));      // dw2 / db1 per run
     L.partial = o; o = up(o + sizeof(float) * part);
     L.total = o;
     return L;
@@ -251,7 +341,7 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         const int rc = arrol_score_partial(ctx, hidden, row_stride, row_index, N, head, nullptr, tmp, tmp + N, nullptr,
                                            tmp + 2 * (size_t)N, s);
         if (rc != ARROL_OK) return rc;
-        head_ds_kernel<T><<<1, DS_THREADS, 0, s>>>(tmp, nullptr, 0, nullptr, N, rewards, mask, ds, loss, db1);
+        head_ds_kernel<<<1, DS_THREADS, 0, s>>>(tmp, N, rewards, mask, ds, loss, db1);
         const int chunks = (N + LIN_ROWS - 1) / LIN_ROWS;
         dim3 grid((d / 8 + 255) / 256, chunks);
         linear_dw_partial_kernel<T><<<grid, 256, 0, s>>>(hid, row_stride, row_index, N, d, ds, partial);
@@ -260,6 +350,19 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
     } else {
         float* u = reinterpret_cast<float*>(ws + L.u);
         float* du = reinterpret_cast<float*>(ws + L.du);
+        auto launch_du = [&](const float* score, const float* tile_partial, int h_tiles, float* du_f, __nv_bfloat16* hi,
+                             __nv_bfloat16* lo) -> int {
+            const int rows_per = ((N + DU_RUNS - 1) / DU_RUNS + 7) / 8 * 8;
+            const int runs = (N + rows_per - 1) / rows_per;
+            ARROL_CUDA_OK(arrol_launch_pdl(head_du_kernel<T>, dim3((h + 31) / 32, runs), dim3(DU_THREADS), sizeof(float) * rows_per, s,
+                                           static_cast<const float*>(u), score, tile_partial, h_tiles,
+                                           score ? nullptr : static_cast<const T*>(head->b2), rewards, mask,
+                                           static_cast<const T*>(head->w2), N, h, rows_per, du_f, hi, lo,
+                                           reinterpret_cast<float*>(ws + L.run_sums), reinterpret_cast<double*>(ws + L.run_loss),
+                                           ctx->d_head_counters, dw2, db1, loss, db2));
+            ctx->launches += 1;
+            return ARROL_OK;
+        };
         if constexpr (sizeof(T) == 2) {
             // bf16 head: both contractions on the tensor cores.  Forward with the pre-activations kept, du split into
             // two bf16 planes, dW1 = du_hi^T X + du_lo^T X with X the packed rows (or the rows in place).
@@ -270,38 +373,21 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
                 if (rc == ARROL_OK) {
                     __nv_bfloat16* du_hi = reinterpret_cast<__nv_bfloat16*>(ws + L.du);
                     __nv_bfloat16* du_lo = reinterpret_cast<__nv_bfloat16*>(ws + L.du + L.du_plane);
-                    head_ds_kernel<T><<<1, DS_THREADS, 0, s>>>(tmp, nullptr, 0, nullptr, N, rewards, mask, ds, loss, db2);
-                    // the tile partials are consumed by now: the region holds the per-run sums of dw2 and db1
-                    const int rows_per = ((N + DU_RUNS - 1) / DU_RUNS + 7) / 8 * 8;
-                    const int runs = (N + rows_per - 1) / rows_per;
-                    float* dw2_runs = partial;
-                    float* db1_runs = partial + (size_t)DU_RUNS * h;
-                    mlp_du_kernel<T><<<dim3((h + 31) / 32, runs), 256, 0, s>>>(u, ds, static_cast<const T*>(head->w2), N, h,
-                                                                               nullptr, du_hi, du_lo, dw2_runs, db1_runs,
-                                                                               rows_per);
-                    column_sum_kernel<<<(h + 255) / 256, 256, 0, s>>>(dw2_runs, runs, h, dw2);
-                    column_sum_kernel<<<(h + 255) / 256, 256, 0, s>>>(db1_runs, runs, h, db1);
-                    ctx->launches += 4;
-                    ARROL_CUDA_OK(cudaGetLastError());
-                    const void* x = row_index ? ctx->d_pack : hidden;
-                    const int64_t ldx = row_index ? d : row_stride;
-                    int rg = arrol_internal_gemm_tn(ctx, du_hi, h, x, ldx, h, d, N, dW1, d, 0, s);
-                    if (rg == ARROL_OK) rg = arrol_internal_gemm_tn(ctx, du_lo, h, x, ldx, h, d, N, dW1, d, 1, s);
-                    return rg;
+                    const int rd = launch_du(tmp, nullptr, 0, nullptr, du_hi, du_lo);
+                    if (rd != ARROL_OK) return rd;
+                    return arrol_internal_head_dw1(ctx, du_hi, du_lo, row_index ? ctx->d_pack : hidden,
+                                                   row_index ? (int64_t)d : row_stride, N, d, h, dW1, s);
                 }
                 if (rc != ARROL_ERR_UNSUPPORTED) return rc;
             }
         }
         const int rc = arrol_internal_mlp_tiles(ctx, hidden, row_stride, row_index, N, head, partial, u, s);
         if (rc != ARROL_OK) return rc;
-        const int h_tiles = (h + ARROL_MLP_TH - 1) / ARROL_MLP_TH;
-        head_ds_kernel<T><<<1, DS_THREADS, 0, s>>>(nullptr, partial, h_tiles, static_cast<const T*>(head->b2), N,
-                                                   rewards, mask, ds, loss, db2);
-        mlp_du_kernel<T><<<(h + 31) / 32, 256, 0, s>>>(u, ds, static_cast<const T*>(head->w2), N, h, du, nullptr,
-                                                       nullptr, dw2, db1, N);
+        const int rd = launch_du(nullptr, partial, (h + ARROL_MLP_TH - 1) / ARROL_MLP_TH, du, nullptr, nullptr);
+        if (rd != ARROL_OK) return rd;
         dim3 grid((d + GT - 1) / GT, (h + GT - 1) / GT);
         mlp_dw1_kernel<T><<<grid, 128, 0, s>>>(du, hid, row_stride, row_index, N, d, h, dW1);
-        ctx->launches += 3;
+        ctx->launches += 1;
     }
     ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;

@@ -671,31 +671,6 @@ BackwardLayout backward_layout(int64_t T_max, int d, int V) {
 
 }  // namespace
 
-int arrol_internal_gemm_tn(arrol_ctx* ctx, const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N, int K,
-                           float* C, int64_t ldc, int accumulate, cudaStream_t s) {
-    if (M <= 0 || N <= 0 || K <= 0 || lda % 8 != 0 || ldb % 8 != 0) return ARROL_ERR_UNSUPPORTED;
-    if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
-    CUtensorMap map_a, map_b, map_c;
-    if (make_map_f32_tile(ctx, &map_c, C, (uint64_t)M, (uint64_t)N, (uint64_t)ldc) != ARROL_OK) return ARROL_ERR_CUDA;
-    bool a3 = M % 64 == 0, b3 = N % 64 == 0;
-    if (a3 && make_map_mn3d(ctx, &map_a, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM / 64) != ARROL_OK) a3 = false;
-    if (b3 && make_map_mn3d(ctx, &map_b, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BN / 2 / 64) != ARROL_OK) b3 = false;
-    if (!a3 && make_map_ld(ctx, &map_a, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK) != ARROL_OK) return ARROL_ERR_CUDA;
-    if (!b3 && make_map_ld(ctx, &map_b, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BK) != ARROL_OK) return ARROL_ERR_CUDA;
-    GemmParams g = {};
-    g.M = M; g.N = N; g.K = K; g.accumulate = accumulate;
-    // the last words of ctx->d_tile_counters: zeroed before every launch (calls on a context's buffers are ordered by the caller)
-    g.lock_counter = ctx->d_tile_counters + ARROL_SCORE_ROW_TILES;
-    ARROL_CUDA_OK(cudaMemsetAsync(g.lock_counter, 0, sizeof(unsigned int), s));
-    g.a3d = a3; g.b3d = b3; g.T_max = 1; g.d_status = ctx->d_status;
-    const int n_tiles = (N + BN - 1) / BN;
-    g.group_n = group_columns(n_tiles);
-    const int64_t items = (int64_t)((M + TILE_ROWS - 1) / TILE_ROWS) * n_tiles;
-    ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, items, s, map_a, map_b, map_b, map_c, g));
-    ctx->launches += 1;
-    return ARROL_OK;
-}
-
 extern "C" size_t arrol_lm_head_backward_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
     return backward_layout(T_max, d, V).total;

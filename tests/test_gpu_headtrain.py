@@ -49,6 +49,14 @@ def test_head_grad_matches_oracle(N, d, h, dtype, use_mask):
     ctx.close()
 
 
+# the MLP head's tensor-core path at its edges: one rollout, a K step of 64 rollouts and one more, hidden units and columns that do
+# not fill a tile, K split over 1, 2 and 4 blocks, column tiles of 128 (more tiles of 64 than SMs), a run longer than one pass
+@pytest.mark.parametrize("N,d,h", [(1, 64, 8), (64, 72, 136), (65, 200, 128), (300, 264, 264), (1100, 128, 64), (700, 2048, 640),
+                                   (2500, 520, 16)])
+def test_head_grad_at_the_edges_of_its_tiles(N, d, h):
+    test_head_grad_matches_oracle(N, d, h, torch.bfloat16, N % 2 == 0)
+
+
 def test_head_grad_empty_inputs():
     ctx = B.Context(0)
     d = 64
