@@ -8,16 +8,17 @@
 //                         copies into the swizzled stage layout, was built and measured: correct, but the
 //                         load/store path holds about 20 KB in flight per SM against the ring's 192 KB by TMA, and
 //                         every block of a row tile fetches the same rows: 18.5 us per call against 14.6 us.)
-//   score_mlp_tc_kernel   one block per (128 rollouts x 64 hidden units); shared memory is one ring of eight stages
-//                         (128 x 64 of X, 64 x 64 of W1 per K step of 64), filled by two TMA producer threads on
-//                         alternate K steps.  Four MMA issuer threads take the K steps round robin (ks mod 4), each
-//                         into its own 64-column tensor-memory accumulator: one thread's wait -> four MMAs -> commit
-//                         round costs several hundred cycles per K step against the 32 cycles a 128 x 64 x 16 MMA
-//                         keeps the tensor pipe busy, so the loop's length is rounds / issuers.
-//                         Eight epilogue warps: thread = rollout x half of the tile's 64 hidden units; accumulators
-//                         added in index order, then sum_j w2_j gelu(u_j + b1_j) over the 32 units in index order,
-//                         the two halves added low + high -> partial[h_tile][N].  The last block of a row tile to
-//                         finish (a counter per row tile) adds the h tiles in index order, adds b2 and applies the
+//   score_mlp_tc_kernel   one block per (128 rollouts x 64 or 128 hidden units); shared memory is one ring of stages
+//                         (128 x 64 of X and the tile's 64 columns of W1 per K step of 64), filled by two TMA producer threads
+//                         on alternate K steps.  Two (tiles of 128) or four (64) issuing warps take the K steps round robin: one
+//                         warp's wait -> four MMAs -> commit round costs nearly 500 cycles, the MMAs of a 128 x 64 x 64 step
+//                         128, and a step's operands come in in about 290.  K step ks goes to accumulator ks mod 4.  The ring's
+//                         length is a multiple of the number of issuers, so that a stage always belongs to the same one: a parity
+//                         wait cannot tell a round from the one before the last.
+//                         Eight epilogue warps: thread = rollout x half of the tile's hidden units; accumulators added in
+//                         index order, then sum_j w2_j gelu(u_j + b1_j) over 32 units in index order, two such sums added
+//                         low + high -> partial[64-unit block][N], whatever the tile's width.  The last block of a row tile to
+//                         finish (a counter per row tile) adds the partial sums in index order, adds b2 and applies the
 //                         probability map, so the result does not depend on block order.
 // Every wait is bounded; on expiry the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
 #include <cuda.h>
@@ -29,50 +30,47 @@
 
 namespace {
 
-constexpr int SBN = 64;                      // hidden units per tile (MMA N)
-constexpr int S_ISSUERS = 4;                 // MMA issuer threads, each with its own accumulator
+constexpr int SUB_H = 64;                    // hidden units per partial sum: the same for every tile width
+constexpr int S_ACCS = 4;                    // accumulators; K step ks goes to accumulator ks % 4
 constexpr int S_PRODUCERS = 2;               // TMA producer threads (lane 0 of the first warps)
 constexpr int S_PRODUCER_WARPS = 4;          // warps before the issuers (two of them idle: the epilogue warps start at a multiple of 4)
-constexpr int S_EPI_WARP0 = S_PRODUCER_WARPS + S_ISSUERS;      // a multiple of 4: epilogue warp w reads lane quarter w % 4
+constexpr int S_EPI_WARP0 = 8;               // a multiple of 4: epilogue warp w reads lane quarter w % 4
 constexpr int S_EPI_WARPS = 8;
-constexpr int SB_BYTES = SBN * BK * 2;       //  8 KB
-constexpr int S_TMEM_COLS = S_ISSUERS * SBN; // a power of two >= 32
 constexpr int S_THREADS = (S_EPI_WARP0 + S_EPI_WARPS) * 32;
-constexpr int S_TAIL_BYTES = 2048;           // barriers, tensor-memory slot, flags | b1, w2 of the tile | half sums
+constexpr int S_TAIL_BYTES = 2560;           // barriers, tensor-memory slot, flags | b1, w2 of the tile | half sums
 constexpr int TM = 128;                      // rollouts per tile (MMA M)
-constexpr int STAGES = 8;
 constexpr int A_BYTES = TM * BK * 2;         // 16 KB
-constexpr int STAGE_BYTES = A_BYTES + SB_BYTES;
-constexpr size_t S_SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 1024 + S_TAIL_BYTES;
+// by tile width (hidden units, MMA N): 64 or 128
+template <int SBN> __host__ __device__ constexpr int ring_stages() { return SBN == 64 ? 8 : 6; }
+template <int SBN> __host__ __device__ constexpr int issuers() { return SBN == 64 ? 4 : 2; }
+template <int SBN> __host__ __device__ constexpr int stage_bytes() { return A_BYTES + SBN * BK * 2; }
+template <int SBN> __host__ __device__ constexpr size_t smem_bytes() { return (size_t)ring_stages<SBN>() * stage_bytes<SBN>() + 1024 + S_TAIL_BYTES; }
 
-// one warp per rollout: 16-byte copies, all of a row's loads in flight before the first store
+// one warp per 4 KB of a row: 16-byte copies, all of its loads in flight before the first store
+constexpr int PACK_VECS = 256;
 __global__ void __launch_bounds__(128)
 pack_rows_kernel(const __nv_bfloat16* __restrict__ hidden, int64_t row_stride, const int64_t* __restrict__ row_index,
-                 int N, int d, __nv_bfloat16* __restrict__ out, int64_t source_rows, uint32_t* d_status) {
+                 int N, int d, int slices, __nv_bfloat16* __restrict__ out, int64_t source_rows, uint32_t* d_status) {
     pdl_launch_dependents();
     pdl_wait();
     hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index);
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    const int i = w / slices, c0 = (w - i * slices) * PACK_VECS + lane;
     if (i >= N) return;
     const int64_t row = row_index[i];
     const uint4* src = reinterpret_cast<const uint4*>(hidden + row * row_stride);
     uint4* dst = reinterpret_cast<uint4*>(out + (int64_t)i * d);
     const int nvec = d / 8;
-    if (source_rows > 0 && (row < 0 || row >= source_rows)) {   // outside the caller's buffer: never read, packed as zeros
-        if (lane == 0) atomicOr(d_status, ARROL_DEV_BAD_INDEX);
-        for (int c = lane; c < nvec; c += 32) dst[c] = make_uint4(0u, 0u, 0u, 0u);
-        return;
-    }
-    for (int c0 = lane; c0 < nvec; c0 += 256) {
-        uint4 v[8];
+    // outside the caller's buffer: never read, packed as zeros
+    const bool read = !(source_rows > 0 && (row < 0 || row >= source_rows));
+    if (!read && c0 == 0) atomicOr(d_status, ARROL_DEV_BAD_INDEX);
+    uint4 v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (c0 + 32 * u < nvec) v[u] = __ldg(src + c0 + 32 * u);
+    for (int u = 0; u < 8; ++u) v[u] = read && c0 + 32 * u < nvec ? __ldg(src + c0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (c0 + 32 * u < nvec) dst[c0 + 32 * u] = v[u];
-    }
+    for (int u = 0; u < 8; ++u)
+        if (c0 + 32 * u < nvec) dst[c0 + 32 * u] = v[u];
 }
 
 struct ScoreTcParams {
@@ -81,7 +79,7 @@ struct ScoreTcParams {
     const __nv_bfloat16* b1;           // [h] or NULL
     const __nv_bfloat16* w2;           // [h]
     const __nv_bfloat16* b2;           // [1] or NULL
-    float* partial;                    // [h_tiles][N]
+    float* partial;                    // [ceil(h / 64)][N]
     float* u_out;                      // [N][h] pre-activations (bias included) for the head training step, or NULL
     uint32_t* counters;                // [row tiles], zero between calls
     int B;
@@ -93,9 +91,15 @@ struct ScoreTcParams {
     uint32_t* d_status;
 };
 
+template <int SBN>
 __global__ void __launch_bounds__(S_THREADS, 1)
 score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                     const ScoreTcParams p) {
+    constexpr int STAGES = ring_stages<SBN>(), STAGE_BYTES = stage_bytes<SBN>(), SB_BYTES = SBN * BK * 2;
+    constexpr int ISSUERS = issuers<SBN>();
+    static_assert(STAGES % ISSUERS == 0 && S_ACCS % ISSUERS == 0 && STAGES % S_PRODUCERS == 0,
+                  "a stage and an accumulator belong to one issuer, a stage to one producer");
+    constexpr int S_TMEM_COLS = S_ACCS * SBN;                    // a power of two >= 32
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* stage_a = smem;
@@ -109,14 +113,14 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     volatile uint32_t* is_last = tmem_slot + 2;
     float* b1_s = reinterpret_cast<float*>(tail + 256);          // [SBN]
     float* w2_s = b1_s + SBN;                                    // [SBN]
-    float* half_s = reinterpret_cast<float*>(tail + 1024);       // [TM] sums over the tile's upper 32 hidden units
+    float* half_s = reinterpret_cast<float*>(tail + 2048);       // [TM] sums over a 64-unit tile's upper 32 hidden units
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * TM, j0 = blockIdx.y * SBN;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        mbar_init(acc_full, S_ISSUERS);
+        mbar_init(acc_full, ISSUERS);
         *abort_flag = 0u;
         *is_last = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -142,7 +146,7 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    // K step ks uses stage ks % STAGES in round ks / STAGES of the ring and issuer / accumulator ks % S_ISSUERS.
+    // K step ks uses stage ks % STAGES in round ks / STAGES of the ring, issuer ks % ISSUERS and accumulator ks % S_ACCS.
     if (warp < S_PRODUCER_WARPS) {
         if (lane == 0 && warp < S_PRODUCERS) {
             int last = -1;
@@ -163,73 +167,90 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             }
         }
     } else if (warp < S_EPI_WARP0) {
-        if (lane == 0) {
-            const int r = warp - S_PRODUCER_WARPS;
-            const uint32_t d_tmem = tmem_base + (uint32_t)(r * SBN);
+        const int r = warp - S_PRODUCER_WARPS;
+        if (r < ISSUERS) {
+            const uint32_t a0 = smem_u32(stage_a), b0 = smem_u32(stage_b);
             constexpr uint32_t idesc = make_idesc(TM, SBN);
-            for (int ks = r; ks < p.k_steps; ks += S_ISSUERS) {
+            bool ok = true;
+            for (int ks = r; ks < p.k_steps; ks += ISSUERS) {
                 const int st = ks % STAGES;
-                if (!mbar_wait(&full[st], (uint32_t)(ks / STAGES) & 1u, abort_flag)) break;
+                if (!mbar_wait_warp(&full[st], (uint32_t)(ks / STAGES) & 1u, abort_flag)) { ok = false; break; }
                 tcgen05_fence_after();
-                const uint64_t a_desc = make_smem_desc(smem_u32(stage_a + (size_t)st * A_BYTES));
-                const uint64_t b_desc = make_smem_desc(smem_u32(stage_b + (size_t)st * SB_BYTES));
+                const uint64_t a_desc = make_smem_desc(a0 + st * A_BYTES);
+                const uint64_t b_desc = make_smem_desc(b0 + st * SB_BYTES);
+                const uint32_t d_tmem = tmem_base + (uint32_t)((ks % S_ACCS) * SBN);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / UMMA_K; ++k)
-                    tcgen05_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
-                                     (ks >= S_ISSUERS || k > 0) ? 1u : 0u);
-                tcgen05_commit(&empty[st]);
+                    for (int k = 0; k < BK / UMMA_K; ++k)
+                        tcgen05_mma_bf16(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
+                                         (ks >= S_ACCS || k > 0) ? 1u : 0u);
+                    tcgen05_commit(&empty[st]);
+                }
+                __syncwarp();
             }
-            // Arrives once every MMA issued by this thread has finished: publishes the accumulator on the normal
-            // path, and on the give-up path it is what this thread waits for before shared and tensor memory go away.
-            tcgen05_commit(acc_full);
-            if (*abort_flag)
+            // Arrives once every MMA issued by this warp has finished: publishes its accumulators on the normal path, and on the
+            // give-up path it is what this warp waits for before shared and tensor memory go away.
+            if (elect_one()) tcgen05_commit(acc_full);
+            __syncwarp();
+            if (!ok || *abort_flag)
                 for (uint32_t it = 0; it < SPIN_LIMIT; ++it)
                     if (mbar_try_wait(acc_full, 0u)) break;
         }
     } else {
         const int quarter = warp & 3;                           // accumulator row r is tensor-memory lane r
-        const int half = (warp - S_EPI_WARP0) >> 2;             // which 32 of the tile's 64 hidden units
+        const int half = (warp - S_EPI_WARP0) >> 2;             // which half of the tile's hidden units
         const int r_tile = quarter * 32 + lane;
         const int m = m0 + r_tile;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        const int used_accs = p.k_steps < S_ISSUERS ? p.k_steps : S_ISSUERS;   // an issuer without K steps wrote nothing
+        const int used_accs = p.k_steps < S_ACCS ? p.k_steps : S_ACCS;         // an accumulator without K steps holds nothing
         bool ok = mbar_wait(acc_full, 0u, abort_flag);
         ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
-        float part = 0.f;
-        if (ok) {
-            tcgen05_fence_after();
+        // sum_j w2_j gelu(u_j + b1_j) over 32 hidden units in index order; two of these, low + high, make a partial sum
+        auto units32 = [&](int j32) {
+            float part = 0.f;
             float v[32];
-            tcgen05_ld_32x32(tmem_base + lane_addr + half * 32, v);
+            tcgen05_ld_32x32(tmem_base + lane_addr + j32, v);
             for (int a = 1; a < used_accs; ++a) {      // fixed order: ((acc0 + acc1) + acc2) + acc3
                 float w[32];
-                tcgen05_ld_32x32(tmem_base + lane_addr + a * SBN + half * 32, w);
+                tcgen05_ld_32x32(tmem_base + lane_addr + a * SBN + j32, w);
 #pragma unroll
                 for (int jj = 0; jj < 32; ++jj) v[jj] += w[jj];
             }
 #pragma unroll
             for (int jj = 0; jj < 32; ++jj) {
-                const float u = v[jj] + b1_s[half * 32 + jj];
+                const float u = v[jj] + b1_s[j32 + jj];
                 v[jj] = u;
                 const float g = 0.5f * u * (1.0f + erff(u * 0.70710678118654752440f));
-                part = fmaf(w2_s[half * 32 + jj], g, part);
+                part = fmaf(w2_s[j32 + jj], g, part);
             }
             if (p.u_out && m < p.N) {
-                float* urow = p.u_out + (int64_t)m * p.h + j0 + half * 32;
+                float* urow = p.u_out + (int64_t)m * p.h + j0 + j32;
 #pragma unroll
                 for (int jj = 0; jj < 32; jj += 4)      // h % 4 == 0: a float4 never straddles the edge
-                    if (j0 + half * 32 + jj < p.h)
+                    if (j0 + j32 + jj < p.h)
                         *reinterpret_cast<float4*>(urow + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
             }
+            return part;
+        };
+        float part = 0.f;
+        if (ok) {
+            tcgen05_fence_after();
+            part = units32(half * (SBN / 2));
+            if constexpr (SBN == 128) part += units32(half * 64 + 32);
         }
-        if (half == 1) half_s[r_tile] = part;
-        asm volatile("bar.sync 2, 256;" ::: "memory");
-        if (half == 0) {
-            part += half_s[r_tile];                             // low half + high half
+        if constexpr (SBN == 64) {
+            if (half == 1) half_s[r_tile] = part;
+            asm volatile("bar.sync 2, 256;" ::: "memory");
+        }
+        if (SBN == 128 || half == 0) {
+            constexpr int PARTS = SBN == 128 ? 256 : 128;       // threads that hold a partial sum
+            if constexpr (SBN == 64) part += half_s[r_tile];    // low half + high half
+            const int sub = (int)blockIdx.y * (SBN / SUB_H) + (SBN == 128 ? half : 0);
             // The counter protocol runs whatever happened above, so the counters are back at zero after every launch
             // (after an expired wait the scores of the call are not meaningful and the status word says so).
-            if (m < p.N) p.partial[(int64_t)blockIdx.y * p.N + m] = part;
+            if (m < p.N && sub * SUB_H < p.h) p.partial[(int64_t)sub * p.N + m] = part;
             __threadfence();
-            asm volatile("bar.sync 1, 128;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
             if (threadIdx.x == S_EPI_WARP0 * 32) {
                 const uint32_t done = atomicAdd(&p.counters[blockIdx.x], 1u);
                 if (done == gridDim.y - 1) {
@@ -237,11 +258,11 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                     p.counters[blockIdx.x] = 0u;    // every block of this row tile has arrived: ready for the next call
                 }
             }
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            if (*is_last && m < p.N) {
+            asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
+            if (*is_last && half == 0 && m < p.N) {
                 __threadfence();
                 float s = 0.f;
-                for (int t = 0; t < (int)gridDim.y; ++t) s += __ldcg(&p.partial[(int64_t)t * p.N + m]);
+                for (int t = 0; t * SUB_H < p.h; ++t) s += __ldcg(&p.partial[(int64_t)t * p.N + m]);
                 if (p.b2) s += __bfloat162float(p.b2[0]);
                 probability_map(s, m, p.B, p.q_lut, p.score, p.prob, p.bin, p.q);
             }
@@ -266,9 +287,9 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
                                 int N, const arrol_head* head, int B, const float* q_lut, float* score, float* prob,
                                 int32_t* bin, float* q, float* u_out, cudaStream_t s) {
     const int d = head->d, h = head->h;
-    const int h_tiles = (h + SBN - 1) / SBN;
+    const int subs = (h + SUB_H - 1) / SUB_H;
     const int m_tiles = (N + TM - 1) / TM;
-    if ((size_t)N * (size_t)h_tiles > ARROL_SCRATCH_FLOATS || m_tiles > ARROL_SCORE_ROW_TILES)
+    if ((size_t)N * (size_t)subs > ARROL_SCRATCH_FLOATS || m_tiles > ARROL_SCORE_ROW_TILES)
         return ARROL_ERR_UNSUPPORTED;
     const bool pack = row_index != nullptr;
     if (pack && (size_t)N * (size_t)d * 2 > ARROL_PACK_BYTES) return ARROL_ERR_UNSUPPORTED;
@@ -277,15 +298,21 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     const void* x = hidden;
     int64_t ld = row_stride;
     if (pack) {
-        ARROL_CUDA_OK(arrol_launch_pdl(pack_rows_kernel, dim3((N + 3) / 4), dim3(128), 0, s,
-                                       static_cast<const __nv_bfloat16*>(hidden), row_stride, row_index, N, d,
+        const int slices = (d / 8 + PACK_VECS - 1) / PACK_VECS;
+        ARROL_CUDA_OK(arrol_launch_pdl(pack_rows_kernel, dim3((unsigned)(((int64_t)N * slices + 3) / 4)), dim3(128), 0, s,
+                                       static_cast<const __nv_bfloat16*>(hidden), row_stride, row_index, N, d, slices,
                                        static_cast<__nv_bfloat16*>(ctx->d_pack), ctx->source_rows, ctx->d_status));
         ctx->launches += 1;
         x = ctx->d_pack;
         ld = d;
     }
+    // Tiles of 64 hidden units while they fit one wave of blocks (more SMs share the way in for the operands), of 128 beyond
+    // that (a third fewer operand bytes and half as many blocks); the bits are the same.  Without / with the wide tiles:
+    // N = 4,096, d = 4,096, h = 512 39.0 -> 28.4 us (8 of them the packing), N = 8,192 80.7 -> 64.7, N = 3,000, d = 1,024
+    // 17.1 -> 14.6; within one wave they lose: N = 2,048, d = 2,048, h = 256 14.2 -> 15.1.
+    const bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
     CUtensorMap map_x, map_w;
-    if (make_map(ctx, &map_w, head->W1, (uint64_t)h, (uint64_t)d, SBN) != ARROL_OK) return ARROL_ERR_CUDA;
+    if (make_map(ctx, &map_w, head->W1, (uint64_t)h, (uint64_t)d, wide ? 128 : 64) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map_ld(ctx, &map_x, x, (uint64_t)N, (uint64_t)d, (uint64_t)ld, TM) != ARROL_OK) return ARROL_ERR_CUDA;
 
     ScoreTcParams p;
@@ -305,13 +332,16 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     p.bin = bin;
     p.q = q;
     p.d_status = ctx->d_status;
-    dim3 grid(m_tiles, h_tiles);
     if (!ctx->score_tc_smem_set) {      // once per context: this call is on the prune step's microsecond path
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)S_SMEM_BYTES));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
         ctx->score_tc_smem_set = true;
     }
-    ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tc_kernel, grid, dim3(S_THREADS), S_SMEM_BYTES, s, map_x, map_w, p));
+    if (wide)
+        ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tc_kernel<128>, dim3(m_tiles, (h + 127) / 128), dim3(S_THREADS), smem_bytes<128>(), s,
+                                       map_x, map_w, p));
+    else
+        ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tc_kernel<64>, dim3(m_tiles, subs), dim3(S_THREADS), smem_bytes<64>(), s, map_x, map_w, p));
     ctx->launches += 1;
     return ARROL_OK;
 }

@@ -114,6 +114,22 @@ def test_mlp_head_larger_than_the_packing_buffer_takes_the_simt_path(ctx):
     _score_case(ctx, 8448, 4096, 64, torch.bfloat16, True, False, seed=4)     # same size, rows in place
 
 
+# more 128 x 64 tiles than SMs: tiles of 128 hidden units, the last of them partly or wholly past h, one to nine K steps
+@pytest.mark.parametrize("N,d,h", [(9600, 64, 72), (5000, 520, 260), (9500, 328, 128), (19001, 136, 136)])
+def test_mlp_head_scores_do_not_depend_on_how_many_rollouts_are_scored(ctx, N, d, h):
+    _score_case(ctx, N, d, h, torch.bfloat16, True, True, seed=N)
+    g = torch.Generator().manual_seed(N)
+    mk = lambda *s: (torch.randn(s, generator=g) * 0.1).to(torch.bfloat16).cuda()
+    x, head = mk(N, d), {"W1": mk(h, d), "b1": mk(h), "w2": mk(h), "b2": mk(1), "h": h}
+    out = []
+    for n in (N, 130):                                            # the second call's tiles fit one wave: tiles of 64
+        o = [torch.full((n,), 7.0, device="cuda") for _ in range(3)]
+        B.arrol_score_partial(ctx, x, head, n, *o)
+        out.append(o)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a[:130], b) for a, b in zip(*out))
+
+
 def test_mlp_head_strided_rows_without_index(ctx):
     """Evenly strided rows (a column slice of a wider buffer) go to the tensor-core path without packing."""
     g = np.random.default_rng(5)
