@@ -128,15 +128,18 @@ gather_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_
 }
 
 // Per-token outputs without a payload plane (token ids, survivor ordinal, advantage): one block per survivor walks
-// its run of tokens with coalesced 4-byte accesses, so nothing has to be searched.  Blocks past S return at once.
-constexpr int TOKENS_THREADS = 128;
-constexpr int TOKENS_PER_THREAD = 16;   // token ids in flight per thread (4: 28.7 us, 8: 26.4, 16: 24.6 for the Qwen-3-4B-shaped step)
+// its run of tokens, so nothing has to be searched.  Blocks past S return at once.  Bound by the bytes it moves (16 per
+// token, 12 of them written): all three outputs leave as 16-byte stores, four tokens per thread.  The source run is aligned
+// differently from the destination, so a thread reads the two aligned 16-byte words that hold its four ids (the second one
+// is its neighbour's first, in L1 by then) and picks them out.  FIGURES_TOKENS
+constexpr int TOKENS_THREADS = 256;
+constexpr int TOKENS_QUADS = 4;          // groups of four tokens in flight per thread
 __global__ void __launch_bounds__(TOKENS_THREADS)
 gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_seqlens,
                      const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off,
                      const int32_t* __restrict__ src_tokens, const float* __restrict__ adv, int64_t capacity,
                      int32_t* __restrict__ dst_tokens, float* __restrict__ tok_adv, int32_t* __restrict__ tok_seq,
-                     const uint32_t* __restrict__ gate) {
+                     const uint32_t* __restrict__ gate, int vector_stores) {
     pdl_launch_dependents();
     pdl_wait();
     d_num = pdl_acquire(d_num); cu_seqlens = pdl_acquire(cu_seqlens); survivor_idx = pdl_acquire(survivor_idx);
@@ -149,21 +152,50 @@ gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restric
         const int len = (int)(__ldg(cu_seqlens + s + 1) - c0);
         const int64_t src0 = __ldg(src_tok_off + __ldg(survivor_idx + s));
         const float a = __ldg(adv + s);
-        for (int t0 = threadIdx.x; t0 < len; t0 += TOKENS_PER_THREAD * TOKENS_THREADS) {
-            int32_t tok[TOKENS_PER_THREAD];
+        auto one = [&](int t) {
+            if (dst_tokens) dst_tokens[c0 + t] = __ldg(src_tokens + src0 + t);
+            if (tok_seq) tok_seq[c0 + t] = s;
+            if (tok_adv) tok_adv[c0 + t] = a;
+        };
+        // up to three tokens before the first 16-byte boundary of the outputs, then groups of four, then up to three
+        const int head = vector_stores ? min(len, (int)((4 - (c0 & 3)) & 3)) : len;
+        const int quads = (len - head) / 4;
+        for (int t = threadIdx.x; t < head; t += TOKENS_THREADS) one(t);
+        if ((int)threadIdx.x < (vector_stores ? len - head - 4 * quads : 0)) one(head + 4 * quads + threadIdx.x);
+        const int32_t* src = src_tokens + src0 + head;
+        const int shift = (int)((reinterpret_cast<uintptr_t>(src) & 15) >> 2);      // ids before src in its 16-byte word
+        const int4* words = reinterpret_cast<const int4*>(src - shift);
+        // both words lie inside the run: nothing outside the rollout's own ids is read
+        auto whole_words = [&](int k) { return shift == 0 || (head + 4 * k >= shift && head + 4 * k - shift + 8 <= len); };
+        for (int k0 = threadIdx.x; k0 < quads; k0 += TOKENS_QUADS * TOKENS_THREADS) {
+            int4 lo[TOKENS_QUADS], hi[TOKENS_QUADS];
 #pragma unroll
-            for (int u = 0; u < TOKENS_PER_THREAD; ++u) {
-                const int t = t0 + u * TOKENS_THREADS;
-                if (dst_tokens && t < len) tok[u] = __ldg(src_tokens + src0 + t);
+            for (int u = 0; u < TOKENS_QUADS; ++u) {
+                const int k = k0 + u * TOKENS_THREADS;
+                if (dst_tokens && k < quads) {
+                    if (whole_words(k)) {
+                        lo[u] = __ldg(words + k);
+                        if (shift) hi[u] = __ldg(words + k + 1);
+                    } else {
+                        lo[u] = make_int4(__ldg(src + 4 * k), __ldg(src + 4 * k + 1), __ldg(src + 4 * k + 2), __ldg(src + 4 * k + 3));
+                    }
+                }
             }
 #pragma unroll
-            for (int u = 0; u < TOKENS_PER_THREAD; ++u) {
-                const int t = t0 + u * TOKENS_THREADS;
-                if (t < len) {
-                    if (dst_tokens) dst_tokens[c0 + t] = tok[u];
-                    if (tok_seq) tok_seq[c0 + t] = s;
-                    if (tok_adv) tok_adv[c0 + t] = a;
+            for (int u = 0; u < TOKENS_QUADS; ++u) {
+                const int k = k0 + u * TOKENS_THREADS;
+                if (k >= quads) break;
+                const int64_t at = c0 + head + 4 * k;
+                if (dst_tokens) {
+                    int4 v = lo[u];
+                    const int by = whole_words(k) ? shift : 0;
+                    if (by == 1) v = make_int4(lo[u].y, lo[u].z, lo[u].w, hi[u].x);
+                    else if (by == 2) v = make_int4(lo[u].z, lo[u].w, hi[u].x, hi[u].y);
+                    else if (by == 3) v = make_int4(lo[u].w, hi[u].x, hi[u].y, hi[u].z);
+                    *reinterpret_cast<int4*>(dst_tokens + at) = v;
                 }
+                if (tok_seq) *reinterpret_cast<int4*>(tok_seq + at) = make_int4(s, s, s, s);
+                if (tok_adv) *reinterpret_cast<float4*>(tok_adv + at) = make_float4(a, a, a, a);
             }
         }
     }
@@ -232,7 +264,9 @@ int arrol_internal_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* l
         int64_t blocks = N < (int64_t)ctx->sm_count * 16 ? N : (int64_t)ctx->sm_count * 16;
         ARROL_CUDA_OK(arrol_launch_pdl(gather_tokens_kernel, dim3((unsigned)blocks), dim3(TOKENS_THREADS), 0, s, d_num,
                                        cu_seqlens, survivor_idx, src_tok_off, src_tokens, adv, dst_capacity_tokens,
-                                       dst_tokens, tok_adv, tok_seq, ctx->d_status + 1));
+                                       dst_tokens, tok_adv, tok_seq, ctx->d_status + 1,
+                                       arrol_aligned(dst_tokens, 16) && arrol_aligned(tok_adv, 16) && arrol_aligned(tok_seq, 16) &&
+                                               arrol_aligned(src_tokens, 4) ? 1 : 0));
         ctx->launches += 1;
         return ARROL_OK;
     }

@@ -81,7 +81,8 @@ struct PartialLse {   // of one token over some columns: running maximum and sum
 // into a block, block by block into a group, then group by group, by whichever kernel holds them.
 struct VocabPlan {
     int total_chunks, n_sub, n_mid, splits;
-    __host__ __device__ int chunk_of_sub(int i) const { return (int)((int64_t)i * total_chunks / n_sub); }
+    // n_sub <= SMs and total_chunks < 2^23: the product stays below 2^31 for any vocabulary that a TMA coordinate reaches
+    __host__ __device__ int chunk_of_sub(int i) const { return (int)((unsigned)i * (unsigned)total_chunks / (unsigned)n_sub); }
     __host__ __device__ int sub_of_mid(int i) const { return i * n_sub / n_mid; }
     __host__ __device__ int mid_of_group(int g) const { return g * n_mid / splits; }
     __host__ __device__ int sub_of_group(int g) const { return sub_of_mid(mid_of_group(g)); }
@@ -102,42 +103,41 @@ __device__ __forceinline__ void merge_record(PartialLse& a, const PartialLse& b)
 }
 __device__ __forceinline__ PartialLse empty_record() { return PartialLse{-INFINITY, 0.f, -INFINITY, 0.f}; }
 
-// Work of one launch on `tiles` token tiles (128 rows, or 256 for a pair of blocks).
+// Work of one launch on `tiles` token tiles (128 rows, or 256 for a pair of blocks).  32-bit throughout (fewer than 2^24 tiles
+// and at most 64 groups): the divisions are on the way of every work item and of the combining kernel.
 struct WorkList {
-    int64_t body_tiles, body_items, tail_items, waves;   // waves: those of the body, plus one for the tail
-    int tail_tiles;                                      // at most units / splits + 1
-};
-__host__ __device__ inline WorkList make_work_list(int64_t tiles, int64_t units, const VocabPlan& v) {
+    int body_tiles, body_items, tail_tiles, tail_items, waves;   // tail_tiles: at most units / splits + 1;  waves: those of the
+};                                                               // body, plus one for the tail
+__host__ __device__ inline WorkList make_work_list(int tiles, int units, const VocabPlan& v) {
     WorkList w;
     w.body_tiles = tiles * v.splits / units * units / v.splits;    // whole waves only
     w.body_items = w.body_tiles * v.splits;
-    w.tail_tiles = (int)(tiles - w.body_tiles);
-    w.tail_items = (int64_t)w.tail_tiles * v.n_sub;
+    w.tail_tiles = tiles - w.body_tiles;
+    w.tail_items = w.tail_tiles * v.n_sub;
     w.waves = (w.body_items + units - 1) / units + (w.tail_items > 0 ? 1 : 0);
     return w;
 }
 struct WorkItem {
-    int64_t tile, wave;
+    int tile, wave;
     int group, sub0, sub1;      // group < 0: a tail item
 };
 // k-th item of a unit; false when it has none left.  The tail walks the segments as the slow index: at any time the
 // units work on neighbouring segments of all tail tiles and share W_vocab through L2.
-__device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v, int64_t unit, int64_t units, int64_t k,
-                                          WorkItem& it) {
-    int64_t i = unit + k * units;               // body items, then tail items, in one numbering
+__device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v, int unit, int units, int k, WorkItem& it) {
+    int i = unit + k * units;                   // body items, then tail items, in one numbering
     it.wave = k < w.waves ? k : w.waves - 1;
     if (i < w.body_items) {
         it.tile = i / v.splits;
-        it.group = (int)(i - it.tile * v.splits);
+        it.group = i - it.tile * v.splits;
         it.sub0 = v.sub_of_group(it.group);
         it.sub1 = v.sub_of_group(it.group + 1);
         return true;
     }
     i -= w.body_items;
     if (i >= w.tail_items) return false;
-    it.sub0 = (int)(i / w.tail_tiles);
+    it.sub0 = i / w.tail_tiles;
     it.sub1 = it.sub0 + 1;
-    it.tile = w.body_tiles + (i - (int64_t)it.sub0 * w.tail_tiles);
+    it.tile = w.body_tiles + (i - it.sub0 * w.tail_tiles);
     it.group = -1;
     return true;
 }
@@ -256,8 +256,8 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // pair: rank of this block in its cluster (block 0 leads), unit = cluster; otherwise unit = block
     const uint32_t rank = PAIR ? cluster_cta_rank() : 0u;
-    const int64_t unit = PAIR ? (int64_t)(blockIdx.x >> 1) : (int64_t)blockIdx.x;
-    const int64_t units = PAIR ? (int64_t)(gridDim.x >> 1) : (int64_t)gridDim.x;
+    const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int units = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
 
     const int k_steps = (p.d + BK - 1) / BK;
 
@@ -291,7 +291,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
     pdl_wait();                    // the set-up above overlaps the end of the preceding kernel
     int64_t T = p.T_max;
     if (p.d_T) { const int64_t t = *pdl_acquire(p.d_T); T = t < 0 ? 0 : (t < T ? t : T); }
-    const int64_t m_tiles = (T + BM - 1) / BM;
+    const int m_tiles = (int)((T + BM - 1) / BM);
     const WorkList work = make_work_list(PAIR ? (m_tiles + 1) / 2 : m_tiles, units, p.plan);
 
     if (warp == 0) {
@@ -303,17 +303,17 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
             const int32_t* tile_row = pdl_acquire(p.tile_row);
             // first of the 128 source rows of this block's tile (gathered variant; requested one item ahead)
             auto source_row = [&](const WorkItem& it) {
-                return tile_row[PAIR ? 2 * it.tile + (int64_t)rank : it.tile];
+                return tile_row[PAIR ? 2 * it.tile + (int)rank : it.tile];
             };
             WorkItem it, next;
             bool have = !p.mute_producer && work_item(work, p.plan, unit, units, 0, it);
             int row = 0;
             if constexpr (GATHER) if (have) row = source_row(it);
-            int64_t arrived = 0, waited = 0;        // waves
-            for (int64_t k = 0; !p.mute_producer; ++k) {
+            int arrived = 0, waited = 0;            // waves
+            for (int k = 0; !p.mute_producer; ++k) {
                 // hold the blocks in step: arrive for the item's wave (one arrival per unit and wave), then wait for
                 // everybody; a unit without an item in a partial wave arrives as well
-                const int64_t wave = have ? it.wave : work.waves - 1;
+                const int wave = have ? it.wave : work.waves - 1;
                 for (; arrived < wave; ++arrived)
                     if (rank == 0) { __threadfence(); atomicAdd(p.wave_counter, 1u); }
                 if (!have) break;
@@ -333,7 +333,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                 const int c0 = p.plan.chunk_of_sub(it.sub0), c1 = p.plan.chunk_of_sub(it.sub1);
                 // where the tile's 128 rows come from: the packed rows, a run of source rows, or a scratch slot
                 const CUtensorMap* a_map = &map_h;
-                int a_row = (int)(PAIR ? 2 * it.tile + (int64_t)rank : it.tile) * BM;
+                int a_row = (PAIR ? 2 * it.tile + (int)rank : it.tile) * BM;
                 if constexpr (GATHER) {
                     a_row = row;
                     if (row < 0) { a_map = &map_s; a_row = ~row; }
@@ -390,7 +390,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
             uint32_t acc = 0, acc_phase = 0;
             bool ok = true;
             WorkItem it;
-            for (int64_t k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
+            for (int k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
                 const int c0 = p.plan.chunk_of_sub(it.sub0), c1 = p.plan.chunk_of_sub(it.sub1);
                 for (int c = c0; c < c1 && ok; ++c) {
                     const uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, chunk_columns(p.V, c));
@@ -452,11 +452,11 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
         WorkItem it;
-        for (int64_t k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
-            const int64_t t = (PAIR ? 2 * it.tile + (int64_t)rank : it.tile) * BM + row_in_tile;
+        for (int k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
+            const int64_t t = (int64_t)(PAIR ? 2 * it.tile + (int)rank : it.tile) * BM + row_in_tile;
             const int y = (t < T) ? targets[t] : -1;
             PartialLse sub = empty_record(), mid = empty_record(), group = empty_record();
-            const int64_t stamp_at = it.tile * p.plan.splits + it.group;
+            const int64_t stamp_at = (int64_t)it.tile * p.plan.splits + it.group;
             const bool stamp = p.timing != nullptr && threadIdx.x == 64 && rank == 0 && it.group >= 0 && stamp_at < p.timing_items;
             if (stamp) { p.timing[4 * stamp_at] = global_timer_ns(); p.timing[4 * stamp_at + 2] = (unsigned long long)clock64(); }
             int mid_i = it.group >= 0 ? p.plan.mid_of_group(it.group) : 0;
@@ -502,7 +502,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                 if (it.group >= 0) {
                     dst = p.body + ((int64_t)it.group * HALVES + half) * p.T_max + t;
                 } else {
-                    const int64_t tail_row = t - work.body_tiles * ((PAIR ? 2 : 1) * BM);
+                    const int64_t tail_row = t - (int64_t)work.body_tiles * ((PAIR ? 2 : 1) * BM);
                     dst = p.tail + (tail_row * p.plan.n_sub + it.sub0) * HALVES + half;
                 }
                 *reinterpret_cast<float4*>(dst) = make_float4(r.m2, r.l, r.zy2, r.sumz);
@@ -593,14 +593,14 @@ constexpr int COMBINE_THREADS = 256;
 template <int HALVES>
 __global__ void __launch_bounds__(COMBINE_THREADS)
 combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
-                      int64_t T_max, int V, VocabPlan plan, int tile_rows, int64_t units, float* __restrict__ logp,
+                      int64_t T_max, int V, VocabPlan plan, int tile_rows, int units, float* __restrict__ logp,
                       float* __restrict__ lse, float* __restrict__ conf, float inv_temp, uint32_t* d_status) {
     pdl_wait();
     body = pdl_acquire(body); tail = pdl_acquire(tail); targets = pdl_acquire(targets); d_T = pdl_acquire(d_T);
     int64_t T = T_max;
     if (d_T) { const int64_t t = *d_T; T = t < 0 ? 0 : (t < T ? t : T); }
-    const WorkList work = make_work_list((T + tile_rows - 1) / tile_rows, units, plan);
-    const int64_t body_rows = min(T, work.body_tiles * tile_rows);
+    const WorkList work = make_work_list((int)(((unsigned)T + tile_rows - 1) / (unsigned)tile_rows), units, plan);   // T < 2^31
+    const int64_t body_rows = min(T, (int64_t)work.body_tiles * tile_rows);
     auto load = [](const PartialLse* p) {
         const float4 r = *reinterpret_cast<const float4*>(p);
         return PartialLse{r.x, r.y, r.z, r.w};
@@ -638,7 +638,7 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
         PartialLse total[HALVES], group[HALVES];
 #pragma unroll
         for (int h = 0; h < HALVES; ++h) total[h] = group[h] = empty_record();
-        int g = 0;
+        int g = 0, group_end = plan.mid_of_group(1);
         for (int base = 0; base < plan.n_mid; base += COMBINE_BLOCKS) {
             const int b = base + lane / HALVES;
             PartialLse mine = empty_record();
@@ -648,6 +648,7 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
                 for (int s = plan.sub_of_mid(b); s < s1; ++s) merge_record(mine, load(rec + s * HALVES + lane % HALVES));
             }
             const int in_base = min(COMBINE_BLOCKS, plan.n_mid - base);
+#pragma unroll 4
             for (int j = 0; j < in_base; ++j) {
 #pragma unroll
                 for (int h = 0; h < HALVES; ++h) {
@@ -655,10 +656,11 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
                     merge_record(group[h], PartialLse{__shfl_sync(0xffffffffu, mine.m2, from), __shfl_sync(0xffffffffu, mine.l, from),
                                                       __shfl_sync(0xffffffffu, mine.zy2, from), __shfl_sync(0xffffffffu, mine.sumz, from)});
                 }
-                if (base + j + 1 == plan.mid_of_group(g + 1)) {
+                if (base + j + 1 == group_end) {
 #pragma unroll
                     for (int h = 0; h < HALVES; ++h) { merge_record(total[h], group[h]); group[h] = empty_record(); }
                     ++g;
+                    group_end = plan.mid_of_group(g + 1);
                 }
             }
         }
@@ -873,7 +875,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     if (units > tiles_max * p.plan.n_sub) units = tiles_max * p.plan.n_sub;
     const int64_t grid = pair ? 2 * units : units;
     // more than one wave: the blocks wait for one another, so they must all be resident (single blocks: cooperative launch)
-    const bool several_waves = make_work_list(tiles_max, units, p.plan).waves > 1;
+    const bool several_waves = make_work_list((int)tiles_max, (int)units, p.plan).waves > 1;
     if (several_waves) ARROL_CUDA_OK(cudaMemsetAsync(p.wave_counter, 0, sizeof(unsigned int), s));
     if (several_waves && !pair) {
         attr[n_attr].id = cudaLaunchAttributeCooperative;
@@ -906,7 +908,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
     ARROL_CUDA_OK(arrol_launch_pdl(halves == 2 ? combine_splits_kernel<2> : combine_splits_kernel<1>, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
                                    static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
-                                   T_max, V, p.plan, (int)tile_rows, units, logp, lse, conf, inv_temperature, ctx->d_status));
+                                   T_max, V, p.plan, (int)tile_rows, (int)units, logp, lse, conf, inv_temperature, ctx->d_status));
     ctx->launches += 1;
     return ARROL_OK;
 }
