@@ -123,6 +123,17 @@ def load_library():
     lib.arrol_prune_step.restype = C.c_int
     lib.arrol_launch_count.argtypes = [C.c_void_p]
     lib.arrol_launch_count.restype = C.c_int64
+    for fn, res, args in (
+            ("arrol_token_logprob_form", C.c_int32, [C.c_void_p, C.c_int64, C.c_int32, C.c_int32]),
+            ("arrol_token_logprob_splits", C.c_int32, [C.c_void_p, C.c_int64, C.c_int32, C.c_int32]),
+            ("arrol_token_logprob_gathered_workspace", C.c_size_t, [C.c_void_p, C.c_int32, C.c_int64, C.c_int32, C.c_int32]),
+            ("arrol_token_logprob_gathered", C.c_int, lib.arrol_token_logprob_gathered.argtypes),
+            ("arrol_test_hook", C.c_int, [C.c_void_p, C.c_int32, C.c_int64]),
+            ("arrol_set_source_rows", C.c_int, [C.c_void_p, C.c_int64]),
+            ("arrol_rank_vote", C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p,
+                                          C.c_void_p, C.c_void_p])):
+        getattr(lib, fn).restype = res
+        getattr(lib, fn).argtypes = args
     for fn in ("arrol_create", "arrol_destroy", "arrol_poll_status", "arrol_calib_counts", "arrol_build_q_lut",
                "arrol_score_partial", "arrol_select", "arrol_compact", "arrol_token_logprob"):
         getattr(lib, fn).restype = C.c_int
@@ -143,13 +154,17 @@ def _check(code: int, where: str):
         raise ArrolError(code, where)
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+# Small calls are bound by the host, so the marshalling is kept lean: plain integers for pointers and streams (the argument
+# types are set once, when the library is loaded), structures filled in one constructor call, and the current stream's handle
+# asked for directly (a torch.cuda.Stream object costs 3 us, half of what a whole call should).
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+def _stream(stream=None) -> int:
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -217,23 +232,29 @@ def arrol_build_q_lut(cpos, cneg, alpha: float = 1.0):
     return q
 
 
+_HEAD_TENSORS = ("W1", "b1", "w2", "b2")
+
+
+def _head_struct(hidden_dtype_code: int, d: int, head: dict) -> _Head:
+    return _Head(int(d), int(head.get("h", 0)), hidden_dtype_code, 0, *[_ptr(head.get(name)) for name in _HEAD_TENSORS])
+
+
+def _calib_struct(q_lut: Optional[torch.Tensor]) -> _Calib:
+    return _Calib() if q_lut is None else _Calib(q_lut.shape[0], 0, q_lut.data_ptr())
+
+
 def arrol_score_partial(ctx: Context, hidden: torch.Tensor, head: dict, N: int, score: torch.Tensor,
                         prob: torch.Tensor, q: torch.Tensor, bin: Optional[torch.Tensor] = None,
                         row_index: Optional[torch.Tensor] = None, q_lut: Optional[torch.Tensor] = None,
                         row_stride: Optional[int] = None, stream=None):
     """head = {"W1", "b1", "w2", "b2", "h"} (device tensors or None).  Outputs are written in place."""
-    hs = _Head()
-    hs.d = hidden.shape[-1]
-    hs.h = int(head.get("h", 0))
-    hs.dtype = _dtype_code(hidden)
-    for name in ("W1", "b1", "w2", "b2"):
+    dtype = hidden.dtype
+    for name in _HEAD_TENSORS:
         t = head.get(name)
-        if t is not None and t.dtype != hidden.dtype:
+        if t is not None and t.dtype != dtype:
             raise TypeError("head tensors share the hidden dtype")
-        setattr(hs, name, None if t is None else t.data_ptr())
-    cs = _Calib()
-    cs.B = 0 if q_lut is None else q_lut.shape[0]
-    cs.q_lut = None if q_lut is None else q_lut.data_ptr()
+    hs = _head_struct(_dtype_code(hidden), hidden.shape[-1], head)
+    cs = _calib_struct(q_lut)
     stride = hidden.stride(-2) if row_stride is None else int(row_stride)
     _check(load_library().arrol_score_partial(ctx.handle, _ptr(hidden), stride, _ptr(row_index), int(N),
                                               C.byref(hs), C.byref(cs), _ptr(score), _ptr(prob), _ptr(bin),
@@ -264,17 +285,11 @@ def arrol_token_logprob_workspace(ctx: Context, T_max: int, d: int, V: int) -> i
 
 def arrol_token_logprob_form(ctx: Context, T_max: int, d: int, V: int) -> int:
     """2 = the kernel runs as pairs of blocks on 256-row tiles for these sizes, 1 = one block per 128-row tile."""
-    lib = load_library()
-    lib.arrol_token_logprob_form.restype = C.c_int32
-    lib.arrol_token_logprob_form.argtypes = [C.c_void_p, C.c_int64, C.c_int32, C.c_int32]
-    return int(lib.arrol_token_logprob_form(ctx.handle, int(T_max), int(d), int(V)))
+    return int(load_library().arrol_token_logprob_form(ctx.handle, int(T_max), int(d), int(V)))
 
 
 def arrol_token_logprob_splits(ctx: Context, T_max: int, d: int, V: int) -> int:
-    lib = load_library()
-    lib.arrol_token_logprob_splits.restype = C.c_int32
-    lib.arrol_token_logprob_splits.argtypes = [C.c_void_p, C.c_int64, C.c_int32, C.c_int32]
-    return int(lib.arrol_token_logprob_splits(ctx.handle, int(T_max), int(d), int(V)))
+    return int(load_library().arrol_token_logprob_splits(ctx.handle, int(T_max), int(d), int(V)))
 
 
 def arrol_token_logprob(ctx: Context, hidden, W_vocab, targets, T_max: int, d: int, V: int, logp, workspace,
@@ -287,10 +302,7 @@ def arrol_token_logprob(ctx: Context, hidden, W_vocab, targets, T_max: int, d: i
 
 
 def arrol_token_logprob_gathered_workspace(ctx: Context, S_max: int, T_max: int, d: int, V: int) -> int:
-    lib = load_library()
-    lib.arrol_token_logprob_gathered_workspace.restype = C.c_size_t
-    lib.arrol_token_logprob_gathered_workspace.argtypes = [C.c_void_p, C.c_int32, C.c_int64, C.c_int32, C.c_int32]
-    return int(lib.arrol_token_logprob_gathered_workspace(ctx.handle, int(S_max), int(T_max), int(d), int(V)))
+    return int(load_library().arrol_token_logprob_gathered_workspace(ctx.handle, int(S_max), int(T_max), int(d), int(V)))
 
 
 def arrol_token_logprob_gathered(ctx: Context, src_rows, W_vocab, targets, cu_seqlens, survivor_idx, src_tok_off, d_num,
@@ -310,29 +322,16 @@ HOOK_SPIN_LIMIT, HOOK_MUTE_LOGPROB_PRODUCER, HOOK_LOGPROB_TIMING_BUFFER, HOOK_LO
 
 def arrol_test_hook(ctx: Context, key: int, value: int):
     """Test hook: bounds the log-prob kernel's pipeline waits / silences its producer (see include/arrol.h)."""
-    lib = load_library()
-    lib.arrol_test_hook.argtypes = [C.c_void_p, C.c_int32, C.c_int64]
-    _check(lib.arrol_test_hook(ctx.handle, int(key), int(value)), "arrol_test_hook")
+    _check(load_library().arrol_test_hook(ctx.handle, int(key), int(value)), "arrol_test_hook")
 
 
 def arrol_set_source_rows(ctx: Context, source_rows: int):
     """Switches on (source_rows > 0) or off (0) the device-side range checks of row_index / src_tok_off + lengths."""
-    lib = load_library()
-    lib.arrol_set_source_rows.argtypes = [C.c_void_p, C.c_int64]
-    _check(lib.arrol_set_source_rows(ctx.handle, int(source_rows)), "arrol_set_source_rows")
+    _check(load_library().arrol_set_source_rows(ctx.handle, int(source_rows)), "arrol_set_source_rows")
 
 
 def arrol_launch_count(ctx: Context) -> int:
     return int(load_library().arrol_launch_count(ctx.handle))
-
-
-def _fill_head(hs: _Head, hidden_dtype_code: int, d: int, head: dict):
-    hs.d = int(d)
-    hs.h = int(head.get("h", 0))
-    hs.dtype = hidden_dtype_code
-    for name in ("W1", "b1", "w2", "b2"):
-        t = head.get(name)
-        setattr(hs, name, None if t is None else t.data_ptr())
 
 
 def make_host_step(scalars: dict, head: dict, q_lut: Optional[torch.Tensor], tensors: dict) -> _HostStep:
@@ -342,9 +341,8 @@ def make_host_step(scalars: dict, head: dict, q_lut: Optional[torch.Tensor], ten
     st = _HostStep()
     for k, v in scalars.items():
         setattr(st, k, v)
-    _fill_head(st.head, ARROL_BF16, scalars["d"], head)
-    st.calib.B = 0 if q_lut is None else q_lut.shape[0]
-    st.calib.q_lut = None if q_lut is None else q_lut.data_ptr()
+    st.head = _head_struct(ARROL_BF16, scalars["d"], head)
+    st.calib = _calib_struct(q_lut)
     for k, t in tensors.items():
         if k.startswith("h_") and t.is_cuda:
             raise ValueError("%s must be a host tensor" % k)
@@ -369,11 +367,8 @@ def arrol_score_partial_static(hidden: torch.Tensor, head: dict, N: int, score: 
     a fixed 128 KiB array inside the library.  Limits: MLP head only, N <= 4096, h <= 512.  Runs on the current
     device; calls that overlap on one GPU race on the shared scratch.  The first call per device does a one-time
     address look-up and should come before any stream capture."""
-    hs = _Head()
-    _fill_head(hs, _dtype_code(hidden), hidden.shape[-1], head)
-    cs = _Calib()
-    cs.B = 0 if q_lut is None else q_lut.shape[0]
-    cs.q_lut = None if q_lut is None else q_lut.data_ptr()
+    hs = _head_struct(_dtype_code(hidden), hidden.shape[-1], head)
+    cs = _calib_struct(q_lut)
     stride = hidden.stride(-2) if row_stride is None else int(row_stride)
     _check(load_library().arrol_score_partial_static(_ptr(hidden), stride, _ptr(row_index), int(N), C.byref(hs),
                                                      C.byref(cs), _ptr(score), _ptr(prob), _ptr(bin), _ptr(q),
@@ -387,9 +382,8 @@ def make_prune_step(hidden: torch.Tensor, head: dict, q_lut: Optional[torch.Tens
     a = _PruneStep()
     a.hidden = hidden.data_ptr()
     a.row_stride_elems = hidden.stride(-2) if row_stride is None else int(row_stride)
-    _fill_head(a.head, _dtype_code(hidden), hidden.shape[-1], head)
-    a.calib.B = 0 if q_lut is None else q_lut.shape[0]
-    a.calib.q_lut = None if q_lut is None else q_lut.data_ptr()
+    a.head = _head_struct(_dtype_code(hidden), hidden.shape[-1], head)
+    a.calib = _calib_struct(q_lut)
     for k, v in scalars.items():
         setattr(a, k, v)
     for k, t in tensors.items():

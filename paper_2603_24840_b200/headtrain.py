@@ -29,8 +29,7 @@ def arrol_head_grad_workspace(ctx: B.Context, N: int, d: int, h: int) -> int:
 def arrol_head_grad(ctx: B.Context, hidden: torch.Tensor, head: dict, N: int, rewards, grads: dict, loss, workspace,
                     row_index: Optional[torch.Tensor] = None, mask: Optional[torch.Tensor] = None, stream=None):
     """grads = {"W1", "b1"[, "w2", "b2"]} float32 device tensors, overwritten; loss = float64 device tensor [1]."""
-    hs = B._Head()
-    B._fill_head(hs, B._dtype_code(hidden), hidden.shape[-1], head)
+    hs = B._head_struct(B._dtype_code(hidden), hidden.shape[-1], head)
     B._check(_lib().arrol_head_grad(ctx.handle, B._ptr(hidden), hidden.stride(-2), B._ptr(row_index), int(N),
                                     C.byref(hs), B._ptr(rewards), B._ptr(mask), B._ptr(grads["W1"]), B._ptr(grads["b1"]),
                                     B._ptr(grads.get("w2")), B._ptr(grads.get("b2")), B._ptr(loss), B._ptr(workspace),

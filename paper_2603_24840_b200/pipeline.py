@@ -72,6 +72,7 @@ class PruneRebatch:
         self.cu_seqlens = torch.empty(N + 1, dtype=i64, device=dev)
         self.adv = torch.empty(N, dtype=f32, device=dev)
         self.d_num = torch.zeros(2, dtype=i64, device=dev)
+        self.d_T = self.d_num[1:]
         self.dst_tokens = torch.empty(cap, dtype=i32, device=dev)
         self.tok_adv = torch.empty(cap, dtype=f32, device=dev)
         self.tok_seq = torch.empty(cap, dtype=i32, device=dev)
@@ -126,6 +127,7 @@ class PruneRebatch:
             for name, t in bufs.items():
                 setattr(v, name, t)
             v.d_num = torch.zeros(2, dtype=i64, device=dev)      # every view keeps its own {S, T}
+            v.d_T = v.d_num[1:]
             views.append(v)
         return views
 
@@ -148,7 +150,7 @@ class PruneRebatch:
     def token_logprob(self, hidden: Optional[torch.Tensor] = None):
         h = self.dst_rows if hidden is None else hidden
         B.arrol_token_logprob(self.ctx, h, self.W_vocab, self.dst_tokens, self.cap, self.w.d, self.w.V, self.logp,
-                              self.workspace, lse=self.lse, d_T=self.d_num[1:])
+                              self.workspace, lse=self.lse, d_T=self.d_T)
 
     def token_logprob_gathered(self):
         """Log-probs with the survivors' rows read in place from the source buffer (no packed copy needed)."""
