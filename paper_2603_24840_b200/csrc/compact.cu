@@ -243,7 +243,9 @@ int arrol_internal_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* l
     if (!guard.ok) return ARROL_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     if (!scan_done) {
-        ARROL_CUDA_OK(arrol_launch_pdl(scan_adv_kernel, dim3(1), dim3(SCAN_THREADS), 0, s, keep, lengths, N, G, rewards,
+        int threads = (N + 4 * 32 - 1) / (4 * 32) * 32;      // four rollouts per thread; a small call pays for few warps only
+        threads = threads < 32 ? 32 : (threads > SCAN_THREADS ? SCAN_THREADS : threads);
+        ARROL_CUDA_OK(arrol_launch_pdl(scan_adv_kernel, dim3(1), dim3(threads), 0, s, keep, lengths, N, G, rewards,
                                        (double)eps, ddof, dst_capacity_tokens, survivor_idx, cu_seqlens, adv, d_num,
                                        ctx->d_status, src_tok_off, ctx->source_rows));
         ctx->launches += 1;

@@ -605,13 +605,12 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
         const float4 r = *reinterpret_cast<const float4*>(p);
         return PartialLse{r.x, r.y, r.z, r.w};
     };
-    auto finish = [&](int64_t t, const PartialLse (&halves)[HALVES]) {
+    auto finish = [&](int64_t t, int y, const PartialLse (&halves)[HALVES]) {
         PartialLse r = halves[0];
 #pragma unroll
         for (int h = 1; h < HALVES; ++h) merge_record(r, halves[h]);
         const float lse2 = r.m2 + log2f(r.l);
         const float ln2 = 0.69314718055994530942f;
-        const int y = targets[t];
         float out = 0.f;
         if (y >= 0) {
             if (y < V) out = (r.zy2 - lse2) * ln2;
@@ -624,17 +623,19 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
     const int64_t thread = blockIdx.x * (int64_t)COMBINE_THREADS + threadIdx.x;
     const int64_t threads = (int64_t)gridDim.x * COMBINE_THREADS;
     for (int64_t t = thread; t < body_rows; t += threads) {
+        const int y = targets[t];
         PartialLse total[HALVES];
 #pragma unroll
         for (int h = 0; h < HALVES; ++h) total[h] = empty_record();
         for (int g = 0; g < plan.splits; ++g)
 #pragma unroll
             for (int h = 0; h < HALVES; ++h) merge_record(total[h], load(body + ((int64_t)g * HALVES + h) * T_max + t));
-        finish(t, total);
+        finish(t, y, total);
     }
     const int lane = threadIdx.x & 31;
     for (int64_t t = body_rows + (thread >> 5); t < T; t += threads >> 5) {
         const PartialLse* rec = tail + (t - body_rows) * plan.n_sub * HALVES;
+        const int y = targets[t];                // requested now, used at the end
         PartialLse total[HALVES], group[HALVES];
 #pragma unroll
         for (int h = 0; h < HALVES; ++h) total[h] = group[h] = empty_record();
@@ -664,7 +665,7 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
                 }
             }
         }
-        if (lane == 0) finish(t, total);
+        if (lane == 0) finish(t, y, total);
     }
 }
 

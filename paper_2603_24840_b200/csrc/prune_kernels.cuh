@@ -56,17 +56,28 @@ template <> struct Vec16<__nv_bfloat16> {
 // is one round trip), four accumulators per lane, shuffle reduction; every lane returns the row's sum (without the
 // bias); nvec = d / Vec16<T>::N, or 0 to skip the row (sum 0).  Products and sums are taken in exactly the order of
 // score_linear_kernel, which keeps w's vectors in registers beside the row's, so the two give the same bits.
+// The first eight loads are a function of their own (linear_row_begin), so that a caller can have them in flight while it
+// waits for something else.
 template <typename T>
-__device__ __forceinline__ float linear_row_dot_ws(const T* __restrict__ x, const typename Vec16<T>::Raw* w_s, int nvec,
-                                                   int lane) {
+__device__ __forceinline__ void linear_row_begin(const T* __restrict__ x, int nvec, int lane, typename Vec16<T>::Raw (&xr)[8]) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int c = lane + 32 * u;
+        if (c < nvec) xr[u] = Vec16<T>::load_raw(x + (int64_t)c * Vec16<T>::N);
+    }
+}
+template <typename T>
+__device__ __forceinline__ float linear_row_dot_ws(const T* __restrict__ x, typename Vec16<T>::Raw (&xr)[8],
+                                                   const typename Vec16<T>::Raw* w_s, int nvec, int lane) {
     constexpr int VN = Vec16<T>::N;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     for (int c0 = lane; c0 < nvec; c0 += 256) {
-        typename Vec16<T>::Raw xr[8];
+        if (c0 != lane) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int c = c0 + 32 * u;
-            if (c < nvec) xr[u] = Vec16<T>::load_raw(x + (int64_t)c * VN);
+            for (int u = 0; u < 8; ++u) {
+                const int c = c0 + 32 * u;
+                if (c < nvec) xr[u] = Vec16<T>::load_raw(x + (int64_t)c * VN);
+            }
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
@@ -85,13 +96,6 @@ __device__ __forceinline__ double shfl_double(double v, int src_lane, int width)
     return __hiloint2double(hi, lo);
 }
 
-__device__ __forceinline__ double shfl_xor_double(double v, int mask, int width) {
-    int lo = __double2loint(v), hi = __double2hiint(v);
-    lo = __shfl_xor_sync(0xffffffffu, lo, mask, width);
-    hi = __shfl_xor_sync(0xffffffffu, hi, mask, width);
-    return __hiloint2double(hi, lo);
-}
-
 // Per-group correctness-balancing selection (Section 4.1; Theorem 1's rule j^ = argmin_j |mu_{-j} - rho| applied
 // G - K times) for the groups held by one warp: a group occupies a segment of `seg` = next power of two >= G lanes,
 // lane j of the segment holds rollout j's q in double (`member` false for padding lanes and groups past the end).
@@ -106,13 +110,14 @@ __device__ __forceinline__ bool select_lanes(double qj, bool member, int j, int 
     for (int i = 0; i < G; ++i) sigma = __dadd_rn(sigma, shfl_double(qj, i, seg));
     for (int n = G; n > K; --n) {
         const double tau = __dsub_rn(sigma, __dmul_rn(rho, (double)(n - 1)));
-        double key = alive ? fabs(__dsub_rn(qj, tau)) : __longlong_as_double(0x7ff0000000000000LL);
+        // non-negative doubles order like their bit patterns, and an integer compare is several times faster than fp64's
+        unsigned long long key = alive ? (unsigned long long)__double_as_longlong(fabs(__dsub_rn(qj, tau))) : 0x7ff0000000000000ull;
         int idx = alive ? j : -1;
         // segmented arg-min; ties -> the higher index
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             if (o < seg) {
-                const double okey = shfl_xor_double(key, o, seg);
+                const unsigned long long okey = __shfl_xor_sync(0xffffffffu, key, o, seg);
                 const int oidx = __shfl_xor_sync(0xffffffffu, idx, o, seg);
                 if (okey < key || (okey == key && oidx > idx)) { key = okey; idx = oidx; }
             }
@@ -187,7 +192,8 @@ constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 4;      // consecutive rollouts per thread and pass: N <= 4096 is one pass
 constexpr int SCAN_GROUPS = SCAN_THREADS * SCAN_ITEMS / 4 + 2;   // groups of size >= 4 that one pass can touch
 
-// Survivor scan and advantages of arrol_compact (Section 4.3 (ii); Section 3) by ONE block of SCAN_THREADS threads.
+// Survivor scan and advantages of arrol_compact (Section 4.3 (ii); Section 3) by ONE block of up to SCAN_THREADS threads (a
+// multiple of 32; four rollouts per thread and pass).
 // `keep` may have been written earlier in the same kernel by other blocks (the fused prune step): it is read with
 // L2-coherent loads, never through the read-only path.
 __device__ __forceinline__ void scan_adv_block(const uint8_t* keep, const int32_t* __restrict__ lengths, int N, int G,
@@ -211,7 +217,8 @@ __device__ __forceinline__ void scan_adv_block(const uint8_t* keep, const int32_
     int64_t carry_t = 0;
 
     // statistics over the kept rollouts of a group (Section 3, on survivors): sums in index order, fp64
-    constexpr int PASS = SCAN_THREADS * SCAN_ITEMS;
+    const int threads = (int)blockDim.x, warps = threads >> 5;
+    const int PASS = threads * SCAN_ITEMS;
     // Statistics of group g over its kept rollouts: mean and 1 / (std + eps), in fp64.  A double-precision division
     // or square root costs this one-block kernel about half a microsecond each, so the reciprocals of the small
     // counts come from a table and sqrt / reciprocal are Newton steps from single-precision seeds (relative error
@@ -227,7 +234,7 @@ __device__ __forceinline__ void scan_adv_block(const uint8_t* keep, const int32_
         group_statistics(g0, g1, ddof, eps, s_inv, flag, rew, mean, inv_den);
     };
 
-    if (threadIdx.x >= 1 && threadIdx.x < SCAN_INV) s_inv[threadIdx.x] = 1.0 / (double)threadIdx.x;   // before the first barrier below
+    for (int c = threadIdx.x + 1; c < SCAN_INV; c += threads) s_inv[c] = 1.0 / (double)c;                // before the first barrier below
 
     for (int base = 0; base < N; base += PASS) {
         const int i0 = base + threadIdx.x * SCAN_ITEMS;
@@ -236,7 +243,7 @@ __device__ __forceinline__ void scan_adv_block(const uint8_t* keep, const int32_
         int32_t c = 0;
         int64_t t = 0;
         // one round of coalesced loads: flags and rewards of the pass into shared memory, lengths into registers
-        for (int e = threadIdx.x; e < PASS; e += SCAN_THREADS) {
+        for (int e = threadIdx.x; e < PASS; e += threads) {
             const int i = base + e;
             s_keep[e] = i < N ? __ldcg(keep + i) : (uint8_t)0;
             s_rew[e] = i < N ? rewards[i] : 0.f;
@@ -256,7 +263,7 @@ __device__ __forceinline__ void scan_adv_block(const uint8_t* keep, const int32_
         const int g_lo = base / G;
         if (shared_stats) {          // one thread per group of this pass; visible after the scan's first barrier
             const int g_hi = (min(N, base + PASS) - 1) / G;
-            for (int gi = threadIdx.x; gi <= g_hi - g_lo; gi += SCAN_THREADS)
+            for (int gi = threadIdx.x; gi <= g_hi - g_lo; gi += threads)
                 group_stats(g_lo + gi, base, g_mean[gi], g_den[gi]);
         }
 #pragma unroll
@@ -273,8 +280,8 @@ __device__ __forceinline__ void scan_adv_block(const uint8_t* keep, const int32_
         if (lane == 31) { warp_cnt[wid] = c; warp_tok[wid] = t; }
         __syncthreads();
         // every warp scans the 32 warp totals itself (no second barrier, no single-warp phase)
-        int32_t wc = warp_cnt[lane];
-        int64_t wt = warp_tok[lane];
+        int32_t wc = lane < warps ? warp_cnt[lane] : 0;
+        int64_t wt = lane < warps ? warp_tok[lane] : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int32_t oc = __shfl_up_sync(0xffffffffu, wc, o);

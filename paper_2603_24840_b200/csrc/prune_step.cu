@@ -59,6 +59,7 @@ struct FusedParams {
     uint32_t spin_limit;
 };
 
+constexpr int LUT_STAGED = 1024;
 constexpr unsigned long long PUBLISHED = 1ull << 63;
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
@@ -76,6 +77,7 @@ prune_fused_kernel(const FusedParams p) {
     __shared__ uint8_t keep_s[32];
     __shared__ int32_t len_s[32];
     __shared__ double inv_count[SCAN_INV], g_mean[32], g_den[32];
+    __shared__ float lut_s[LUT_STAGED];                      // the posterior table, or its first use would be one more round trip
     extern __shared__ uint4 w_stage[];                       // linear head: the weights, d * sizeof(T) bytes
     pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -103,21 +105,27 @@ prune_fused_kernel(const FusedParams p) {
             row = row_index ? row_index[i] : (int64_t)i;
         }
         const T* w = pdl_acquire(static_cast<const T*>(p.w));
+        const float* q_lut = pdl_acquire(p.q_lut);
+        const bool lut_staged = q_lut && p.B <= LUT_STAGED;
         for (int c = threadIdx.x; c < p.d / VN; c += blockDim.x) w_s[c] = Vec16<T>::load_raw(w + (int64_t)c * VN);
+        if (lut_staged)
+            for (int c = threadIdx.x; c < p.B; c += blockDim.x) lut_s[c] = q_lut[c];
+        const T* x = pdl_acquire(static_cast<const T*>(p.hidden)) + row * p.row_stride;
+        const T* bias_ptr = pdl_acquire(static_cast<const T*>(p.bias));
+        const float bias = bias_ptr ? to_f32(bias_ptr[0]) : 0.f;
+        int nvec = warp < n_here ? p.d / VN : 0;
+        if (nvec && p.source_rows > 0 && (row < 0 || row >= p.source_rows)) {   // never read, scored as zeros
+            if (lane == 0) atomicOr(p.d_status, ARROL_DEV_BAD_INDEX);
+            nvec = 0;
+        }
+        Raw xr[8];
+        linear_row_begin<T>(x, nvec, lane, xr);              // the row is on its way while the block waits for the weights
         __syncthreads();
         if (warp < n_here) {
-            const T* hidden = pdl_acquire(static_cast<const T*>(p.hidden));
-            const T* bias = pdl_acquire(static_cast<const T*>(p.bias));
-            const float* q_lut = pdl_acquire(p.q_lut);
-            int nvec = p.d / VN;
-            if (p.source_rows > 0 && (row < 0 || row >= p.source_rows)) {   // never read, scored as zeros
-                if (lane == 0) atomicOr(p.d_status, ARROL_DEV_BAD_INDEX);
-                nvec = 0;
-            }
-            float s = linear_row_dot_ws<T>(hidden + row * p.row_stride, w_s, nvec, lane);
+            float s = linear_row_dot_ws<T>(x, xr, w_s, nvec, lane);
             if (lane == 0) {
-                if (bias) s += to_f32(bias[0]);
-                q_s[warp] = probability_map(s, i, p.B, q_lut, p.score, p.prob, p.bin, p.q);
+                if (bias_ptr) s += bias;
+                q_s[warp] = probability_map(s, i, p.B, lut_staged ? lut_s : q_lut, p.score, p.prob, p.bin, p.q);
             }
         }
     } else {
@@ -209,18 +217,21 @@ prune_fused_kernel(const FusedParams p) {
     }
     const bool any_bad = __any_sync(0xffffffffu, bad_index);
     const bool any_expired = __any_sync(0xffffffffu, expired);
+    unsigned long long done = 0;
     if (lane == 0) {
         if (any_expired) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
         if (any_bad) atomicOr(reinterpret_cast<unsigned int*>(p.chain + 1), 1u);
         __threadfence();
-        // the block that finishes last has seen every block read what it needed: clear the chain for the next call
-        const unsigned long long done = atomicAdd(p.chain, 1ull);
-        if (done == gridDim.x - 1) {
-            __threadfence();
+        done = atomicAdd(p.chain, 1ull);
+    }
+    // the block that finishes last has seen every block read what it needed: clear the chain for the next call
+    if (__shfl_sync(0xffffffffu, done, 0) == gridDim.x - 1) {
+        __threadfence();
+        for (unsigned int b = lane; b < 2 * gridDim.x; b += 32) totals[b] = 0ull;
+        if (lane == 0) {
             const unsigned int bad = *reinterpret_cast<volatile unsigned int*>(p.chain + 1);
             if (bad) atomicOr(p.d_status, ARROL_DEV_BAD_INDEX);
             p.d_status[1] = bad ? 1u : 0u;       // gate word: the gather kernels of this call copy nothing when set
-            for (unsigned int b = 0; b < 2 * gridDim.x; ++b) totals[b] = 0ull;
             p.chain[1] = 0ull;
             p.chain[0] = 0ull;
         }

@@ -14,7 +14,7 @@ __device__ __forceinline__ float probability_map(float s, int i, int B, const fl
     score[i] = s;
     prob[i] = sp;
     if (bin) bin[i] = b;
-    const float qv = (q_lut != nullptr) ? __ldg(q_lut + b) : sp;
+    const float qv = (q_lut != nullptr) ? q_lut[b] : sp;      // global or shared memory
     q[i] = qv;
     return qv;
 }
