@@ -34,8 +34,8 @@ __device__ __forceinline__ void bulk_store(void* gdst, const void* smem_src, uin
                  ::"l"(gdst), "r"(smem_u32(smem_src)), "r"(bytes), "l"(l2_policy) : "memory");
 }
 // L2 eviction priority of the stored rows.  Packed rows that outgrow L2 are gone before anybody reads them: written back
-// first they leave the cache's share to the reads (1.67 GB of rows of 4 KB: 580 -> 570 us for the prune step, of 8 KB:
-// 2,088 -> 2,073; the same hint on the loads instead 571 and 2,088).  A packed block that fits stays for the log-prob kernel.
+// first they leave the cache's share to the reads (1.67 GB of rows of 4 KB: 579 -> 569 us for the prune step, 6.7 GB of 8 KB:
+// 2,093 -> 2,074; the same hint on the loads instead 571 and 2,088).  A packed block that fits stays for the log-prob kernel.
 constexpr int64_t L2_BYTES = (int64_t)126 << 20;
 __device__ __forceinline__ uint64_t store_policy(bool streamed) {
     uint64_t p;
@@ -133,7 +133,8 @@ gather_rows_bulk_kernel(const int64_t* __restrict__ d_num, const int64_t* __rest
             const int rows_here = (int)min((int64_t)tile_rows, T - t0);
             if (!mbar_wait(&full[stage], phase, abort_flag)) break;
             fence_proxy_async_smem();
-            bulk_store(dst_rows + t0 * row_bytes, smem + (size_t)stage * GB_TILE_BYTES, (uint32_t)(rows_here * row_bytes));
+            bulk_store(dst_rows + t0 * row_bytes, smem + (size_t)stage * GB_TILE_BYTES, (uint32_t)(rows_here * row_bytes),
+                       policy);
             bulk_commit_group();
             if (prev_stage >= 0) {                        // the store before this one has read its stage: free it
                 bulk_wait_read_but_one();
