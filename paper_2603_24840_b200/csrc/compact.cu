@@ -153,16 +153,24 @@ gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restric
         const int len = (int)(__ldg(cu_seqlens + s + 1) - c0);
         const int64_t src0 = __ldg(src_tok_off + __ldg(survivor_idx + s));
         const float a = __ldg(adv + s);
-        auto one = [&](int t) {
-            if (dst_tokens) dst_tokens[c0 + t] = __ldg(src_tokens + src0 + t);
+        auto store_one = [&](int t, int32_t id) {
+            if (dst_tokens) dst_tokens[c0 + t] = id;
             if (tok_seq) tok_seq[c0 + t] = s;
             if (tok_adv) tok_adv[c0 + t] = a;
         };
+        if (!vector_stores) {
+            for (int t = threadIdx.x; t < len; t += TOKENS_THREADS) store_one(t, dst_tokens ? __ldg(src_tokens + src0 + t) : 0);
+            continue;
+        }
         // up to three tokens before the first 16-byte boundary of the outputs, then groups of four, then up to three
-        const int head = vector_stores ? min(len, (int)((4 - (c0 & 3)) & 3)) : len;
+        const int head = min(len, (int)((4 - (c0 & 3)) & 3));
         const int quads = (len - head) / 4;
-        for (int t = threadIdx.x; t < head; t += TOKENS_THREADS) one(t);
-        if ((int)threadIdx.x < (vector_stores ? len - head - 4 * quads : 0)) one(head + 4 * quads + threadIdx.x);
+        // (one each for six threads; stored after the groups, or the first warp's group loads would wait for a store that
+        // waits for its id: one group of 16 rollouts 27.4 -> 26.8 us, with the linear head 19.8 -> 19.3)
+        const int edge = (int)threadIdx.x < 3 ? ((int)threadIdx.x < head ? (int)threadIdx.x : -1)
+                                              : ((int)threadIdx.x < 6 && head + 4 * quads + (int)threadIdx.x - 3 < len
+                                                     ? head + 4 * quads + (int)threadIdx.x - 3 : -1);
+        const int32_t edge_id = edge >= 0 && dst_tokens ? __ldg(src_tokens + src0 + edge) : 0;
         const int32_t* src = src_tokens + src0 + head;
         const int shift = (int)((reinterpret_cast<uintptr_t>(src) & 15) >> 2);      // ids before src in its 16-byte word
         const int4* words = reinterpret_cast<const int4*>(src - shift);
@@ -199,6 +207,7 @@ gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restric
                 if (tok_adv) *reinterpret_cast<float4*>(tok_adv + at) = make_float4(a, a, a, a);
             }
         }
+        if (edge >= 0) store_one(edge, edge_id);
     }
 }
 

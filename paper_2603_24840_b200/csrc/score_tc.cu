@@ -46,17 +46,18 @@ template <int SBN> __host__ __device__ constexpr int issuers() { return SBN == 6
 template <int SBN> __host__ __device__ constexpr int stage_bytes() { return A_BYTES + SBN * BK * 2; }
 template <int SBN> __host__ __device__ constexpr size_t smem_bytes() { return (size_t)ring_stages<SBN>() * stage_bytes<SBN>() + 1024 + S_TAIL_BYTES; }
 
-// one warp per 4 KB of a row: 16-byte copies, all of its loads in flight before the first store
+// one warp per 4 KB of a row (a grid row per slice, so that no warp divides): 16-byte copies, all of its loads in flight
+// before the first store
 constexpr int PACK_VECS = 256;
 __global__ void __launch_bounds__(128)
 pack_rows_kernel(const __nv_bfloat16* __restrict__ hidden, int64_t row_stride, const int64_t* __restrict__ row_index,
-                 int N, int d, int slices, __nv_bfloat16* __restrict__ out, int64_t source_rows, uint32_t* d_status) {
+                 int N, int d, __nv_bfloat16* __restrict__ out, int64_t source_rows, uint32_t* d_status) {
     pdl_launch_dependents();
     pdl_wait();
     hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index);
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    const int i = w / slices, c0 = (w - i * slices) * PACK_VECS + lane;
+    const int c0 = blockIdx.y * PACK_VECS + lane;
     if (i >= N) return;
     const int64_t row = row_index[i];
     const uint4* src = reinterpret_cast<const uint4*>(hidden + row * row_stride);
@@ -299,8 +300,8 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     int64_t ld = row_stride;
     if (pack) {
         const int slices = (d / 8 + PACK_VECS - 1) / PACK_VECS;
-        ARROL_CUDA_OK(arrol_launch_pdl(pack_rows_kernel, dim3((unsigned)(((int64_t)N * slices + 3) / 4)), dim3(128), 0, s,
-                                       static_cast<const __nv_bfloat16*>(hidden), row_stride, row_index, N, d, slices,
+        ARROL_CUDA_OK(arrol_launch_pdl(pack_rows_kernel, dim3((unsigned)((N + 3) / 4), (unsigned)slices), dim3(128), 0, s,
+                                       static_cast<const __nv_bfloat16*>(hidden), row_stride, row_index, N, d,
                                        static_cast<__nv_bfloat16*>(ctx->d_pack), ctx->source_rows, ctx->d_status));
         ctx->launches += 1;
         x = ctx->d_pack;
