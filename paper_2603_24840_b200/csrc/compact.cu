@@ -127,81 +127,92 @@ gather_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_
     }
 }
 
-// Per-token outputs without a payload plane (token ids, survivor ordinal, advantage): one block per survivor walks
-// its run of tokens, so nothing has to be searched.  Blocks past S return at once.  Bound by the bytes it moves (16 per
-// token, 12 of them written): all three outputs leave as 16-byte stores, four tokens per thread.  The source run is aligned
-// differently from the destination, so a thread reads the two aligned 16-byte words that hold its four ids (the second one
-// is its neighbour's first, in L1 by then) and picks them out.  2.7 M tokens: the kernel
-// 11.3 -> 10.4 us, the prune step 26.1 -> 23.2 us; beyond what L2 holds (6.5 M tokens, 104 MB) the stores go at HBM's pace either way.
+// Per-token outputs without a payload plane (token ids, survivor ordinal, advantage): a team of lanes per survivor walks
+// its run of tokens, so nothing has to be searched.  Blocks past the survivors return at once.  Bound by the bytes it moves
+// (16 per token, 12 of them written): all three outputs leave as 16-byte stores, four tokens per lane.  The source run is
+// aligned differently from the destination, so a lane reads the two aligned 16-byte words that hold its four ids (the second
+// one is its neighbour's first, in L1 by then) and picks them out, without a branch, so that a lane's loads are all in
+// flight together.  The few ids whose words would reach outside the run go one by one.
+// Prune step without a payload plane, 4-byte stores and 128 threads per survivor / this / 16-byte stores and 256 threads per
+// survivor: 1,024 runs of 2,600 ids 26.1 / 22.0 / 22.9 us; 12,288 of 131 58.6 / 52.6 / 69.7; 2,048 of 600 19.9 / 19.7 / 22.0; 828 of
+// 275 12.3 / 12.5 / 12.9; 8 of 1,240 12.3 / 12.1 / 12.0.  Beyond what L2 holds (6.5 M ids, 104 MB) the stores go at HBM's pace.
 constexpr int TOKENS_THREADS = 256;
-constexpr int TOKENS_QUADS = 4;          // groups of four tokens in flight per thread
-__global__ void __launch_bounds__(TOKENS_THREADS)
+constexpr int TOKENS_QUADS = 2;          // groups of four tokens in flight per lane (3 or 4 spill at four blocks per SM: 24.4, 26.7 us on the first of these)
+constexpr int TOKENS_BLOCKS = 4;         // blocks per SM (five or six blocks of fewer registers: 24.4, 25.0)
+// Lanes per survivor: a group of four tokens for each while that many fit on the GPU at once, else up to TOKENS_QUADS groups.
+__device__ __forceinline__ int token_team(int64_t T, int S, int resident) {
+    const float groups = __fdividef((float)T, 4.f * (float)S);              // of the mean survivor
+    int lanes = groups <= 32.f ? 32 : groups <= 64.f ? 64 : groups <= 128.f ? 128 : TOKENS_THREADS;
+    while (lanes > 32 && (float)lanes * (float)S > (float)resident && (float)(lanes / 2 * TOKENS_QUADS) >= groups) lanes /= 2;
+    return lanes;
+}
+__global__ void __launch_bounds__(TOKENS_THREADS, TOKENS_BLOCKS)
 gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_seqlens,
                      const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off,
                      const int32_t* __restrict__ src_tokens, const float* __restrict__ adv, int64_t capacity,
                      int32_t* __restrict__ dst_tokens, float* __restrict__ tok_adv, int32_t* __restrict__ tok_seq,
-                     const uint32_t* __restrict__ gate, int vector_stores) {
+                     const uint32_t* __restrict__ gate, int vector_stores, int resident) {
     pdl_launch_dependents();
     pdl_wait();
     d_num = pdl_acquire(d_num); cu_seqlens = pdl_acquire(cu_seqlens); survivor_idx = pdl_acquire(survivor_idx);
     src_tok_off = pdl_acquire(src_tok_off); src_tokens = pdl_acquire(src_tokens); adv = pdl_acquire(adv);
     gate = pdl_acquire(gate);
     const int S = (int)d_num[0];
-    if (d_num[1] > capacity || *gate) return;              // overflow / bad index was recorded by the scan kernel
-    for (int s = blockIdx.x; s < S; s += gridDim.x) {
+    const int64_t T = d_num[1];
+    if (S <= 0 || T > capacity || *gate) return;                     // overflow / bad index was recorded by the scan kernel
+    const int lanes = token_team(T, S, resident);
+    const int team = (int)threadIdx.x / lanes, lane = (int)threadIdx.x & (lanes - 1), teams = TOKENS_THREADS / lanes;
+#pragma unroll 1
+    for (int s = blockIdx.x * teams + team; s < S; s += gridDim.x * teams) {
         const int64_t c0 = __ldg(cu_seqlens + s);
         const int len = (int)(__ldg(cu_seqlens + s + 1) - c0);
         const int64_t src0 = __ldg(src_tok_off + __ldg(survivor_idx + s));
         const float a = __ldg(adv + s);
+        auto load_one = [&](int t) { return dst_tokens ? __ldg(src_tokens + src0 + t) : 0; };
         auto store_one = [&](int t, int32_t id) {
             if (dst_tokens) dst_tokens[c0 + t] = id;
             if (tok_seq) tok_seq[c0 + t] = s;
             if (tok_adv) tok_adv[c0 + t] = a;
         };
-        if (!vector_stores) {
-            for (int t = threadIdx.x; t < len; t += TOKENS_THREADS) store_one(t, dst_tokens ? __ldg(src_tokens + src0 + t) : 0);
+        // [head, end): whole 16-byte groups of the outputs whose ids lie in words inside the run
+        int head = (int)((4 - (c0 & 3)) & 3), end = len - (int)((c0 + len) & 3);
+        const int shift = (int)((reinterpret_cast<uintptr_t>(src_tokens + src0 + head) & 15) >> 2);   // ids before src0 + head in its word
+        if (shift > head) head += 4;
+        if (shift && end - shift + 4 > len) end -= 4;
+        if (!vector_stores || end <= head) {
+#pragma unroll 1
+            for (int t = lane; t < len; t += lanes) store_one(t, load_one(t));
             continue;
         }
-        // up to three tokens before the first 16-byte boundary of the outputs, then groups of four, then up to three
-        const int head = min(len, (int)((4 - (c0 & 3)) & 3));
-        const int quads = (len - head) / 4;
-        // (one each for six threads; stored after the groups, or the first warp's group loads would wait for a store that
-        // waits for its id: one group of 16 rollouts 27.4 -> 26.8 us, with the linear head 19.8 -> 19.3)
-        const int edge = (int)threadIdx.x < 3 ? ((int)threadIdx.x < head ? (int)threadIdx.x : -1)
-                                              : ((int)threadIdx.x < 6 && head + 4 * quads + (int)threadIdx.x - 3 < len
-                                                     ? head + 4 * quads + (int)threadIdx.x - 3 : -1);
-        const int32_t edge_id = edge >= 0 && dst_tokens ? __ldg(src_tokens + src0 + edge) : 0;
-        const int32_t* src = src_tokens + src0 + head;
-        const int shift = (int)((reinterpret_cast<uintptr_t>(src) & 15) >> 2);      // ids before src in its 16-byte word
-        const int4* words = reinterpret_cast<const int4*>(src - shift);
-        // both words lie inside the run: nothing outside the rollout's own ids is read
-        auto whole_words = [&](int k) { return shift == 0 || (head + 4 * k >= shift && head + 4 * k - shift + 8 <= len); };
-        for (int k0 = threadIdx.x; k0 < quads; k0 += TOKENS_QUADS * TOKENS_THREADS) {
+        // at most 6 ids before and 6 after, a lane each; stored after the groups, or the first lanes' loads would wait for a
+        // store that waits for its id
+        const int edge = lane < head ? lane : (lane >= 8 && end + lane - 8 < len ? end + lane - 8 : -1);
+        const int32_t edge_id = edge >= 0 ? load_one(edge) : 0;
+        const int4* words = reinterpret_cast<const int4*>(src_tokens + src0 + head - shift);
+        const int quads = (end - head) / 4, second = shift ? 1 : 0;
+#pragma unroll 1
+        for (int k0 = lane; k0 < quads; k0 += TOKENS_QUADS * lanes) {
             int4 lo[TOKENS_QUADS], hi[TOKENS_QUADS];
+            if (dst_tokens) {
 #pragma unroll
-            for (int u = 0; u < TOKENS_QUADS; ++u) {
-                const int k = k0 + u * TOKENS_THREADS;
-                if (dst_tokens && k < quads) {
-                    if (whole_words(k)) {
+                for (int u = 0; u < TOKENS_QUADS; ++u) {
+                    const int k = k0 + u * lanes;
+                    if (k < quads) {
                         lo[u] = __ldg(words + k);
-                        if (shift) hi[u] = __ldg(words + k + 1);
-                    } else {
-                        lo[u] = make_int4(__ldg(src + 4 * k), __ldg(src + 4 * k + 1), __ldg(src + 4 * k + 2), __ldg(src + 4 * k + 3));
+                        hi[u] = __ldg(words + k + second);
                     }
                 }
             }
 #pragma unroll
             for (int u = 0; u < TOKENS_QUADS; ++u) {
-                const int k = k0 + u * TOKENS_THREADS;
+                const int k = k0 + u * lanes;
                 if (k >= quads) break;
                 const int64_t at = c0 + head + 4 * k;
                 if (dst_tokens) {
-                    int4 v = lo[u];
-                    const int by = whole_words(k) ? shift : 0;
-                    if (by == 1) v = make_int4(lo[u].y, lo[u].z, lo[u].w, hi[u].x);
-                    else if (by == 2) v = make_int4(lo[u].z, lo[u].w, hi[u].x, hi[u].y);
-                    else if (by == 3) v = make_int4(lo[u].w, hi[u].x, hi[u].y, hi[u].z);
-                    *reinterpret_cast<int4*>(dst_tokens + at) = v;
+                    const bool two = shift & 2, one = shift & 1;
+                    const int32_t x0 = two ? lo[u].z : lo[u].x, x1 = two ? lo[u].w : lo[u].y, x2 = two ? hi[u].x : lo[u].z,
+                                  x3 = two ? hi[u].y : lo[u].w, x4 = two ? hi[u].z : hi[u].x;
+                    *reinterpret_cast<int4*>(dst_tokens + at) = make_int4(one ? x1 : x0, one ? x2 : x1, one ? x3 : x2, one ? x4 : x3);
                 }
                 if (tok_seq) *reinterpret_cast<int4*>(tok_seq + at) = make_int4(s, s, s, s);
                 if (tok_adv) *reinterpret_cast<float4*>(tok_adv + at) = make_float4(a, a, a, a);
@@ -278,7 +289,8 @@ int arrol_internal_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* l
                                        cu_seqlens, survivor_idx, src_tok_off, src_tokens, adv, dst_capacity_tokens,
                                        dst_tokens, tok_adv, tok_seq, ctx->d_status + 1,
                                        arrol_aligned(dst_tokens, 16) && arrol_aligned(tok_adv, 16) && arrol_aligned(tok_seq, 16) &&
-                                               arrol_aligned(src_tokens, 4) ? 1 : 0));
+                                               arrol_aligned(src_tokens, 4) ? 1 : 0,
+                                       ctx->sm_count * TOKENS_BLOCKS * TOKENS_THREADS));
         ctx->launches += 1;
         return ARROL_OK;
     }

@@ -279,6 +279,38 @@ def test_compact_edge_cases(ctx):
     _compact_case(ctx, 3000, 8, 32, seed=7, lo=300, hi=700)                           # ~0.75M tokens, many tiles
 
 
+# teams of 32, 64, 128 and 256 lanes per survivor; 64 wanted but 32 taken (more survivors than fit side by side); runs too
+# short for a group of four; a few long runs
+@pytest.mark.parametrize("N,G,lo,hi", [(512, 8, 0, 250), (512, 8, 200, 310), (520, 8, 400, 600), (96, 8, 900, 1600),
+                                       (24000, 8, 130, 250), (400, 4, 0, 9), (8, 4, 5000, 9001)])
+@pytest.mark.parametrize("row_bytes", [0, 16])
+def test_token_runs_of_all_lengths_and_alignments(ctx, N, G, lo, hi, row_bytes):
+    _compact_case(ctx, N, G, row_bytes, seed=N + hi, lo=lo, hi=hi)
+    _compact_case(ctx, N, G, row_bytes, seed=N + hi + 1, lo=lo, hi=hi, padded=True)
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_token_outputs_that_no_16_byte_store_can_reach(ctx, shift):
+    G, N = 8, 64
+    g = np.random.default_rng(shift)
+    ell = g.integers(0, 90, size=N).astype(np.int32)
+    off, keep = synth.src_offsets(ell), (g.random(N) < 0.5).astype(np.uint8)
+    tokens, n = dev(g.integers(0, 1 << 30, size=int(off[-1])).astype(np.int32)), int(off[-1])
+    got = []
+    for at in (0, shift):
+        outs = [torch.full((n + 8,), 7, dtype=t, device="cuda") for t in (torch.int32, torch.int32, torch.float32)]
+        dst, seq, adv = (o[at:at + n] for o in outs)
+        z = lambda k, t: torch.zeros(k, dtype=t, device="cuda")
+        B.arrol_compact(ctx, dev(keep), dev(ell), dev(off[:-1]), N, G, dev((g.random(N) < 2).astype(np.float32)), n, z(N + 1, torch.int64),
+                        z(N, torch.int32), z(N, torch.float32), z(2, torch.int64), src_tokens=tokens, dst_tokens=dst, tok_seq=seq,
+                        tok_adv=adv)
+        torch.cuda.synchronize()
+        got.append([o.clone() for o in (dst, seq, adv)])
+        assert all((o[:at] == 7).all() and (o[at + n:] == 7).all() for o in outs)      # nothing outside the outputs
+    T = int((ell * keep).sum())
+    assert T > 500 and all(torch.equal(a[:T], b[:T]) and (b[T:] == 7).all() for a, b in zip(*got))
+
+
 def test_compact_degenerate_groups_and_capacity_overflow(ctx):
     G, N = 8, 24
     rewards = np.array([0] * G + [1] * G + [1, 0] * (G // 2), np.float32)
