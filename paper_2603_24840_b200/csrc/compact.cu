@@ -4,14 +4,15 @@
 // Kernel 1 (one block): stable partition by a block-wide prefix sum over (kept flag, kept length):
 //   survivor_idx, cu_seqlens, {S, T}, and per-survivor advantages (fp64 statistics over the kept rollouts of
 //   the group, in index order, rounded once to fp32).
-// Kernel 2: the per-token outputs (token id, survivor ordinal, advantage), one block per survivor, and, when there is
-//   a hidden-row plane, the rows themselves by bulk copies through shared memory (gather_bulk.cu).  Rows too large
+// Kernel 2: the per-token outputs (token id, survivor ordinal, advantage), a team of lanes per survivor, and, when there is
+//   a hidden-row plane, beside them the rows by bulk copies through shared memory (gather_bulk.cu).  Rows too large
 //   for a bulk stage take gather_kernel below: one wave of persistent blocks, each owning a contiguous run of
 //   destination tiles; one thread per row finds its survivor (binary search once per block, then a forward walk in
 //   cu_seqlens), then the block streams the tile's payload with 16-byte loads/stores, eight in flight per thread.
 //   T is read from device memory, so there is no host synchronisation between the kernels.
 #include "arrol_internal.h"
 #include "prune_kernels.cuh"
+#include "token_runs.cuh"
 
 namespace {
 
@@ -127,99 +128,24 @@ gather_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_
     }
 }
 
-// Per-token outputs without a payload plane (token ids, survivor ordinal, advantage): a team of lanes per survivor walks
-// its run of tokens, so nothing has to be searched.  Blocks past the survivors return at once.  Bound by the bytes it moves
-// (16 per token, 12 of them written): all three outputs leave as 16-byte stores, four tokens per lane.  The source run is
-// aligned differently from the destination, so a lane reads the two aligned 16-byte words that hold its four ids (the second
-// one is its neighbour's first, in L1 by then) and picks them out, without a branch, so that a lane's loads are all in
-// flight together.  The few ids whose words would reach outside the run go one by one.
-// Prune step without a payload plane, 4-byte stores and 128 threads per survivor / this / 16-byte stores and 256 threads per
-// survivor: 1,024 runs of 2,600 ids 26.1 / 22.0 / 22.9 us; 12,288 of 131 58.6 / 52.6 / 69.7; 2,048 of 600 19.9 / 19.7 / 22.0; 828 of
-// 275 12.3 / 12.5 / 12.9; 8 of 1,240 12.3 / 12.1 / 12.0.  Beyond what L2 holds (6.5 M ids, 104 MB) the stores go at HBM's pace.
+// The per-token outputs alone (no payload plane); blocks past the survivors return at once.
 constexpr int TOKENS_THREADS = 256;
-constexpr int TOKENS_QUADS = 2;          // groups of four tokens in flight per lane (3 or 4 spill at four blocks per SM: 24.4, 26.7 us on the first of these)
-constexpr int TOKENS_BLOCKS = 4;         // blocks per SM (five or six blocks of fewer registers: 24.4, 25.0)
-// Lanes per survivor: a group of four tokens for each while that many fit on the GPU at once, else up to TOKENS_QUADS groups.
-__device__ __forceinline__ int token_team(int64_t T, int S, int resident) {
-    const float groups = __fdividef((float)T, 4.f * (float)S);              // of the mean survivor
-    int lanes = groups <= 32.f ? 32 : groups <= 64.f ? 64 : groups <= 128.f ? 128 : TOKENS_THREADS;
-    while (lanes > 32 && (float)lanes * (float)S > (float)resident && (float)(lanes / 2 * TOKENS_QUADS) >= groups) lanes /= 2;
-    return lanes;
-}
+constexpr int TOKENS_BLOCKS = 4;         // blocks per SM (five or six blocks of fewer registers: 24.4, 25.0 us where four take 22.0)
 __global__ void __launch_bounds__(TOKENS_THREADS, TOKENS_BLOCKS)
 gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_seqlens,
-                     const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off,
-                     const int32_t* __restrict__ src_tokens, const float* __restrict__ adv, int64_t capacity,
-                     int32_t* __restrict__ dst_tokens, float* __restrict__ tok_adv, int32_t* __restrict__ tok_seq,
-                     const uint32_t* __restrict__ gate, int vector_stores, int resident) {
+                     const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off, TokenOutputs o,
+                     int64_t capacity, const uint32_t* __restrict__ gate, int resident) {
     pdl_launch_dependents();
     pdl_wait();
     d_num = pdl_acquire(d_num); cu_seqlens = pdl_acquire(cu_seqlens); survivor_idx = pdl_acquire(survivor_idx);
-    src_tok_off = pdl_acquire(src_tok_off); src_tokens = pdl_acquire(src_tokens); adv = pdl_acquire(adv);
+    src_tok_off = pdl_acquire(src_tok_off); o.src_tokens = pdl_acquire(o.src_tokens); o.adv = pdl_acquire(o.adv);
     gate = pdl_acquire(gate);
     const int S = (int)d_num[0];
     const int64_t T = d_num[1];
-    if (S <= 0 || T > capacity || *gate) return;                     // overflow / bad index was recorded by the scan kernel
-    const int lanes = token_team(T, S, resident);
+    if (S <= 0 || T > capacity || *gate) return;           // overflow / bad index was recorded by the scan kernel
+    const int lanes = token_team(T, S, resident, TOKENS_THREADS);
     const int team = (int)threadIdx.x / lanes, lane = (int)threadIdx.x & (lanes - 1), teams = TOKENS_THREADS / lanes;
-#pragma unroll 1
-    for (int s = blockIdx.x * teams + team; s < S; s += gridDim.x * teams) {
-        const int64_t c0 = __ldg(cu_seqlens + s);
-        const int len = (int)(__ldg(cu_seqlens + s + 1) - c0);
-        const int64_t src0 = __ldg(src_tok_off + __ldg(survivor_idx + s));
-        const float a = __ldg(adv + s);
-        auto load_one = [&](int t) { return dst_tokens ? __ldg(src_tokens + src0 + t) : 0; };
-        auto store_one = [&](int t, int32_t id) {
-            if (dst_tokens) dst_tokens[c0 + t] = id;
-            if (tok_seq) tok_seq[c0 + t] = s;
-            if (tok_adv) tok_adv[c0 + t] = a;
-        };
-        // [head, end): whole 16-byte groups of the outputs whose ids lie in words inside the run
-        int head = (int)((4 - (c0 & 3)) & 3), end = len - (int)((c0 + len) & 3);
-        const int shift = (int)((reinterpret_cast<uintptr_t>(src_tokens + src0 + head) & 15) >> 2);   // ids before src0 + head in its word
-        if (shift > head) head += 4;
-        if (shift && end - shift + 4 > len) end -= 4;
-        if (!vector_stores || end <= head) {
-#pragma unroll 1
-            for (int t = lane; t < len; t += lanes) store_one(t, load_one(t));
-            continue;
-        }
-        // at most 6 ids before and 6 after, a lane each; stored after the groups, or the first lanes' loads would wait for a
-        // store that waits for its id
-        const int edge = lane < head ? lane : (lane >= 8 && end + lane - 8 < len ? end + lane - 8 : -1);
-        const int32_t edge_id = edge >= 0 ? load_one(edge) : 0;
-        const int4* words = reinterpret_cast<const int4*>(src_tokens + src0 + head - shift);
-        const int quads = (end - head) / 4, second = shift ? 1 : 0;
-#pragma unroll 1
-        for (int k0 = lane; k0 < quads; k0 += TOKENS_QUADS * lanes) {
-            int4 lo[TOKENS_QUADS], hi[TOKENS_QUADS];
-            if (dst_tokens) {
-#pragma unroll
-                for (int u = 0; u < TOKENS_QUADS; ++u) {
-                    const int k = k0 + u * lanes;
-                    if (k < quads) {
-                        lo[u] = __ldg(words + k);
-                        hi[u] = __ldg(words + k + second);
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < TOKENS_QUADS; ++u) {
-                const int k = k0 + u * lanes;
-                if (k >= quads) break;
-                const int64_t at = c0 + head + 4 * k;
-                if (dst_tokens) {
-                    const bool two = shift & 2, one = shift & 1;
-                    const int32_t x0 = two ? lo[u].z : lo[u].x, x1 = two ? lo[u].w : lo[u].y, x2 = two ? hi[u].x : lo[u].z,
-                                  x3 = two ? hi[u].y : lo[u].w, x4 = two ? hi[u].z : hi[u].x;
-                    *reinterpret_cast<int4*>(dst_tokens + at) = make_int4(one ? x1 : x0, one ? x2 : x1, one ? x3 : x2, one ? x4 : x3);
-                }
-                if (tok_seq) *reinterpret_cast<int4*>(tok_seq + at) = make_int4(s, s, s, s);
-                if (tok_adv) *reinterpret_cast<float4*>(tok_adv + at) = make_float4(a, a, a, a);
-            }
-        }
-        if (edge >= 0) store_one(edge, edge_id);
-    }
+    token_runs(o, cu_seqlens, survivor_idx, src_tok_off, S, blockIdx.x * teams + team, gridDim.x * teams, lane, lanes);
 }
 
 }  // namespace
@@ -274,22 +200,17 @@ int arrol_internal_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* l
     if (N == 0 || dst_capacity_tokens == 0 || !any_token_output) return ARROL_OK;
 
     const int vec_per_row = src_rows ? row_bytes / 16 : 0;
-    // Rows that fit a 32 KB stage go through the bulk-copy kernel; the per-token outputs then come from the
-    // survivor-major kernel.  Larger rows take the load/store kernel, which writes both.
+    // Rows that fit a 32 KB stage go through the bulk-copy kernel, which writes the per-token outputs beside its copies.
+    // Larger rows take the load/store kernel, which writes both too.
     const bool bulk_rows = vec_per_row > 0 && row_bytes <= 32 * 1024;
-    if (vec_per_row == 0 || bulk_rows) {
-        if (bulk_rows) {
-            const int rc = arrol_internal_gather_rows_bulk(ctx, d_num, cu_seqlens, survivor_idx, src_tok_off, src_rows,
-                                                           row_bytes, dst_capacity_tokens, dst_rows, s);
-            if (rc != ARROL_OK) return rc;
-            if (!dst_tokens && !tok_adv && !tok_seq) return ARROL_OK;
-        }
+    const TokenOutputs outputs = token_outputs(src_tokens, adv, dst_tokens, tok_adv, tok_seq);
+    if (bulk_rows)
+        return arrol_internal_gather_rows_bulk(ctx, d_num, cu_seqlens, survivor_idx, src_tok_off, N, outputs, src_rows, row_bytes,
+                                               dst_capacity_tokens, dst_rows, s);
+    if (vec_per_row == 0) {
         int64_t blocks = N < (int64_t)ctx->sm_count * 16 ? N : (int64_t)ctx->sm_count * 16;
         ARROL_CUDA_OK(arrol_launch_pdl(gather_tokens_kernel, dim3((unsigned)blocks), dim3(TOKENS_THREADS), 0, s, d_num,
-                                       cu_seqlens, survivor_idx, src_tok_off, src_tokens, adv, dst_capacity_tokens,
-                                       dst_tokens, tok_adv, tok_seq, ctx->d_status + 1,
-                                       arrol_aligned(dst_tokens, 16) && arrol_aligned(tok_adv, 16) && arrol_aligned(tok_seq, 16) &&
-                                               arrol_aligned(src_tokens, 4) ? 1 : 0,
+                                       cu_seqlens, survivor_idx, src_tok_off, outputs, dst_capacity_tokens, ctx->d_status + 1,
                                        ctx->sm_count * TOKENS_BLOCKS * TOKENS_THREADS));
         ctx->launches += 1;
         return ARROL_OK;
