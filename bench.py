@@ -833,7 +833,7 @@ def report(res, peaks, tokens_all, ms_per_step, e2e_ms, world):
                          "token_logprob": logp_ms_step},
         "logprob_tokens_per_s": T / (logp_ms_step * 1e-3),
         "prune_step_us": res["prune_us"],
-        "compact_roofline": {"kernel": "gather_rows_bulk_kernel (+ scan_adv_kernel)", "bound": "hbm",
+        "compact_roofline": {"kernel": "gather_rows_bulk_kernel (+ scan_adv_kernel, gather_tokens_kernel)", "bound": "hbm",
                              "achieved": compact_gbs, "peak": float(peaks["hbm_gbs"]), "unit": "GB/s",
                              "frac": compact_gbs / float(peaks["hbm_gbs"]), "frac_of_nominal_8000": compact_gbs / 8000.0,
                              "algorithmic_bytes_per_launch": gather_bytes / C},

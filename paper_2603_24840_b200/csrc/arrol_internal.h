@@ -145,6 +145,7 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
 // gather_bulk.cu: the survivors' rows moved by bulk copies through shared memory.  ARROL_ERR_UNSUPPORTED (nothing
 // launched) when a row does not fit a 32 KB stage.
 struct TokenOutputs;   // token_runs.cuh
+bool arrol_internal_gather_rows_writes_tokens(int64_t row_bytes, int64_t capacity);   // gather_bulk.cu
 int arrol_internal_gather_rows_bulk(arrol_ctx* ctx, const int64_t* d_num, const int64_t* cu_seqlens,
                                     const int32_t* survivor_idx, const int64_t* src_tok_off, int N, const TokenOutputs& outputs,
                                     const void* src_rows, int64_t row_bytes, int64_t capacity, void* dst_rows, cudaStream_t s);

@@ -5,7 +5,8 @@
 //   survivor_idx, cu_seqlens, {S, T}, and per-survivor advantages (fp64 statistics over the kept rollouts of
 //   the group, in index order, rounded once to fp32).
 // Kernel 2: the per-token outputs (token id, survivor ordinal, advantage), a team of lanes per survivor, and, when there is
-//   a hidden-row plane, beside them the rows by bulk copies through shared memory (gather_bulk.cu).  Rows too large
+//   a hidden-row plane, the rows by bulk copies through shared memory (gather_bulk.cu), which writes the per-token outputs
+//   too while the packed rows fit L2.  Rows too large
 //   for a bulk stage take gather_kernel below: one wave of persistent blocks, each owning a contiguous run of
 //   destination tiles; one thread per row finds its survivor (binary search once per block, then a forward walk in
 //   cu_seqlens), then the block streams the tile's payload with 16-byte loads/stores, eight in flight per thread.
@@ -131,6 +132,13 @@ gather_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_
 // The per-token outputs alone (no payload plane); blocks past the survivors return at once.
 constexpr int TOKENS_THREADS = 256;
 constexpr int TOKENS_BLOCKS = 4;         // blocks per SM (five or six blocks of fewer registers: 24.4, 25.0 us where four take 22.0)
+// Lanes per survivor: a group of four tokens for each while that many fit on the GPU at once, else up to TOKENS_QUADS groups.
+__device__ __forceinline__ int token_team(int64_t T, int S, int resident) {
+    const float groups = __fdividef((float)T, 4.f * (float)S);              // of the mean survivor
+    int lanes = groups <= 32.f ? 32 : groups <= 64.f ? 64 : groups <= 128.f ? 128 : TOKENS_THREADS;
+    while (lanes > 32 && (float)lanes * (float)S > (float)resident && (float)(lanes / 2 * TOKENS_QUADS) >= groups) lanes /= 2;
+    return lanes;
+}
 __global__ void __launch_bounds__(TOKENS_THREADS, TOKENS_BLOCKS)
 gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_seqlens,
                      const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off, TokenOutputs o,
@@ -143,7 +151,7 @@ gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restric
     const int S = (int)d_num[0];
     const int64_t T = d_num[1];
     if (S <= 0 || T > capacity || *gate) return;           // overflow / bad index was recorded by the scan kernel
-    const int lanes = token_team(T, S, resident, TOKENS_THREADS);
+    const int lanes = token_team(T, S, resident);
     const int team = (int)threadIdx.x / lanes, lane = (int)threadIdx.x & (lanes - 1), teams = TOKENS_THREADS / lanes;
     token_runs(o, cu_seqlens, survivor_idx, src_tok_off, S, blockIdx.x * teams + team, gridDim.x * teams, lane, lanes);
 }
@@ -200,14 +208,18 @@ int arrol_internal_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* l
     if (N == 0 || dst_capacity_tokens == 0 || !any_token_output) return ARROL_OK;
 
     const int vec_per_row = src_rows ? row_bytes / 16 : 0;
-    // Rows that fit a 32 KB stage go through the bulk-copy kernel, which writes the per-token outputs beside its copies.
+    // Rows that fit a 32 KB stage go through the bulk-copy kernel; the per-token outputs are written beside its copies or after.
     // Larger rows take the load/store kernel, which writes both too.
     const bool bulk_rows = vec_per_row > 0 && row_bytes <= 32 * 1024;
     const TokenOutputs outputs = token_outputs(src_tokens, adv, dst_tokens, tok_adv, tok_seq);
-    if (bulk_rows)
-        return arrol_internal_gather_rows_bulk(ctx, d_num, cu_seqlens, survivor_idx, src_tok_off, N, outputs, src_rows, row_bytes,
-                                               dst_capacity_tokens, dst_rows, s);
-    if (vec_per_row == 0) {
+    if (vec_per_row == 0 || bulk_rows) {
+        if (bulk_rows) {
+            const bool beside = arrol_internal_gather_rows_writes_tokens(row_bytes, dst_capacity_tokens);
+            const int rc = arrol_internal_gather_rows_bulk(ctx, d_num, cu_seqlens, survivor_idx, src_tok_off, N,
+                                                           beside ? outputs : TokenOutputs{}, src_rows, row_bytes, dst_capacity_tokens,
+                                                           dst_rows, s);
+            if (rc != ARROL_OK || beside || !outputs.any()) return rc;
+        }
         int64_t blocks = N < (int64_t)ctx->sm_count * 16 ? N : (int64_t)ctx->sm_count * 16;
         ARROL_CUDA_OK(arrol_launch_pdl(gather_tokens_kernel, dim3((unsigned)blocks), dim3(TOKENS_THREADS), 0, s, d_num,
                                        cu_seqlens, survivor_idx, src_tok_off, outputs, dst_capacity_tokens, ctx->d_status + 1,

@@ -12,10 +12,8 @@
 //                        shared-memory stages; completion by transaction count on the stage's mbarrier
 //   thread 32 (storer)   waits for a stage, issues one bulk store of the tile to its (contiguous) destination, and
 //                        frees a stage once the store that used it has finished reading shared memory
-//   threads 64 ...       write the per-token outputs (token_runs.cuh) meanwhile: they need only what the row copies need, and
-//                        neither the queues nor HBM notice.  A kernel of its own after this one cost 2-5 us a
-//                        call: 16 rollouts 18.7 -> 16.5 us for the prune step, 256 141 -> 137, 6,144 runs of 131 ids 314 -> 309,
-//                        1.67 GB of rows 575 -> 572
+//   threads 64 ... 95    a warp that writes the per-token outputs meanwhile (token_runs.cuh), when asked to: see
+//                        gather_rows_writes_tokens for when
 // Every wait is bounded; on expiry the block records ARROL_DEV_WAIT_EXPIRED, lets its copies land and returns.
 #include "arrol_internal.h"
 #include "tc_common.cuh"
@@ -27,8 +25,8 @@ constexpr int GB_STAGES = 2;
 constexpr int GB_BLOCKS_PER_SM = 3;
 static_assert(GB_STAGES >= 2, "the storer frees a stage only after it has issued the following store");
 constexpr int GB_TILE_BYTES = 32 * 1024;
-constexpr int GB_TOKEN_THREADS = 128;    // behind the producer's and the storer's warp
-constexpr int GB_THREADS = 64 + GB_TOKEN_THREADS;
+constexpr int GB_COPY_THREADS = 64;        // the producer's warp and the storer's
+constexpr int GB_THREADS = GB_COPY_THREADS + 32;   // and one for the per-token outputs
 constexpr size_t GB_SMEM = (size_t)GB_STAGES * GB_TILE_BYTES + 1024 + 256;
 
 __device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
@@ -151,11 +149,9 @@ gather_rows_bulk_kernel(const int64_t* __restrict__ d_num, const int64_t* __rest
             if (++stage == GB_STAGES) { stage = 0; phase ^= 1u; }
         }
         bulk_wait_all();                                  // stores complete before the block's shared memory goes
-    } else if (threadIdx.x >= 64 && o.any()) {
+    } else if (threadIdx.x >= GB_COPY_THREADS) {
         // ---------------- per-token outputs ----------------
-        const int lanes = token_team(T, S, (int)gridDim.x * GB_TOKEN_THREADS, GB_TOKEN_THREADS);
-        const int t = (int)threadIdx.x - 64, teams = GB_TOKEN_THREADS / lanes;
-        token_runs(o, cu_seqlens, survivor_idx, src_tok_off, S, blockIdx.x * teams + t / lanes, gridDim.x * teams, t & (lanes - 1), lanes);
+        token_runs(o, cu_seqlens, survivor_idx, src_tok_off, S, blockIdx.x, gridDim.x, (int)threadIdx.x - GB_COPY_THREADS, 32);
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort_flag) atomicOr(d_status, ARROL_DEV_WAIT_EXPIRED);
@@ -163,7 +159,13 @@ gather_rows_bulk_kernel(const int64_t* __restrict__ d_num, const int64_t* __rest
 
 }  // namespace
 
-// Moves the survivors' rows with bulk copies.  ARROL_ERR_UNSUPPORTED (nothing launched) for rows that do not fit a
+// Per-token outputs beside the row copies, or by a kernel of their own after them.  Beside them they save that kernel's launch
+// and round trips: prune step of 16 rollouts 18.9 -> 16.5 us, 512 in runs of 200 32.2 -> 27.5.  Only while the packed rows stay in L2: a
+// gather at HBM's pace gained 0.1-3 % on most shapes, but lost 5-15 % on some with long runs (1.0 M tokens in runs of 1,500 to 4,500,
+// 4.6 KB rows 1,312 -> 1,434 us with one warp; 2.7 M tokens, 5 KB rows 4,377 -> 5,055 with four), for a reason that was not found.
+bool arrol_internal_gather_rows_writes_tokens(int64_t row_bytes, int64_t capacity) { return capacity <= L2_BYTES / row_bytes; }
+
+// Moves the survivors' rows with bulk copies, and writes the per-token outputs unless `outputs` is empty.  ARROL_ERR_UNSUPPORTED (nothing launched) for rows that do not fit a
 // stage; the caller then takes the load/store kernel.
 int arrol_internal_gather_rows_bulk(arrol_ctx* ctx, const int64_t* d_num, const int64_t* cu_seqlens,
                                     const int32_t* survivor_idx, const int64_t* src_tok_off, int N, const TokenOutputs& outputs,
@@ -183,7 +185,7 @@ int arrol_internal_gather_rows_bulk(arrol_ctx* ctx, const int64_t* d_num, const 
     const int64_t wanted = max_tiles > N || !outputs.any() ? max_tiles : N;
     if (blocks > wanted) blocks = wanted;
     if (blocks < 1) blocks = 1;
-    ARROL_CUDA_OK(arrol_launch_pdl(gather_rows_bulk_kernel, dim3((unsigned)blocks), dim3(GB_THREADS), GB_SMEM, s, d_num,
+    ARROL_CUDA_OK(arrol_launch_pdl(gather_rows_bulk_kernel, dim3((unsigned)blocks), dim3(outputs.any() ? GB_THREADS : GB_COPY_THREADS), GB_SMEM, s, d_num,
                                    cu_seqlens, survivor_idx, src_tok_off, static_cast<const uint8_t*>(src_rows),
                                    row_bytes, capacity, tile_rows, static_cast<uint8_t*>(dst_rows), outputs, ctx->d_status));
     ctx->launches += 1;

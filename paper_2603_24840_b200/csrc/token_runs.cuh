@@ -1,5 +1,5 @@
 // Per-token outputs of the compaction (token ids, survivor ordinal, advantage): device code of the kernel that writes them
-// alone (gather_tokens_kernel) and of the row gather, which writes them beside its copies (gather_rows_bulk_kernel).
+// alone (gather_tokens_kernel) and of the row gather, which writes them beside its copies while these fit L2 (gather_rows_bulk_kernel).
 #pragma once
 #include "arrol_internal.h"
 
@@ -27,14 +27,6 @@ inline TokenOutputs token_outputs(const int32_t* src_tokens, const float* adv, i
 // survivor: 1,024 runs of 2,600 ids 26.1 / 22.0 / 22.9 us; 12,288 of 131 58.6 / 52.6 / 69.7; 2,048 of 600 19.9 / 19.7 / 22.0; 828 of
 // 275 12.3 / 12.5 / 12.9; 8 of 1,240 12.3 / 12.1 / 12.0.  Beyond what L2 holds (6.5 M ids, 104 MB) the stores go at HBM's pace.
 constexpr int TOKENS_QUADS = 2;          // groups of four tokens in flight per lane (3 or 4 spill at four blocks per SM: 24.4, 26.7 us on the first of these)
-// Lanes per survivor: a group of four tokens for each while that many fit on the GPU at once, else up to TOKENS_QUADS groups.
-__device__ __forceinline__ int token_team(int64_t T, int S, int resident, int most) {
-    const float groups = __fdividef((float)T, 4.f * (float)S);              // of the mean survivor
-    int lanes = groups <= 32.f ? 32 : groups <= 64.f ? 64 : groups <= 128.f ? 128 : most;
-    if (lanes > most) lanes = most;
-    while (lanes > 32 && (float)lanes * (float)S > (float)resident && (float)(lanes / 2 * TOKENS_QUADS) >= groups) lanes /= 2;
-    return lanes;
-}
 // Survivors first, first + step, ... by lane `lane` of a team of `lanes`.
 __device__ __forceinline__ void token_runs(const TokenOutputs& o, const int64_t* __restrict__ cu_seqlens, const int32_t* __restrict__ survivor_idx,
                                            const int64_t* __restrict__ src_tok_off, int S, int first, int step, int lane, int lanes) {
