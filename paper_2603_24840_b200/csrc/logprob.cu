@@ -48,6 +48,7 @@
 // fell from 1.27 to 0.8 GHz under the power cap).
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <float.h>
 
 #include "arrol_internal.h"
 #include "tc_common.cuh"
@@ -91,7 +92,7 @@ struct VocabPlan {
 // (M, L) <- (M, L) + (m, l): M = max, L = sum of 2^(. - M).  One rounding per operation, so that the main kernel (body)
 // and the combining kernel (tail) get the same bits.
 __device__ __forceinline__ void merge_lse(float& M, float& L, float m, float l) {
-    if (m == -INFINITY) return;                                 // no column in the record
+    if (l == 0.f) return;                                       // nothing in the record (a NaN is something)
     const float Mn = fmaxf(M, m);
     L = __fadd_rn(__fmul_rn(L, ex2_approx(M - Mn)), __fmul_rn(l, ex2_approx(m - Mn)));
     M = Mn;
@@ -101,7 +102,9 @@ __device__ __forceinline__ void merge_record(PartialLse& a, const PartialLse& b)
     a.zy2 = fmaxf(a.zy2, b.zy2);        // exactly one record holds the target column, the others hold -inf
     a.sumz = __fadd_rn(a.sumz, b.sumz);
 }
-__device__ __forceinline__ PartialLse empty_record() { return PartialLse{-INFINITY, 0.f, -INFINITY, 0.f}; }
+// The maximum starts at the lowest finite number: columns that are all -inf then add 2^(-inf) = 0 and leave the record empty, while
+// NaN columns, which no maximum shows, make the sum NaN.  (From -inf both would end as -inf - -inf = NaN.)
+__device__ __forceinline__ PartialLse empty_record() { return PartialLse{-FLT_MAX, 0.f, -INFINITY, 0.f}; }
 
 // Work of one launch on `tiles` token tiles (128 rows, or 256 for a pair of blocks).  32-bit throughout (fewer than 2^24 tiles
 // and at most 64 groups): the divisions are on the way of every work item and of the combining kernel.
