@@ -117,7 +117,8 @@ int arrol_score_partial(arrol_ctx* ctx, const void* hidden, int64_t row_stride_e
  * is the member whose removal leaves the group mean closest to rho; of equal candidates the one with the
  * highest index is removed, so the lower index survives.  Keys are evaluated in double, one rounding per
  * operation, so the result is reproducible bit for bit.  keep [P*G] uint8 receives 1 (kept) / 0 (pruned).
- * mode must be 0.  Supported: 1 <= K <= G <= 32.  q must be finite.  P == 0 is a no-op. */
+ * mode must be 0.  Supported: 1 <= K <= G <= 32.  q must be finite (of a group with a NaN or an infinity K members stay as well,
+ * but which ones is not defined).  P == 0 is a no-op. */
 int arrol_select(arrol_ctx* ctx, const float* q, int32_t P, int32_t G, int32_t K, double rho, int32_t mode,
                  uint8_t* keep, void* stream);
 

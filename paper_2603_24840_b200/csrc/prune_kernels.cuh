@@ -110,8 +110,9 @@ __device__ __forceinline__ bool select_lanes(double qj, bool member, int j, int 
     for (int i = 0; i < G; ++i) sigma = __dadd_rn(sigma, shfl_double(qj, i, seg));
     for (int n = G; n > K; --n) {
         const double tau = __dsub_rn(sigma, __dmul_rn(rho, (double)(n - 1)));
-        // non-negative doubles order like their bit patterns, and an integer compare is several times faster than fp64's
-        unsigned long long key = alive ? (unsigned long long)__double_as_longlong(fabs(__dsub_rn(qj, tau))) : 0x7ff0000000000000ull;
+        // non-negative doubles order like their bit patterns, and an integer compare is several times faster than fp64's; lanes
+        // that are out take the largest pattern, above a NaN's, so that a member goes whatever the keys are
+        unsigned long long key = alive ? (unsigned long long)__double_as_longlong(fabs(__dsub_rn(qj, tau))) : ~0ull;
         int idx = alive ? j : -1;
         // segmented arg-min; ties -> the higher index
 #pragma unroll
@@ -122,7 +123,7 @@ __device__ __forceinline__ bool select_lanes(double qj, bool member, int j, int 
                 if (okey < key || (okey == key && oidx > idx)) { key = okey; idx = oidx; }
             }
         }
-        const double q_removed = shfl_double(qj, idx < 0 ? 0 : idx, seg);
+        const double q_removed = shfl_double(qj, idx < 0 ? 0 : idx, seg);   // idx < 0: no member at all (padding segment)
         if (idx == j) alive = false;
         sigma = __dsub_rn(sigma, q_removed);
     }

@@ -1,10 +1,13 @@
 """Non-finite values stay where they belong: a NaN logit makes its token's log-prob and log-sum-exp NaN wherever in the
-vocabulary it stands, a logit of minus infinity only leaves the sum, and other tokens keep their bits."""
+vocabulary it stands, a logit of minus infinity only leaves the sum, and other tokens keep their bits; a group with a
+non-finite score keeps K members like any other, and the other groups keep theirs."""
 import numpy as np
 import pytest
 import torch
 
 from paper_2603_24840_b200 import binding as B
+from paper_2603_24840_b200 import synth
+from paper_2603_24840_b200.pipeline import PruneRebatch, host_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +62,48 @@ def test_logprob_of_non_finite_logits(T, d, V):
         hit = ref_p.isinf()
         assert torch.equal(logp[some][hit], ref_p[hit].float()) and (logp[some][~hit].double() - ref_p[~hit]).abs().max() <= 2e-3
     ctx.close()
+
+
+@pytest.mark.parametrize("G,K", [(8, 4), (12, 6), (32, 1), (5, 5), (2, 1)])
+def test_a_group_with_a_non_finite_score_keeps_exactly_k(G, K):
+    """All keys of such a group are NaN or infinite: whoever goes, exactly K of it stay, and the other groups keep theirs."""
+    ctx = B.Context(0)
+    P = 9
+    q = np.random.default_rng(G).random((P, G)).astype(np.float32)
+    want = torch.full((P, G), 9, dtype=torch.uint8, device="cuda")
+    B.arrol_select(ctx, torch.from_numpy(q).cuda(), P, G, K, 0.5, want)
+    bad = q.copy()
+    bad[1, 0] = np.nan
+    bad[3, :] = np.nan
+    bad[4, G - 1] = np.inf
+    bad[7, G // 2] = -np.inf
+    keep = torch.full((P, G), 9, dtype=torch.uint8, device="cuda")
+    B.arrol_select(ctx, torch.from_numpy(bad).cuda(), P, G, K, 0.5, keep)
+    torch.cuda.synchronize()
+    assert (keep.sum(1) == K).all() and keep.max() <= 1
+    rest = [0, 2, 5, 6, 8]
+    assert torch.equal(keep[rest], want[rest])
+    ctx.close()
+
+
+@pytest.mark.parametrize("name", ["mini", "profile-mlp"])
+def test_a_rollout_with_a_nan_hidden_row_leaves_the_other_groups_alone(name):
+    w = synth.WORKLOADS[name]
+    pr = PruneRebatch(w, inputs=host_inputs(w))
+    pr.q_lut = None                                    # q is the score's sigmoid itself: NaN for a NaN row
+    pr.prune_step()
+    torch.cuda.synchronize()
+    want = pr.keep.clone().view(w.P, w.G)
+    bad = 2 * w.G + 1
+    pr.hidden_score[pr.row_index[bad]] = float("nan")
+    rest = [p for p in range(w.P) if p != 2]
+    for run in (pr.prune_step, lambda: B.arrol_prune_step(pr.ctx, pr.prune_step_args())):
+        pr.keep.fill_(9)
+        run()
+        torch.cuda.synchronize()
+        keep = pr.keep.view(w.P, w.G)
+        assert pr.q[bad].isnan()
+        assert (keep.sum(1) == w.K).all() and torch.equal(keep[rest], want[rest])
+        assert pr.counts()[0] == w.P * w.K
+        assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == 0
+    pr.ctx.close()
