@@ -227,7 +227,8 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     // evaluates 31 points a round (one warp each) and the first warp replays the bisection as far as the settled points
     // reach.  Rounds 0 and 1 take the 31 midpoints of the next five levels; round 2 takes points at growing distances around
     // the root of the linear piece that E is on by then, which settles most of the remaining levels; then five levels a
-    // round again until the bracket stops shrinking.
+    // round again until the bracket stops shrinking.  Every round of midpoints settles one step at least (its first point is
+    // the next midpoint), so 65 rounds are always enough, and no more are made.
     //   One evaluation: the lanes form the per-bin products c_b p_b (all >= 0) and a butterfly sum S of them; the in-order sum
     // differs from S by at most (B + 8) 2^-53 S (both are within their standard error bounds of the exact sum), so when S is
     // further from kappa n than four times that bound plus the roundings of the division and of kappa n, S < kappa n already
@@ -248,8 +249,11 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
         double lo = -(1.0 + lambda), hi = 1.0 + lambda;           // the first warp's
         double known_below = lo - 1.0, known_above = hi + 1.0;    // settled points next to the threshold
         double sum_at = 0.0, slope_at = 0.0;                      // S and dS/d(delta) at known_below
-        int step = 0;
-        for (int round = 0;; ++round) {
+        // infinite lambda: the first midpoint is NaN, no comparison holds, and a plain loop ends at NaN.  (A finite bracket
+        // never gets there: its midpoints can overflow, but not with opposite signs.)
+        int step = isinf(lambda) ? 64 : 0;
+        if (step) hi = midpoint(lo, hi);
+        for (int round = 0; round <= 65; ++round) {
             if (wid == 0) {
                 for (; step < 64; ++step) {
                     const double m = midpoint(lo, hi);

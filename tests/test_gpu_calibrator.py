@@ -88,6 +88,25 @@ def test_delta_is_bit_equal_over_many_states_and_parameters(ctx):
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
 
 
+@pytest.mark.parametrize("lam", [0.0, 1e17, 1e300, 1.7e308, float("inf")])
+@pytest.mark.parametrize("alpha", [1.0, 0.0])                 # alpha = 0: empty bins have the posterior 0 / 0
+def test_delta_of_extreme_parameters_ends_where_a_plain_loop_does(ctx, lam, alpha):
+    g = np.random.default_rng(9)
+    for n_bins in (1, 16, 720):
+        cal = CAL.Calibrator(ctx, n_bins, 300, alpha=alpha)
+        prob = g.beta(2, 2, size=200).astype(np.float32)
+        rew = (g.random(200) < prob).astype(np.float32)
+        bins = np.array([oracle.bin_index(float(v), n_bins) for v in prob], dtype=np.int32)
+        for kappa, pmin, pmax in ((0.5, 0.05, 0.95), (0.0, 0.0, 1.0), (1.0, 0.0, 1.0)):
+            cal.update(torch.from_numpy(bins).cuda(), torch.from_numpy(rew).cuda(), CAL.survival(kappa, lam, 0.5, pmin, pmax))
+            torch.cuda.synchronize()
+            snap = cal.snapshot()
+            with np.errstate(all="ignore"):
+                delta = oracle.solve_delta(snap["cpos"], snap["cneg"], snap["q_lut"], kappa, lam, 0.5, pmin, pmax, iters=64)
+            assert np.array_equal(snap["delta"], delta, equal_nan=True), (n_bins, kappa)
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+
+
 def test_stochastic_selection_matches_oracle(ctx):
     g = np.random.default_rng(5)
     N = 100003
