@@ -71,8 +71,11 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 // One block, bound by latency: a handful of dependent round trips to memory and a serial search.  Every input is read once
 // (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
 // that one block scan ranks all of them, and the bisection is settled in about five rounds of 31 points (see below) instead
-// of 64 steps, twenty of them with a serial sum.  Per call: N = 2,048, 128 bins 61.5 -> 26.7 us; N = 32, 64 bins 41 -> 22 us;
-// N = 8,192, 256 bins 100 -> 37 us.
+// of 64 steps, twenty of them with a serial sum.  Per call, timed back to back: N = 2,048, 128 bins 61.5 -> 26.7 us; N = 32,
+// 64 bins 41 -> 22 us; N = 8,192, 256 bins 100 -> 37 us.  More rollouts go through shared memory in pieces of CAL_STAGED,
+// after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
+// touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
+// per thread and scan, as it was before the runs, 460 and 1,570).
 constexpr int CAL_STAGED = 8192;
 constexpr int CAL_POINTS = 31;                 // points per round, one warp each
 __host__ __device__ inline int product_pitch(int B) { return B | 1; }      // odd: 31 lanes walk 31 rows without bank conflicts
@@ -95,17 +98,20 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     extern __shared__ double products[];        // [31][B rounded up to odd]: c_b p_b of a round's points
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
-    auto code_of = [&](int i) {
+    auto code_of = [&](int64_t i) {
         if (mask && !mask[i]) return -1;
         int b = bin[i];
         b = b < 0 ? 0 : (b >= B ? B - 1 : b);
         return 2 * b + (rewards[i] > 0.5f ? 1 : 0);
     };
-    const bool in_shared = N <= CAL_STAGED;
-    if (in_shared) {
+    auto stage = [&](int64_t from) {
+        const int n = (int)min((int64_t)CAL_STAGED, N - from);
 #pragma unroll 4
-        for (int i = tid; i < N; i += CAL_THREADS) staged[i] = (int16_t)code_of(i);
-    }
+        for (int j = tid; j < n; j += CAL_THREADS) staged[j] = (int16_t)code_of(from + j);
+        return n;
+    };
+    const bool one_piece = N <= CAL_STAGED;
+    if (one_piece) stage(0);
     // The byte layout L comes from the call's (B, cap); the state must have been initialised with the same pair.
     // A mismatched or uninitialised state is left untouched and reported (uniform over the block: no barrier yet).
     if (hd->B != B || hd->cap != cap) {
@@ -121,40 +127,59 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     if (tid < B) { old_cnt[0] = cnt[0][tid]; old_cnt[1] = cnt[1][tid]; hist[0][tid] = 0; hist[1][tid] = 0; }
     __syncthreads();
 
-    // rank of every new entry among those of its label, in index order
-    const int per = (N + CAL_THREADS - 1) / CAL_THREADS;
-    const int i0 = min(N, tid * per), i1 = min(N, i0 + per);
-    auto code = [&](int i) { return in_shared ? (int)staged[i] : code_of(i); };
-    int32_t mine[2] = {0, 0};
-    for (int i = i0; i < i1; ++i) {
-        const int c = code(i);
-        if (c >= 0) mine[c & 1] += 1;
-    }
-    int32_t incl[2];
+    // Sums over the block of two counts per thread (one barrier), and the sums of the threads before this one.
+    auto block_scan = [&](const int32_t (&mine)[2], int64_t (&before)[2], int64_t (&total)[2]) {
+        int32_t incl[2];
 #pragma unroll
-    for (int l = 0; l < 2; ++l) {
-        int32_t v = mine[l];
+        for (int l = 0; l < 2; ++l) {
+            int32_t v = mine[l];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += t;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += t;
+            }
+            incl[l] = v;
+            if (lane == 31) warp_sum[l][wid] = v;
         }
-        incl[l] = v;
-        if (lane == 31) warp_sum[l][wid] = v;
-    }
-    __syncthreads();
+        __syncthreads();
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {            // every warp scans the warp totals for itself
+            int32_t v = warp_sum[l][lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += t;
+            }
+            total[l] = __shfl_sync(0xffffffffu, v, 31);
+            const int32_t warps_before = __shfl_sync(0xffffffffu, v, wid > 0 ? wid - 1 : 0);
+            before[l] = (wid > 0 ? warps_before : 0) + incl[l] - mine[l];
+        }
+    };
+    // This thread's run [j0, j1) of the n staged entries, and the rank of its first one among those of its label.
+    auto rank_run = [&](int n, int& j0, int& j1, int64_t (&first_rank)[2], int64_t (&total)[2]) {
+        const int per = (n + CAL_THREADS - 1) / CAL_THREADS;
+        j0 = min(n, tid * per);
+        j1 = min(n, j0 + per);
+        int32_t mine[2] = {0, 0};
+        for (int j = j0; j < j1; ++j) {
+            const int c = staged[j];
+            if (c >= 0) mine[c & 1] += 1;
+        }
+        block_scan(mine, first_rank, total);
+    };
+    int j0 = 0, j1 = 0;
     int64_t total_new[2], first_rank[2];
-#pragma unroll
-    for (int l = 0; l < 2; ++l) {                // every warp scans the warp totals for itself
-        int32_t v = warp_sum[l][lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += t;
+    if (one_piece) {
+        rank_run(N, j0, j1, first_rank, total_new);
+    } else {                                     // how many there are of each label decides what is evicted and what stays
+        int32_t mine[2] = {0, 0};
+#pragma unroll 8
+        for (int64_t i = tid; i < N; i += CAL_THREADS) {
+            const bool on = !mask || mask[i], pos = rewards[i] > 0.5f;
+            mine[0] += on && !pos ? 1 : 0;
+            mine[1] += on && pos ? 1 : 0;
         }
-        total_new[l] = __shfl_sync(0xffffffffu, v, 31);
-        const int32_t before = __shfl_sync(0xffffffffu, v, wid > 0 ? wid - 1 : 0);
-        first_rank[l] = (wid > 0 ? before : 0) + incl[l] - mine[l];
+        block_scan(mine, first_rank, total_new);
     }
 
     // evict the oldest entries that the push displaces (read the rings before they are overwritten)
@@ -172,18 +197,33 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     // entry r of m lands in slot (head + n + r) mod cap, and only the last `cap` of them survive the call
     {
         const int64_t slot0[2] = {(head0[0] + n0[0]) % cap, (head0[1] + n0[1]) % cap};
-        int64_t r[2] = {first_rank[0], first_rank[1]};
-        for (int i = i0; i < i1; ++i) {
-            const int c = code(i);
-            if (c < 0) continue;
-            const int l = c & 1;
-            const int64_t rank = l ? r[1]++ : r[0]++;
-            if (rank >= total_new[l] - cap) {
-                const int64_t at = slot0[l] + (rank < cap ? rank : rank % cap);
-                ring[l][at < cap ? at : at - cap] = (int16_t)(c >> 1);
-                atomicAdd(&hist[l][c >> 1], 1);
+        auto write_run = [&](const int64_t (&before)[2]) {
+            int64_t r[2] = {before[0] + first_rank[0], before[1] + first_rank[1]};
+            for (int j = j0; j < j1; ++j) {
+                const int c = staged[j];
+                if (c < 0) continue;
+                const int l = c & 1;
+                const int64_t rank = l ? r[1]++ : r[0]++;
+                if (rank >= total_new[l] - cap) {
+                    const int64_t at = slot0[l] + (rank < cap ? rank : rank % cap);
+                    ring[l][at < cap ? at : at - cap] = (int16_t)(c >> 1);
+                    atomicAdd(&hist[l][c >> 1], 1);
+                }
             }
-        }
+        };
+        int64_t before[2] = {0, 0};
+        if (one_piece) write_run(before);
+        else
+            for (int64_t from = 0; from < N; from += CAL_STAGED) {
+                int64_t here[2];
+                const int n = stage(from);
+                __syncthreads();
+                rank_run(n, j0, j1, first_rank, here);
+                write_run(before);
+                before[0] += here[0];
+                before[1] += here[1];
+                __syncthreads();                 // the staged entries and the warp sums are overwritten by the next piece
+            }
     }
     __syncthreads();
 

@@ -60,6 +60,11 @@ def test_calibrator_update_beyond_the_staged_rollouts(ctx, n_bins, cap, sizes):
     test_calibrator_update_matches_oracle(ctx, n_bins, cap, sizes)
 
 
+@pytest.mark.parametrize("n_bins,cap,sizes", [(128, 5000, [30000, 16385, 8193]), (16, 40000, [24577, 30000, 16384])])
+def test_calibrator_update_of_several_pieces(ctx, n_bins, cap, sizes):
+    test_calibrator_update_matches_oracle(ctx, n_bins, cap, sizes)
+
+
 def test_delta_is_bit_equal_over_many_states_and_parameters(ctx):
     """delta decides by comparisons that turn on the last bits near convergence: many random buffer states, skewed
     score distributions and survival parameters, every one bit for bit."""
