@@ -113,16 +113,20 @@ __device__ __forceinline__ void pipe_teardown(const PipeSmem& ps, uint32_t* d_st
 // Pairs in step.  The pairs of a launch share operand panels through L2, but only while they read them at about the same
 // time, and nothing in a persistent kernel keeps them together: measured at d = 4,096, the dH contraction of a chunk read 33 GB
 // from HBM where 11 would do and ran at 1.09 GHz under the power cap, the dz kernel beside it, with its little traffic, at 1.27.
-// So about every EPOCH K steps the leading producer of a pair reports on a counter in global memory and waits until all
-// pairs have reported two epochs ago; none gets further ahead of the others than that.  The counter is fetched an epoch
+// So about every EPOCH K steps the leading producer of a pair reports on a counter in global memory and waits until there are
+// as many reports as all pairs make up to two epochs ago: no pair gets more than two epochs ahead of the average.  (A single
+// straggler is not waited for by name: the reports of the pairs ahead stand in for its own.)  The counter is fetched an epoch
 // ahead by an asynchronous copy into shared memory, so a pair that is not ahead does not wait for memory either.
 // (A plain load of the counter by one thread at every epoch cost the tensor pipe 6-14 % of the cycles.)  One chunk alone, without
 // and with it: d = 2,048, V = 128,256 HBM reads of dH 12.0 -> 6.8 GB, of dW 8.9 -> 6.1, the three kernels 10.4 -> 10.0 ms; d = 4,096,
 // V = 151,936 34 -> 17 and 25 -> 15.5 GB, 25.7 -> 24.0 ms.  Over seconds, where the power cap evens it out, an update of a
 // DAPO-shaped micro-batch takes 70.3 -> 69.4 ms.  Epochs of 8 steps reach the least traffic (4.9 and 4.7 GB, 11.7 and 11.2) but
-// gain nothing more over seconds.  All pairs must be resident: no more are launched than the occupancy query allows, and the wait is bounded
-// like every other.
+// gain nothing more over seconds.
+//   The results do not depend on it, and nothing may: the pairs of another launch, on another stream, can hold the SMs that some
+// of these pairs still need, and wait for their own absent pairs in turn.  So the wait is a short one, far above what pairs
+// that run side by side ever wait, and a pair that has waited that long goes on, reports as before and waits no more.
 constexpr int EPOCH = 16;
+constexpr uint32_t LOCK_TRIES = 128;   // of half a microsecond or more; an epoch takes about three
 constexpr size_t LOCK_BYTES = 16;      // per counter
 struct Lockstep {
     unsigned int* counter;      // zero before the launch, 16-byte aligned
@@ -139,18 +143,16 @@ __device__ __forceinline__ Lockstep lockstep_for(unsigned int* counter, int64_t 
                                            : (most + l.items_per_epoch - 1) / l.items_per_epoch);
     return l;
 }
-// One thread, at the beginning of its pair's epoch `epoch`.  False: the wait ran out.
-__device__ __forceinline__ bool begin_epoch(const Lockstep& lock, volatile uint32_t* seen, uint32_t epoch,
-                                            volatile uint32_t* abort_flag) {
+// One thread, at the beginning of its pair's epoch `epoch`.  False: waited in vain.
+__device__ __forceinline__ bool begin_epoch(const Lockstep& lock, volatile uint32_t* seen, uint32_t epoch) {
     atomicAdd(lock.counter, 1u);
     cp_async_wait_all();
-    const uint32_t target = epoch < 2 ? 0u : (epoch - 1) * lock.units;       // everybody has begun epoch - 2
-    if (target != 0u && *seen < target) {
+    const uint32_t target = epoch < 2 ? 0u : (epoch - 1) * lock.units;       // the average pair has begun epoch - 2
+    if (*seen < target)
         for (uint32_t spin = 0; ld_relaxed_u32(lock.counter) < target; ++spin) {
+            if (spin >= LOCK_TRIES) return false;
             __nanosleep(32);
-            if (spin >= SPIN_LIMIT || ((spin & 1023u) == 1023u && *abort_flag)) { *abort_flag = 1u; return false; }
         }
-    }
     cp_async_16(seen, lock.counter);                                          // looked at when the next epoch begins
     return true;
 }
@@ -171,7 +173,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
                                               const CUtensorMap* mb_tail = nullptr, int tail_ks = -1) {
     const uint32_t a0 = smem_u32(ps.stage_a), b0 = smem_u32(ps.stage_b);
     uint32_t stage = 0, phase = 0, issued = 0, epoch = 0;
-    bool ok = true;
+    bool ok = true, in_step = true;
     TileAt tile;
     int to_epoch = 0;                     // items until the next epoch
     for (int64_t it = 0; ok && coords(it, tile); ++it) {
@@ -179,9 +181,11 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
         for (int ks0 = 0; ks0 < k_steps && ok; ks0 += EPOCH) {
             if (ks0 > 0 || to_epoch == 0) {
                 if (ps.rank == 0) {
-                    if (elect_one()) ok = begin_epoch(lock, ps.lock_seen, epoch, ps.abort_flag);
-                    ok = __all_sync(0xffffffffu, ok) != 0;
-                    if (!ok) break;
+                    if (elect_one()) {
+                        if (in_step) in_step = begin_epoch(lock, ps.lock_seen, epoch);
+                        else atomicAdd(lock.counter, 1u);
+                    }
+                    in_step = __all_sync(0xffffffffu, in_step) != 0;
                 }
                 ++epoch;
                 if (ks0 == 0) to_epoch = lock.items_per_epoch;
@@ -628,7 +632,7 @@ cudaError_t launch_pairs(arrol_ctx* ctx, int which, void (*kernel)(KArgs...), in
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    // the pairs wait for one another: never more of them than are resident at once (asked once per context and kernel)
+    // the pairs are persistent and kept in step: no more of them than the GPU holds at once (asked once per context and kernel)
     if (ctx->backward_max_pairs[which] == 0) {
         int fit = 0;
         cudaLaunchConfig_t ask = cfg;

@@ -124,6 +124,44 @@ def test_lm_head_backward_without_a_live_token(ctx):
     assert torch.all(dW == 0.0) and torch.all((dH == 0.0) | (dH == 9.0))
 
 
+def test_lm_head_backwards_in_flight_on_two_streams(ctx):
+    """Each launch fills the GPU and keeps its pairs of blocks in step; two at once get a part of the SMs each, so neither can
+    count on all of its pairs running."""
+    T, d, V = 6000, 1024, 12000
+    g = np.random.default_rng(3)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    calls = []
+    for i in range(2):
+        H = torch.from_numpy(g.normal(size=(T, d)).astype(np.float32)).to(torch.bfloat16).cuda()
+        W = torch.from_numpy(g.normal(0, 0.02, size=(V, d)).astype(np.float32)).to(torch.bfloat16).cuda()
+        y = dv(g.integers(0, V, size=T).astype(np.int32))
+        gl = dv(g.normal(size=T).astype(np.float32))
+        lse = torch.full((T,), float(np.log(V)) + 0.2, device="cuda")
+        out = [torch.full((T, d), 9.0, device="cuda"), torch.full((V, d), 9.0, device="cuda")]
+        ws = torch.empty(U.arrol_lm_head_backward_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+        calls.append((H, W, y, gl, lse, out, ws))
+
+    def run(i, stream=None):
+        H, W, y, gl, lse, out, ws = calls[i]
+        U.arrol_lm_head_backward(ctx, H, W, y, gl, lse, T, d, V, out[0], out[1], ws, stream=stream)
+
+    want = []
+    for i in range(2):
+        run(i)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in calls[i][5]])
+        for t in calls[i][5]:
+            t.fill_(9.0)
+    torch.cuda.synchronize()
+    for _ in range(6):
+        for i in range(2):
+            run(i, streams[i])
+    torch.cuda.synchronize()
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    for i in range(2):
+        assert all(torch.equal(a, b) for a, b in zip(calls[i][5], want[i]))
+
+
 def test_update_argument_errors(ctx):
     z = torch.zeros(8, device="cuda")
     with pytest.raises(B.ArrolError) as e:
