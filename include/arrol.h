@@ -59,8 +59,12 @@ const char* arrol_status_string(int status); /* static string, never NULL */
 /* Creates a context on CUDA device `device` (made current for the calling thread during the call).
  * Allocates the context's device status word, a 16 MB scratch buffer and a 64 MB row-packing buffer (MLP head),
  * 65 MB of pinned host memory, a second stream and a few events (used by arrol_prune_rebatch_host); nothing is
- * allocated later.  Calls that use the context's buffers (MLP-head scoring, the policy loss, the head training
- * step) must be ordered on the device with respect to one another, e.g. by issuing them on one stream. */
+ * allocated later.  Calls that use the context's buffers (MLP-head scoring, arrol_compact, arrol_prune_step and
+ * arrol_prune_rebatch_host, the policy loss, the head training step) must be ordered on the device with respect to one
+ * another, e.g. by issuing them on one stream.  Calls that work in the caller's buffers alone may be in flight on several
+ * streams at once, each with a workspace and outputs of its own: arrol_token_logprob and its variants,
+ * arrol_lm_head_backward, linear-head scoring, arrol_select, the vote, the trace confidence, and the calibrator's calls
+ * (those on one state in order).  They share the GPU then; results do not depend on it. */
 int arrol_create(arrol_ctx** out, int device);
 int arrol_destroy(arrol_ctx* ctx);
 

@@ -29,11 +29,13 @@
 // its chunks from HBM, falls further behind, and the extra HBM traffic costs power: the SM clock under the 1 kW cap
 // fell from 1.40 GHz in the first waves to 0.72 GHz.  So the blocks are held in step: before issuing the loads of
 // wave k (its k-th work item) every producer arrives on a counter in global memory and waits until all blocks have
-// arrived for that wave.  All blocks must then be resident: single blocks are launched cooperatively whenever there is
-// more than one wave; for pairs the host asks cudaOccupancyMaxActiveClusters how many fit at once and launches no
-// more (a cooperative launch of clusters that fills the GPU is the one launch the profiler cannot make).  Like every
-// other wait this one is bounded.
-// Every wait is bounded; when one runs out the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
+// arrived for that wave.  Single blocks are launched cooperatively whenever there is more than one wave, so that they are
+// all resident; of pairs no more are launched than cudaOccupancyMaxActiveClusters says fit at once (a cooperative launch of
+// clusters that fills the GPU is the one launch the profiler cannot make), which another launch on another stream can
+// still keep from being resident together.  The results do not depend on the step, so a producer waits half as long as its own
+// last item took (side by side they are within a few per cent of one another), or STEP_WAIT_CYCLES if that is longer, then goes on
+// and waits no more.
+// Every other wait is bounded too; when one runs out the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
 //
 // Gathered variant (arrol_token_logprob_gathered; Section 4.3 (ii): the survivors are re-batched "to compute
 // log-probabilities"): the token rows are read straight from the pre-prune source buffer, so the packed copy of the
@@ -70,6 +72,7 @@ constexpr int PAIR_STAGE_BYTES = A_STAGE_BYTES + PAIR_B_STAGE_BYTES;
 static_assert(PAIR_STAGES * PAIR_STAGE_BYTES == SOLO_STAGES * SOLO_STAGE_BYTES, "both variants fill the same shared memory");
 constexpr int TMEM_COLS = 512;   // two fp32 accumulators of BN columns
 constexpr int num_threads(int halves) { return 64 + 128 * halves; }     // producer, issuer, four epilogue warps per column half
+constexpr long long STEP_WAIT_CYCLES = 100000;   // what a producer waits at least for the others of its wave (50 us or more)
 constexpr int COMBINE_BLOCKS = 16;           // blocks of segments (n_mid) that one warp merges side by side
 constexpr size_t SMEM_BYTES = (size_t)SOLO_STAGES * SOLO_STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
 
@@ -162,12 +165,6 @@ struct LogprobParams {
     unsigned long long* timing;   // test hook: per body item {globaltimer start, end, clock64 start, end}, or NULL
     int64_t timing_items;
 };
-
-__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 
 __device__ __forceinline__ unsigned long long global_timer_ns() {
     unsigned long long t;
@@ -313,22 +310,26 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
             int row = 0;
             if constexpr (GATHER) if (have) row = source_row(it);
             int arrived = 0, waited = 0;            // waves
+            bool in_step = true;
+            long long item_begun = clock64();
             for (int k = 0; !p.mute_producer; ++k) {
                 // hold the blocks in step: arrive for the item's wave (one arrival per unit and wave), then wait for
                 // everybody; a unit without an item in a partial wave arrives as well
                 const int wave = have ? it.wave : work.waves - 1;
                 for (; arrived < wave; ++arrived)
-                    if (rank == 0) { __threadfence(); atomicAdd(p.wave_counter, 1u); }
+                    if (rank == 0) atomicAdd(p.wave_counter, 1u);
                 if (!have) break;
-                if (wave > waited) {
+                if (wave > waited && in_step) {
                     const unsigned int target = (unsigned int)wave * (unsigned int)units;
-                    uint32_t spin = 0;
-                    while (ld_acquire_u32(p.wave_counter) < target) {
+                    long long now = clock64();
+                    const long long until = now + max((now - item_begun) / 2, STEP_WAIT_CYCLES);
+                    while (ld_relaxed_u32(p.wave_counter) < target) {
+                        if (now >= until) { in_step = false; break; }
                         __nanosleep(64);
-                        if (++spin >= p.spin_limit || ((spin & 1023u) == 1023u && *abort_flag)) { ok = false; break; }
+                        now = clock64();
                     }
-                    if (!ok) { *abort_flag = 1u; break; }
                     waited = wave;
+                    item_begun = now;
                 }
                 const bool have_next = work_item(work, p.plan, unit, units, k + 1, next);
                 int row_next = 0;
@@ -860,11 +861,10 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         attr[n_attr].val.clusterDim.y = 1;
         attr[n_attr].val.clusterDim.z = 1;
         ++n_attr;
-        // Pairs that wait for one another per wave must all be resident.  The cooperative attribute would have the
-        // driver check that, but the profiler cannot launch a cooperative grid of clusters that fills the GPU
-        // ("LaunchFailed"; the same grid without the attribute profiles), so the check is made here instead: never
-        // more pairs than the occupancy query says fit at once (asked once per context and kernel variant).  The
-        // waits themselves are bounded either way.
+        // Pairs are kept in step per wave, so no more of them than fit the GPU at once (asked once per context and kernel
+        // variant).  The cooperative attribute would have the driver see to it that they also are resident at once, but the
+        // profiler cannot launch a cooperative grid of clusters that fills the GPU ("LaunchFailed"; the same grid without the
+        // attribute profiles), and the waits do without (see the top of this file).
         if (ctx->pair_max_clusters[halves - 1][variant] == 0) {
             cfg.gridDim = dim3((unsigned)(2 * units));
             cfg.attrs = attr;
@@ -878,7 +878,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     }
     if (units > tiles_max * p.plan.n_sub) units = tiles_max * p.plan.n_sub;
     const int64_t grid = pair ? 2 * units : units;
-    // more than one wave: the blocks wait for one another, so they must all be resident (single blocks: cooperative launch)
+    // more than one wave: the blocks are kept in step, and should all be resident (single blocks: cooperative launch)
     const bool several_waves = make_work_list((int)tiles_max, (int)units, p.plan).waves > 1;
     if (several_waves) ARROL_CUDA_OK(cudaMemsetAsync(p.wave_counter, 0, sizeof(unsigned int), s));
     if (several_waves && !pair) {

@@ -626,3 +626,39 @@ def test_logprob_bits_do_not_depend_on_the_token_count(V, d, pair):
     assert np.abs(full[1].cpu().numpy()[rows] - lse_ref).max() <= LOGP_TOL
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("d", [448, 640])                # single blocks, pairs
+def test_logprob_calls_of_several_waves_in_flight_on_two_streams(ctx, d):
+    """Each launch fills the GPU and holds its blocks in step wave by wave; two at once get a part of the SMs each, so neither
+    can count on all of its blocks running."""
+    T, V = 60000, 3000
+    g = np.random.default_rng(d)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    calls = []
+    for _ in range(2):
+        H = torch.from_numpy(g.normal(size=(T, d)).astype(np.float32)).to(torch.bfloat16).cuda()
+        W = torch.from_numpy(g.normal(0, 0.03, size=(V, d)).astype(np.float32)).to(torch.bfloat16).cuda()
+        y = dev(g.integers(0, V, size=T).astype(np.int32))
+        ws = torch.empty(B.arrol_token_logprob_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+        calls.append((H, W, y, torch.empty(T, device="cuda"), torch.empty(T, device="cuda"), ws))
+
+    def run(i, stream=None):
+        H, W, y, logp, lse, ws = calls[i]
+        B.arrol_token_logprob(ctx, H, W, y, T, d, V, logp, ws, lse=lse, stream=stream)
+
+    want = []
+    for i in range(2):
+        run(i)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in calls[i][3:5]])
+        for t in calls[i][3:5]:
+            t.fill_(7.0)
+    torch.cuda.synchronize()
+    for _ in range(6):
+        for i in range(2):
+            run(i, streams[i])
+    torch.cuda.synchronize()
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    for i in range(2):
+        assert all(torch.equal(a, b) for a, b in zip(calls[i][3:5], want[i]))
