@@ -291,8 +291,7 @@ int arrol_select_stochastic(arrol_ctx* ctx, const float* q, const float* u, cons
  *   hidden rows t in [T, T_max) are never read by the contractions (the last, partly live block of rows goes
  *   through a zero-padded copy), so they may hold anything.
  *   workspace: arrol_lm_head_backward_workspace(ctx, T_max, d, V) bytes, 256-byte aligned (one chunk of 9,472 tokens
- *   of dz in bf16, one 64-row block of hidden, 48 bytes per chunk): 9472 * 2 * V + 128 * d + 48 * ceil(T_max / 9472)
- *   bytes (V rounded up to 8, every part to 256). */
+ *   of dz in bf16 and one 64-row block of hidden): 9472 * 2 * V + 128 * d bytes (V rounded up to 8), whatever T_max is. */
 int arrol_policy_loss(arrol_ctx* ctx, const float* logp, const float* logp_old, const float* logp_ref,
                       const float* tok_adv, const int32_t* tok_seq, const int64_t* cu_seqlens, const int64_t* d_num,
                       int64_t T_max, float eps_low, float eps_high, float beta, int32_t agg_mode, float* grad_logp,

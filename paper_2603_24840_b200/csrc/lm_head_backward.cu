@@ -127,15 +127,20 @@ __device__ __forceinline__ void pipe_teardown(const PipeSmem& ps, uint32_t* d_st
 // that run side by side ever wait, and a pair that has waited that long goes on, reports as before and waits no more.
 constexpr int EPOCH = 16;
 constexpr uint32_t LOCK_TRIES = 128;   // of half a microsecond or more; an epoch takes about three
-constexpr size_t LOCK_BYTES = 16;      // per counter
+// The counters of a call, one per kernel, in one 16-byte group.  Each kernel zeroes the next one's, which its last user, a
+// chunk ago, is done with and its next one, the following launch, has not begun to use.
+enum LockWord { LOCK_DZ, LOCK_DH, LOCK_DW, LOCK_WORDS };
+constexpr size_t LOCK_BYTES = 16;
 struct Lockstep {
-    unsigned int* counter;      // zero before the launch, 16-byte aligned
+    unsigned int* words;        // 16-byte aligned; this kernel's is zero before the launch
+    int word;
     uint32_t units, epochs;     // epochs of the pair with the most work
     int items_per_epoch;        // > 1 when a tile has few K steps
 };
-__device__ __forceinline__ Lockstep lockstep_for(unsigned int* counter, int64_t units, int64_t items, int k_steps) {
+__device__ __forceinline__ Lockstep lockstep_for(unsigned int* words, int word, int64_t units, int64_t items, int k_steps) {
     Lockstep l;
-    l.counter = counter;
+    l.words = words;
+    l.word = word;
     l.units = (uint32_t)units;
     l.items_per_epoch = k_steps >= EPOCH ? 1 : EPOCH / max(k_steps, 1);
     const int64_t most = (items + units - 1) / units;
@@ -145,15 +150,16 @@ __device__ __forceinline__ Lockstep lockstep_for(unsigned int* counter, int64_t 
 }
 // One thread, at the beginning of its pair's epoch `epoch`.  False: waited in vain.
 __device__ __forceinline__ bool begin_epoch(const Lockstep& lock, volatile uint32_t* seen, uint32_t epoch) {
-    atomicAdd(lock.counter, 1u);
+    unsigned int* counter = lock.words + lock.word;
+    atomicAdd(counter, 1u);
     cp_async_wait_all();
     const uint32_t target = epoch < 2 ? 0u : (epoch - 1) * lock.units;       // the average pair has begun epoch - 2
-    if (*seen < target)
-        for (uint32_t spin = 0; ld_relaxed_u32(lock.counter) < target; ++spin) {
+    if (seen[lock.word] < target)
+        for (uint32_t spin = 0; ld_relaxed_u32(counter) < target; ++spin) {
             if (spin >= LOCK_TRIES) return false;
             __nanosleep(32);
         }
-    cp_async_16(seen, lock.counter);                                          // looked at when the next epoch begins
+    cp_async_16(seen, lock.words);                                            // looked at when the next epoch begins
     return true;
 }
 
@@ -176,6 +182,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
     bool ok = true, in_step = true;
     TileAt tile;
     int to_epoch = 0;                     // items until the next epoch
+    if (blockIdx.x == 0 && elect_one()) lock.words[(lock.word + 1) % LOCK_WORDS] = 0u;
     for (int64_t it = 0; ok && coords(it, tile); ++it) {
         const int ay = tile.a0 + (int)ps.rank * BM, by = tile.b0 + (int)ps.rank * (tile.n / 2);
         for (int ks0 = 0; ks0 < k_steps && ok; ks0 += EPOCH) {
@@ -183,7 +190,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
                 if (ps.rank == 0) {
                     if (elect_one()) {
                         if (in_step) in_step = begin_epoch(lock, ps.lock_seen, epoch);
-                        else atomicAdd(lock.counter, 1u);
+                        else atomicAdd(lock.words + lock.word, 1u);
                     }
                     in_step = __all_sync(0xffffffffu, in_step) != 0;
                 }
@@ -233,7 +240,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
     }
     if (ps.rank == 0 && elect_one()) {
         cp_async_wait_all();
-        if (epoch < lock.epochs) atomicAdd(lock.counter, lock.epochs - epoch);   // done: nobody waits for this pair
+        if (epoch < lock.epochs) atomicAdd(lock.words + lock.word, lock.epochs - epoch);   // done: nobody waits for this pair
     }
     if (!ok && ps.rank == 0 && elect_one()) {
         // gave up: let the copies already issued land before shared memory goes away (bounded); the peer's copies are
@@ -319,8 +326,8 @@ struct DzParams {
     int group_tiles;
     float scale2, inv_temp;
     const uint16_t* hidden;
-    unsigned int* lock_counter;
-    uint16_t* tail;           // [64, d]: the last, partly live 64-row block of the chunk's hidden rows, zero-padded
+    unsigned int* lock_words;
+    uint16_t* tail;           // [63, d]: the last, partly live 64-row block of the chunk's hidden rows, zero-padded
     uint32_t* d_status;
 };
 
@@ -359,7 +366,7 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
     const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
 
     if (warp == 0) {
-        const Lockstep lock = lockstep_for(p.lock_counter, units, (int64_t)m_tiles * total_chunks, k_steps);
+        const Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, (int64_t)m_tiles * total_chunks, k_steps);
         producer_loop<false, false>(ps, &map_h, &map_w, k_steps, lock, [&](int64_t it, TileAt& t) {
             int m, c;
             if (!dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c)) return false;
@@ -376,11 +383,12 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
             });
     } else {
         // The last, partly live 64-row block of the chunk's hidden rows, padded with zeros, for the dW contraction: rows past
-        // the live tokens (caller memory that may hold anything) never reach the tensor core.
+        // the live tokens (caller memory that may hold anything) never reach the tensor core.  At most 63 rows live in it; the
+        // copy fills the 64th with zeros by itself.
         if (live % BK != 0) {
             const int r0 = live / BK * BK, vec_per_row = p.d / 8;
             const uint16_t* hidden = pdl_acquire(p.hidden);
-            for (int i = (int)blockIdx.x * 32 * EPI_WARPS + (int)threadIdx.x - 64; i < BK * vec_per_row; i += (int)gridDim.x * 32 * EPI_WARPS) {
+            for (int i = (int)blockIdx.x * 32 * EPI_WARPS + (int)threadIdx.x - 64; i < (BK - 1) * vec_per_row; i += (int)gridDim.x * 32 * EPI_WARPS) {
                 const int r = i / vec_per_row, v = i - r * vec_per_row;
                 uint4 x = make_uint4(0u, 0u, 0u, 0u);
                 if (r0 + r < live) x = *reinterpret_cast<const uint4*>(hidden + (p.t0 + r0 + r) * p.d + v * 8);
@@ -494,7 +502,8 @@ struct GemmParams {
     int a3d, b3d;             // the MN-major operand's maps are three-dimensional (one copy per stage)
     const int64_t* d_T;
     int64_t T_max, t0;
-    unsigned int* lock_counter;
+    unsigned int* lock_words;
+    int lock_word;
     uint32_t* d_status;
 };
 
@@ -537,7 +546,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 
     if (warp == 0) {
         const int tail_ks = (p.k_is_tokens && (K % BK) != 0) ? k_steps - 1 : -1;
-        const Lockstep lock = lockstep_for(p.lock_counter, units, (int64_t)m_tiles * n_tiles, k_steps);
+        const Lockstep lock = lockstep_for(p.lock_words, p.lock_word, units, (int64_t)m_tiles * n_tiles, k_steps);
         producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, k_steps, lock, [&](int64_t it, TileAt& t) {
             GemmTile g;
             if (!gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g)) return false;
@@ -660,16 +669,17 @@ int raise_smem_limits(arrol_ctx* ctx) {
 
 struct BackwardLayout {
     int64_t ldz;       // V rounded up to 8
-    size_t dz, tail, counters, total;
+    size_t dz, tail, lock, total;
 };
 
-BackwardLayout backward_layout(int64_t T_max, int d, int V) {
+BackwardLayout backward_layout(int d, int V) {
     BackwardLayout L;
     L.ldz = ((int64_t)V + 7) & ~(int64_t)7;
     L.dz = 0;
     L.tail = (((size_t)TC * L.ldz * 2) + 255) & ~(size_t)255;
-    L.counters = L.tail + (((size_t)BK * d * 2 + 255) & ~(size_t)255);
-    L.total = L.counters + (((size_t)((T_max + TC - 1) / TC) * 3 * LOCK_BYTES + 255) & ~(size_t)255);   // one per kernel
+    L.lock = L.tail + (size_t)(BK - 1) * d * 2;      // in the block's last row, which never holds a hidden row; d >= 8
+    static_assert(LOCK_WORDS * sizeof(unsigned int) <= LOCK_BYTES && LOCK_BYTES <= 8 * 2, "the counters fit the narrowest row");
+    L.total = L.tail + (((size_t)BK * d * 2 + 255) & ~(size_t)255);
     return L;
 }
 
@@ -677,7 +687,7 @@ BackwardLayout backward_layout(int64_t T_max, int d, int V) {
 
 extern "C" size_t arrol_lm_head_backward_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    return backward_layout(T_max, d, V).total;
+    return backward_layout(d, V).total;
 }
 
 extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const void* W_vocab, const int32_t* targets,
@@ -698,12 +708,12 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     if (!hidden || !W_vocab || !targets || !grad_logp || !lse || !dH) return ARROL_ERR_INVALID_ARG;
     if (!arrol_aligned(hidden, 16) || !arrol_aligned(W_vocab, 16) || !arrol_aligned(dH, 16) || !arrol_aligned(dW, 16))
         return ARROL_ERR_INVALID_ARG;
-    const BackwardLayout L = backward_layout(T_max, d, V);
+    const BackwardLayout L = backward_layout(d, V);
     if (!workspace || workspace_bytes < L.total || !arrol_aligned(workspace, 256)) return ARROL_ERR_WORKSPACE;
     __nv_bfloat16* dZ = reinterpret_cast<__nv_bfloat16*>(static_cast<uint8_t*>(workspace) + L.dz);
     uint16_t* Htail = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + L.tail);
-    unsigned int* counters = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + L.counters);
-    ARROL_CUDA_OK(cudaMemsetAsync(counters, 0, L.total - L.counters, s));
+    unsigned int* lock_words = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + L.lock);
+    ARROL_CUDA_OK(cudaMemsetAsync(lock_words, 0, LOCK_BYTES, s));
     if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
 
     // tensor maps: K-major operands are fetched as [128 MN rows x 64 K columns] boxes; MN-major ones (the same row-major
@@ -718,12 +728,12 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     if (make_map_f32_tile(ctx, &map_dw, dW, (uint64_t)V, (uint64_t)d, (uint64_t)d) != ARROL_OK) return ARROL_ERR_CUDA;
     bool d3 = d % 64 == 0, v3 = V % 64 == 0;
     if (d3 && (make_map_mn3d(ctx, &map_w_mn, W_vocab, (uint64_t)V, (uint64_t)d, (uint64_t)d, BN / 2 / 64) != ARROL_OK ||
-               make_map_mn3d(ctx, &map_h_tail, Htail, (uint64_t)BK, (uint64_t)d, (uint64_t)d, BN / 2 / 64) != ARROL_OK))
+               make_map_mn3d(ctx, &map_h_tail, Htail, (uint64_t)BK - 1, (uint64_t)d, (uint64_t)d, BN / 2 / 64) != ARROL_OK))
         d3 = false;
     if (v3 && make_map_mn3d(ctx, &map_dz_mn, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BM / 64) != ARROL_OK) v3 = false;
     if (!d3) {
         if (make_map(ctx, &map_w_mn, W_vocab, (uint64_t)V, (uint64_t)d, BK) != ARROL_OK) return ARROL_ERR_CUDA;
-        if (make_map(ctx, &map_h_tail, Htail, (uint64_t)BK, (uint64_t)d, BK) != ARROL_OK) return ARROL_ERR_CUDA;
+        if (make_map(ctx, &map_h_tail, Htail, (uint64_t)BK - 1, (uint64_t)d, BK) != ARROL_OK) return ARROL_ERR_CUDA;
     }
     if (!v3 && make_map_ld(ctx, &map_dz_mn, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BK) != ARROL_OK) return ARROL_ERR_CUDA;
 
@@ -744,13 +754,13 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         zp.targets = targets; zp.grad_logp = grad_logp; zp.lse = lse; zp.d_T = d_T; zp.T_max = T_max; zp.t0 = t0;
         zp.d = d; zp.V = V; zp.group_tiles = (TC / TILE_ROWS + m_groups - 1) / m_groups;
         zp.scale2 = inv_temperature * 1.44269504088896340736f; zp.inv_temp = inv_temperature;
-        zp.lock_counter = counters; counters += LOCK_BYTES / sizeof(unsigned int);
+        zp.lock_words = lock_words;
         zp.hidden = static_cast<const uint16_t*>(hidden); zp.tail = Htail; zp.d_status = ctx->d_status;
         ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, (int64_t)m_tiles * total_chunks, s, map_h_k, map_w_k, map_dz_st, zp));
 
         GemmParams gh = {};    // dH[chunk] = dZ . W
         gh.M = (int)rows; gh.N = d; gh.K = V; gh.group_n = group_columns(n_tiles);
-        gh.m_is_tokens = 1; gh.b3d = d3; gh.lock_counter = counters; counters += LOCK_BYTES / sizeof(unsigned int);
+        gh.m_is_tokens = 1; gh.b3d = d3; gh.lock_words = lock_words; gh.lock_word = LOCK_DH;
         gh.d_T = d_T; gh.T_max = T_max; gh.t0 = t0; gh.d_status = ctx->d_status;
         CUtensorMap map_dh;      // this chunk's rows of dH: rows past the chunk are clipped by the tile stores
         if (make_map_f32_tile(ctx, &map_dh, dH + t0 * d, (uint64_t)rows, (uint64_t)d, (uint64_t)d) != ARROL_OK)
@@ -760,7 +770,7 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         GemmParams gw = {};    // dW (+)= dZ^T . H[chunk]; the first chunk writes dW, zeros where no token lives
         gw.M = V; gw.N = d; gw.K = (int)rows; gw.group_n = group_columns(n_tiles);
         gw.accumulate = t0 > 0; gw.k_is_tokens = 1; gw.zero_if_dead = t0 == 0; gw.a3d = v3; gw.b3d = d3;
-        gw.lock_counter = counters; counters += LOCK_BYTES / sizeof(unsigned int);
+        gw.lock_words = lock_words; gw.lock_word = LOCK_DW;
         gw.d_T = d_T; gw.T_max = T_max; gw.t0 = t0; gw.d_status = ctx->d_status;
         ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, (int64_t)((V + TILE_ROWS - 1) / TILE_ROWS) * n_tiles, s,
                                    map_dz_mn, map_h_mn, map_h_tail, map_dw, gw));

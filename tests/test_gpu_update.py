@@ -124,6 +124,14 @@ def test_lm_head_backward_without_a_live_token(ctx):
     assert torch.all(dW == 0.0) and torch.all((dH == 0.0) | (dH == 9.0))
 
 
+def test_lm_head_backward_workspace_serves_any_number_of_tokens(ctx):
+    for d, V in ((8, 300), (72, 301), (4096, 151936)):
+        want = 9472 * 2 * ((V + 7) // 8 * 8) + 128 * d
+        assert all(U.arrol_lm_head_backward_workspace(ctx, T, d, V) == want for T in (1, 9472, 9473, 60000, 1 << 30))
+    for d, T, T_live in ((8, 9700, 9500), (16, 20000, 18945), (24, 9473, None)):   # the narrowest rows, several chunks
+        _backward_case(ctx, T, d, 300, seed=d, T_live=T_live)
+
+
 def test_lm_head_backwards_in_flight_on_two_streams(ctx):
     """Each launch fills the GPU and keeps its pairs of blocks in step; two at once get a part of the SMs each, so neither can
     count on all of its pairs running."""
