@@ -60,11 +60,11 @@ const char* arrol_status_string(int status); /* static string, never NULL */
  * Allocates the context's device status word, a 16 MB scratch buffer and a 64 MB row-packing buffer (MLP head),
  * 65 MB of pinned host memory, a second stream and a few events (used by arrol_prune_rebatch_host); nothing is
  * allocated later.  Calls that use the context's buffers (MLP-head scoring, arrol_compact, arrol_prune_step and
- * arrol_prune_rebatch_host, the policy loss, the head training step) must be ordered on the device with respect to one
+ * arrol_prune_rebatch_host, the policy loss, the training step of a bf16 MLP head) must be ordered on the device with respect to one
  * another, e.g. by issuing them on one stream.  Calls that work in the caller's buffers alone may be in flight on several
  * streams at once, each with a workspace and outputs of its own: arrol_token_logprob and its variants,
- * arrol_lm_head_backward, linear-head scoring, arrol_select, the vote, the trace confidence, and the calibrator's calls
- * (those on one state in order).  They share the GPU then; results do not depend on it. */
+ * arrol_lm_head_backward, scoring and training of a linear head, training of an fp32 head, arrol_select, the vote, the
+ * trace confidence, and the calibrator's calls (those on one state in order).  They share the GPU then; results do not depend on it. */
 int arrol_create(arrol_ctx** out, int device);
 int arrol_destroy(arrol_ctx* ctx);
 
@@ -332,8 +332,9 @@ int arrol_trace_confidence(arrol_ctx* ctx, const float* token_conf, const int64_
  * hidden / row_stride_elems / row_index / N / head as in arrol_score_partial (the scores are recomputed here).
  * Outputs are float (loss: device double [1]) and are overwritten; dw2, db2 are ignored for a linear head.
  * fp32 arithmetic, fixed-order reductions.  N <= 65536.  N == 0 or an all-zero mask gives zero loss and gradients.
- * workspace: arrol_head_grad_workspace(ctx, N, d, h) bytes, 256-byte aligned.  Uses the context scratch for the
- * linear head's scores: one stream at a time per context. */
+ * workspace: arrol_head_grad_workspace(ctx, N, d, h) bytes, 256-byte aligned.  A bf16 MLP head uses the context's
+ * buffers too (the packed rows, the scoring counters): one stream at a time per context.  Linear heads and fp32 heads work
+ * in the workspace alone. */
 size_t arrol_head_grad_workspace(arrol_ctx* ctx, int32_t N, int32_t d, int32_t h);
 int arrol_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride_elems, const int64_t* row_index, int32_t N,
                     const arrol_head* head, const float* rewards, const uint8_t* mask, float* dW1, float* db1,

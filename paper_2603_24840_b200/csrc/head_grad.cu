@@ -4,7 +4,7 @@
 //   linear head:  dw = sum_i ds_i x_i, db = sum_i ds_i
 //   MLP head:     dw2_j = sum_i ds_i gelu(u_ij), db2 = sum_i ds_i, du_ij = ds_i w2_j gelu'(u_ij),
 //                 dW1 = du^T X, db1_j = sum_i du_ij.
-// All reductions run in a fixed order (no atomics), so the gradients are reproducible run to run.
+// All reductions run in a fixed order (the only atomics count arrivals), so the gradients are reproducible run to run.
 #include <cuda_bf16.h>
 
 #include "arrol_internal.h"
@@ -102,7 +102,7 @@ __global__ void column_sum_kernel(const float* __restrict__ partial, int chunks,
 // MLP head: everything between the forward and the dW1 contraction in one launch: ds_i, the loss, du_ij, and per hidden unit
 // the sums dw2_j = sum_i ds_i gelu(u_ij), db1_j = sum_i du_ij.  (It was four launches: ds by one block, du, two column sums,
 // 22 us at N = 2,048, h = 256 against 9 now.)  Block (x, y): 32 hidden units, a run of rollouts.  Every block counts the labelled rollouts itself and forms the
-// ds of its own run; the last block of a column tile to arrive (a counter per tile, reset by that block) adds the runs' sums in
+// ds of its own run; the last block of a column tile to arrive (a counter per tile, zero again when that block is through) adds the runs' sums in
 // index order, the one of tile 0 the loss and db2 as well.  The score is given, or the sum of the forward's tile partials + b2.
 // du goes out as float (SIMT contraction) or as the sum of two bf16 planes (error 2^-17 relative: the tensor-core operand).
 template <int THREADS>
@@ -304,7 +304,7 @@ mlp_dw1_kernel(const float* __restrict__ du, const T* __restrict__ hidden, int64
 }
 
 struct GradLayout {
-    size_t tmp3, ds, u, du, run_loss, run_sums, partial, total;   // byte offsets
+    size_t tmp3, ds, u, du, run_loss, run_sums, counters, partial, total;   // byte offsets
     size_t du_plane;                          // bytes of one bf16 plane of du (hi at du, lo at du + du_plane)
 };
 GradLayout grad_layout(int N, int d, int h) {
@@ -323,6 +323,7 @@ GradLayout grad_layout(int N, int d, int h) {
     size_t part = h > 0 ? tiles * (size_t)N : chunks * (size_t)d;
     L.run_loss = o; o = up(o + sizeof(double) * 2 * DU_RUNS);                                       // loss / db2 per run
     L.run_sums = o; o = up(o + sizeof(float) * 2 * (size_t)DU_RUNS * (size_t)(h > 0 ? h : 0));      // dw2 / db1 per run
+    L.counters = o; o = up(o + sizeof(uint32_t) * (size_t)(((h > 0 ? h : 0) + 31) / 32));             // finished runs per column tile
     L.partial = o; o = up(o + sizeof(float) * part);
     L.total = o;
     return L;
@@ -351,7 +352,7 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         float* u = reinterpret_cast<float*>(ws + L.u);
         float* du = reinterpret_cast<float*>(ws + L.du);
         auto launch_du = [&](const float* score, const float* tile_partial, int h_tiles, float* du_f, __nv_bfloat16* hi,
-                             __nv_bfloat16* lo) -> int {
+                             __nv_bfloat16* lo, uint32_t* counters) -> int {
             const int rows_per = ((N + DU_RUNS - 1) / DU_RUNS + 7) / 8 * 8;
             const int runs = (N + rows_per - 1) / rows_per;
             ARROL_CUDA_OK(arrol_launch_pdl(head_du_kernel<T>, dim3((h + 31) / 32, runs), dim3(DU_THREADS), sizeof(float) * rows_per, s,
@@ -359,7 +360,7 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
                                            score ? nullptr : static_cast<const T*>(head->b2), rewards, mask,
                                            static_cast<const T*>(head->w2), N, h, rows_per, du_f, hi, lo,
                                            reinterpret_cast<float*>(ws + L.run_sums), reinterpret_cast<double*>(ws + L.run_loss),
-                                           ctx->d_head_counters, dw2, db1, loss, db2));
+                                           counters, dw2, db1, loss, db2));
             ctx->launches += 1;
             return ARROL_OK;
         };
@@ -373,7 +374,7 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
                 if (rc == ARROL_OK) {
                     __nv_bfloat16* du_hi = reinterpret_cast<__nv_bfloat16*>(ws + L.du);
                     __nv_bfloat16* du_lo = reinterpret_cast<__nv_bfloat16*>(ws + L.du + L.du_plane);
-                    const int rd = launch_du(tmp, nullptr, 0, nullptr, du_hi, du_lo);
+                    const int rd = launch_du(tmp, nullptr, 0, nullptr, du_hi, du_lo, ctx->d_head_counters);
                     if (rd != ARROL_OK) return rd;
                     return arrol_internal_head_dw1(ctx, du_hi, du_lo, row_index ? ctx->d_pack : hidden,
                                                    row_index ? (int64_t)d : row_stride, N, d, h, dW1, s);
@@ -381,9 +382,13 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
                 if (rc != ARROL_ERR_UNSUPPORTED) return rc;
             }
         }
+        // this path works in the call's own workspace alone, so that calls on several streams do not meet; its counters too
+        // (a call on the tensor cores shares the context's packing buffer and scoring counters with others anyway)
+        uint32_t* counters = reinterpret_cast<uint32_t*>(ws + L.counters);
+        ARROL_CUDA_OK(cudaMemsetAsync(counters, 0, sizeof(uint32_t) * (size_t)((h + 31) / 32), s));
         const int rc = arrol_internal_mlp_tiles(ctx, hidden, row_stride, row_index, N, head, partial, u, s);
         if (rc != ARROL_OK) return rc;
-        const int rd = launch_du(nullptr, partial, (h + ARROL_MLP_TH - 1) / ARROL_MLP_TH, du, nullptr, nullptr);
+        const int rd = launch_du(nullptr, partial, (h + ARROL_MLP_TH - 1) / ARROL_MLP_TH, du, nullptr, nullptr, counters);
         if (rd != ARROL_OK) return rd;
         dim3 grid((d + GT - 1) / GT, (h + GT - 1) / GT);
         mlp_dw1_kernel<T><<<grid, 128, 0, s>>>(du, hid, row_stride, row_index, N, d, h, dW1);

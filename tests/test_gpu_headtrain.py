@@ -57,6 +57,41 @@ def test_head_grad_at_the_edges_of_its_tiles(N, d, h):
     test_head_grad_matches_oracle(N, d, h, torch.bfloat16, N % 2 == 0)
 
 
+@pytest.mark.parametrize("h", [0, 260])
+def test_head_grads_of_an_fp32_head_in_flight_on_two_streams(h):
+    """These calls work in their own workspaces alone, so two at once give what each gives by itself."""
+    ctx = B.Context(0)
+    g = np.random.default_rng(h)
+    N, d, hh = 5000, 64, max(h, 1)
+    mk = lambda *s: torch.from_numpy(g.normal(0, 0.05, size=s).astype(np.float32)).cuda()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    calls = []
+    for _ in range(2):
+        head = {"W1": mk(d), "b1": mk(1), "w2": None, "b2": None} if h == 0 else {"W1": mk(h, d), "b1": mk(h), "w2": mk(h), "b2": mk(1)}
+        head["h"] = h
+        grads = dict(W1=mk(hh, d), b1=mk(hh), **({"w2": mk(h), "b2": mk(1)} if h else {}))
+        ws = torch.empty(HT.arrol_head_grad_workspace(ctx, N, d, h), dtype=torch.uint8, device="cuda")
+        calls.append((mk(N, d) * 20, head, (mk(N) > 0).float(), grads, torch.zeros(1, dtype=torch.float64, device="cuda"), ws))
+
+    def run(i, stream=None):
+        x, head, rew, grads, loss, ws = calls[i]
+        HT.arrol_head_grad(ctx, x, head, N, rew, grads, loss, ws, stream=stream)
+
+    want = []
+    for i in range(2):
+        run(i)
+        torch.cuda.synchronize()
+        want.append({k: t.clone() for k, t in dict(calls[i][3], loss=calls[i][4]).items()})
+    for _ in range(50):
+        for i in range(2):
+            run(i, streams[i])
+    torch.cuda.synchronize()
+    for i in range(2):
+        assert all(torch.equal(t, want[i][k]) for k, t in dict(calls[i][3], loss=calls[i][4]).items())
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    ctx.close()
+
+
 def test_head_grad_empty_inputs():
     ctx = B.Context(0)
     d = 64
