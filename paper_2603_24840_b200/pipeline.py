@@ -72,7 +72,6 @@ class PruneRebatch:
         self.cu_seqlens = torch.empty(N + 1, dtype=i64, device=dev)
         self.adv = torch.empty(N, dtype=f32, device=dev)
         self.d_num = torch.zeros(2, dtype=i64, device=dev)
-        self.d_T = self.d_num[1:]
         self.dst_tokens = torch.empty(cap, dtype=i32, device=dev)
         self.tok_adv = torch.empty(cap, dtype=f32, device=dev)
         self.tok_seq = torch.empty(cap, dtype=i32, device=dev)
@@ -127,9 +126,17 @@ class PruneRebatch:
             for name, t in bufs.items():
                 setattr(v, name, t)
             v.d_num = torch.zeros(2, dtype=i64, device=dev)      # every view keeps its own {S, T}
-            v.d_T = v.d_num[1:]
             views.append(v)
         return views
+
+    # {S, T} on the device.  The view of T that the log-prob call takes is made with it, not on every step (about 2 us).
+    @property
+    def d_num(self) -> torch.Tensor:
+        return self._d_num
+
+    @d_num.setter
+    def d_num(self, t: torch.Tensor):
+        self._d_num, self.d_T = t, t[1:]
 
     # ---- the four calls -------------------------------------------------------------------------------
     def score_partial(self):
