@@ -80,22 +80,34 @@ struct PartialLse {   // of one token over some columns: running maximum and sum
     float m2, l, zy2, sumz;   // sum of the raw accumulators (only when the confidence is asked for)
 };
 
+// a / b of small whole numbers by b's rounded reciprocal, taken half a unit above a: exact while a < 2^16 and b < 2^10 (the margin is
+// 0.5 / b, the error a / b 2^-22).  An item of a small call would wait for the division of integers.
+__device__ __forceinline__ int quotient(int a, float inv_b) { return (int)(((float)a + 0.5f) * inv_b); }
+
 // How the vocabulary is cut: total_chunks chunks of BN columns -> n_sub segments -> n_mid blocks of segments -> splits
 // groups.  A body item covers a whole group, a tail item one segment; a token's records are merged segment by segment
 // into a block, block by block into a group, then group by group, by whichever kernel holds them.
 struct VocabPlan {
     int total_chunks, n_sub, n_mid, splits;
+    int n_long;           // segments that hold a chunk more than the others: total_chunks mod n_sub
+    float inv_long, inv_short;   // 1 / n_long, 1 / (n_sub - n_long)
     // n_sub <= SMs and total_chunks < 2^23: the product stays below 2^31 for any vocabulary that a TMA coordinate reaches
     __host__ __device__ int chunk_of_sub(int i) const { return (int)((unsigned)i * (unsigned)total_chunks / (unsigned)n_sub); }
+    // j-th segment in the order of dealing: the long ones first.  Segment i is long where floor(i n_long / n_sub) steps after i,
+    // short where ceil(i (n_sub - n_long) / n_sub) does.
+    __device__ int nth_sub(int j) const {
+        const bool is_long = j < n_long;
+        const int a = is_long ? (j + 1) * n_sub + n_long - 1 : (j - n_long) * n_sub;
+        return quotient(a, is_long ? inv_long : inv_short) - (is_long ? 1 : 0);
+    }
     __host__ __device__ int sub_of_mid(int i) const { return i * n_sub / n_mid; }
     __host__ __device__ int mid_of_group(int g) const { return g * n_mid / splits; }
     __host__ __device__ int sub_of_group(int g) const { return sub_of_mid(mid_of_group(g)); }
 };
 
 // (M, L) <- (M, L) + (m, l): M = max, L = sum of 2^(. - M).  One rounding per operation, so that the main kernel (body)
-// and the combining kernel (tail) get the same bits.
+// and the combining kernel (tail) get the same bits.  An empty record (below) changes nothing: L 2^0 + 0.
 __device__ __forceinline__ void merge_lse(float& M, float& L, float m, float l) {
-    if (l == 0.f) return;                                       // nothing in the record (a NaN is something)
     const float Mn = fmaxf(M, m);
     L = __fadd_rn(__fmul_rn(L, ex2_approx(M - Mn)), __fmul_rn(l, ex2_approx(m - Mn)));
     M = Mn;
@@ -113,13 +125,15 @@ __device__ __forceinline__ PartialLse empty_record() { return PartialLse{-FLT_MA
 // and at most 64 groups): the divisions are on the way of every work item and of the combining kernel.
 struct WorkList {
     int body_tiles, body_items, tail_tiles, tail_items, waves;   // tail_tiles: at most units / splits + 1;  waves: those of the
-};                                                               // body, plus one for the tail
+    float inv_tail_tiles;                                        // body, plus one for the tail
+};
 __host__ __device__ inline WorkList make_work_list(int tiles, int units, const VocabPlan& v) {
     WorkList w;
     w.body_tiles = tiles * v.splits / units * units / v.splits;    // whole waves only
     w.body_items = w.body_tiles * v.splits;
     w.tail_tiles = tiles - w.body_tiles;
     w.tail_items = w.tail_tiles * v.n_sub;
+    w.inv_tail_tiles = w.tail_tiles > 0 ? 1.0f / (float)w.tail_tiles : 0.f;
     w.waves = (w.body_items + units - 1) / units + (w.tail_items > 0 ? 1 : 0);
     return w;
 }
@@ -128,7 +142,11 @@ struct WorkItem {
     int group, sub0, sub1;      // group < 0: a tail item
 };
 // k-th item of a unit; false when it has none left.  The tail walks the segments as the slow index: at any time the
-// units work on neighbouring segments of all tail tiles and share W_vocab through L2.
+// units work on neighbouring segments of all tail tiles and share W_vocab through L2.  The segments that are a chunk longer go
+// first: dealt round robin, no unit then has a chunk more than it must.  In the order of the vocabulary they fell to some units
+// more often (19 pair tiles x 160 chunks: 44 chunks on the busiest of 74 pairs against 42; 24 tiles 60 against 52).  Single
+// launches at the full clock in that order / this one: d = 1,856, V = 40,945: 1,000 tokens 132 / 110 us, 4,645 458 / 441, 6,000
+// 615 / 550; d = 2,560, V = 50,257: 3,000 517 / 474, 5,000 794 / 783.
 __device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v, int unit, int units, int k, WorkItem& it) {
     int i = unit + k * units;                   // body items, then tail items, in one numbering
     it.wave = k < w.waves ? k : w.waves - 1;
@@ -141,9 +159,10 @@ __device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v,
     }
     i -= w.body_items;
     if (i >= w.tail_items) return false;
-    it.sub0 = i / w.tail_tiles;
+    const int turn = quotient(i, w.inv_tail_tiles);
+    it.sub0 = v.nth_sub(turn);
     it.sub1 = it.sub0 + 1;
-    it.tile = w.body_tiles + (i - it.sub0 * w.tail_tiles);
+    it.tile = w.body_tiles + (i - turn * w.tail_tiles);
     it.group = -1;
     return true;
 }
@@ -721,6 +740,9 @@ VocabPlan plan_for(const arrol_ctx* ctx, int d, int V) {
     v.splits = splits_for(ctx, d, V, pair_for(ctx, d));
     // one segment per SM: then the tail's items fill the units (SMs, or half as many pairs) a whole number of times
     v.n_sub = v.total_chunks < ctx->sm_count ? v.total_chunks : ctx->sm_count;
+    v.n_long = v.total_chunks % v.n_sub;
+    v.inv_long = v.n_long > 0 ? 1.0f / (float)v.n_long : 0.f;
+    v.inv_short = 1.0f / (float)(v.n_sub - v.n_long);
     if (v.n_sub < v.splits) v.splits = v.n_sub;
     const int per_group = COMBINE_BLOCKS / v.splits > 1 ? COMBINE_BLOCKS / v.splits : 1;
     v.n_mid = v.splits * per_group < v.n_sub ? v.splits * per_group : v.n_sub;

@@ -628,6 +628,14 @@ def test_logprob_bits_do_not_depend_on_the_token_count(V, d, pair):
     ctx.close()
 
 
+# one segment longer than the others, half of them, all but one; single blocks and pairs
+@pytest.mark.parametrize("d", [72, 520])
+@pytest.mark.parametrize("V", [148 * 256 + 1, 222 * 256, 296 * 256 - 255 - 1, 2 * 148 * 256 + 7])
+def test_logprob_with_vocabulary_segments_of_two_sizes(ctx, V, d):
+    for T in (1, 300, 1500):
+        _logprob_case(ctx, T, d, V, seed=V + T, sample=min(T, 12), wstd=0.8 / d ** 0.5)
+
+
 @pytest.mark.parametrize("d", [448, 640])                # single blocks, pairs
 def test_logprob_calls_of_several_waves_in_flight_on_two_streams(ctx, d):
     """Each launch fills the GPU and holds its blocks in step wave by wave; two at once get a part of the SMs each, so neither
