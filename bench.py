@@ -5,8 +5,9 @@ A step is one pass of the whole path over one batch of synthetic input shaped li
   arrol_score_partial -> arrol_select -> arrol_compact (token ids + hidden rows) -> arrol_token_logprob.
 `value` = survivor tokens processed per second over the whole step, inputs resident in HBM.
 `e2e`   = the same metric through arrol_prune_rebatch_host: inputs in pinned host memory, results read back.
-The headline workload is the largest one (Qwen-3-8B DAPO-shaped); `per_workload` carries the same figures for the
-other four at a reduced step count.  `--impl reference` times the CPU oracle (the plain fp64 program the GPU path is
+The headline workload is the largest one (Qwen-3-8B DAPO-shaped); the other four are run at a reduced step count.
+One JSON line on stdout carries the contract's figures (a few KB, so that whoever reads only the end of the output gets all
+of it); the whole report, with every workload's break-down, goes to stderr as a second JSON line.  `--impl reference` times the CPU oracle (the plain fp64 program the GPU path is
 checked against) on host cores.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--impl ours|reference]
@@ -35,7 +36,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # profiler captures on the small cases of the same d and V (the Llama-shaped and the DAPO-shaped one): (bytes read +
 # bytes written) / tokens of the launch.  At fixed d, V and split count the traffic grows in proportion to the tokens
 # of the launch.
-LOGPROB_DRAM_BYTES_PER_TOKEN = {(2048, 128256, 2): 60090.0, (4096, 151936, 2): 155108.0}
+LOGPROB_DRAM_BYTES_PER_TOKEN = {(2048, 128256, 2): 60090.0}
 # DRAM bytes per scored row of score_linear_kernel streamed over consecutive rows (same kind of capture)
 SCORE_LINEAR_DRAM_BYTES_PER_ROW = {(2048, 2): 4129.8}
 
@@ -884,6 +885,34 @@ def report(res, peaks, tokens_all, ms_per_step, e2e_ms, world):
     return out
 
 
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+             "dtype", "data", "config", "gpu_launches", "clocks", "e2e", "breakdown_ms", "logprob_tokens_per_s")
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac", "launch_ms", "launches_per_step", "vocab_splits", "traffic")
+
+
+def finite(x):
+    """The same with NaN and infinities as null: they are no JSON."""
+    if isinstance(x, dict):
+        return {k: finite(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [finite(v) for v in x]
+    return None if isinstance(x, float) and not np.isfinite(x) else x
+
+
+def contract_line(out):
+    """The line for stdout: the contract's keys, the roofline without its notes, one row per other workload."""
+    line = {k: out[k] for k in LINE_KEYS if k in out}
+    line["roofline"] = {k: out["roofline"][k] for k in ROOFLINE_KEYS if k in out["roofline"]}
+    cpu = out.get("cpu_baseline")
+    line["cpu_baseline"] = None if cpu is None else dict(cpu, sample=cpu["sample"][:200])
+    per = out.get("per_workload")
+    if per is not None:
+        line["per_workload"] = {name: {"skipped": b["skipped"][:100]} if "skipped" in b else
+                                {"value": b["value"], "ms_per_step": b["ms_per_step"], "e2e": b["e2e"]["value"],
+                                 "roofline_frac": b["roofline"]["frac"]} for name, b in per.items()}
+    return json.dumps(finite(line))
+
+
 def run_ours(args, w):
     import torch
     import torch.distributed as dist
@@ -958,7 +987,8 @@ def run_ours(args, w):
                                    "survivor_tokens": T_cpu, "gpu_arm_survivor_tokens": T_gpu}
         else:
             out["cpu_baseline"] = None
-        print(json.dumps(out), flush=True)
+        print(json.dumps(finite(out)), file=sys.stderr, flush=True)
+        print(contract_line(out), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
