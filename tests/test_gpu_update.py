@@ -111,6 +111,38 @@ def test_lm_head_backward_at_the_edges_of_a_pairs_tile(ctx, T, d, V, T_live):
     assert np.all(dH[n:] == 0.0)
 
 
+# tile orders of wide heads: columns in two uneven groups (6 + 5 tiles, the last one ragged or whole), token tiles in two groups
+# (22 pair tiles, 19 to a group); gradients on sampled rows, so that the oracle stays cheap
+@pytest.mark.parametrize("d", [2808, 2816])
+def test_lm_head_backward_with_groups_of_tiles(ctx, d):
+    T, V = 5500, 600
+    g = np.random.default_rng(d)
+    H = torch.from_numpy(g.normal(size=(T, d)).astype(np.float32)).to(torch.bfloat16)
+    W = torch.from_numpy(g.normal(0, 0.02, size=(V, d)).astype(np.float32)).to(torch.bfloat16)
+    y = g.integers(0, V, size=T).astype(np.int32)
+    rows = np.unique(np.concatenate([[0, 255, 256, 19 * 256 - 1, 19 * 256, T - 1], g.integers(0, T, size=40)]))
+    gl = np.zeros(T, np.float32)
+    gl[rows] = g.normal(size=len(rows))
+    dH_ref, dW_ref = ou.lm_head_backward(synth.as_oracle_array(H[rows]), synth.as_oracle_array(W), y[rows], gl[rows].astype(np.float64))
+    Hd, Wd, yd = H.cuda(), W.cuda(), dv(y)
+    logp, lse = torch.empty(T, device="cuda"), torch.empty(T, device="cuda")
+    ws = torch.empty(B.arrol_token_logprob_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+    B.arrol_token_logprob(ctx, Hd, Wd, yd, T, d, V, logp, ws, lse=lse)
+    dH, dW = torch.full((T, d), 9.0, device="cuda"), torch.full((V, d), 9.0, device="cuda")
+    ws2 = torch.empty(U.arrol_lm_head_backward_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+    U.arrol_lm_head_backward(ctx, Hd, Wd, yd, dv(gl), lse, T, d, V, dH, dW, ws2)
+    torch.cuda.synchronize()
+    dH, dW = dH.cpu().numpy().astype(np.float64), dW.cpu().numpy().astype(np.float64)
+    for got, ref in ((dH[rows], dH_ref), (dW, dW_ref)):
+        assert np.abs(got - ref).max() <= 1e-2 * np.abs(ref).max()
+        assert np.linalg.norm(got - ref) <= 5e-3 * np.linalg.norm(ref)
+    assert np.all(np.delete(dH, rows, axis=0) == 0.0)
+
+
+def test_lm_head_backward_with_a_dead_chunk_after_a_live_one(ctx):
+    _backward_case(ctx, 9700, 72, 300, seed=6, T_live=300)
+
+
 def test_lm_head_backward_without_a_live_token(ctx):
     T, d, V = 300, 136, 700
     Z = torch.full((T, d), float("nan"), device="cuda", dtype=torch.bfloat16)
