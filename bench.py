@@ -36,7 +36,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # profiler captures on the small cases of the same d and V (the Llama-shaped and the DAPO-shaped one): (bytes read +
 # bytes written) / tokens of the launch.  At fixed d, V and split count the traffic grows in proportion to the tokens
 # of the launch.
-LOGPROB_DRAM_BYTES_PER_TOKEN = {(2048, 128256, 2): 60090.0}
+LOGPROB_DRAM_BYTES_PER_TOKEN = {(2048, 128256, 2): 62484.0, (4096, 151936, 4): 340069.0}
 # DRAM bytes per scored row of score_linear_kernel streamed over consecutive rows (same kind of capture)
 SCORE_LINEAR_DRAM_BYTES_PER_ROW = {(2048, 2): 4129.8}
 

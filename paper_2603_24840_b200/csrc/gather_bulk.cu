@@ -38,8 +38,9 @@ __device__ __forceinline__ void bulk_store(void* gdst, const void* smem_src, uin
                  ::"l"(gdst), "r"(smem_u32(smem_src)), "r"(bytes), "l"(l2_policy) : "memory");
 }
 // L2 eviction priority of the stored rows.  Packed rows that outgrow L2 are gone before anybody reads them: written back
-// first they leave the cache's share to the reads (1.67 GB of rows of 4 KB: 579 -> 569 us for the prune step, 6.7 GB of 8 KB:
-// 2,093 -> 2,074; the same hint on the loads instead 571 and 2,088).  A packed block that fits stays for the log-prob kernel.
+// first they leave the cache's share to the reads.  arrol_compact with normal / evict-first stores, four runs of each in turn (spread
+// of all runs): 1.77 GB of rows of 4 KB 593 (591-598) / 582 us (578-588), 7.1 GB of 8 KB 2,270 (2,261-2,279) / 2,249 (2,243-2,257);
+// the same hint on the loads instead gains less.  A packed block that fits stays for the log-prob kernel.
 constexpr int64_t L2_BYTES = (int64_t)126 << 20;
 __device__ __forceinline__ uint64_t store_policy(bool streamed) {
     uint64_t p;

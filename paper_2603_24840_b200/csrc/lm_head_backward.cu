@@ -27,7 +27,7 @@
 
 namespace {
 
-constexpr int BM = 128, BN = 256;        // rows of a block, columns of a tile
+constexpr int BM = 128, BN = CHUNK_COLUMNS;   // rows of a block, columns of a tile
 constexpr int TILE_ROWS = 2 * BM;        // rows of a pair's tile
 constexpr int STAGES = 6;
 constexpr int A_STAGE_BYTES = BM * BK * 2;
@@ -342,12 +342,6 @@ __device__ __forceinline__ bool dz_item(int64_t i, int m_tiles, int total_chunks
     c = (int)(i / size);
     m = first + (int)(i - (int64_t)c * size);
     return true;
-}
-
-// Columns of vocabulary chunk c that the MMA computes: a multiple of 32 (the granularity of N for a pair).
-__device__ __forceinline__ int chunk_columns(int V, int c) {
-    const int left = V - c * BN;
-    return left >= BN ? BN : (left + 31) & ~31;
 }
 
 __global__ void __launch_bounds__(NUM_THREADS, 1)

@@ -58,7 +58,7 @@
 namespace {
 
 constexpr int BM = 128;          // token rows per tile  (MMA M)
-constexpr int BN = 256;          // vocabulary columns per chunk (MMA N)
+constexpr int BN = CHUNK_COLUMNS;   // vocabulary columns per chunk (MMA N)
 constexpr int SOLO_STAGES = 4;
 constexpr int A_STAGE_BYTES = BM * BK * 2;   // 16 KB
 constexpr int SOLO_B_STAGE_BYTES = BN * BK * 2;   // 32 KB
@@ -189,13 +189,6 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
-}
-
-// Columns of chunk c that the MMA computes: BN, or what is left of the vocabulary rounded up to 32 (the granularity of
-// N for a pair of blocks, each of which brings half of the rows of W_vocab).
-__device__ __forceinline__ int chunk_columns(int V, int c) {
-    const int left = V - c * BN;
-    return left >= BN ? BN : (left + 31) & ~31;
 }
 
 // 32 columns pc0 ... of one token row into its running record.

@@ -11,8 +11,7 @@
 //                        two warps run the per-group selection (select_lanes, as select_kernel) and write the keep
 //                        flags.  The first warp then scans the block's rollouts (kept, kept length), publishes the
 //                        block's totals, adds up the totals of the blocks before it as they appear (a chained scan:
-//                        every block only waits for lower-numbered blocks, and the grid never exceeds the SM count, so
-//                        all blocks are resident), and writes survivor_idx, cu_seqlens and the advantages of its own
+//                        every block only waits for lower-numbered blocks, of at most two per SM), and writes survivor_idx, cu_seqlens and the advantages of its own
 //                        groups (group_statistics, as scan_adv_kernel); the last block writes {S, T}.  Nothing is
 //                        re-read from global memory and no block waits for the whole grid.  The block that finishes
 //                        last clears the published totals for the next call.
@@ -275,12 +274,11 @@ extern "C" int arrol_prune_step(arrol_ctx* ctx, const arrol_prune_step_args* a, 
     }
     const int64_t fused_blocks = ((int64_t)a->P + gpb - 1) / gpb;
     const size_t w_bytes = linear ? (size_t)a->head.d * (a->head.dtype == ARROL_F32 ? 4 : 2) : 0;
-    // the chained scan needs every block resident: at most (SMs x blocks that fit an SM) blocks
+    // blocks of the chained scan, which wait for lower-numbered ones: at most two per SM
     const int per_sm = 2048 / threads < 1 ? 1 : 2048 / threads;
     if (fused_blocks > (int64_t)ctx->sm_count * (per_sm > 2 ? 2 : per_sm) || fused_blocks > ARROL_CHAIN_BLOCKS ||
         w_bytes > 40 * 1024) {
-        // too many blocks for the chained scan to be resident at once (or a head too wide to stage): the three calls,
-        // back to back
+        // more than the chained scan is made for, or a head too wide to stage: the three calls, back to back
         rc = arrol_score_partial(ctx, a->hidden, a->row_stride_elems, a->row_index, N, &a->head, &a->calib, a->score,
                                  a->prob, a->bin, a->q, stream);
         if (rc != ARROL_OK) return rc;

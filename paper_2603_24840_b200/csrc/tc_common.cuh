@@ -79,12 +79,6 @@ __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m
         ::"r"(smem_u32(smem_dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
 }
 
-__device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_u32(smem_dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)) : "memory");
-}
-
 // Shared memory -> global tile store (bulk async-group completion) and the fences / waits that go with it.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, const void* smem_src) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
@@ -268,7 +262,13 @@ __host__ __device__ constexpr uint32_t make_idesc(int m, int n, bool a_mn = fals
     return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) |
            ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
-
+// Columns of chunk c of 256 vocabulary columns that the MMA computes: 256, or what is left of the vocabulary rounded up to 32 (the
+// granularity of N for a pair of blocks, each of which brings half of the rows of W_vocab).
+constexpr int CHUNK_COLUMNS = 256;
+__device__ __forceinline__ int chunk_columns(int V, int c) {
+    const int left = V - c * CHUNK_COLUMNS;
+    return left >= CHUNK_COLUMNS ? CHUNK_COLUMNS : (left + 31) & ~31;
+}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
