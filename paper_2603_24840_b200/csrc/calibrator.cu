@@ -75,11 +75,13 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 // 64 bins 41 -> 22 us; N = 8,192, 256 bins 100 -> 37 us.  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
-// per thread and scan, as it was before the runs, 460 and 1,570).
+// per thread and scan, as it was before the runs, 460 and 1,570).  An instance each, because the pieces' code in the same one cost
+// small calls 0.3 us and 12,000 rollouts 1.5 (graph of 20 calls: 2,048 25.6 / 25.4 us, 12,000 37.4 / 36.0).
 constexpr int CAL_STAGED = 8192;
 constexpr int CAL_POINTS = 31;                 // points per round, one warp each
 __host__ __device__ inline int product_pitch(int B) { return B | 1; }      // odd: 31 lanes walk 31 rows without bank conflicts
 constexpr int CAL_PRODUCT_BINS = 704;          // most bins whose products are held in shared memory (31 x 705 x 8 = 175 KB)
+template <bool ONE_PIECE>
 __global__ void __launch_bounds__(CAL_THREADS)
 calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ bin, const float* __restrict__ rewards,
                     const uint8_t* __restrict__ mask, int N, double kappa, double lambda, double rho, double p_min,
@@ -110,8 +112,7 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
         for (int j = tid; j < n; j += CAL_THREADS) staged[j] = (int16_t)code_of(from + j);
         return n;
     };
-    const bool one_piece = N <= CAL_STAGED;
-    if (one_piece) stage(0);
+    if constexpr (ONE_PIECE) stage(0);
     // The byte layout L comes from the call's (B, cap); the state must have been initialised with the same pair.
     // A mismatched or uninitialised state is left untouched and reported (uniform over the block: no barrier yet).
     if (hd->B != B || hd->cap != cap) {
@@ -169,7 +170,7 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     };
     int j0 = 0, j1 = 0;
     int64_t total_new[2], first_rank[2];
-    if (one_piece) {
+    if constexpr (ONE_PIECE) {
         rank_run(N, j0, j1, first_rank, total_new);
     } else {                                     // how many there are of each label decides what is evicted and what stays
         int32_t mine[2] = {0, 0};
@@ -212,7 +213,7 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
             }
         };
         int64_t before[2] = {0, 0};
-        if (one_piece) write_run(before);
+        if constexpr (ONE_PIECE) write_run(before);
         else
             for (int64_t from = 0; from < N; from += CAL_STAGED) {
                 int64_t here[2];
@@ -458,15 +459,17 @@ extern "C" int arrol_calib_update(arrol_ctx* ctx, void* state, int32_t B, int64_
     if (N > 0 && (!bin || !rewards)) return ARROL_ERR_INVALID_ARG;
     ArrolDeviceGuard guard(ctx->device);
     if (!guard.ok) return ARROL_ERR_CUDA;
+    const auto one_piece = calib_update_kernel<true>, pieces = calib_update_kernel<false>;
     if (!ctx->calib_smem_set) {
-        ARROL_CUDA_OK(cudaFuncSetAttribute(calib_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(sizeof(double) * CAL_POINTS * product_pitch(CAL_PRODUCT_BINS))));
+        const int most = (int)(sizeof(double) * CAL_POINTS * product_pitch(CAL_PRODUCT_BINS));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(one_piece, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(pieces, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
         ctx->calib_smem_set = true;
     }
     const size_t smem = B <= CAL_PRODUCT_BINS ? sizeof(double) * CAL_POINTS * product_pitch(B) : 0;
-    calib_update_kernel<<<1, CAL_THREADS, smem, (cudaStream_t)stream>>>(static_cast<uint8_t*>(state), layout_of(B, cap), bin,
-                                                                  rewards, mask, N, sp->kappa, sp->lambda, sp->rho,
-                                                                  sp->p_min, sp->p_max, B, cap, ctx->d_status);
+    (N <= CAL_STAGED ? one_piece : pieces)<<<1, CAL_THREADS, smem, (cudaStream_t)stream>>>(
+        static_cast<uint8_t*>(state), layout_of(B, cap), bin, rewards, mask, N, sp->kappa, sp->lambda, sp->rho, sp->p_min, sp->p_max,
+        B, cap, ctx->d_status);
     ctx->launches += 1;
     ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;
