@@ -137,15 +137,17 @@ struct Lockstep {
     uint32_t units, epochs;     // epochs of the pair with the most work
     int items_per_epoch;        // > 1 when a tile has few K steps
 };
-__device__ __forceinline__ Lockstep lockstep_for(unsigned int* words, int word, int64_t units, int64_t items, int k_steps) {
+// `body` items of k_steps K steps each, then `tail` items of at most tail_steps (the same number where k_steps < EPOCH)
+__device__ __forceinline__ Lockstep lockstep_for(unsigned int* words, int word, int64_t units, int64_t body, int k_steps, int64_t tail,
+                                                 int tail_steps) {
     Lockstep l;
     l.words = words;
     l.word = word;
     l.units = (uint32_t)units;
     l.items_per_epoch = k_steps >= EPOCH ? 1 : EPOCH / max(k_steps, 1);
-    const int64_t most = (items + units - 1) / units;
-    l.epochs = (uint32_t)(k_steps >= EPOCH ? most * ((k_steps + EPOCH - 1) / EPOCH)
-                                           : (most + l.items_per_epoch - 1) / l.items_per_epoch);
+    const int64_t most = (body + units - 1) / units, most_tail = (tail + units - 1) / units;
+    l.epochs = (uint32_t)(k_steps >= EPOCH ? most * ((k_steps + EPOCH - 1) / EPOCH) + most_tail * ((tail_steps + EPOCH - 1) / EPOCH)
+                                           : (most + most_tail + l.items_per_epoch - 1) / l.items_per_epoch);
     return l;
 }
 // One thread, at the beginning of its pair's epoch `epoch`.  False: waited in vain.
@@ -163,8 +165,9 @@ __device__ __forceinline__ bool begin_epoch(const Lockstep& lock, volatile uint3
     return true;
 }
 
-// One accumulator tile's operands: origin of the tile's rows (A) and columns (B), and the columns that the MMA computes.
-struct TileAt { int a0, b0, n; };
+// One accumulator tile's operands: origin of the tile's rows (A) and columns (B), the columns that the MMA computes, the K steps
+// [k0, k1), and where the result goes: the output (slot < 0) or a slot of partial sums.
+struct TileAt { int a0, b0, n, k0, k1, slot; };
 
 // Producer role (one warp of each block; the warp walks the loops and waits, one elected lane issues).  For every accumulator tile `coords(it, tile)` gives the operands' MN origins
 // (false when the list is exhausted); this block loads rows a0 + 128 rank ... of A and b0 + (n / 2) rank ... of B.  Per K step
@@ -175,7 +178,7 @@ struct TileAt { int a0, b0, n; };
 // Both blocks' bytes are counted on the leading block's barrier.
 template <bool A_MN, bool B_MN, typename Coords>
 __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensorMap* ma, const CUtensorMap* mb,
-                                              int k_steps, const Lockstep& lock, Coords coords, bool a3d = false, bool b3d = false,
+                                              const Lockstep& lock, Coords coords, bool a3d = false, bool b3d = false,
                                               const CUtensorMap* mb_tail = nullptr, int tail_ks = -1) {
     const uint32_t a0 = smem_u32(ps.stage_a), b0 = smem_u32(ps.stage_b);
     uint32_t stage = 0, phase = 0, issued = 0, epoch = 0;
@@ -185,8 +188,8 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
     if (blockIdx.x == 0 && elect_one()) lock.words[(lock.word + 1) % LOCK_WORDS] = 0u;
     for (int64_t it = 0; ok && coords(it, tile); ++it) {
         const int ay = tile.a0 + (int)ps.rank * BM, by = tile.b0 + (int)ps.rank * (tile.n / 2);
-        for (int ks0 = 0; ks0 < k_steps && ok; ks0 += EPOCH) {
-            if (ks0 > 0 || to_epoch == 0) {
+        for (int ks0 = tile.k0; ks0 < tile.k1 && ok; ks0 += EPOCH) {
+            if (ks0 > tile.k0 || to_epoch == 0) {
                 if (ps.rank == 0) {
                     if (elect_one()) {
                         if (in_step) in_step = begin_epoch(lock, ps.lock_seen, epoch);
@@ -195,9 +198,9 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
                     in_step = __all_sync(0xffffffffu, in_step) != 0;
                 }
                 ++epoch;
-                if (ks0 == 0) to_epoch = lock.items_per_epoch;
+                if (ks0 == tile.k0) to_epoch = lock.items_per_epoch;
             }
-            const int ks1 = min(ks0 + EPOCH, k_steps);
+            const int ks1 = min(ks0 + EPOCH, tile.k1);
             for (int ks = ks0; ks < ks1; ++ks) {
                 if (!mbar_wait_warp(&ps.empty[stage], phase ^ 1u, ps.abort_flag)) { ok = false; break; }
                 if (elect_one()) {
@@ -256,26 +259,26 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
     __syncwarp();
 }
 
-// MMA role (one warp of the leading block): the accumulator tiles that `columns(it)` lists (their MMA columns, 0 = no
-// more), k_steps K steps each (the last one of k_last slices of 16), alternating the two accumulators.  The whole warp
+// MMA role (one warp of the leading block): the accumulator tiles that `coords(it, tile)` lists (false: no more), the last of all
+// k_steps K steps having k_last slices of 16, alternating the two accumulators.  The whole warp
 // walks the loops and waits, one elected lane issues.
 // Inside a stage the four K = 16 slices are 32 bytes apart for a K-major operand (columns of the swizzled row) and
 // 16 rows = 2048 bytes apart for an MN-major one.
-template <bool A_MN, bool B_MN, typename Columns>
-__device__ __forceinline__ void mma_loop(const PipeSmem& ps, int k_steps, int k_last, Columns columns) {
+template <bool A_MN, bool B_MN, typename Coords>
+__device__ __forceinline__ void mma_loop(const PipeSmem& ps, int k_steps, int k_last, Coords coords) {
     constexpr uint64_t a_step = A_MN ? (UMMA_K * 128) >> 4 : (UMMA_K * 2) >> 4;
     constexpr uint64_t b_step = B_MN ? (UMMA_K * 128) >> 4 : (UMMA_K * 2) >> 4;
     const uint32_t a0 = smem_u32(ps.stage_a), b0 = smem_u32(ps.stage_b);
     uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
     bool ok = true;
-    for (int64_t it = 0; ok; ++it) {
-        const int n = columns(it);
-        if (n == 0) break;
-        const uint32_t idesc = make_idesc(TILE_ROWS, n, A_MN, B_MN);
+    TileAt tile;
+    for (int64_t it = 0; ok && coords(it, tile); ++it) {
+        const uint32_t idesc = make_idesc(TILE_ROWS, tile.n, A_MN, B_MN);
         if (!mbar_wait_warp(&ps.acc_empty[acc], acc_phase ^ 1u, ps.abort_flag)) { ok = false; break; }
         tcgen05_fence_after();
         const uint32_t d_tmem = ps.tmem_base + acc * BN;
-        for (int ks = 0; ks < k_steps; ++ks) {
+        const int k0 = tile.k0, k1 = tile.k1;
+        for (int ks = k0; ks < k1; ++ks) {
             if (!mbar_wait_warp(&ps.full[stage], phase, ps.abort_flag)) { ok = false; break; }
             tcgen05_fence_after();
             const uint32_t sa = a0 + stage * A_STAGE_BYTES, sb = b0 + stage * B_STAGE_BYTES;
@@ -285,13 +288,13 @@ __device__ __forceinline__ void mma_loop(const PipeSmem& ps, int k_steps, int k_
                 if (ks + 1 < k_steps || k_last == BK / UMMA_K) {
 #pragma unroll
                     for (int k = 0; k < BK / UMMA_K; ++k)
-                        tcgen05_mma_bf16_pair(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, (ks | k) != 0 ? 1u : 0u);
+                        tcgen05_mma_bf16_pair(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, ((ks - k0) | k) != 0 ? 1u : 0u);
                 } else {
                     for (int k = 0; k < k_last; ++k)         // slices past the end of K are zeros
-                        tcgen05_mma_bf16_pair(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, (ks | k) != 0 ? 1u : 0u);
+                        tcgen05_mma_bf16_pair(d_tmem, a_desc + a_step * k, b_desc + b_step * k, idesc, ((ks - k0) | k) != 0 ? 1u : 0u);
                 }
                 tcgen05_commit_pair(&ps.empty[stage], (uint16_t)3);
-                if (ks + 1 == k_steps) tcgen05_commit_pair(&ps.acc_full[acc], (uint16_t)3);
+                if (ks + 1 == k1) tcgen05_commit_pair(&ps.acc_full[acc], (uint16_t)3);
             }
             __syncwarp();
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -331,17 +334,43 @@ struct DzParams {
     uint32_t* d_status;
 };
 
-__device__ __forceinline__ bool dz_item(int64_t i, int m_tiles, int total_chunks, int group_tiles, int& m, int& c) {
+// The last items, which would keep at most half of the pairs busy for one more wave, go as two halves of their columns each:
+// the last wave then takes about 0.6 of a whole one (an operand of the rows for half the MMAs).
+struct DzWork { int m_tiles, total_chunks, group_tiles; int64_t body, items; };
+__device__ __forceinline__ DzWork make_dz_work(int m_tiles, int total_chunks, int group_tiles, int64_t units) {
+    DzWork w;
+    w.m_tiles = m_tiles;
+    w.total_chunks = total_chunks;
+    w.group_tiles = group_tiles;
+    const int64_t tiles = (int64_t)m_tiles * total_chunks, tail = tiles % units;
+    const bool halves = 2 * tail <= units;
+    w.body = halves ? tiles - tail : tiles;
+    w.items = halves ? tiles + tail : tiles;
+    return w;
+}
+// (m, c): token tile and vocabulary chunk; half: 0 or 1, -1 for the whole chunk
+__device__ __forceinline__ bool dz_item(const DzWork& w, int64_t i, int& m, int& c, int& half) {
+    const int m_tiles = w.m_tiles, total_chunks = w.total_chunks, group_tiles = w.group_tiles;
+    if (i >= w.items) return false;
+    half = -1;
+    if (i >= w.body) {
+        half = (int)((i - w.body) & 1);
+        i = w.body + ((i - w.body) >> 1);
+    }
     const int64_t per_group = (int64_t)group_tiles * total_chunks;
     const int64_t g = i / per_group;
     const int first = (int)g * group_tiles;
-    if (first >= m_tiles) return false;
     const int size = min(group_tiles, m_tiles - first);
     i -= g * per_group;
-    if (i >= (int64_t)size * total_chunks) return false;
     c = (int)(i / size);
     m = first + (int)(i - (int64_t)c * size);
     return true;
+}
+// first column of an item and how many the MMA computes (32 at least: a half that lies past V is zeros, which nobody stores)
+__device__ __forceinline__ int dz_column(int c, int half) { return c * BN + (half > 0 ? BN / 2 : 0); }
+__device__ __forceinline__ int dz_columns(int V, int c, int half) {
+    const int left = (max(V - dz_column(c, half), 1) + 31) & ~31;
+    return min(left, half >= 0 ? BN / 2 : BN);
 }
 
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -358,23 +387,23 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
     const int k_last = (p.d - (k_steps - 1) * BK + UMMA_K - 1) / UMMA_K;
     const int total_chunks = (p.V + BN - 1) / BN;
     const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
+    const DzWork work = make_dz_work(m_tiles, total_chunks, p.group_tiles, units);
+    auto coords = [&](int64_t it, TileAt& t) {
+        int m, c, half;
+        if (!dz_item(work, unit + it * units, m, c, half)) return false;
+        t.a0 = (int)p.t0 + m * TILE_ROWS;
+        t.b0 = dz_column(c, half);
+        t.n = dz_columns(p.V, c, half);
+        t.k0 = 0;
+        t.k1 = k_steps;
+        return true;
+    };
 
     if (warp == 0) {
-        const Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, (int64_t)m_tiles * total_chunks, k_steps);
-        producer_loop<false, false>(ps, &map_h, &map_w, k_steps, lock, [&](int64_t it, TileAt& t) {
-            int m, c;
-            if (!dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c)) return false;
-            t.a0 = (int)p.t0 + m * TILE_ROWS;
-            t.b0 = c * BN;
-            t.n = chunk_columns(p.V, c);
-            return true;
-        });
+        const Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, work.body, k_steps, work.items - work.body, k_steps);
+        producer_loop<false, false>(ps, &map_h, &map_w, lock, coords);
     } else if (warp == 1) {
-        if (ps.rank == 0)
-            mma_loop<false, false>(ps, k_steps, k_last, [&](int64_t it) {
-                int m, c;
-                return dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c) ? chunk_columns(p.V, c) : 0;
-            });
+        if (ps.rank == 0) mma_loop<false, false>(ps, k_steps, k_last, coords);
     } else {
         // The last, partly live 64-row block of the chunk's hidden rows, padded with zeros, for the dW contraction: rows past
         // the live tokens (caller memory that may hold anything) never reach the tensor core.  At most 63 rows live in it; the
@@ -402,8 +431,9 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
         uint8_t* stg = dz_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        int m, c;
-        for (int64_t item = unit; ok && dz_item(item, m_tiles, total_chunks, p.group_tiles, m, c); item += units) {
+        int m, c, half;
+        for (int64_t item = unit; ok && dz_item(work, item, m, c, half); item += units) {
+            const int first_col = dz_column(c, half);
             const int row0 = m * TILE_ROWS + (int)ps.rank * BM + quarter * 32;
             const int64_t t = p.t0 + row0 + lane;
             int y = -1;
@@ -425,7 +455,7 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
             // into dz and staged.
             const uint32_t tacc = ps.tmem_base + lane_addr + acc * BN;
             auto to_dz = [&](const uint32_t (&raw)[32], int piece, uint32_t (&packed)[16]) {
-                const int pc0 = c * BN + piece * 32;
+                const int pc0 = first_col + piece * 32;
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
                     // dz = coef ([v = y] - 2^(z log2e - lse log2e)); coef = 0 for rows that carry no gradient
@@ -446,7 +476,8 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
                         make_uint4(packed[4 * q4], packed[4 * q4 + 1], packed[4 * q4 + 2], packed[4 * q4 + 3]);
             };
             uint32_t ra[32], rb[32];
-            const int p0 = col_half * EPI_PIECES, p1 = p0 + EPI_PIECES;   // this warp's pieces of the accumulator
+            const int pieces = half >= 0 ? EPI_PIECES / 2 : EPI_PIECES;
+            const int p0 = col_half * pieces, p1 = p0 + pieces;           // this warp's pieces of the accumulator
             tcgen05_ld_32x32_issue(tacc + p0 * 32, ra);
 #pragma unroll 1
             for (int piece = p0; piece < p1; piece += 2) {
@@ -463,7 +494,7 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
                 stage_piece(pb, piece + 1);
                 fence_proxy_async_smem();
                 __syncwarp();
-                const int col0 = c * BN + piece * 32;
+                const int col0 = first_col + piece * 32;
                 if (lane == 0 && col0 < p.V) {
                     tma_store_2d(&map_dz, col0, row0, stg);
                     bulk_commit_group();
@@ -485,6 +516,18 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
 // Tiles of 256 x 256, dealt to the pairs in groups of `group_n` column tiles: within a group consecutive pairs share the
 // A panel and walk the B panels.  group_n keeps the B panels of a group (for dW a whole chunk of hidden rows) in L2 and the
 // wave of 74 tiles near square, which is what it reads least bytes per K step with.
+//   Whole waves of tiles are the body; the tiles left over (all of them where there are fewer than pairs) would keep part of the
+// pairs busy for a whole wave, which is what a call of a few hundred tokens, with dH tiles of thousands of K steps on a handful
+// of pairs, spent its time on.  So they are cut (GemmWork): for dH into ranges of K, the first of which writes dH and the others
+// partial sums (in the rows of dZ that the chunk's tokens leave unused), added to dH in the order of the ranges by the epilogue
+// warps of the dW kernel, which wait for their first tile at that time; where there is no room for partial sums, and for
+// dW, into halves of their columns.  Neither depends on anything but the sizes, so results are the same from run to run.
+struct SumParams {            // dW kernel: the dH contraction whose partial sums it adds up
+    const float* part;
+    float* out;
+    int M, N, K, group_n, slots;
+    int64_t units;
+};
 struct GemmParams {
     int M, N, K;
     int group_n;
@@ -498,6 +541,8 @@ struct GemmParams {
     int64_t T_max, t0;
     unsigned int* lock_words;
     int lock_word;
+    int slots;                // partial sums of a tile that fit the workspace (dH)
+    SumParams sum;
     uint32_t* d_status;
 };
 
@@ -516,11 +561,91 @@ __device__ __forceinline__ bool gemm_item(int64_t i, int m_tiles, int n_tiles, i
     return true;
 }
 
+// How the tiles of a launch are dealt.  Items [0, body) are whole tiles in the order of gemm_item; then the tail, by range of K and
+// tile (segs > 1; the tile as the fast index, so that the pairs that work at the same time share operand panels) or by tile and
+// half.  Where all tiles are tail, and the last column tile is half as wide as the others, its tiles are cut into half as many
+// ranges and come last.
+constexpr int MIN_SEG = 16;              // K steps of a range at least: an epoch of the lock-step, and ten times what its set-up takes
+constexpr int SEG_COST = 12;             // K steps that a wave of ranges costs beside its own (writing and adding 256 KB a pair)
+struct GemmWork {
+    int m_tiles, n_tiles, group_n, k_steps;
+    int body, tail, items;
+    int segs, narrow_segs;               // ranges of K per tail tile; of the narrow ones at the end of the tail
+    int wide;                            // tail tiles before the narrow ones
+};
+__device__ __forceinline__ GemmWork make_gemm_work(int m_tiles, int n_tiles, int group_n, int k_steps, int N, int units, int slots) {
+    GemmWork w;
+    w.m_tiles = m_tiles; w.n_tiles = n_tiles; w.group_n = group_n; w.k_steps = k_steps;
+    const int tiles = m_tiles * n_tiles;
+    int tail = tiles % units;
+    w.segs = w.narrow_segs = 1;
+    const bool narrow = tail == tiles && n_tiles > 1 && N - (n_tiles - 1) * BN <= BN / 2;
+    w.wide = narrow ? tail - m_tiles : tail;
+    bool halves = false;
+    if (tail > 0) {
+        const int load = 2 * w.wide + (narrow ? m_tiles : 0);        // in half tiles
+        int best = k_steps;
+        if (2 * tail <= units && !narrow) { halves = true; best = k_steps * 5 / 8; }
+#pragma unroll 1
+        for (int waves = 1; waves <= 3; ++waves) {
+            int s = min(2 * waves * units / load, min(k_steps / MIN_SEG, 2 * (slots + tail) / load));
+            if (narrow) s &= ~1;
+            if (s < 2 || s > 2 * units) continue;
+            const int cost = waves * ((k_steps + s - 1) / s + SEG_COST);
+            if (cost < best) { best = cost; w.segs = s; halves = false; }
+        }
+        w.narrow_segs = narrow && w.segs > 1 ? w.segs / 2 : w.segs;
+        if (w.segs == 1 && !halves) tail = 0;                        // nothing to gain: whole tiles to the end
+    }
+    w.tail = tail;
+    w.body = tiles - tail;
+    w.items = w.body + (w.segs > 1 ? w.wide * w.segs + (tail - w.wide) * w.narrow_segs : halves ? 2 * tail : 0);
+    return w;
+}
+// slot of range seg > 0 of tail tile idx
+__device__ __forceinline__ int gemm_slot(const GemmWork& w, int idx, int seg) {
+    return idx < w.wide ? (seg - 1) * w.wide + idx : (w.segs - 1) * w.wide + (seg - 1) * (w.tail - w.wide) + idx - w.wide;
+}
+__device__ __forceinline__ GemmTile gemm_tail_tile(const GemmWork& w, int idx) {
+    GemmTile g;
+    if (w.body > 0) gemm_item(w.body + idx, w.m_tiles, w.n_tiles, w.group_n, g);
+    else { g.n = idx / w.m_tiles; g.m = idx - g.n * w.m_tiles; }
+    return g;
+}
+__device__ __forceinline__ bool gemm_work_item(const GemmWork& w, int N, int64_t item, GemmTile& g, TileAt& t) {
+    if (item >= w.items) return false;
+    int i = (int)item, half = -1;
+    t.k0 = 0;
+    t.k1 = w.k_steps;
+    t.slot = -1;
+    if (i < w.body) {
+        gemm_item(i, w.m_tiles, w.n_tiles, w.group_n, g);
+    } else if (w.segs > 1) {
+        i -= w.body;
+        const bool wide = i < w.wide * w.segs;
+        const int count = wide ? w.wide : w.tail - w.wide, segs = wide ? w.segs : w.narrow_segs;
+        if (!wide) i -= w.wide * w.segs;
+        const int seg = i / count, idx = i - seg * count + (wide ? 0 : w.wide);
+        t.k0 = (int)((unsigned)seg * (unsigned)w.k_steps / (unsigned)segs);            // segs <= 2 units, k_steps < 2^25 / 64 columns a step
+        t.k1 = (int)((unsigned)(seg + 1) * (unsigned)w.k_steps / (unsigned)segs);
+        if (seg > 0) t.slot = gemm_slot(w, idx, seg);
+        g = gemm_tail_tile(w, idx);
+    } else {
+        half = (i - w.body) & 1;
+        g = gemm_tail_tile(w, (i - w.body) >> 1);
+    }
+    t.a0 = g.m * TILE_ROWS;
+    t.b0 = g.n * BN + (half > 0 ? BN / 2 : 0);
+    // 64 columns per block at least: the granularity of an MN-major B tile's blocks
+    t.n = half < 0 && N - t.b0 > BN / 2 ? BN : BN / 2;
+    return true;
+}
+
 template <bool A_MN, bool B_MN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_b_tail, const __grid_constant__ CUtensorMap map_c,
-            const GemmParams p) {
+            const __grid_constant__ CUtensorMap map_part, const GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     const PipeSmem ps = pipe_setup(smem_raw, &map_a, &map_b);
     uint8_t* c_stage = ps.stage_a + EPI_STAGE_OFFSET;      // one 32 x 32 fp32 staging tile per epilogue warp
@@ -535,26 +660,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int m_tiles = K == 0 ? 0 : p.m_is_tokens ? (int)min((int64_t)all_m_tiles, (live + TILE_ROWS - 1) / TILE_ROWS) : all_m_tiles;
     const int zero_m_tiles = live > 0 || p.zero_if_dead ? all_m_tiles - m_tiles : 0;
     const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
-    // 64 columns per block at least: the granularity of an MN-major B tile's blocks
-    auto columns = [&](int n) { const int left = p.N - n * BN; return left > BN / 2 ? BN : BN / 2; };
+    const GemmWork work = make_gemm_work(m_tiles, n_tiles, p.group_n, k_steps, p.N, (int)units, p.slots);
+    auto coords = [&](int64_t it, TileAt& t) {
+        GemmTile g;
+        return gemm_work_item(work, p.N, unit + it * units, g, t);
+    };
 
     if (warp == 0) {
         const int tail_ks = (p.k_is_tokens && (K % BK) != 0) ? k_steps - 1 : -1;
-        const Lockstep lock = lockstep_for(p.lock_words, p.lock_word, units, (int64_t)m_tiles * n_tiles, k_steps);
-        producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, k_steps, lock, [&](int64_t it, TileAt& t) {
-            GemmTile g;
-            if (!gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g)) return false;
-            t.a0 = g.m * TILE_ROWS;
-            t.b0 = g.n * BN;
-            t.n = columns(g.n);
-            return true;
-        }, p.a3d != 0, p.b3d != 0, &map_b_tail, tail_ks);
+        const Lockstep lock = lockstep_for(p.lock_words, p.lock_word, units, work.body, k_steps, work.items - work.body,
+                                           (k_steps + work.narrow_segs - 1) / work.narrow_segs);
+        producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, lock, coords, p.a3d != 0, p.b3d != 0, &map_b_tail, tail_ks);
     } else if (warp == 1) {
-        if (ps.rank == 0)
-            mma_loop<A_MN, B_MN>(ps, k_steps, k_last, [&](int64_t it) {
-                GemmTile g;
-                return gemm_item(unit + it * units, m_tiles, n_tiles, p.group_n, g) ? columns(g.n) : 0;
-            });
+        if (ps.rank == 0) mma_loop<A_MN, B_MN>(ps, k_steps, k_last, coords);
     } else {
         const int quarter = warp & 3;
         const int col_half = (warp - 2) >> 2;           // 0 or 1: which half of the accumulator's columns
@@ -563,12 +681,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         // as one TMA reduction (global += tile) when the result is accumulated: whole 128-byte lines, no read of C by
         // the SM, and rows / columns past M / N are clipped by the copy.
         uint8_t* stg = c_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
-        auto store_tile = [&](const GemmTile& g, bool zero, uint32_t tacc) {
-            const int row0 = g.m * TILE_ROWS + (int)ps.rank * BM + quarter * 32;
+        auto store_tile = [&](const TileAt& t, bool zero, uint32_t tacc) {
+            const bool partial = t.slot >= 0;
+            const int row0 = (partial ? t.slot * TILE_ROWS : t.a0) + (int)ps.rank * BM + quarter * 32;
+            const int pieces = t.n / 32 / (EPI_WARPS / 4);              // of this warp
 #pragma unroll 1
-            for (int piece = col_half * EPI_PIECES; piece < (col_half + 1) * EPI_PIECES; ++piece) {
-                const int pc0 = g.n * BN + piece * 32;
-                if (pc0 >= p.N) break;
+            for (int piece = col_half * pieces; piece < (col_half + 1) * pieces; ++piece) {
+                if (t.b0 + piece * 32 >= p.N) break;
+                const int pc0 = (partial ? 0 : t.b0) + piece * 32;
                 float v[32];
                 if (zero) {
 #pragma unroll
@@ -584,32 +704,57 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                         make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
                 fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0 && row0 < p.M) {
-                    if (p.accumulate) tma_reduce_add_2d(&map_c, pc0, row0, stg);
+                if (lane == 0 && (partial || row0 < p.M)) {
+                    if (partial) tma_store_2d(&map_part, pc0, row0, stg);
+                    else if (p.accumulate) tma_reduce_add_2d(&map_c, pc0, row0, stg);
                     else tma_store_2d(&map_c, pc0, row0, stg);
                     bulk_commit_group();
                 }
             }
         };
+        if constexpr (A_MN) {       // dH += its partial sums, in the order of the ranges of K
+            const SumParams& h = p.sum;
+            const int h_tiles = (int)min((int64_t)((h.M + TILE_ROWS - 1) / TILE_ROWS), (live + TILE_ROWS - 1) / TILE_ROWS);
+            const GemmWork hw = make_gemm_work(h_tiles, n_tiles, h.group_n, (h.K + BK - 1) / BK, h.N, (int)h.units, h.slots);
+            if (hw.segs > 1) {
+                constexpr int QUADS = TILE_ROWS * BN / 4;                // of a tile
+                const float* part = pdl_acquire(h.part);
+                const int stride = (int)gridDim.x * 32 * EPI_WARPS;
+                for (int i = (int)blockIdx.x * 32 * EPI_WARPS + (int)threadIdx.x - 64; i < hw.tail * QUADS; i += stride) {
+                    const int idx = i / QUADS, r = i / (BN / 4) % TILE_ROWS, q = i % (BN / 4);
+                    const GemmTile g = gemm_tail_tile(hw, idx);
+                    const int row = g.m * TILE_ROWS + r, col = g.n * BN + 4 * q;
+                    if (row >= h.M || col >= h.N) continue;              // N is a multiple of 8
+                    float4* out = reinterpret_cast<float4*>(h.out + (int64_t)row * h.N + col);
+                    float4 v = __ldcg(out);
+                    const int segs = idx < hw.wide ? hw.segs : hw.narrow_segs;
+#pragma unroll 8
+                    for (int seg = 1; seg < segs; ++seg) {
+                        const float4 x = __ldcg(reinterpret_cast<const float4*>(part + ((int64_t)gemm_slot(hw, idx, seg) * TILE_ROWS + r) * BN + 4 * q));
+                        v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+                    }
+                    *out = v;
+                }
+            }
+        }
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
         GemmTile g;
-        for (int64_t item = unit; ok && gemm_item(item, m_tiles, n_tiles, p.group_n, g); item += units) {
+        TileAt t;
+        for (int64_t item = unit; ok && gemm_work_item(work, p.N, item, g, t); item += units) {
             ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
             ok = __all_sync(0xffffffffu, ok) != 0;
             if (!ok) break;
             tcgen05_fence_after();
-            store_tile(g, false, ps.tmem_base + lane_addr + acc * BN);
+            store_tile(t, false, ps.tmem_base + lane_addr + acc * BN);
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (!p.accumulate)
-            for (int64_t item = unit; gemm_item(item, zero_m_tiles, n_tiles, p.group_n, g); item += units) {
-                g.m += m_tiles;
-                store_tile(g, true, 0u);
-            }
+            for (int64_t item = unit; gemm_item(item, zero_m_tiles, n_tiles, p.group_n, g); item += units)
+                store_tile(TileAt{(m_tiles + g.m) * TILE_ROWS, g.n * BN, BN, 0, 0, -1}, true, 0u);
         if (lane == 0) bulk_wait_all();       // the tile copies have completed before the block's shared memory goes
     }
     pipe_teardown(ps, p.d_status);
@@ -620,9 +765,9 @@ int group_columns(int n_tiles) {          // column tiles per group: at most 10 
     return (n_tiles + groups - 1) / groups;
 }
 
+// As many pairs as fit the GPU at once: those without a tile of their own take part of another's.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pairs(arrol_ctx* ctx, int which, void (*kernel)(KArgs...), int64_t items, cudaStream_t s, Args&&... args) {
-    int64_t pairs = items < 1 ? 1 : (items < ctx->sm_count / 2 ? items : ctx->sm_count / 2);
+cudaError_t launch_pairs(arrol_ctx* ctx, int which, void (*kernel)(KArgs...), cudaStream_t s, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(NUM_THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
@@ -646,8 +791,7 @@ cudaError_t launch_pairs(arrol_ctx* ctx, int which, void (*kernel)(KArgs...), in
         if (fit < 1) return cudaErrorInvalidConfiguration;
         ctx->backward_max_pairs[which] = fit;
     }
-    if (pairs > ctx->backward_max_pairs[which]) pairs = ctx->backward_max_pairs[which];
-    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.gridDim = dim3((unsigned)(2 * ctx->backward_max_pairs[which]));
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
@@ -731,7 +875,7 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     }
     if (!v3 && make_map_ld(ctx, &map_dz_mn, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BK) != ARROL_OK) return ARROL_ERR_CUDA;
 
-    const int total_chunks = (V + BN - 1) / BN, n_tiles = (d + BN - 1) / BN;
+    const int n_tiles = (d + BN - 1) / BN;
     int m_groups = 1;
     while ((double)TC / m_groups * d * 2 > 50.0 * 1024 * 1024) ++m_groups;
 
@@ -750,7 +894,7 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         zp.scale2 = inv_temperature * 1.44269504088896340736f; zp.inv_temp = inv_temperature;
         zp.lock_words = lock_words;
         zp.hidden = static_cast<const uint16_t*>(hidden); zp.tail = Htail; zp.d_status = ctx->d_status;
-        ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, (int64_t)m_tiles * total_chunks, s, map_h_k, map_w_k, map_dz_st, zp));
+        ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, s, map_h_k, map_w_k, map_dz_st, zp));
 
         GemmParams gh = {};    // dH[chunk] = dZ . W
         gh.M = (int)rows; gh.N = d; gh.K = V; gh.group_n = group_columns(n_tiles);
@@ -759,15 +903,23 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         CUtensorMap map_dh;      // this chunk's rows of dH: rows past the chunk are clipped by the tile stores
         if (make_map_f32_tile(ctx, &map_dh, dH + t0 * d, (uint64_t)rows, (uint64_t)d, (uint64_t)d) != ARROL_OK)
             return ARROL_ERR_CUDA;
-        ARROL_CUDA_OK(launch_pairs(ctx, 1, gemm_kernel<false, true>, (int64_t)m_tiles * n_tiles, s, map_dz_k, map_w_mn, map_w_mn,
-                                   map_dh, gh));
+        // partial sums of dH tiles lie in the rows of dZ that no tile of this chunk reaches
+        constexpr size_t SLOT_BYTES = sizeof(float) * TILE_ROWS * BN;
+        const size_t part_at = ((size_t)m_tiles * TILE_ROWS * L.ldz * 2 + 255) & ~(size_t)255;
+        float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + L.dz + part_at);
+        const size_t room = (L.tail - part_at) / SLOT_BYTES;
+        gh.slots = room < 4096 ? (int)room : 4096;
+        CUtensorMap map_part = map_dh;
+        if (gh.slots > 0 && make_map_f32_tile(ctx, &map_part, part, (uint64_t)gh.slots * TILE_ROWS, BN, BN) != ARROL_OK) return ARROL_ERR_CUDA;
+        ARROL_CUDA_OK(launch_pairs(ctx, 1, gemm_kernel<false, true>, s, map_dz_k, map_w_mn, map_w_mn, map_dh, map_part, gh));
         GemmParams gw = {};    // dW (+)= dZ^T . H[chunk]; the first chunk writes dW, zeros where no token lives
         gw.M = V; gw.N = d; gw.K = (int)rows; gw.group_n = group_columns(n_tiles);
         gw.accumulate = t0 > 0; gw.k_is_tokens = 1; gw.zero_if_dead = t0 == 0; gw.a3d = v3; gw.b3d = d3;
         gw.lock_words = lock_words; gw.lock_word = LOCK_DW;
         gw.d_T = d_T; gw.T_max = T_max; gw.t0 = t0; gw.d_status = ctx->d_status;
-        ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, (int64_t)((V + TILE_ROWS - 1) / TILE_ROWS) * n_tiles, s,
-                                   map_dz_mn, map_h_mn, map_h_tail, map_dw, gw));
+        gw.sum.part = part; gw.sum.out = dH + t0 * d; gw.sum.M = gh.M; gw.sum.N = gh.N; gw.sum.K = gh.K;
+        gw.sum.group_n = gh.group_n; gw.sum.slots = gh.slots; gw.sum.units = ctx->backward_max_pairs[1];
+        ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, s, map_dz_mn, map_h_mn, map_h_tail, map_dw, map_dw, gw));
         ctx->launches += 3;
     }
     return ARROL_OK;

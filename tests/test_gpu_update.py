@@ -139,6 +139,43 @@ def test_lm_head_backward_with_groups_of_tiles(ctx, d):
     assert np.all(np.delete(dH, rows, axis=0) == 0.0)
 
 
+# tiles that are cut: all of dH along K, with a last column tile of half width (600) or one column tile and dead rows (900); 10 tiles
+# beyond a whole wave of 74 along K (7,000); 37 tiles in halves of their columns, without room for partial sums (9,472); vocabulary
+# chunks in halves, the last one with nothing in its second half (600, 257)
+@pytest.mark.parametrize("T,d,V,T_live", [(600, 320, 20000, None), (900, 72, 9001, 777), (7000, 768, 12000, None), (9472, 256, 700, None),
+                                          (257, 520, 5000, 256)])
+def test_lm_head_backward_with_cut_tiles(ctx, T, d, V, T_live):
+    g = np.random.default_rng(T + d)
+    n = T if T_live is None else T_live
+    H = torch.from_numpy(g.normal(size=(T, d)).astype(np.float32)).to(torch.bfloat16)
+    W = torch.from_numpy(g.normal(0, 0.04, size=(V, d)).astype(np.float32)).to(torch.bfloat16)
+    y = g.integers(0, V, size=T).astype(np.int32)
+    rows = np.unique(np.concatenate([[0, 255, n - 1], g.integers(0, n, size=40)]))
+    gl = np.zeros(T, np.float32)
+    gl[rows] = g.normal(size=len(rows))
+    dH_ref, dW_ref = ou.lm_head_backward(synth.as_oracle_array(H[rows]), synth.as_oracle_array(W), y[rows], gl[rows].astype(np.float64))
+    Hd, Wd, yd = H.cuda(), W.cuda(), dv(y)
+    Hd[n:] = float("nan")
+    d_T = torch.tensor([n], dtype=torch.int64, device="cuda")
+    logp, lse = torch.empty(T, device="cuda"), torch.empty(T, device="cuda")
+    ws = torch.empty(B.arrol_token_logprob_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+    B.arrol_token_logprob(ctx, Hd, Wd, yd, T, d, V, logp, ws, lse=lse, d_T=d_T)
+    outs = []
+    for _ in range(2):
+        dH, dW = torch.full((T, d), 9.0, device="cuda"), torch.full((V, d), 9.0, device="cuda")
+        ws2 = torch.full((U.arrol_lm_head_backward_workspace(ctx, T, d, V),), 255, dtype=torch.uint8, device="cuda")
+        U.arrol_lm_head_backward(ctx, Hd, Wd, yd, dv(gl), lse, T, d, V, dH, dW, ws2, d_T=d_T)
+        torch.cuda.synchronize()
+        outs.append((dH, dW))
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+    dH, dW = dH.cpu().numpy().astype(np.float64), dW.cpu().numpy().astype(np.float64)
+    for got, ref in ((dH[rows], dH_ref), (dW, dW_ref)):
+        assert np.abs(got - ref).max() <= 1e-2 * np.abs(ref).max()
+        assert np.linalg.norm(got - ref) <= 5e-3 * np.linalg.norm(ref)
+    assert np.all(np.delete(dH, rows, axis=0) == 0.0)
+
+
 def test_lm_head_backward_with_a_dead_chunk_after_a_live_one(ctx):
     _backward_case(ctx, 9700, 72, 300, seed=6, T_live=300)
 
