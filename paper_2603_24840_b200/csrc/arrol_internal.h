@@ -24,6 +24,7 @@ struct arrol_ctx {
     bool head_dw1_smem_set[2]; // likewise for the head training step's contraction (column tiles of 64, 128)
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
+    bool prune_smem_set;       // likewise for the fused prune step
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
     uint32_t test_spin_limit;  // arrol_test_hook: tries per pipeline wait of the log-prob kernel, 0 = the normal limit

@@ -50,6 +50,7 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
     ctx->logprob_smem_set = false;
     ctx->calib_smem_set = false;
     ctx->backward_smem_set = false;
+    ctx->prune_smem_set = false;
     for (int& n : ctx->backward_max_pairs) n = 0;
     ctx->score_tc_smem_set = false;
     ctx->gather_bulk_smem_set = false;

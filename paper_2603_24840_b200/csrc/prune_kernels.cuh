@@ -66,17 +66,33 @@ __device__ __forceinline__ void linear_row_begin(const T* __restrict__ x, int nv
         if (c < nvec) xr[u] = Vec16<T>::load_raw(x + (int64_t)c * Vec16<T>::N);
     }
 }
+// rest_s: the vectors past the first 256 in shared memory, copied there by the lanes that read them (linear_row_rest), or NULL.
+constexpr int ROW_BEGIN_VECS = 256;
+template <typename T>
+__device__ __forceinline__ void linear_row_rest(const T* __restrict__ x, int nvec, int lane, typename Vec16<T>::Raw* rest_s) {
+    for (int c = ROW_BEGIN_VECS + lane; c < nvec; c += 32)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(rest_s + c - ROW_BEGIN_VECS)),
+                     "l"(x + (int64_t)c * Vec16<T>::N) : "memory");
+}
 template <typename T>
 __device__ __forceinline__ float linear_row_dot_ws(const T* __restrict__ x, typename Vec16<T>::Raw (&xr)[8],
-                                                   const typename Vec16<T>::Raw* w_s, int nvec, int lane) {
+                                                   const typename Vec16<T>::Raw* w_s, int nvec, int lane,
+                                                   const typename Vec16<T>::Raw* rest_s) {
     constexpr int VN = Vec16<T>::N;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int c0 = lane; c0 < nvec; c0 += 256) {
+    for (int c0 = lane; c0 < nvec; c0 += ROW_BEGIN_VECS) {
         if (c0 != lane) {
+            if (rest_s) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int c = c0 + 32 * u;
-                if (c < nvec) xr[u] = Vec16<T>::load_raw(x + (int64_t)c * VN);
+                for (int u = 0; u < 8; ++u)
+                    if (c0 + 32 * u < nvec) xr[u] = rest_s[c0 + 32 * u - ROW_BEGIN_VECS];
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int c = c0 + 32 * u;
+                    if (c < nvec) xr[u] = Vec16<T>::load_raw(x + (int64_t)c * VN);
+                }
             }
         }
 #pragma unroll
@@ -103,8 +119,13 @@ __device__ __forceinline__ double shfl_double(double v, int src_lane, int width)
 // segmented shuffle arg-min on (key, index) where of equal keys the higher index wins, then the winner leaves the
 // group and Sigma -= q_winner.  Sigma starts as the index-order sum, built with broadcasts so that every lane of the
 // segment adds the same values in the same order.  All 32 lanes must call this.  Returns whether the lane's rollout
-// is kept.
-__device__ __forceinline__ bool select_lanes(double qj, bool member, int j, int G, int K, double rho, int seg) {
+// is kept.  A chain of G - K rounds, so a round's latency is all that counts: the smallest key by shuffles, then its highest lane by
+// a ballot; SEG, the segment where it is known, leaves no branches between the shuffles.
+template <int SEG>
+__device__ __forceinline__ bool select_lanes_seg(double qj, bool member, int j, int G, int K, double rho, int seg_arg) {
+    const int seg = SEG ? SEG : seg_arg;
+    const int seg0 = (int)(threadIdx.x & 31) & ~(seg - 1);                 // the segment's first lane and its lanes
+    const unsigned int seg_lanes = (0xffffffffu >> (32 - seg)) << seg0;
     bool alive = member;
     double sigma = 0.0;
     for (int i = 0; i < G; ++i) sigma = __dadd_rn(sigma, shfl_double(qj, i, seg));
@@ -112,22 +133,26 @@ __device__ __forceinline__ bool select_lanes(double qj, bool member, int j, int 
         const double tau = __dsub_rn(sigma, __dmul_rn(rho, (double)(n - 1)));
         // non-negative doubles order like their bit patterns, and an integer compare is several times faster than fp64's; lanes
         // that are out take the largest pattern, above a NaN's, so that a member goes whatever the keys are
-        unsigned long long key = alive ? (unsigned long long)__double_as_longlong(fabs(__dsub_rn(qj, tau))) : ~0ull;
-        int idx = alive ? j : -1;
-        // segmented arg-min; ties -> the higher index
+        const unsigned long long mine = alive ? (unsigned long long)__double_as_longlong(fabs(__dsub_rn(qj, tau))) : ~0ull;
+        unsigned long long key = mine;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = 16; o > 0; o >>= 1)
             if (o < seg) {
-                const unsigned long long okey = __shfl_xor_sync(0xffffffffu, key, o, seg);
-                const int oidx = __shfl_xor_sync(0xffffffffu, idx, o, seg);
-                if (okey < key || (okey == key && oidx > idx)) { key = okey; idx = oidx; }
+                const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o, seg);
+                key = other < key ? other : key;
             }
-        }
+        const unsigned int hits = __ballot_sync(0xffffffffu, alive && mine == key) & seg_lanes;
+        const int idx = hits ? 31 - __clz(hits) - seg0 : -1;               // ties -> the higher index
         const double q_removed = shfl_double(qj, idx < 0 ? 0 : idx, seg);   // idx < 0: no member at all (padding segment)
         if (idx == j) alive = false;
         sigma = __dsub_rn(sigma, q_removed);
     }
     return alive;
+}
+__device__ __forceinline__ bool select_lanes(double qj, bool member, int j, int G, int K, double rho, int seg) {
+    if (seg == 16) return select_lanes_seg<16>(qj, member, j, G, K, rho, seg);
+    if (seg == 8) return select_lanes_seg<8>(qj, member, j, G, K, rho, seg);
+    return select_lanes_seg<0>(qj, member, j, G, K, rho, seg);
 }
 
 // Statistics of one group over its kept rollouts r in [g0, g1) (Section 3, on the survivors): mean and

@@ -56,6 +56,7 @@ struct FusedParams {
     // {kept tokens, kept rollouts}, each with bit 63 set once published; all zero between calls
     unsigned long long* chain;
     uint32_t spin_limit;
+    int rest_vecs;             // 16-byte vectors of a row past the first 256 that a warp has room for in shared memory: all of them, or 0
 };
 
 constexpr int LUT_STAGED = 1024;
@@ -117,11 +118,15 @@ prune_fused_kernel(const FusedParams p) {
             if (lane == 0) atomicOr(p.d_status, ARROL_DEV_BAD_INDEX);
             nvec = 0;
         }
+        // the whole row is on its way while the block waits for the weights: 4 KB in registers, what is past them by asynchronous
+        // copies (a second round trip to HBM after the first one otherwise)
         Raw xr[8];
-        linear_row_begin<T>(x, nvec, lane, xr);              // the row is on its way while the block waits for the weights
+        Raw* rest_s = p.rest_vecs > 0 ? w_s + p.d / VN + warp * p.rest_vecs : nullptr;
+        linear_row_begin<T>(x, nvec, lane, xr);
+        if (rest_s) linear_row_rest<T>(x, nvec, lane, rest_s);
         __syncthreads();
         if (warp < n_here) {
-            float s = linear_row_dot_ws<T>(x, xr, w_s, nvec, lane);
+            float s = linear_row_dot_ws<T>(x, xr, w_s, nvec, lane, rest_s);
             if (lane == 0) {
                 if (bias_ptr) s += bias;
                 q_s[warp] = probability_map(s, i, p.B, lut_staged ? lut_s : q_lut, p.score, p.prob, p.bin, p.q);
@@ -145,6 +150,19 @@ prune_fused_kernel(const FusedParams p) {
         }
     }
     __syncthreads();
+    // statistics of the block's groups by the second warp, one lane per group, while the first one scans
+    if (warp == 1) {
+        if (lane < groups_here) {
+            auto flag = [&](int r) { return keep_s[r] != 0; };
+            auto rew = [&](int r) { return rew_s[r]; };
+            double mean, den;
+            group_statistics(lane * p.G, lane * p.G + p.G, p.ddof, p.eps, inv_count, flag, rew, mean, den);
+            g_mean[lane] = mean;
+            g_den[lane] = den;
+        }
+        __threadfence_block();
+        asm volatile("bar.arrive 1, 64;" ::: "memory");
+    }
     if (warp != 0) return;
 
     // ---- first warp: scan of the block's rollouts, chained over the blocks, outputs of the block's groups ----
@@ -170,15 +188,6 @@ prune_fused_kernel(const FusedParams p) {
         totals[2 * blockIdx.x] = PUBLISHED | (unsigned long long)block_t;
         totals[2 * blockIdx.x + 1] = PUBLISHED | (unsigned long long)block_c;
     }
-    // statistics of the block's groups, one lane per group, while the other blocks publish
-    if (lane < groups_here) {
-        auto flag = [&](int r) { return keep_s[r] != 0; };
-        auto rew = [&](int r) { return rew_s[r]; };
-        double mean, den;
-        group_statistics(lane * p.G, lane * p.G + p.G, p.ddof, p.eps, inv_count, flag, rew, mean, den);
-        g_mean[lane] = mean;
-        g_den[lane] = den;
-    }
     // totals of the blocks before this one (each lane takes every 32nd of them)
     int64_t base_t = 0;
     int32_t base_c = 0;
@@ -200,9 +209,19 @@ prune_fused_kernel(const FusedParams p) {
         base_t += __shfl_xor_sync(0xffffffffu, base_t, o);
         base_c += __shfl_xor_sync(0xffffffffu, base_c, o);
     }
-    __syncwarp();
+    // this block has read what it needed: it says so before it writes, so that the arrival does not wait for the stores
+    const bool any_bad = __any_sync(0xffffffffu, bad_index);
+    const bool any_expired = __any_sync(0xffffffffu, expired);
+    unsigned long long done = 0;
+    if (lane == 0) {
+        if (any_expired) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
+        if (any_bad) atomicOr(reinterpret_cast<unsigned int*>(p.chain + 1), 1u);
+        __threadfence();
+        done = atomicAdd(p.chain, 1ull);
+    }
+    asm volatile("bar.sync 1, 64;" ::: "memory");            // the groups' statistics
     if (kept) {
-        const int32_t pos = base_c + (c - own_c);
+        const int pos = base_c + (c - own_c);
         p.survivor_idx[pos] = first + lane;
         p.cu_seqlens[pos + 1] = base_t + t;
         const int g = lane / p.G;
@@ -213,15 +232,6 @@ prune_fused_kernel(const FusedParams p) {
         p.d_num[0] = base_c + block_c;
         p.d_num[1] = base_t + block_t;
         if (base_t + block_t > p.capacity) atomicOr(p.d_status, ARROL_DEV_CAPACITY);
-    }
-    const bool any_bad = __any_sync(0xffffffffu, bad_index);
-    const bool any_expired = __any_sync(0xffffffffu, expired);
-    unsigned long long done = 0;
-    if (lane == 0) {
-        if (any_expired) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
-        if (any_bad) atomicOr(reinterpret_cast<unsigned int*>(p.chain + 1), 1u);
-        __threadfence();
-        done = atomicAdd(p.chain, 1ull);
     }
     // the block that finishes last has seen every block read what it needed: clear the chain for the next call
     if (__shfl_sync(0xffffffffu, done, 0) == gridDim.x - 1) {
@@ -274,6 +284,11 @@ extern "C" int arrol_prune_step(arrol_ctx* ctx, const arrol_prune_step_args* a, 
     }
     const int64_t fused_blocks = ((int64_t)a->P + gpb - 1) / gpb;
     const size_t w_bytes = linear ? (size_t)a->head.d * (a->head.dtype == ARROL_F32 ? 4 : 2) : 0;
+    // what is past the first 4 KB of a block's rows is staged too while the blocks of an SM have room for it side by side
+    const size_t first_bytes = (size_t)ROW_BEGIN_VECS * 16;
+    size_t rest_bytes = w_bytes > first_bytes ? (w_bytes - first_bytes) * (size_t)(threads / 32) : 0;
+    if (rest_bytes + w_bytes > (fused_blocks > ctx->sm_count ? (size_t)96 : (size_t)200) * 1024) rest_bytes = 0;
+    const size_t smem = w_bytes + rest_bytes;
     // blocks of the chained scan, which wait for lower-numbered ones: at most two per SM
     const int per_sm = 2048 / threads < 1 ? 1 : 2048 / threads;
     if (fused_blocks > (int64_t)ctx->sm_count * (per_sm > 2 ? 2 : per_sm) || fused_blocks > ARROL_CHAIN_BLOCKS ||
@@ -317,14 +332,20 @@ extern "C" int arrol_prune_step(arrol_ctx* ctx, const arrol_prune_step_args* a, 
     p.d_status = ctx->d_status;
     p.chain = ctx->d_chain;
     p.spin_limit = ctx->test_spin_limit ? ctx->test_spin_limit : (1u << 22);
+    p.rest_vecs = (int)(rest_bytes / 16 / (size_t)(threads / 32));
+    if (smem > 40 * 1024 && !ctx->prune_smem_set) {
+        ARROL_CUDA_OK(cudaFuncSetAttribute(prune_fused_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(prune_fused_kernel<__nv_bfloat16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+        ctx->prune_smem_set = true;
+    }
     const dim3 grid((unsigned)fused_blocks), block((unsigned)threads);
     cudaStream_t s = (cudaStream_t)stream;
     if (!linear)
         ARROL_CUDA_OK(arrol_launch_pdl(prune_fused_kernel<float, false>, grid, block, 0, s, p));
     else if (a->head.dtype == ARROL_F32)
-        ARROL_CUDA_OK(arrol_launch_pdl(prune_fused_kernel<float, true>, grid, block, w_bytes, s, p));
+        ARROL_CUDA_OK(arrol_launch_pdl(prune_fused_kernel<float, true>, grid, block, smem, s, p));
     else
-        ARROL_CUDA_OK(arrol_launch_pdl(prune_fused_kernel<__nv_bfloat16, true>, grid, block, w_bytes, s, p));
+        ARROL_CUDA_OK(arrol_launch_pdl(prune_fused_kernel<__nv_bfloat16, true>, grid, block, smem, s, p));
     ctx->launches += 1;
     return arrol_internal_compact(ctx, a->keep, a->lengths, a->src_tok_off, N, a->G, a->src_tokens, a->src_rows,
                                   a->row_bytes, a->rewards, a->eps, a->ddof, a->dst_capacity_tokens, a->dst_tokens,

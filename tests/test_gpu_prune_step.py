@@ -147,3 +147,25 @@ def test_fused_prune_step_over_group_shapes(P, G, K):
             assert torch.equal(getattr(pr, k)[:T], want[k][:T]), k
     assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == 0
     pr.ctx.close()
+
+
+# rows past the 4 KB that a warp holds in registers: one vector more (2,056 bf16, 1,032 fp32), twice as many, a block of few warps, and
+# rows too long to be staged for a block of 32 of them
+@pytest.mark.parametrize("P,G,K,d,dtype", [(9, 16, 8, 2056, "bf16"), (150, 16, 8, 4096, "bf16"), (1, 3, 1, 3000, "bf16"),
+                                           (5, 4, 2, 1032, "f32"), (3, 32, 7, 9000, "f32")])
+def test_fused_prune_step_on_wide_rows(P, G, K, d, dtype):
+    import dataclasses
+    w = dataclasses.replace(synth.WORKLOADS["mini"], P=P, G=G, K=K, h=0, d=d, dtype=dtype, seed=P + d)
+    pr = PruneRebatch(w, inputs=host_inputs(w), with_rows=False)
+    pr.prune_step(with_rows=False)
+    torch.cuda.synchronize()
+    keys = ("score", "prob", "q", "bin", "keep", "d_num")
+    want = {k: getattr(pr, k).clone() for k in keys}
+    for k in keys:
+        getattr(pr, k).fill_(0)
+    B.arrol_prune_step(pr.ctx, pr.prune_step_args(with_rows=False))
+    torch.cuda.synchronize()
+    for k in keys:
+        assert torch.equal(getattr(pr, k), want[k]), k
+    assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == 0
+    pr.ctx.close()
