@@ -95,16 +95,18 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     __shared__ double term[MAX_BINS];           // lambda (rho - q_b)
     __shared__ double weight[MAX_BINS];         // c_b^+ + c_b^-
     __shared__ double point_at[32], point_sum[32], point_slope[32];
-    __shared__ double round_lo, round_hi, round_at;
-    __shared__ int round_kind;                  // 0 = done, 1 = tree, 2 = around the linear estimate
+    __shared__ double round_lo, round_hi, round_at, round_unit;
+    __shared__ int round_kind;
+    enum { DONE, EVEN, AROUND, ADJACENT, TREE };        // of a round's points, see below
     extern __shared__ double products[];        // [31][B rounded up to odd]: c_b p_b of a round's points
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
-    auto code_of = [&](int64_t i) {
-        if (mask && !mask[i]) return -1;
+    auto code_of = [&](int64_t i) {             // the three loads do not wait for one another
+        const bool on = !mask || mask[i];
         int b = bin[i];
+        const bool positive = rewards[i] > 0.5f;
         b = b < 0 ? 0 : (b >= B ? B - 1 : b);
-        return 2 * b + (rewards[i] > 0.5f ? 1 : 0);
+        return on ? 2 * b + (positive ? 1 : 0) : -1;
     };
     auto stage = [&](int64_t from) {
         const int n = (int)min((int64_t)CAL_STAGED, N - from);
@@ -112,19 +114,30 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
         for (int j = tid; j < n; j += CAL_THREADS) staged[j] = (int16_t)code_of(from + j);
         return n;
     };
+    pdl_launch_dependents();
+    pdl_wait();
+    hd = pdl_acquire(hd); bin = pdl_acquire(bin); rewards = pdl_acquire(rewards); mask = pdl_acquire(mask); state = pdl_acquire(state);
+    const int32_t state_B = hd->B;
+    const int64_t state_cap = hd->cap;
+    const int64_t head0[2] = {hd->head_neg, hd->head_pos}, n0[2] = {hd->n_neg, hd->n_pos};
+    const double alpha = hd->alpha;
     if constexpr (ONE_PIECE) stage(0);
     // The byte layout L comes from the call's (B, cap); the state must have been initialised with the same pair.
     // A mismatched or uninitialised state is left untouched and reported (uniform over the block: no barrier yet).
-    if (hd->B != B || hd->cap != cap) {
+    if (state_B != B || state_cap != cap) {
         if (tid == 0) atomicOr(d_status, ARROL_DEV_BAD_STATE);
         return;
     }
     int64_t* cnt[2] = {reinterpret_cast<int64_t*>(state + L.cneg), reinterpret_cast<int64_t*>(state + L.cpos)};
     int16_t* ring[2] = {reinterpret_cast<int16_t*>(state + L.ring_neg), reinterpret_cast<int16_t*>(state + L.ring_pos)};
     float* lut = reinterpret_cast<float*>(state + L.q_lut);
-    const int64_t head0[2] = {hd->head_neg, hd->head_pos}, n0[2] = {hd->n_neg, hd->n_pos};
-    const double alpha = hd->alpha;
     int64_t old_cnt[2] = {0, 0};                // B <= MAX_BINS = CAL_THREADS: thread b owns bin b
+    int16_t oldest[2];                          // this thread's first candidates for eviction, requested before it is known how many go
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        const int64_t at = head0[l] + tid;      // head0 < cap
+        oldest[l] = tid < n0[l] ? ring[l][at < cap ? at : at - cap] : (int16_t)0;
+    }
     if (tid < B) { old_cnt[0] = cnt[0][tid]; old_cnt[1] = cnt[1][tid]; hist[0][tid] = 0; hist[1][tid] = 0; }
     __syncthreads();
 
@@ -164,7 +177,8 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
         int32_t mine[2] = {0, 0};
         for (int j = j0; j < j1; ++j) {
             const int c = staged[j];
-            if (c >= 0) mine[c & 1] += 1;
+            mine[0] += c >= 0 && (c & 1) == 0 ? 1 : 0;
+            mine[1] += c >= 0 && (c & 1) != 0 ? 1 : 0;
         }
         block_scan(mine, first_rank, total);
     };
@@ -190,14 +204,16 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
         const int64_t evict = over <= 0 ? 0 : (over < n0[l] ? over : n0[l]);
         for (int64_t j = tid; j < evict; j += CAL_THREADS) {
             const int64_t at = head0[l] + j;     // head0, j < cap
-            atomicSub(&hist[l][ring[l][at < cap ? at : at - cap]], 1);
+            atomicSub(&hist[l][j == tid ? oldest[l] : ring[l][at < cap ? at : at - cap]], 1);
         }
     }
     __syncthreads();
 
     // entry r of m lands in slot (head + n + r) mod cap, and only the last `cap` of them survive the call
     {
-        const int64_t slot0[2] = {(head0[0] + n0[0]) % cap, (head0[1] + n0[1]) % cap};
+        int64_t slot0[2] = {head0[0] + n0[0], head0[1] + n0[1]};         // below 2 cap
+#pragma unroll
+        for (int l = 0; l < 2; ++l) slot0[l] -= slot0[l] >= cap ? cap : 0;
         auto write_run = [&](const int64_t (&before)[2]) {
             int64_t r[2] = {before[0] + first_rank[0], before[1] + first_rank[1]};
             for (int j = j0; j < j1; ++j) {
@@ -205,9 +221,9 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
                 if (c < 0) continue;
                 const int l = c & 1;
                 const int64_t rank = l ? r[1]++ : r[0]++;
-                if (rank >= total_new[l] - cap) {
-                    const int64_t at = slot0[l] + (rank < cap ? rank : rank % cap);
-                    ring[l][at < cap ? at : at - cap] = (int16_t)(c >> 1);
+                if (rank >= (l ? total_new[1] : total_new[0]) - cap) {
+                    const int64_t at = (l ? slot0[1] : slot0[0]) + (rank < cap ? rank : rank % cap);
+                    (l ? ring[1] : ring[0])[at < cap ? at : at - cap] = (int16_t)(c >> 1);
                     atomicAdd(&hist[l][c >> 1], 1);
                 }
             }
@@ -234,7 +250,7 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     for (int l = 0; l < 2; ++l) {
         const int64_t over = n0[l] + total_new[l] - cap;
         n1[l] = over > 0 ? cap : n0[l] + total_new[l];
-        if (tid == l) {
+        if (tid == CAL_THREADS - 1 - l) {        // a warp without a bin to work on, most often
             const int64_t h1 = over > 0 ? (head0[l] + over) % cap : head0[l];
             if (l == 0) { hd->head_neg = h1; hd->n_neg = n1[l]; } else { hd->head_pos = h1; hd->n_pos = n1[l]; }
         }
@@ -264,12 +280,16 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     // delta: 64 bisection steps on E[p](delta) = kappa.  The value that decides a step is the expected keep rate summed over
     // the bins in index order, one rounding per operation (so that delta agrees bit for bit with a plain loop).
     //   Rounded addition, multiplication, clamping and division are all monotone, so the decision "below" is a monotone
-    // function of the midpoint, bit for bit: one evaluation at x settles every midpoint on its side of x.  So the block
-    // evaluates 31 points a round (one warp each) and the first warp replays the bisection as far as the settled points
-    // reach.  Rounds 0 and 1 take the 31 midpoints of the next five levels; round 2 takes points at growing distances around
-    // the root of the linear piece that E is on by then, which settles most of the remaining levels; then five levels a
-    // round again until the bracket stops shrinking.  Every round of midpoints settles one step at least (its first point is
-    // the next midpoint), so 65 rounds are always enough, and no more are made.
+    // function of the midpoint x, bit for bit, and one of kappa + x (rounded), through which alone x enters: one evaluation at x
+    // settles every midpoint whose kappa + x lies on its side.  So the block evaluates 31 points a round (one warp each, in
+    // ascending order), whatever they are, and at the end the first warp replays the bisection against the two settled points next to
+    // the threshold.  E is piecewise linear, and its root needs few rounds:
+    //   EVEN      points evenly over the bracket: after it the piece that the root lies on is known
+    //   AROUND    points at growing distances around the root of that piece, with the sum as a butterfly gives it
+    //   ADJACENT  neighbouring values of kappa + x around the root that the sum in index order at the best point gives
+    // and, where that does not settle all (breakpoints next to the root, or no slope), the 31 midpoints of the replay's next five levels
+    // (TREE) until it does: a round of those settles a step at least, so 64 of them are always enough.
+    // (Before, midpoints only, but for one round around the linear root: six rounds where three do now, with two replays between.)
     //   One evaluation: the lanes form the per-bin products c_b p_b (all >= 0) and a butterfly sum S of them; the in-order sum
     // differs from S by at most (B + 8) 2^-53 S (both are within their standard error bounds of the exact sum), so when S is
     // further from kappa n than four times that bound plus the roundings of the division and of kappa n, S < kappa n already
@@ -280,6 +300,7 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     if (n > 0.0) {                                   // uniform for the block
         const double u = 1.1102230246251565e-16;     // 2^-53
         const double goal = kappa * n;
+        const double inf = __longlong_as_double(0x7ff0000000000000ll);
         const int pitch = product_pitch(B);
         auto midpoint = [](double a, double b) { return __dmul_rn(0.5, __dadd_rn(a, b)); };
         auto clipped = [&](double p) {
@@ -287,46 +308,68 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
             if (p > p_max) p = p_max;
             return p;
         };
-        double lo = -(1.0 + lambda), hi = 1.0 + lambda;           // the first warp's
-        double known_below = lo - 1.0, known_above = hi + 1.0;    // settled points next to the threshold
-        double sum_at = 0.0, slope_at = 0.0;                      // S and dS/d(delta) at known_below
+        // the first warp's: the bracket of the replay, the settled points next to the threshold, S and dS/d(delta) at the lower one
+        double lo = -(1.0 + lambda), hi = 1.0 + lambda;
+        const double first_lo = lo, first_hi = hi;
+        double known_below = -inf, known_above = inf;
+        double sum_at = 0.0, slope_at = 0.0;
+        bool sum_in_order = false;
         // infinite lambda: the first midpoint is NaN, no comparison holds, and a plain loop ends at NaN.  (A finite bracket
         // never gets there: its midpoints can overflow, but not with opposite signs.)
         int step = isinf(lambda) ? 64 : 0;
         if (step) hi = midpoint(lo, hi);
-        for (int round = 0; round <= 65; ++round) {
+        for (int round = 0; round <= 3 + 64; ++round) {
             if (wid == 0) {
-                for (; step < 64; ++step) {
-                    const double m = midpoint(lo, hi);
-                    if (m <= known_below) { if (m == lo) step = 64; lo = m; }        // an unchanged bracket stays unchanged
-                    else if (m >= known_above) { if (m == hi) step = 64; hi = m; }
-                    else break;
+                int kind = TREE;
+                double a = fmax(known_below, first_lo), b = fmin(known_above, first_hi), at = 0.0, unit = 0.0;
+                if (step >= 64) {
+                    kind = DONE;
+                } else if (round < 3) {
+                    kind = EVEN;
+                    if (round > 0 && known_below > -inf && slope_at > 0.0) {
+                        at = fmin(fmax(known_below + (goal - sum_at) / slope_at, a), b);
+                        kind = round == 2 && sum_in_order ? ADJACENT : AROUND;
+                        unit = kind == AROUND ? 1.0 + lambda : scalbn(1.0, ilogb(fmax(fmax(fabs(kappa + at), fabs(at)), 1e-200)) - 52);
+                    }
+                } else {                             // replay as far as the settled points reach
+                    const double base_below = __dadd_rn(kappa, known_below), base_above = __dadd_rn(kappa, known_above);
+                    double m = midpoint(lo, hi);
+                    for (; step < 64; ++step) {
+                        const double base = __dadd_rn(kappa, m), m_up = midpoint(m, hi), m_down = midpoint(lo, m);    // side by side
+                        if (base <= base_below) { if (m == lo) step = 64; lo = m; m = m_up; }      // an unchanged bracket stays unchanged
+                        else if (base >= base_above) { if (m == hi) step = 64; hi = m; m = m_down; }
+                        else break;
+                    }
+                    if (step >= 64) kind = DONE;
+                    a = lo;
+                    b = hi;
                 }
-                if (lane == 0) {
-                    const bool linear = round == 2 && slope_at > 0.0;
-                    round_kind = step >= 64 ? 0 : (linear ? 2 : 1);
-                    round_lo = lo; round_hi = hi;
-                    round_at = linear ? fmin(fmax(known_below + (goal - sum_at) / slope_at, lo), hi) : 0.0;
-                }
+                if (lane == 0) { round_kind = kind; round_lo = a; round_hi = b; round_at = at; round_unit = unit; }
             }
             __syncthreads();
             const int kind = round_kind;
-            if (kind == 0) break;
-            // this warp's point
+            if (kind == DONE) break;
+            // this warp's point, in ascending order
             double x = 0.0;
-            if (kind == 1) {                         // node of the binary tree of midpoints, 1 = the next one; children 2k, 2k + 1
+            const int i = wid - 15;                  // -15 .. 15
+            if (kind == EVEN) {
+                const double t = (double)(wid + 1) * 0.03125;
+                x = (1.0 - t) * round_lo + t * round_hi;
+            } else if (kind == AROUND) {             // 2^-51 ... 2^-44 away, then coarser
+                const int k = i < 0 ? -i : i;
+                const int e = k <= 8 ? k - 52 : (k == 9 ? -42 : k == 10 ? -39 : k == 11 ? -36 : k == 12 ? -32 : k == 13 ? -26 : k == 14 ? -18 : -10);
+                const double off = k == 0 ? 0.0 : scalbn(round_unit, e);
+                x = i < 0 ? round_at - off : round_at + off;
+            } else if (kind == ADJACENT) {
+                x = round_at + (double)i * round_unit;
+            } else {                                 // in-order traversal of the tree of the next five levels' midpoints
                 double a = round_lo, b = round_hi;
-                const int node = wid < CAL_POINTS ? wid + 1 : 1;
-                for (int bit = 30 - __clz(node); bit >= 0; --bit) {
-                    const double m = midpoint(a, b);
-                    if ((node >> bit) & 1) a = m; else b = m;
-                }
+                const int want = wid < CAL_POINTS ? wid + 1 : 1;
                 x = midpoint(a, b);
-            } else {
-                const int i = wid < 15 ? 15 - wid : wid - 15;       // 0 .. 15 steps away: 2^-51 ... 2^-44, then coarser
-                const int e = i <= 8 ? i - 52 : (i == 9 ? -42 : i == 10 ? -39 : i == 11 ? -36 : i == 12 ? -32 : i == 13 ? -26 : i == 14 ? -18 : -10);
-                const double off = i == 0 ? 0.0 : scalbn(1.0 + lambda, e);
-                x = wid < 15 ? round_at - off : round_at + off;
+                for (int node = 16, half = 8; node != want; half >>= 1) {
+                    if (want > node) { a = x; node += half; } else { b = x; node -= half; }
+                    x = midpoint(a, b);
+                }
             }
             if (wid < CAL_POINTS) {
                 const double base = __dadd_rn(kappa, x);
@@ -350,35 +393,34 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
             if (wid == 0) {
                 const bool has = lane < CAL_POINTS;
                 const double S = has ? point_sum[lane] : 0.0;
-                const double at = has ? point_at[lane] : 0.0;
                 const double slack = 4.0 * ((double)(B + 8) * u * S + 3.0 * u * (S + goal));
                 const bool near = has && fabs(S - goal) <= slack;
                 bool below = S < goal;
+                double e = S;
                 if (__any_sync(0xffffffffu, near)) {
-                    double e = 0.0;
+                    e = 0.0;
                     if (B <= CAL_PRODUCT_BINS) {
                         const double* row = products + (has ? lane : 0) * pitch;
 #pragma unroll 8
                         for (int k = 0; k < B; ++k) e = __dadd_rn(e, row[k]);
                     } else {
-                        const double base = __dadd_rn(kappa, at);
+                        const double base = __dadd_rn(kappa, has ? point_at[lane] : 0.0);
 #pragma unroll 4
                         for (int k = 0; k < B; ++k) e = __dadd_rn(e, __dmul_rn(weight[k], clipped(__dadd_rn(base, term[k]))));
                     }
                     if (near) below = __ddiv_rn(e, n) < kappa;
+                    if (has) point_sum[lane] = e;
+                    __syncwarp();
                 }
-                // settled points next to the threshold, over the warp
-                double best_below = has && below ? at : known_below, best_above = has && !below ? at : known_above;
-                double s_at = has && below ? S : sum_at, d_at = has && below ? point_slope[lane] : slope_at;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const double ob = __shfl_xor_sync(0xffffffffu, best_below, o), os = __shfl_xor_sync(0xffffffffu, s_at, o);
-                    const double od = __shfl_xor_sync(0xffffffffu, d_at, o), oa = __shfl_xor_sync(0xffffffffu, best_above, o);
-                    if (ob > best_below) { best_below = ob; s_at = os; d_at = od; }
-                    best_above = fmin(best_above, oa);
+                // ascending points: the ones below come first
+                const int count = __popc(__ballot_sync(0xffffffffu, has && below));
+                if (count > 0 && point_at[count - 1] > known_below) {
+                    known_below = point_at[count - 1];
+                    sum_at = point_sum[count - 1];
+                    slope_at = point_slope[count - 1];
+                    sum_in_order = __any_sync(0xffffffffu, near);
                 }
-                if (best_below > known_below) { known_below = best_below; sum_at = s_at; slope_at = d_at; }
-                known_above = fmin(known_above, best_above);
+                if (count < CAL_POINTS) known_above = fmin(known_above, point_at[count]);
             }
         }
         delta = midpoint(lo, hi);                    // meaningful in the first warp
@@ -391,6 +433,9 @@ __global__ void select_stochastic_kernel(const float* __restrict__ q, const floa
                                          const double* __restrict__ d_delta, double delta_value, double lambda,
                                          double rho, double p_min, double p_max, uint8_t* __restrict__ keep,
                                          float* __restrict__ p_out) {
+    pdl_launch_dependents();
+    pdl_wait();
+    q = pdl_acquire(q); u = pdl_acquire(u); eligible = pdl_acquire(eligible); d_delta = pdl_acquire(d_delta);
     const double delta = d_delta ? *d_delta : delta_value;
     const double base = __dadd_rn(kappa, delta);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -467,11 +512,10 @@ extern "C" int arrol_calib_update(arrol_ctx* ctx, void* state, int32_t B, int64_
         ctx->calib_smem_set = true;
     }
     const size_t smem = B <= CAL_PRODUCT_BINS ? sizeof(double) * CAL_POINTS * product_pitch(B) : 0;
-    (N <= CAL_STAGED ? one_piece : pieces)<<<1, CAL_THREADS, smem, (cudaStream_t)stream>>>(
-        static_cast<uint8_t*>(state), layout_of(B, cap), bin, rewards, mask, N, sp->kappa, sp->lambda, sp->rho, sp->p_min, sp->p_max,
-        B, cap, ctx->d_status);
+    ARROL_CUDA_OK(arrol_launch_pdl(N <= CAL_STAGED ? one_piece : pieces, dim3(1), dim3(CAL_THREADS), smem, (cudaStream_t)stream,
+                                   static_cast<uint8_t*>(state), layout_of(B, cap), bin, rewards, mask, N, sp->kappa, sp->lambda,
+                                   sp->rho, sp->p_min, sp->p_max, B, cap, ctx->d_status));
     ctx->launches += 1;
-    ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;
 }
 
@@ -485,9 +529,8 @@ extern "C" int arrol_select_stochastic(arrol_ctx* ctx, const float* q, const flo
     if (!guard.ok) return ARROL_ERR_CUDA;
     int64_t blocks = (N + 255) / 256;
     if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
-    select_stochastic_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(
-        q, u, eligible, N, sp->kappa, d_delta, delta, sp->lambda, sp->rho, sp->p_min, sp->p_max, keep, p_out);
+    ARROL_CUDA_OK(arrol_launch_pdl(select_stochastic_kernel, dim3((unsigned)blocks), dim3(256), 0, (cudaStream_t)stream, q, u, eligible,
+                                   N, sp->kappa, d_delta, delta, sp->lambda, sp->rho, sp->p_min, sp->p_max, keep, p_out));
     ctx->launches += 1;
-    ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;
 }
