@@ -29,17 +29,17 @@ namespace {
 
 constexpr int BM = 128, BN = CHUNK_COLUMNS;   // rows of a block, columns of a tile
 constexpr int TILE_ROWS = 2 * BM;        // rows of a pair's tile
-constexpr int STAGES = 6;
 constexpr int A_STAGE_BYTES = BM * BK * 2;
 constexpr int B_STAGE_BYTES = BN / 2 * BK * 2;
 constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
 constexpr int MN_BLOCK_BYTES = BK * 128;   // one 64-element MN block of an MN-major stage: BK rows of 128 bytes
 constexpr int TMEM_COLS = 512;
+constexpr int STAGES = 6;
 constexpr int EPI_WARPS = 8;            // two warps per tensor-memory lane quarter, each takes half of the columns
 constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 constexpr int EPI_PIECES = BN / 32 / (EPI_WARPS / 4);   // 32-column pieces per epilogue warp and accumulator
-// every kernel: one 32-row x 128-byte staging tile per epilogue warp behind the barrier block (1 KB), 1024-byte
-// aligned, from which the results leave as TMA tile stores / reductions
+// one 32-row x 128-byte staging tile per epilogue warp behind the barrier block (1 KB), 1024-byte aligned: results go through it to
+// leave in whole 128-byte lines
 constexpr int EPI_STAGE_TILE = 32 * 128;
 constexpr size_t EPI_STAGE_OFFSET = (size_t)STAGES * STAGE_BYTES + 1024;
 constexpr size_t SMEM_BYTES = EPI_STAGE_OFFSET + (size_t)EPI_WARPS * EPI_STAGE_TILE + 1024;
@@ -330,52 +330,36 @@ struct DzParams {
     float scale2, inv_temp;
     const uint16_t* hidden;
     unsigned int* lock_words;
+    uint16_t* dz;             // [TC, ldz]
+    int64_t ldz;
     uint16_t* tail;           // [63, d]: the last, partly live 64-row block of the chunk's hidden rows, zero-padded
     uint32_t* d_status;
 };
 
-// The last items, which would keep at most half of the pairs busy for one more wave, go as two halves of their columns each:
-// the last wave then takes about 0.6 of a whole one (an operand of the rows for half the MMAs).
-struct DzWork { int m_tiles, total_chunks, group_tiles; int64_t body, items; };
-__device__ __forceinline__ DzWork make_dz_work(int m_tiles, int total_chunks, int group_tiles, int64_t units) {
-    DzWork w;
-    w.m_tiles = m_tiles;
-    w.total_chunks = total_chunks;
-    w.group_tiles = group_tiles;
-    const int64_t tiles = (int64_t)m_tiles * total_chunks, tail = tiles % units;
-    const bool halves = 2 * tail <= units;
-    w.body = halves ? tiles - tail : tiles;
-    w.items = halves ? tiles + tail : tiles;
-    return w;
-}
-// (m, c): token tile and vocabulary chunk; half: 0 or 1, -1 for the whole chunk
-__device__ __forceinline__ bool dz_item(const DzWork& w, int64_t i, int& m, int& c, int& half) {
-    const int m_tiles = w.m_tiles, total_chunks = w.total_chunks, group_tiles = w.group_tiles;
-    if (i >= w.items) return false;
-    half = -1;
-    if (i >= w.body) {
-        half = (int)((i - w.body) & 1);
-        i = w.body + ((i - w.body) >> 1);
-    }
+__device__ __forceinline__ bool dz_item(int64_t i, int m_tiles, int total_chunks, int group_tiles, int& m, int& c) {
     const int64_t per_group = (int64_t)group_tiles * total_chunks;
     const int64_t g = i / per_group;
     const int first = (int)g * group_tiles;
+    if (first >= m_tiles) return false;
     const int size = min(group_tiles, m_tiles - first);
     i -= g * per_group;
+    if (i >= (int64_t)size * total_chunks) return false;
     c = (int)(i / size);
     m = first + (int)(i - (int64_t)c * size);
     return true;
 }
-// first column of an item and how many the MMA computes (32 at least: a half that lies past V is zeros, which nobody stores)
-__device__ __forceinline__ int dz_column(int c, int half) { return c * BN + (half > 0 ? BN / 2 : 0); }
-__device__ __forceinline__ int dz_columns(int V, int c, int half) {
-    const int left = (max(V - dz_column(c, half), 1) + 31) & ~31;
-    return min(left, half >= 0 ? BN / 2 : BN);
-}
 
+// What bounds it: the MMAs (8 d cycles of an SM per tile) from d of about 400 on.  Below that the epilogue: 32,768 exponentials a tile and
+// SM take the special-function units 2,048 cycles, and what a warp does for its 32 x 128 share takes it about 3,800.  It took 5,500 to
+// 8,000 while results left by TMA tile stores, which queue behind the operand copies in flight, from a staging tile that had to be free
+// again; while the accumulator was handed back by a release, which waited for those stores; and while the row's target and gradient
+// were fetched when the tile had already arrived.  Now whole lines are read back from the staging tile and stored directly, rows are
+// requested a tile ahead, and an element costs 3 to 4 instructions: two at a time in packed fp32, the target column, which few
+// pieces hold, by a loop of its own.  (Sixteen warps with less staging each: no gain with tile stores, 10 % slower with direct ones.)
+// 700 tokens, d = 320, V = 151,936: whole update 358 -> 303 us, with the dH kernel's epilogue in the same manner; 12,000, d = 512,
+// V = 30,000 1,025 -> 970; 12,000, d = 2,048, V = 60,000 6,430 -> 6,250.
 __global__ void __launch_bounds__(NUM_THREADS, 1)
-dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w,
-          const __grid_constant__ CUtensorMap map_dz, const DzParams p) {
+dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUtensorMap map_w, const DzParams p) {
     extern __shared__ uint8_t smem_raw[];
     const PipeSmem ps = pipe_setup(smem_raw, &map_h, &map_w);
     uint8_t* dz_stage = ps.stage_a + EPI_STAGE_OFFSET;
@@ -387,20 +371,19 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
     const int k_last = (p.d - (k_steps - 1) * BK + UMMA_K - 1) / UMMA_K;
     const int total_chunks = (p.V + BN - 1) / BN;
     const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
-    const DzWork work = make_dz_work(m_tiles, total_chunks, p.group_tiles, units);
     auto coords = [&](int64_t it, TileAt& t) {
-        int m, c, half;
-        if (!dz_item(work, unit + it * units, m, c, half)) return false;
+        int m, c;
+        if (!dz_item(unit + it * units, m_tiles, total_chunks, p.group_tiles, m, c)) return false;
         t.a0 = (int)p.t0 + m * TILE_ROWS;
-        t.b0 = dz_column(c, half);
-        t.n = dz_columns(p.V, c, half);
+        t.b0 = c * BN;
+        t.n = chunk_columns(p.V, c);
         t.k0 = 0;
         t.k1 = k_steps;
         return true;
     };
 
     if (warp == 0) {
-        const Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, work.body, k_steps, work.items - work.body, k_steps);
+        const Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, (int64_t)m_tiles * total_chunks, k_steps, 0, 0);
         producer_loop<false, false>(ps, &map_h, &map_w, lock, coords);
     } else if (warp == 1) {
         if (ps.rank == 0) mma_loop<false, false>(ps, k_steps, k_last, coords);
@@ -422,50 +405,66 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
         const float* grad_logp = pdl_acquire(p.grad_logp);
         const float* lse = pdl_acquire(p.lse);
         const int quarter = warp & 3;
-        const int col_half = (warp - 2) >> 2;           // 0 or 1: which half of the accumulator's columns
+        const int col_half = (warp - 2) >> 2;           // which half of the accumulator's columns
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         // dz leaves through shared memory: the warp's 32 rows x 64 columns (two pieces, 128 bytes per row, 128-byte
-        // swizzle) are staged and written by one TMA tile store, i.e. in whole 128-byte lines; columns past V are
-        // clipped by the copy.  (16-byte stores straight from the registers touch 32 lines per instruction and
-        // cost the kernel 14 %.)
+        // swizzle) are staged and written in whole 128-byte lines.  (16-byte stores straight from the registers touch 32 lines per
+        // instruction and cost the kernel 14 %.)  Columns past V go as far as the row's padding, which nobody reads.
         uint8_t* stg = dz_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        int m, c, half;
-        for (int64_t item = unit; ok && dz_item(work, item, m, c, half); item += units) {
-            const int first_col = dz_column(c, half);
-            const int row0 = m * TILE_ROWS + (int)ps.rank * BM + quarter * 32;
-            const int64_t t = p.t0 + row0 + lane;
-            int y = -1;
-            float coef = 0.f, lse2 = 0.f;
+        int m, c, m_next = 0, c_next = 0;
+        // the row's target, gradient and log-sum-exp, requested a tile ahead
+        int y_raw = -1;
+        float grad_raw = 0.f, lse_raw = 0.f;
+        auto request_row = [&](int tile) {
+            const int64_t t = p.t0 + tile * TILE_ROWS + (int)ps.rank * BM + quarter * 32 + lane;
+            y_raw = -1;
             if (t < T) {
-                y = targets[t];
-                if (y >= 0 && y < p.V) {
-                    coef = grad_logp[t] * p.inv_temp;
-                    lse2 = lse[t] * 1.44269504088896340736f;
-                } else {
-                    y = -1;
-                }
+                y_raw = targets[t];
+                grad_raw = grad_logp[t];
+                lse_raw = lse[t];
             }
+        };
+        int64_t item = unit;
+        bool have = dz_item(item, m_tiles, total_chunks, p.group_tiles, m, c);
+        if (have) request_row(m);
+        while (ok && have) {
+            item += units;
+            const bool have_next = dz_item(item, m_tiles, total_chunks, p.group_tiles, m_next, c_next);
+            const int row0 = m * TILE_ROWS + (int)ps.rank * BM + quarter * 32, first_col = c * BN;
+            const bool valid = y_raw >= 0 && y_raw < p.V;
+            const int y = valid ? y_raw : -1;
+            const float coef = valid ? grad_raw * p.inv_temp : 0.f;
+            const float lse2 = valid ? lse_raw * 1.44269504088896340736f : 0.f;
+            if (have_next) request_row(m_next);
             ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
             ok = __all_sync(0xffffffffu, ok) != 0;
             if (!ok) break;
             tcgen05_fence_after();
-            // Two register buffers: the tensor-memory load of piece i + 1 is in flight while piece i is turned
-            // into dz and staged.
             const uint32_t tacc = ps.tmem_base + lane_addr + acc * BN;
+            const uint32_t live_mask = coef == 0.f ? 0u : ~0u;    // rows that carry no gradient are zeros whatever their logits and lse hold
+            const uint64_t scale_2 = pack_f32x2(p.scale2, p.scale2), lse_2 = pack_f32x2(-lse2, -lse2), coef_2 = pack_f32x2(-coef, -coef);
+            // dz = coef ([v = y] - 2^(z log2e - lse log2e)), two columns at a time
             auto to_dz = [&](const uint32_t (&raw)[32], int piece, uint32_t (&packed)[16]) {
                 const int pc0 = first_col + piece * 32;
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
-                    // dz = coef ([v = y] - 2^(z log2e - lse log2e)); coef = 0 for rows that carry no gradient
-                    float d0 = -coef * ex2_approx(fmaf(__uint_as_float(raw[j]), p.scale2, -lse2));
-                    float d1 = -coef * ex2_approx(fmaf(__uint_as_float(raw[j + 1]), p.scale2, -lse2));
-                    if (pc0 + j == y) d0 += coef;
-                    if (pc0 + j + 1 == y) d1 += coef;
-                    if (coef == 0.f) { d0 = 0.f; d1 = 0.f; }      // also guards 0 * inf from stale lse values
+                    float e0, e1, d0, d1;
+                    unpack_f32x2(fma_f32x2(((uint64_t)raw[j + 1] << 32) | raw[j], scale_2, lse_2), e0, e1);
+                    unpack_f32x2(mul_f32x2(pack_f32x2(ex2_approx(e0), ex2_approx(e1)), coef_2), d0, d1);
                     const __nv_bfloat162 h2 = __floats2bfloat162_rn(d0, d1);
-                    packed[j >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+                    packed[j >> 1] = *reinterpret_cast<const uint32_t*>(&h2) & live_mask;
+                }
+                if (__any_sync(0xffffffffu, (unsigned)(y - pc0) < 32u)) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (pc0 + j == y) {
+                            const float e = fmaf(__uint_as_float(raw[j]), p.scale2, -lse2);
+                            const __nv_bfloat16 h = __float2bfloat16_rn(-coef * ex2_approx(e) + coef);
+                            const uint32_t bits = (uint32_t)*reinterpret_cast<const uint16_t*>(&h) & live_mask;
+                            packed[j >> 1] = (j & 1) ? (packed[j >> 1] & 0xffffu) | (bits << 16) : (packed[j >> 1] & 0xffff0000u) | bits;
+                        }
                 }
             };
             auto stage_piece = [&](const uint32_t (&packed)[16], int piece) {
@@ -475,37 +474,50 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
                     *reinterpret_cast<uint4*>(stg + lane * 128 + (((chunk0 + q4) ^ (lane & 7)) << 4)) =
                         make_uint4(packed[4 * q4], packed[4 * q4 + 1], packed[4 * q4 + 2], packed[4 * q4 + 3]);
             };
+            // Two register buffers: the tensor-memory load of piece i + 1 is in flight while piece i is turned into dz and staged.
+            // The accumulator is handed back as soon as its last piece has been read.
+            static_assert(EPI_PIECES % 2 == 0, "pieces go in pairs");
+            const int p0 = col_half * EPI_PIECES;
             uint32_t ra[32], rb[32];
-            const int pieces = half >= 0 ? EPI_PIECES / 2 : EPI_PIECES;
-            const int p0 = col_half * pieces, p1 = p0 + pieces;           // this warp's pieces of the accumulator
             tcgen05_ld_32x32_issue(tacc + p0 * 32, ra);
 #pragma unroll 1
-            for (int piece = p0; piece < p1; piece += 2) {
+            for (int piece = p0; piece < p0 + EPI_PIECES; piece += 2) {
+                uint32_t pa[16], pb[16];
                 tcgen05_ld_wait(ra);
                 tcgen05_ld_32x32_issue(tacc + (piece + 1) * 32, rb);
-                uint32_t pa[16], pb[16];
                 to_dz(ra, piece, pa);
                 tcgen05_ld_wait(rb);
-                if (piece + 2 < p1) tcgen05_ld_32x32_issue(tacc + (piece + 2) * 32, ra);
+                if (piece + 2 < p0 + EPI_PIECES) {
+                    tcgen05_ld_32x32_issue(tacc + (piece + 2) * 32, ra);
+                } else {
+                    tcgen05_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
+                }
                 to_dz(rb, piece + 1, pb);
-                if (lane == 0) bulk_wait_read_all();          // the previous tile store has read the staging tile
-                __syncwarp();
+                const int col0 = first_col + piece * 32;
+                __syncwarp();                                     // the staging tile has been read
                 stage_piece(pa, piece);
                 stage_piece(pb, piece + 1);
-                fence_proxy_async_smem();
                 __syncwarp();
-                const int col0 = first_col + piece * 32;
-                if (lane == 0 && col0 < p.V) {
-                    tma_store_2d(&map_dz, col0, row0, stg);
-                    bulk_commit_group();
+                const int q = lane & 7;                           // eight lanes per row
+                uint16_t* out = p.dz + (int64_t)(row0 + (lane >> 3)) * p.ldz + col0 + 8 * q;
+                uint4 line[8];                                    // all of them read before the first store
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int row = 4 * i + (lane >> 3);
+                    line[i] = *reinterpret_cast<const uint4*>(stg + row * 128 + ((q ^ (row & 7)) << 4));
+                }
+                if (col0 + 8 * q < p.ldz) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(out + 4 * i * p.ldz) = line[i];
                 }
             }
-            tcgen05_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            have = have_next;
+            m = m_next;
+            c = c_next;
         }
-        if (lane == 0) bulk_wait_all();       // the tile stores have completed before the block's shared memory goes
     }
     pipe_teardown(ps, p.d_status);
 }
@@ -520,8 +532,8 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
 // pairs busy for a whole wave, which is what a call of a few hundred tokens, with dH tiles of thousands of K steps on a handful
 // of pairs, spent its time on.  So they are cut (GemmWork): for dH into ranges of K, the first of which writes dH and the others
 // partial sums (in the rows of dZ that the chunk's tokens leave unused), added to dH in the order of the ranges by the epilogue
-// warps of the dW kernel, which wait for their first tile at that time; where there is no room for partial sums, and for
-// dW, into halves of their columns.  Neither depends on anything but the sizes, so results are the same from run to run.
+// warps of the dW kernel, which wait for their first tile at that time.  How they are cut depends on the sizes alone, so results are
+// the same from run to run.
 struct SumParams {            // dW kernel: the dH contraction whose partial sums it adds up
     const float* part;
     float* out;
@@ -541,7 +553,9 @@ struct GemmParams {
     int64_t T_max, t0;
     unsigned int* lock_words;
     int lock_word;
-    int slots;                // partial sums of a tile that fit the workspace (dH)
+    float* c;                 // [M, N], for direct stores
+    float* part;              // partial sums of a tile, 256 x 256 each (dH): as many as fit the workspace
+    int slots;
     SumParams sum;
     uint32_t* d_status;
 };
@@ -562,49 +576,31 @@ __device__ __forceinline__ bool gemm_item(int64_t i, int m_tiles, int n_tiles, i
 }
 
 // How the tiles of a launch are dealt.  Items [0, body) are whole tiles in the order of gemm_item; then the tail, by range of K and
-// tile (segs > 1; the tile as the fast index, so that the pairs that work at the same time share operand panels) or by tile and
-// half.  Where all tiles are tail, and the last column tile is half as wide as the others, its tiles are cut into half as many
-// ranges and come last.
-constexpr int MIN_SEG = 16;              // K steps of a range at least: an epoch of the lock-step, and ten times what its set-up takes
+// tile, the tile as the fast index, so that the pairs that work at the same time share operand panels.  (A column tile of half the
+// width counts like the others: a K step takes the issuing warp about 500 cycles whatever the MMAs' width.)
+constexpr int MIN_SEG = 16;              // K steps of a range at least: an epoch of the lock-step
 constexpr int SEG_COST = 12;             // K steps that a wave of ranges costs beside its own (writing and adding 256 KB a pair)
 struct GemmWork {
     int m_tiles, n_tiles, group_n, k_steps;
-    int body, tail, items;
-    int segs, narrow_segs;               // ranges of K per tail tile; of the narrow ones at the end of the tail
-    int wide;                            // tail tiles before the narrow ones
+    int body, tail, segs, items;         // tiles, tail tiles, ranges of K per tail tile
 };
-__device__ __forceinline__ GemmWork make_gemm_work(int m_tiles, int n_tiles, int group_n, int k_steps, int N, int units, int slots) {
+__device__ __forceinline__ GemmWork make_gemm_work(int m_tiles, int n_tiles, int group_n, int k_steps, int units, int slots) {
     GemmWork w;
     w.m_tiles = m_tiles; w.n_tiles = n_tiles; w.group_n = group_n; w.k_steps = k_steps;
-    const int tiles = m_tiles * n_tiles;
-    int tail = tiles % units;
-    w.segs = w.narrow_segs = 1;
-    const bool narrow = tail == tiles && n_tiles > 1 && N - (n_tiles - 1) * BN <= BN / 2;
-    w.wide = narrow ? tail - m_tiles : tail;
-    bool halves = false;
-    if (tail > 0) {
-        const int load = 2 * w.wide + (narrow ? m_tiles : 0);        // in half tiles
-        int best = k_steps;
-        if (2 * tail <= units && !narrow) { halves = true; best = k_steps * 5 / 8; }
+    const int tiles = m_tiles * n_tiles, tail = tiles % units;
+    w.segs = 1;
+    int best = k_steps;
+    if (tail > 0 && slots > 0)
 #pragma unroll 1
         for (int waves = 1; waves <= 3; ++waves) {
-            int s = min(2 * waves * units / load, min(k_steps / MIN_SEG, 2 * (slots + tail) / load));
-            if (narrow) s &= ~1;
-            if (s < 2 || s > 2 * units) continue;
-            const int cost = waves * ((k_steps + s - 1) / s + SEG_COST);
-            if (cost < best) { best = cost; w.segs = s; halves = false; }
+            const int s = min(waves * units / tail, min(k_steps / MIN_SEG, slots / tail + 1));
+            const int cost = waves * ((k_steps + s - 1) / max(s, 1) + SEG_COST);
+            if (s > 1 && cost < best) { best = cost; w.segs = s; }
         }
-        w.narrow_segs = narrow && w.segs > 1 ? w.segs / 2 : w.segs;
-        if (w.segs == 1 && !halves) tail = 0;                        // nothing to gain: whole tiles to the end
-    }
-    w.tail = tail;
-    w.body = tiles - tail;
-    w.items = w.body + (w.segs > 1 ? w.wide * w.segs + (tail - w.wide) * w.narrow_segs : halves ? 2 * tail : 0);
+    w.tail = w.segs > 1 ? tail : 0;      // nothing to gain: whole tiles to the end
+    w.body = tiles - w.tail;
+    w.items = w.body + w.tail * w.segs;
     return w;
-}
-// slot of range seg > 0 of tail tile idx
-__device__ __forceinline__ int gemm_slot(const GemmWork& w, int idx, int seg) {
-    return idx < w.wide ? (seg - 1) * w.wide + idx : (w.segs - 1) * w.wide + (seg - 1) * (w.tail - w.wide) + idx - w.wide;
 }
 __device__ __forceinline__ GemmTile gemm_tail_tile(const GemmWork& w, int idx) {
     GemmTile g;
@@ -612,40 +608,37 @@ __device__ __forceinline__ GemmTile gemm_tail_tile(const GemmWork& w, int idx) {
     else { g.n = idx / w.m_tiles; g.m = idx - g.n * w.m_tiles; }
     return g;
 }
-__device__ __forceinline__ bool gemm_work_item(const GemmWork& w, int N, int64_t item, GemmTile& g, TileAt& t) {
+// slot of range seg > 0 of tail tile idx
+__device__ __forceinline__ int gemm_slot(const GemmWork& w, int idx, int seg) { return (seg - 1) * w.tail + idx; }
+__device__ __forceinline__ bool gemm_work_item(const GemmWork& w, int N, int64_t item, TileAt& t) {
     if (item >= w.items) return false;
-    int i = (int)item, half = -1;
+    GemmTile g;
     t.k0 = 0;
     t.k1 = w.k_steps;
     t.slot = -1;
-    if (i < w.body) {
-        gemm_item(i, w.m_tiles, w.n_tiles, w.group_n, g);
-    } else if (w.segs > 1) {
-        i -= w.body;
-        const bool wide = i < w.wide * w.segs;
-        const int count = wide ? w.wide : w.tail - w.wide, segs = wide ? w.segs : w.narrow_segs;
-        if (!wide) i -= w.wide * w.segs;
-        const int seg = i / count, idx = i - seg * count + (wide ? 0 : w.wide);
-        t.k0 = (int)((unsigned)seg * (unsigned)w.k_steps / (unsigned)segs);            // segs <= 2 units, k_steps < 2^25 / 64 columns a step
-        t.k1 = (int)((unsigned)(seg + 1) * (unsigned)w.k_steps / (unsigned)segs);
+    if (item < w.body) {
+        gemm_item(item, w.m_tiles, w.n_tiles, w.group_n, g);
+    } else {
+        const int i = (int)item - w.body, seg = i / w.tail, idx = i - seg * w.tail;
+        t.k0 = (int)((unsigned)seg * (unsigned)w.k_steps / (unsigned)w.segs);          // segs <= 3 units, k_steps < 2^20
+        t.k1 = (int)((unsigned)(seg + 1) * (unsigned)w.k_steps / (unsigned)w.segs);
         if (seg > 0) t.slot = gemm_slot(w, idx, seg);
         g = gemm_tail_tile(w, idx);
-    } else {
-        half = (i - w.body) & 1;
-        g = gemm_tail_tile(w, (i - w.body) >> 1);
     }
     t.a0 = g.m * TILE_ROWS;
-    t.b0 = g.n * BN + (half > 0 ? BN / 2 : 0);
-    // 64 columns per block at least: the granularity of an MN-major B tile's blocks
-    t.n = half < 0 && N - t.b0 > BN / 2 ? BN : BN / 2;
+    t.b0 = g.n * BN;
+    t.n = N - t.b0 > BN / 2 ? BN : BN / 2;     // 64 columns per block at least: the granularity of an MN-major B tile's blocks
     return true;
 }
 
+// How results leave.  dH (written once, partial sums too): as 16-byte stores of whole lines, because a pair often has a single tile
+// and its last store is what the kernel waits for.  dW: by TMA tile stores and reductions, beside the MMAs of the next tile; direct
+// stores were no faster there (400 tokens, d = 512, V = 60,000 whole update 120 us, 124 with them; 12,000, d = 1,024, V = 30,000 1,662, 1,700).
 template <bool A_MN, bool B_MN>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_b_tail, const __grid_constant__ CUtensorMap map_c,
-            const __grid_constant__ CUtensorMap map_part, const GemmParams p) {
+            const GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     const PipeSmem ps = pipe_setup(smem_raw, &map_a, &map_b);
     uint8_t* c_stage = ps.stage_a + EPI_STAGE_OFFSET;      // one 32 x 32 fp32 staging tile per epilogue warp
@@ -660,34 +653,33 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int m_tiles = K == 0 ? 0 : p.m_is_tokens ? (int)min((int64_t)all_m_tiles, (live + TILE_ROWS - 1) / TILE_ROWS) : all_m_tiles;
     const int zero_m_tiles = live > 0 || p.zero_if_dead ? all_m_tiles - m_tiles : 0;
     const int64_t unit = blockIdx.x >> 1, units = gridDim.x >> 1;
-    const GemmWork work = make_gemm_work(m_tiles, n_tiles, p.group_n, k_steps, p.N, (int)units, p.slots);
-    auto coords = [&](int64_t it, TileAt& t) {
-        GemmTile g;
-        return gemm_work_item(work, p.N, unit + it * units, g, t);
-    };
+    const GemmWork work = make_gemm_work(m_tiles, n_tiles, p.group_n, k_steps, (int)units, p.slots);
+    auto coords = [&](int64_t it, TileAt& t) { return gemm_work_item(work, p.N, unit + it * units, t); };
 
     if (warp == 0) {
         const int tail_ks = (p.k_is_tokens && (K % BK) != 0) ? k_steps - 1 : -1;
         const Lockstep lock = lockstep_for(p.lock_words, p.lock_word, units, work.body, k_steps, work.items - work.body,
-                                           (k_steps + work.narrow_segs - 1) / work.narrow_segs);
+                                           (k_steps + work.segs - 1) / work.segs);
         producer_loop<A_MN, B_MN>(ps, &map_a, &map_b, lock, coords, p.a3d != 0, p.b3d != 0, &map_b_tail, tail_ks);
     } else if (warp == 1) {
         if (ps.rank == 0) mma_loop<A_MN, B_MN>(ps, k_steps, k_last, coords);
     } else {
         const int quarter = warp & 3;
-        const int col_half = (warp - 2) >> 2;           // 0 or 1: which half of the accumulator's columns
+        const int col_half = (warp - 2) >> 2;           // which half of the accumulator's columns
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        // The warp's 32 rows x 32 columns leave through shared memory (128-byte swizzle) as one TMA tile store, or
-        // as one TMA reduction (global += tile) when the result is accumulated: whole 128-byte lines, no read of C by
-        // the SM, and rows / columns past M / N are clipped by the copy.
+        // The warp's 32 rows x 32 columns leave through shared memory (128-byte swizzle): as one TMA tile store, or as one TMA
+        // reduction (global += tile) when the result is accumulated: whole 128-byte lines, no read of C by the SM, and rows / columns
+        // past M / N are clipped by the copy; or as 16-byte stores of whole lines.
+        constexpr bool DIRECT = !A_MN;
         uint8_t* stg = c_stage + (size_t)(warp - 2) * EPI_STAGE_TILE;
-        auto store_tile = [&](const TileAt& t, bool zero, uint32_t tacc) {
+        auto store_tile = [&](const TileAt& t, bool zero, uint32_t tacc, auto release) {
             const bool partial = t.slot >= 0;
             const int row0 = (partial ? t.slot * TILE_ROWS : t.a0) + (int)ps.rank * BM + quarter * 32;
             const int pieces = t.n / 32 / (EPI_WARPS / 4);              // of this warp
 #pragma unroll 1
-            for (int piece = col_half * pieces; piece < (col_half + 1) * pieces; ++piece) {
-                if (t.b0 + piece * 32 >= p.N) break;
+            for (int i = 0; i < pieces; ++i) {
+                const int piece = col_half * pieces + i;
+                const bool inside = t.b0 + piece * 32 < p.N;
                 const int pc0 = (partial ? 0 : t.b0) + piece * 32;
                 float v[32];
                 if (zero) {
@@ -695,27 +687,46 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     for (int j = 0; j < 32; ++j) v[j] = 0.f;
                 } else {
                     tcgen05_ld_32x32(tacc + piece * 32, v);
+                    if (i + 1 == pieces) release();
                 }
-                if (lane == 0) bulk_wait_read_all();          // the previous tile copy has read the staging tile
+                if (!inside) continue;
+                if (!DIRECT && lane == 0) bulk_wait_read_all();          // the previous tile copy has read the staging tile
                 __syncwarp();
 #pragma unroll
                 for (int q4 = 0; q4 < 8; ++q4)
                     *reinterpret_cast<float4*>(stg + lane * 128 + ((q4 ^ (lane & 7)) << 4)) =
                         make_float4(v[4 * q4], v[4 * q4 + 1], v[4 * q4 + 2], v[4 * q4 + 3]);
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0 && (partial || row0 < p.M)) {
-                    if (partial) tma_store_2d(&map_part, pc0, row0, stg);
-                    else if (p.accumulate) tma_reduce_add_2d(&map_c, pc0, row0, stg);
-                    else tma_store_2d(&map_c, pc0, row0, stg);
-                    bulk_commit_group();
+                if constexpr (DIRECT) {
+                    __syncwarp();
+                    const int q = lane & 7;                              // eight lanes per row
+                    const int64_t ld = partial ? BN : p.N;
+                    float* out = (partial ? p.part : p.c) + (int64_t)(row0 + (lane >> 3)) * ld + pc0 + 4 * q;
+                    float4 line[8];                                      // all of them read before the first store
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int row = 4 * k + (lane >> 3);
+                        line[k] = *reinterpret_cast<const float4*>(stg + row * 128 + ((q ^ (row & 7)) << 4));
+                    }
+                    if (partial || pc0 + 4 * q < p.N) {                  // N is a multiple of 8
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            if (partial || row0 + 4 * k + (lane >> 3) < p.M) *reinterpret_cast<float4*>(out + 4 * k * ld) = line[k];
+                    }
+                } else {
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0 && row0 < p.M) {
+                        if (p.accumulate) tma_reduce_add_2d(&map_c, pc0, row0, stg);
+                        else tma_store_2d(&map_c, pc0, row0, stg);
+                        bulk_commit_group();
+                    }
                 }
             }
         };
         if constexpr (A_MN) {       // dH += its partial sums, in the order of the ranges of K
             const SumParams& h = p.sum;
             const int h_tiles = (int)min((int64_t)((h.M + TILE_ROWS - 1) / TILE_ROWS), (live + TILE_ROWS - 1) / TILE_ROWS);
-            const GemmWork hw = make_gemm_work(h_tiles, n_tiles, h.group_n, (h.K + BK - 1) / BK, h.N, (int)h.units, h.slots);
+            const GemmWork hw = make_gemm_work(h_tiles, n_tiles, h.group_n, (h.K + BK - 1) / BK, (int)h.units, h.slots);
             if (hw.segs > 1) {
                 constexpr int QUADS = TILE_ROWS * BN / 4;                // of a tile
                 const float* part = pdl_acquire(h.part);
@@ -727,9 +738,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     if (row >= h.M || col >= h.N) continue;              // N is a multiple of 8
                     float4* out = reinterpret_cast<float4*>(h.out + (int64_t)row * h.N + col);
                     float4 v = __ldcg(out);
-                    const int segs = idx < hw.wide ? hw.segs : hw.narrow_segs;
 #pragma unroll 8
-                    for (int seg = 1; seg < segs; ++seg) {
+                    for (int seg = 1; seg < hw.segs; ++seg) {
                         const float4 x = __ldcg(reinterpret_cast<const float4*>(part + ((int64_t)gemm_slot(hw, idx, seg) * TILE_ROWS + r) * BN + 4 * q));
                         v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
                     }
@@ -739,22 +749,23 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         }
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        GemmTile g;
         TileAt t;
-        for (int64_t item = unit; ok && gemm_work_item(work, p.N, item, g, t); item += units) {
+        for (int64_t item = unit; ok && gemm_work_item(work, p.N, item, t); item += units) {
             ok = mbar_wait(&ps.acc_full[acc], acc_phase, ps.abort_flag);
             ok = __all_sync(0xffffffffu, ok) != 0;
             if (!ok) break;
             tcgen05_fence_after();
-            store_tile(t, false, ps.tmem_base + lane_addr + acc * BN);
-            tcgen05_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
+            store_tile(t, false, ps.tmem_base + lane_addr + acc * BN, [&]() {
+                tcgen05_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(ps.lead_acc_empty + acc * (uint32_t)sizeof(uint64_t));
+            });
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
+        GemmTile g;
         if (!p.accumulate)
             for (int64_t item = unit; gemm_item(item, zero_m_tiles, n_tiles, p.group_n, g); item += units)
-                store_tile(TileAt{(m_tiles + g.m) * TILE_ROWS, g.n * BN, BN, 0, 0, -1}, true, 0u);
+                store_tile(TileAt{(m_tiles + g.m) * TILE_ROWS, g.n * BN, BN, 0, 0, -1}, true, 0u, []() {});
         if (lane == 0) bulk_wait_all();       // the tile copies have completed before the block's shared memory goes
     }
     pipe_teardown(ps, p.d_status);
@@ -857,11 +868,10 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     // tensor maps: K-major operands are fetched as [128 MN rows x 64 K columns] boxes; MN-major ones (the same row-major
     // storage read the other way) as one three-dimensional box per stage when the MN extent is a whole number of
     // 64-element blocks, else as one [64 K rows x 64 MN columns] box per block
-    CUtensorMap map_h_k, map_w_k, map_dz_k, map_dz_st, map_w_mn, map_dz_mn, map_h_mn, map_h_tail;
+    CUtensorMap map_h_k, map_w_k, map_dz_k, map_w_mn, map_dz_mn, map_h_mn, map_h_tail;
     if (make_map(ctx, &map_h_k, hidden, (uint64_t)T_max, (uint64_t)d, BM) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map(ctx, &map_w_k, W_vocab, (uint64_t)V, (uint64_t)d, BN / 2) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map_ld(ctx, &map_dz_k, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BM) != ARROL_OK) return ARROL_ERR_CUDA;
-    if (make_map_ld(ctx, &map_dz_st, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, 32) != ARROL_OK) return ARROL_ERR_CUDA;   // store tiles
     CUtensorMap map_dw;
     if (make_map_f32_tile(ctx, &map_dw, dW, (uint64_t)V, (uint64_t)d, (uint64_t)d) != ARROL_OK) return ARROL_ERR_CUDA;
     bool d3 = d % 64 == 0, v3 = V % 64 == 0;
@@ -892,26 +902,23 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         zp.targets = targets; zp.grad_logp = grad_logp; zp.lse = lse; zp.d_T = d_T; zp.T_max = T_max; zp.t0 = t0;
         zp.d = d; zp.V = V; zp.group_tiles = (TC / TILE_ROWS + m_groups - 1) / m_groups;
         zp.scale2 = inv_temperature * 1.44269504088896340736f; zp.inv_temp = inv_temperature;
-        zp.lock_words = lock_words;
+        zp.lock_words = lock_words; zp.dz = reinterpret_cast<uint16_t*>(dZ); zp.ldz = L.ldz;
         zp.hidden = static_cast<const uint16_t*>(hidden); zp.tail = Htail; zp.d_status = ctx->d_status;
-        ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, s, map_h_k, map_w_k, map_dz_st, zp));
+        ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, s, map_h_k, map_w_k, zp));
 
         GemmParams gh = {};    // dH[chunk] = dZ . W
         gh.M = (int)rows; gh.N = d; gh.K = V; gh.group_n = group_columns(n_tiles);
         gh.m_is_tokens = 1; gh.b3d = d3; gh.lock_words = lock_words; gh.lock_word = LOCK_DH;
         gh.d_T = d_T; gh.T_max = T_max; gh.t0 = t0; gh.d_status = ctx->d_status;
-        CUtensorMap map_dh;      // this chunk's rows of dH: rows past the chunk are clipped by the tile stores
-        if (make_map_f32_tile(ctx, &map_dh, dH + t0 * d, (uint64_t)rows, (uint64_t)d, (uint64_t)d) != ARROL_OK)
-            return ARROL_ERR_CUDA;
         // partial sums of dH tiles lie in the rows of dZ that no tile of this chunk reaches
         constexpr size_t SLOT_BYTES = sizeof(float) * TILE_ROWS * BN;
         const size_t part_at = ((size_t)m_tiles * TILE_ROWS * L.ldz * 2 + 255) & ~(size_t)255;
         float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + L.dz + part_at);
         const size_t room = (L.tail - part_at) / SLOT_BYTES;
         gh.slots = room < 4096 ? (int)room : 4096;
-        CUtensorMap map_part = map_dh;
-        if (gh.slots > 0 && make_map_f32_tile(ctx, &map_part, part, (uint64_t)gh.slots * TILE_ROWS, BN, BN) != ARROL_OK) return ARROL_ERR_CUDA;
-        ARROL_CUDA_OK(launch_pairs(ctx, 1, gemm_kernel<false, true>, s, map_dz_k, map_w_mn, map_w_mn, map_dh, map_part, gh));
+        gh.part = part;
+        gh.c = dH + t0 * d;
+        ARROL_CUDA_OK(launch_pairs(ctx, 1, gemm_kernel<false, true>, s, map_dz_k, map_w_mn, map_w_mn, map_dw, gh));      // dH does not go through a map
         GemmParams gw = {};    // dW (+)= dZ^T . H[chunk]; the first chunk writes dW, zeros where no token lives
         gw.M = V; gw.N = d; gw.K = (int)rows; gw.group_n = group_columns(n_tiles);
         gw.accumulate = t0 > 0; gw.k_is_tokens = 1; gw.zero_if_dead = t0 == 0; gw.a3d = v3; gw.b3d = d3;
@@ -919,7 +926,7 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         gw.d_T = d_T; gw.T_max = T_max; gw.t0 = t0; gw.d_status = ctx->d_status;
         gw.sum.part = part; gw.sum.out = dH + t0 * d; gw.sum.M = gh.M; gw.sum.N = gh.N; gw.sum.K = gh.K;
         gw.sum.group_n = gh.group_n; gw.sum.slots = gh.slots; gw.sum.units = ctx->backward_max_pairs[1];
-        ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, s, map_dz_mn, map_h_mn, map_h_tail, map_dw, map_dw, gw));
+        ARROL_CUDA_OK(launch_pairs(ctx, 2, gemm_kernel<true, true>, s, map_dz_mn, map_h_mn, map_h_tail, map_dw, gw));
         ctx->launches += 3;
     }
     return ARROL_OK;
