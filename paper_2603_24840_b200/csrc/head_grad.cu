@@ -30,6 +30,9 @@ __global__ void __launch_bounds__(DS_THREADS)
 head_ds_kernel(const float* __restrict__ score, int N, const float* __restrict__ rewards, const uint8_t* __restrict__ mask, float* __restrict__ ds,
                double* __restrict__ loss, float* __restrict__ dbias) {
     __shared__ double sh[32];
+    pdl_launch_dependents();
+    pdl_wait();
+    score = pdl_acquire(score); rewards = pdl_acquire(rewards); mask = pdl_acquire(mask);
     double cnt = 0.0;
     for (int i = threadIdx.x; i < N; i += DS_THREADS) cnt += (!mask || mask[i]) ? 1.0 : 0.0;
     const double n = block_sum(cnt, sh);
@@ -67,34 +70,56 @@ __device__ __forceinline__ void widen8(const float* p, float (&o)[8]) {
     o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
 }
 
-// Linear head: partial[c][k] = sum over the rows of row-chunk c of ds_i x_ik.  Thread = 8 consecutive columns.
-constexpr int LIN_ROWS = 32;
+// Linear head: partial[c][k] = sum over the rows of row-chunk c of ds_i x_ik, in index order.  Thread = 8 consecutive columns.  Bound by
+// the latency of its loads where the rollouts are few: the chunk's factors and row numbers come in one round trip and eight
+// rows are in flight (a row at a time, each behind its factor and its number: 15.4 us under the profiler at N = 172, d = 1,464).
+// Rows without a factor are not read.
+constexpr int LIN_ROWS = 32, LIN_AHEAD = 8;
 template <typename T>
 __global__ void __launch_bounds__(256)
 linear_dw_partial_kernel(const T* __restrict__ hidden, int64_t row_stride, const int64_t* __restrict__ row_index,
                          int N, int d, const float* __restrict__ ds, float* __restrict__ partial) {
+    __shared__ float g_s[LIN_ROWS];
+    __shared__ int64_t row_s[LIN_ROWS];
+    pdl_launch_dependents();
+    pdl_wait();
+    hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); ds = pdl_acquire(ds);
     const int k0 = (blockIdx.x * 256 + threadIdx.x) * 8;
+    const int i0 = blockIdx.y * LIN_ROWS;
+    if (threadIdx.x < LIN_ROWS) {
+        const int i = i0 + threadIdx.x;
+        g_s[threadIdx.x] = i < N ? ds[i] : 0.f;
+        row_s[threadIdx.x] = i < N ? (row_index ? row_index[i] : (int64_t)i) : 0;
+    }
+    __syncthreads();
     if (k0 >= d) return;
-    const int i0 = blockIdx.y * LIN_ROWS, i1 = min(N, i0 + LIN_ROWS);
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int i = i0; i < i1; ++i) {
-        const float g = ds[i];
-        if (g == 0.f) continue;
-        const int64_t row = row_index ? row_index[i] : (int64_t)i;
-        float x[8];
-        widen8(hidden + row * row_stride + k0, x);
+#pragma unroll 1
+    for (int r0 = 0; r0 < LIN_ROWS; r0 += LIN_AHEAD) {
+        float x[LIN_AHEAD][8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = fmaf(g, x[e], acc[e]);
+        for (int r = 0; r < LIN_AHEAD; ++r)
+            if (g_s[r0 + r] != 0.f) widen8(hidden + row_s[r0 + r] * row_stride + k0, x[r]);
+#pragma unroll
+        for (int r = 0; r < LIN_AHEAD; ++r)
+            if (g_s[r0 + r] != 0.f) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[e] = fmaf(g_s[r0 + r], x[r][e], acc[e]);
+            }
     }
     float* out = partial + (int64_t)blockIdx.y * d + k0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) out[e] = acc[e];
+    *reinterpret_cast<float4*>(out) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    *reinterpret_cast<float4*>(out + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
 }
 
 __global__ void column_sum_kernel(const float* __restrict__ partial, int chunks, int d, float* __restrict__ out) {
+    pdl_launch_dependents();
+    pdl_wait();
+    partial = pdl_acquire(partial);
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= d) return;
     float s = 0.f;
+#pragma unroll 8
     for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * d + k];
     out[k] = s;
 }
@@ -342,11 +367,11 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         const int rc = arrol_score_partial(ctx, hidden, row_stride, row_index, N, head, nullptr, tmp, tmp + N, nullptr,
                                            tmp + 2 * (size_t)N, s);
         if (rc != ARROL_OK) return rc;
-        head_ds_kernel<<<1, DS_THREADS, 0, s>>>(tmp, N, rewards, mask, ds, loss, db1);
+        ARROL_CUDA_OK(arrol_launch_pdl(head_ds_kernel, dim3(1), dim3(DS_THREADS), 0, s, static_cast<const float*>(tmp), N, rewards, mask, ds, loss, db1));
         const int chunks = (N + LIN_ROWS - 1) / LIN_ROWS;
         dim3 grid((d / 8 + 255) / 256, chunks);
-        linear_dw_partial_kernel<T><<<grid, 256, 0, s>>>(hid, row_stride, row_index, N, d, ds, partial);
-        column_sum_kernel<<<(d + 255) / 256, 256, 0, s>>>(partial, chunks, d, dW1);
+        ARROL_CUDA_OK(arrol_launch_pdl(linear_dw_partial_kernel<T>, grid, dim3(256), 0, s, hid, row_stride, row_index, N, d, static_cast<const float*>(ds), partial));
+        ARROL_CUDA_OK(arrol_launch_pdl(column_sum_kernel, dim3((d + 255) / 256), dim3(256), 0, s, static_cast<const float*>(partial), chunks, d, dW1));
         ctx->launches += 3;
     } else {
         float* u = reinterpret_cast<float*>(ws + L.u);
