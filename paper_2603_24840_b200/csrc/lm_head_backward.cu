@@ -136,6 +136,7 @@ struct Lockstep {
     int word;
     uint32_t units, epochs;     // epochs of the pair with the most work
     int items_per_epoch;        // > 1 when a tile has few K steps
+    bool on;                    // false: the pairs go as they like, and the counter is not touched
 };
 // `body` items of k_steps K steps each, then `tail` items of at most tail_steps (the same number where k_steps < EPOCH)
 __device__ __forceinline__ Lockstep lockstep_for(unsigned int* words, int word, int64_t units, int64_t body, int k_steps, int64_t tail,
@@ -144,6 +145,7 @@ __device__ __forceinline__ Lockstep lockstep_for(unsigned int* words, int word, 
     l.words = words;
     l.word = word;
     l.units = (uint32_t)units;
+    l.on = true;
     l.items_per_epoch = k_steps >= EPOCH ? 1 : EPOCH / max(k_steps, 1);
     const int64_t most = (body + units - 1) / units, most_tail = (tail + units - 1) / units;
     l.epochs = (uint32_t)(k_steps >= EPOCH ? most * ((k_steps + EPOCH - 1) / EPOCH) + most_tail * ((tail_steps + EPOCH - 1) / EPOCH)
@@ -182,7 +184,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
                                               const CUtensorMap* mb_tail = nullptr, int tail_ks = -1) {
     const uint32_t a0 = smem_u32(ps.stage_a), b0 = smem_u32(ps.stage_b);
     uint32_t stage = 0, phase = 0, issued = 0, epoch = 0;
-    bool ok = true, in_step = true;
+    bool ok = true, in_step = lock.on;
     TileAt tile;
     int to_epoch = 0;                     // items until the next epoch
     if (blockIdx.x == 0 && elect_one()) lock.words[(lock.word + 1) % LOCK_WORDS] = 0u;
@@ -190,7 +192,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
         const int ay = tile.a0 + (int)ps.rank * BM, by = tile.b0 + (int)ps.rank * (tile.n / 2);
         for (int ks0 = tile.k0; ks0 < tile.k1 && ok; ks0 += EPOCH) {
             if (ks0 > tile.k0 || to_epoch == 0) {
-                if (ps.rank == 0) {
+                if (lock.on && ps.rank == 0) {
                     if (elect_one()) {
                         if (in_step) in_step = begin_epoch(lock, ps.lock_seen, epoch);
                         else atomicAdd(lock.words + lock.word, 1u);
@@ -241,7 +243,7 @@ __device__ __forceinline__ void producer_loop(const PipeSmem& ps, const CUtensor
         }
         --to_epoch;
     }
-    if (ps.rank == 0 && elect_one()) {
+    if (lock.on && ps.rank == 0 && elect_one()) {
         cp_async_wait_all();
         if (epoch < lock.epochs) atomicAdd(lock.words + lock.word, lock.epochs - epoch);   // done: nobody waits for this pair
     }
@@ -330,6 +332,7 @@ struct DzParams {
     float scale2, inv_temp;
     const uint16_t* hidden;
     unsigned int* lock_words;
+    int lock_on;
     uint16_t* dz;             // [TC, ldz]
     int64_t ldz;
     uint16_t* tail;           // [63, d]: the last, partly live 64-row block of the chunk's hidden rows, zero-padded
@@ -383,7 +386,8 @@ dz_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_constant__ CUt
     };
 
     if (warp == 0) {
-        const Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, (int64_t)m_tiles * total_chunks, k_steps, 0, 0);
+        Lockstep lock = lockstep_for(p.lock_words, LOCK_DZ, units, (int64_t)m_tiles * total_chunks, k_steps, 0, 0);
+        lock.on = p.lock_on != 0;
         producer_loop<false, false>(ps, &map_h, &map_w, lock, coords);
     } else if (warp == 1) {
         if (ps.rank == 0) mma_loop<false, false>(ps, k_steps, k_last, coords);
@@ -816,6 +820,8 @@ int raise_smem_limits(arrol_ctx* ctx) {
     return ARROL_OK;
 }
 
+constexpr int FREE_TILES = 8;          // tiles per pair that are not kept in step
+
 struct BackwardLayout {
     int64_t ldz;       // V rounded up to 8
     size_t dz, tail, lock, total;
@@ -862,7 +868,11 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     __nv_bfloat16* dZ = reinterpret_cast<__nv_bfloat16*>(static_cast<uint8_t*>(workspace) + L.dz);
     uint16_t* Htail = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + L.tail);
     unsigned int* lock_words = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + L.lock);
-    ARROL_CUDA_OK(cudaMemsetAsync(lock_words, 0, LOCK_BYTES, s));
+    // The dz kernel's counter has to be zero before the first chunk (the later ones are zeroed by the kernels).  Clearing it costs a
+    // call about 2 us and keeps the dz kernel's start from overlapping the end of the kernel before it, so calls of which a pair has
+    // few tiles do without the step: they are over before pairs drift apart.
+    const bool first_in_step = (T_max + TILE_ROWS - 1) / TILE_ROWS * ((V + BN - 1) / BN) > (int64_t)FREE_TILES * (ctx->sm_count / 2);
+    if (first_in_step) ARROL_CUDA_OK(cudaMemsetAsync(lock_words, 0, LOCK_BYTES, s));
     if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
 
     // tensor maps: K-major operands are fetched as [128 MN rows x 64 K columns] boxes; MN-major ones (the same row-major
@@ -902,7 +912,7 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
         zp.targets = targets; zp.grad_logp = grad_logp; zp.lse = lse; zp.d_T = d_T; zp.T_max = T_max; zp.t0 = t0;
         zp.d = d; zp.V = V; zp.group_tiles = (TC / TILE_ROWS + m_groups - 1) / m_groups;
         zp.scale2 = inv_temperature * 1.44269504088896340736f; zp.inv_temp = inv_temperature;
-        zp.lock_words = lock_words; zp.dz = reinterpret_cast<uint16_t*>(dZ); zp.ldz = L.ldz;
+        zp.lock_words = lock_words; zp.lock_on = t0 > 0 || first_in_step; zp.dz = reinterpret_cast<uint16_t*>(dZ); zp.ldz = L.ldz;
         zp.hidden = static_cast<const uint16_t*>(hidden); zp.tail = Htail; zp.d_status = ctx->d_status;
         ARROL_CUDA_OK(launch_pairs(ctx, 0, dz_kernel, s, map_h_k, map_w_k, zp));
 

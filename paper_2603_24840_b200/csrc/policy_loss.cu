@@ -18,6 +18,10 @@ policy_loss_kernel(const float* __restrict__ logp, const float* __restrict__ log
                    const int32_t* __restrict__ tok_seq, const int64_t* __restrict__ cu_seqlens,
                    const int64_t* __restrict__ d_num, int64_t T_max, float eps_low, float eps_high, float beta,
                    int agg_mode, float* __restrict__ grad, double* __restrict__ block_partial) {
+    pdl_launch_dependents();
+    pdl_wait();
+    logp = pdl_acquire(logp); logp_old = pdl_acquire(logp_old); logp_ref = pdl_acquire(logp_ref); tok_adv = pdl_acquire(tok_adv);
+    tok_seq = pdl_acquire(tok_seq); cu_seqlens = pdl_acquire(cu_seqlens); d_num = pdl_acquire(d_num);
     const int64_t S = d_num[0];
     int64_t T = d_num[1];
     if (T > T_max) T = T_max;
@@ -61,12 +65,17 @@ policy_loss_kernel(const float* __restrict__ logp, const float* __restrict__ log
     }
 }
 
+// One warp: lane l adds every 32nd partial sum from l on, the lanes' sums by a butterfly: one order for a number of blocks.
 __global__ void policy_loss_finish_kernel(const double* __restrict__ block_partial, int n, double* __restrict__ loss) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double tot = 0.0;
-        for (int i = 0; i < n; ++i) tot += block_partial[i];
-        *loss = tot;
-    }
+    pdl_launch_dependents();
+    pdl_wait();
+    block_partial = pdl_acquire(block_partial);
+    double tot = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += 32) tot += block_partial[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (threadIdx.x == 0) *loss = tot;
 }
 
 }  // namespace
@@ -87,11 +96,9 @@ extern "C" int arrol_policy_loss(arrol_ctx* ctx, const float* logp, const float*
     if (blocks > PL_MAX_BLOCKS) blocks = PL_MAX_BLOCKS;
     if (blocks < 1) blocks = 1;
     double* partial = reinterpret_cast<double*>(ctx->d_scratch);
-    policy_loss_kernel<<<(unsigned)blocks, PL_THREADS, 0, s>>>(logp, logp_old, logp_ref, tok_adv, tok_seq, cu_seqlens,
-                                                              d_num, T_max, eps_low, eps_high, beta, agg_mode,
-                                                              grad_logp, partial);
-    policy_loss_finish_kernel<<<1, 32, 0, s>>>(partial, (int)blocks, loss);
+    ARROL_CUDA_OK(arrol_launch_pdl(policy_loss_kernel, dim3((unsigned)blocks), dim3(PL_THREADS), 0, s, logp, logp_old, logp_ref, tok_adv,
+                                   tok_seq, cu_seqlens, d_num, T_max, eps_low, eps_high, beta, (int)agg_mode, grad_logp, partial));
+    ARROL_CUDA_OK(arrol_launch_pdl(policy_loss_finish_kernel, dim3(1), dim3(32), 0, s, static_cast<const double*>(partial), (int)blocks, loss));
     ctx->launches += 2;
-    ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;
 }
