@@ -184,8 +184,10 @@ class PruneRebatch:
         return B.make_prune_step(self.hidden_score, self.head, self.q_lut, scal, tensors)
 
     def step(self):
-        """One pass of the whole path: score -> select -> compact (tokens + hidden rows) -> token log-prob."""
-        self.prune_step()
+        """One pass of the whole path: score -> select -> compact (tokens + hidden rows) -> token log-prob.  The first three through
+        the one-call prune step: the same results, two launches instead of four to seven and one call instead of three (a
+        debugging-size step is bound by them: 36 -> 31 us)."""
+        B.arrol_prune_step(self.ctx, self.prune_step_args())
         self.token_logprob()
 
     def counts(self):
