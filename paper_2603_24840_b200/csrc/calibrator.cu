@@ -70,9 +70,10 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 
 // One block, bound by latency: a handful of dependent round trips to memory and a serial search.  Every input is read once
 // (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
-// that one block scan ranks all of them, and the bisection is settled in about five rounds of 31 points (see below) instead
-// of 64 steps, twenty of them with a serial sum.  Per call, timed back to back: N = 2,048, 128 bins 61.5 -> 26.7 us; N = 32,
-// 64 bins 41 -> 22 us; N = 8,192, 256 bins 100 -> 37 us.  More rollouts go through shared memory in pieces of CAL_STAGED,
+// that one block scan ranks all of them, and the bisection is settled in three rounds of 31 points (see below) instead of 64
+// steps.  Per call, in a graph of 20 (with six rounds, separate round trips for mask, bin and reward, and a later one for
+// the evicted entries before): N = 2,048, 128 bins 25.6 -> 17.4 us; N = 32, 64 bins 21.1 -> 14.4; N = 8,192, 256 bins 34.9 -> 24.1; 13 of
+// the 17 us are the search.  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
 // per thread and scan, as it was before the runs, 460 and 1,570).  An instance each, because the pieces' code in the same one cost
@@ -169,18 +170,36 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
             before[l] = (wid > 0 ? warps_before : 0) + incl[l] - mine[l];
         }
     };
-    // This thread's run [j0, j1) of the n staged entries, and the rank of its first one among those of its label.
+    // This thread's run [j0, j1) of the n staged entries, and the rank of its first one among those of its label.  Both labels'
+    // counts in one word, 16 bits each: at most CAL_STAGED entries.
+    static_assert(CAL_STAGED < 1 << 15, "two counts in one word");
     auto rank_run = [&](int n, int& j0, int& j1, int64_t (&first_rank)[2], int64_t (&total)[2]) {
         const int per = (n + CAL_THREADS - 1) / CAL_THREADS;
         j0 = min(n, tid * per);
         j1 = min(n, j0 + per);
-        int32_t mine[2] = {0, 0};
+        int32_t mine = 0;
         for (int j = j0; j < j1; ++j) {
             const int c = staged[j];
-            mine[0] += c >= 0 && (c & 1) == 0 ? 1 : 0;
-            mine[1] += c >= 0 && (c & 1) != 0 ? 1 : 0;
+            mine += c < 0 ? 0 : (c & 1) ? 1 << 16 : 1;
         }
-        block_scan(mine, first_rank, total);
+        int32_t incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) warp_sum[0][wid] = incl;
+        __syncthreads();
+        int32_t v = warp_sum[0][lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t t = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += t;
+        }
+        const int32_t all = __shfl_sync(0xffffffffu, v, 31), warps_before = __shfl_sync(0xffffffffu, v, wid > 0 ? wid - 1 : 0);
+        const int32_t before = (wid > 0 ? warps_before : 0) + incl - mine;
+        first_rank[0] = before & 0xffff; first_rank[1] = before >> 16;
+        total[0] = all & 0xffff; total[1] = all >> 16;
     };
     int j0 = 0, j1 = 0;
     int64_t total_new[2], first_rank[2];
@@ -334,11 +353,15 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
                 } else {                             // replay as far as the settled points reach
                     const double base_below = __dadd_rn(kappa, known_below), base_above = __dadd_rn(kappa, known_above);
                     double m = midpoint(lo, hi);
-                    for (; step < 64; ++step) {
-                        const double base = __dadd_rn(kappa, m), m_up = midpoint(m, hi), m_down = midpoint(lo, m);    // side by side
-                        if (base <= base_below) { if (m == lo) step = 64; lo = m; m = m_up; }      // an unchanged bracket stays unchanged
-                        else if (base >= base_above) { if (m == hi) step = 64; hi = m; m = m_down; }
-                        else break;
+                    while (step < 64) {              // both next midpoints while the comparison is under way
+                        const double base = __dadd_rn(kappa, m), m_up = midpoint(m, hi), m_down = midpoint(lo, m);
+                        const bool below = base <= base_below;
+                        if (!(below || base >= base_above)) break;
+                        const bool unchanged = below ? m == lo : m == hi;                          // then it stays unchanged
+                        lo = below ? m : lo;
+                        hi = below ? hi : m;
+                        m = below ? m_up : m_down;
+                        step = unchanged ? 64 : step + 1;
                     }
                     if (step >= 64) kind = DONE;
                     a = lo;
@@ -374,6 +397,7 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
             if (wid < CAL_POINTS) {
                 const double base = __dadd_rn(kappa, x);
                 double part = 0.0, slope = 0.0;
+#pragma unroll 4
                 for (int k = lane; k < B; k += 32) {
                     const double raw = __dadd_rn(base, term[k]), p = clipped(raw);
                     const double v = __dmul_rn(weight[k], p);
