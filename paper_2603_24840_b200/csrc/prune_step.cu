@@ -209,14 +209,17 @@ prune_fused_kernel(const FusedParams p) {
         base_t += __shfl_xor_sync(0xffffffffu, base_t, o);
         base_c += __shfl_xor_sync(0xffffffffu, base_c, o);
     }
-    // this block has read what it needed: it says so before it writes, so that the arrival does not wait for the stores
+    // This block has read what it needed (`expired` comes from the values read): it says so before it writes, without a fence, which
+    // would wait for the published totals to be performed (1.5 us).
     const bool any_bad = __any_sync(0xffffffffu, bad_index);
     const bool any_expired = __any_sync(0xffffffffu, expired);
     unsigned long long done = 0;
     if (lane == 0) {
         if (any_expired) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
-        if (any_bad) atomicOr(reinterpret_cast<unsigned int*>(p.chain + 1), 1u);
-        __threadfence();
+        if (any_bad) {
+            atomicOr(reinterpret_cast<unsigned int*>(p.chain + 1), 1u);
+            __threadfence();
+        }
         done = atomicAdd(p.chain, 1ull);
     }
     asm volatile("bar.sync 1, 64;" ::: "memory");            // the groups' statistics
