@@ -539,8 +539,10 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
 
 // Gathered variant, first kernel: copies every token tile that crosses a survivor boundary into its scratch slot.
 // Block s looks at the tile that holds survivor s's last row: if that tile starts inside s (so s owns it) and runs on
-// past the end of s, its rows are copied, run by run, with 16-byte loads/stores (eight in flight per thread).
-constexpr int PACK_THREADS = 256;
+// past the end of s, its rows are copied, run by run, with 16-byte loads/stores (eight in flight per thread).  Bound by latency: a
+// pass of 32 KB takes a block about 2 us and a tile of d = 2,240 has 18 of them, so the passes of a tile are dealt to the blocks of a
+// column of the grid while that leaves SMs without one.
+constexpr int PACK_THREADS = 256, PACK_PASS = 8 * PACK_THREADS;
 __global__ void __launch_bounds__(PACK_THREADS)
 pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __restrict__ cu_seqlens,
                            const int32_t* __restrict__ survivor_idx, const int64_t* __restrict__ src_tok_off,
@@ -556,7 +558,8 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
     T = T < 0 ? 0 : (T < T_max ? T : T_max);
     // where every token tile's rows come from (an even number of entries: a pair's second tile may lie past T)
     const int64_t tiles = ((T + BM - 1) / BM + 1) / 2 * 2;
-    for (int64_t i = blockIdx.x * (int64_t)PACK_THREADS + threadIdx.x; i < tiles; i += (int64_t)gridDim.x * PACK_THREADS) {
+    const int64_t block = (int64_t)blockIdx.y * gridDim.x + blockIdx.x, blocks = (int64_t)gridDim.x * gridDim.y;
+    for (int64_t i = block * PACK_THREADS + threadIdx.x; i < tiles; i += blocks * PACK_THREADS) {
         const int64_t t0 = i * BM;
         int32_t row = 0;
         if (t0 < T) {
@@ -584,7 +587,7 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
         __syncthreads();
         uint4* dst = scratch + (int64_t)s0 * BM * vec_per_row;
         const int total = rows * vec_per_row;
-        for (int v0 = 0; v0 < total; v0 += 8 * PACK_THREADS) {
+        for (int v0 = (int)blockIdx.y * PACK_PASS; v0 < total; v0 += (int)gridDim.y * PACK_PASS) {
             uint4 buf[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
@@ -909,8 +912,11 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     cfg.attrs = attr;
     cfg.numAttrs = n_attr;
     if (ga) {
-        int blocks = ga->S_max < ctx->sm_count * 4 ? ga->S_max : ctx->sm_count * 4;
-        ARROL_CUDA_OK(arrol_launch_pdl(pack_boundary_tiles_kernel, dim3((unsigned)blocks), dim3(PACK_THREADS), 0, s,
+        const int blocks = ga->S_max < ctx->sm_count * 4 ? ga->S_max : ctx->sm_count * 4;
+        const int passes = (BM * (d / 8) + PACK_PASS - 1) / PACK_PASS;
+        int columns = ctx->sm_count * 4 / blocks;
+        if (columns > passes) columns = passes;
+        ARROL_CUDA_OK(arrol_launch_pdl(pack_boundary_tiles_kernel, dim3((unsigned)blocks, (unsigned)columns), dim3(PACK_THREADS), 0, s,
                                        static_cast<const uint4*>(hidden), ga->cu_seqlens, ga->survivor_idx,
                                        ga->src_tok_off, ga->d_num, ga->S_max, T_max, d / 8, static_cast<uint4*>(scratch), tile_row));
         ctx->launches += 1;
