@@ -164,8 +164,8 @@ size_t arrol_token_logprob_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, i
  * Token tiles that would not fill a whole wave of blocks are cut finer; the results do not depend on it. */
 int32_t arrol_token_logprob_splits(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V);
 /* Form of the kernel for these sizes: 2 = pairs of thread blocks on 256-row token tiles (tcgen05 cta_group::2), 1 = one
- * block per 128-row tile.  Pairs are used for hidden widths above 512; see ARROL_HOOK_LOGPROB_PAIR.  0 for invalid
- * arguments. */
+ * block per 128-row tile.  Pairs are used for hidden widths above 512 and, where T_max d >= 800,000, from 320; see
+ * ARROL_HOOK_LOGPROB_PAIR.  0 for invalid arguments. */
 int32_t arrol_token_logprob_form(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V);
 int arrol_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_vocab, const int32_t* targets,
                         int64_t T_max, const int64_t* d_T, int32_t d, int32_t V, float inv_temperature,
@@ -474,7 +474,7 @@ int64_t arrol_launch_count(arrol_ctx* ctx);
  *   ARROL_HOOK_LOGPROB_PAIR          form of the log-prob kernel.  0: one thread block per 128-row token tile (tcgen05
  *                                    cta_group::1, cooperative launch).  1: clusters of two thread blocks that share
  *                                    one 256-row tile (tcgen05 cta_group::2; the same results bit for bit at equal
- *                                    split counts).  2 (the default): pairs for hidden widths above 512.
+ *                                    split counts).  2 (the default): pairs where arrol_token_logprob_form says so.
  *                                    Pairs wait for one another per wave, so no more
  *                                    of them are launched than cudaOccupancyMaxActiveClusters says are resident at
  *                                    once (asked once per context).  Set it before sizing the workspace.

@@ -191,37 +191,51 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
     return t;
 }
 
-// 32 columns pc0 ... of one token row into its running record.
+// 32 columns pc0 ... of one token row into its running record.  2.5 instructions a column: maxima three at a time, the exponents'
+// arguments and the sums two at a time in packed fp32, and four chains of either, so that a warp does not wait for its own additions.
 template <bool CONF>
-__device__ __forceinline__ void accumulate_piece(float (&v)[32], int pc0, int y, int V, float scale2, PartialLse& r) {
+__device__ __forceinline__ void accumulate_piece(uint32_t (&raw)[32], int pc0, int y, int V, float scale2, PartialLse& r) {
+    auto v = [&](int j) { return __uint_as_float(raw[j]); };
     if constexpr (CONF) {                   // sum of the valid logits of the piece (before masking)
         float ps[4] = {0.f, 0.f, 0.f, 0.f};           // four chains; only the last piece needs the mask
         if (pc0 + 32 <= V) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) ps[j & 3] += v[j];
+            for (int j = 0; j < 32; ++j) ps[j & 3] += v(j);
         } else {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) ps[j & 3] += (pc0 + j < V) ? v[j] : 0.f;
+            for (int j = 0; j < 32; ++j) ps[j & 3] += (pc0 + j < V) ? v(j) : 0.f;
         }
         r.sumz += (ps[0] + ps[1]) + (ps[2] + ps[3]);
     }
     if (pc0 + 32 > V) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) if (pc0 + j >= V) v[j] = -INFINITY;
+        for (int j = 0; j < 32; ++j) if (pc0 + j >= V) raw[j] = 0xff800000u;      // -inf
     }
     if ((unsigned)(y - pc0) < 32u) {
         const int jy = y - pc0;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) if (j == jy) r.zy2 = v[j] * scale2;
+        for (int j = 0; j < 32; ++j) if (j == jy) r.zy2 = v(j) * scale2;
     }
-    float bmax = v[0];
+    float top[4] = {v(0), v(1), v(2), v(3)};
 #pragma unroll
-    for (int j = 1; j < 32; ++j) bmax = fmaxf(bmax, v[j]);
+    for (int j = 4; j < 28; j += 8)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) top[c] = fmaxf(fmaxf(top[c], v(j + c)), v(j + 4 + c));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) top[c] = fmaxf(top[c], v(28 + c));
+    const float bmax = fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
     const float m_new = fmaxf(r.m2, bmax * scale2);
-    float sum = 0.f;
+    const uint64_t scale = pack_f32x2(scale2, scale2), minus_m = pack_f32x2(-m_new, -m_new);
+    uint64_t sum[2] = {0ull, 0ull};
 #pragma unroll
-    for (int j = 0; j < 32; ++j) sum += ex2_approx(fmaf(v[j], scale2, -m_new));
-    r.l = fmaf(r.l, ex2_approx(r.m2 - m_new), sum);
+    for (int j = 0; j < 32; j += 2) {
+        float a, b;
+        unpack_f32x2(fma_f32x2(((uint64_t)raw[j + 1] << 32) | raw[j], scale, minus_m), a, b);
+        sum[(j >> 1) & 1] = add_f32x2(sum[(j >> 1) & 1], pack_f32x2(ex2_approx(a), ex2_approx(b)));
+    }
+    float s0, s1;
+    unpack_f32x2(add_f32x2(sum[0], sum[1]), s0, s1);
+    r.l = fmaf(r.l, ex2_approx(r.m2 - m_new), s0 + s1);
     r.m2 = m_new;
 }
 
@@ -489,8 +503,9 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                     for (int piece = 0; piece < EPI_COLS / 32; ++piece) {
                         const int pc0 = col0 + piece * 32;
                         if (pc0 >= p.V) break;                  // columns past the vocabulary
-                        float v[32];
-                        tcgen05_ld_32x32(tmem_base + lane_addr + acc * BN + half * EPI_COLS + piece * 32, v);
+                        uint32_t v[32];
+                        tcgen05_ld_32x32_issue(tmem_base + lane_addr + acc * BN + half * EPI_COLS + piece * 32, v);
+                        tcgen05_ld_wait(v);
                         accumulate_piece<CONF>(v, pc0, y, p.V, p.scale2, sub);
                     }
                     tcgen05_fence_before();
@@ -713,27 +728,30 @@ int splits_for(const arrol_ctx* ctx, int d, int V, bool pair) {
     return splits < total_chunks ? splits : total_chunks;
 }
 
-// The form of the kernel for these sizes (V = 61,125, 100,000 tokens; us as single blocks with 4 / 8 epilogue warps and as
-// pairs with 4 / 8):
-//   d = 256   3,676 / 3,090   3,935 / 3,514        d = 640    6,006 / 6,120    6,297 / 5,877
-//   d = 384   4,393 / 3,879   4,616 / 4,385        d = 768    7,140 / 7,242    6,954 / 6,653
-//   d = 512   5,077 / 5,000   5,595 / 5,168        d = 1,024  9,376 / 9,445    8,798 / 8,854
+// The form of the kernel for these sizes (V = 61,125, 100,000 tokens; us as single blocks and as pairs, eight epilogue warps up to
+// 768, four beyond):
+//   d = 256   2,865 / 2,850    d = 320 (20,000 tokens, V = 40,000)  456 / 425    d = 384   3,757 / 3,530    d = 512   4,710 / 4,290
+//   d = 768 (four / eight warps)  7,140 / 7,242, pairs 6,954 / 6,653             d = 1,024 9,376 / 8,798
 //   d = 4,096 (V = 151,936, 287,000 tokens): single blocks with two splits 250.6 ms, pairs with four 247.9 ms
 // A chunk's 128 x 256 exponentials take an SM's special-function units 2,048 cycles, its MMAs 8 d: at small d the epilogue
 // sets the pace.  Two warps per scheduler then hide the latency of one another's tensor-memory loads, and single blocks
-// hand an accumulator back without waiting for a peer's epilogue.  At large d the tensor pipe and the power cap set it:
-// pairs move fewer operand bytes, and the fewer epilogue warps draw less power.
-constexpr int PAIR_MIN_WIDTH = 513, EIGHT_WARPS_MAX_WIDTH = 896;
-bool pair_for(const arrol_ctx* ctx, int d) {
+// hand an accumulator back without waiting for a peer's epilogue.  At larger d pairs move fewer operand bytes, and fewer
+// epilogue warps draw less power.  A call of few tokens pays for a pair's 256-row tiles and its
+// start (V = 32,379, single blocks / pairs): d = 320, 286 tokens 17.8 / 25.2, 2,000 47.8 / 48.2, 5,000 115 / 109; d = 512, 1,000 tokens
+// 32.7 / 32.8, 2,000 66.2 / 58.9, 5,000 159 / 145.
+constexpr int PAIR_MIN_WIDTH = 320, PAIR_ALWAYS_WIDTH = 513, EIGHT_WARPS_MAX_WIDTH = 896;
+constexpr int64_t PAIR_MIN_WORK = 800000;      // T_max d, for widths in between
+bool pair_for(const arrol_ctx* ctx, int64_t T_max, int d) {
     if (ctx->sm_count < 2 || ctx->logprob_pair == 0) return false;
-    return ctx->logprob_pair == 1 || d >= PAIR_MIN_WIDTH;
+    return ctx->logprob_pair == 1 || d >= PAIR_ALWAYS_WIDTH || (d >= PAIR_MIN_WIDTH && T_max >= (PAIR_MIN_WORK + d - 1) / d);
 }
 int halves_for(int d) { return d <= EIGHT_WARPS_MAX_WIDTH ? 2 : 1; }
 
 VocabPlan plan_for(const arrol_ctx* ctx, int d, int V) {
     VocabPlan v;
     v.total_chunks = (V + BN - 1) / BN;
-    v.splits = splits_for(ctx, d, V, pair_for(ctx, d));
+    // the same for every token count: where the form depends on that, both forms' resident tiles are far below either budget
+    v.splits = splits_for(ctx, d, V, pair_for(ctx, INT64_MAX, d));
     // one segment per SM: then the tail's items fill the units (SMs, or half as many pairs) a whole number of times
     v.n_sub = v.total_chunks < ctx->sm_count ? v.total_chunks : ctx->sm_count;
     v.n_long = v.total_chunks % v.n_sub;
@@ -772,7 +790,7 @@ extern "C" size_t arrol_token_logprob_workspace(arrol_ctx* ctx, int64_t T_max, i
 
 extern "C" int32_t arrol_token_logprob_form(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
     if (!ctx || T_max <= 0 || d <= 0 || V <= 0) return 0;
-    return pair_for(ctx, d) ? 2 : 1;
+    return pair_for(ctx, T_max, d) ? 2 : 1;
 }
 
 extern "C" int32_t arrol_token_logprob_splits(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V) {
@@ -823,7 +841,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         map_s = map_h;
     }
     // pair variant (clusters of two blocks): every block loads half of a chunk's W_vocab rows
-    const bool pair = pair_for(ctx, d);
+    const bool pair = pair_for(ctx, T_max, d);
     if (make_map(ctx, &map_w, W_vocab, (uint64_t)V, (uint64_t)d, pair ? PAIR_B_ROWS : BN) != ARROL_OK) return ARROL_ERR_CUDA;
 
     LogprobParams p;

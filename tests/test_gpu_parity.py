@@ -670,3 +670,31 @@ def test_logprob_calls_of_several_waves_in_flight_on_two_streams(ctx, d):
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
     for i in range(2):
         assert all(torch.equal(a, b) for a, b in zip(calls[i][3:5], want[i]))
+
+
+# the widths and token counts where the form of the kernel changes: single blocks on one side, pairs on the other, the same bits
+@pytest.mark.parametrize("T,d,form", [(4000, 312, 1), (2500, 320, 2), (2499, 320, 1), (1563, 512, 2), (1562, 512, 1), (300, 520, 2)])
+def test_logprob_forms_give_the_same_bits_where_they_meet(T, d, form):
+    V = 3001
+    ctx = B.Context(0)
+    assert B.arrol_token_logprob_form(ctx, T, d, V) == form
+    g = np.random.default_rng(T + d)
+    H = torch.from_numpy(g.normal(size=(T, d)).astype(np.float32)).to(torch.bfloat16).cuda()
+    W = torch.from_numpy(g.normal(0, 0.05, size=(V, d)).astype(np.float32)).to(torch.bfloat16).cuda()
+    y = dev(g.integers(0, V, size=T).astype(np.int32))
+    outs = []
+    for hook in (2, 0, 1):
+        B.arrol_test_hook(ctx, B.HOOK_LOGPROB_PAIR, hook)
+        ws = torch.empty(B.arrol_token_logprob_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+        lp, lse = torch.empty(T, device="cuda"), torch.empty(T, device="cuda")
+        B.arrol_token_logprob(ctx, H, W, y, T, d, V, lp, ws, lse=lse)
+        torch.cuda.synchronize()
+        outs.append((lp, lse))
+    assert all(torch.equal(a, b) for o in outs[1:] for a, b in zip(outs[0], o))
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("d", [256])                     # single blocks
+def test_logprob_calls_of_single_blocks_in_flight_on_two_streams(ctx, d):
+    test_logprob_calls_of_several_waves_in_flight_on_two_streams(ctx, d)
