@@ -72,8 +72,8 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 // (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
 // that one block scan ranks all of them, and the bisection is settled in three rounds of 31 points (see below) instead of 64
 // steps.  Per call, in a graph of 20 (with six rounds, separate round trips for mask, bin and reward, and a later one for
-// the evicted entries before): N = 2,048, 128 bins 25.6 -> 17.4 us; N = 32, 64 bins 21.1 -> 14.4; N = 8,192, 256 bins 34.9 -> 24.1; 13 of
-// the 17 us are the search.  More rollouts go through shared memory in pieces of CAL_STAGED,
+// the evicted entries before): N = 2,048, 128 bins 25.6 -> 15.9 us; N = 32, 64 bins 21.1 -> 12.9; N = 8,192, 256 bins 34.9 -> 23.0; 12 of
+// the 16 us are the search.  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
 // per thread and scan, as it was before the runs, 460 and 1,570).  An instance each, because the pieces' code in the same one cost

@@ -140,10 +140,10 @@ def test_lm_head_backward_with_groups_of_tiles(ctx, d):
 
 
 # tiles that are cut: all of dH along K, with a last column tile of half width (600) or one column tile and dead rows (900); 10 tiles
-# beyond a whole wave of 74 along K (7,000); 37 tiles in halves of their columns, without room for partial sums (9,472); vocabulary
-# chunks in halves, the last one with nothing in its second half (600, 257)
+# beyond a whole wave of 74 along K (7,000); 37 tiles without room for partial sums (9,472); a second chunk whose tiles are cut while
+# dW is added to (9,900)
 @pytest.mark.parametrize("T,d,V,T_live", [(600, 320, 20000, None), (900, 72, 9001, 777), (7000, 768, 12000, None), (9472, 256, 700, None),
-                                          (257, 520, 5000, 256)])
+                                          (257, 520, 5000, 256), (9900, 136, 9001, 9800)])
 def test_lm_head_backward_with_cut_tiles(ctx, T, d, V, T_live):
     g = np.random.default_rng(T + d)
     n = T if T_live is None else T_live
