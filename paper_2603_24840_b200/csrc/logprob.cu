@@ -623,8 +623,13 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
 
 // Merges every token's records.  Tokens of the body: one thread each, splits x HALVES records.  Tokens of the tail: one
 // warp each; lane (block of segments, column half) merges its segments, then all lanes walk the blocks in order.
-constexpr int COMBINE_THREADS = 256;
-template <int HALVES>
+// AHEAD: a lane has all records of its block on their way before it merges the first (148 segments in 16 blocks are ten at most).
+// Where the tail has many tokens, and their blocks more segments than the other loop has in flight, the loads are what the kernel waits
+// for; elsewhere the loop without conditions is quicker (a step of a debugging size, one segment per block, 31.3 / 32.4 us):
+// V = 32,379, d = 320, whole call without / with it, 286 tokens 17.8 / 18.3 us, 1,500 41.8 / 36.6, 2,000 50.0 / 44.5; 3,000 and more the same.
+constexpr int COMBINE_THREADS = 256, COMBINE_AHEAD = 10;
+constexpr int64_t COMBINE_AHEAD_TOKENS = 1024;
+template <int HALVES, bool AHEAD>
 __global__ void __launch_bounds__(COMBINE_THREADS)
 combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
                       int64_t T_max, int V, VocabPlan plan, int tile_rows, int units, float* __restrict__ logp,
@@ -679,8 +684,20 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
             PartialLse mine = empty_record();
             if (b < plan.n_mid && lane < COMBINE_BLOCKS * HALVES) {
                 const int s1 = plan.sub_of_mid(b + 1);
+                if constexpr (AHEAD) {
+                    for (int s = plan.sub_of_mid(b); s < s1; s += COMBINE_AHEAD) {
+                        PartialLse r[COMBINE_AHEAD];
+#pragma unroll
+                        for (int k = 0; k < COMBINE_AHEAD; ++k)
+                            if (s + k < s1) r[k] = load(rec + (s + k) * HALVES + lane % HALVES);
+#pragma unroll
+                        for (int k = 0; k < COMBINE_AHEAD; ++k)
+                            if (s + k < s1) merge_record(mine, r[k]);
+                    }
+                } else {
 #pragma unroll 4
-                for (int s = plan.sub_of_mid(b); s < s1; ++s) merge_record(mine, load(rec + s * HALVES + lane % HALVES));
+                    for (int s = plan.sub_of_mid(b); s < s1; ++s) merge_record(mine, load(rec + s * HALVES + lane % HALVES));
+                }
             }
             const int in_base = min(COMBINE_BLOCKS, plan.n_mid - base);
 #pragma unroll 4
@@ -949,7 +966,9 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     const int64_t tail_blocks = (tail_rows * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
     if (blocks < tail_blocks) blocks = tail_blocks;
     if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
-    ARROL_CUDA_OK(arrol_launch_pdl(halves == 2 ? combine_splits_kernel<2> : combine_splits_kernel<1>, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
+    const auto combine = T_max >= COMBINE_AHEAD_TOKENS && p.plan.n_sub > 4 * p.plan.n_mid ? (halves == 2 ? combine_splits_kernel<2, true> : combine_splits_kernel<1, true>)
+                                                       : (halves == 2 ? combine_splits_kernel<2, false> : combine_splits_kernel<1, false>);
+    ARROL_CUDA_OK(arrol_launch_pdl(combine, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
                                    static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
                                    T_max, V, p.plan, (int)tile_rows, (int)units, logp, lse, conf, inv_temperature, ctx->d_status));
     ctx->launches += 1;
