@@ -18,7 +18,7 @@ struct arrol_ctx {
     uint32_t* d_tile_counters; // MLP head on the tensor cores: finished blocks per row tile, zero between calls
     void* d_pack;              // MLP head on the tensor cores: the scored rows packed as bf16 [N][d], ARROL_PACK_BYTES
     uint32_t* d_head_counters; // head training step: finished runs per column tile, zero between calls
-    unsigned long long* d_chain;   // fused prune step: finished blocks, index-check flag, per-block totals; zero between calls
+    unsigned long long* d_chain;   // fused prune step: finished blocks (and failed index checks), per-block totals; zero between calls
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
     int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
     bool head_dw1_smem_set[2]; // likewise for the head training step's contraction (column tiles of 64, 128)

@@ -149,6 +149,59 @@ def test_fused_prune_step_over_group_shapes(P, G, K):
     pr.ctx.close()
 
 
+ROLLOUT_OUT, SURVIVOR_OUT, TOKEN_OUT = ("score", "prob", "q", "bin", "keep"), ("survivor_idx", "adv"), ("dst_tokens", "tok_adv", "tok_seq")
+
+
+def _snapshot(pr):
+    return {k: getattr(pr, k).clone() for k in ROLLOUT_OUT + SURVIVOR_OUT + TOKEN_OUT + ("cu_seqlens", "d_num")}
+
+
+def _clear(pr):
+    for k in ROLLOUT_OUT + SURVIVOR_OUT + TOKEN_OUT + ("cu_seqlens", "d_num"):
+        getattr(pr, k).fill_(0)
+
+
+def _assert_equals(pr, want):
+    """Everything that a call writes: what lies past the survivors and their tokens belongs to nobody."""
+    S, T = (int(x) for x in want["d_num"].cpu())
+    assert pr.counts() == (S, T)
+    for k in ROLLOUT_OUT:
+        assert torch.equal(getattr(pr, k), want[k]), k
+    for k in SURVIVOR_OUT:
+        assert torch.equal(getattr(pr, k)[:S], want[k][:S]), k
+    assert torch.equal(pr.cu_seqlens[:S + 1], want["cu_seqlens"][:S + 1])
+    for k in TOKEN_OUT:
+        assert torch.equal(getattr(pr, k)[:T], want[k][:T]), k
+
+
+def test_fused_prune_steps_of_changing_size_on_one_context():
+    """The blocks of a call find each other's totals in the context's chain.  Calls of 1 to 290 blocks (the last one: an MLP
+    head, blocks of two warps) follow one another on one context without a host synchronisation: whatever a call leaves
+    there must not be taken for a later and larger call's totals."""
+    import dataclasses
+    import random
+    ctx = B.Context(0)
+    states = []
+    for P, h in ((1, 0), (2, 0), (40, 0), (300, 0), (580, 0), (450, 24)):
+        w = dataclasses.replace(synth.WORKLOADS["mini"], P=P, G=16, K=8, h=h, seed=P)
+        pr = PruneRebatch(w, inputs=host_inputs(w), with_rows=False, ctx=ctx)
+        pr.prune_step(with_rows=False)
+        torch.cuda.synchronize()
+        states.append((pr, pr.prune_step_args(with_rows=False), _snapshot(pr)))
+    rng = random.Random(3)
+    for _ in range(20):
+        for pr, _, _ in states:
+            _clear(pr)
+        order = [rng.randrange(len(states)) for _ in range(40)] + rng.sample(range(len(states)), len(states))
+        for i in order:
+            B.arrol_prune_step(ctx, states[i][1])
+        torch.cuda.synchronize()
+        for pr, _, want in states:
+            _assert_equals(pr, want)
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+    ctx.close()
+
+
 # rows past the 4 KB that a warp holds in registers: one vector more (2,056 bf16, 1,032 fp32), twice as many, a block of few warps, and
 # rows too long to be staged for a block of 32 of them
 @pytest.mark.parametrize("P,G,K,d,dtype", [(9, 16, 8, 2056, "bf16"), (150, 16, 8, 4096, "bf16"), (1, 3, 1, 3000, "bf16"),
