@@ -171,6 +171,7 @@ prune_fused_kernel(const FusedParams p) {
             g_den[lane] = den;
         }
         __threadfence_block();
+        __syncwarp();                                        // the named barriers want their warps converged
         asm volatile("bar.arrive 1, 64;" ::: "memory");
         // The block is done with the chain when the first warp has published its totals and read the others'.  The count's release is what
         // the clearing rests on: every block's stores have been performed before the last one to be counted zeroes the
