@@ -49,7 +49,7 @@ typedef enum {
 /* Device status bits accumulated in the context's status word (see arrol_poll_status). */
 #define ARROL_DEV_CAPACITY 1u      /* arrol_compact: T > dst_capacity_tokens, nothing was gathered */
 #define ARROL_DEV_BAD_TARGET 2u    /* arrol_token_logprob: a target id >= V (its logp is set to 0) */
-#define ARROL_DEV_WAIT_EXPIRED 4u  /* arrol_token_logprob: a pipeline wait hit its iteration limit */
+#define ARROL_DEV_WAIT_EXPIRED 4u  /* a wait inside a kernel hit its iteration limit; arrol_prune_step then reports {0, 0} survivors, tokens */
 #define ARROL_DEV_BAD_STATE 8u     /* arrol_calib_update: the state's header does not match (B, cap); state untouched */
 #define ARROL_DEV_BAD_INDEX 16u    /* a source row outside the bound set with arrol_set_source_rows; access skipped */
 

@@ -53,14 +53,14 @@ struct FusedParams {
     int64_t* d_num;
     uint32_t* d_status;
     // chained scan: word [0] blocks that are done with it, from LEFT_ONE on those of which a kept rollout left the source (index
-    // check), then from [2] per block {kept tokens, kept rollouts}, each with bit 63 set once published; all zero between calls
+    // check), from EXPIRED_ONE on those that waited in vain; then from [2] per block {kept tokens, kept rollouts}, each with bit 63 set once published; all zero between calls
     unsigned long long* chain;
     uint32_t spin_limit;
     int rest_vecs;             // 16-byte vectors of a row past the first 256 that a warp has room for in shared memory: all of them, or 0
 };
 
 constexpr int LUT_STAGED = 1024;
-constexpr unsigned long long PUBLISHED = 1ull << 63, LEFT_ONE = 1ull << 32;
+constexpr unsigned long long PUBLISHED = 1ull << 63, LEFT_ONE = 1ull << 32, EXPIRED_ONE = 1ull << 48;     // at most ARROL_CHAIN_BLOCKS of either
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
     unsigned long long v;
@@ -84,7 +84,7 @@ prune_fused_kernel(const FusedParams p) {
     __shared__ float q_s[32], rew_s[32];
     __shared__ uint8_t keep_s[32];
     __shared__ int32_t len_s[32];
-    __shared__ bool block_left;                              // a kept rollout of this block leaves the source
+    __shared__ bool block_left, block_expired;               // a kept rollout of this block leaves the source; a wait ran out
     __shared__ double inv_count[SCAN_INV], g_mean[32], g_den[32];
     __shared__ float lut_s[LUT_STAGED];                      // the posterior table, or its first use would be one more round trip
     extern __shared__ uint4 w_stage[];                       // linear head: the weights, d * sizeof(T) bytes
@@ -182,14 +182,19 @@ prune_fused_kernel(const FusedParams p) {
         // after an MLP head 70.4 / 70.6 / 70.0, 32 rollouts 9.4 / 10.3 / 9.9.
         asm volatile("bar.sync 2, 64;" ::: "memory");
         unsigned long long done = 0;
-        if (lane == 0) done = count_acq_rel(p.chain, block_left ? 1ull + LEFT_ONE : 1ull);
+        if (lane == 0) done = count_acq_rel(p.chain, 1ull + (block_left ? LEFT_ONE : 0ull) + (block_expired ? EXPIRED_ONE : 0ull));
         done = __shfl_sync(0xffffffffu, done, 0);
         if ((done & (LEFT_ONE - 1)) == gridDim.x - 1) {
             for (unsigned int b = lane; b < 2 * gridDim.x; b += 32) totals[b] = 0ull;
             if (lane == 0) {
-                const bool left = block_left || done >= LEFT_ONE;
+                const bool left = block_left || done % EXPIRED_ONE >= LEFT_ONE, expired = block_expired || done >= EXPIRED_ONE;
                 if (left) atomicOr(p.d_status, ARROL_DEV_BAD_INDEX);
-                p.d_status[1] = left ? 1u : 0u;      // gate word: the gather kernels of this call copy nothing when set
+                if (expired) {                       // the survivors' list has holes: nobody is to follow it
+                    atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
+                    p.d_num[0] = 0;
+                    p.d_num[1] = 0;
+                }
+                p.d_status[1] = left || expired ? 1u : 0u;      // gate word: the gather kernels of this call copy nothing when set
                 p.chain[0] = 0ull;
             }
         }
@@ -242,8 +247,13 @@ prune_fused_kernel(const FusedParams p) {
     const bool any_bad = __any_sync(0xffffffffu, bad_index);
     const bool any_expired = __any_sync(0xffffffffu, expired);
     if (lane == 0) {
-        if (any_expired) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
         block_left = any_bad;
+        block_expired = any_expired;
+        if (blockIdx.x == gridDim.x - 1) {                   // before the block is counted: the last one may take it back
+            p.d_num[0] = base_c + block_c;
+            p.d_num[1] = base_t + block_t;
+            if (base_t + block_t > p.capacity) atomicOr(p.d_status, ARROL_DEV_CAPACITY);
+        }
     }
     __syncwarp();
     asm volatile("bar.arrive 2, 64;" ::: "memory");          // done with the chain
@@ -256,11 +266,6 @@ prune_fused_kernel(const FusedParams p) {
         p.adv[pos] = (float)(((double)rew_s[lane] - g_mean[g]) * g_den[g]);      // den holds 1 / (std + eps), or 0
     }
     if (blockIdx.x == 0 && lane == 0) p.cu_seqlens[0] = 0;
-    if (blockIdx.x == gridDim.x - 1 && lane == 0) {
-        p.d_num[0] = base_c + block_c;
-        p.d_num[1] = base_t + block_t;
-        if (base_t + block_t > p.capacity) atomicOr(p.d_status, ARROL_DEV_CAPACITY);
-    }
 }
 
 }  // namespace

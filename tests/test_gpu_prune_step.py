@@ -202,6 +202,36 @@ def test_fused_prune_steps_of_changing_size_on_one_context():
     ctx.close()
 
 
+def test_an_expired_wait_of_the_fused_prune_step_leaves_nothing_to_follow():
+    """A block that gives up waiting for the totals before it leaves holes in the survivors' list.  The call reports it, as
+    {0, 0} survivors and tokens, gathers nothing, and leaves nothing behind for the next call."""
+    import dataclasses
+    w = dataclasses.replace(synth.WORKLOADS["mini"], P=580, G=16, K=8, h=0, seed=12)
+    pr = PruneRebatch(w, inputs=host_inputs(w), with_rows=False)
+    args = pr.prune_step_args(with_rows=False)
+    pr.prune_step(with_rows=False)
+    torch.cuda.synchronize()
+    want = _snapshot(pr)
+    expired = 0
+    for _ in range(8):
+        _clear(pr)
+        B.arrol_test_hook(pr.ctx, B.HOOK_SPIN_LIMIT, 1)          # one look at every total
+        B.arrol_prune_step(pr.ctx, args)
+        torch.cuda.synchronize()
+        if B.arrol_poll_status(pr.ctx, raise_on_error=False) & B.DEV_WAIT_EXPIRED:
+            expired += 1
+            assert pr.counts() == (0, 0)
+            assert all(int(getattr(pr, k).abs().max()) == 0 for k in TOKEN_OUT)
+        B.arrol_test_hook(pr.ctx, B.HOOK_SPIN_LIMIT, 0)
+        _clear(pr)
+        B.arrol_prune_step(pr.ctx, args)
+        torch.cuda.synchronize()
+        _assert_equals(pr, want)
+    assert expired > 0
+    assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == 0
+    pr.ctx.close()
+
+
 # rows past the 4 KB that a warp holds in registers: one vector more (2,056 bf16, 1,032 fp32), twice as many, a block of few warps, and
 # rows too long to be staged for a block of 32 of them
 @pytest.mark.parametrize("P,G,K,d,dtype", [(9, 16, 8, 2056, "bf16"), (150, 16, 8, 4096, "bf16"), (1, 3, 1, 3000, "bf16"),
