@@ -235,6 +235,14 @@ def arrol_build_q_lut(cpos, cneg, alpha: float = 1.0):
 _HEAD_TENSORS = ("W1", "b1", "w2", "b2")
 
 
+def _check_head(hidden: torch.Tensor, head: dict):
+    dtype = hidden.dtype
+    for name in _HEAD_TENSORS:
+        t = head.get(name)
+        if t is not None and t.dtype != dtype:
+            raise TypeError("head tensors share the hidden dtype")
+
+
 def _head_struct(hidden_dtype_code: int, d: int, head: dict) -> _Head:
     return _Head(int(d), int(head.get("h", 0)), hidden_dtype_code, 0, *[_ptr(head.get(name)) for name in _HEAD_TENSORS])
 
@@ -248,11 +256,7 @@ def arrol_score_partial(ctx: Context, hidden: torch.Tensor, head: dict, N: int, 
                         row_index: Optional[torch.Tensor] = None, q_lut: Optional[torch.Tensor] = None,
                         row_stride: Optional[int] = None, stream=None):
     """head = {"W1", "b1", "w2", "b2", "h"} (device tensors or None).  Outputs are written in place."""
-    dtype = hidden.dtype
-    for name in _HEAD_TENSORS:
-        t = head.get(name)
-        if t is not None and t.dtype != dtype:
-            raise TypeError("head tensors share the hidden dtype")
+    _check_head(hidden, head)
     hs = _head_struct(_dtype_code(hidden), hidden.shape[-1], head)
     cs = _calib_struct(q_lut)
     stride = hidden.stride(-2) if row_stride is None else int(row_stride)
@@ -379,6 +383,7 @@ def make_prune_step(hidden: torch.Tensor, head: dict, q_lut: Optional[torch.Tens
                     row_stride: Optional[int] = None) -> _PruneStep:
     """Argument block of arrol_prune_step.  scalars: P, G, K, rho, eps, ddof, dst_capacity_tokens, row_bytes;
     tensors: the device tensors by field name (missing / None = NULL).  The caller keeps the tensors alive."""
+    _check_head(hidden, head)
     a = _PruneStep()
     a.hidden = hidden.data_ptr()
     a.row_stride_elems = hidden.stride(-2) if row_stride is None else int(row_stride)
