@@ -623,12 +623,14 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
 
 // Merges every token's records.  Tokens of the body: one thread each, splits x HALVES records.  Tokens of the tail: one
 // warp each; lane (block of segments, column half) merges its segments, then all lanes walk the blocks in order.
-// AHEAD: a lane has all records of its block on their way before it merges the first (148 segments in 16 blocks are ten at most).
-// Where the tail has many tokens, and their blocks more segments than the other loop has in flight, the loads are what the kernel waits
-// for; elsewhere the loop without conditions is quicker (a step of a debugging size, one segment per block, 31.3 / 32.4 us):
-// V = 32,379, d = 320, whole call without / with it, 286 tokens 17.8 / 18.3 us, 1,500 41.8 / 36.6, 2,000 50.0 / 44.5; 3,000 and more the same.
+// AHEAD: a lane has all records of its block on their way before it merges the first (148 segments in 16 blocks are ten at most).  It
+// takes 102 registers where the other loop takes 60, and that is what counts: one block waits on every SM beside the log-prob
+// kernel, and of those past them (a warp merges a token) up to three more go to the SM that is free first, whose 32 warps then merge
+// one another out of the way; of AHEAD's only one.  So it is taken where the tail has more blocks than that, and no more than two an SM, past
+// which they take a wave more.  Whole call without / with it, d = 256, V = 6,000 (us): 148 blocks (1,184 tokens) 14.3 / 15.0, 149
+// 14.7 / 14.9, 150 15.8 / 15.0, 151 17.1 / 14.9, 256 19.9 / 17.8, 296 21.6 / 20.0, 297 21.7 / 22.7, 5,000 tokens 31.3 / 35.0; V = 32,379: 1,280 tokens
+// 35.7 / 32.1, 2,048 46.8 / 43.4, 2,500 54.8 / 55.6, 5,000 95.4 / 98.0.  T_max draws the line: 300 live tokens of 2,048 at V = 16,640 14.4 / 15.1.
 constexpr int COMBINE_THREADS = 256, COMBINE_AHEAD = 10;
-constexpr int64_t COMBINE_AHEAD_TOKENS = 1024;
 template <int HALVES, bool AHEAD>
 __global__ void __launch_bounds__(COMBINE_THREADS)
 combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
@@ -966,8 +968,10 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     const int64_t tail_blocks = (tail_rows * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
     if (blocks < tail_blocks) blocks = tail_blocks;
     if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
-    const auto combine = T_max >= COMBINE_AHEAD_TOKENS && p.plan.n_sub > 4 * p.plan.n_mid ? (halves == 2 ? combine_splits_kernel<2, true> : combine_splits_kernel<1, true>)
-                                                       : (halves == 2 ? combine_splits_kernel<2, false> : combine_splits_kernel<1, false>);
+    const int64_t token_blocks = ((T_max < tail_rows ? T_max : tail_rows) * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
+    const bool ahead = token_blocks > ctx->sm_count + 1 && token_blocks <= 2 * (int64_t)ctx->sm_count;
+    const auto combine = ahead ? (halves == 2 ? combine_splits_kernel<2, true> : combine_splits_kernel<1, true>)
+                               : (halves == 2 ? combine_splits_kernel<2, false> : combine_splits_kernel<1, false>);
     ARROL_CUDA_OK(arrol_launch_pdl(combine, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
                                    static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
                                    T_max, V, p.plan, (int)tile_rows, (int)units, logp, lse, conf, inv_temperature, ctx->d_status));

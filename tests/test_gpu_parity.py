@@ -628,6 +628,32 @@ def test_logprob_bits_do_not_depend_on_the_token_count(V, d, pair):
     ctx.close()
 
 
+# the token counts where the combining kernel changes: 149 and 150 blocks of 8 tokens, 296 and 297; one to ten segments a lane
+@pytest.mark.parametrize("V,d", [(700, 72), (4096, 72), (12000, 904), (40000, 72)])
+def test_logprob_bits_on_both_sides_of_the_combining_kernels(ctx, V, d):
+    g = np.random.default_rng(V + 1)
+    T_max = 2400
+    H = torch.from_numpy(g.normal(size=(T_max, d)).astype(np.float32)).to(torch.bfloat16)
+    W = torch.from_numpy(g.normal(0, 0.8 / d ** 0.5, size=(V, d)).astype(np.float32)).to(torch.bfloat16)
+    y = g.integers(0, V, size=T_max).astype(np.int32)
+    Hd, Wd, yd = H.cuda(), W.cuda(), dev(y)
+    full = None
+    for T, live in ((2400, 2400), (2369, 2369), (2368, 2368), (2368, 300), (1193, 1193), (1192, 1192), (600, 600)):
+        ws = torch.empty(B.arrol_token_logprob_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+        lp, lse = torch.full((T,), 7.0, device="cuda"), torch.full((T,), 7.0, device="cuda")
+        B.arrol_token_logprob(ctx, Hd, Wd, yd, T, d, V, lp, ws, lse=lse, d_T=torch.tensor([live], dtype=torch.int64, device="cuda"))
+        torch.cuda.synchronize()
+        if full is None:
+            full = (lp, lse)
+        assert torch.equal(lp[:live], full[0][:live]) and torch.equal(lse[:live], full[1][:live])
+        assert bool((lp[live:] == 7.0).all())
+    rows = np.unique(np.concatenate([[0, 1191, 1192, 2367, 2368, 2399], g.integers(0, T_max, size=20)])).astype(np.int64)
+    lp_ref, lse_ref = oracle.token_logprob(synth.as_oracle_array(H), synth.as_oracle_array(W), y, rows=rows)
+    assert np.abs(full[0].cpu().numpy()[rows] - lp_ref).max() <= LOGP_TOL
+    assert np.abs(full[1].cpu().numpy()[rows] - lse_ref).max() <= LOGP_TOL
+    assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
+
+
 # one segment longer than the others, half of them, all but one; single blocks and pairs
 @pytest.mark.parametrize("d", [72, 520])
 @pytest.mark.parametrize("V", [148 * 256 + 1, 222 * 256, 296 * 256 - 255 - 1, 2 * 148 * 256 + 7])
