@@ -8,6 +8,8 @@ from paper_2603_24840_b200.pipeline import PruneRebatch, host_inputs
 
 pytestmark = pytest.mark.gpu
 
+BAD_INDEX = 16
+
 
 @pytest.mark.parametrize("name,rows", [("tiny", True), ("mini", True), ("mini", False), ("profile-mlp", True)])
 def test_one_call_prune_step_equals_three_calls(name, rows):
@@ -242,13 +244,30 @@ def test_fused_prune_step_on_wide_rows(P, G, K, d, dtype):
     pr = PruneRebatch(w, inputs=host_inputs(w), with_rows=False)
     pr.prune_step(with_rows=False)
     torch.cuda.synchronize()
-    keys = ("score", "prob", "q", "bin", "keep", "d_num")
-    want = {k: getattr(pr, k).clone() for k in keys}
-    for k in keys:
-        getattr(pr, k).fill_(0)
+    want = _snapshot(pr)
+    _clear(pr)
     B.arrol_prune_step(pr.ctx, pr.prune_step_args(with_rows=False))
     torch.cuda.synchronize()
-    for k in keys:
-        assert torch.equal(getattr(pr, k), want[k]), k
+    _assert_equals(pr, want)
     assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == 0
+    pr.ctx.close()
+
+
+def test_fused_prune_step_on_wide_rows_checks_their_numbers():
+    """Rows that go through shared memory (d = 4,096): numbers outside the source are reported and scored as zeros, as by the
+    three calls, and their rows are not asked for."""
+    import dataclasses
+    w = dataclasses.replace(synth.WORKLOADS["mini"], P=20, G=16, K=8, h=0, d=4096, seed=41)
+    pr = PruneRebatch(w, inputs=host_inputs(w), with_rows=False)
+    pr.row_index[5], pr.row_index[100], pr.row_index[319] = pr.T_src, -1, 1 << 40
+    B.arrol_set_source_rows(pr.ctx, pr.T_src)
+    pr.prune_step(with_rows=False)
+    torch.cuda.synchronize()
+    assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == BAD_INDEX
+    want = _snapshot(pr)
+    _clear(pr)
+    B.arrol_prune_step(pr.ctx, pr.prune_step_args(with_rows=False))
+    torch.cuda.synchronize()
+    _assert_equals(pr, want)
+    assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == BAD_INDEX
     pr.ctx.close()
