@@ -165,7 +165,10 @@ size_t arrol_token_logprob_workspace(arrol_ctx* ctx, int64_t T_max, int32_t d, i
 int32_t arrol_token_logprob_splits(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V);
 /* Form of the kernel for these sizes: 2 = pairs of thread blocks on 256-row token tiles (tcgen05 cta_group::2), 1 = one
  * block per 128-row tile.  Pairs are used for hidden widths above 512 and, where T_max d >= 800,000, from 320; see
- * ARROL_HOOK_LOGPROB_PAIR.  0 for invalid arguments. */
+ * ARROL_HOOK_LOGPROB_PAIR.  0 for invalid arguments.
+ * The capacity T_max decides, not the live tokens, which only the device knows: between 320 and 512 a generous capacity with
+ * few hundred live tokens pays for 256-row tiles (d = 320, V = 151,936, T_max = 2,500: 625 live 64.8 us, as single blocks 55.7; 1,250
+ * live 100.6, 102.0).  Results do not depend on it. */
 int32_t arrol_token_logprob_form(arrol_ctx* ctx, int64_t T_max, int32_t d, int32_t V);
 int arrol_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_vocab, const int32_t* targets,
                         int64_t T_max, const int64_t* d_T, int32_t d, int32_t V, float inv_temperature,

@@ -583,7 +583,10 @@ __device__ __forceinline__ bool gemm_item(int64_t i, int m_tiles, int n_tiles, i
 // tile, the tile as the fast index, so that the pairs that work at the same time share operand panels.  (A column tile of half the
 // width counts like the others: a K step takes the issuing warp about 500 cycles whatever the MMAs' width.)
 constexpr int MIN_SEG = 16;              // K steps of a range at least: an epoch of the lock-step
-constexpr int SEG_COST = 12;             // K steps that a wave of ranges costs beside its own (writing and adding 256 KB a pair)
+// K steps that a wave of ranges costs beside its own (writing and adding 256 KB a pair).  Policy loss and backward with 0 / 12 / 40 (us): d = 320,
+// V = 8,192, 2,500 tokens 71 / 68 / 68, 5,000 127 / 113 / 124; d = 1,024, 1,200 78 / 72 / 72, 2,500 124 / 112 / 123; d = 320, V = 30,000, 1,200
+// 113 / 101 / 101, 4,700 320 / 320 / 324, and the one shape found where it is not the best, 2,400 180 / 185 / 181.
+constexpr int SEG_COST = 12;
 struct GemmWork {
     int m_tiles, n_tiles, group_n, k_steps;
     int body, tail, segs, items;         // tiles, tail tiles, ranges of K per tail tile
@@ -780,7 +783,10 @@ int group_columns(int n_tiles) {          // column tiles per group: at most 10 
     return (n_tiles + groups - 1) / groups;
 }
 
-// As many pairs as fit the GPU at once: those without a tile of their own take part of another's.
+// As many pairs as fit the GPU at once, whatever the work: in the dH kernel those without a tile of their own take part of another's, and in
+// the dW kernel all of them add the partial sums.  Grids cut to the pairs with work do not leave more to a launch on another stream
+// (two calls on one stream / two, us a call, all pairs and cut ones: T = 200, d = 256, V = 4,096 27.8 / 14.3, 29.8 / 15.2; 600, 512, 4,096 32.1 / 21.1,
+// 33.9 / 20.4; 1,000, 256, 8,000 36.7 / 26.2, 36.4 / 25.8).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pairs(arrol_ctx* ctx, int which, void (*kernel)(KArgs...), cudaStream_t s, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
@@ -869,8 +875,10 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     uint16_t* Htail = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + L.tail);
     unsigned int* lock_words = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + L.lock);
     // The dz kernel's counter has to be zero before the first chunk (the later ones are zeroed by the kernels).  Clearing it costs a
-    // call about 2 us and keeps the dz kernel's start from overlapping the end of the kernel before it, so calls of which a pair has
-    // few tiles do without the step: they are over before pairs drift apart.
+    // call 4 to 5 us, most of it because the dz kernel's start no longer overlaps the end of the kernel before it, so calls of which a pair
+    // has few tiles do without the step: they are over before pairs drift apart.  Policy loss and backward, in step / not: d = 512, V = 20,000,
+    // 1,500 tokens (6.4 tiles a pair) 101 / 95 us, 2,048 (8.5) 123 / 118, 5,000 (21) 273 / 269; d = 2,048, V = 12,000, 3,072 (7.6) 322 / 319, 6,144 (15)
+    // 615 / 612.  So at the line the step is not yet worth its clearing; it stays well below the launches that drift.
     const bool first_in_step = (T_max + TILE_ROWS - 1) / TILE_ROWS * ((V + BN - 1) / BN) > (int64_t)FREE_TILES * (ctx->sm_count / 2);
     if (first_in_step) ARROL_CUDA_OK(cudaMemsetAsync(lock_words, 0, LOCK_BYTES, s));
     if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;

@@ -748,7 +748,7 @@ int splits_for(const arrol_ctx* ctx, int d, int V, bool pair) {
 }
 
 // The form of the kernel for these sizes (V = 61,125, 100,000 tokens; us as single blocks and as pairs, eight epilogue warps up to
-// 768, four beyond):
+// 896, four beyond):
 //   d = 256   2,865 / 2,850    d = 320 (20,000 tokens, V = 40,000)  456 / 425    d = 384   3,757 / 3,530    d = 512   4,710 / 4,290
 //   d = 768 (four / eight warps)  7,140 / 7,242, pairs 6,954 / 6,653             d = 1,024 9,376 / 8,798
 //   d = 4,096 (V = 151,936, 287,000 tokens): single blocks with two splits 250.6 ms, pairs with four 247.9 ms
@@ -757,7 +757,9 @@ int splits_for(const arrol_ctx* ctx, int d, int V, bool pair) {
 // hand an accumulator back without waiting for a peer's epilogue.  At larger d pairs move fewer operand bytes, and fewer
 // epilogue warps draw less power.  A call of few tokens pays for a pair's 256-row tiles and its
 // start (V = 32,379, single blocks / pairs): d = 320, 286 tokens 17.8 / 25.2, 2,000 47.8 / 48.2, 5,000 115 / 109; d = 512, 1,000 tokens
-// 32.7 / 32.8, 2,000 66.2 / 58.9, 5,000 159 / 145.
+// 32.7 / 32.8, 2,000 66.2 / 58.9, 5,000 159 / 145.  The line is drawn by T_max, the live tokens being on the device: with V = 151,936, capacities of
+// 2,500 and 5,000, a quarter / half / all of it live, d = 320: 56 / 65, 102 / 101, 195 / 190 and 102 / 101, 196 / 192, 389 / 368; d = 512:
+// 82 / 90, 150 / 140, 283 / 259 and 150 / 139, 287 / 263, 555 / 504.  What few tokens lose is the half tile at their end.
 constexpr int PAIR_MIN_WIDTH = 320, PAIR_ALWAYS_WIDTH = 513, EIGHT_WARPS_MAX_WIDTH = 896;
 constexpr int64_t PAIR_MIN_WORK = 800000;      // T_max d, for widths in between
 bool pair_for(const arrol_ctx* ctx, int64_t T_max, int d) {
