@@ -25,6 +25,7 @@ struct arrol_ctx {
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool prune_smem_set;       // likewise for the fused prune step
+    int score_max_clusters[9]; // scoring kernel: clusters of so many blocks of 64 hidden units that are resident at once; 0 = not asked yet
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
     uint32_t test_spin_limit;  // arrol_test_hook: tries per pipeline wait of the log-prob kernel, 0 = the normal limit

@@ -9,17 +9,27 @@
 //                         load/store path holds about 20 KB in flight per SM against the ring's 192 KB by TMA, and
 //                         every block of a row tile fetches the same rows: 18.5 us per call against 14.6 us.)
 //   score_mlp_tc_kernel   one block per (128 rollouts x 64 or 128 hidden units); shared memory is one ring of stages
-//                         (128 x 64 of X and the tile's 64 columns of W1 per K step of 64), filled by two TMA producer threads
-//                         on alternate K steps.  Two (tiles of 128) or four (64) issuing warps take the K steps round robin: one
+//                         (128 x 64 of X and the tile's 64 columns of W1 per K step of 64), filled by four TMA producer threads,
+//                         two for X and two for W1, on alternate K steps (one thread for all of W1 takes 300 cycles a step:
+//                         N = 2,048, d = 2,048, h = 256, rows in place 8.7 -> 12.6 us).  Two (tiles of 128) or four (64) issuing warps take the K steps round robin: one
 //                         warp's wait -> four MMAs -> commit round costs nearly 500 cycles, the MMAs of a 128 x 64 x 64 step
 //                         128, and a step's operands come in in about 290.  K step ks goes to accumulator ks mod 4.  The ring's
 //                         length is a multiple of the number of issuers, so that a stage always belongs to the same one: a parity
 //                         wait cannot tell a round from the one before the last.
 //                         Eight epilogue warps: thread = rollout x half of the tile's hidden units; accumulators added in
 //                         index order, then sum_j w2_j gelu(u_j + b1_j) over 32 units in index order, two such sums added
-//                         low + high -> partial[64-unit block][N], whatever the tile's width.  The last block of a row tile to
-//                         finish (a counter per row tile) adds the partial sums in index order, adds b2 and applies the
-//                         probability map, so the result does not depend on block order.
+//                         low + high -> a partial sum per 64 units and rollout, whatever the tile's width.
+//                         The blocks of a row tile are a cluster and put their partial sums into the first block's shared
+//                         memory, which adds them in index order, adds b2 and applies the probability map.  More than 1,024
+//                         hidden units are more than eight blocks of 128: there the partial sums go through global memory and
+//                         the last block to arrive (a counter per row tile) adds them.  The result does not depend on block
+//                         order, nor on which of the two it was.  Per call of 20 in a graph, partial sums through global memory ->
+//                         cluster: N = 2,048, d = 2,048, h = 256 13.5 -> 12.0 us (rows in place 10.3 -> 8.7); 4,096, 4,096, 512 29.1 ->
+//                         26.5; 394, 1,664, 256 10.8 -> 9.3; 32, 256, 64 7.1 -> 6.0.
+//   What the N = 2,048 call spends (in-kernel stamps, before): 0.7 us to the first stage, 3.7 for 32 K steps (192 KB in flight per
+//   SM and a copy's latency of 0.85 us), 1.6 of erff (45 instructions a unit and rollout), 2.2 in counting and adding up.
+//   Packing inside this kernel, each block of a cluster a share of the row tile and the contraction following chunk by chunk,
+//   was built and measured: 17.7 us, because every chunk's report waits 2 us for the stores before it.
 // Every wait is bounded; on expiry the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -37,7 +47,10 @@ constexpr int S_PRODUCER_WARPS = 4;          // warps before the issuers (two of
 constexpr int S_EPI_WARP0 = 8;               // a multiple of 4: epilogue warp w reads lane quarter w % 4
 constexpr int S_EPI_WARPS = 8;
 constexpr int S_THREADS = (S_EPI_WARP0 + S_EPI_WARPS) * 32;
-constexpr int S_TAIL_BYTES = 2560;           // barriers, tensor-memory slot, flags | b1, w2 of the tile | half sums
+constexpr uint32_t DRAIN_LIMIT = 1u << 16;   // tries per wait of a producer that gave up, for copies in flight
+constexpr int MAX_SUBS = 16;                 // partial sums of a row tile whose blocks form a cluster: 8 blocks of 128 hidden units
+// barriers, tensor-memory slot, flags | b1 and w2 of the tile, sums over a 64-unit tile's upper 32 hidden units | partial sums
+constexpr int S_TAIL_BYTES = 2048 + MAX_SUBS * 128 * 4;
 constexpr int TM = 128;                      // rollouts per tile (MMA M)
 constexpr int A_BYTES = TM * BK * 2;         // 16 KB
 // by tile width (hidden units, MMA N): 64 or 128
@@ -92,7 +105,8 @@ struct ScoreTcParams {
     uint32_t* d_status;
 };
 
-template <int SBN>
+// CLUSTER: the blocks of a row tile (gridDim.y of them, at most eight) are a cluster and finish the scores among themselves.
+template <int SBN, bool CLUSTER>
 __global__ void __launch_bounds__(S_THREADS, 1)
 score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                     const ScoreTcParams p) {
@@ -112,15 +126,16 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
     volatile uint32_t* abort_flag = tmem_slot + 1;
     volatile uint32_t* is_last = tmem_slot + 2;
-    float* b1_s = reinterpret_cast<float*>(tail + 256);          // [SBN]
-    float* w2_s = b1_s + SBN;                                    // [SBN]
-    float* half_s = reinterpret_cast<float*>(tail + 2048);       // [TM] sums over a 64-unit tile's upper 32 hidden units
+    float* b1_s = reinterpret_cast<float*>(tail + 512);          // [SBN]
+    float* w2_s = reinterpret_cast<float*>(tail + 1024);         // [SBN]
+    float* half_s = reinterpret_cast<float*>(tail + 1536);       // [TM] sums over a 64-unit tile's upper 32 hidden units
+    float* subs_s = reinterpret_cast<float*>(tail + 2048);       // [MAX_SUBS][TM] partial sums of the row tile (first block of a cluster)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * TM, j0 = blockIdx.y * SBN;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], 1); }
         mbar_init(acc_full, ISSUERS);
         *abort_flag = 0u;
         *is_last = 0u;
@@ -132,38 +147,36 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         tcgen05_alloc(tmem_slot, S_TMEM_COLS);
         tcgen05_relinquish();
     }
-    pdl_launch_dependents();
-    pdl_wait();                  // set-up above overlaps the previous kernel; global memory is read from here on
-    if (warp >= S_EPI_WARP0) {   // the tile's slice of b1 and w2, zero past h so that padded columns add nothing
-        const int e = threadIdx.x - S_EPI_WARP0 * 32;
-        if (e < SBN) {
-            const int j = j0 + e;
-            b1_s[e] = (j < p.h && p.b1) ? __bfloat162float(p.b1[j]) : 0.f;
-            w2_s[e] = (j < p.h) ? __bfloat162float(p.w2[j]) : 0.f;
-        }
-    }
     tcgen05_fence_before();
     __syncthreads();
+    if constexpr (CLUSTER) cluster_sync_all();      // the other blocks' barriers exist before anything arrives on them
     tcgen05_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_launch_dependents();
+    pdl_wait();                  // set-up above overlaps the previous kernel; global memory is read from here on
 
     // K step ks uses stage ks % STAGES in round ks / STAGES of the ring, issuer ks % ISSUERS and accumulator ks % S_ACCS.
     if (warp < S_PRODUCER_WARPS) {
-        if (lane == 0 && warp < S_PRODUCERS) {
+        if (lane == 0) {         // two threads for the rows, two for W1, on alternate K steps
+            const bool rows = warp < S_PRODUCERS;
             int last = -1;
             bool ok = true;
-            for (int ks = warp; ks < p.k_steps; ks += S_PRODUCERS) {
+            for (int ks = warp % S_PRODUCERS; ks < p.k_steps; ks += S_PRODUCERS) {
                 const int st = ks % STAGES;
                 const uint32_t round = (uint32_t)(ks / STAGES);
                 if (!mbar_wait(&empty[st], (round & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                mbar_expect_tx(&full[st], STAGE_BYTES);
-                tma_load_2d(stage_a + (size_t)st * A_BYTES, &map_x, ks * BK, m0, &full[st]);
-                tma_load_2d(stage_b + (size_t)st * SB_BYTES, &map_w, ks * BK, j0, &full[st]);
+                if (rows) {
+                    mbar_expect_tx(&full[st], A_BYTES);
+                    tma_load_2d(stage_a + (size_t)st * A_BYTES, &map_x, ks * BK, m0, &full[st]);
+                } else {
+                    mbar_expect_tx(&full[st], SB_BYTES);
+                    tma_load_2d(stage_b + (size_t)st * SB_BYTES, &map_w, ks * BK, j0, &full[st]);
+                }
                 last = ks;
             }
             if (!ok || *abort_flag) {   // let this thread's copies in flight land before the block's shared memory goes away
                 for (int ks = last; ks >= 0 && ks > last - STAGES; ks -= S_PRODUCERS)
-                    for (uint32_t it = 0; it < SPIN_LIMIT; ++it)
+                    for (uint32_t it = 0; it < DRAIN_LIMIT; ++it)       // (the stage's other operand may never have been asked for)
                         if (mbar_try_wait(&full[ks % STAGES], (uint32_t)(ks / STAGES) & 1u)) break;
             }
         }
@@ -204,6 +217,15 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         const int m = m0 + r_tile;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const int used_accs = p.k_steps < S_ACCS ? p.k_steps : S_ACCS;         // an accumulator without K steps holds nothing
+        {   // the tile's slice of b1 and w2, zero past h so that padded columns add nothing
+            const int e = threadIdx.x - S_EPI_WARP0 * 32;
+            if (e < SBN) {
+                const int j = j0 + e;
+                b1_s[e] = (j < p.h && p.b1) ? __bfloat162float(pdl_acquire(p.b1)[j]) : 0.f;
+                w2_s[e] = (j < p.h) ? __bfloat162float(pdl_acquire(p.w2)[j]) : 0.f;
+            }
+        }
+        asm volatile("bar.sync 2, 256;" ::: "memory");
         bool ok = mbar_wait(acc_full, 0u, abort_flag);
         ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
         // sum_j w2_j gelu(u_j + b1_j) over 32 hidden units in index order; two of these, low + high, make a partial sum
@@ -244,39 +266,73 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             asm volatile("bar.sync 2, 256;" ::: "memory");
         }
         if (SBN == 128 || half == 0) {
-            constexpr int PARTS = SBN == 128 ? 256 : 128;       // threads that hold a partial sum
             if constexpr (SBN == 64) part += half_s[r_tile];    // low half + high half
             const int sub = (int)blockIdx.y * (SBN / SUB_H) + (SBN == 128 ? half : 0);
-            // The counter protocol runs whatever happened above, so the counters are back at zero after every launch
-            // (after an expired wait the scores of the call are not meaningful and the status word says so).
-            if (m < p.N && sub * SUB_H < p.h) p.partial[(int64_t)sub * p.N + m] = part;
-            __threadfence();
-            asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
-            if (threadIdx.x == S_EPI_WARP0 * 32) {
-                const uint32_t done = atomicAdd(&p.counters[blockIdx.x], 1u);
-                if (done == gridDim.y - 1) {
-                    *is_last = 1u;
-                    p.counters[blockIdx.x] = 0u;    // every block of this row tile has arrived: ready for the next call
-                }
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
-            if (*is_last && half == 0 && m < p.N) {
+            if constexpr (CLUSTER) {
+                if (sub * SUB_H < p.h) st_shared_cluster_f32(map_to_cta(smem_u32(&subs_s[sub * TM + r_tile]), 0u), part);
+            } else {
+                constexpr int PARTS = SBN == 128 ? 256 : 128;   // threads that hold a partial sum
+                // The counter protocol runs whatever happened above, so the counters are back at zero after every launch
+                // (after an expired wait the scores of the call are not meaningful and the status word says so).
+                if (m < p.N && sub * SUB_H < p.h) p.partial[(int64_t)sub * p.N + m] = part;
                 __threadfence();
-                float s = 0.f;
-                for (int t = 0; t * SUB_H < p.h; ++t) s += __ldcg(&p.partial[(int64_t)t * p.N + m]);
-                if (p.b2) s += __bfloat162float(p.b2[0]);
-                probability_map(s, m, p.B, p.q_lut, p.score, p.prob, p.bin, p.q);
+                asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
+                if (threadIdx.x == S_EPI_WARP0 * 32) {
+                    const uint32_t done = atomicAdd(&p.counters[blockIdx.x], 1u);
+                    if (done == gridDim.y - 1) {
+                        *is_last = 1u;
+                        p.counters[blockIdx.x] = 0u;    // every block of this row tile has arrived: ready for the next call
+                    }
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
+                if (*is_last && half == 0 && m < p.N) {
+                    __threadfence();
+                    float s = 0.f;
+                    for (int t = 0; t * SUB_H < p.h; ++t) s += __ldcg(&p.partial[(int64_t)t * p.N + m]);
+                    if (p.b2) s += __bfloat162float(p.b2[0]);
+                    probability_map(s, m, p.B, p.q_lut, p.score, p.prob, p.bin, p.q);
+                }
             }
         }
     }
 
     tcgen05_fence_before();
     __syncthreads();
+    if constexpr (CLUSTER) {
+        cluster_sync_all();             // the first block has everybody's partial sums; the others need nothing from here on
+        const int r = threadIdx.x, m = m0 + r;
+        if (blockIdx.y == 0 && r < TM && m < p.N) {
+            float s = 0.f;
+            for (int t = 0; t * SUB_H < p.h; ++t) s += subs_s[t * TM + r];
+            if (p.b2) s += __bfloat162float(pdl_acquire(p.b2)[0]);
+            probability_map(s, m, p.B, pdl_acquire(p.q_lut), p.score, p.prob, p.bin, p.q);
+        }
+    }
     if (threadIdx.x == 0 && *abort_flag) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
     if (warp == S_PRODUCER_WARPS) {
         tcgen05_fence_after();
         tcgen05_dealloc(tmem_base, S_TMEM_COLS);
     }
+}
+
+// Clusters of `blocks` blocks with tiles of 64 hidden units that are resident at once (asked once per context and size).
+int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
+    if (ctx->score_max_clusters[blocks] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, (unsigned)blocks);
+        cfg.blockDim = dim3(S_THREADS);
+        cfg.dynamicSmemBytes = smem_bytes<64>();
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = (unsigned)blocks;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&ctx->score_max_clusters[blocks], score_mlp_tc_kernel<64, true>, &cfg));
+    }
+    *fit = ctx->score_max_clusters[blocks];
+    return ARROL_OK;
 }
 
 }  // namespace
@@ -295,7 +351,26 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     const bool pack = row_index != nullptr;
     if (pack && (size_t)N * (size_t)d * 2 > ARROL_PACK_BYTES) return ARROL_ERR_UNSUPPORTED;
     if (!row_index && ((uint64_t)row_stride * 2) >= (1ull << 40)) return ARROL_ERR_UNSUPPORTED;
-
+    if (!ctx->score_tc_smem_set) {      // once per context: this call is on the prune step's microsecond path
+        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
+        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
+        ctx->score_tc_smem_set = true;
+    }
+    // Tiles of 64 hidden units while they fit one wave of blocks (more SMs share the way in for the operands), of 128 beyond
+    // that (a third fewer operand bytes and half as many blocks); the bits are the same.  As clusters fewer blocks fit: GPCs are
+    // not filled by clusters of any size.  Without / with the wide tiles (rows packed before, partial sums through global memory):
+    // N = 4,096, d = 4,096, h = 512 39.0 -> 28.4 us (8 of them the packing), N = 8,192 80.7 -> 64.7, N = 3,000, d = 1,024
+    // 17.1 -> 14.6; within one wave they lose: N = 2,048, d = 2,048, h = 256 14.2 -> 15.1.
+    const bool cluster = subs <= MAX_SUBS;
+    bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
+    if (cluster && !wide && subs > 1) {
+        int fit = 0;                    // clusters of more than eight blocks are not portable
+        if (subs <= 8 && narrow_clusters(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
+        wide = m_tiles > fit;
+    }
+    const int tiles_h = wide ? (h + 127) / 128 : subs;
     const void* x = hidden;
     int64_t ld = row_stride;
     if (pack) {
@@ -307,11 +382,6 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
         x = ctx->d_pack;
         ld = d;
     }
-    // Tiles of 64 hidden units while they fit one wave of blocks (more SMs share the way in for the operands), of 128 beyond
-    // that (a third fewer operand bytes and half as many blocks); the bits are the same.  Without / with the wide tiles:
-    // N = 4,096, d = 4,096, h = 512 39.0 -> 28.4 us (8 of them the packing), N = 8,192 80.7 -> 64.7, N = 3,000, d = 1,024
-    // 17.1 -> 14.6; within one wave they lose: N = 2,048, d = 2,048, h = 256 14.2 -> 15.1.
-    const bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
     CUtensorMap map_x, map_w;
     if (make_map(ctx, &map_w, head->W1, (uint64_t)h, (uint64_t)d, wide ? 128 : 64) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map_ld(ctx, &map_x, x, (uint64_t)N, (uint64_t)d, (uint64_t)ld, TM) != ARROL_OK) return ARROL_ERR_CUDA;
@@ -333,16 +403,23 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     p.bin = bin;
     p.q = q;
     p.d_status = ctx->d_status;
-    if (!ctx->score_tc_smem_set) {      // once per context: this call is on the prune step's microsecond path
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
-        ctx->score_tc_smem_set = true;
-    }
-    if (wide)
-        ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tc_kernel<128>, dim3(m_tiles, (h + 127) / 128), dim3(S_THREADS), smem_bytes<128>(), s,
-                                       map_x, map_w, p));
-    else
-        ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tc_kernel<64>, dim3(m_tiles, subs), dim3(S_THREADS), smem_bytes<64>(), s, map_x, map_w, p));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)m_tiles, (unsigned)tiles_h);
+    cfg.blockDim = dim3(S_THREADS);
+    cfg.dynamicSmemBytes = wide ? smem_bytes<128>() : smem_bytes<64>();
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = tiles_h;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster ? 2 : 1;
+    const auto kernel = cluster ? (wide ? score_mlp_tc_kernel<128, true> : score_mlp_tc_kernel<64, true>)
+                                : (wide ? score_mlp_tc_kernel<128, false> : score_mlp_tc_kernel<64, false>);
+    ARROL_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, map_x, map_w, p));
     ctx->launches += 1;
     return ARROL_OK;
 }

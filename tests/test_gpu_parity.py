@@ -130,6 +130,14 @@ def test_mlp_head_scores_do_not_depend_on_how_many_rollouts_are_scored(ctx, N, d
     assert all(torch.equal(a[:130], b) for a, b in zip(*out))
 
 
+# a row tile's blocks as a cluster of 1 to 8 (tiles of 64 hidden units; of 128 past 512), the last one partly past h, one row tile and two
+# with one row in the second, one K step and several; 1,028 hidden units go without clusters
+@pytest.mark.parametrize("h", [4, 64, 68, 192, 260, 512, 516, 1024, 1028])
+def test_mlp_head_clusters_of_every_size(ctx, h):
+    _score_case(ctx, 129, 72, h, torch.bfloat16, True, True, seed=h)
+    _score_case(ctx, 1, 648, h, torch.bfloat16, False, False, seed=h + 1, bias=False)
+
+
 def test_mlp_head_strided_rows_without_index(ctx):
     """Evenly strided rows (a column slice of a wider buffer) go to the tensor-core path without packing."""
     g = np.random.default_rng(5)
