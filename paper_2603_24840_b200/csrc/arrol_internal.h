@@ -22,6 +22,7 @@ struct arrol_ctx {
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
     int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
     bool head_dw1_smem_set[2]; // likewise for the head training step's contraction (column tiles of 64, 128)
+    int head_dw1_max_clusters[2];   // clusters of eight blocks of that kernel that are resident at once; 0 = not asked yet
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool prune_smem_set;       // likewise for the fused prune step
@@ -143,6 +144,9 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
                                 int N, const arrol_head* head, int B, const float* q_lut, float* score, float* prob,
                                 int32_t* bin, float* q, float* u_out /* [N][h] pre-activations, or NULL */,
                                 cudaStream_t s);
+int arrol_internal_head_train_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
+                                 const arrol_head* head, const float* rewards, const uint8_t* mask, void* du_hi, void* du_lo,
+                                 float* tile_sums, double* tile_loss, cudaStream_t s);
 
 // gather_bulk.cu: the survivors' rows moved by bulk copies through shared memory.  ARROL_ERR_UNSUPPORTED (nothing
 // launched) when a row does not fit a 32 KB stage.
@@ -152,6 +156,15 @@ int arrol_internal_gather_rows_bulk(arrol_ctx* ctx, const int64_t* d_num, const 
                                     const int32_t* survivor_idx, const int64_t* src_tok_off, int N, const TokenOutputs& outputs,
                                     const void* src_rows, int64_t row_bytes, int64_t capacity, void* dst_rows, cudaStream_t s);
 
-// head_grad_tc.cu: dW1[h, d] = (du_hi + du_lo)^T X on the tensor cores, du planes [N, h] bf16, X [N, d] bf16 with rows ldx apart.
+// head_grad_tc.cu: dW1[h, d] = (du_hi + du_lo)^T X on the tensor cores, du planes [N, h] bf16, X [N, d] bf16 with rows ldx apart; and
+// the sums over the tiles of 128 rollouts that arrol_internal_head_train_tc left, where tile_sums is given.
+struct HeadTileSums {
+    const float* tile_sums;     // [2][tiles][h] -> dw2, db1
+    const double* tile_loss;    // [2][tiles] -> loss, db2
+    float* dw2;
+    float* db1;
+    double* loss;
+    float* db2;
+};
 int arrol_internal_head_dw1(arrol_ctx* ctx, const void* du_hi, const void* du_lo, const void* X, int64_t ldx, int N, int d,
-                            int h, float* dW1, cudaStream_t s);
+                            int h, float* dW1, const HeadTileSums& sums, cudaStream_t s);

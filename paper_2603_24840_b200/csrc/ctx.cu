@@ -48,6 +48,7 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
     ctx->d_tile_counters = nullptr;
     ctx->d_chain = nullptr;
     ctx->logprob_smem_set = false;
+    ctx->head_dw1_max_clusters[0] = ctx->head_dw1_max_clusters[1] = 0;
     ctx->calib_smem_set = false;
     ctx->backward_smem_set = false;
     ctx->prune_smem_set = false;

@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "arrol_internal.h"
+#include "score_common.cuh"
 
 namespace {
 
@@ -130,21 +131,6 @@ __global__ void column_sum_kernel(const float* __restrict__ partial, int chunks,
 // ds of its own run; the last block of a column tile to arrive (a counter per tile, zero again when that block is through) adds the runs' sums in
 // index order, the one of tile 0 the loss and db2 as well.  The score is given, or the sum of the forward's tile partials + b2.
 // du goes out as float (SIMT contraction) or as the sum of two bf16 planes (error 2^-17 relative: the tensor-core operand).
-template <int THREADS>
-__device__ __forceinline__ int count_labelled(const uint8_t* mask, int N) {
-    if (!mask) return N;
-    int c = 0;
-    const int vec = (reinterpret_cast<uintptr_t>(mask) & 15) == 0 ? N / 16 : 0;
-    for (int i = threadIdx.x; i < vec; i += THREADS) {
-        const uint4 v = reinterpret_cast<const uint4*>(mask)[i];
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) c += __popc(__vcmpne4(w[k], 0u)) >> 3;
-    }
-    for (int i = vec * 16 + threadIdx.x; i < N; i += THREADS) c += mask[i] ? 1 : 0;
-    return c;
-}
-
 constexpr int DU_THREADS = 256;
 template <typename T>
 __global__ void __launch_bounds__(DU_THREADS)
@@ -175,9 +161,9 @@ head_du_kernel(const float* u, const float* score, const float* partial, int h_t
     }
     const float wj = j < h ? widen(w2[j]) : 0.f;
     {
-        int c = count_labelled<DU_THREADS>(mask, N);
+        int c = mask ? count_labelled(mask, N, threadIdx.x, DU_THREADS) : 0;
         c = __reduce_add_sync(0xffffffffu, c);
-        if (tx == 0) warp_n[ty] = mask ? c : 0;
+        if (tx == 0) warp_n[ty] = c;
     }
     __syncthreads();
     int n = mask ? 0 : N;
@@ -393,17 +379,25 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
             // bf16 head: both contractions on the tensor cores.  Forward with the pre-activations kept, du split into
             // two bf16 planes, dW1 = du_hi^T X + du_lo^T X with X the packed rows (or the rows in place).
             if (h % 8 == 0) {
-                float* tmp = reinterpret_cast<float*>(ws + L.tmp3);
-                const int rc = arrol_internal_score_mlp_tc(ctx, hidden, row_stride, row_index, N, head, 0, nullptr, tmp,
-                                                           tmp + N, nullptr, tmp + 2 * (size_t)N, u, s);
-                if (rc == ARROL_OK) {
-                    __nv_bfloat16* du_hi = reinterpret_cast<__nv_bfloat16*>(ws + L.du);
-                    __nv_bfloat16* du_lo = reinterpret_cast<__nv_bfloat16*>(ws + L.du + L.du_plane);
-                    const int rd = launch_du(tmp, nullptr, 0, nullptr, du_hi, du_lo, ctx->d_head_counters);
-                    if (rd != ARROL_OK) return rd;
-                    return arrol_internal_head_dw1(ctx, du_hi, du_lo, row_index ? ctx->d_pack : hidden,
-                                                   row_index ? (int64_t)d : row_stride, N, d, h, dW1, s);
+                __nv_bfloat16* du_hi = reinterpret_cast<__nv_bfloat16*>(ws + L.du);
+                __nv_bfloat16* du_lo = reinterpret_cast<__nv_bfloat16*>(ws + L.du + L.du_plane);
+                // sums per tile of 128 rollouts: where the other path keeps those of its runs, of more tiles where it keeps u and ds
+                const bool few = (N + 127) / 128 <= DU_RUNS;
+                float* tile_sums = few ? reinterpret_cast<float*>(ws + L.run_sums) : u;
+                double* tile_loss = few ? reinterpret_cast<double*>(ws + L.run_loss) : reinterpret_cast<double*>(ds);
+                HeadTileSums sums = {tile_sums, tile_loss, dw2, db1, loss, db2};
+                int rc = arrol_internal_head_train_tc(ctx, hidden, row_stride, row_index, N, head, rewards, mask, du_hi, du_lo,
+                                                      tile_sums, tile_loss, s);
+                if (rc == ARROL_ERR_UNSUPPORTED) {      // more than 1,024 hidden units, or beyond the context's buffers
+                    float* tmp = reinterpret_cast<float*>(ws + L.tmp3);
+                    sums.tile_sums = nullptr;
+                    rc = arrol_internal_score_mlp_tc(ctx, hidden, row_stride, row_index, N, head, 0, nullptr, tmp, tmp + N, nullptr,
+                                                     tmp + 2 * (size_t)N, u, s);
+                    if (rc == ARROL_OK) rc = launch_du(tmp, nullptr, 0, nullptr, du_hi, du_lo, ctx->d_head_counters);
                 }
+                if (rc == ARROL_OK)
+                    return arrol_internal_head_dw1(ctx, du_hi, du_lo, row_index ? ctx->d_pack : hidden,
+                                                   row_index ? (int64_t)d : row_stride, N, d, h, dW1, sums, s);
                 if (rc != ARROL_ERR_UNSUPPORTED) return rc;
             }
         }

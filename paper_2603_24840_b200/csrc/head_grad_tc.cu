@@ -7,6 +7,8 @@
 // blocks while SMs are idle (their accumulators meet in shared memory, added in rank order) and TN is 128 where tiles of 64
 // would need more than one wave.  N = 2,048, d = 2,048, h = 256: 12.7 us (7 of them launch, set-up and finish) against 35.7 for a
 // launch per plane on eight 128 x 256 tiles; N = 4,096, d = 4,096, h = 512: 33 us.
+// The epilogue warps, which wait for the contraction, add up the row tiles' sums that dw2, db1, db2 and the loss are made of; the forward
+// kernel's last blocks did, behind a fence, a counter and a reload (N = 2,048, d = 2,048, h = 256: whole call 32.3 -> 29.2 us).
 // Every wait is bounded; on expiry the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -30,6 +32,7 @@ struct Dw1Params {
     int N, d, h;
     int k_steps;                                  // ceil(N / 64)
     float* dW1;
+    HeadTileSums sums;
     uint32_t* d_status;
 };
 
@@ -129,6 +132,28 @@ head_dw1_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constan
     } else {
         // thread = one hidden unit: its TN sums go to shared memory (the stages are free: every MMA has finished)
         const int quarter = warp & 3, r = quarter * 32 + lane;
+        if (c0 == 0 && rank == 0 && p.sums.tile_sums) {        // the row tiles' sums, in index order, while the contraction runs
+            const int tiles = (p.N + 127) / 128, j = j0 + r;
+            const float* tile_sums = pdl_acquire(p.sums.tile_sums);
+            if (j < p.h) {
+                double w2 = 0.0, b1 = 0.0;          // up to 512 tiles
+#pragma unroll 8
+                for (int t = 0; t < tiles; ++t) {
+                    w2 += tile_sums[(int64_t)t * p.h + j];
+                    b1 += tile_sums[(int64_t)(tiles + t) * p.h + j];
+                }
+                p.sums.dw2[j] = (float)w2;
+                p.sums.db1[j] = (float)b1;
+            }
+            if (j0 == 0 && r < 2) {
+                const double* tile_loss = pdl_acquire(p.sums.tile_loss);
+                double t = 0.0;
+#pragma unroll 8
+                for (int i = 0; i < tiles; ++i) t += tile_loss[r * tiles + i];
+                if (r == 0) *p.sums.loss = t;
+                else *p.sums.db2 = (float)t;
+            }
+        }
         bool ok = mbar_wait(acc_full, 0u, abort_flag);
         ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
         float* row = reinterpret_cast<float*>(smem) + r * PITCH;
@@ -177,10 +202,7 @@ int launch_dw1(arrol_ctx* ctx, const CUtensorMap& hi, const CUtensorMap& lo, con
         ctx->head_dw1_smem_set[TN == 128] = true;
     }
     const int tiles = ((p.d + TN - 1) / TN) * ((p.h + GM - 1) / GM);
-    int splits = 1;                     // blocks per cluster: at least four K steps each, no more blocks than SMs
-    while (splits < 4 && tiles * splits * 2 <= ctx->sm_count && p.k_steps >= splits * 2 * 4) splits *= 2;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((p.d + TN - 1) / TN, (p.h + GM - 1) / GM, splits);
     cfg.blockDim = dim3(G_THREADS);
     cfg.dynamicSmemBytes = smem_bytes<TN>();
     cfg.stream = s;
@@ -188,10 +210,28 @@ int launch_dw1(arrol_ctx* ctx, const CUtensorMap& hi, const CUtensorMap& lo, con
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1;
     attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = splits;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
+    auto shape = [&](int splits) {
+        cfg.gridDim = dim3((p.d + TN - 1) / TN, (p.h + GM - 1) / GM, splits);
+        attr[0].val.clusterDim.z = splits;
+    };
+    // Blocks per cluster: at least four K steps each, and no more blocks than SMs; eight only where so many clusters fit at once
+    // (asked once per context).  N = 5,000, d = 520, h = 72 (nine tiles) with four / eight: 28.5 / 24.5 us; where they do not fit, N = 8,000,
+    // d = 1,024, h = 64 (16 tiles) 30.3 / 35.8.
+    int splits = 1;
+    while (splits < 4 && tiles * splits * 2 <= ctx->sm_count && p.k_steps >= splits * 2 * 4) splits *= 2;
+    if (splits == 4 && tiles * 8 <= ctx->sm_count && p.k_steps >= 32) {
+        int& fit = ctx->head_dw1_max_clusters[TN == 128];
+        if (fit == 0) {
+            shape(8);
+            cfg.numAttrs = 1;
+            ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&fit, head_dw1_kernel<TN>, &cfg));
+        }
+        if (tiles <= fit) splits = 8;
+    }
+    shape(splits);
     cfg.numAttrs = 2;
     ARROL_CUDA_OK(cudaLaunchKernelEx(&cfg, head_dw1_kernel<TN>, hi, lo, x, p));
     ctx->launches += 1;
@@ -201,7 +241,7 @@ int launch_dw1(arrol_ctx* ctx, const CUtensorMap& hi, const CUtensorMap& lo, con
 }  // namespace
 
 int arrol_internal_head_dw1(arrol_ctx* ctx, const void* du_hi, const void* du_lo, const void* X, int64_t ldx, int N, int d,
-                            int h, float* dW1, cudaStream_t s) {
+                            int h, float* dW1, const HeadTileSums& sums, cudaStream_t s) {
     CUtensorMap map_hi, map_lo, map_x;
     if (make_map(ctx, &map_hi, du_hi, (uint64_t)N, (uint64_t)h, BK) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map(ctx, &map_lo, du_lo, (uint64_t)N, (uint64_t)h, BK) != ARROL_OK) return ARROL_ERR_CUDA;
@@ -210,6 +250,7 @@ int arrol_internal_head_dw1(arrol_ctx* ctx, const void* du_hi, const void* du_lo
     p.N = N; p.d = d; p.h = h;
     p.k_steps = (N + BK - 1) / BK;
     p.dW1 = dW1;
+    p.sums = sums;
     p.d_status = ctx->d_status;
     const int tiles64 = ((d + 63) / 64) * ((h + GM - 1) / GM);
     return tiles64 > ctx->sm_count ? launch_dw1<128>(ctx, map_hi, map_lo, map_x, p, s)

@@ -16,8 +16,8 @@
 //                         128, and a step's operands come in in about 290.  K step ks goes to accumulator ks mod 4.  The ring's
 //                         length is a multiple of the number of issuers, so that a stage always belongs to the same one: a parity
 //                         wait cannot tell a round from the one before the last.
-//                         Eight epilogue warps: thread = rollout x half of the tile's hidden units; accumulators added in
-//                         index order, then sum_j w2_j gelu(u_j + b1_j) over 32 units in index order, two such sums added
+//                         Epilogue by all sixteen warps (with eight, two a scheduler, the chains of erff wait for themselves: 3.0 us
+//                         for 64 units): thread = rollout x a quarter of the tile's hidden units; accumulators added in index order, then sum_j w2_j gelu(u_j + b1_j) over 32 units in index order, two such sums added
 //                         low + high -> a partial sum per 64 units and rollout, whatever the tile's width.
 //                         The blocks of a row tile are a cluster and put their partial sums into the first block's shared
 //                         memory, which adds them in index order, adds b2 and applies the probability map.  More than 1,024
@@ -43,14 +43,15 @@ namespace {
 constexpr int SUB_H = 64;                    // hidden units per partial sum: the same for every tile width
 constexpr int S_ACCS = 4;                    // accumulators; K step ks goes to accumulator ks % 4
 constexpr int S_PRODUCERS = 2;               // TMA producer threads (lane 0 of the first warps)
-constexpr int S_PRODUCER_WARPS = 4;          // warps before the issuers (two of them idle: the epilogue warps start at a multiple of 4)
-constexpr int S_EPI_WARP0 = 8;               // a multiple of 4: epilogue warp w reads lane quarter w % 4
-constexpr int S_EPI_WARPS = 8;
-constexpr int S_THREADS = (S_EPI_WARP0 + S_EPI_WARPS) * 32;
+constexpr int S_PRODUCER_WARPS = 4;          // warps before the issuers
+constexpr int S_HELPER_WARP0 = 8;            // warps without a role in the contraction fetch what the epilogue needs
+constexpr int S_HELPER_WARPS = 8;
+constexpr int S_WARPS = S_HELPER_WARP0 + S_HELPER_WARPS, S_THREADS = S_WARPS * 32;     // the epilogue is all warps' work
 constexpr uint32_t DRAIN_LIMIT = 1u << 16;   // tries per wait of a producer that gave up, for copies in flight
 constexpr int MAX_SUBS = 16;                 // partial sums of a row tile whose blocks form a cluster: 8 blocks of 128 hidden units
-// barriers, tensor-memory slot, flags | b1 and w2 of the tile, sums over a 64-unit tile's upper 32 hidden units | partial sums
-constexpr int S_TAIL_BYTES = 2048 + MAX_SUBS * 128 * 4;
+// barriers, tensor-memory slot, flags | b1 and w2 of the tile, sums over 16 hidden units | sums over 32
+// | the training step's ds of the tile's rollouts, sums over its warps
+constexpr int S_TAIL_BYTES = 2560 + 2 * MAX_SUBS * 128 * 4 + 512 + 256;
 constexpr int TM = 128;                      // rollouts per tile (MMA M)
 constexpr int A_BYTES = TM * BK * 2;         // 16 KB
 // by tile width (hidden units, MMA N): 64 or 128
@@ -93,7 +94,7 @@ struct ScoreTcParams {
     const __nv_bfloat16* b1;           // [h] or NULL
     const __nv_bfloat16* w2;           // [h]
     const __nv_bfloat16* b2;           // [1] or NULL
-    float* partial;                    // [ceil(h / 64)][N]
+    float* partial;                    // PARTIALS: [ceil(h / 64)][N]
     float* u_out;                      // [N][h] pre-activations (bias included) for the head training step, or NULL
     uint32_t* counters;                // [row tiles], zero between calls
     int B;
@@ -103,10 +104,24 @@ struct ScoreTcParams {
     int32_t* bin;
     float* q;
     uint32_t* d_status;
+    // TRAIN
+    const float* rewards;
+    const uint8_t* mask;               // or NULL
+    __nv_bfloat16* du_hi;              // [N][h], du as the sum of two bf16 planes
+    __nv_bfloat16* du_lo;
+    float* tile_sums;                  // [2][row tiles][h]: sums of ds gelu(u) and of du over a tile's rollouts
+    double* tile_loss;                 // [2][row tiles]: sums of the losses, divided by their number, and of ds
 };
 
-// CLUSTER: the blocks of a row tile (gridDim.y of them, at most eight) are a cluster and finish the scores among themselves.
-template <int SBN, bool CLUSTER>
+// PARTIALS: row tiles of more than eight blocks; the scores are finished through global memory.  SCORES: the blocks of a row tile
+// (gridDim.y of them) are a cluster and finish the scores among themselves.  TRAIN: the head training step's forward and all
+// of its backward but the dW1 contraction: as SCORES, but every block gets all partial sums, forms the scores' gradients ds and
+// finishes its own hidden units: du = ds w2 gelu'(u), and the sums over the tile's rollouts that dw2 and db1 are made of, which the dW1 kernel adds up while it waits
+// for its contraction.  Both addends go to the operand ring's
+// shared memory, [unit][rollout], where the sums over rollouts are read along rows.  A kernel of its
+// own with u through global memory between took 9.4 us at N = 2,048, h = 256 (ncu).
+enum Mode { PARTIALS, SCORES, TRAIN };
+template <int SBN, Mode MODE>
 __global__ void __launch_bounds__(S_THREADS, 1)
 score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                     const ScoreTcParams p) {
@@ -115,6 +130,8 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     static_assert(STAGES % ISSUERS == 0 && S_ACCS % ISSUERS == 0 && STAGES % S_PRODUCERS == 0,
                   "a stage and an accumulator belong to one issuer, a stage to one producer");
     constexpr int S_TMEM_COLS = S_ACCS * SBN;                    // a power of two >= 32
+    constexpr bool CLUSTER = MODE != PARTIALS;
+    static_assert(2 * SBN * TM * 4 <= STAGES * STAGE_BYTES, "both planes fit the stages");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* stage_a = smem;
@@ -128,8 +145,13 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     volatile uint32_t* is_last = tmem_slot + 2;
     float* b1_s = reinterpret_cast<float*>(tail + 512);          // [SBN]
     float* w2_s = reinterpret_cast<float*>(tail + 1024);         // [SBN]
-    float* half_s = reinterpret_cast<float*>(tail + 1536);       // [TM] sums over a 64-unit tile's upper 32 hidden units
-    float* subs_s = reinterpret_cast<float*>(tail + 2048);       // [MAX_SUBS][TM] partial sums of the row tile (first block of a cluster)
+    float* half_s = reinterpret_cast<float*>(tail + 1536);       // [2][TM] sums over 16 hidden units of a tile of 64
+    float* runs_s = reinterpret_cast<float*>(tail + 2560);       // [2 MAX_SUBS][TM] sums over 32 (of the row tile in the first block of a cluster; TRAIN: in every block)
+    float* ds_s = runs_s + 2 * MAX_SUBS * TM;                    // [TM]
+    double* warp_d = reinterpret_cast<double*>(ds_s + TM);       // [2][4]
+    int* warp_n = reinterpret_cast<int*>(warp_d + 8);            // [S_HELPER_WARPS]
+    float* gelu_s = reinterpret_cast<float*>(smem);              // [SBN][TM] ds gelu(u), once every MMA has finished
+    float* du_s = gelu_s + SBN * TM;                             // [SBN][TM]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * TM, j0 = blockIdx.y * SBN;
@@ -155,6 +177,8 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     pdl_launch_dependents();
     pdl_wait();                  // set-up above overlaps the previous kernel; global memory is read from here on
 
+    bool labelled = false;       // TRAIN, warps 8 to 11: of rollout r_tile
+    float reward = 0.f;
     // K step ks uses stage ks % STAGES in round ks / STAGES of the ring, issuer ks % ISSUERS and accumulator ks % S_ACCS.
     if (warp < S_PRODUCER_WARPS) {
         if (lane == 0) {         // two threads for the rows, two for W1, on alternate K steps
@@ -180,7 +204,7 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                         if (mbar_try_wait(&full[ks % STAGES], (uint32_t)(ks / STAGES) & 1u)) break;
             }
         }
-    } else if (warp < S_EPI_WARP0) {
+    } else if (warp < S_HELPER_WARP0) {
         const int r = warp - S_PRODUCER_WARPS;
         if (r < ISSUERS) {
             const uint32_t a0 = smem_u32(stage_a), b0 = smem_u32(stage_b);
@@ -211,101 +235,207 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                     if (mbar_try_wait(acc_full, 0u)) break;
         }
     } else {
-        const int quarter = warp & 3;                           // accumulator row r is tensor-memory lane r
-        const int half = (warp - S_EPI_WARP0) >> 2;             // which half of the tile's hidden units
-        const int r_tile = quarter * 32 + lane;
-        const int m = m0 + r_tile;
-        const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-        const int used_accs = p.k_steps < S_ACCS ? p.k_steps : S_ACCS;         // an accumulator without K steps holds nothing
-        {   // the tile's slice of b1 and w2, zero past h so that padded columns add nothing
-            const int e = threadIdx.x - S_EPI_WARP0 * 32;
-            if (e < SBN) {
-                const int j = j0 + e;
-                b1_s[e] = (j < p.h && p.b1) ? __bfloat162float(pdl_acquire(p.b1)[j]) : 0.f;
-                w2_s[e] = (j < p.h) ? __bfloat162float(pdl_acquire(p.w2)[j]) : 0.f;
-            }
+        const int e = threadIdx.x - S_HELPER_WARP0 * 32;
+        if (e < SBN) {          // the tile's slice of b1 and w2, zero past h so that padded columns add nothing
+            const int j = j0 + e;
+            b1_s[e] = (j < p.h && p.b1) ? __bfloat162float(pdl_acquire(p.b1)[j]) : 0.f;
+            w2_s[e] = (j < p.h) ? __bfloat162float(pdl_acquire(p.w2)[j]) : 0.f;
         }
-        asm volatile("bar.sync 2, 256;" ::: "memory");
-        bool ok = mbar_wait(acc_full, 0u, abort_flag);
-        ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
-        // sum_j w2_j gelu(u_j + b1_j) over 32 hidden units in index order; two of these, low + high, make a partial sum
-        auto units32 = [&](int j32) {
-            float part = 0.f;
-            float v[32];
-            tcgen05_ld_32x32(tmem_base + lane_addr + j32, v);
-            for (int a = 1; a < used_accs; ++a) {      // fixed order: ((acc0 + acc1) + acc2) + acc3
-                float w[32];
-                tcgen05_ld_32x32(tmem_base + lane_addr + a * SBN + j32, w);
-#pragma unroll
-                for (int jj = 0; jj < 32; ++jj) v[jj] += w[jj];
+        if constexpr (MODE == TRAIN) {      // every block counts the labelled rollouts itself
+            const uint8_t* mask = pdl_acquire(p.mask);
+            if (e < TM && m0 + e < p.N) {
+                labelled = !mask || mask[m0 + e];
+                reward = pdl_acquire(p.rewards)[m0 + e];
             }
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-                const float u = v[jj] + b1_s[j32 + jj];
-                v[jj] = u;
-                const float g = 0.5f * u * (1.0f + erff(u * 0.70710678118654752440f));
-                part = fmaf(w2_s[j32 + jj], g, part);
-            }
-            if (p.u_out && m < p.N) {
-                float* urow = p.u_out + (int64_t)m * p.h + j0 + j32;
-#pragma unroll
-                for (int jj = 0; jj < 32; jj += 4)      // h % 4 == 0: a float4 never straddles the edge
-                    if (j0 + j32 + jj < p.h)
-                        *reinterpret_cast<float4*>(urow + jj) = make_float4(v[jj], v[jj + 1], v[jj + 2], v[jj + 3]);
-            }
-            return part;
-        };
-        float part = 0.f;
-        if (ok) {
-            tcgen05_fence_after();
-            part = units32(half * (SBN / 2));
-            if constexpr (SBN == 128) part += units32(half * 64 + 32);
+            const int c = __reduce_add_sync(0xffffffffu, mask ? count_labelled(mask, p.N, e, S_HELPER_WARPS * 32) : 0);
+            if (lane == 0) warp_n[warp - S_HELPER_WARP0] = c;
         }
-        if constexpr (SBN == 64) {
-            if (half == 1) half_s[r_tile] = part;
-            asm volatile("bar.sync 2, 256;" ::: "memory");
+    }
+    __syncwarp();
+
+    // Epilogue: all warps; thread = rollout x a quarter of the tile's hidden units.  Accumulator row r is tensor-memory lane r, and a
+    // warp reads the lanes of its number mod 4.
+    constexpr int UNITS = SBN / 4;
+    const int quarter = warp & 3, cg = warp >> 2;
+    const int r_tile = quarter * 32 + lane, m = m0 + r_tile;
+    const int used_accs = p.k_steps < S_ACCS ? p.k_steps : S_ACCS;         // an accumulator without K steps holds nothing
+    bool ok = mbar_wait(acc_full, 0u, abort_flag);
+    ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
+    __syncthreads();                        // b1_s, w2_s
+    float v[UNITS], cdf[UNITS];             // u = pre-activations, then gelu(u); 2 Phi(u)
+    if (ok) {
+        tcgen05_fence_after();
+        const uint32_t at = tmem_base + ((uint32_t)(quarter * 32) << 16) + cg * UNITS;
+        tcgen05_ld_32(at, v);
+        for (int a = 1; a < used_accs; ++a) {      // fixed order: ((acc0 + acc1) + acc2) + acc3
+            float w[UNITS];
+            tcgen05_ld_32(at + a * SBN, w);
+#pragma unroll
+            for (int j = 0; j < UNITS; ++j) v[j] += w[j];
         }
-        if (SBN == 128 || half == 0) {
-            if constexpr (SBN == 64) part += half_s[r_tile];    // low half + high half
-            const int sub = (int)blockIdx.y * (SBN / SUB_H) + (SBN == 128 ? half : 0);
-            if constexpr (CLUSTER) {
-                if (sub * SUB_H < p.h) st_shared_cluster_f32(map_to_cta(smem_u32(&subs_s[sub * TM + r_tile]), 0u), part);
-            } else {
-                constexpr int PARTS = SBN == 128 ? 256 : 128;   // threads that hold a partial sum
-                // The counter protocol runs whatever happened above, so the counters are back at zero after every launch
-                // (after an expired wait the scores of the call are not meaningful and the status word says so).
-                if (m < p.N && sub * SUB_H < p.h) p.partial[(int64_t)sub * p.N + m] = part;
-                __threadfence();
-                asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
-                if (threadIdx.x == S_EPI_WARP0 * 32) {
-                    const uint32_t done = atomicAdd(&p.counters[blockIdx.x], 1u);
-                    if (done == gridDim.y - 1) {
-                        *is_last = 1u;
-                        p.counters[blockIdx.x] = 0u;    // every block of this row tile has arrived: ready for the next call
-                    }
-                }
-                asm volatile("bar.sync 1, %0;" ::"n"(PARTS) : "memory");
-                if (*is_last && half == 0 && m < p.N) {
-                    __threadfence();
-                    float s = 0.f;
-                    for (int t = 0; t * SUB_H < p.h; ++t) s += __ldcg(&p.partial[(int64_t)t * p.N + m]);
-                    if (p.b2) s += __bfloat162float(p.b2[0]);
-                    probability_map(s, m, p.B, p.q_lut, p.score, p.prob, p.bin, p.q);
-                }
-            }
+    } else {
+#pragma unroll
+        for (int j = 0; j < UNITS; ++j) v[j] = 0.f;
+    }
+    float slope[MODE == TRAIN ? UNITS : 1];        // gelu'(u) w2
+#pragma unroll
+    for (int j = 0; j < UNITS; ++j) {
+        const float u = v[j] + b1_s[cg * UNITS + j];
+        v[j] = u;
+        cdf[j] = 1.0f + erff(u * 0.70710678118654752440f);
+    }
+    if constexpr (MODE == PARTIALS) {
+        if (p.u_out && m < p.N) {
+            float* urow = p.u_out + (int64_t)m * p.h + j0 + cg * UNITS;
+#pragma unroll
+            for (int j = 0; j < UNITS; j += 4)      // h % 4 == 0: a float4 never straddles the edge
+                if (j0 + cg * UNITS + j < p.h) *reinterpret_cast<float4*>(urow + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        }
+    }
+    // sum_j w2_j gelu(u_j) over 32 hidden units in index order; two of these, low + high, make a partial sum.  Of a tile of 64 two
+    // threads have 16 each, and the second one goes on where the first one ends.
+    const float* w2 = w2_s + cg * UNITS;
+    float part = 0.f;
+    if constexpr (SBN == 64) {
+        if ((cg & 1) == 0) {
+#pragma unroll
+            for (int j = 0; j < UNITS; ++j) part = fmaf(w2[j], 0.5f * v[j] * cdf[j], part);
+            half_s[(cg >> 1) * TM + r_tile] = part;
+        }
+        __syncthreads();
+        if ((cg & 1) == 1) part = half_s[(cg >> 1) * TM + r_tile];
+    }
+    if (SBN == 128 || (cg & 1) == 1) {
+#pragma unroll
+        for (int j = 0; j < UNITS; ++j) part = fmaf(w2[j], 0.5f * v[j] * cdf[j], part);
+        const int run = SBN == 128 ? cg : cg >> 1;                       // of 32 hidden units, in the tile
+        const int all = MODE == PARTIALS ? run : (int)blockIdx.y * (SBN / 32) + run;
+        if (MODE == PARTIALS || (all >> 1) * SUB_H < p.h) {
+            const uint32_t to = smem_u32(&runs_s[all * TM + r_tile]);
+            if constexpr (MODE == PARTIALS) runs_s[all * TM + r_tile] = part;
+            if constexpr (MODE == SCORES) st_shared_cluster_f32(map_to_cta(to, 0u), part);
+            if constexpr (MODE == TRAIN)
+                for (uint32_t b = 0; b < gridDim.y; ++b) st_shared_cluster_f32(map_to_cta(to, b), part);
         }
     }
 
     tcgen05_fence_before();
-    __syncthreads();
-    if constexpr (CLUSTER) {
-        cluster_sync_all();             // the first block has everybody's partial sums; the others need nothing from here on
-        const int r = threadIdx.x, m = m0 + r;
-        if (blockIdx.y == 0 && r < TM && m < p.N) {
+    if constexpr (MODE == PARTIALS) {
+        __syncthreads();
+        // The counter protocol runs whatever happened above, so the counters are back at zero after every launch
+        // (after an expired wait the scores of the call are not meaningful and the status word says so).
+        const int sub = (int)blockIdx.y * (SBN / SUB_H) + cg;
+        if (cg < SBN / SUB_H && m < p.N && sub * SUB_H < p.h)
+            p.partial[(int64_t)sub * p.N + m] = runs_s[2 * cg * TM + r_tile] + runs_s[(2 * cg + 1) * TM + r_tile];
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const uint32_t done = atomicAdd(&p.counters[blockIdx.x], 1u);
+            if (done == gridDim.y - 1) {
+                *is_last = 1u;
+                p.counters[blockIdx.x] = 0u;    // every block of this row tile has arrived: ready for the next call
+            }
+        }
+        __syncthreads();
+        if (*is_last && cg == 0 && m < p.N) {
+            __threadfence();
             float s = 0.f;
-            for (int t = 0; t * SUB_H < p.h; ++t) s += subs_s[t * TM + r];
-            if (p.b2) s += __bfloat162float(pdl_acquire(p.b2)[0]);
-            probability_map(s, m, p.B, pdl_acquire(p.q_lut), p.score, p.prob, p.bin, p.q);
+            for (int t = 0; t * SUB_H < p.h; ++t) s += __ldcg(&p.partial[(int64_t)t * p.N + m]);
+            if (p.b2) s += __bfloat162float(p.b2[0]);
+            probability_map(s, m, p.B, p.q_lut, p.score, p.prob, p.bin, p.q);
+        }
+    } else {
+        cluster_arrive();
+        if constexpr (MODE == TRAIN) {          // what needs no score is done while the partial sums are on their way
+#pragma unroll
+            for (int j = 0; j < UNITS; ++j) {
+                const float u = v[j], half_cdf = 0.5f * cdf[j];
+                slope[j] = w2[j] * (half_cdf + u * (expf(-0.5f * u * u) * 0.39894228040143267794f));
+                v[j] = u * half_cdf;
+            }
+        }
+        cluster_wait();             // the partial sums are there; nobody's shared memory is written from here on
+    }
+    auto score_of = [&](int r) {
+        float s = 0.f;
+        for (int t = 0; t * SUB_H < p.h; ++t) s += runs_s[2 * t * TM + r] + runs_s[(2 * t + 1) * TM + r];
+        return p.b2 ? s + __bfloat162float(pdl_acquire(p.b2)[0]) : s;
+    };
+    if constexpr (MODE == SCORES) {
+        if (blockIdx.y == 0 && cg == 0 && m < p.N)
+            probability_map(score_of(r_tile), m, p.B, pdl_acquire(p.q_lut), p.score, p.prob, p.bin, p.q);
+    }
+    if constexpr (MODE == TRAIN) {
+        const bool live = m < p.N;
+        if (warp >= S_HELPER_WARP0 && warp < S_HELPER_WARP0 + 4) {       // the warps that have the labels
+            int n = p.N;
+            if (p.mask) {
+                n = 0;
+#pragma unroll
+                for (int w = 0; w < S_HELPER_WARPS; ++w) n += warp_n[w];
+            }
+            double l = 0.0, sd = 0.0;
+            float ds = 0.f;
+            if (labelled) {
+                const float s = score_of(r_tile);
+                const float y = reward > 0.5f ? 1.f : 0.f;
+                ds = (1.0f / (1.0f + expf(-s)) - y) / (float)n;
+                sd = (double)ds;
+                if (blockIdx.y == 0) l = (double)((s > 0.f ? s + log1pf(expf(-s)) : log1pf(expf(s))) - y * s);
+            }
+            ds_s[r_tile] = ds;
+            if (blockIdx.y == 0) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    l += __shfl_xor_sync(0xffffffffu, l, o);
+                    sd += __shfl_xor_sync(0xffffffffu, sd, o);
+                }
+                if (lane == 0) { warp_d[quarter] = n > 0 ? l / (double)n : 0.0; warp_d[4 + quarter] = sd; }
+            }
+        }
+        __syncthreads();
+        if (blockIdx.y == 0 && threadIdx.x < 2) {
+            const double* d = warp_d + 4 * threadIdx.x;
+            p.tile_loss[threadIdx.x * gridDim.x + blockIdx.x] = ((d[0] + d[1]) + d[2]) + d[3];
+        }
+        const float g = ds_s[r_tile];
+        const int64_t out = (int64_t)m * p.h + j0 + cg * UNITS;
+#pragma unroll
+        for (int jj = 0; jj < UNITS; jj += 8) {
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float d_u = g * slope[jj + k];
+                const __nv_bfloat16 top = __float2bfloat16_rn(d_u);
+                const uint32_t h16 = __bfloat16_as_ushort(top), l16 = __bfloat16_as_ushort(__float2bfloat16_rn(d_u - __bfloat162float(top)));
+                hi[k >> 1] = (k & 1) ? hi[k >> 1] | h16 << 16 : h16;
+                lo[k >> 1] = (k & 1) ? lo[k >> 1] | l16 << 16 : l16;
+                gelu_s[(cg * UNITS + jj + k) * TM + r_tile] = live ? g * v[jj + k] : 0.f;       // rows past N: zeros, whatever b1 made of them
+                du_s[(cg * UNITS + jj + k) * TM + r_tile] = live ? d_u : 0.f;
+            }
+            if (live && j0 + cg * UNITS + jj < p.h) {                       // h % 8 == 0
+                *reinterpret_cast<uint4*>(p.du_hi + out + jj) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4*>(p.du_lo + out + jj) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            }
+        }
+        __syncthreads();
+        constexpr int ABREAST = 4;              // a warp per hidden unit, four of them side by side
+        for (int j = ABREAST * warp; j < SBN && j0 + j < p.h; j += ABREAST * S_WARPS) {
+            float sum[2 * ABREAST];
+#pragma unroll
+            for (int i = 0; i < ABREAST; ++i) {
+                const float* a = gelu_s + (j + i) * TM + lane;
+                const float* b = du_s + (j + i) * TM + lane;
+                sum[2 * i] = (a[0] + a[32]) + (a[64] + a[96]);
+                sum[2 * i + 1] = (b[0] + b[32]) + (b[64] + b[96]);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < 2 * ABREAST; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
+            if (lane < 2)                       // j0 + j + 3 < h: h % 8 == 0
+                *reinterpret_cast<float4*>(p.tile_sums + ((int64_t)lane * gridDim.x + blockIdx.x) * p.h + j0 + j) =
+                    lane == 0 ? make_float4(sum[0], sum[2], sum[4], sum[6]) : make_float4(sum[1], sum[3], sum[5], sum[7]);
         }
     }
     if (threadIdx.x == 0 && *abort_flag) atomicOr(p.d_status, ARROL_DEV_WAIT_EXPIRED);
@@ -329,7 +459,7 @@ int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&ctx->score_max_clusters[blocks], score_mlp_tc_kernel<64, true>, &cfg));
+        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&ctx->score_max_clusters[blocks], score_mlp_tc_kernel<64, SCORES>, &cfg));
     }
     *fit = ctx->score_max_clusters[blocks];
     return ARROL_OK;
@@ -337,12 +467,10 @@ int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
 
 }  // namespace
 
-// Scores of a bf16 MLP head on the tensor cores.  Returns ARROL_ERR_UNSUPPORTED (nothing launched) when the sizes
-// do not fit the context's buffers; the caller then takes the SIMT path.  Indexed rows are left packed as bf16
-// [N][d] in the context's packing buffer (the head training step's second contraction reads them there).
-int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index,
-                                int N, const arrol_head* head, int B, const float* q_lut, float* score, float* prob,
-                                int32_t* bin, float* q, float* u_out, cudaStream_t s) {
+// Launches the packing kernel and the contraction in one of its modes; p holds the mode's own outputs.  ARROL_ERR_UNSUPPORTED
+// (nothing launched) when the sizes do not fit the context's buffers, or the mode.
+static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
+                         const arrol_head* head, bool train, ScoreTcParams& p, cudaStream_t s) {
     const int d = head->d, h = head->h;
     const int subs = (h + SUB_H - 1) / SUB_H;
     const int m_tiles = (N + TM - 1) / TM;
@@ -352,10 +480,10 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     if (pack && (size_t)N * (size_t)d * 2 > ARROL_PACK_BYTES) return ARROL_ERR_UNSUPPORTED;
     if (!row_index && ((uint64_t)row_stride * 2) >= (1ull << 40)) return ARROL_ERR_UNSUPPORTED;
     if (!ctx->score_tc_smem_set) {      // once per context: this call is on the prune step's microsecond path
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
-        ARROL_CUDA_OK(cudaFuncSetAttribute(score_mlp_tc_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
+        for (const auto f : {score_mlp_tc_kernel<64, PARTIALS>, score_mlp_tc_kernel<64, SCORES>, score_mlp_tc_kernel<64, TRAIN>})
+            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
+        for (const auto f : {score_mlp_tc_kernel<128, PARTIALS>, score_mlp_tc_kernel<128, SCORES>, score_mlp_tc_kernel<128, TRAIN>})
+            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
         ctx->score_tc_smem_set = true;
     }
     // Tiles of 64 hidden units while they fit one wave of blocks (more SMs share the way in for the operands), of 128 beyond
@@ -363,8 +491,12 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     // not filled by clusters of any size.  Without / with the wide tiles (rows packed before, partial sums through global memory):
     // N = 4,096, d = 4,096, h = 512 39.0 -> 28.4 us (8 of them the packing), N = 8,192 80.7 -> 64.7, N = 3,000, d = 1,024
     // 17.1 -> 14.6; within one wave they lose: N = 2,048, d = 2,048, h = 256 14.2 -> 15.1.
-    const bool cluster = subs <= MAX_SUBS;
+    // Up to eight blocks of 64 are a cluster, or of 128; nine to sixteen blocks of 64 that fit one wave stay without (N = 300, d = 4,096,
+    // h = 1,024 15.7 us, as cluster of wide ones 17.1), but for the training step, which needs the cluster (N = 300, d = 512, h = 1,024
+    // 23.8 -> 21.2).
     bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
+    const bool cluster = subs <= 8 || (subs <= MAX_SUBS && (wide || train));
+    if (train && (!cluster || h % 8 != 0)) return ARROL_ERR_UNSUPPORTED;
     if (cluster && !wide && subs > 1) {
         int fit = 0;                    // clusters of more than eight blocks are not portable
         if (subs <= 8 && narrow_clusters(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
@@ -386,7 +518,6 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     if (make_map(ctx, &map_w, head->W1, (uint64_t)h, (uint64_t)d, wide ? 128 : 64) != ARROL_OK) return ARROL_ERR_CUDA;
     if (make_map_ld(ctx, &map_x, x, (uint64_t)N, (uint64_t)d, (uint64_t)ld, TM) != ARROL_OK) return ARROL_ERR_CUDA;
 
-    ScoreTcParams p;
     p.N = N;
     p.h = h;
     p.k_steps = (d + BK - 1) / BK;
@@ -394,14 +525,7 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     p.w2 = static_cast<const __nv_bfloat16*>(head->w2);
     p.b2 = static_cast<const __nv_bfloat16*>(head->b2);
     p.partial = ctx->d_scratch;
-    p.u_out = u_out;
     p.counters = ctx->d_tile_counters;
-    p.B = B;
-    p.q_lut = q_lut;
-    p.score = score;
-    p.prob = prob;
-    p.bin = bin;
-    p.q = q;
     p.d_status = ctx->d_status;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)m_tiles, (unsigned)tiles_h);
@@ -417,9 +541,46 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = cluster ? 2 : 1;
-    const auto kernel = cluster ? (wide ? score_mlp_tc_kernel<128, true> : score_mlp_tc_kernel<64, true>)
-                                : (wide ? score_mlp_tc_kernel<128, false> : score_mlp_tc_kernel<64, false>);
+    const Mode mode = train ? TRAIN : cluster ? SCORES : PARTIALS;
+    const auto kernel = wide ? (mode == TRAIN ? score_mlp_tc_kernel<128, TRAIN> : mode == SCORES ? score_mlp_tc_kernel<128, SCORES>
+                                                                                          : score_mlp_tc_kernel<128, PARTIALS>)
+                             : (mode == TRAIN ? score_mlp_tc_kernel<64, TRAIN> : mode == SCORES ? score_mlp_tc_kernel<64, SCORES>
+                                                                                         : score_mlp_tc_kernel<64, PARTIALS>);
     ARROL_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, map_x, map_w, p));
     ctx->launches += 1;
     return ARROL_OK;
+}
+
+// Scores of a bf16 MLP head on the tensor cores.  Returns ARROL_ERR_UNSUPPORTED (nothing launched) when the sizes
+// do not fit the context's buffers; the caller then takes the SIMT path.  Indexed rows are left packed as bf16
+// [N][d] in the context's packing buffer (the head training step's second contraction reads them there).
+// u_out [N][h]: the pre-activations as well, of more than 1,024 hidden units only.
+int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index,
+                                int N, const arrol_head* head, int B, const float* q_lut, float* score, float* prob,
+                                int32_t* bin, float* q, float* u_out, cudaStream_t s) {
+    if (u_out && head->h <= MAX_SUBS * SUB_H) return ARROL_ERR_UNSUPPORTED;
+    ScoreTcParams p = {};
+    p.u_out = u_out;
+    p.B = B;
+    p.q_lut = q_lut;
+    p.score = score;
+    p.prob = prob;
+    p.bin = bin;
+    p.q = q;
+    return launch_mlp_tc(ctx, hidden, row_stride, row_index, N, head, false, p, s);
+}
+
+// The head training step up to the dW1 contraction, for at most 1,024 hidden units, a multiple of 8: du as two bf16 planes [N][h]; per tile of
+// 128 rollouts what dw2 and db1 (tile_sums [2][tiles][h]), loss and db2 (tile_loss [2][tiles]) are the sums of.  Rows as above.
+int arrol_internal_head_train_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
+                                 const arrol_head* head, const float* rewards, const uint8_t* mask, void* du_hi, void* du_lo,
+                                 float* tile_sums, double* tile_loss, cudaStream_t s) {
+    ScoreTcParams p = {};
+    p.rewards = rewards;
+    p.mask = mask;
+    p.du_hi = static_cast<__nv_bfloat16*>(du_hi);
+    p.du_lo = static_cast<__nv_bfloat16*>(du_lo);
+    p.tile_sums = tile_sums;
+    p.tile_loss = tile_loss;
+    return launch_mlp_tc(ctx, hidden, row_stride, row_index, N, head, true, p, s);
 }

@@ -50,9 +50,10 @@ def test_head_grad_matches_oracle(N, d, h, dtype, use_mask):
 
 
 # the MLP head's tensor-core path at its edges: one rollout, a K step of 64 rollouts and one more, hidden units and columns that do
-# not fill a tile, K split over 1, 2 and 4 blocks, column tiles of 128 (more tiles of 64 than SMs), a run longer than one pass
+# not fill a tile, K split over 1, 2, 4 and 8 blocks, column tiles of 128 (more tiles of 64 than SMs), more than 32 tiles of rollouts, the most
+# hidden units whose blocks form a cluster and more
 @pytest.mark.parametrize("N,d,h", [(1, 64, 8), (64, 72, 136), (65, 200, 128), (300, 264, 264), (1100, 128, 64), (700, 2048, 640),
-                                   (2500, 520, 16)])
+                                   (2500, 520, 16), (4200, 64, 136), (2100, 128, 72), (130, 72, 1024), (40, 64, 1032)])
 def test_head_grad_at_the_edges_of_its_tiles(N, d, h):
     test_head_grad_matches_oracle(N, d, h, torch.bfloat16, N % 2 == 0)
 
