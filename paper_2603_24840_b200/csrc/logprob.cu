@@ -73,8 +73,9 @@ static_assert(PAIR_STAGES * PAIR_STAGE_BYTES == SOLO_STAGES * SOLO_STAGE_BYTES, 
 constexpr int TMEM_COLS = 512;   // two fp32 accumulators of BN columns
 constexpr int num_threads(int halves) { return 64 + 128 * halves; }     // producer, issuer, four epilogue warps per column half
 constexpr long long STEP_WAIT_CYCLES = 100000;   // what a producer waits at least for the others of its wave (50 us or more)
-constexpr int COMBINE_BLOCKS = 16;           // blocks of segments (n_mid) that one warp merges side by side
-constexpr size_t SMEM_BYTES = (size_t)SOLO_STAGES * SOLO_STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */;
+constexpr int ITEMS_AHEAD = 64;              // work items of a unit that are listed in shared memory
+constexpr size_t SMEM_BYTES = (size_t)SOLO_STAGES * SOLO_STAGE_BYTES + 1024 /* alignment slack */ + 256 /* barriers */ +
+                              ITEMS_AHEAD * 28 /* WorkItem */;
 
 struct PartialLse {   // of one token over some columns: running maximum and sum in the base-2 domain, target logit,
     float m2, l, zy2, sumz;   // sum of the raw accumulators (only when the confidence is asked for)
@@ -87,12 +88,16 @@ __device__ __forceinline__ int quotient(int a, float inv_b) { return (int)(((flo
 // How the vocabulary is cut: total_chunks chunks of BN columns -> n_sub segments -> n_mid blocks of segments -> splits
 // groups.  A body item covers a whole group, a tail item one segment; a token's records are merged segment by segment
 // into a block, block by block into a group, then group by group, by whichever kernel holds them.
+constexpr int MAX_SPLITS = 64;
 struct VocabPlan {
     int total_chunks, n_sub, n_mid, splits;
-    int n_long;           // segments that hold a chunk more than the others: total_chunks mod n_sub
-    float inv_long, inv_short;   // 1 / n_long, 1 / (n_sub - n_long)
-    // n_sub <= SMs and total_chunks < 2^23: the product stays below 2^31 for any vocabulary that a TMA coordinate reaches
-    __host__ __device__ int chunk_of_sub(int i) const { return (int)((unsigned)i * (unsigned)total_chunks / (unsigned)n_sub); }
+    int per_sub;          // whole chunks per segment, n_long segments hold one more
+    int n_long;           // total_chunks mod n_sub
+    float inv_sub, inv_long, inv_short;   // 1 / n_sub, 1 / n_long, 1 / (n_sub - n_long)
+    uint8_t mid_begin[MAX_SPLITS + 1];    // first segment of every block of segments (n_sub <= SMs < 256)
+    uint8_t group_begin[MAX_SPLITS + 1];  // first block of every group
+    // floor(i total_chunks / n_sub), without a division
+    __device__ int chunk_of_sub(int i) const { return i * per_sub + quotient(i * n_long, inv_sub); }
     // j-th segment in the order of dealing: the long ones first.  Segment i is long where floor(i n_long / n_sub) steps after i,
     // short where ceil(i (n_sub - n_long) / n_sub) does.
     __device__ int nth_sub(int j) const {
@@ -100,9 +105,7 @@ struct VocabPlan {
         const int a = is_long ? (j + 1) * n_sub + n_long - 1 : (j - n_long) * n_sub;
         return quotient(a, is_long ? inv_long : inv_short) - (is_long ? 1 : 0);
     }
-    __host__ __device__ int sub_of_mid(int i) const { return i * n_sub / n_mid; }
-    __host__ __device__ int mid_of_group(int g) const { return g * n_mid / splits; }
-    __host__ __device__ int sub_of_group(int g) const { return sub_of_mid(mid_of_group(g)); }
+    __device__ int sub_of_group(int g) const { return mid_begin[group_begin[g]]; }
 };
 
 // (M, L) <- (M, L) + (m, l): M = max, L = sum of 2^(. - M).  One rounding per operation, so that the main kernel (body)
@@ -140,6 +143,7 @@ __host__ __device__ inline WorkList make_work_list(int tiles, int units, const V
 struct WorkItem {
     int tile, wave;
     int group, sub0, sub1;      // group < 0: a tail item
+    int c0, c1;                 // chunks of columns
 };
 // k-th item of a unit; false when it has none left.  The tail walks the segments as the slow index: at any time the
 // units work on neighbouring segments of all tail tiles and share W_vocab through L2.  The segments that are a chunk longer go
@@ -155,6 +159,8 @@ __device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v,
         it.group = i - it.tile * v.splits;
         it.sub0 = v.sub_of_group(it.group);
         it.sub1 = v.sub_of_group(it.group + 1);
+        it.c0 = v.chunk_of_sub(it.sub0);
+        it.c1 = v.chunk_of_sub(it.sub1);
         return true;
     }
     i -= w.body_items;
@@ -164,6 +170,8 @@ __device__ __forceinline__ bool work_item(const WorkList& w, const VocabPlan& v,
     it.sub1 = it.sub0 + 1;
     it.tile = w.body_tiles + (i - turn * w.tail_tiles);
     it.group = -1;
+    it.c0 = v.chunk_of_sub(it.sub0);
+    it.c1 = v.chunk_of_sub(it.sub1);
     return true;
 }
 
@@ -173,6 +181,7 @@ struct LogprobParams {
     int64_t T_max;
     int d, V;
     VocabPlan plan;
+    WorkList work;         // of T_max tokens
     float scale2;          // inv_temperature * log2(e)
     PartialLse* body;      // [splits][column halves][T_max]: records of the tokens in whole waves
     PartialLse* tail;      // [token of the tail][n_sub][column halves]
@@ -264,7 +273,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
     constexpr int STAGES = PAIR ? PAIR_STAGES : SOLO_STAGES;
     constexpr int B_STAGE_BYTES = PAIR ? PAIR_B_STAGE_BYTES : SOLO_B_STAGE_BYTES;
     constexpr int STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES;
-    constexpr int EPI_WARPS = 4 * HALVES, EPI_COLS = BN / HALVES;
+    constexpr int EPI_WARPS = 4 * HALVES, EPI_COLS = BN / HALVES, TILE_ROWS = PAIR ? 2 * BM : BM;
     extern __shared__ uint8_t smem_raw[];
     // stage buffers need 1024-byte alignment for the 128-byte swizzle pattern
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -278,6 +287,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
     uint64_t* drain = acc_empty + 2;          // [1]       used only when giving up: MMAs in flight -> done
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile uint32_t* abort_flag = tmem_slot + 1;
+    WorkItem* items_s = reinterpret_cast<WorkItem*>(smem + (size_t)STAGES * STAGE_BYTES + 256);   // [ITEMS_AHEAD] this unit's first items
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // pair: rank of this block in its cluster (block 0 leads), unit = cluster; otherwise unit = block
@@ -302,6 +312,22 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
         if constexpr (PAIR) { tcgen05_alloc_pair(tmem_slot, TMEM_COLS); tcgen05_relinquish_pair(); }
         else { tcgen05_alloc(tmem_slot, TMEM_COLS); tcgen05_relinquish(); }
     }
+    // The unit's first items, a thread each.  Every role would work them out for itself, one behind the other, and the first time
+    // through that code costs a microsecond of instruction and constant fetches: here it overlaps the preceding kernel.
+    WorkList work = p.work;
+    auto list_items = [&] {
+        if (threadIdx.x < ITEMS_AHEAD) {
+            WorkItem it = {};
+            if (!work_item(work, p.plan, unit, units, threadIdx.x, it)) it.c0 = it.c1 = -1;
+            items_s[threadIdx.x] = it;
+        }
+    };
+    list_items();
+    auto get_item = [&](int k, WorkItem& it) {
+        if (k >= ITEMS_AHEAD) return work_item(work, p.plan, unit, units, k, it);
+        it = items_s[k];
+        return it.c0 >= 0;
+    };
     tcgen05_fence_before();
     __syncthreads();
     if constexpr (PAIR) cluster_sync_all();     // the peer's barriers exist before anything arrives on them
@@ -316,9 +342,16 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
     pdl_launch_dependents();       // the combining kernel may be set up while this one runs
     pdl_wait();                    // the set-up above overlaps the end of the preceding kernel
     int64_t T = p.T_max;
-    if (p.d_T) { const int64_t t = *pdl_acquire(p.d_T); T = t < 0 ? 0 : (t < T ? t : T); }
-    const int m_tiles = (int)((T + BM - 1) / BM);
-    const WorkList work = make_work_list(PAIR ? (m_tiles + 1) / 2 : m_tiles, units, p.plan);
+    if (p.d_T) {
+        const int64_t t = *pdl_acquire(p.d_T);
+        T = t < 0 ? 0 : (t < T ? t : T);
+        const int tiles = (int)((T + TILE_ROWS - 1) / TILE_ROWS);
+        if (tiles != work.body_tiles + work.tail_tiles) {          // uniform over the block
+            work = make_work_list(tiles, units, p.plan);
+            list_items();
+            __syncthreads();
+        }
+    }
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -332,7 +365,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                 return tile_row[PAIR ? 2 * it.tile + (int)rank : it.tile];
             };
             WorkItem it, next;
-            bool have = !p.mute_producer && work_item(work, p.plan, unit, units, 0, it);
+            bool have = !p.mute_producer && get_item(0, it);
             int row = 0;
             if constexpr (GATHER) if (have) row = source_row(it);
             int arrived = 0, waited = 0;            // waves
@@ -357,10 +390,9 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                     waited = wave;
                     item_begun = now;
                 }
-                const bool have_next = work_item(work, p.plan, unit, units, k + 1, next);
+                const bool have_next = get_item(k + 1, next);
                 int row_next = 0;
                 if constexpr (GATHER) if (have_next) row_next = source_row(next);
-                const int c0 = p.plan.chunk_of_sub(it.sub0), c1 = p.plan.chunk_of_sub(it.sub1);
                 // where the tile's 128 rows come from: the packed rows, a run of source rows, or a scratch slot
                 const CUtensorMap* a_map = &map_h;
                 int a_row = (PAIR ? 2 * it.tile + (int)rank : it.tile) * BM;
@@ -368,7 +400,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                     a_row = row;
                     if (row < 0) { a_map = &map_s; a_row = ~row; }
                 }
-                for (int c = c0; c < c1 && ok; ++c) {
+                for (int c = it.c0; c < it.c1 && ok; ++c) {
                     for (int ks = 0; ks < k_steps; ++ks) {
                         if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
                         if constexpr (PAIR) {
@@ -420,9 +452,8 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
             uint32_t acc = 0, acc_phase = 0;
             bool ok = true;
             WorkItem it;
-            for (int k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
-                const int c0 = p.plan.chunk_of_sub(it.sub0), c1 = p.plan.chunk_of_sub(it.sub1);
-                for (int c = c0; c < c1 && ok; ++c) {
+            for (int k = 0; ok && get_item(k, it); ++k) {
+                for (int c = it.c0; c < it.c1 && ok; ++c) {
                     const uint32_t idesc = make_idesc(PAIR ? 2 * BM : BM, chunk_columns(p.V, c));
                     if (!mbar_wait_warp(&acc_empty[acc], acc_phase ^ 1u, abort_flag, p.spin_limit)) { ok = false; break; }
                     tcgen05_fence_after();
@@ -481,39 +512,50 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
         const int32_t* targets = pdl_acquire(p.targets);
         uint32_t acc = 0, acc_phase = 0;
         bool ok = true;
-        WorkItem it;
-        for (int k = 0; ok && work_item(work, p.plan, unit, units, k, it); ++k) {
-            const int64_t t = (int64_t)(PAIR ? 2 * it.tile + (int)rank : it.tile) * BM + row_in_tile;
-            const int y = (t < T) ? targets[t] : -1;
+        auto token_of = [&](const WorkItem& it) { return (int64_t)(PAIR ? 2 * it.tile + (int)rank : it.tile) * BM + row_in_tile; };
+        auto target_of = [&](const WorkItem& it) { const int64_t t = token_of(it); return t < T ? targets[t] : -1; };
+        // The next item and its target are requested before this one's columns: an item of one chunk would wait for them longer
+        // than a quarter of its time.
+        WorkItem it, next;
+        bool have = get_item(0, it), have_next = false;
+        int y = have ? target_of(it) : -1, y_next = -1;
+        for (int k = 0; ok && have; ++k, it = next, y = y_next, have = have_next) {
+            have_next = get_item(k + 1, next);
+            y_next = have_next ? target_of(next) : -1;
+            const int64_t t = token_of(it);
             PartialLse sub = empty_record(), mid = empty_record(), group = empty_record();
             const int64_t stamp_at = (int64_t)it.tile * p.plan.splits + it.group;
             const bool stamp = p.timing != nullptr && threadIdx.x == 64 && rank == 0 && it.group >= 0 && stamp_at < p.timing_items;
             if (stamp) { p.timing[4 * stamp_at] = global_timer_ns(); p.timing[4 * stamp_at + 2] = (unsigned long long)clock64(); }
-            int mid_i = it.group >= 0 ? p.plan.mid_of_group(it.group) : 0;
-            int mid_end = p.plan.sub_of_mid(mid_i + 1);
+            int mid_i = it.group >= 0 ? p.plan.group_begin[it.group] : 0;
+            int mid_end = p.plan.mid_begin[mid_i + 1];
+            int c = it.c0;
             for (int s = it.sub0; s < it.sub1 && ok; ++s) {
-                const int c1 = p.plan.chunk_of_sub(s + 1);
-                for (int c = p.plan.chunk_of_sub(s); c < c1 && ok; ++c) {
+                const int c1 = s + 1 == it.sub1 ? it.c1 : p.plan.chunk_of_sub(s + 1);
+                for (; c < c1 && ok; ++c) {
                     ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit);
                     ok = __all_sync(0xffffffffu, ok) != 0;     // keep the warp converged for the aligned tensor-memory loads
                     if (!ok) break;
                     tcgen05_fence_after();
                     const int col0 = c * BN + half * EPI_COLS;
+                    const int pieces = min(EPI_COLS / 32, (p.V - col0 + 31) / 32);        // none past the vocabulary
+                    auto hand_back = [&] {
+                        tcgen05_fence_before();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if constexpr (PAIR) mbar_arrive_cluster(lead_acc_empty0 + acc * (uint32_t)sizeof(uint64_t));
+                            else mbar_arrive(&acc_empty[acc]);
+                        }
+                    };
 #pragma unroll 1
-                    for (int piece = 0; piece < EPI_COLS / 32; ++piece) {
-                        const int pc0 = col0 + piece * 32;
-                        if (pc0 >= p.V) break;                  // columns past the vocabulary
+                    for (int piece = 0; piece < pieces; ++piece) {
                         uint32_t v[32];
                         tcgen05_ld_32x32_issue(tmem_base + lane_addr + acc * BN + half * EPI_COLS + piece * 32, v);
                         tcgen05_ld_wait(v);
-                        accumulate_piece<CONF>(v, pc0, y, p.V, p.scale2, sub);
+                        if (piece + 1 == pieces) hand_back();
+                        accumulate_piece<CONF>(v, col0 + piece * 32, y, p.V, p.scale2, sub);
                     }
-                    tcgen05_fence_before();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if constexpr (PAIR) mbar_arrive_cluster(lead_acc_empty0 + acc * (uint32_t)sizeof(uint64_t));
-                        else mbar_arrive(&acc_empty[acc]);
-                    }
+                    if (pieces <= 0) hand_back();
                     if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
                 }
                 if (it.group >= 0) {                           // the segment is complete: segment -> block -> group
@@ -522,7 +564,7 @@ token_logprob_kernel(const __grid_constant__ CUtensorMap map_h, const __grid_con
                     if (s + 1 == mid_end) {
                         merge_record(group, mid);
                         mid = empty_record();
-                        mid_end = p.plan.sub_of_mid(++mid_i + 1);
+                        if (s + 1 < it.sub1) mid_end = p.plan.mid_begin[++mid_i + 1];
                     }
                 }
             }
@@ -621,35 +663,45 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
     }
 }
 
-// Merges every token's records.  Tokens of the body: one thread each, splits x HALVES records.  Tokens of the tail: one
-// warp each; lane (block of segments, column half) merges its segments, then all lanes walk the blocks in order.
-// AHEAD: a lane has all records of its block on their way before it merges the first (148 segments in 16 blocks are ten at most).  It
-// takes 102 registers where the other loop takes 60, and that is what counts: one block waits on every SM beside the log-prob
-// kernel, and of those past them (a warp merges a token) up to three more go to the SM that is free first, whose 32 warps then merge
-// one another out of the way; of AHEAD's only one.  So it is taken where the tail has more blocks than that, and no more than two an SM, past
-// which they take a wave more.  Whole call without / with it, d = 256, V = 6,000 (us): 148 blocks (1,184 tokens) 14.3 / 15.0, 149
-// 14.7 / 14.9, 150 15.8 / 15.0, 151 17.1 / 14.9, 256 19.9 / 17.8, 296 21.6 / 20.0, 297 21.7 / 22.7, 5,000 tokens 31.3 / 35.0; V = 32,379: 1,280 tokens
-// 35.7 / 32.1, 2,048 46.8 / 43.4, 2,500 54.8 / 55.6, 5,000 95.4 / 98.0.  T_max draws the line: 300 live tokens of 2,048 at V = 16,640 14.4 / 15.1.
-constexpr int COMBINE_THREADS = 256, COMBINE_AHEAD = 10;
-template <int HALVES, bool AHEAD>
-__global__ void __launch_bounds__(COMBINE_THREADS)
+// Merges every token's records.  Tokens of the body: one thread each, splits x HALVES records.  Tokens of the tail: a block takes
+// `group` consecutive ones, whose records lie one after another and come into shared memory by asynchronous copies; a thread
+// merges the segments of one block of segments (and column half), then a thread per token and half walks the blocks in order.
+// Bound by latency: one round trip for the length, the targets and the records together (where no call of T_max tokens has a body the
+// records' place does not depend on the length), then some 25 dependent merges of 50 cycles.  Registers and shared memory leave
+// room for one block beside the log-prob kernel's on every SM, where it waits; blocks past that would pile up on the SM that is
+// free first.  A warp per token, its lanes the blocks of segments and then all of them the same chain of 16 merges, took 4.5 to 6.5 us
+// of a call of 2,800 tokens on V = 4,096 (d = 256), and takes 2.8 to 3.4 now.  With the items listed ahead the whole call went from 18.9 to
+// 14.4 us (graph of 20), 3,636 tokens at d = 320 on V = 14,170 from 41.9 to 35.0.
+constexpr int COMBINE_THREADS = 256;
+constexpr int COMBINE_GROUP = 32;                  // most tokens per block
+constexpr size_t COMBINE_SMEM = 32 * 1024;
+// tokens of the tail per block, `per_token` records each
+__host__ __device__ inline size_t combine_bytes(const VocabPlan& v, int halves) { return (size_t)(v.n_sub + (v.n_mid < v.n_sub ? v.n_mid : 0)) * halves * 16; }
+template <int HALVES>
+__global__ void __launch_bounds__(COMBINE_THREADS, 4)
 combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
-                      int64_t T_max, int V, VocabPlan plan, int tile_rows, int units, float* __restrict__ logp,
-                      float* __restrict__ lse, float* __restrict__ conf, float inv_temp, uint32_t* d_status) {
+                      int64_t T_max, int V, VocabPlan plan, int tile_rows, int units, int group, int block_lanes, bool tail_only,
+                      float* __restrict__ logp, float* __restrict__ lse, float* __restrict__ conf, float inv_temp, uint32_t* d_status) {
+    extern __shared__ __align__(16) float4 records_s[];    // [group][n_sub][HALVES], then [group][n_mid][HALVES] where that is less
     pdl_wait();
     body = pdl_acquire(body); tail = pdl_acquire(tail); targets = pdl_acquire(targets); d_T = pdl_acquire(d_T);
+    const int tid = threadIdx.x;
+    const int per_token = plan.n_sub * HALVES;
+    auto fetch = [&](int64_t row0, int n) {
+        const float4* from = reinterpret_cast<const float4*>(tail + row0 * per_token);
+        for (int i = tid; i < n * per_token; i += COMBINE_THREADS) cp_async_16(records_s + i, from + i);
+    };
+    const int64_t first = (int64_t)blockIdx.x * group;
+    if (tail_only && first < T_max) fetch(first, (int)min((int64_t)group, T_max - first));
     int64_t T = T_max;
     if (d_T) { const int64_t t = *d_T; T = t < 0 ? 0 : (t < T ? t : T); }
     const WorkList work = make_work_list((int)(((unsigned)T + tile_rows - 1) / (unsigned)tile_rows), units, plan);   // T < 2^31
     const int64_t body_rows = min(T, (int64_t)work.body_tiles * tile_rows);
-    auto load = [](const PartialLse* p) {
-        const float4 r = *reinterpret_cast<const float4*>(p);
+    auto load = [](const float4* p) {
+        const float4 r = *p;
         return PartialLse{r.x, r.y, r.z, r.w};
     };
-    auto finish = [&](int64_t t, int y, const PartialLse (&halves)[HALVES]) {
-        PartialLse r = halves[0];
-#pragma unroll
-        for (int h = 1; h < HALVES; ++h) merge_record(r, halves[h]);
+    auto finish = [&](int64_t t, int y, const PartialLse& r) {
         const float lse2 = r.m2 + log2f(r.l);
         const float ln2 = 0.69314718055994530942f;
         float out = 0.f;
@@ -661,7 +713,7 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
         if (lse) lse[t] = lse2 * ln2;
         if (conf) conf[t] = (float)V * (lse2 * ln2) - r.sumz * inv_temp;
     };
-    const int64_t thread = blockIdx.x * (int64_t)COMBINE_THREADS + threadIdx.x;
+    const int64_t thread = blockIdx.x * (int64_t)COMBINE_THREADS + tid;
     const int64_t threads = (int64_t)gridDim.x * COMBINE_THREADS;
     for (int64_t t = thread; t < body_rows; t += threads) {
         const int y = targets[t];
@@ -670,55 +722,53 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
         for (int h = 0; h < HALVES; ++h) total[h] = empty_record();
         for (int g = 0; g < plan.splits; ++g)
 #pragma unroll
-            for (int h = 0; h < HALVES; ++h) merge_record(total[h], load(body + ((int64_t)g * HALVES + h) * T_max + t));
-        finish(t, y, total);
+            for (int h = 0; h < HALVES; ++h)
+                merge_record(total[h], load(reinterpret_cast<const float4*>(body + ((int64_t)g * HALVES + h) * T_max + t)));
+#pragma unroll
+        for (int h = 1; h < HALVES; ++h) merge_record(total[0], total[h]);
+        finish(t, y, total[0]);
     }
-    const int lane = threadIdx.x & 31;
-    for (int64_t t = body_rows + (thread >> 5); t < T; t += threads >> 5) {
-        const PartialLse* rec = tail + (t - body_rows) * plan.n_sub * HALVES;
-        const int y = targets[t];                // requested now, used at the end
-        PartialLse total[HALVES], group[HALVES];
-#pragma unroll
-        for (int h = 0; h < HALVES; ++h) total[h] = group[h] = empty_record();
-        int g = 0, group_end = plan.mid_of_group(1);
-        for (int base = 0; base < plan.n_mid; base += COMBINE_BLOCKS) {
-            const int b = base + lane / HALVES;
-            PartialLse mine = empty_record();
-            if (b < plan.n_mid && lane < COMBINE_BLOCKS * HALVES) {
-                const int s1 = plan.sub_of_mid(b + 1);
-                if constexpr (AHEAD) {
-                    for (int s = plan.sub_of_mid(b); s < s1; s += COMBINE_AHEAD) {
-                        PartialLse r[COMBINE_AHEAD];
-#pragma unroll
-                        for (int k = 0; k < COMBINE_AHEAD; ++k)
-                            if (s + k < s1) r[k] = load(rec + (s + k) * HALVES + lane % HALVES);
-#pragma unroll
-                        for (int k = 0; k < COMBINE_AHEAD; ++k)
-                            if (s + k < s1) merge_record(mine, r[k]);
-                    }
-                } else {
+    const int per_block = plan.n_mid * HALVES, lanes = 1 << block_lanes;       // lanes >= per_block
+    float4* blocks_s = plan.n_mid < plan.n_sub ? records_s + group * per_token : records_s;
+    for (int64_t row0 = first; row0 < T - body_rows; row0 += (int64_t)gridDim.x * group) {
+        const int n = (int)min((int64_t)group, T - body_rows - row0);
+        if (!tail_only) fetch(row0, n);
+        const int token = tid / HALVES, h = tid % HALVES;
+        const int y = token < n ? targets[body_rows + row0 + token] : -1;           // requested now, used at the end
+        cp_async_wait_all();
+        __syncthreads();
+        if (plan.n_mid < plan.n_sub) {
+            const int i = tid & (lanes - 1), b = i / HALVES;
+            if (i < per_block)
+                for (int of = tid >> block_lanes; of < n; of += COMBINE_THREADS >> block_lanes) {
+                    const float4* rec = records_s + of * per_token + i % HALVES;
+                    PartialLse mine = empty_record();
+                    const int s1 = plan.mid_begin[b + 1];
 #pragma unroll 4
-                    for (int s = plan.sub_of_mid(b); s < s1; ++s) merge_record(mine, load(rec + s * HALVES + lane % HALVES));
+                    for (int s = plan.mid_begin[b]; s < s1; ++s) merge_record(mine, load(rec + s * HALVES));
+                    blocks_s[of * per_block + i] = make_float4(mine.m2, mine.l, mine.zy2, mine.sumz);
                 }
-            }
-            const int in_base = min(COMBINE_BLOCKS, plan.n_mid - base);
-#pragma unroll 4
-            for (int j = 0; j < in_base; ++j) {
-#pragma unroll
-                for (int h = 0; h < HALVES; ++h) {
-                    const int from = j * HALVES + h;
-                    merge_record(group[h], PartialLse{__shfl_sync(0xffffffffu, mine.m2, from), __shfl_sync(0xffffffffu, mine.l, from),
-                                                      __shfl_sync(0xffffffffu, mine.zy2, from), __shfl_sync(0xffffffffu, mine.sumz, from)});
-                }
-                if (base + j + 1 == group_end) {
-#pragma unroll
-                    for (int h = 0; h < HALVES; ++h) { merge_record(total[h], group[h]); group[h] = empty_record(); }
-                    ++g;
-                    group_end = plan.mid_of_group(g + 1);
-                }
-            }
+            __syncthreads();
         }
-        if (lane == 0) finish(t, y, total);
+        // warps come along whole
+        if (tid / 32 * 32 < n * HALVES) {
+            PartialLse total = empty_record(), in_group = empty_record();
+            if (token < n) {
+                const float4* rec = blocks_s + token * per_block + h;
+                for (int g = 0; g < plan.splits; ++g) {
+                    const int b1 = plan.group_begin[g + 1];
+#pragma unroll 4
+                    for (int b = plan.group_begin[g]; b < b1; ++b) merge_record(in_group, load(rec + b * HALVES));
+                    merge_record(total, in_group);
+                    in_group = empty_record();
+                }
+            }
+            if constexpr (HALVES == 2)
+                merge_record(total, PartialLse{__shfl_down_sync(0xffffffffu, total.m2, 1), __shfl_down_sync(0xffffffffu, total.l, 1),
+                                               __shfl_down_sync(0xffffffffu, total.zy2, 1), __shfl_down_sync(0xffffffffu, total.sumz, 1)});
+            if (token < n && h == 0) finish(body_rows + row0 + token, y, total);
+        }
+        __syncthreads();                    // the records are overwritten by the next ones
     }
 }
 
@@ -778,9 +828,15 @@ VocabPlan plan_for(const arrol_ctx* ctx, int d, int V) {
     v.n_long = v.total_chunks % v.n_sub;
     v.inv_long = v.n_long > 0 ? 1.0f / (float)v.n_long : 0.f;
     v.inv_short = 1.0f / (float)(v.n_sub - v.n_long);
+    v.per_sub = v.total_chunks / v.n_sub;
+    v.inv_sub = 1.0f / (float)v.n_sub;
     if (v.n_sub < v.splits) v.splits = v.n_sub;
-    const int per_group = COMBINE_BLOCKS / v.splits > 1 ? COMBINE_BLOCKS / v.splits : 1;
+    // as many blocks as there are segments in each, so that the two chains of merges together are shortest
+    int per_group = 1;
+    while (v.splits * per_group * v.splits * per_group < v.n_sub) ++per_group;
     v.n_mid = v.splits * per_group < v.n_sub ? v.splits * per_group : v.n_sub;
+    for (int i = 0; i <= v.n_mid; ++i) v.mid_begin[i] = (uint8_t)(i * v.n_sub / v.n_mid);
+    for (int g = 0; g <= v.splits; ++g) v.group_begin[g] = (uint8_t)(g * v.n_mid / v.splits);
     return v;
 }
 
@@ -936,7 +992,8 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     if (units > tiles_max * p.plan.n_sub) units = tiles_max * p.plan.n_sub;
     const int64_t grid = pair ? 2 * units : units;
     // more than one wave: the blocks are kept in step, and should all be resident (single blocks: cooperative launch)
-    const bool several_waves = make_work_list((int)tiles_max, (int)units, p.plan).waves > 1;
+    p.work = make_work_list((int)tiles_max, (int)units, p.plan);
+    const bool several_waves = p.work.waves > 1;
     if (several_waves) ARROL_CUDA_OK(cudaMemsetAsync(p.wave_counter, 0, sizeof(unsigned int), s));
     if (several_waves && !pair) {
         attr[n_attr].id = cudaLaunchAttributeCooperative;
@@ -963,20 +1020,26 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     ARROL_CUDA_OK(cudaLaunchKernelEx(&cfg, fn, map_h, map_s, map_w, p));
     ctx->launches += 1;
     ARROL_CUDA_OK(cudaGetLastError());
-    // one thread per token of the body, one warp per token of the tail
+    // a thread per token of the body; tokens of the tail a few per block, so that the blocks are as many as SMs if they can be
     const int64_t tile_rows = (pair ? 2 : 1) * BM;
-    const int64_t tail_rows = (tiles_max < units / p.plan.splits + 1 ? tiles_max : units / p.plan.splits + 1) * tile_rows;
-    int64_t blocks = (T_max + COMBINE_THREADS - 1) / COMBINE_THREADS;
-    const int64_t tail_blocks = (tail_rows * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
-    if (blocks < tail_blocks) blocks = tail_blocks;
-    if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
-    const int64_t token_blocks = ((T_max < tail_rows ? T_max : tail_rows) * 32 + COMBINE_THREADS - 1) / COMBINE_THREADS;
-    const bool ahead = token_blocks > ctx->sm_count + 1 && token_blocks <= 2 * (int64_t)ctx->sm_count;
-    const auto combine = ahead ? (halves == 2 ? combine_splits_kernel<2, true> : combine_splits_kernel<1, true>)
-                               : (halves == 2 ? combine_splits_kernel<2, false> : combine_splits_kernel<1, false>);
-    ARROL_CUDA_OK(arrol_launch_pdl(combine, dim3((unsigned)blocks), dim3(COMBINE_THREADS), 0, s,
+    const bool tail_only = p.work.body_tiles == 0;      // fewer tokens have none either
+    int64_t tail_rows = (tiles_max < units / p.plan.splits + 1 ? tiles_max : units / p.plan.splits + 1) * tile_rows;
+    if (tail_rows > T_max) tail_rows = T_max;
+    const size_t token_bytes = combine_bytes(p.plan, halves);
+    int64_t group = (tail_rows + ctx->sm_count - 1) / ctx->sm_count;
+    if (group > COMBINE_GROUP) group = COMBINE_GROUP;
+    if (group > (int64_t)(COMBINE_SMEM / token_bytes)) group = (int64_t)(COMBINE_SMEM / token_bytes);
+    int64_t blocks = (tail_rows + group - 1) / group;
+    int block_lanes = 0;
+    while ((1 << block_lanes) < p.plan.n_mid * halves) ++block_lanes;
+    if (!tail_only) {
+        if (blocks < (T_max + COMBINE_THREADS - 1) / COMBINE_THREADS) blocks = (T_max + COMBINE_THREADS - 1) / COMBINE_THREADS;
+        if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
+    }
+    const auto combine = halves == 2 ? combine_splits_kernel<2> : combine_splits_kernel<1>;
+    ARROL_CUDA_OK(arrol_launch_pdl(combine, dim3((unsigned)blocks), dim3(COMBINE_THREADS), (size_t)group * token_bytes, s,
                                    static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
-                                   T_max, V, p.plan, (int)tile_rows, (int)units, logp, lse, conf, inv_temperature, ctx->d_status));
+                                   T_max, V, p.plan, (int)tile_rows, (int)units, (int)group, block_lanes, tail_only, logp, lse, conf, inv_temperature, ctx->d_status));
     ctx->launches += 1;
     return ARROL_OK;
 }

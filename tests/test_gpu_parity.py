@@ -395,6 +395,14 @@ def test_token_logprob_matches_oracle(ctx, T, d, V):
     _logprob_case(ctx, T, d, V, seed=T + d + V)
 
 
+# the tail alone: more items per unit than are listed ahead (73 tiles of 128 rows, 36 of 256 in pairs, 149 chunks of the vocabulary);
+# one token and three per block of the combining kernel, 148 segments of one chunk and of several; live tokens in fewer tiles than the capacity
+@pytest.mark.parametrize("T,d,V,T_live", [(9344, 64, 38000, None), (9216, 328, 38000, 9000), (150, 64, 38000, 140), (444, 328, 76000, 1),
+                                          (2900, 64, 5000, 130)])
+def test_token_logprob_of_the_tail(ctx, T, d, V, T_live):
+    _logprob_case(ctx, T, d, V, seed=T + d, T_live=T_live, sample=30)
+
+
 def test_token_logprob_dominant_logits_temperature_and_device_T(ctx):
     _logprob_case(ctx, 200, 256, 3000, seed=1, scale=30.0)                   # one logit dominates: lse ~ max
     _logprob_case(ctx, 200, 256, 3000, seed=2, inv_temp=0.6)
