@@ -3,8 +3,11 @@
 //
 // Only what the step needs crosses the bus: the N hidden rows at the detection length (for the head; packed into a
 // pinned staging block on the host and sent as one copy), the small per-rollout arrays, and then -- once the keep
-// mask is known -- the survivors' hidden rows and token ids, which are copied straight into their packed positions
-// (the copy engine does the compaction).  Those uploads run on a
+// mask is known -- the survivors' hidden rows and token ids.  The rows are copied straight into their packed positions (the
+// copy engine does the compaction), a run of survivors that are neighbours in the source as one copy; the ids are packed in the
+// staging block and sent once per chunk.  A copy costs the host 2 to 3 us and the engine about one whatever its size, which is
+// what bounds a step of many short rollouts (copies of their own for ids and rows -> now): 96 survivors of about 93 tokens, d = 2,592
+// 2,352 -> 1,477 us, 192 of 90, d = 2,368 5,880 -> 4,090, 44 of 1,038, d = 640 1,546 -> 1,332.  Those uploads run on a
 // second stream in token chunks, and the log-prob kernel of chunk c starts as soon as chunk c has landed, so the
 // upload of the survivors is hidden behind the tensor-core work.  One host synchronisation in the middle (the mask
 // must reach the host to plan the copies) and one at the end.
@@ -111,16 +114,36 @@ extern "C" int arrol_prune_rebatch_host(arrol_ctx* ctx, const arrol_host_step* s
     if (T > 0 && T <= st->dst_capacity_tokens) {
         const int64_t chunk = chunk_for(T);
         int64_t c = 0;                       // next chunk to launch: tokens [c*chunk, min(T, (c+1)*chunk))
+        const bool stage_ids = (size_t)T * sizeof(int32_t) <= ARROL_STAGE_BYTES;     // the scored rows have left it: the stream is idle
+        int32_t* ids = reinterpret_cast<int32_t*>(ctx->h_stage);
+        int64_t ids_sent = 0;
+        int64_t run_at = 0, run_src = 0, run_len = 0;          // rows that are not sent yet: neighbours in the source
+        auto send_rows = [&]() -> cudaError_t {
+            if (run_len == 0) return cudaSuccess;
+            const size_t bytes = (size_t)run_len * rb;
+            run_len = 0;
+            return cudaMemcpyAsync(d_dst_rows + (size_t)run_at * rb, h_hidden + (size_t)run_src * rb, bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
+        };
         for (size_t k = 0; k < surv.size(); ++k) {
-            const int64_t len = cu[k + 1] - cu[k];
+            const int64_t len = cu[k + 1] - cu[k], src = st->h_src_tok_off[surv[k]];
             if (len > 0) {
-                ARROL_CUDA_OK(cudaMemcpyAsync(d_dst_rows + (size_t)cu[k] * rb,
-                                              h_hidden + (size_t)st->h_src_tok_off[surv[k]] * rb, (size_t)len * rb,
-                                              cudaMemcpyHostToDevice, ctx->copy_stream));
-                ARROL_CUDA_OK(cudaMemcpyAsync(st->d_dst_tokens + cu[k], st->h_src_tokens + st->h_src_tok_off[surv[k]],
-                                              (size_t)len * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->copy_stream));
+                if (run_len > 0 && src != run_src + run_len) ARROL_CUDA_OK(send_rows());
+                if (run_len == 0) { run_at = cu[k]; run_src = src; }
+                run_len += len;
+                if (stage_ids)
+                    std::memcpy(ids + cu[k], st->h_src_tokens + src, (size_t)len * sizeof(int32_t));
+                else
+                    ARROL_CUDA_OK(cudaMemcpyAsync(st->d_dst_tokens + cu[k], st->h_src_tokens + src, (size_t)len * sizeof(int32_t),
+                                                  cudaMemcpyHostToDevice, ctx->copy_stream));
             }
             const bool last = (k + 1 == surv.size());
+            if (c * chunk < T && (cu[k + 1] >= (c + 1) * chunk || last)) {       // what the next launches need
+                ARROL_CUDA_OK(send_rows());
+                if (stage_ids && cu[k + 1] > ids_sent)
+                    ARROL_CUDA_OK(cudaMemcpyAsync(st->d_dst_tokens + ids_sent, ids + ids_sent, (size_t)(cu[k + 1] - ids_sent) * sizeof(int32_t),
+                                                  cudaMemcpyHostToDevice, ctx->copy_stream));
+                ids_sent = cu[k + 1];
+            }
             while (c * chunk < T && (cu[k + 1] >= (c + 1) * chunk || last)) {
                 const int64_t t0 = c * chunk, t1 = (t0 + chunk < T) ? t0 + chunk : T;
                 cudaEvent_t ev = ctx->copy_events[c % ARROL_COPY_EVENTS];

@@ -1,5 +1,7 @@
 """arrol_prune_rebatch_host (the whole step from host buffers, uploads overlapped with the log-prob kernel) against
 the oracle and against the device-resident path."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -64,6 +66,28 @@ def test_host_step_matches_device_path_and_oracle(name):
                                      pr.dst_tokens.cpu().numpy()[rows])
     assert np.abs(h["h_logp"].numpy()[rows] - lp_ref).max() <= 2e-3
     assert B.arrol_poll_status(pr.ctx, raise_on_error=False) == 0
+    pr.ctx.close()
+
+
+@pytest.mark.parametrize("all_kept,d", [(True, 64), (False, 64), (True, 8)])
+def test_host_step_sends_neighbours_together(all_kept, d):
+    """Survivors that are neighbours in the source go as one copy, up to the end of a chunk of 18,944 tokens: with every rollout kept
+    the runs are longest and cross the chunks' ends; gaps in the source (a rollout shorter than its slot) and empty rollouts lie among them."""
+    w = dataclasses.replace(synth.WORKLOADS["mini"], P=24, G=8, K=8 if all_kept else 4, L_max=600, len_dist=("uniform", 100, 600), d=d,
+                            V=500, cutoff=40, h=0)
+    inp = host_inputs(w)
+    inp["lengths"][3::7] = 0
+    inp["lengths"][5::7] -= 1
+    pr = PruneRebatch(w, inputs=inp)
+    pr.step()
+    torch.cuda.synchronize()
+    S, T = pr.counts()
+    assert not all_kept or T > 3 * 18944
+    h, dv, _keepalive = _host_step(pr, w)
+    assert h["h_num"].tolist() == [S, T]
+    assert torch.equal(dv["d_dst_tokens"][:T], pr.dst_tokens[:T])
+    assert torch.equal(dv["d_dst_rows"][:T], pr.dst_rows[:T])
+    assert (h["h_logp"][:T] - pr.logp.cpu()[:T]).abs().max().item() <= 1e-4
     pr.ctx.close()
 
 
