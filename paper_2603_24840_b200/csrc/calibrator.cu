@@ -70,10 +70,10 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 
 // One block, bound by latency: a handful of dependent round trips to memory and a serial search.  Every input is read once
 // (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
-// that one block scan ranks all of them, and the bisection is settled in three rounds of 31 points (see below) instead of 64
-// steps.  Per call, in a graph of 20 (with six rounds, separate round trips for mask, bin and reward, and a later one for
-// the evicted entries before): N = 2,048, 128 bins 25.6 -> 15.9 us; N = 32, 64 bins 21.1 -> 12.9; N = 8,192, 256 bins 34.9 -> 23.0; 12 of
-// the 16 us are the search.  More rollouts go through shared memory in pieces of CAL_STAGED,
+// that one block scan ranks all of them, and the bisection is settled in two or three rounds of 31 points (see below) instead of 64
+// steps.  Per call, in a graph of 40 over changing states, mean of six (always three rounds before): N = 2,048, 128 bins 15.7 -> 13.3 us;
+// N = 32, 64 bins 12.5 -> 11.3; N = 8,192, 256 bins 24.5 -> 19.1; N = 3,000, 256 bins, lambda = 1.3 21.7 -> 19.5 (17.4 to 23.8: where
+// the threshold is not among the first neighbours it is three rounds still, with a second chain of additions).  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
 // per thread and scan, as it was before the runs, 460 and 1,570).  An instance each, because the pieces' code in the same one cost
@@ -304,8 +304,10 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
     // ascending order), whatever they are, and at the end the first warp replays the bisection against the two settled points next to
     // the threshold.  E is piecewise linear, and its root needs few rounds:
     //   EVEN      points evenly over the bracket: after it the piece that the root lies on is known
-    //   AROUND    points at growing distances around the root of that piece, with the sum as a butterfly gives it
-    //   ADJACENT  neighbouring values of kappa + x around the root that the sum in index order at the best point gives
+    //   AROUND    the root of that piece, with the sum as a butterfly gives it: 17 neighbouring values of kappa + x, then points at
+    //             growing distances.  The sum in index order is a few roundings from the butterfly's, so that the threshold lies
+    //             among the neighbours most often, and nothing is left to settle
+    //   ADJACENT  where it does not: 31 neighbours around the root that the sum in index order at the best point gives
     // and, where that does not settle all (breakpoints next to the root, or no slope), the 31 midpoints of the replay's next five levels
     // (TREE) until it does: a round of those settles a step at least, so 64 of them are always enough.
     // (Before, midpoints only, but for one round around the linear root: six rounds where three do now, with two replays between.)
@@ -343,12 +345,12 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
                 double a = fmax(known_below, first_lo), b = fmin(known_above, first_hi), at = 0.0, unit = 0.0;
                 if (step >= 64) {
                     kind = DONE;
-                } else if (round < 3) {
+                } else if (round < 3 && !(__dadd_rn(kappa, known_above) <= nextafter(__dadd_rn(kappa, known_below), inf))) {
                     kind = EVEN;
                     if (round > 0 && known_below > -inf && slope_at > 0.0) {
                         at = fmin(fmax(known_below + (goal - sum_at) / slope_at, a), b);
                         kind = round == 2 && sum_in_order ? ADJACENT : AROUND;
-                        unit = kind == AROUND ? 1.0 + lambda : scalbn(1.0, ilogb(fmax(fmax(fabs(kappa + at), fabs(at)), 1e-200)) - 52);
+                        unit = scalbn(1.0, ilogb(fmax(fmax(fabs(kappa + at), fabs(at)), 1e-200)) - 52);
                     }
                 } else {                             // replay as far as the settled points reach
                     const double base_below = __dadd_rn(kappa, known_below), base_above = __dadd_rn(kappa, known_above);
@@ -378,12 +380,11 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
             if (kind == EVEN) {
                 const double t = (double)(wid + 1) * 0.03125;
                 x = (1.0 - t) * round_lo + t * round_hi;
-            } else if (kind == AROUND) {             // 2^-51 ... 2^-44 away, then coarser
-                const int k = i < 0 ? -i : i;
-                const int e = k <= 8 ? k - 52 : (k == 9 ? -42 : k == 10 ? -39 : k == 11 ? -36 : k == 12 ? -32 : k == 13 ? -26 : k == 14 ? -18 : -10);
-                const double off = k == 0 ? 0.0 : scalbn(round_unit, e);
+            } else if (kind == AROUND && (i < -8 || i > 8)) {
+                const int k = i < 0 ? -i : i;        // unit <= (1 + lambda + kappa) 2^-52: past the eighth neighbour
+                const double off = scalbn(1.0 + lambda + fabs(kappa), k == 9 ? -46 : k == 10 ? -43 : k == 11 ? -40 : k == 12 ? -35 : k == 13 ? -28 : k == 14 ? -19 : -10);
                 x = i < 0 ? round_at - off : round_at + off;
-            } else if (kind == ADJACENT) {
+            } else if (kind == ADJACENT || kind == AROUND) {
                 x = round_at + (double)i * round_unit;
             } else {                                 // in-order traversal of the tree of the next five levels' midpoints
                 double a = round_lo, b = round_hi;
