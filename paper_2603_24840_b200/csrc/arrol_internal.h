@@ -53,7 +53,8 @@ constexpr size_t ARROL_PACK_BYTES = (size_t)64 << 20;
 constexpr int ARROL_TILE_COUNTERS = 1024;   // [0, 1020) row tiles of the MLP head
 constexpr int ARROL_HEAD_COUNTERS = ARROL_MAX_H / 32;   // column tiles of the head training step
 constexpr int ARROL_SCORE_ROW_TILES = 1020;
-constexpr int ARROL_CHAIN_BLOCKS = 510;      // blocks of the fused prune step's chained scan (2 + 2 * 510 words = 8 KB)
+constexpr int ARROL_CHAIN_BLOCKS = 510;      // blocks of the fused prune step's chained scan
+constexpr int ARROL_CHAIN_WORDS = 4;         // 8-byte words per block, after two for the call (16 KB)
 
 #define ARROL_CUDA_OK(expr)                      \
     do {                                         \

@@ -80,8 +80,8 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
               cudaMemset(ctx->d_head_counters, 0, ARROL_HEAD_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_tile_counters, ARROL_TILE_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMemset(ctx->d_tile_counters, 0, ARROL_TILE_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
-              cudaMalloc(&ctx->d_chain, (2 + 2 * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
-              cudaMemset(ctx->d_chain, 0, (2 + 2 * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMalloc(&ctx->d_chain, (2 + ARROL_CHAIN_WORDS * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMemset(ctx->d_chain, 0, (2 + ARROL_CHAIN_WORDS * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
               cudaMallocHost(&ctx->h_keep, ARROL_MAX_HOST_N) == cudaSuccess &&
               cudaMallocHost(&ctx->h_stage, ARROL_STAGE_BYTES) == cudaSuccess &&
               cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) == cudaSuccess;

@@ -7,7 +7,7 @@
 // Llama- / Qwen-3-4B-shaped steps, two blocks with three stages 5,288 / 5,708, three blocks with two stages
 // 5,540-5,562 / 6,036-6,082 (the same bytes in flight, more threads issuing copies), four blocks of two 24 KB stages
 // 5,473 / 6,114.  A ring needs at least two stages: a stage is freed when the NEXT store has been issued.
-//   thread 0 (producer)  for each tile: finds the survivors its rows belong to (binary search once, then a forward
+//   thread 0 (producer)  for each tile: finds the survivors its rows belong to (a search by its warp once, then a forward
 //                        walk in cu_seqlens) and issues one bulk load per contiguous source segment into a ring of
 //                        shared-memory stages; completion by transaction count on the stage's mbarrier
 //   thread 32 (storer)   waits for a stage, issues one bulk store of the tile to its (contiguous) destination, and
@@ -51,11 +51,15 @@ __device__ __forceinline__ uint64_t store_policy(bool streamed) {
 // all but the most recent bulk store of this thread have finished reading shared memory
 __device__ __forceinline__ void bulk_wait_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 
-// Largest s in [lo, hi) with cu_seqlens[s] <= t (skips zero-length survivors), given cu_seqlens[lo] <= t < cu_seqlens[hi].
-__device__ __forceinline__ int find_survivor_of(const int64_t* __restrict__ cu_seqlens, int lo, int hi, int64_t t) {
+// Largest s in [lo, hi) with cu_seqlens[s] <= t (skips zero-length survivors), given cu_seqlens[lo] <= t < cu_seqlens[hi], by a whole warp:
+// 32 points a round trip, where a thread halving the range waits for log2(S) of them.
+__device__ __forceinline__ int find_survivor_of(const int64_t* __restrict__ cu_seqlens, int lo, int hi, int64_t t, int lane) {
     while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(cu_seqlens + mid) <= t) lo = mid; else hi = mid;
+        const int stride = (hi - lo + 31) / 32;              // points lo + stride (lane + 1), those below hi
+        const int at = lo + stride * (lane + 1);
+        const int below = __popc(__ballot_sync(0xffffffffu, at < hi && __ldg(cu_seqlens + at) <= t));
+        lo += stride * below;                                // ascending: the ones below come first
+        hi = min(hi, lo + stride);
     }
     return lo;
 }
@@ -91,9 +95,10 @@ gather_rows_bulk_kernel(const int64_t* __restrict__ d_num, const int64_t* __rest
     const int64_t tile_begin = (int64_t)blockIdx.x * per_block;
     const int64_t tile_end = min(n_tiles, tile_begin + per_block);
 
+    int s = 0;
+    if (threadIdx.x < 32 && tile_begin < tile_end) s = find_survivor_of(cu_seqlens, 0, S, tile_begin * tile_rows, threadIdx.x);
     if (threadIdx.x == 0 && tile_begin < tile_end) {
         // ---------------- producer ----------------
-        int s = find_survivor_of(cu_seqlens, 0, S, tile_begin * tile_rows);
         int64_t s_begin = __ldg(cu_seqlens + s), s_end = __ldg(cu_seqlens + s + 1);
         int64_t s_src = __ldg(src_tok_off + __ldg(survivor_idx + s));
         uint32_t stage = 0, phase = 0, issued = 0;

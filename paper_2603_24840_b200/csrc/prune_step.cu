@@ -9,9 +9,9 @@
 //                        leaves q in shared memory; MLP head: q comes from the scoring kernel that ran before (blocks
 //                        of two warps then, always 32 / G groups each).  One or
 //                        two warps run the per-group selection (select_lanes, as select_kernel) and write the keep
-//                        flags.  The first warp then scans the block's rollouts (kept, kept length), publishes the
-//                        block's totals, adds up the totals of the blocks before it as they appear (a chained scan:
-//                        every block only waits for lower-numbered blocks, of at most two per SM), and writes survivor_idx, cu_seqlens and the advantages of its own
+//                        flags.  The first warp then scans the block's rollouts (kept, kept length), adds the block's
+//                        tokens to the sums of the blocks after it, waits until those before have added theirs to its own (a chained scan:
+//                        every block only waits for lower-numbered blocks, of at most two per SM; how many rollouts they keep is known), and writes survivor_idx, cu_seqlens and the advantages of its own
 //                        groups (group_statistics, as scan_adv_kernel); the last block writes {S, T}.  Nothing is
 //                        re-read from global memory and no block waits for the whole grid.  The second warp counts
 //                        the blocks that are done with the chain; the last one clears it for the next call.
@@ -53,22 +53,24 @@ struct FusedParams {
     int64_t* d_num;
     uint32_t* d_status;
     // chained scan: word [0] blocks that are done with it, from LEFT_ONE on those of which a kept rollout left the source (index
-    // check), from EXPIRED_ONE on those that waited in vain; then from [2] per block {kept tokens, kept rollouts}, each with bit 63 set once published; all zero between calls
+    // check), from EXPIRED_ONE on those that waited in vain; then from [2] a word per block, SUM_WORDS apart: the kept tokens of the blocks before
+    // it, from ARRIVED_ONE on how many of these have added theirs; all zero between calls
     unsigned long long* chain;
     uint32_t spin_limit;
     int rest_vecs;             // 16-byte vectors of a row past the first 256 that a warp has room for in shared memory: all of them, or 0
 };
 
 constexpr int LUT_STAGED = 1024;
-constexpr unsigned long long PUBLISHED = 1ull << 63, LEFT_ONE = 1ull << 32, EXPIRED_ONE = 1ull << 48;     // at most ARROL_CHAIN_BLOCKS of either
+constexpr int SUM_WORDS = ARROL_CHAIN_WORDS;       // a sector of its own for every block
+constexpr unsigned long long ARRIVED_ONE = 1ull << 54, LEFT_ONE = 1ull << 32, EXPIRED_ONE = 1ull << 48;     // at most ARROL_CHAIN_BLOCKS of either
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
     unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void red_add_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ unsigned long long count_acq_rel(unsigned long long* p, unsigned long long n) {
     unsigned long long before;
@@ -159,7 +161,7 @@ prune_fused_kernel(const FusedParams p) {
         }
     }
     __syncthreads();
-    unsigned long long* totals = p.chain + 2;
+    unsigned long long* sums = p.chain + 2;
     if (warp == 1) {
         // statistics of the block's groups, one lane per group, while the first warp scans
         if (lane < groups_here) {
@@ -173,10 +175,10 @@ prune_fused_kernel(const FusedParams p) {
         __threadfence_block();
         __syncwarp();                                        // the named barriers want their warps converged
         asm volatile("bar.arrive 1, 64;" ::: "memory");
-        // The block is done with the chain when the first warp has published its totals and read the others'.  The count's release is what
+        // The block is done with the chain when the first warp has added its total to the sums of the blocks after it and read its own.  The count's release is what
         // the clearing rests on: every block's stores have been performed before the last one to be counted zeroes the
-        // words.  Without it the totals of the highest block, which nobody reads, or of a block that another one has given up waiting
-        // for, could land after the zeros and be taken for that block's totals by a later call.  The release waits for
+        // words.  Without it what a block adds to the sum of one that has given up waiting could land after the zeros and be counted by a
+        // later call.  The release waits for
         // those stores, so it is this warp's, beside the outputs that the first one writes.  Graphs of 20 calls, this / with a fence and
         // the count in the first warp / with nothing between stores and count: 2,048 rollouts at d = 2,560 19.5 / 20.3 / 20.1 us, 4,096
         // after an MLP head 70.4 / 70.6 / 70.0, 32 rollouts 9.4 / 10.3 / 9.9.
@@ -185,7 +187,7 @@ prune_fused_kernel(const FusedParams p) {
         if (lane == 0) done = count_acq_rel(p.chain, 1ull + (block_left ? LEFT_ONE : 0ull) + (block_expired ? EXPIRED_ONE : 0ull));
         done = __shfl_sync(0xffffffffu, done, 0);
         if ((done & (LEFT_ONE - 1)) == gridDim.x - 1) {
-            for (unsigned int b = lane; b < 2 * gridDim.x; b += 32) totals[b] = 0ull;
+            for (unsigned int b = lane; b < gridDim.x; b += 32) sums[b * SUM_WORDS] = 0ull;
             if (lane == 0) {
                 const bool left = block_left || done % EXPIRED_ONE >= LEFT_ONE, expired = block_expired || done >= EXPIRED_ONE;
                 if (left) atomicOr(p.d_status, ARROL_DEV_BAD_INDEX);
@@ -203,47 +205,34 @@ prune_fused_kernel(const FusedParams p) {
 
     // ---- first warp: scan of the block's rollouts, chained over the blocks, outputs of the block's groups ----
     const bool kept = lane < n_here && keep_s[lane] != 0;
-    const int32_t own_c = kept ? 1 : 0;
     const int64_t own_t = kept ? (int64_t)len_s[lane] : 0;
     if (kept && p.source_rows > 0) {
         const int64_t o = pdl_acquire(p.src_tok_off)[first + lane];
         bad_index = o < 0 || o + own_t > p.source_rows;
     }
-    int32_t c = own_c;
+    const unsigned int kept_lanes = __ballot_sync(0xffffffffu, kept);
     int64_t t = own_t;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int32_t oc = __shfl_up_sync(0xffffffffu, c, o);
         const int64_t ot = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) { c += oc; t += ot; }
+        if (lane >= o) t += ot;
     }
-    const int32_t block_c = __shfl_sync(0xffffffffu, c, 31);
     const int64_t block_t = __shfl_sync(0xffffffffu, t, 31);
-    if (lane == 0) {
-        st_relaxed_u64(totals + 2 * blockIdx.x, PUBLISHED | (unsigned long long)block_t);
-        st_relaxed_u64(totals + 2 * blockIdx.x + 1, PUBLISHED | (unsigned long long)block_c);
-    }
-    // totals of the blocks before this one (each lane takes every 32nd of them)
-    int64_t base_t = 0;
-    int32_t base_c = 0;
+    const int32_t block_c = __popc(kept_lanes);
+    // The block adds its total to the sums of all blocks after it, and waits for its own sum to be complete: every block polls a word
+    // of its own.  When each read all totals before it, 128 blocks polled the same lines, and the last total took 3.8 us to get
+    // through to them (relaxed loads, eight at a time, 5 us: the more polls the later).
+    for (unsigned int b = blockIdx.x + 1 + lane; b < gridDim.x; b += 32) red_add_u64(sums + (size_t)b * SUM_WORDS, ARRIVED_ONE + (unsigned long long)block_t);
+    unsigned long long sum = 0;
     bool expired = false;
-    for (int b = lane; b < (int)blockIdx.x; b += 32) {
-        unsigned long long wt = 0, wc = 0;
-        uint32_t it = 0;
-        for (;;) {
-            wt = ld_acquire_u64(totals + 2 * b);
-            wc = ld_acquire_u64(totals + 2 * b + 1);
-            if ((wt & wc & PUBLISHED) != 0) break;
+    if (lane == 0 && blockIdx.x > 0)
+        for (uint32_t it = 0;;) {
+            sum = ld_relaxed_u64(sums + (size_t)blockIdx.x * SUM_WORDS);
+            if (sum / ARRIVED_ONE == blockIdx.x) break;
             if (++it >= p.spin_limit) { expired = true; break; }
         }
-        base_t += (int64_t)(wt & ~PUBLISHED);
-        base_c += (int32_t)(wc & ~PUBLISHED);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        base_t += __shfl_xor_sync(0xffffffffu, base_t, o);
-        base_c += __shfl_xor_sync(0xffffffffu, base_c, o);
-    }
+    const int64_t base_t = (int64_t)(__shfl_sync(0xffffffffu, sum, 0) % ARRIVED_ONE);
+    const int32_t base_c = group0 * p.K;                     // every group before these keeps exactly K
     const bool any_bad = __any_sync(0xffffffffu, bad_index);
     const bool any_expired = __any_sync(0xffffffffu, expired);
     if (lane == 0) {
@@ -259,7 +248,7 @@ prune_fused_kernel(const FusedParams p) {
     asm volatile("bar.arrive 2, 64;" ::: "memory");          // done with the chain
     asm volatile("bar.sync 1, 64;" ::: "memory");            // the groups' statistics
     if (kept) {
-        const int pos = base_c + (c - own_c);
+        const int pos = base_c + __popc(kept_lanes & ((1u << lane) - 1u));
         p.survivor_idx[pos] = first + lane;
         p.cu_seqlens[pos + 1] = base_t + t;
         const int g = lane / p.G;
