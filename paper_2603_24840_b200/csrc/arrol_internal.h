@@ -19,6 +19,7 @@ struct arrol_ctx {
     void* d_pack;              // MLP head on the tensor cores: the scored rows packed as bf16 [N][d], ARROL_PACK_BYTES
     uint32_t* d_head_counters; // head training step: finished runs per column tile, zero between calls
     unsigned long long* d_chain;   // fused prune step: finished blocks (and failed index checks), per-block totals; zero between calls
+    void* d_runs;              // fused prune step: the survivors' runs for the kernel that writes the per-token outputs, ARROL_CHAIN_BLOCKS * 32
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
     int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
     bool head_dw1_smem_set[2]; // likewise for the head training step's contraction (column tiles of 64, 128)
@@ -128,7 +129,8 @@ int arrol_internal_compact(arrol_ctx* ctx, const uint8_t* keep, const int32_t* l
                            int32_t N, int32_t G, const int32_t* src_tokens, const void* src_rows, int32_t row_bytes,
                            const float* rewards, float eps, int32_t ddof, int64_t dst_capacity_tokens,
                            int32_t* dst_tokens, void* dst_rows, int64_t* cu_seqlens, int32_t* survivor_idx, float* adv,
-                           float* tok_adv, int32_t* tok_seq, int64_t* d_num, void* stream, bool scan_done);
+                           float* tok_adv, int32_t* tok_seq, int64_t* d_num, void* stream, bool scan_done,
+                           const struct SurvivorRun* runs, int survivors);
 int arrol_internal_check_compact(const uint8_t* keep, const int32_t* lengths, const int64_t* src_tok_off, int32_t N,
                                  int32_t G, const int32_t* src_tokens, const void* src_rows, int32_t row_bytes,
                                  const float* rewards, float eps, int32_t ddof, int64_t dst_capacity_tokens,

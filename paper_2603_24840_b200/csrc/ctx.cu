@@ -3,6 +3,7 @@
 #include <new>
 
 #include "arrol_internal.h"
+#include "token_runs.cuh"
 
 extern "C" int arrol_version(void) { return 100; }
 
@@ -47,6 +48,7 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
     ctx->head_dw1_smem_set[0] = ctx->head_dw1_smem_set[1] = false;
     ctx->d_tile_counters = nullptr;
     ctx->d_chain = nullptr;
+    ctx->d_runs = nullptr;
     ctx->logprob_smem_set = false;
     ctx->head_dw1_max_clusters[0] = ctx->head_dw1_max_clusters[1] = 0;
     ctx->calib_smem_set = false;
@@ -80,6 +82,7 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
               cudaMemset(ctx->d_head_counters, 0, ARROL_HEAD_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMalloc(&ctx->d_tile_counters, ARROL_TILE_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
               cudaMemset(ctx->d_tile_counters, 0, ARROL_TILE_COUNTERS * sizeof(uint32_t)) == cudaSuccess &&
+              cudaMalloc(&ctx->d_runs, (size_t)ARROL_CHAIN_BLOCKS * 32 * sizeof(SurvivorRun)) == cudaSuccess &&
               cudaMalloc(&ctx->d_chain, (2 + ARROL_CHAIN_WORDS * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
               cudaMemset(ctx->d_chain, 0, (2 + ARROL_CHAIN_WORDS * ARROL_CHAIN_BLOCKS) * sizeof(unsigned long long)) == cudaSuccess &&
               cudaMallocHost(&ctx->h_keep, ARROL_MAX_HOST_N) == cudaSuccess &&
@@ -111,6 +114,7 @@ extern "C" int arrol_destroy(arrol_ctx* ctx) {
     if (ctx->d_scratch) (void)cudaFree(ctx->d_scratch);
     if (ctx->d_pack) (void)cudaFree(ctx->d_pack);
     if (ctx->d_head_counters) (void)cudaFree(ctx->d_head_counters);
+    if (ctx->d_runs) (void)cudaFree(ctx->d_runs);
     if (ctx->d_tile_counters) (void)cudaFree(ctx->d_tile_counters);
     if (ctx->d_chain) (void)cudaFree(ctx->d_chain);
     if (ctx->h_keep) (void)cudaFreeHost(ctx->h_keep);

@@ -22,6 +22,7 @@
 
 #include "arrol_internal.h"
 #include "prune_kernels.cuh"
+#include "token_runs.cuh"
 
 namespace {
 
@@ -56,6 +57,7 @@ struct FusedParams {
     // check), from EXPIRED_ONE on those that waited in vain; then from [2] a word per block, SUM_WORDS apart: the kept tokens of the blocks before
     // it, from ARRIVED_ONE on how many of these have added theirs; all zero between calls
     unsigned long long* chain;
+    SurvivorRun* runs;         // or NULL: no per-token outputs
     uint32_t spin_limit;
     int rest_vecs;             // 16-byte vectors of a row past the first 256 that a warp has room for in shared memory: all of them, or 0
 };
@@ -86,6 +88,7 @@ prune_fused_kernel(const FusedParams p) {
     __shared__ float q_s[32], rew_s[32];
     __shared__ uint8_t keep_s[32];
     __shared__ int32_t len_s[32];
+    __shared__ int64_t src_s[32];
     __shared__ bool block_left, block_expired;               // a kept rollout of this block leaves the source; a wait ran out
     __shared__ double inv_count[SCAN_INV], g_mean[32], g_den[32];
     __shared__ float lut_s[LUT_STAGED];                      // the posterior table, or its first use would be one more round trip
@@ -103,6 +106,7 @@ prune_fused_kernel(const FusedParams p) {
         const int i = first + lane;
         len_s[lane] = max(pdl_acquire(p.lengths)[i], 0);
         rew_s[lane] = pdl_acquire(p.rewards)[i];
+        if (p.runs || p.source_rows > 0) src_s[lane] = pdl_acquire(p.src_tok_off)[i];
     }
     if constexpr (SCORE) {
         // every warp fetches its row number while the block stages the head's weights
@@ -207,7 +211,7 @@ prune_fused_kernel(const FusedParams p) {
     const bool kept = lane < n_here && keep_s[lane] != 0;
     const int64_t own_t = kept ? (int64_t)len_s[lane] : 0;
     if (kept && p.source_rows > 0) {
-        const int64_t o = pdl_acquire(p.src_tok_off)[first + lane];
+        const int64_t o = src_s[lane];
         bad_index = o < 0 || o + own_t > p.source_rows;
     }
     const unsigned int kept_lanes = __ballot_sync(0xffffffffu, kept);
@@ -252,7 +256,14 @@ prune_fused_kernel(const FusedParams p) {
         p.survivor_idx[pos] = first + lane;
         p.cu_seqlens[pos + 1] = base_t + t;
         const int g = lane / p.G;
-        p.adv[pos] = (float)(((double)rew_s[lane] - g_mean[g]) * g_den[g]);      // den holds 1 / (std + eps), or 0
+        const float adv = (float)(((double)rew_s[lane] - g_mean[g]) * g_den[g]);      // den holds 1 / (std + eps), or 0
+        p.adv[pos] = adv;
+        if (p.runs) {
+            const int64_t c0 = base_t + t - own_t, src0 = src_s[lane];
+            int4* run = reinterpret_cast<int4*>(p.runs + pos);
+            run[0] = make_int4((int)c0, (int)(c0 >> 32), (int)src0, (int)(src0 >> 32));
+            run[1] = make_int4(len_s[lane], __float_as_int(adv), 0, 0);
+        }
     }
     if (blockIdx.x == 0 && lane == 0) p.cu_seqlens[0] = 0;
 }
@@ -341,6 +352,7 @@ extern "C" int arrol_prune_step(arrol_ctx* ctx, const arrol_prune_step_args* a, 
     p.survivor_idx = a->survivor_idx; p.cu_seqlens = a->cu_seqlens; p.adv = a->adv; p.d_num = a->d_num;
     p.d_status = ctx->d_status;
     p.chain = ctx->d_chain;
+    p.runs = a->dst_tokens || a->tok_adv || a->tok_seq ? static_cast<SurvivorRun*>(ctx->d_runs) : nullptr;
     p.spin_limit = ctx->test_spin_limit ? ctx->test_spin_limit : (1u << 22);
     p.rest_vecs = (int)(rest_bytes / 16 / (size_t)(threads / 32));
     if (smem > 40 * 1024 && !ctx->prune_smem_set) {
@@ -360,5 +372,5 @@ extern "C" int arrol_prune_step(arrol_ctx* ctx, const arrol_prune_step_args* a, 
     return arrol_internal_compact(ctx, a->keep, a->lengths, a->src_tok_off, N, a->G, a->src_tokens, a->src_rows,
                                   a->row_bytes, a->rewards, a->eps, a->ddof, a->dst_capacity_tokens, a->dst_tokens,
                                   a->dst_rows, a->cu_seqlens, a->survivor_idx, a->adv, a->tok_adv, a->tok_seq, a->d_num,
-                                  stream, true);
+                                  stream, true, p.runs, a->P * a->K);
 }

@@ -18,6 +18,23 @@ inline TokenOutputs token_outputs(const int32_t* src_tokens, const float* adv, i
     return o;
 }
 
+// A survivor's run of tokens, left by the fused prune step for the kernel that writes the per-token outputs.
+struct alignas(16) SurvivorRun {
+    int64_t c0, src0;              // where it begins in the packed outputs and in the source
+    int32_t len;
+    float adv;
+    int32_t pad[2];
+};
+__device__ __forceinline__ SurvivorRun load_run(const SurvivorRun* p) {
+    const int4 a = *reinterpret_cast<const int4*>(p), b = *(reinterpret_cast<const int4*>(p) + 1);
+    SurvivorRun r;
+    r.c0 = (int64_t)(uint32_t)a.x | (int64_t)a.y << 32;
+    r.src0 = (int64_t)(uint32_t)a.z | (int64_t)a.w << 32;
+    r.len = b.x;
+    r.adv = __int_as_float(b.y);
+    return r;
+}
+
 // A team of lanes per survivor walks its run of tokens, so nothing has to be searched.  Bound by the bytes it moves
 // (16 per token, 12 of them written): all three outputs leave as 16-byte stores, four tokens per lane.  The source run is
 // aligned differently from the destination, so a lane reads the two aligned 16-byte words that hold its four ids (the second
@@ -27,20 +44,19 @@ inline TokenOutputs token_outputs(const int32_t* src_tokens, const float* adv, i
 // survivor: 1,024 runs of 2,600 ids 26.1 / 22.0 / 22.9 us; 12,288 of 131 58.6 / 52.6 / 69.7; 2,048 of 600 19.9 / 19.7 / 22.0; 828 of
 // 275 12.3 / 12.5 / 12.9; 8 of 1,240 12.3 / 12.1 / 12.0.  Beyond what L2 holds (6.5 M ids, 104 MB) the stores go at HBM's pace.
 constexpr int TOKENS_QUADS = 2;          // groups of four tokens in flight per lane (3 or 4 spill at four blocks per SM: 24.4, 26.7 us on the first of these)
-// Survivors first, first + step, ... by lane `lane` of a team of `lanes`.
-__device__ __forceinline__ void token_runs(const TokenOutputs& o, const int64_t* __restrict__ cu_seqlens, const int32_t* __restrict__ survivor_idx,
-                                           const int64_t* __restrict__ src_tok_off, int S, int first, int step, int lane, int lanes) {
+// Survivors first, first + step, ... by lane `lane` of a team of `lanes`; next_run(s) gives survivor s's run.
+template <typename NextRun>
+__device__ __forceinline__ void token_runs(const TokenOutputs& o, NextRun next_run, int S, int first, int step, int lane, int lanes) {
     const int32_t* __restrict__ src_tokens = o.src_tokens;
-    const float* __restrict__ adv = o.adv;
     int32_t* __restrict__ dst_tokens = o.dst_tokens;
     float* __restrict__ tok_adv = o.tok_adv;
     int32_t* __restrict__ tok_seq = o.tok_seq;
 #pragma unroll 1
     for (int s = first; s < S; s += step) {
-        const int64_t c0 = __ldg(cu_seqlens + s);
-        const int len = (int)(__ldg(cu_seqlens + s + 1) - c0);
-        const int64_t src0 = __ldg(src_tok_off + __ldg(survivor_idx + s));
-        const float a = __ldg(adv + s);
+        const SurvivorRun run = next_run(s);
+        const int64_t c0 = run.c0, src0 = run.src0;
+        const int len = run.len;
+        const float a = run.adv;
         auto load_one = [&](int t) { return dst_tokens ? __ldg(src_tokens + src0 + t) : 0; };
         auto store_one = [&](int t, int32_t id) {
             if (dst_tokens) dst_tokens[c0 + t] = id;
@@ -93,4 +109,18 @@ __device__ __forceinline__ void token_runs(const TokenOutputs& o, const int64_t*
         }
         if (edge >= 0) store_one(edge, edge_id);
     }
+}
+
+// the same, each run from the scan's outputs: two dependent round trips more than a SurvivorRun
+__device__ __forceinline__ void token_runs(const TokenOutputs& o, const int64_t* __restrict__ cu_seqlens, const int32_t* __restrict__ survivor_idx,
+                                           const int64_t* __restrict__ src_tok_off, int S, int first, int step, int lane, int lanes) {
+    auto next_run = [&](int s) {
+        SurvivorRun r;
+        r.c0 = __ldg(cu_seqlens + s);
+        r.len = (int)(__ldg(cu_seqlens + s + 1) - r.c0);
+        r.src0 = __ldg(src_tok_off + __ldg(survivor_idx + s));
+        r.adv = __ldg(o.adv + s);
+        return r;
+    };
+    token_runs(o, next_run, S, first, step, lane, lanes);
 }
