@@ -9,6 +9,7 @@
 
 #include "arrol_internal.h"
 #include "score_common.cuh"
+#include "tc_common.cuh"
 
 namespace {
 
@@ -69,6 +70,12 @@ __device__ __forceinline__ void widen8(const __nv_bfloat16* p, float (&o)[8]) {
 __device__ __forceinline__ void widen8(const float* p, float (&o)[8]) {
     const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
     o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+}
+
+__device__ __forceinline__ void load_vector(const __nv_bfloat16* p, float (&o)[8]) { widen8(p, o); }
+__device__ __forceinline__ void load_vector(const float* p, float (&o)[4]) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
 }
 
 // Linear head: partial[c][k] = sum over the rows of row-chunk c of ds_i x_ik, in index order.  Thread = 8 consecutive columns.  Bound by
@@ -255,63 +262,111 @@ head_du_kernel(const float* u, const float* score, const float* partial, int h_t
     }
 }
 
-// dW1[j][k] = sum_i du[i][j] x[i][k]: 64 x 64 output tile per block, 8 x 4 per thread, rollouts in chunks of 32.
-constexpr int GT = 64, GK = 32, GPAD = 4;
+// dW1[j][k] = sum_i du[i][j] x[i][k]: 64 x 64 output tile per block, 8 x 4 per thread, rollouts in chunks of 32.  A head has few such tiles (d = 512,
+// h = 256: 32) and each contracts all rollouts, so the rollouts are cut into ranges over the blocks of a cluster, whose sums meet in
+// shared memory and are added in rank order; and a chunk waits for its row numbers and then for its rows, so they are requested
+// two chunks and one ahead.  N = 2,000, d = 512, h = 256 (fp32): this
+// kernel 292 us under the profiler as 32 blocks that waited for every load; whole call, with the forward's K over a cluster
+// too, graph of 20: 234 -> 74 us, N = 8,000, d = 1,024, h = 256 962 -> 336, 5,000, 256, 64 488 -> 65, 283, 288, 64 55 -> 27.
+constexpr int GT = 64, GK = 32, GPAD = 4, DW1_THREADS = 128, DW1_SPLITS = 8;
 template <typename T>
-__global__ void __launch_bounds__(128)
-mlp_dw1_kernel(const float* __restrict__ du, const T* __restrict__ hidden, int64_t row_stride,
-               const int64_t* __restrict__ row_index, int N, int d, int h, float* __restrict__ dW1) {
-    __shared__ __align__(16) float as[GK][GT + GPAD];   // du rows
-    __shared__ __align__(16) float bs[GK][GT + GPAD];   // x rows
-    const int j0 = blockIdx.y * GT, c0 = blockIdx.x * GT;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+__global__ void __launch_bounds__(DW1_THREADS)
+mlp_dw1_kernel(const float* du, const T* hidden, int64_t row_stride, const int64_t* row_index, int N, int d, int h, float* __restrict__ dW1) {
+    constexpr int VN = 16 / (int)sizeof(T);                      // columns per 16-byte vector of x
+    constexpr int XV = GK * GT / VN / DW1_THREADS, AV = GK * GT / 4 / DW1_THREADS;       // vectors per thread and chunk
+    constexpr int X_STEP = DW1_THREADS * VN / GT;                // rows between a thread's vectors of x
+    __shared__ __align__(16) float as[2][GK][GT + GPAD];         // du rows
+    __shared__ __align__(16) float bs[2][GK][GT + GPAD];         // x rows
+    static_assert(sizeof(float) * GT * (GT + GPAD) <= sizeof(as), "the block's sums fit the du rows");
+    const int tid = threadIdx.x, j0 = blockIdx.y * GT, c0 = blockIdx.x * GT;
+    const int tx = tid & 15, ty = tid >> 4;
+    const int splits = gridDim.z, rank = blockIdx.z;             // the cluster's blocks
+    const int chunks = (N + GK - 1) / GK;
+    const int first = (int)((int64_t)rank * chunks / splits), last = (int)((int64_t)(rank + 1) * chunks / splits);
+    const int xr = tid * VN / GT, xc = c0 + tid * VN % GT;       // this thread's first vector of x
+    const int ar = tid / (GT / 4), aj = j0 + tid % (GT / 4) * 4; // and of du
+    pdl_launch_dependents();
+    pdl_wait();
+    du = pdl_acquire(du); hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index);
+    int64_t row[XV];                                             // of the chunk that is requested next
+    float4 a_next[AV];
+    float x_next[XV][VN];
+    auto rows_of = [&](int chunk) {
+#pragma unroll
+        for (int i = 0; i < XV; ++i) {
+            const int r = chunk * GK + xr + X_STEP * i;
+            row[i] = chunk < last && r < N ? (row_index ? row_index[r] : (int64_t)r) : -1;
+        }
+    };
+    auto fetch = [&](int chunk) {
+#pragma unroll
+        for (int i = 0; i < AV; ++i) {
+            const int r = chunk * GK + ar + 8 * i;
+            a_next[i] = chunk < last && r < N && aj < h ? *reinterpret_cast<const float4*>(du + (int64_t)r * h + aj)    // h % 4 == 0
+                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < XV; ++i) {
+            const int r = chunk * GK + xr + X_STEP * i;
+            if (chunk < last && r < N && xc < d) {
+                load_vector(hidden + row[i] * row_stride + xc, x_next[i]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < VN; ++e) x_next[i][e] = 0.f;
+            }
+        }
+    };
     float acc[8][4];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-    for (int i0 = 0; i0 < N; i0 += GK) {
-        // du tile: 32 rows x 64 floats = 512 float4, 4 per thread
-        for (int v = threadIdx.x; v < GK * (GT / 4); v += 128) {
-            const int r = v / (GT / 4), c4 = v % (GT / 4);
-            float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-            const int i = i0 + r, j = j0 + c4 * 4;
-            if (i < N && j < h) val = __ldg(reinterpret_cast<const float4*>(du + (int64_t)i * h + j));   // h % 4 == 0
-            *reinterpret_cast<float4*>(&as[r][c4 * 4]) = val;
-        }
-        // x tile: 32 rows x 64 columns, 8 columns per load
-        for (int v = threadIdx.x; v < GK * (GT / 8); v += 128) {
-            const int r = v / (GT / 8), c8 = v % (GT / 8);
-            float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const int i = i0 + r, k = c0 + c8 * 8;
-            if (i < N && k < d) {
-                const int64_t row = row_index ? row_index[i] : (int64_t)i;
-                widen8(hidden + row * row_stride + k, x);
-            }
+    rows_of(first);
+    fetch(first);
+    rows_of(first + 1);
+    int buf = 0;
+    for (int c = first; c < last; ++c, buf ^= 1) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) bs[r][c8 * 8 + e] = x[e];
-        }
-        __syncthreads();
+        for (int i = 0; i < AV; ++i) *reinterpret_cast<float4*>(&as[buf][ar + 8 * i][aj - j0]) = a_next[i];
+#pragma unroll
+        for (int i = 0; i < XV; ++i)
+#pragma unroll
+            for (int e = 0; e < VN; e += 4)
+                *reinterpret_cast<float4*>(&bs[buf][xr + X_STEP * i][xc - c0 + e]) = make_float4(x_next[i][e], x_next[i][e + 1], x_next[i][e + 2], x_next[i][e + 3]);
+        fetch(c + 1);
+        rows_of(c + 2);
+        __syncthreads();                                         // the other buffer was last read before the previous one
 #pragma unroll
         for (int kk = 0; kk < GK; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&as[kk][ty * 8]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&as[kk][ty * 8 + 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&bs[kk][tx * 4]);
-            const float ar[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float br[4] = {b0.x, b0.y, b0.z, b0.w};
+            const float4 a0 = *reinterpret_cast<const float4*>(&as[buf][kk][ty * 8]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&as[buf][kk][ty * 8 + 4]);
+            const float4 b0 = *reinterpret_cast<const float4*>(&bs[buf][kk][tx * 4]);
+            const float ar8[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float br4[4] = {b0.x, b0.y, b0.z, b0.w};
 #pragma unroll
             for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ar[a], br[b], acc[a][b]);
+                for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ar8[a], br4[b], acc[a][b]);
         }
-        __syncthreads();
     }
+    __syncthreads();
+    float* sums = &as[0][0][0];                                  // [GT][GT + GPAD]
 #pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        const int j = j0 + ty * 8 + a, k = c0 + tx * 4;
-        if (j < h && k < d)     // d % 8 == 0: a float4 never straddles the edge
-            *reinterpret_cast<float4*>(dW1 + (int64_t)j * d + k) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+    for (int a = 0; a < 8; ++a)
+        *reinterpret_cast<float4*>(sums + (ty * 8 + a) * (GT + GPAD) + tx * 4) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+    cluster_sync_all();
+    const int rows_each = GT / splits;                           // every block finishes its share of the tile's rows
+    for (int i = tid; i < rows_each * (GT / 4); i += DW1_THREADS) {
+        const int r = rank * rows_each + i / (GT / 4), c = i % (GT / 4) * 4;
+        const uint32_t at = smem_u32(sums + r * (GT + GPAD) + c);
+        float4 sum = ld_shared_cluster_v4(map_to_cta(at, 0u));
+        for (int z = 1; z < splits; ++z) {
+            const float4 v = ld_shared_cluster_v4(map_to_cta(at, (uint32_t)z));
+            sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+        }
+        if (j0 + r < h && c0 + c < d) *reinterpret_cast<float4*>(dW1 + (int64_t)(j0 + r) * d + c0 + c) = sum;      // d % 8 == 0
     }
+    cluster_sync_all();                 // nobody's shared memory goes away while it is being read
 }
 
 struct GradLayout {
@@ -409,8 +464,11 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         if (rc != ARROL_OK) return rc;
         const int rd = launch_du(nullptr, partial, (h + ARROL_MLP_TH - 1) / ARROL_MLP_TH, du, nullptr, nullptr, counters);
         if (rd != ARROL_OK) return rd;
-        dim3 grid((d + GT - 1) / GT, (h + GT - 1) / GT);
-        mlp_dw1_kernel<T><<<grid, 128, 0, s>>>(du, hid, row_stride, row_index, N, d, h, dW1);
+        const int tiles = ((d + GT - 1) / GT) * ((h + GT - 1) / GT), row_chunks = (N + GK - 1) / GK;
+        int splits = 1;                     // two chunks at least, and no more than about four blocks per SM
+        while (splits < DW1_SPLITS && tiles * splits * 2 <= 4 * ctx->sm_count && row_chunks >= splits * 2 * 2) splits *= 2;
+        ARROL_CUDA_OK(arrol_launch_pdl_cluster(mlp_dw1_kernel<T>, dim3((d + GT - 1) / GT, (h + GT - 1) / GT, splits), dim3(DW1_THREADS),
+                                               dim3(1, 1, splits), s, static_cast<const float*>(du), hid, row_stride, row_index, N, d, h, dW1));
         ctx->launches += 1;
     }
     ARROL_CUDA_OK(cudaGetLastError());

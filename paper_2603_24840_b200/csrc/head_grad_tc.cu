@@ -36,12 +36,6 @@ struct Dw1Params {
     uint32_t* d_status;
 };
 
-__device__ __forceinline__ float4 ld_shared_cluster_v4(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-
 template <int TN>
 __global__ void __launch_bounds__(G_THREADS, 1)
 head_dw1_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,

@@ -58,6 +58,13 @@ def test_head_grad_at_the_edges_of_its_tiles(N, d, h):
     test_head_grad_matches_oracle(N, d, h, torch.bfloat16, N % 2 == 0)
 
 
+# the fp32 kernels at their edges: K ranges over clusters of 1, 2 and 4 blocks (forward) and of 1 to 8 (dW1), one of them without a chunk,
+# tiles of 64 rollouts, hidden units and columns partly filled
+@pytest.mark.parametrize("N,d,h", [(1, 64, 8), (33, 1000, 68), (65, 264, 64), (130, 72, 132), (300, 600, 36), (700, 520, 260)])
+def test_fp32_head_grad_at_the_edges_of_its_tiles(N, d, h):
+    test_head_grad_matches_oracle(N, d, h, torch.float32, N % 2 == 0)
+
+
 @pytest.mark.parametrize("h", [0, 260])
 def test_head_grads_of_an_fp32_head_in_flight_on_two_streams(h):
     """These calls work in their own workspaces alone, so two at once give what each gives by itself."""
