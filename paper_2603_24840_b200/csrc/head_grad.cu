@@ -13,106 +13,112 @@
 
 namespace {
 
-constexpr int DS_THREADS = 1024;
 constexpr int DU_RUNS = 32;          // runs of rollouts of head_du_kernel
-
-__device__ __forceinline__ double block_sum(double v, double* sh /* [32] */) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    return t;
-}
-
-// Linear head: ds_i, loss, sum of ds.  One block.
-__global__ void __launch_bounds__(DS_THREADS)
-head_ds_kernel(const float* __restrict__ score, int N, const float* __restrict__ rewards, const uint8_t* __restrict__ mask, float* __restrict__ ds,
-               double* __restrict__ loss, float* __restrict__ dbias) {
-    __shared__ double sh[32];
-    pdl_launch_dependents();
-    pdl_wait();
-    score = pdl_acquire(score); rewards = pdl_acquire(rewards); mask = pdl_acquire(mask);
-    double cnt = 0.0;
-    for (int i = threadIdx.x; i < N; i += DS_THREADS) cnt += (!mask || mask[i]) ? 1.0 : 0.0;
-    const double n = block_sum(cnt, sh);
-    double l = 0.0, sd = 0.0;
-    for (int i = threadIdx.x; i < N; i += DS_THREADS) {
-        float v = 0.f;
-        if (!mask || mask[i]) {
-            const float s = score[i];
-            const float y = rewards[i] > 0.5f ? 1.f : 0.f;
-            const float softplus = s > 0.f ? s + log1pf(expf(-s)) : log1pf(expf(s));
-            l += (double)(softplus - y * s);
-            v = (1.0f / (1.0f + expf(-s)) - y) / (float)n;
-            sd += (double)v;
-        }
-        ds[i] = v;
-    }
-    l = block_sum(l, sh);
-    sd = block_sum(sd, sh);
-    if (threadIdx.x == 0) {
-        *loss = n > 0.0 ? l / n : 0.0;
-        *dbias = (float)sd;
-    }
-}
 
 __device__ __forceinline__ float widen(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float widen(float x) { return x; }
-__device__ __forceinline__ void widen8(const __nv_bfloat16* p, float (&o)[8]) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// eight consecutive elements of a row as they are loaded
+template <typename T> struct Row8;
+template <> struct Row8<__nv_bfloat16> {
+    uint4 v;
+    __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = __ldg(reinterpret_cast<const uint4*>(p)); }
+    __device__ __forceinline__ void widen(float (&o)[8]) const {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { o[2 * i] = __uint_as_float(w[i] << 16); o[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
-}
-__device__ __forceinline__ void widen8(const float* p, float (&o)[8]) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-    o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-}
+        for (int i = 0; i < 4; ++i) { o[2 * i] = __uint_as_float(w[i] << 16); o[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+    }
+};
+template <> struct Row8<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float* p) {
+        a = __ldg(reinterpret_cast<const float4*>(p));
+        b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    }
+    __device__ __forceinline__ void widen(float (&o)[8]) const {
+        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+    }
+};
 
-__device__ __forceinline__ void load_vector(const __nv_bfloat16* p, float (&o)[8]) { widen8(p, o); }
+__device__ __forceinline__ void load_vector(const __nv_bfloat16* p, float (&o)[8]) {
+    Row8<__nv_bfloat16> x;
+    x.load(p);
+    x.widen(o);
+}
 __device__ __forceinline__ void load_vector(const float* p, float (&o)[4]) {
     const float4 v = __ldg(reinterpret_cast<const float4*>(p));
     o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
 }
 
-// Linear head: partial[c][k] = sum over the rows of row-chunk c of ds_i x_ik, in index order.  Thread = 8 consecutive columns.  Bound by
-// the latency of its loads where the rollouts are few: the chunk's factors and row numbers come in one round trip and eight
-// rows are in flight (a row at a time, each behind its factor and its number: 15.4 us under the profiler at N = 172, d = 1,464).
-// Rows without a factor are not read.
-constexpr int LIN_ROWS = 32, LIN_AHEAD = 8;
+// Linear head, first kernel: ds_i = (sigmoid(s_i) - y_i) / n of the row-chunk's rollouts (every block counts the labelled ones itself), their losses
+// and sum, and partial[c][k] = sum over the rows of row-chunk c of ds_i x_ik, in index order.  Thread = 8 consecutive columns.  Bound by
+// the latency of its loads: the row numbers come with what ds is made of, and sixteen rows are in flight.  Rows without a factor are
+// not read.  Second kernel: the chunks' sums.  As three kernels, ds by one block, blocks of 2,048 columns with eight rows in flight, a thread per
+// column for the sums, a whole call took 19.6 us where it takes 9.4 now (graph of 20, N = 2,048, d = 2,048, bf16; 172, 1,464 15.2 -> 7.7; 8,192,
+// 4,096 48.6 -> 25.6; 8,192, 512, fp32 30.4 -> 11.5).
+constexpr int LIN_ROWS = 32, LIN_AHEAD = 16, LIN_THREADS = 128;
 template <typename T>
-__global__ void __launch_bounds__(256)
-linear_dw_partial_kernel(const T* __restrict__ hidden, int64_t row_stride, const int64_t* __restrict__ row_index,
-                         int N, int d, const float* __restrict__ ds, float* __restrict__ partial) {
+__global__ void __launch_bounds__(LIN_THREADS)
+linear_dw_partial_kernel(const T* hidden, int64_t row_stride, const int64_t* row_index, int N, int d, const float* score, const float* rewards,
+                         const uint8_t* mask, float* __restrict__ partial, double* __restrict__ chunk_loss /* [2][chunks]: losses / n, ds */) {
     __shared__ float g_s[LIN_ROWS];
     __shared__ int64_t row_s[LIN_ROWS];
+    __shared__ int warp_n[LIN_THREADS / 32];
     pdl_launch_dependents();
     pdl_wait();
-    hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); ds = pdl_acquire(ds);
-    const int k0 = (blockIdx.x * 256 + threadIdx.x) * 8;
-    const int i0 = blockIdx.y * LIN_ROWS;
+    hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); score = pdl_acquire(score); rewards = pdl_acquire(rewards);
+    mask = pdl_acquire(mask);
+    const int k0 = (blockIdx.x * LIN_THREADS + threadIdx.x) * 8;
+    const int i0 = blockIdx.y * LIN_ROWS, i = i0 + (int)threadIdx.x;
+    const bool mine = threadIdx.x < LIN_ROWS && i < N;           // the first warp's lanes: a rollout each
+    bool labelled = false;
+    float s = 0.f, y = 0.f;
+    if (mine) {
+        labelled = !mask || mask[i];
+        s = score[i];
+        y = rewards[i] > 0.5f ? 1.f : 0.f;
+        row_s[threadIdx.x] = row_index ? row_index[i] : (int64_t)i;
+    }
+    const int c = __reduce_add_sync(0xffffffffu, mask ? count_labelled(mask, N, threadIdx.x, LIN_THREADS) : 0);
+    if ((threadIdx.x & 31) == 0) warp_n[threadIdx.x >> 5] = c;
+    __syncthreads();
     if (threadIdx.x < LIN_ROWS) {
-        const int i = i0 + threadIdx.x;
-        g_s[threadIdx.x] = i < N ? ds[i] : 0.f;
-        row_s[threadIdx.x] = i < N ? (row_index ? row_index[i] : (int64_t)i) : 0;
+        int n = mask ? 0 : N;
+#pragma unroll
+        for (int w = 0; w < LIN_THREADS / 32; ++w) n += warp_n[w];
+        float v = 0.f;
+        double l = 0.0, sd = 0.0;
+        if (labelled) {
+            const float softplus = s > 0.f ? s + log1pf(expf(-s)) : log1pf(expf(s));
+            l = (double)(softplus - y * s) / (double)n;
+            v = (1.0f / (1.0f + expf(-s)) - y) / (float)n;
+            sd = (double)v;
+        }
+        g_s[threadIdx.x] = v;
+        if (blockIdx.x == 0) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                l += __shfl_xor_sync(0xffffffffu, l, o);
+                sd += __shfl_xor_sync(0xffffffffu, sd, o);
+            }
+            if (threadIdx.x == 0) { chunk_loss[blockIdx.y] = l; chunk_loss[gridDim.y + blockIdx.y] = sd; }
+        }
     }
     __syncthreads();
     if (k0 >= d) return;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
     for (int r0 = 0; r0 < LIN_ROWS; r0 += LIN_AHEAD) {
-        float x[LIN_AHEAD][8];
+        Row8<T> x[LIN_AHEAD];
 #pragma unroll
         for (int r = 0; r < LIN_AHEAD; ++r)
-            if (g_s[r0 + r] != 0.f) widen8(hidden + row_s[r0 + r] * row_stride + k0, x[r]);
+            if (g_s[r0 + r] != 0.f) x[r].load(hidden + row_s[r0 + r] * row_stride + k0);
 #pragma unroll
         for (int r = 0; r < LIN_AHEAD; ++r)
             if (g_s[r0 + r] != 0.f) {
+                float w[8];
+                x[r].widen(w);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc[e] = fmaf(g_s[r0 + r], x[r][e], acc[e]);
+                for (int e = 0; e < 8; ++e) acc[e] = fmaf(g_s[r0 + r], w[e], acc[e]);
             }
     }
     float* out = partial + (int64_t)blockIdx.y * d + k0;
@@ -120,16 +126,40 @@ linear_dw_partial_kernel(const T* __restrict__ hidden, int64_t row_stride, const
     *reinterpret_cast<float4*>(out + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
 }
 
-__global__ void column_sum_kernel(const float* __restrict__ partial, int chunks, int d, float* __restrict__ out) {
+// A block per 32 columns: eight warps take every eighth chunk, their sums are added in order.  The first block's last warp: loss and db.
+__global__ void __launch_bounds__(288)
+column_sum_kernel(const float* partial, const double* chunk_loss, int chunks, int d, float* __restrict__ out, double* __restrict__ loss,
+                  float* __restrict__ dbias) {
+    __shared__ float sums[8][32];
     pdl_launch_dependents();
     pdl_wait();
-    partial = pdl_acquire(partial);
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= d) return;
-    float s = 0.f;
+    partial = pdl_acquire(partial); chunk_loss = pdl_acquire(chunk_loss);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = blockIdx.x * 32 + lane;
+    if (warp < 8) {
+        float s = 0.f;
+        if (k < d)
 #pragma unroll 8
-    for (int c = 0; c < chunks; ++c) s += partial[(int64_t)c * d + k];
-    out[k] = s;
+            for (int c = warp; c < chunks; c += 8) s += partial[(int64_t)c * d + k];
+        sums[warp][lane] = s;
+    } else if (blockIdx.x == 0) {
+        double l = 0.0, sd = 0.0;
+#pragma unroll 4
+        for (int c = lane; c < chunks; c += 32) { l += chunk_loss[c]; sd += chunk_loss[chunks + c]; }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            l += __shfl_xor_sync(0xffffffffu, l, o);
+            sd += __shfl_xor_sync(0xffffffffu, sd, o);
+        }
+        if (lane == 0) { *loss = l; *dbias = (float)sd; }
+    }
+    __syncthreads();
+    if (warp == 0 && k < d) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += sums[w][lane];
+        out[k] = s;
+    }
 }
 
 // MLP head: everything between the forward and the dW1 contraction in one launch: ds_i, the loss, du_ij, and per hidden unit
@@ -408,12 +438,13 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         const int rc = arrol_score_partial(ctx, hidden, row_stride, row_index, N, head, nullptr, tmp, tmp + N, nullptr,
                                            tmp + 2 * (size_t)N, s);
         if (rc != ARROL_OK) return rc;
-        ARROL_CUDA_OK(arrol_launch_pdl(head_ds_kernel, dim3(1), dim3(DS_THREADS), 0, s, static_cast<const float*>(tmp), N, rewards, mask, ds, loss, db1));
         const int chunks = (N + LIN_ROWS - 1) / LIN_ROWS;
-        dim3 grid((d / 8 + 255) / 256, chunks);
-        ARROL_CUDA_OK(arrol_launch_pdl(linear_dw_partial_kernel<T>, grid, dim3(256), 0, s, hid, row_stride, row_index, N, d, static_cast<const float*>(ds), partial));
-        ARROL_CUDA_OK(arrol_launch_pdl(column_sum_kernel, dim3((d + 255) / 256), dim3(256), 0, s, static_cast<const float*>(partial), chunks, d, dW1));
-        ctx->launches += 3;
+        double* chunk_loss = reinterpret_cast<double*>(ds);          // 16 bytes per 32 rollouts
+        ARROL_CUDA_OK(arrol_launch_pdl(linear_dw_partial_kernel<T>, dim3((d / 8 + LIN_THREADS - 1) / LIN_THREADS, chunks), dim3(LIN_THREADS), 0, s, hid,
+                                       row_stride, row_index, N, d, static_cast<const float*>(tmp), rewards, mask, partial, chunk_loss));
+        ARROL_CUDA_OK(arrol_launch_pdl(column_sum_kernel, dim3((d + 31) / 32), dim3(288), 0, s, static_cast<const float*>(partial),
+                                       static_cast<const double*>(chunk_loss), chunks, d, dW1, loss, db1));
+        ctx->launches += 2;
     } else {
         float* u = reinterpret_cast<float*>(ws + L.u);
         float* du = reinterpret_cast<float*>(ws + L.du);

@@ -65,6 +65,13 @@ def test_fp32_head_grad_at_the_edges_of_its_tiles(N, d, h):
     test_head_grad_matches_oracle(N, d, h, torch.float32, N % 2 == 0)
 
 
+# the linear head's: one rollout, one past a row-chunk, columns that end a thread's eight into the second block, more chunks than warps add
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("N,d", [(1, 8), (33, 8), (65, 1032), (700, 2056), (32, 1024)])
+def test_linear_head_grad_at_the_edges_of_its_blocks(N, d, dtype):
+    test_head_grad_matches_oracle(N, d, 0, dtype, N % 2 == 0)
+
+
 @pytest.mark.parametrize("h", [0, 260])
 def test_head_grads_of_an_fp32_head_in_flight_on_two_streams(h):
     """These calls work in their own workspaces alone, so two at once give what each gives by itself."""
