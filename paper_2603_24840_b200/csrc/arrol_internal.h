@@ -27,7 +27,7 @@ struct arrol_ctx {
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool prune_smem_set;       // likewise for the fused prune step
-    int score_max_clusters[9]; // scoring kernel: clusters of so many blocks of 64 hidden units that are resident at once; 0 = not asked yet
+    int score_max_clusters[2][9]; // scoring kernel, tiles of 128 / 64 rollouts x 64 hidden units: clusters of so many blocks that are resident at once; 0 = not asked yet
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
     uint32_t test_spin_limit;  // arrol_test_hook: tries per pipeline wait of the log-prob kernel, 0 = the normal limit
@@ -167,7 +167,7 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
                                 cudaStream_t s);
 int arrol_internal_head_train_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
                                  const arrol_head* head, const float* rewards, const uint8_t* mask, void* du_hi, void* du_lo,
-                                 float* tile_sums, double* tile_loss, cudaStream_t s);
+                                 float* tile_sums, double* tile_loss, int* tile_rows, cudaStream_t s);
 
 // gather_bulk.cu: the survivors' rows moved by bulk copies through shared memory.  ARROL_ERR_UNSUPPORTED (nothing
 // launched) when a row does not fit a 32 KB stage.
@@ -178,8 +178,9 @@ int arrol_internal_gather_rows_bulk(arrol_ctx* ctx, const int64_t* d_num, const 
                                     const void* src_rows, int64_t row_bytes, int64_t capacity, void* dst_rows, cudaStream_t s);
 
 // head_grad_tc.cu: dW1[h, d] = (du_hi + du_lo)^T X on the tensor cores, du planes [N, h] bf16, X [N, d] bf16 with rows ldx apart; and
-// the sums over the tiles of 128 rollouts that arrol_internal_head_train_tc left, where tile_sums is given.
+// the sums over the tiles of rollouts that arrol_internal_head_train_tc left, where tile_sums is given.
 struct HeadTileSums {
+    int tiles;
     const float* tile_sums;     // [2][tiles][h] -> dw2, db1
     const double* tile_loss;    // [2][tiles] -> loss, db2
     float* dw2;

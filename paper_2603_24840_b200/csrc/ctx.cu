@@ -55,7 +55,8 @@ extern "C" int arrol_create(arrol_ctx** out, int device) {
     ctx->backward_smem_set = false;
     ctx->prune_smem_set = false;
     for (int& n : ctx->backward_max_pairs) n = 0;
-    for (int& n : ctx->score_max_clusters) n = 0;
+    for (auto& rows : ctx->score_max_clusters)
+        for (int& n : rows) n = 0;
     ctx->score_tc_smem_set = false;
     ctx->gather_bulk_smem_set = false;
     ctx->test_spin_limit = 0;

@@ -467,13 +467,14 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
             if (h % 8 == 0) {
                 __nv_bfloat16* du_hi = reinterpret_cast<__nv_bfloat16*>(ws + L.du);
                 __nv_bfloat16* du_lo = reinterpret_cast<__nv_bfloat16*>(ws + L.du + L.du_plane);
-                // sums per tile of 128 rollouts: where the other path keeps those of its runs, of more tiles where it keeps u and ds
-                const bool few = (N + 127) / 128 <= DU_RUNS;
+                // sums per tile of 64 rollouts or more: where the other path keeps those of its runs, of more tiles where it keeps u and ds
+                const bool few = (N + 63) / 64 <= DU_RUNS;
                 float* tile_sums = few ? reinterpret_cast<float*>(ws + L.run_sums) : u;
                 double* tile_loss = few ? reinterpret_cast<double*>(ws + L.run_loss) : reinterpret_cast<double*>(ds);
-                HeadTileSums sums = {tile_sums, tile_loss, dw2, db1, loss, db2};
+                int tile_rows = 128;
                 int rc = arrol_internal_head_train_tc(ctx, hidden, row_stride, row_index, N, head, rewards, mask, du_hi, du_lo,
-                                                      tile_sums, tile_loss, s);
+                                                      tile_sums, tile_loss, &tile_rows, s);
+                HeadTileSums sums = {(N + tile_rows - 1) / tile_rows, tile_sums, tile_loss, dw2, db1, loss, db2};
                 if (rc == ARROL_ERR_UNSUPPORTED) {      // more than 1,024 hidden units, or beyond the context's buffers
                     float* tmp = reinterpret_cast<float*>(ws + L.tmp3);
                     sums.tile_sums = nullptr;

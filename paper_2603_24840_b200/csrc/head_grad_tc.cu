@@ -7,7 +7,8 @@
 // blocks while SMs are idle (their accumulators meet in shared memory, added in rank order) and TN is 128 where tiles of 64
 // would need more than one wave.  N = 2,048, d = 2,048, h = 256: 12.7 us (7 of them launch, set-up and finish) against 35.7 for a
 // launch per plane on eight 128 x 256 tiles; N = 4,096, d = 4,096, h = 512: 33 us.
-// The epilogue warps, which wait for the contraction, add up the row tiles' sums that dw2, db1, db2 and the loss are made of; the forward
+// The epilogue warps, which wait for the contraction, add up the row tiles' sums that dw2, db1, db2 and the loss are made of (32 hidden units
+// a block: by one block's threads alone 125 tiles took longer than its share of the contraction); the forward
 // kernel's last blocks did, behind a fence, a counter and a reload (N = 2,048, d = 2,048, h = 256: whole call 32.3 -> 29.2 us).
 // Every wait is bounded; on expiry the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
 #include <cuda.h>
@@ -22,7 +23,7 @@ constexpr int GM = 128;                           // hidden units per tile (MMA 
 constexpr int PLANE_BYTES = GM * BK * 2;          // one plane's part of a stage: two blocks of [64 rollouts x 64 units]
 constexpr int G_THREADS = 192;                    // producer, issuer, four epilogue warps
 constexpr int MN_BLOCK = BK * 128;                // bytes of a [64 x 64] MN-major block
-constexpr int G_TAIL_BYTES = 512;
+constexpr int G_TAIL_BYTES = 512 + 2048;           // barriers | quarters of the row tiles' sums
 
 template <int TN> __host__ __device__ constexpr int stage_bytes() { return 2 * PLANE_BYTES + TN * BK * 2; }
 template <int TN> __host__ __device__ constexpr int stages() { return TN == 64 ? 5 : 4; }
@@ -50,6 +51,7 @@ head_dw1_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constan
     uint64_t* acc_full = empty + STAGES;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
     volatile uint32_t* abort_flag = tmem_slot + 1;
+    double* quarter_s = reinterpret_cast<double*>(smem + (size_t)STAGES * STAGE_BYTES + 512);     // [2][4][32]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c0 = blockIdx.x * TN, j0 = blockIdx.y * GM;
     const int splits = gridDim.z, rank = blockIdx.z;              // the cluster's blocks: ranges of the K steps
@@ -126,26 +128,39 @@ head_dw1_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constan
     } else {
         // thread = one hidden unit: its TN sums go to shared memory (the stages are free: every MMA has finished)
         const int quarter = warp & 3, r = quarter * 32 + lane;
-        if (c0 == 0 && rank == 0 && p.sums.tile_sums) {        // the row tiles' sums, in index order, while the contraction runs
-            const int tiles = (p.N + 127) / 128, j = j0 + r;
+        if (p.sums.tile_sums) {          // the row tiles' sums, while the contraction runs: 32 hidden units a block, a quarter of the tiles a warp
+            const int tiles = p.sums.tiles, w = warp - 2;
+            const int block = (int)blockIdx.x * splits + rank, blocks = (int)gridDim.x * splits;
             const float* tile_sums = pdl_acquire(p.sums.tile_sums);
-            if (j < p.h) {
-                double w2 = 0.0, b1 = 0.0;          // up to 512 tiles
+            for (int u0 = block * 32; u0 < GM && j0 + u0 < p.h; u0 += blocks * 32) {
+                const int j = j0 + u0 + lane;
+                double w2 = 0.0, b1 = 0.0;           // up to 1,024 tiles
+                if (j < p.h)
 #pragma unroll 8
-                for (int t = 0; t < tiles; ++t) {
-                    w2 += tile_sums[(int64_t)t * p.h + j];
-                    b1 += tile_sums[(int64_t)(tiles + t) * p.h + j];
+                    for (int t = w; t < tiles; t += 4) {
+                        w2 += (double)tile_sums[(int64_t)t * p.h + j];
+                        b1 += (double)tile_sums[(int64_t)(tiles + t) * p.h + j];
+                    }
+                quarter_s[w * 32 + lane] = w2;
+                quarter_s[128 + w * 32 + lane] = b1;
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                if (w < 2 && j < p.h) {
+                    const double* q = quarter_s + 128 * w + lane;
+                    (w == 0 ? p.sums.dw2 : p.sums.db1)[j] = (float)(((q[0] + q[32]) + q[64]) + q[96]);
                 }
-                p.sums.dw2[j] = (float)w2;
-                p.sums.db1[j] = (float)b1;
+                asm volatile("bar.sync 1, 128;" ::: "memory");
             }
-            if (j0 == 0 && r < 2) {
-                const double* tile_loss = pdl_acquire(p.sums.tile_loss);
+            if (j0 == 0 && block == blocks - 1 && w >= 2) {
+                const double* tile_loss = pdl_acquire(p.sums.tile_loss) + (w - 2) * tiles;
                 double t = 0.0;
-#pragma unroll 8
-                for (int i = 0; i < tiles; ++i) t += tile_loss[r * tiles + i];
-                if (r == 0) *p.sums.loss = t;
-                else *p.sums.db2 = (float)t;
+#pragma unroll 4
+                for (int i = lane; i < tiles; i += 32) t += tile_loss[i];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                if (lane == 0) {
+                    if (w == 2) *p.sums.loss = t;
+                    else *p.sums.db2 = (float)t;
+                }
             }
         }
         bool ok = mbar_wait(acc_full, 0u, abort_flag);

@@ -8,8 +8,8 @@
 //                         copies into the swizzled stage layout, was built and measured: correct, but the
 //                         load/store path holds about 20 KB in flight per SM against the ring's 192 KB by TMA, and
 //                         every block of a row tile fetches the same rows: 18.5 us per call against 14.6 us.)
-//   score_mlp_tc_kernel   one block per (128 rollouts x 64 or 128 hidden units); shared memory is one ring of stages
-//                         (128 x 64 of X and the tile's 64 columns of W1 per K step of 64), filled by four TMA producer threads,
+//   score_mlp_tc_kernel   one block per (64 or 128 rollouts x 64 hidden units, or 128 x 128); shared memory is one ring of stages
+//                         (the tile's 64 columns of X and of W1 per K step of 64), filled by four TMA producer threads,
 //                         two for X and two for W1, on alternate K steps (one thread for all of W1 takes 300 cycles a step:
 //                         N = 2,048, d = 2,048, h = 256, rows in place 8.7 -> 12.6 us).  Two (tiles of 128) or four (64) issuing warps take the K steps round robin: one
 //                         warp's wait -> four MMAs -> commit round costs nearly 500 cycles, the MMAs of a 128 x 64 x 64 step
@@ -52,13 +52,15 @@ constexpr int MAX_SUBS = 16;                 // partial sums of a row tile whose
 // barriers, tensor-memory slot, flags | b1 and w2 of the tile, sums over 16 hidden units | sums over 32
 // | the training step's ds of the tile's rollouts, sums over its warps
 constexpr int S_TAIL_BYTES = 2560 + 2 * MAX_SUBS * 128 * 4 + 512 + 256;
-constexpr int TM = 128;                      // rollouts per tile (MMA M)
-constexpr int A_BYTES = TM * BK * 2;         // 16 KB
-// by tile width (hidden units, MMA N): 64 or 128
-template <int SBN> __host__ __device__ constexpr int ring_stages() { return SBN == 64 ? 8 : 6; }
+constexpr int MAX_ROWS = 128;
+// by tile: rollouts (MMA M: 64 or 128) x hidden units (MMA N: 64 or 128); 64 x 64, 128 x 64 and 128 x 128
+template <int ROWS> __host__ __device__ constexpr int a_bytes() { return ROWS * BK * 2; }
+template <int SBN, int ROWS> __host__ __device__ constexpr int ring_stages() { return SBN == 128 ? 6 : ROWS == 128 ? 8 : 12; }
 template <int SBN> __host__ __device__ constexpr int issuers() { return SBN == 64 ? 4 : 2; }
-template <int SBN> __host__ __device__ constexpr int stage_bytes() { return A_BYTES + SBN * BK * 2; }
-template <int SBN> __host__ __device__ constexpr size_t smem_bytes() { return (size_t)ring_stages<SBN>() * stage_bytes<SBN>() + 1024 + S_TAIL_BYTES; }
+template <int SBN, int ROWS> __host__ __device__ constexpr int stage_bytes() { return a_bytes<ROWS>() + SBN * BK * 2; }
+template <int SBN, int ROWS> __host__ __device__ constexpr size_t smem_bytes() {
+    return (size_t)ring_stages<SBN, ROWS>() * stage_bytes<SBN, ROWS>() + 1024 + S_TAIL_BYTES;
+}
 
 // one warp per 4 KB of a row (a grid row per slice, so that no warp divides): 16-byte copies, all of its loads in flight
 // before the first store
@@ -121,17 +123,20 @@ struct ScoreTcParams {
 // shared memory, [unit][rollout], where the sums over rollouts are read along rows.  A kernel of its
 // own with u through global memory between took 9.4 us at N = 2,048, h = 256 (ncu).
 enum Mode { PARTIALS, SCORES, TRAIN };
-template <int SBN, Mode MODE>
+template <int SBN, Mode MODE, int ROWS>
 __global__ void __launch_bounds__(S_THREADS, 1)
 score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                     const ScoreTcParams p) {
-    constexpr int STAGES = ring_stages<SBN>(), STAGE_BYTES = stage_bytes<SBN>(), SB_BYTES = SBN * BK * 2;
+    constexpr int TM = ROWS, A_BYTES = a_bytes<ROWS>();
+    constexpr int STAGES = ring_stages<SBN, ROWS>(), STAGE_BYTES = stage_bytes<SBN, ROWS>(), SB_BYTES = SBN * BK * 2;
     constexpr int ISSUERS = issuers<SBN>();
     static_assert(STAGES % ISSUERS == 0 && S_ACCS % ISSUERS == 0 && STAGES % S_PRODUCERS == 0,
                   "a stage and an accumulator belong to one issuer, a stage to one producer");
     constexpr int S_TMEM_COLS = S_ACCS * SBN;                    // a power of two >= 32
     constexpr bool CLUSTER = MODE != PARTIALS;
-    static_assert(2 * SBN * TM * 4 <= STAGES * STAGE_BYTES, "both planes fit the stages");
+    constexpr int PITCH = TM == 128 ? TM : TM + 2;               // of the training step's planes: lanes l and l + 16 on different banks
+    static_assert(2 * SBN * PITCH * 4 <= STAGES * STAGE_BYTES, "both planes fit the stages");
+    static_assert(TM == 128 || (SBN == 64 && MODE != PARTIALS), "tiles of 64 rollouts: narrow ones, in clusters");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* stage_a = smem;
@@ -147,11 +152,11 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     float* w2_s = reinterpret_cast<float*>(tail + 1024);         // [SBN]
     float* half_s = reinterpret_cast<float*>(tail + 1536);       // [2][TM] sums over 16 hidden units of a tile of 64
     float* runs_s = reinterpret_cast<float*>(tail + 2560);       // [2 MAX_SUBS][TM] sums over 32 (of the row tile in the first block of a cluster; TRAIN: in every block)
-    float* ds_s = runs_s + 2 * MAX_SUBS * TM;                    // [TM]
+    float* ds_s = runs_s + 2 * MAX_SUBS * MAX_ROWS;                    // [TM]
     double* warp_d = reinterpret_cast<double*>(ds_s + TM);       // [2][4]
     int* warp_n = reinterpret_cast<int*>(warp_d + 8);            // [S_HELPER_WARPS]
-    float* gelu_s = reinterpret_cast<float*>(smem);              // [SBN][TM] ds gelu(u), once every MMA has finished
-    float* du_s = gelu_s + SBN * TM;                             // [SBN][TM]
+    float* gelu_s = reinterpret_cast<float*>(smem);              // [SBN][PITCH] ds gelu(u), once every MMA has finished
+    float* du_s = gelu_s + SBN * PITCH;                          // [SBN][PITCH]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * TM, j0 = blockIdx.y * SBN;
@@ -177,7 +182,7 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     pdl_launch_dependents();
     pdl_wait();                  // set-up above overlaps the previous kernel; global memory is read from here on
 
-    bool labelled = false;       // TRAIN, warps 8 to 11: of rollout r_tile
+    bool labelled = false;       // TRAIN: of rollout threadIdx.x - 256 of the tile
     float reward = 0.f;
     // K step ks uses stage ks % STAGES in round ks / STAGES of the ring, issuer ks % ISSUERS and accumulator ks % S_ACCS.
     if (warp < S_PRODUCER_WARPS) {
@@ -253,64 +258,87 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
     __syncwarp();
 
-    // Epilogue: all warps; thread = rollout x a quarter of the tile's hidden units.  Accumulator row r is tensor-memory lane r, and a
-    // warp reads the lanes of its number mod 4.
-    constexpr int UNITS = SBN / 4;
+    // Epilogue: all warps; thread = rollout x UNITS hidden units.  128 rollouts: accumulator row r is tensor-memory lane r, a warp reads the lanes of its
+    // number mod 4 and a quarter of the columns.  64 rollouts: row r is lane 32 (r / 16) + r mod 16, so that the upper half of a warp's
+    // lanes holds nothing; it takes over the upper half of the warp's columns.
+    constexpr int COLS = SBN / 4, UNITS = TM == 128 ? COLS : COLS / 2;
     const int quarter = warp & 3, cg = warp >> 2;
-    const int r_tile = quarter * 32 + lane, m = m0 + r_tile;
+    const bool upper = TM == 64 && lane >= 16;
+    const int r_tile = TM == 128 ? quarter * 32 + lane : quarter * 16 + (lane & 15), m = m0 + r_tile;
+    const int unit0 = cg * COLS + (upper ? UNITS : 0);                     // of this thread's, in the tile
     const int used_accs = p.k_steps < S_ACCS ? p.k_steps : S_ACCS;         // an accumulator without K steps holds nothing
     bool ok = mbar_wait(acc_full, 0u, abort_flag);
     ok = __all_sync(0xffffffffu, ok && !*abort_flag) != 0;
     __syncthreads();                        // b1_s, w2_s
     float v[UNITS], cdf[UNITS];             // u = pre-activations, then gelu(u); 2 Phi(u)
-    if (ok) {
-        tcgen05_fence_after();
-        const uint32_t at = tmem_base + ((uint32_t)(quarter * 32) << 16) + cg * UNITS;
-        tcgen05_ld_32(at, v);
-        for (int a = 1; a < used_accs; ++a) {      // fixed order: ((acc0 + acc1) + acc2) + acc3
-            float w[UNITS];
-            tcgen05_ld_32(at + a * SBN, w);
+    {
+        float sum[COLS];
+        if (ok) {
+            tcgen05_fence_after();
+            const uint32_t at = tmem_base + ((uint32_t)(quarter * 32) << 16) + cg * COLS;
+            tcgen05_ld_32(at, sum);
+            for (int a = 1; a < used_accs; ++a) {      // fixed order: ((acc0 + acc1) + acc2) + acc3
+                float w[COLS];
+                tcgen05_ld_32(at + a * SBN, w);
 #pragma unroll
-            for (int j = 0; j < UNITS; ++j) v[j] += w[j];
+                for (int j = 0; j < COLS; ++j) sum[j] += w[j];
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) sum[j] = 0.f;
         }
-    } else {
 #pragma unroll
-        for (int j = 0; j < UNITS; ++j) v[j] = 0.f;
+        for (int j = 0; j < UNITS; ++j) {
+            v[j] = sum[j];
+            if constexpr (TM == 64) {
+                const float other = __shfl_sync(0xffffffffu, sum[UNITS + j], lane & 15);
+                if (upper) v[j] = other;
+            }
+        }
     }
     float slope[MODE == TRAIN ? UNITS : 1];        // gelu'(u) w2
 #pragma unroll
     for (int j = 0; j < UNITS; ++j) {
-        const float u = v[j] + b1_s[cg * UNITS + j];
+        const float u = v[j] + b1_s[unit0 + j];
         v[j] = u;
         cdf[j] = 1.0f + erff(u * 0.70710678118654752440f);
     }
     if constexpr (MODE == PARTIALS) {
         if (p.u_out && m < p.N) {
-            float* urow = p.u_out + (int64_t)m * p.h + j0 + cg * UNITS;
+            float* urow = p.u_out + (int64_t)m * p.h + j0 + unit0;
 #pragma unroll
             for (int j = 0; j < UNITS; j += 4)      // h % 4 == 0: a float4 never straddles the edge
-                if (j0 + cg * UNITS + j < p.h) *reinterpret_cast<float4*>(urow + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                if (j0 + unit0 + j < p.h) *reinterpret_cast<float4*>(urow + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
         }
     }
     // sum_j w2_j gelu(u_j) over 32 hidden units in index order; two of these, low + high, make a partial sum.  Of a tile of 64 two
-    // threads have 16 each, and the second one goes on where the first one ends.
-    const float* w2 = w2_s + cg * UNITS;
+    // threads (four where a tile has 64 rollouts) have a part each, and the next one goes on where the one before ends.
+    const float* w2 = w2_s + unit0;
+    auto go_on = [&](float part) {
+        auto units = [&](float start) {
+#pragma unroll
+            for (int j = 0; j < UNITS; ++j) start = fmaf(w2[j], 0.5f * v[j] * cdf[j], start);
+            return start;
+        };
+        part = units(part);
+        if constexpr (TM == 64) part = units(__shfl_sync(0xffffffffu, part, lane & 15));     // the upper lanes' after the lower ones'
+        return part;
+    };
+    const bool ends = TM == 128 || upper;       // this thread's part is the last one of its warp
     float part = 0.f;
     if constexpr (SBN == 64) {
         if ((cg & 1) == 0) {
-#pragma unroll
-            for (int j = 0; j < UNITS; ++j) part = fmaf(w2[j], 0.5f * v[j] * cdf[j], part);
-            half_s[(cg >> 1) * TM + r_tile] = part;
+            part = go_on(0.f);
+            if (ends) half_s[(cg >> 1) * TM + r_tile] = part;
         }
         __syncthreads();
         if ((cg & 1) == 1) part = half_s[(cg >> 1) * TM + r_tile];
     }
     if (SBN == 128 || (cg & 1) == 1) {
-#pragma unroll
-        for (int j = 0; j < UNITS; ++j) part = fmaf(w2[j], 0.5f * v[j] * cdf[j], part);
+        part = go_on(part);
         const int run = SBN == 128 ? cg : cg >> 1;                       // of 32 hidden units, in the tile
         const int all = MODE == PARTIALS ? run : (int)blockIdx.y * (SBN / 32) + run;
-        if (MODE == PARTIALS || (all >> 1) * SUB_H < p.h) {
+        if (ends && (MODE == PARTIALS || (all >> 1) * SUB_H < p.h)) {
             const uint32_t to = smem_u32(&runs_s[all * TM + r_tile]);
             if constexpr (MODE == PARTIALS) runs_s[all * TM + r_tile] = part;
             if constexpr (MODE == SCORES) st_shared_cluster_f32(map_to_cta(to, 0u), part);
@@ -362,12 +390,14 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         return p.b2 ? s + __bfloat162float(pdl_acquire(p.b2)[0]) : s;
     };
     if constexpr (MODE == SCORES) {
-        if (blockIdx.y == 0 && cg == 0 && m < p.N)
+        if (blockIdx.y == 0 && cg == 0 && !upper && m < p.N)
             probability_map(score_of(r_tile), m, p.B, pdl_acquire(p.q_lut), p.score, p.prob, p.bin, p.q);
     }
     if constexpr (MODE == TRAIN) {
         const bool live = m < p.N;
-        if (warp >= S_HELPER_WARP0 && warp < S_HELPER_WARP0 + 4) {       // the warps that have the labels
+        const int labels = warp - S_HELPER_WARP0;                        // the first of these warps have the labels
+        if (labels >= 0 && labels < TM / 32) {
+            const int r = labels * 32 + lane;
             int n = p.N;
             if (p.mask) {
                 n = 0;
@@ -377,29 +407,29 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             double l = 0.0, sd = 0.0;
             float ds = 0.f;
             if (labelled) {
-                const float s = score_of(r_tile);
+                const float s = score_of(r);
                 const float y = reward > 0.5f ? 1.f : 0.f;
                 ds = (1.0f / (1.0f + expf(-s)) - y) / (float)n;
                 sd = (double)ds;
                 if (blockIdx.y == 0) l = (double)((s > 0.f ? s + log1pf(expf(-s)) : log1pf(expf(s))) - y * s);
             }
-            ds_s[r_tile] = ds;
+            ds_s[r] = ds;
             if (blockIdx.y == 0) {
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
                     l += __shfl_xor_sync(0xffffffffu, l, o);
                     sd += __shfl_xor_sync(0xffffffffu, sd, o);
                 }
-                if (lane == 0) { warp_d[quarter] = n > 0 ? l / (double)n : 0.0; warp_d[4 + quarter] = sd; }
+                if (lane == 0) { warp_d[labels] = n > 0 ? l / (double)n : 0.0; warp_d[4 + labels] = sd; }
             }
         }
         __syncthreads();
         if (blockIdx.y == 0 && threadIdx.x < 2) {
             const double* d = warp_d + 4 * threadIdx.x;
-            p.tile_loss[threadIdx.x * gridDim.x + blockIdx.x] = ((d[0] + d[1]) + d[2]) + d[3];
+            p.tile_loss[threadIdx.x * gridDim.x + blockIdx.x] = TM == 128 ? ((d[0] + d[1]) + d[2]) + d[3] : d[0] + d[1];
         }
         const float g = ds_s[r_tile];
-        const int64_t out = (int64_t)m * p.h + j0 + cg * UNITS;
+        const int64_t out = (int64_t)m * p.h + j0 + unit0;
 #pragma unroll
         for (int jj = 0; jj < UNITS; jj += 8) {
             uint32_t hi[4], lo[4];
@@ -410,10 +440,10 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 const uint32_t h16 = __bfloat16_as_ushort(top), l16 = __bfloat16_as_ushort(__float2bfloat16_rn(d_u - __bfloat162float(top)));
                 hi[k >> 1] = (k & 1) ? hi[k >> 1] | h16 << 16 : h16;
                 lo[k >> 1] = (k & 1) ? lo[k >> 1] | l16 << 16 : l16;
-                gelu_s[(cg * UNITS + jj + k) * TM + r_tile] = live ? g * v[jj + k] : 0.f;       // rows past N: zeros, whatever b1 made of them
-                du_s[(cg * UNITS + jj + k) * TM + r_tile] = live ? d_u : 0.f;
+                gelu_s[(unit0 + jj + k) * PITCH + r_tile] = live ? g * v[jj + k] : 0.f;       // rows past N: zeros, whatever b1 made of them
+                du_s[(unit0 + jj + k) * PITCH + r_tile] = live ? d_u : 0.f;
             }
-            if (live && j0 + cg * UNITS + jj < p.h) {                       // h % 8 == 0
+            if (live && j0 + unit0 + jj < p.h) {                       // h % 8 == 0
                 *reinterpret_cast<uint4*>(p.du_hi + out + jj) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                 *reinterpret_cast<uint4*>(p.du_lo + out + jj) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
@@ -424,10 +454,11 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             float sum[2 * ABREAST];
 #pragma unroll
             for (int i = 0; i < ABREAST; ++i) {
-                const float* a = gelu_s + (j + i) * TM + lane;
-                const float* b = du_s + (j + i) * TM + lane;
-                sum[2 * i] = (a[0] + a[32]) + (a[64] + a[96]);
-                sum[2 * i + 1] = (b[0] + b[32]) + (b[64] + b[96]);
+                const float* a = gelu_s + (j + i) * PITCH + lane;
+                const float* b = du_s + (j + i) * PITCH + lane;
+                sum[2 * i] = a[0] + a[32];
+                sum[2 * i + 1] = b[0] + b[32];
+                if constexpr (TM == 128) { sum[2 * i] += a[64] + a[96]; sum[2 * i + 1] += b[64] + b[96]; }
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1)
@@ -445,13 +476,15 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
 }
 
-// Clusters of `blocks` blocks with tiles of 64 hidden units that are resident at once (asked once per context and size).
+// Clusters of `blocks` blocks with tiles of ROWS rollouts x 64 hidden units that are resident at once (asked once per context and size).
+template <int ROWS>
 int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
-    if (ctx->score_max_clusters[blocks] == 0) {
+    int& known = ctx->score_max_clusters[ROWS == 64][blocks];
+    if (known == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(1, (unsigned)blocks);
         cfg.blockDim = dim3(S_THREADS);
-        cfg.dynamicSmemBytes = smem_bytes<64>();
+        cfg.dynamicSmemBytes = smem_bytes<64, ROWS>();
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 1;
@@ -459,9 +492,9 @@ int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&ctx->score_max_clusters[blocks], score_mlp_tc_kernel<64, SCORES>, &cfg));
+        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&known, score_mlp_tc_kernel<64, SCORES, ROWS>, &cfg));
     }
-    *fit = ctx->score_max_clusters[blocks];
+    *fit = known;
     return ARROL_OK;
 }
 
@@ -470,20 +503,22 @@ int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
 // Launches the packing kernel and the contraction in one of its modes; p holds the mode's own outputs.  ARROL_ERR_UNSUPPORTED
 // (nothing launched) when the sizes do not fit the context's buffers, or the mode.
 static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
-                         const arrol_head* head, bool train, ScoreTcParams& p, cudaStream_t s) {
+                         const arrol_head* head, bool train, ScoreTcParams& p, cudaStream_t s, int* tile_rows = nullptr) {
     const int d = head->d, h = head->h;
     const int subs = (h + SUB_H - 1) / SUB_H;
-    const int m_tiles = (N + TM - 1) / TM;
+    int m_tiles = (N + 127) / 128;
     if ((size_t)N * (size_t)subs > ARROL_SCRATCH_FLOATS || m_tiles > ARROL_SCORE_ROW_TILES)
         return ARROL_ERR_UNSUPPORTED;
     const bool pack = row_index != nullptr;
     if (pack && (size_t)N * (size_t)d * 2 > ARROL_PACK_BYTES) return ARROL_ERR_UNSUPPORTED;
     if (!row_index && ((uint64_t)row_stride * 2) >= (1ull << 40)) return ARROL_ERR_UNSUPPORTED;
     if (!ctx->score_tc_smem_set) {      // once per context: this call is on the prune step's microsecond path
-        for (const auto f : {score_mlp_tc_kernel<64, PARTIALS>, score_mlp_tc_kernel<64, SCORES>, score_mlp_tc_kernel<64, TRAIN>})
-            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64>()));
-        for (const auto f : {score_mlp_tc_kernel<128, PARTIALS>, score_mlp_tc_kernel<128, SCORES>, score_mlp_tc_kernel<128, TRAIN>})
-            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128>()));
+        for (const auto f : {score_mlp_tc_kernel<64, PARTIALS, 128>, score_mlp_tc_kernel<64, SCORES, 128>, score_mlp_tc_kernel<64, TRAIN, 128>})
+            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64, 128>()));
+        for (const auto f : {score_mlp_tc_kernel<128, PARTIALS, 128>, score_mlp_tc_kernel<128, SCORES, 128>, score_mlp_tc_kernel<128, TRAIN, 128>})
+            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<128, 128>()));
+        for (const auto f : {score_mlp_tc_kernel<64, SCORES, 64>, score_mlp_tc_kernel<64, TRAIN, 64>})
+            ARROL_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<64, 64>()));
         ctx->score_tc_smem_set = true;
     }
     // Tiles of 64 hidden units while they fit one wave of blocks (more SMs share the way in for the operands), of 128 beyond
@@ -497,11 +532,25 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
     bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
     const bool cluster = subs <= 8 || (subs <= MAX_SUBS && (wide || train));
     if (train && (!cluster || h % 8 != 0)) return ARROL_ERR_UNSUPPORTED;
-    if (cluster && !wide && subs > 1) {
-        int fit = 0;                    // clusters of more than eight blocks are not portable
-        if (subs <= 8 && narrow_clusters(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
-        wide = m_tiles > fit;
+    // Tiles of 64 rollouts where all of these fit at once: half as much of the epilogue per SM, and a third fewer operand bytes.  Graph
+    // of 20 calls, tiles of 128 / 64: N = 394, d = 1,664, h = 256 9.5 / 8.8 us, 1,000, 1,000, 320 11.2 / 9.5, 283, 600, 512 8.5 / 7.4, 32, 256, 64 6.0 /
+    // 5.4; training steps N = 2,048, d = 2,048, h = 256 26.8 / 25.4, 525, 2,880, 512 27.2 / 23.5.
+    bool half_rows = false;
+    if (cluster && subs <= 8) {         // clusters of more than eight blocks are not portable
+        int fit = 0;
+        if (narrow_clusters<64>(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
+        half_rows = (N + 63) / 64 <= fit;
+        if (half_rows) {
+            wide = false;
+            m_tiles = (N + 63) / 64;
+        } else if (!wide && subs > 1) {
+            if (narrow_clusters<128>(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
+            wide = m_tiles > fit;
+        }
+    } else if (cluster) {
+        wide = true;
     }
+    if (tile_rows) *tile_rows = half_rows ? 64 : 128;
     const int tiles_h = wide ? (h + 127) / 128 : subs;
     const void* x = hidden;
     int64_t ld = row_stride;
@@ -516,7 +565,7 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
     }
     CUtensorMap map_x, map_w;
     if (make_map(ctx, &map_w, head->W1, (uint64_t)h, (uint64_t)d, wide ? 128 : 64) != ARROL_OK) return ARROL_ERR_CUDA;
-    if (make_map_ld(ctx, &map_x, x, (uint64_t)N, (uint64_t)d, (uint64_t)ld, TM) != ARROL_OK) return ARROL_ERR_CUDA;
+    if (make_map_ld(ctx, &map_x, x, (uint64_t)N, (uint64_t)d, (uint64_t)ld, half_rows ? 64 : 128) != ARROL_OK) return ARROL_ERR_CUDA;
 
     p.N = N;
     p.h = h;
@@ -530,7 +579,7 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)m_tiles, (unsigned)tiles_h);
     cfg.blockDim = dim3(S_THREADS);
-    cfg.dynamicSmemBytes = wide ? smem_bytes<128>() : smem_bytes<64>();
+    cfg.dynamicSmemBytes = half_rows ? smem_bytes<64, 64>() : wide ? smem_bytes<128, 128>() : smem_bytes<64, 128>();
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -542,10 +591,11 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
     cfg.attrs = attr;
     cfg.numAttrs = cluster ? 2 : 1;
     const Mode mode = train ? TRAIN : cluster ? SCORES : PARTIALS;
-    const auto kernel = wide ? (mode == TRAIN ? score_mlp_tc_kernel<128, TRAIN> : mode == SCORES ? score_mlp_tc_kernel<128, SCORES>
-                                                                                          : score_mlp_tc_kernel<128, PARTIALS>)
-                             : (mode == TRAIN ? score_mlp_tc_kernel<64, TRAIN> : mode == SCORES ? score_mlp_tc_kernel<64, SCORES>
-                                                                                         : score_mlp_tc_kernel<64, PARTIALS>);
+    const auto kernel = half_rows ? (mode == TRAIN ? score_mlp_tc_kernel<64, TRAIN, 64> : score_mlp_tc_kernel<64, SCORES, 64>)
+                        : wide ? (mode == TRAIN ? score_mlp_tc_kernel<128, TRAIN, 128>
+                                                : mode == SCORES ? score_mlp_tc_kernel<128, SCORES, 128> : score_mlp_tc_kernel<128, PARTIALS, 128>)
+                               : (mode == TRAIN ? score_mlp_tc_kernel<64, TRAIN, 128>
+                                                : mode == SCORES ? score_mlp_tc_kernel<64, SCORES, 128> : score_mlp_tc_kernel<64, PARTIALS, 128>);
     ARROL_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, map_x, map_w, p));
     ctx->launches += 1;
     return ARROL_OK;
@@ -571,10 +621,10 @@ int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_
 }
 
 // The head training step up to the dW1 contraction, for at most 1,024 hidden units, a multiple of 8: du as two bf16 planes [N][h]; per tile of
-// 128 rollouts what dw2 and db1 (tile_sums [2][tiles][h]), loss and db2 (tile_loss [2][tiles]) are the sums of.  Rows as above.
+// *tile_rows rollouts (64 or 128) what dw2 and db1 (tile_sums [2][tiles][h]), loss and db2 (tile_loss [2][tiles]) are the sums of.  Rows as above.
 int arrol_internal_head_train_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
                                  const arrol_head* head, const float* rewards, const uint8_t* mask, void* du_hi, void* du_lo,
-                                 float* tile_sums, double* tile_loss, cudaStream_t s) {
+                                 float* tile_sums, double* tile_loss, int* tile_rows, cudaStream_t s) {
     ScoreTcParams p = {};
     p.rewards = rewards;
     p.mask = mask;
@@ -582,5 +632,5 @@ int arrol_internal_head_train_tc(arrol_ctx* ctx, const void* hidden, int64_t row
     p.du_lo = static_cast<__nv_bfloat16*>(du_lo);
     p.tile_sums = tile_sums;
     p.tile_loss = tile_loss;
-    return launch_mlp_tc(ctx, hidden, row_stride, row_index, N, head, true, p, s);
+    return launch_mlp_tc(ctx, hidden, row_stride, row_index, N, head, true, p, s, tile_rows);
 }

@@ -138,6 +138,13 @@ def test_mlp_head_clusters_of_every_size(ctx, h):
     _score_case(ctx, 1, 648, h, torch.bfloat16, False, False, seed=h + 1, bias=False)
 
 
+# tiles of 64 rollouts: the last one full, with one rollout, with one missing; both sides of what fits at once as clusters of five
+# blocks (fewer than 30 tiles or more than 29), where tiles of 128 take over
+@pytest.mark.parametrize("N", [63, 64, 65, 1024, 1400, 1856, 2113])
+def test_mlp_head_tiles_of_64_rollouts(ctx, N):
+    _score_case(ctx, N, 72, 260, torch.bfloat16, True, True, seed=N)
+
+
 def test_mlp_head_strided_rows_without_index(ctx):
     """Evenly strided rows (a column slice of a wider buffer) go to the tensor-core path without packing."""
     g = np.random.default_rng(5)
