@@ -71,8 +71,8 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 // One block, bound by latency: a handful of dependent round trips to memory and a serial search.  Every input is read once
 // (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
 // that one block scan ranks all of them, and the bisection is settled in two or three rounds of 31 points (see below) instead of 64
-// steps.  Per call, in a graph of 40 over changing states, mean of six (always three rounds before): N = 2,048, 128 bins 15.7 -> 13.3 us;
-// N = 32, 64 bins 12.5 -> 11.3; N = 8,192, 256 bins 24.5 -> 19.1; N = 3,000, 256 bins, lambda = 1.3 21.7 -> 19.5 (17.4 to 23.8: where
+// steps.  Per call, in a graph of 40 over changing states, mean of six (always three rounds, and a replay of all steps, before): N = 2,048, 128
+// bins, lambda = 0.5 15.7 -> 11.3 us; N = 32, 64 bins 12.5 -> 9.5; N = 8,192, 256 bins 24.5 -> 17.2; N = 3,000, 256 bins, lambda = 1.3 21.7 -> 19.5 (17.4 to 23.8: where
 // the threshold is not among the first neighbours it is three rounds still, with a second chain of additions).  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
@@ -354,6 +354,25 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
                     }
                 } else {                             // replay as far as the settled points reach
                     const double base_below = __dadd_rn(kappa, known_below), base_above = __dadd_rn(kappa, known_above);
+                    // The first midpoints are whole multiples of (1 + lambda) 2^-j, without rounding while their bits last: after j steps the bracket
+                    // is the cell of that grid that holds the threshold, found at once where 1 + lambda has few bits (51 steps of
+                    // lambda = 0.5; none of 0.3, whose midpoints are rounded from the third one on).
+                    const int used = 53 - min(52, __ffsll(__double_as_longlong(first_hi) | (1ll << 52)) - 1);      // bits of 1 + lambda
+                    if (step == 0 && used < 44 && known_below > first_lo && known_above < first_hi) {
+                        const int jump = 53 - used;
+                        const double cells = __longlong_as_double((long long)(1023 + jump) << 52), unit_cell = __longlong_as_double((long long)(1023 - jump) << 52);
+                        const double at = floor((known_below / first_hi + 1.0) * 0.5 * cells);
+#pragma unroll 1
+                        for (int k = -1; k <= 1 && step == 0; ++k) {         // one of these three, or none
+                            const double below_k = (2.0 * (at + k) - cells) * unit_cell * first_hi, above_k = (2.0 * (at + k + 1.0) - cells) * unit_cell * first_hi;
+                            if (at + k >= 0.0 && at + k + 1.0 <= cells && (at + k == 0.0 || __dadd_rn(kappa, below_k) <= base_below) &&
+                                (at + k + 1.0 == cells || __dadd_rn(kappa, above_k) >= base_above)) {
+                                lo = below_k;
+                                hi = above_k;
+                                step = jump;
+                            }
+                        }
+                    }
                     double m = midpoint(lo, hi);
                     while (step < 64) {              // both next midpoints while the comparison is under way
                         const double base = __dadd_rn(kappa, m), m_up = midpoint(m, hi), m_down = midpoint(lo, m);

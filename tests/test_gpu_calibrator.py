@@ -93,6 +93,24 @@ def test_delta_is_bit_equal_over_many_states_and_parameters(ctx):
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
 
 
+# 1 + lambda of 1 to 53 bits: the replay begins at the grid that its midpoints lie on without rounding, where that is more than 9 steps
+@pytest.mark.parametrize("lam", [0.0, 0.5, 1.0, 0.25, 1.0 + 2.0 ** -30, 2.0 ** -42, 2.0 ** -43, 2.0 ** -44, 2.0 ** -52, 0.3, 3.0 - 2.0 ** -40])
+def test_delta_for_lambdas_of_few_and_many_bits(ctx, lam):
+    g = np.random.default_rng(19)
+    for case in range(12):
+        n_bins = (16, 128)[case % 2]
+        cal = CAL.Calibrator(ctx, n_bins, 500)
+        prob = g.beta(*((2, 2), (0.5, 0.5), (8, 1))[case % 3], size=int(g.integers(1, 900))).astype(np.float32)
+        rew = (g.random(len(prob)) < prob).astype(np.float32)
+        bins = np.array([oracle.bin_index(float(v), n_bins) for v in prob], dtype=np.int32)
+        kappa, rho = float(g.uniform(0.1, 0.9)), float(g.uniform(0.2, 0.8))
+        cal.update(torch.from_numpy(bins).cuda(), torch.from_numpy(rew).cuda(), CAL.survival(kappa, lam, rho, 0.05, 0.95))
+        torch.cuda.synchronize()
+        snap = cal.snapshot()
+        delta = oracle.solve_delta(snap["cpos"], snap["cneg"], snap["q_lut"], kappa, lam, rho, 0.05, 0.95, iters=64)
+        assert snap["delta"] == delta, (case, kappa, rho)
+
+
 @pytest.mark.parametrize("lam", [0.0, 1e17, 1e300, 1.7e308, float("inf")])
 @pytest.mark.parametrize("alpha", [1.0, 0.0])                 # alpha = 0: empty bins have the posterior 0 / 0
 def test_delta_of_extreme_parameters_ends_where_a_plain_loop_does(ctx, lam, alpha):
