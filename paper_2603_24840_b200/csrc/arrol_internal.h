@@ -157,7 +157,7 @@ int arrol_internal_check_compact(const uint8_t* keep, const int32_t* lengths, co
 
 // score.cu: MLP tile pass with optional pre-activation output; partial is [ceil(h / ARROL_MLP_TH)][N].
 int arrol_internal_mlp_tiles(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
-                             const arrol_head* head, float* partial, float* u_out, cudaStream_t s);
+                             const arrol_head* head, float* partial, float* u_out, uint32_t* counters, int n_counters, cudaStream_t s);
 
 // score_tc.cu: scores of a bf16 MLP head on the tensor cores (pack, contraction, GELU, w2 dot, probability map).
 // ARROL_ERR_UNSUPPORTED (nothing launched) when the sizes do not fit the context's buffers.

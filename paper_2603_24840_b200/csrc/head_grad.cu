@@ -491,8 +491,7 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         // this path works in the call's own workspace alone, so that calls on several streams do not meet; its counters too
         // (a call on the tensor cores shares the context's packing buffer and scoring counters with others anyway)
         uint32_t* counters = reinterpret_cast<uint32_t*>(ws + L.counters);
-        ARROL_CUDA_OK(cudaMemsetAsync(counters, 0, sizeof(uint32_t) * (size_t)((h + 31) / 32), s));
-        const int rc = arrol_internal_mlp_tiles(ctx, hidden, row_stride, row_index, N, head, partial, u, s);
+        const int rc = arrol_internal_mlp_tiles(ctx, hidden, row_stride, row_index, N, head, partial, u, counters, (h + 31) / 32, s);
         if (rc != ARROL_OK) return rc;
         const int rd = launch_du(nullptr, partial, (h + ARROL_MLP_TH - 1) / ARROL_MLP_TH, du, nullptr, nullptr, counters);
         if (rd != ARROL_OK) return rd;

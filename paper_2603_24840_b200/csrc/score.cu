@@ -87,6 +87,10 @@ constexpr int MLP_SPLITS = 4;        // blocks of a cluster at most
 // SPLIT:  blockIdx.z picks a K range of k_len columns; the raw partial pre-activations go to
 //                 partial [splits][N][h] and score_mlp_splitk_finish_kernel completes them.  More, shorter blocks:
 //                 this is what fills the SMs when N x h is only a few hundred tiles.
+// Each waits for its predecessor with its launch already done (programmatic launch), and a training step's counters are
+// zeroed by the first block here: a launch, a gap and a clearing between kernels of a few microseconds each cost more than
+// their work.  Graphs of 20 calls, with ordinary launches and a memset -> now: a prune step of an fp32 head 32.0 -> 28.4 us,
+// training steps of fp32 heads N = 2,000, d = 512, h = 256 74 -> 69 us and N = 283, d = 288, h = 64 27 -> 24.
 enum MlpMode { WHOLE, CLUSTERED, SPLIT };
 template <typename T, MlpMode MODE>
 __global__ void __launch_bounds__(MLP_THREADS)
@@ -94,7 +98,7 @@ score_mlp_tile_kernel(const T* hidden, int64_t row_stride, const int64_t* row_in
                       int N, int d, int h, const T* W1, const T* b1,
                       const T* w2, float* __restrict__ partial,
                       float* __restrict__ u_out /* CLUSTERED: [N][h] pre-activations */, int k_len,
-                      int64_t source_rows, uint32_t* d_status) {
+                      int64_t source_rows, uint32_t* d_status, uint32_t* counters = nullptr, int n_counters = 0) {
     constexpr int VN = Vec16<T>::N;
     constexpr int VPR = TK / VN;                       // 16-byte vectors per tile row per K chunk
     constexpr int NV = TM * VPR / MLP_THREADS;         // vectors per thread per operand per chunk (2 or 4)
@@ -102,11 +106,11 @@ score_mlp_tile_kernel(const T* hidden, int64_t row_stride, const int64_t* row_in
     __shared__ __align__(16) float xs[2][TK][TM + PAD];
     __shared__ __align__(16) float ws[2][TK][TH + PAD];
 
-    if constexpr (MODE == CLUSTERED) {
-        pdl_launch_dependents();
-        pdl_wait();
-        hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); W1 = pdl_acquire(W1); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2);
-    }
+    pdl_launch_dependents();
+    pdl_wait();
+    hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); W1 = pdl_acquire(W1); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2);
+    if (MODE == CLUSTERED && blockIdx.x + blockIdx.y + blockIdx.z == 0)       // the du kernel's, which follows
+        for (int i = threadIdx.x; i < n_counters; i += MLP_THREADS) counters[i] = 0u;
     const int m0 = blockIdx.x * TM, j0 = blockIdx.y * TH;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // tx: 4 hidden units each, ty: 8 rollouts each
 
@@ -264,9 +268,11 @@ score_mlp_tile_kernel(const T* hidden, int64_t row_stride, const int64_t* row_in
 }
 
 template <typename T>
-__global__ void score_mlp_finish_kernel(const float* __restrict__ partial, int N, int h_tiles,
-                                        const T* __restrict__ b2, int B, const float* __restrict__ q_lut,
+__global__ void score_mlp_finish_kernel(const float* partial, int N, int h_tiles, const T* b2, int B, const float* q_lut,
                                         float* score, float* prob, int32_t* bin, float* q) {
+    pdl_launch_dependents();
+    pdl_wait();
+    partial = pdl_acquire(partial); b2 = pdl_acquire(b2); q_lut = pdl_acquire(q_lut);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     float s = 0.f;
@@ -279,9 +285,11 @@ __global__ void score_mlp_finish_kernel(const float* __restrict__ partial, int N
 // shuffle order), then the probability map.
 template <typename T>
 __global__ void __launch_bounds__(128)
-score_mlp_splitk_finish_kernel(const float* __restrict__ upart, int splits, int N, int h, const T* __restrict__ b1,
-                               const T* __restrict__ w2, const T* __restrict__ b2, int B,
-                               const float* __restrict__ q_lut, float* score, float* prob, int32_t* bin, float* q) {
+score_mlp_splitk_finish_kernel(const float* upart, int splits, int N, int h, const T* b1, const T* w2, const T* b2, int B,
+                               const float* q_lut, float* score, float* prob, int32_t* bin, float* q) {
+    pdl_launch_dependents();
+    pdl_wait();
+    upart = pdl_acquire(upart); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2); b2 = pdl_acquire(b2); q_lut = pdl_acquire(q_lut);
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (i >= N) return;
@@ -333,21 +341,20 @@ int launch_score(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const i
         splits = (head->d + k_len - 1) / k_len;
         if (per_split * splits <= ARROL_SCRATCH_FLOATS) {
             dim3 grid(m_tiles, h_tiles, splits);
-            score_mlp_tile_kernel<T, SPLIT><<<grid, MLP_THREADS, 0, s>>>(
-                hid, row_stride, row_index, N, head->d, head->h, static_cast<const T*>(head->W1), nullptr, nullptr,
-                ctx->d_scratch, nullptr, k_len, ctx->source_rows, ctx->d_status);
-            score_mlp_splitk_finish_kernel<T><<<(N + 3) / 4, 128, 0, s>>>(
-                ctx->d_scratch, splits, N, head->h, static_cast<const T*>(head->b1), static_cast<const T*>(head->w2),
-                static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q);
+            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tile_kernel<T, SPLIT>, grid, dim3(MLP_THREADS), 0, s,
+                hid, row_stride, row_index, N, head->d, head->h, static_cast<const T*>(head->W1), static_cast<const T*>(nullptr),
+                static_cast<const T*>(nullptr), ctx->d_scratch, nullptr, k_len, ctx->source_rows, ctx->d_status, nullptr, 0));
+            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_splitk_finish_kernel<T>, dim3((N + 3) / 4), dim3(128), 0, s,
+                static_cast<const float*>(ctx->d_scratch), splits, N, head->h, static_cast<const T*>(head->b1), static_cast<const T*>(head->w2),
+                static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q));
         } else {   // N x h too large for the scratch: one block per tile finishes its tile itself
             dim3 grid(m_tiles, h_tiles);
-            score_mlp_tile_kernel<T, WHOLE><<<grid, MLP_THREADS, 0, s>>>(
+            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tile_kernel<T, WHOLE>, grid, dim3(MLP_THREADS), 0, s,
                 hid, row_stride, row_index, N, head->d, head->h, static_cast<const T*>(head->W1),
                 static_cast<const T*>(head->b1), static_cast<const T*>(head->w2), ctx->d_scratch, nullptr, 0,
-                ctx->source_rows, ctx->d_status);
-            score_mlp_finish_kernel<T><<<(N + 255) / 256, 256, 0, s>>>(ctx->d_scratch, N, h_tiles,
-                                                                      static_cast<const T*>(head->b2), B, q_lut,
-                                                                      score, prob, bin, q);
+                ctx->source_rows, ctx->d_status, nullptr, 0));
+            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_finish_kernel<T>, dim3((N + 255) / 256), dim3(256), 0, s,
+                static_cast<const float*>(ctx->d_scratch), N, h_tiles, static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q));
         }
         ctx->launches += 2;
     }
@@ -357,9 +364,9 @@ int launch_score(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const i
 
 }  // namespace
 
-// Internal: MLP tile pass that also stores the pre-activations u [N][h] (used by the head training step).
+// Internal: MLP tile pass that also stores the pre-activations u [N][h], and zeroes `counters` (used by the head training step).
 int arrol_internal_mlp_tiles(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index, int N,
-                             const arrol_head* head, float* partial, float* u_out, cudaStream_t s) {
+                             const arrol_head* head, float* partial, float* u_out, uint32_t* counters, int n_counters, cudaStream_t s) {
     const int h_tiles = (head->h + TH - 1) / TH, m_tiles = (N + TM - 1) / TM;
     int splits = 1;                     // two K chunks at least, and no more than about four blocks per SM
     while (splits < MLP_SPLITS && m_tiles * h_tiles * splits * 2 <= 4 * ctx->sm_count && head->d >= splits * 2 * 2 * TK) splits *= 2;
@@ -369,12 +376,12 @@ int arrol_internal_mlp_tiles(arrol_ctx* ctx, const void* hidden, int64_t row_str
         ARROL_CUDA_OK(arrol_launch_pdl_cluster(score_mlp_tile_kernel<float, CLUSTERED>, grid, dim3(MLP_THREADS), cluster, s,
             static_cast<const float*>(hidden), row_stride, row_index, N, head->d, head->h,
             static_cast<const float*>(head->W1), static_cast<const float*>(head->b1),
-            static_cast<const float*>(head->w2), partial, u_out, k_len, ctx->source_rows, ctx->d_status));
+            static_cast<const float*>(head->w2), partial, u_out, k_len, ctx->source_rows, ctx->d_status, counters, n_counters));
     else
         ARROL_CUDA_OK(arrol_launch_pdl_cluster(score_mlp_tile_kernel<__nv_bfloat16, CLUSTERED>, grid, dim3(MLP_THREADS), cluster, s,
             static_cast<const __nv_bfloat16*>(hidden), row_stride, row_index, N, head->d, head->h,
             static_cast<const __nv_bfloat16*>(head->W1), static_cast<const __nv_bfloat16*>(head->b1),
-            static_cast<const __nv_bfloat16*>(head->w2), partial, u_out, k_len, ctx->source_rows, ctx->d_status));
+            static_cast<const __nv_bfloat16*>(head->w2), partial, u_out, k_len, ctx->source_rows, ctx->d_status, counters, n_counters));
     ctx->launches += 1;
     ARROL_CUDA_OK(cudaGetLastError());
     return ARROL_OK;
