@@ -826,7 +826,14 @@ int raise_smem_limits(arrol_ctx* ctx) {
     return ARROL_OK;
 }
 
-constexpr int FREE_TILES = 8;          // tiles per pair that are not kept in step
+constexpr int FREE_TILES = 16;         // tiles per pair that are not kept in step
+
+// A kernel, not a memset: the dz kernel can be resident and set up while it waits for this one, and for the kernel before.
+__global__ void clear_lock_kernel(unsigned int* words) {
+    pdl_launch_dependents();
+    pdl_wait();
+    if (threadIdx.x < LOCK_WORDS) words[threadIdx.x] = 0u;
+}
 
 struct BackwardLayout {
     int64_t ldz;       // V rounded up to 8
@@ -874,13 +881,14 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     __nv_bfloat16* dZ = reinterpret_cast<__nv_bfloat16*>(static_cast<uint8_t*>(workspace) + L.dz);
     uint16_t* Htail = reinterpret_cast<uint16_t*>(static_cast<uint8_t*>(workspace) + L.tail);
     unsigned int* lock_words = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + L.lock);
-    // The dz kernel's counter has to be zero before the first chunk (the later ones are zeroed by the kernels).  Clearing it costs a
-    // call 4 to 5 us, most of it because the dz kernel's start no longer overlaps the end of the kernel before it, so calls of which a pair
-    // has few tiles do without the step: they are over before pairs drift apart.  Policy loss and backward, in step / not: d = 512, V = 20,000,
-    // 1,500 tokens (6.4 tiles a pair) 101 / 95 us, 2,048 (8.5) 123 / 118, 5,000 (21) 273 / 269; d = 2,048, V = 12,000, 3,072 (7.6) 322 / 319, 6,144 (15)
-    // 615 / 612.  So at the line the step is not yet worth its clearing; it stays well below the launches that drift.
+    // The dz kernel's counter has to be zero before the first chunk (the later ones are zeroed by the kernels).  Clearing it puts a
+    // kernel's end and start, 3 us, before the dz kernel, and a memset 1.2 us more (backward, memset -> kernel: d = 512, V = 20,000, 2,048 tokens 121.8 ->
+    // 120.5 us; 320, 40,000, 1,536 147.5 -> 146.6), so calls of which a pair has few tiles do without the step: they are over before pairs
+    // drift apart.  Backward, in step / not: d = 512, V = 20,000, 2,048 tokens (8.5 tiles a pair) 120.9 / 118.4 us; 320, 40,000, 1,536 (12.7)
+    // 146.8 / 144.0; 256, 60,000, 1,200 (15.9) 141.2 / 138.5; and past the line 512, 20,000, 5,000 (21) 266 / 264; 320, 151,936, 700 (24) 261.9 / 261.5;
+    // 2,048, 60,000, 1,700 (22) 902 / 902; 4,096, 100,000, 1,000 (21) 1,801 / 1,803; 4,096, 10,000, 9,000 (19) 1,484 / 1,484.  At the line the
+    // step is not yet worth its clearing; it stays well below the launches that drift.
     const bool first_in_step = (T_max + TILE_ROWS - 1) / TILE_ROWS * ((V + BN - 1) / BN) > (int64_t)FREE_TILES * (ctx->sm_count / 2);
-    if (first_in_step) ARROL_CUDA_OK(cudaMemsetAsync(lock_words, 0, LOCK_BYTES, s));
     if (raise_smem_limits(ctx) != ARROL_OK) return ARROL_ERR_CUDA;
 
     // tensor maps: K-major operands are fetched as [128 MN rows x 64 K columns] boxes; MN-major ones (the same row-major
@@ -903,6 +911,10 @@ extern "C" int arrol_lm_head_backward(arrol_ctx* ctx, const void* hidden, const 
     }
     if (!v3 && make_map_ld(ctx, &map_dz_mn, dZ, TC, (uint64_t)V, (uint64_t)L.ldz, BK) != ARROL_OK) return ARROL_ERR_CUDA;
 
+    if (first_in_step) {
+        ARROL_CUDA_OK(arrol_launch_pdl(clear_lock_kernel, dim3(1), dim3(32), 0, s, lock_words));
+        ctx->launches += 1;
+    }
     const int n_tiles = (d + BN - 1) / BN;
     int m_groups = 1;
     while ((double)TC / m_groups * d * 2 > 50.0 * 1024 * 1024) ++m_groups;

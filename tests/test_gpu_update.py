@@ -201,6 +201,33 @@ def test_lm_head_backward_workspace_serves_any_number_of_tokens(ctx):
         _backward_case(ctx, T, d, 300, seed=d, T_live=T_live)
 
 
+# 16 tiles a pair on 74 pairs, the last that are not kept in step, and two tiles more, whose counters are cleared first
+@pytest.mark.parametrize("V", [592 * 256, 592 * 256 + 1])
+def test_lm_head_backward_does_not_depend_on_the_workspace(ctx, V):
+    T, d = 512, 64
+    g = torch.Generator(device="cuda").manual_seed(V)
+    H = torch.randn((T, d), generator=g, device="cuda").to(torch.bfloat16)
+    W = (torch.randn((V, d), generator=g, device="cuda") * 0.2).to(torch.bfloat16)
+    y = torch.randint(0, V, (T,), generator=g, device="cuda", dtype=torch.int32)
+    gl = torch.randn(T, generator=g, device="cuda")
+    z = H.double() @ W.double().T
+    lse = torch.logsumexp(z, dim=1)
+    ws = torch.empty(U.arrol_lm_head_backward_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+    got = []
+    for byte in (0, 255):
+        ws.fill_(byte)
+        dH, dW = torch.full((T, d), 9.0, device="cuda"), torch.full((V, d), 9.0, device="cuda")
+        U.arrol_lm_head_backward(ctx, H, W, y, gl, lse.float(), T, d, V, dH, dW, ws)
+        got.append((dH, dW))
+    assert B.arrol_poll_status(ctx) == 0
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    dz = -torch.exp(z - lse[:, None]) * gl[:, None].double()
+    dz[torch.arange(T, device="cuda"), y.long()] += gl.double()
+    # dz is held in bf16: 2^-9 of each term; the fp32 logits, exponentials and sums err by far less than the other 2^-9
+    for out, ref, bound in ((got[0][0], dz @ W.double(), dz.abs() @ W.double().abs()), (got[0][1], dz.T @ H.double(), dz.abs().T @ H.double().abs())):
+        assert bool(((out.double() - ref).abs() <= 2.0 ** -8 * bound + 1e-6).all())
+
+
 def test_lm_head_backwards_in_flight_on_two_streams(ctx):
     """Each launch fills the GPU and keeps its pairs of blocks in step; two at once get a part of the SMs each, so neither can
     count on all of its pairs running."""
