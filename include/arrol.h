@@ -57,8 +57,9 @@ int arrol_version(void);                    /* major*10000 + minor*100 + patch *
 const char* arrol_status_string(int status); /* static string, never NULL */
 
 /* Creates a context on CUDA device `device` (made current for the calling thread during the call).
- * Allocates the context's device status word, a 16 MB scratch buffer and a 64 MB row-packing buffer (MLP head),
- * 65 MB of pinned host memory, a second stream and a few events (used by arrol_prune_rebatch_host); nothing is
+ * Allocates the context's device status word, a 16 MB scratch buffer, a 64 MB row-packing buffer (MLP head), under 1 MB
+ * of counters and of survivors' records (arrol_prune_step), 65 MB of pinned host memory, a second stream and a few events
+ * (used by arrol_prune_rebatch_host); nothing is
  * allocated later.  Calls that use the context's buffers (MLP-head scoring, arrol_compact, arrol_prune_step and
  * arrol_prune_rebatch_host, the policy loss, the training step of a bf16 MLP head) must be ordered on the device with respect to one
  * another, e.g. by issuing them on one stream.  Calls that work in the caller's buffers alone may be in flight on several
@@ -358,7 +359,8 @@ int arrol_rank_vote(arrol_ctx* ctx, const float* score, const int32_t* answer, i
  * the small per-rollout arrays, the N hidden rows at the detection length (gathered into a pinned staging block of
  * the context and sent as one copy into d_hidden as a packed [N, d] block, for the head), and - once
  * arrol_score_partial and arrol_select have produced the keep mask, which is read back to plan the copies - the
- * survivors' hidden rows and token ids, copied straight into their packed positions in d_dst_rows / d_dst_tokens.
+ * survivors' hidden rows, copied straight into their packed positions in d_dst_rows (neighbours in the source as one
+ * copy), and their token ids, packed in the staging block and sent to d_dst_tokens once per chunk.
  * arrol_compact then produces the scan and the advantages, and arrol_token_logprob runs
  * per chunk of tokens as soon as the chunk's rows have landed (uploads on the context's second stream overlap the
  * tensor-core work).  Results are copied back and the stream is synchronised: the call is synchronous (one
