@@ -102,6 +102,19 @@ __device__ __forceinline__ T* pdl_acquire(T* p) {
 }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Barriers of part of a block.  Like every aligned instruction they want the warp converged; past a branch that its lanes took
+// differently nothing but the compiler's reconvergence would see to that, so the helpers of such instructions do (tc_common.cuh too).
+template <int ID, int THREADS>
+__device__ __forceinline__ void named_barrier_sync() {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+template <int ID, int THREADS>
+__device__ __forceinline__ void named_barrier_arrive() {
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+
 template <typename... KArgs, typename... Args>
 cudaError_t arrol_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                              Args&&... args) {

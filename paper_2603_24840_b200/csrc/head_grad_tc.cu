@@ -143,12 +143,12 @@ head_dw1_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constan
                     }
                 quarter_s[w * 32 + lane] = w2;
                 quarter_s[128 + w * 32 + lane] = b1;
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                named_barrier_sync<1, 128>();
                 if (w < 2 && j < p.h) {
                     const double* q = quarter_s + 128 * w + lane;
                     (w == 0 ? p.sums.dw2 : p.sums.db1)[j] = (float)(((q[0] + q[32]) + q[64]) + q[96]);
                 }
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                named_barrier_sync<1, 128>();
             }
             if (j0 == 0 && block == blocks - 1 && w >= 2) {
                 const double* tile_loss = pdl_acquire(p.sums.tile_loss) + (w - 2) * tiles;

@@ -177,8 +177,7 @@ prune_fused_kernel(const FusedParams p) {
             g_den[lane] = den;
         }
         __threadfence_block();
-        __syncwarp();                                        // the named barriers want their warps converged
-        asm volatile("bar.arrive 1, 64;" ::: "memory");
+        named_barrier_arrive<1, 64>();
         // The block is done with the chain when the first warp has added its total to the sums of the blocks after it and read its own.  The count's release is what
         // the clearing rests on: every block's stores have been performed before the last one to be counted zeroes the
         // words.  Without it what a block adds to the sum of one that has given up waiting could land after the zeros and be counted by a
@@ -186,7 +185,7 @@ prune_fused_kernel(const FusedParams p) {
         // those stores, so it is this warp's, beside the outputs that the first one writes.  Graphs of 20 calls, this / with a fence and
         // the count in the first warp / with nothing between stores and count: 2,048 rollouts at d = 2,560 19.5 / 20.3 / 20.1 us, 4,096
         // after an MLP head 70.4 / 70.6 / 70.0, 32 rollouts 9.4 / 10.3 / 9.9.
-        asm volatile("bar.sync 2, 64;" ::: "memory");
+        named_barrier_sync<2, 64>();
         unsigned long long done = 0;
         if (lane == 0) done = count_acq_rel(p.chain, 1ull + (block_left ? LEFT_ONE : 0ull) + (block_expired ? EXPIRED_ONE : 0ull));
         done = __shfl_sync(0xffffffffu, done, 0);
@@ -248,9 +247,8 @@ prune_fused_kernel(const FusedParams p) {
             if (base_t + block_t > p.capacity) atomicOr(p.d_status, ARROL_DEV_CAPACITY);
         }
     }
-    __syncwarp();
-    asm volatile("bar.arrive 2, 64;" ::: "memory");          // done with the chain
-    asm volatile("bar.sync 1, 64;" ::: "memory");            // the groups' statistics
+    named_barrier_arrive<2, 64>();                           // done with the chain
+    named_barrier_sync<1, 64>();                             // the groups' statistics
     if (kept) {
         const int pos = base_c + __popc(kept_lanes & ((1u << lane) - 1u));
         p.survivor_idx[pos] = first + lane;
