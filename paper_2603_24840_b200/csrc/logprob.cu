@@ -770,6 +770,7 @@ combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int3
         }
         __syncthreads();                    // the records are overwritten by the next ones
     }
+    cp_async_wait_all();                    // of a block past the live tokens: its copies land before its shared memory goes away
 }
 
 // How many vocabulary splits per token tile.  With one split every resident block streams a different token

@@ -26,3 +26,39 @@ def test_aligned_barriers_follow_a_warp_barrier(path):
 
 def test_the_rule_finds_the_barriers():
     assert sum(len(ALIGNED_BARRIER.findall(_code(p))) for p in SOURCES) >= 10
+
+
+def _kernels(code):
+    """(name, body) of every __global__ function."""
+    for m in re.finditer(r"__global__", code):
+        bounds = re.compile(r"__launch_bounds__\([^)]*\)").search(code, m.end(), m.end() + 80)
+        head = re.compile(r"(\w+)\s*\(").search(code, bounds.end() if bounds else m.end())
+        at = code.index("{", head.end())
+        depth, i = 0, at
+        while True:
+            depth += {"{": 1, "}": -1}.get(code[i], 0)
+            if depth == 0:
+                break
+            i += 1
+        yield head.group(1), code[at + 1:i]
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_kernels_wait_for_their_asynchronous_copies_on_every_way_out(path):
+    """A block's shared memory is another block's once it has left: where a kernel issues asynchronous copies, the wait for them stands at
+    the outermost level behind the last of them, and nothing returns in between."""
+    for name, body in _kernels(_code(path)):
+        if "cp_async_16(" not in body:
+            continue
+        depth, waits = 0, []
+        for m in re.finditer(r"[{}]|cp_async_wait_all\(\)", body):
+            depth += {"{": 1, "}": -1}.get(m.group(), 0)
+            if depth == 0 and m.group().startswith("cp_async"):
+                waits.append(m.start())
+        assert waits and waits[-1] > body.rindex("cp_async_16("), name
+        assert not re.search(r"\breturn;", body[body.index("cp_async_16("):waits[-1]]), name
+
+
+def test_the_rule_finds_the_kernels():
+    found = {name for p in SOURCES for name, _ in _kernels(_code(p))}
+    assert {"combine_splits_kernel", "token_logprob_kernel", "prune_fused_kernel", "column_sum_kernel"} <= found
