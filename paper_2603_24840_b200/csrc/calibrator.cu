@@ -356,9 +356,9 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
                     const double base_below = __dadd_rn(kappa, known_below), base_above = __dadd_rn(kappa, known_above);
                     // The first midpoints are whole multiples of (1 + lambda) 2^-j, without rounding while their bits last: after j steps the bracket
                     // is the cell of that grid that holds the threshold, found at once where 1 + lambda has few bits (51 steps of
-                    // lambda = 0.5; none of 0.3, whose midpoints are rounded from the third one on).
+                    // lambda = 0.5; none of 0.3, whose midpoints are rounded from the third one on; none past 2^1023, where lo + hi can overflow).
                     const int used = 53 - min(52, __ffsll(__double_as_longlong(first_hi) | (1ll << 52)) - 1);      // bits of 1 + lambda
-                    if (step == 0 && used < 44 && known_below > first_lo && known_above < first_hi) {
+                    if (step == 0 && used < 44 && first_hi <= 0x1p1023 && known_below > first_lo && known_above < first_hi) {
                         const int jump = 53 - used;
                         const double cells = __longlong_as_double((long long)(1023 + jump) << 52), unit_cell = __longlong_as_double((long long)(1023 - jump) << 52);
                         const double at = floor((known_below / first_hi + 1.0) * 0.5 * cells);

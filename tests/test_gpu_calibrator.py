@@ -130,6 +130,21 @@ def test_delta_of_extreme_parameters_ends_where_a_plain_loop_does(ctx, lam, alph
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
 
 
+# a bracket so wide that lo + hi overflows in its upper part, where the root lies: a plain loop ends at infinity from there on.  1 + lambda of
+# few bits, at and past the widest bracket whose midpoints cannot overflow
+@pytest.mark.parametrize("lam", [2.0 ** 1023, 2.0 ** 1023 + 2.0 ** 1010, 1.5 * 2.0 ** 1023, 1.5 * 2.0 ** 1023 + 2.0 ** 984, 1.75 * 2.0 ** 1023 + 2.0 ** 990])
+@pytest.mark.parametrize("rho", [0.2, 0.5, 0.8])
+def test_delta_where_a_plain_loops_midpoints_overflow(ctx, lam, rho):
+    cal = CAL.Calibrator(ctx, 1, 300)
+    rew = (np.arange(200) < 160).astype(np.float32)               # one bin: its posterior is 0.8
+    cal.update(torch.zeros(200, dtype=torch.int32, device="cuda"), torch.from_numpy(rew).cuda(), CAL.survival(0.5, lam, rho, 0.05, 0.95))
+    torch.cuda.synchronize()
+    snap = cal.snapshot()
+    with np.errstate(all="ignore"):
+        delta = oracle.solve_delta(snap["cpos"], snap["cneg"], snap["q_lut"], 0.5, lam, rho, 0.05, 0.95, iters=64)
+    assert snap["delta"] == delta
+
+
 def test_stochastic_selection_matches_oracle(ctx):
     g = np.random.default_rng(5)
     N = 100003
