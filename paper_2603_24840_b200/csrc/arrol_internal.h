@@ -27,7 +27,7 @@ struct arrol_ctx {
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool prune_smem_set;       // likewise for the fused prune step
-    int score_max_clusters[2][9]; // scoring kernel, tiles of 128 / 64 rollouts x 64 hidden units: clusters of so many blocks that are resident at once; 0 = not asked yet
+    int score_max_clusters[3][9]; // scoring kernel, tiles of 128 x 64, 64 x 64 and 128 x 128 rollouts x hidden units: clusters of so many blocks that are resident at once; 0 = not asked yet
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
     uint32_t test_spin_limit;  // arrol_test_hook: tries per pipeline wait of the log-prob kernel, 0 = the normal limit

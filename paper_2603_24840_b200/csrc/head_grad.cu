@@ -475,7 +475,7 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
                 int rc = arrol_internal_head_train_tc(ctx, hidden, row_stride, row_index, N, head, rewards, mask, du_hi, du_lo,
                                                       tile_sums, tile_loss, &tile_rows, s);
                 HeadTileSums sums = {(N + tile_rows - 1) / tile_rows, tile_sums, tile_loss, dw2, db1, loss, db2};
-                if (rc == ARROL_ERR_UNSUPPORTED) {      // more than 1,024 hidden units, or beyond the context's buffers
+                if (rc == ARROL_ERR_UNSUPPORTED) {      // no clusters for these sizes, or beyond the context's buffers
                     float* tmp = reinterpret_cast<float*>(ws + L.tmp3);
                     sums.tile_sums = nullptr;
                     rc = arrol_internal_score_mlp_tc(ctx, hidden, row_stride, row_index, N, head, 0, nullptr, tmp, tmp + N, nullptr,

@@ -476,15 +476,15 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
 }
 
-// Clusters of `blocks` blocks with tiles of ROWS rollouts x 64 hidden units that are resident at once (asked once per context and size).
-template <int ROWS>
-int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
-    int& known = ctx->score_max_clusters[ROWS == 64][blocks];
+// Clusters of `blocks` blocks with tiles of ROWS rollouts x SBN hidden units that are resident at once (asked once per context and size).
+template <int SBN, int ROWS>
+int resident_clusters(arrol_ctx* ctx, int blocks, int* fit) {
+    int& known = ctx->score_max_clusters[SBN == 128 ? 2 : ROWS == 64][blocks];
     if (known == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(1, (unsigned)blocks);
         cfg.blockDim = dim3(S_THREADS);
-        cfg.dynamicSmemBytes = smem_bytes<64, ROWS>();
+        cfg.dynamicSmemBytes = smem_bytes<SBN, ROWS>();
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 1;
@@ -492,7 +492,7 @@ int narrow_clusters(arrol_ctx* ctx, int blocks, int* fit) {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&known, score_mlp_tc_kernel<64, SCORES, ROWS>, &cfg));
+        ARROL_CUDA_OK(cudaOccupancyMaxActiveClusters(&known, score_mlp_tc_kernel<SBN, SCORES, ROWS>, &cfg));
     }
     *fit = known;
     return ARROL_OK;
@@ -522,36 +522,46 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
         ctx->score_tc_smem_set = true;
     }
     // Tiles of 64 hidden units while they fit one wave of blocks (more SMs share the way in for the operands), of 128 beyond
-    // that (a third fewer operand bytes and half as many blocks); the bits are the same.  As clusters fewer blocks fit: GPCs are
-    // not filled by clusters of any size.  Without / with the wide tiles (rows packed before, partial sums through global memory):
-    // N = 4,096, d = 4,096, h = 512 39.0 -> 28.4 us (8 of them the packing), N = 8,192 80.7 -> 64.7, N = 3,000, d = 1,024
-    // 17.1 -> 14.6; within one wave they lose: N = 2,048, d = 2,048, h = 256 14.2 -> 15.1.
+    // that (a third fewer operand bytes and half as many blocks); the bits are the same.  Without / with the wide tiles (rows packed
+    // before, partial sums through global memory): N = 4,096, d = 4,096, h = 512 39.0 -> 28.4 us (8 of them the packing), N = 8,192
+    // 80.7 -> 64.7, N = 3,000, d = 1,024 17.1 -> 14.6; within one wave they lose: N = 2,048, d = 2,048, h = 256 14.2 -> 15.1.
     // Up to eight blocks of 64 are a cluster, or of 128; nine to sixteen blocks of 64 that fit one wave stay without (N = 300, d = 4,096,
     // h = 1,024 15.7 us, as cluster of wide ones 17.1), but for the training step, which needs the cluster (N = 300, d = 512, h = 1,024
     // 23.8 -> 21.2).
+    // As clusters fewer blocks fit, GPCs not being filled by clusters of any size: 45, 33, 26, 22, 15 and 15 of three to eight blocks.  A
+    // cluster saves a call about 2 us, a wave more costs it more, so scores are clustered where that takes no more waves (asked
+    // once per context).  Without / with clusters, one wave more: d = 512: N = 6,000, h = 320 12.0 / 16.1 us, 9,000, 512 19.1 / 24.0, 2,100,
+    // 896 11.9 / 15.4, 14,000, 1,024 50.3 / 60.9; d = 3,072: 2,100, 1,024 24.0 / 29.7, 9,000, 768 67.0 / 77.4; as many: N = 3,000, d = 1,024,
+    // h = 512 14.7 / 12.9, 20,000, 256, 512 40.8 / 39.0.  The training step saves more, and is clustered unless one wave of the widest
+    // tile rows becomes two: h = 1,024, N = 2,100, d = 512 40.5 / 42.3, d = 3,072 75.9 / 81.5; but h = 896, N = 2,600 45.5 / 44.3 (2,100
+    // 41.7 / 42.5), h = 576, N = 3,300 43.5 / 36.9, h = 1,024, N = 4,200 63.3 / 63.0.
+    const int wide_tiles = (h + 127) / 128;
     bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
-    const bool cluster = subs <= 8 || (subs <= MAX_SUBS && (wide || train));
-    if (train && (!cluster || h % 8 != 0)) return ARROL_ERR_UNSUPPORTED;
+    const int waves = (m_tiles * (wide ? wide_tiles : subs) + ctx->sm_count - 1) / ctx->sm_count;       // without clusters
     // Tiles of 64 rollouts where all of these fit at once: half as much of the epilogue per SM, and a third fewer operand bytes.  Graph
     // of 20 calls, tiles of 128 / 64: N = 394, d = 1,664, h = 256 9.5 / 8.8 us, 1,000, 1,000, 320 11.2 / 9.5, 283, 600, 512 8.5 / 7.4, 32, 256, 64 6.0 /
     // 5.4; training steps N = 2,048, d = 2,048, h = 256 26.8 / 25.4, 525, 2,880, 512 27.2 / 23.5.
-    bool half_rows = false;
-    if (cluster && subs <= 8) {         // clusters of more than eight blocks are not portable
-        int fit = 0;
-        if (narrow_clusters<64>(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
+    bool cluster = false, half_rows = false;
+    int fit = 0;
+    if (!p.u_out && subs <= 8) {        // clusters of more than eight blocks are not portable
+        if (resident_clusters<64, 64>(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
         half_rows = (N + 63) / 64 <= fit;
         if (half_rows) {
             wide = false;
             m_tiles = (N + 63) / 64;
         } else if (!wide && subs > 1) {
-            if (narrow_clusters<128>(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
-            wide = m_tiles > fit;
+            if (resident_clusters<64, 128>(ctx, subs, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
         }
-    } else if (cluster) {
-        wide = true;
+        cluster = half_rows || (!wide && (subs == 1 || m_tiles <= fit));
     }
+    if (!p.u_out && !cluster && subs <= MAX_SUBS && (wide || train)) {
+        if (resident_clusters<128, 128>(ctx, wide_tiles, &fit) != ARROL_OK) return ARROL_ERR_CUDA;
+        cluster = fit > 0 && ((m_tiles + fit - 1) / fit <= waves || (train && (waves > 1 || wide_tiles < 8)));
+        wide = wide || cluster;
+    }
+    if (train && (!cluster || h % 8 != 0)) return ARROL_ERR_UNSUPPORTED;
     if (tile_rows) *tile_rows = half_rows ? 64 : 128;
-    const int tiles_h = wide ? (h + 127) / 128 : subs;
+    const int tiles_h = wide ? wide_tiles : subs;
     const void* x = hidden;
     int64_t ld = row_stride;
     if (pack) {
@@ -604,11 +614,10 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
 // Scores of a bf16 MLP head on the tensor cores.  Returns ARROL_ERR_UNSUPPORTED (nothing launched) when the sizes
 // do not fit the context's buffers; the caller then takes the SIMT path.  Indexed rows are left packed as bf16
 // [N][d] in the context's packing buffer (the head training step's second contraction reads them there).
-// u_out [N][h]: the pre-activations as well, of more than 1,024 hidden units only.
+// u_out [N][h]: the pre-activations as well (never clustered).
 int arrol_internal_score_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const int64_t* row_index,
                                 int N, const arrol_head* head, int B, const float* q_lut, float* score, float* prob,
                                 int32_t* bin, float* q, float* u_out, cudaStream_t s) {
-    if (u_out && head->h <= MAX_SUBS * SUB_H) return ARROL_ERR_UNSUPPORTED;
     ScoreTcParams p = {};
     p.u_out = u_out;
     p.B = B;

@@ -58,6 +58,13 @@ def test_head_grad_at_the_edges_of_its_tiles(N, d, h):
     test_head_grad_matches_oracle(N, d, h, torch.bfloat16, N % 2 == 0)
 
 
+# 1,024 hidden units: one wave of blocks that would be two of clusters goes without them, by way of the pre-activations; fewer and more
+# tiles of rollouts are clustered
+@pytest.mark.parametrize("N", [1792, 2176, 2304, 2305])
+def test_head_grad_on_both_sides_of_one_wave_without_clusters(N):
+    test_head_grad_matches_oracle(N, 72, 1024, torch.bfloat16, N % 2 == 0)
+
+
 # the fp32 kernels at their edges: K ranges over clusters of 1, 2 and 4 blocks (forward) and of 1 to 8 (dW1), one of them without a chunk,
 # tiles of 64 rollouts, hidden units and columns partly filled
 @pytest.mark.parametrize("N,d,h", [(1, 64, 8), (33, 1000, 68), (65, 264, 64), (130, 72, 132), (300, 600, 36), (700, 520, 260)])

@@ -130,6 +130,13 @@ def test_mlp_head_scores_do_not_depend_on_how_many_rollouts_are_scored(ctx, N, d
     assert all(torch.equal(a[:130], b) for a, b in zip(*out))
 
 
+# row tiles that would take a wave more as clusters (of three, seven and eight wide blocks; 27 tiles as clusters of five narrow ones): their
+# blocks go without, and give the bits of clustered ones; (5600, 64, 320) are clusters of wide ones, as many waves as without
+@pytest.mark.parametrize("N,d,h", [(5900, 72, 320), (2100, 136, 900), (2100, 72, 1024), (3400, 64, 320), (5600, 64, 320)])
+def test_mlp_head_scores_are_the_same_with_and_without_clusters(ctx, N, d, h):
+    test_mlp_head_scores_do_not_depend_on_how_many_rollouts_are_scored(ctx, N, d, h)
+
+
 # a row tile's blocks as a cluster of 1 to 8 (tiles of 64 hidden units; of 128 past 512), the last one partly past h, one row tile and two
 # with one row in the second, one K step and several; 1,028 hidden units go without clusters
 @pytest.mark.parametrize("h", [4, 64, 68, 192, 260, 512, 516, 1024, 1028])
