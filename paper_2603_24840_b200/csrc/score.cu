@@ -87,10 +87,14 @@ constexpr int MLP_SPLITS = 4;        // blocks of a cluster at most
 // SPLIT:  blockIdx.z picks a K range of k_len columns; the raw partial pre-activations go to
 //                 partial [splits][N][h] and score_mlp_splitk_finish_kernel completes them.  More, shorter blocks:
 //                 this is what fills the SMs when N x h is only a few hundred tiles.
-// Each waits for its predecessor with its launch already done (programmatic launch), and a training step's counters are
+// A training step's tiles are launched while the kernel before them runs (programmatic launch) and its counters are
 // zeroed by the first block here: a launch, a gap and a clearing between kernels of a few microseconds each cost more than
-// their work.  Graphs of 20 calls, with ordinary launches and a memset -> now: a prune step of an fp32 head 32.0 -> 28.4 us,
-// training steps of fp32 heads N = 2,000, d = 512, h = 256 74 -> 69 us and N = 283, d = 288, h = 64 27 -> 24.
+// their work.  Graphs of 20 calls, with ordinary launches and a memset -> now: N = 2,000, d = 512, h = 256 74 -> 69 us, N = 283, d = 288,
+// h = 64 27 -> 24.  Scores (WHOLE, SPLIT) are not: their blocks, bound by arithmetic, would pile up on the SMs that the finishing kernel of the
+// call before leaves free.  Ordinary / programmatic launches, scores of fp32 heads: N = 500, d = 1,024, h = 256 20.3 / 30.1 us, 1,500, 1,024, 64
+// 16.2 / 24.5, 500, 256, 512 19.7 / 23.7, 12,000, 256, 64 24.3 / 26.3, 64, 256, 64 6.6 / 6.2; prune steps P = 16, G = 8, d = 1,024,
+// h = 256 22.6 / 33.2, P = 128, 512, 128 19.1 / 24.6, P = 4, 256, 64 12.1 / 12.7.  Launching the finishing kernel alone that way: 10.2 / 12.6 at N = 64,
+// d = 256, h = 256, 1,500, 256, 64 8.3 / 8.1; the trigger behind the contraction: prune step P = 64, 512, 128 17.3 / 24.2.
 enum MlpMode { WHOLE, CLUSTERED, SPLIT };
 template <typename T, MlpMode MODE>
 __global__ void __launch_bounds__(MLP_THREADS)
@@ -106,11 +110,13 @@ score_mlp_tile_kernel(const T* hidden, int64_t row_stride, const int64_t* row_in
     __shared__ __align__(16) float xs[2][TK][TM + PAD];
     __shared__ __align__(16) float ws[2][TK][TH + PAD];
 
-    pdl_launch_dependents();
-    pdl_wait();
-    hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); W1 = pdl_acquire(W1); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2);
-    if (MODE == CLUSTERED && blockIdx.x + blockIdx.y + blockIdx.z == 0)       // the du kernel's, which follows
-        for (int i = threadIdx.x; i < n_counters; i += MLP_THREADS) counters[i] = 0u;
+    if constexpr (MODE == CLUSTERED) {
+        pdl_launch_dependents();
+        pdl_wait();
+        hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); W1 = pdl_acquire(W1); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2);
+        if (blockIdx.x + blockIdx.y + blockIdx.z == 0)       // the du kernel's, which follows
+            for (int i = threadIdx.x; i < n_counters; i += MLP_THREADS) counters[i] = 0u;
+    }
     const int m0 = blockIdx.x * TM, j0 = blockIdx.y * TH;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // tx: 4 hidden units each, ty: 8 rollouts each
 
@@ -270,9 +276,6 @@ score_mlp_tile_kernel(const T* hidden, int64_t row_stride, const int64_t* row_in
 template <typename T>
 __global__ void score_mlp_finish_kernel(const float* partial, int N, int h_tiles, const T* b2, int B, const float* q_lut,
                                         float* score, float* prob, int32_t* bin, float* q) {
-    pdl_launch_dependents();
-    pdl_wait();
-    partial = pdl_acquire(partial); b2 = pdl_acquire(b2); q_lut = pdl_acquire(q_lut);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     float s = 0.f;
@@ -287,9 +290,6 @@ template <typename T>
 __global__ void __launch_bounds__(128)
 score_mlp_splitk_finish_kernel(const float* upart, int splits, int N, int h, const T* b1, const T* w2, const T* b2, int B,
                                const float* q_lut, float* score, float* prob, int32_t* bin, float* q) {
-    pdl_launch_dependents();
-    pdl_wait();
-    upart = pdl_acquire(upart); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2); b2 = pdl_acquire(b2); q_lut = pdl_acquire(q_lut);
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (i >= N) return;
@@ -341,20 +341,20 @@ int launch_score(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const i
         splits = (head->d + k_len - 1) / k_len;
         if (per_split * splits <= ARROL_SCRATCH_FLOATS) {
             dim3 grid(m_tiles, h_tiles, splits);
-            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tile_kernel<T, SPLIT>, grid, dim3(MLP_THREADS), 0, s,
-                hid, row_stride, row_index, N, head->d, head->h, static_cast<const T*>(head->W1), static_cast<const T*>(nullptr),
-                static_cast<const T*>(nullptr), ctx->d_scratch, nullptr, k_len, ctx->source_rows, ctx->d_status, nullptr, 0));
-            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_splitk_finish_kernel<T>, dim3((N + 3) / 4), dim3(128), 0, s,
-                static_cast<const float*>(ctx->d_scratch), splits, N, head->h, static_cast<const T*>(head->b1), static_cast<const T*>(head->w2),
-                static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q));
+            score_mlp_tile_kernel<T, SPLIT><<<grid, MLP_THREADS, 0, s>>>(
+                hid, row_stride, row_index, N, head->d, head->h, static_cast<const T*>(head->W1), nullptr, nullptr,
+                ctx->d_scratch, nullptr, k_len, ctx->source_rows, ctx->d_status);
+            score_mlp_splitk_finish_kernel<T><<<(N + 3) / 4, 128, 0, s>>>(
+                ctx->d_scratch, splits, N, head->h, static_cast<const T*>(head->b1), static_cast<const T*>(head->w2),
+                static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q);
         } else {   // N x h too large for the scratch: one block per tile finishes its tile itself
             dim3 grid(m_tiles, h_tiles);
-            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_tile_kernel<T, WHOLE>, grid, dim3(MLP_THREADS), 0, s,
+            score_mlp_tile_kernel<T, WHOLE><<<grid, MLP_THREADS, 0, s>>>(
                 hid, row_stride, row_index, N, head->d, head->h, static_cast<const T*>(head->W1),
                 static_cast<const T*>(head->b1), static_cast<const T*>(head->w2), ctx->d_scratch, nullptr, 0,
-                ctx->source_rows, ctx->d_status, nullptr, 0));
-            ARROL_CUDA_OK(arrol_launch_pdl(score_mlp_finish_kernel<T>, dim3((N + 255) / 256), dim3(256), 0, s,
-                static_cast<const float*>(ctx->d_scratch), N, h_tiles, static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q));
+                ctx->source_rows, ctx->d_status);
+            score_mlp_finish_kernel<T><<<(N + 255) / 256, 256, 0, s>>>(
+                ctx->d_scratch, N, h_tiles, static_cast<const T*>(head->b2), B, q_lut, score, prob, bin, q);
         }
         ctx->launches += 2;
     }
