@@ -71,9 +71,11 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 // One block, bound by latency: a handful of dependent round trips to memory and a serial search.  Every input is read once
 // (the labelled bins are kept in shared memory up to CAL_STAGED rollouts), a thread owns a run of consecutive rollouts so
 // that one block scan ranks all of them, and the bisection is settled in two or three rounds of 31 points (see below) instead of 64
-// steps.  Per call, in a graph of 40 over changing states, mean of six (always three rounds, and a replay of all steps, before): N = 2,048, 128
-// bins, lambda = 0.5 15.7 -> 11.3 us; N = 32, 64 bins 12.5 -> 9.5; N = 8,192, 256 bins 24.5 -> 17.2; N = 3,000, 256 bins, lambda = 1.3 21.7 -> 19.5 (17.4 to 23.8: where
-// the threshold is not among the first neighbours it is three rounds still, with a second chain of additions).  More rollouts go through shared memory in pieces of CAL_STAGED,
+// steps.  Per call, in a graph of 36 over changing states, mean of six (always three rounds, and a replay of all steps, before), lambda = 0.5:
+// N = 2,048, 128 bins 15.7 -> 11.3 us; N = 32, 64 bins 12.9 -> 9.1; N = 8,192, 256 bins 23.5 -> 17.2.  lambda = 0.3, whose replay takes all
+// steps: N = 2,048, 128 bins 16.6 -> 13.9; N = 64, 256 bins 19.1 -> 14.2; N = 4,000, 256 bins 20.8 -> 18.6.  Where bins meet the clip limits the root may
+// lie next to a breakpoint, which more rounds follow: lambda = 1 to 1.3 0.65 to 1.19 of the former time by the state, 0.9 of the rounds in the mean
+// of 48 states each.  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
 // per thread and scan, as it was before the runs, 460 and 1,570).  An instance each, because the pieces' code in the same one cost
@@ -345,10 +347,13 @@ calib_update_kernel(uint8_t* state, CalibLayout L, const int32_t* __restrict__ b
                 double a = fmax(known_below, first_lo), b = fmin(known_above, first_hi), at = 0.0, unit = 0.0;
                 if (step >= 64) {
                     kind = DONE;
-                } else if (round < 3 && !(__dadd_rn(kappa, known_above) <= nextafter(__dadd_rn(kappa, known_below), inf))) {
+                } else if (round < 3 && !(__dadd_rn(kappa, known_above) <= nextafter(__dadd_rn(kappa, known_below), inf) ||
+                                          known_above <= nextafter(known_below, inf))) {
                     kind = EVEN;
                     if (round > 0 && known_below > -inf && slope_at > 0.0) {
+                        // kappa + at without rounding: neighbours taken from halfway between two values would round to every other one
                         at = fmin(fmax(known_below + (goal - sum_at) / slope_at, a), b);
+                        at = __dsub_rn(__dadd_rn(kappa, at), kappa);
                         kind = round == 2 && sum_in_order ? ADJACENT : AROUND;
                         unit = scalbn(1.0, ilogb(fmax(fmax(fabs(kappa + at), fabs(at)), 1e-200)) - 52);
                     }

@@ -130,6 +130,22 @@ def test_delta_of_extreme_parameters_ends_where_a_plain_loop_does(ctx, lam, alph
     assert B.arrol_poll_status(ctx, raise_on_error=False) == 0
 
 
+# kappas of few bits, beside which the root's neighbours may lie halfway between two values of kappa + delta, and roots on both sides of zero
+@pytest.mark.parametrize("kappa", [0.0, 0.125, 0.25, 0.5, 0.75, 1.0])
+def test_delta_beside_kappas_of_few_bits(ctx, kappa):
+    g = np.random.default_rng(23)
+    for case in range(24):
+        lam, rho, n_bins = (0.3, 0.1, 0.7, 0.5)[case % 4], (0.5, 0.2, 0.9)[case % 3], (64, 256)[case % 2]
+        cal = CAL.Calibrator(ctx, n_bins, 2048)
+        prob = g.beta(*((2, 2), (0.6, 0.6), (5, 2))[case % 3], size=int(g.integers(20, 3000))).astype(np.float32)
+        rew = (g.random(len(prob)) < prob).astype(np.float32)
+        bins = np.array([oracle.bin_index(float(v), n_bins) for v in prob], dtype=np.int32)
+        cal.update(torch.from_numpy(bins).cuda(), torch.from_numpy(rew).cuda(), CAL.survival(kappa, lam, rho, 0.0, 1.0))
+        torch.cuda.synchronize()
+        snap = cal.snapshot()
+        assert snap["delta"] == oracle.solve_delta(snap["cpos"], snap["cneg"], snap["q_lut"], kappa, lam, rho, 0.0, 1.0, iters=64), case
+
+
 # a bracket so wide that lo + hi overflows in its upper part, where the root lies: a plain loop ends at infinity from there on.  1 + lambda of
 # few bits, at and past the widest bracket whose midpoints cannot overflow
 @pytest.mark.parametrize("lam", [2.0 ** 1023, 2.0 ** 1023 + 2.0 ** 1010, 1.5 * 2.0 ** 1023, 1.5 * 2.0 ** 1023 + 2.0 ** 984, 1.75 * 2.0 ** 1023 + 2.0 ** 990])
