@@ -4,6 +4,7 @@
 
 #include "arrol_internal.h"
 #include "token_runs.cuh"
+#include "vocab_plan.cuh"
 
 extern "C" int arrol_version(void) { return 100; }
 
@@ -146,7 +147,7 @@ extern "C" int arrol_test_hook(arrol_ctx* ctx, int32_t key, int64_t value) {
             ctx->test_mute_producer = value != 0;
             return ARROL_OK;
         case ARROL_HOOK_LOGPROB_SPLITS:
-            if (value < 0 || value > 64) return ARROL_ERR_INVALID_ARG;
+            if (value < 0 || value > MAX_SPLITS) return ARROL_ERR_INVALID_ARG;
             ctx->logprob_splits = (int)value;
             return ARROL_OK;
         case ARROL_HOOK_LOGPROB_PAIR:

@@ -54,6 +54,7 @@
 
 #include "arrol_internal.h"
 #include "tc_common.cuh"
+#include "vocab_plan.cuh"
 
 namespace {
 
@@ -79,33 +80,6 @@ constexpr size_t SMEM_BYTES = (size_t)SOLO_STAGES * SOLO_STAGE_BYTES + 1024 /* a
 
 struct PartialLse {   // of one token over some columns: running maximum and sum in the base-2 domain, target logit,
     float m2, l, zy2, sumz;   // sum of the raw accumulators (only when the confidence is asked for)
-};
-
-// a / b of small whole numbers by b's rounded reciprocal, taken half a unit above a: exact while a < 2^16 and b < 2^10 (the margin is
-// 0.5 / b, the error a / b 2^-22).  An item of a small call would wait for the division of integers.
-__device__ __forceinline__ int quotient(int a, float inv_b) { return (int)(((float)a + 0.5f) * inv_b); }
-
-// How the vocabulary is cut: total_chunks chunks of BN columns -> n_sub segments -> n_mid blocks of segments -> splits
-// groups.  A body item covers a whole group, a tail item one segment; a token's records are merged segment by segment
-// into a block, block by block into a group, then group by group, by whichever kernel holds them.
-constexpr int MAX_SPLITS = 64;
-struct VocabPlan {
-    int total_chunks, n_sub, n_mid, splits;
-    int per_sub;          // whole chunks per segment, n_long segments hold one more
-    int n_long;           // total_chunks mod n_sub
-    float inv_sub, inv_long, inv_short;   // 1 / n_sub, 1 / n_long, 1 / (n_sub - n_long)
-    uint8_t mid_begin[MAX_SPLITS + 1];    // first segment of every block of segments (n_sub <= SMs < 256)
-    uint8_t group_begin[MAX_SPLITS + 1];  // first block of every group
-    // floor(i total_chunks / n_sub), without a division
-    __device__ int chunk_of_sub(int i) const { return i * per_sub + quotient(i * n_long, inv_sub); }
-    // j-th segment in the order of dealing: the long ones first.  Segment i is long where floor(i n_long / n_sub) steps after i,
-    // short where ceil(i (n_sub - n_long) / n_sub) does.
-    __device__ int nth_sub(int j) const {
-        const bool is_long = j < n_long;
-        const int a = is_long ? (j + 1) * n_sub + n_long - 1 : (j - n_long) * n_sub;
-        return quotient(a, is_long ? inv_long : inv_short) - (is_long ? 1 : 0);
-    }
-    __device__ int sub_of_group(int g) const { return mid_begin[group_begin[g]]; }
 };
 
 // (M, L) <- (M, L) + (m, l): M = max, L = sum of 2^(. - M).  One rounding per operation, so that the main kernel (body)
@@ -820,25 +794,8 @@ bool pair_for(const arrol_ctx* ctx, int64_t T_max, int d) {
 int halves_for(int d) { return d <= EIGHT_WARPS_MAX_WIDTH ? 2 : 1; }
 
 VocabPlan plan_for(const arrol_ctx* ctx, int d, int V) {
-    VocabPlan v;
-    v.total_chunks = (V + BN - 1) / BN;
     // the same for every token count: where the form depends on that, both forms' resident tiles are far below either budget
-    v.splits = splits_for(ctx, d, V, pair_for(ctx, INT64_MAX, d));
-    // one segment per SM: then the tail's items fill the units (SMs, or half as many pairs) a whole number of times
-    v.n_sub = v.total_chunks < ctx->sm_count ? v.total_chunks : ctx->sm_count;
-    v.n_long = v.total_chunks % v.n_sub;
-    v.inv_long = v.n_long > 0 ? 1.0f / (float)v.n_long : 0.f;
-    v.inv_short = 1.0f / (float)(v.n_sub - v.n_long);
-    v.per_sub = v.total_chunks / v.n_sub;
-    v.inv_sub = 1.0f / (float)v.n_sub;
-    if (v.n_sub < v.splits) v.splits = v.n_sub;
-    // as many blocks as there are segments in each, so that the two chains of merges together are shortest
-    int per_group = 1;
-    while (v.splits * per_group * v.splits * per_group < v.n_sub) ++per_group;
-    v.n_mid = v.splits * per_group < v.n_sub ? v.splits * per_group : v.n_sub;
-    for (int i = 0; i <= v.n_mid; ++i) v.mid_begin[i] = (uint8_t)(i * v.n_sub / v.n_mid);
-    for (int g = 0; g <= v.splits; ++g) v.group_begin[g] = (uint8_t)(g * v.n_mid / v.splits);
-    return v;
+    return make_vocab_plan(ctx->sm_count, (V + BN - 1) / BN, splits_for(ctx, d, V, pair_for(ctx, INT64_MAX, d)));
 }
 
 // Workspace: wave counter, body records, tail records, source rows of the token tiles (gathered variant).  Every part
