@@ -641,18 +641,15 @@ pack_boundary_tiles_kernel(const uint4* __restrict__ src_rows, const int64_t* __
 // `group` consecutive ones, whose records lie one after another and come into shared memory by asynchronous copies; a thread
 // merges the segments of one block of segments (and column half), then a thread per token and half walks the blocks in order.
 // Bound by latency: one round trip for the length, the targets and the records together (where no call of T_max tokens has a body the
-// records' place does not depend on the length), then some 25 dependent merges of 50 cycles.  Registers and shared memory leave
-// room for one block beside the log-prob kernel's on every SM, where it waits; blocks past that would pile up on the SM that is
-// free first.  A warp per token, its lanes the blocks of segments and then all of them the same chain of 16 merges, took 4.5 to 6.5 us
+// records' place does not depend on the length), then some 25 dependent merges of 50 cycles.  Of calls with no more blocks than fit at once,
+// registers and shared memory leave room for one beside the log-prob kernel's on every SM, where it waits; blocks past that would pile up
+// on the SM that is free first.  A warp per token, its lanes the blocks of segments and then all of them the same chain of 16 merges, took 4.5 to 6.5 us
 // of a call of 2,800 tokens on V = 4,096 (d = 256), and takes 2.8 to 3.4 now.  With the items listed ahead the whole call went from 18.9 to
 // 14.4 us (graph of 20), 3,636 tokens at d = 320 on V = 14,170 from 41.9 to 35.0.
 constexpr int COMBINE_THREADS = 256;
-constexpr int COMBINE_GROUP = 32;                  // most tokens per block
-constexpr size_t COMBINE_SMEM = 32 * 1024;
-// tokens of the tail per block, `per_token` records each
-__host__ __device__ inline size_t combine_bytes(const VocabPlan& v, int halves) { return (size_t)(v.n_sub + (v.n_mid < v.n_sub ? v.n_mid : 0)) * halves * 16; }
+static_assert((MAX_SEGMENTS + MAX_SPLITS) * 2 * 16 + SMEM_BYTES + 2 * BLOCK_SMEM_RESERVED <= SM_SMEM, "a token's records fit beside the log-prob kernel");
 template <int HALVES>
-__global__ void __launch_bounds__(COMBINE_THREADS, 4)
+__global__ void __launch_bounds__(COMBINE_THREADS, COMBINE_BLOCKS)
 combine_splits_kernel(const PartialLse* body, const PartialLse* tail, const int32_t* targets, const int64_t* d_T,
                       int64_t T_max, int V, VocabPlan plan, int tile_rows, int units, int group, int block_lanes, bool tail_only,
                       float* __restrict__ logp, float* __restrict__ lse, float* __restrict__ conf, float inv_temp, uint32_t* d_status) {
@@ -983,10 +980,7 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
     const bool tail_only = p.work.body_tiles == 0;      // fewer tokens have none either
     int64_t tail_rows = (tiles_max < units / p.plan.splits + 1 ? tiles_max : units / p.plan.splits + 1) * tile_rows;
     if (tail_rows > T_max) tail_rows = T_max;
-    const size_t token_bytes = combine_bytes(p.plan, halves);
-    int64_t group = (tail_rows + ctx->sm_count - 1) / ctx->sm_count;
-    if (group > COMBINE_GROUP) group = COMBINE_GROUP;
-    if (group > (int64_t)(COMBINE_SMEM / token_bytes)) group = (int64_t)(COMBINE_SMEM / token_bytes);
+    const int group = combine_group(p.plan, halves, tail_rows, ctx->sm_count, SMEM_BYTES);
     int64_t blocks = (tail_rows + group - 1) / group;
     int block_lanes = 0;
     while ((1 << block_lanes) < p.plan.n_mid * halves) ++block_lanes;
@@ -995,9 +989,9 @@ static int run_token_logprob(arrol_ctx* ctx, const void* hidden, const void* W_v
         if (blocks > (int64_t)ctx->sm_count * 8) blocks = (int64_t)ctx->sm_count * 8;
     }
     const auto combine = halves == 2 ? combine_splits_kernel<2> : combine_splits_kernel<1>;
-    ARROL_CUDA_OK(arrol_launch_pdl(combine, dim3((unsigned)blocks), dim3(COMBINE_THREADS), (size_t)group * token_bytes, s,
+    ARROL_CUDA_OK(arrol_launch_pdl(combine, dim3((unsigned)blocks), dim3(COMBINE_THREADS), (size_t)group * combine_bytes(p.plan, halves), s,
                                    static_cast<const PartialLse*>(p.body), static_cast<const PartialLse*>(p.tail), targets, d_T,
-                                   T_max, V, p.plan, (int)tile_rows, (int)units, (int)group, block_lanes, tail_only, logp, lse, conf, inv_temperature, ctx->d_status));
+                                   T_max, V, p.plan, (int)tile_rows, (int)units, group, block_lanes, tail_only, logp, lse, conf, inv_temperature, ctx->d_status));
     ctx->launches += 1;
     return ARROL_OK;
 }

@@ -13,7 +13,7 @@ def _run(tmp_path, body):
     if gxx is None:
         pytest.skip("no C++ compiler")
     src = tmp_path / "plan.cpp"
-    src.write_text('#include <cstdio>\n#include <cstdlib>\n#include "vocab_plan.cuh"\n'
+    src.write_text('#include <cstdio>\n#include <cstdlib>\n#include <initializer_list>\n#include "vocab_plan.cuh"\n'
                    '#define CHECK(c) do { if (!(c)) { std::printf("%s: sm %d chunks %d splits %d\\n", #c, sm, chunks, splits); std::exit(1); } } while (0)\n'
                    "int main() {\n" + body + "\n  return 0;\n}\n")
     subprocess.check_call([gxx, "-std=c++17", "-O2", "-Wall", "-I", CSRC, str(src), "-o", str(tmp_path / "plan")])
@@ -45,3 +45,30 @@ def test_segments_blocks_and_groups_cover_the_vocabulary_on_any_number_of_sms(tm
       dealt[s] = true;
     }
   }""")
+
+
+def test_the_combining_kernel_fits_beside_the_log_prob_kernel(tmp_path):
+    """Whatever the vocabulary and the tail: where all blocks of the combining kernel fit at once, four an SM, one of them and one of the
+    log-prob kernel (its 195 KB) are within the shared memory of an SM; and no block takes fewer tokens than that, 32 KB, 32 tokens or an
+    SM's share of the tail allow."""
+    _run(tmp_path, r"""
+  const size_t beside = 4 * 48 * 1024 + 1024 + 256 + 64 * 28, sm_bytes = 228 * 1024, reserved = 1024;
+  const int sm = 148;
+  int most = 0, beyond = 0;
+  for (int chunks = 1; chunks <= 600; ++chunks) for (int splits = 1; splits <= 64 && splits <= chunks; splits += splits < 8 ? 1 : 7) for (int halves = 1; halves <= 2; ++halves) {
+    const VocabPlan v = make_vocab_plan(sm, chunks, splits);
+    for (long rows : {1L, 100L, 148L, 149L, 888L, 1000L, 2800L, 3552L, 3553L, 3996L, 4200L, 9472L}) {
+      const int group = combine_group(v, halves, rows, sm, beside);
+      CHECK(group >= 1 && group <= 32 && group <= (rows + sm - 1) / sm);
+      const size_t token = combine_bytes(v, halves), bytes = group * token;
+      const bool fits = beside + bytes + 2 * reserved <= sm_bytes, at_once = (rows + group - 1) / group <= 4 * sm;
+      CHECK(bytes <= 32 * 1024);
+      CHECK(group == 32 || group == (rows + sm - 1) / sm || bytes + token > (fits ? sm_bytes - beside - 2 * reserved : 32 * 1024));
+      // past the line only where the smaller blocks would not fit at once
+      if (!fits) { ++beyond; CHECK(rows > (long)((sm_bytes - beside - 2 * reserved) / token) * 4 * sm); }
+      CHECK(fits || !at_once || rows > (long)((sm_bytes - beside - 2 * reserved) / token) * 4 * sm);
+      most = group > most ? group : most;
+    }
+  }
+  const int chunks = 0, splits = 0;
+  CHECK(most == 32 && beyond > 0);""")
