@@ -228,6 +228,24 @@ def test_lm_head_backward_does_not_depend_on_the_workspace(ctx, V):
         assert bool(((out.double() - ref).abs() <= 2.0 ** -8 * bound + 1e-6).all())
 
 
+def test_lm_head_backward_clears_its_counters_past_16_tiles_a_pair(ctx):
+    """One kernel more, which clears the counters that keep the pairs in step: results do not show whether it ran, launches do."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the line is drawn by the number of SMs")
+    T, d = 512, 64
+    H, gl = torch.zeros((T, d), dtype=torch.bfloat16, device="cuda"), torch.zeros(T, device="cuda")
+    y = torch.zeros(T, dtype=torch.int32, device="cuda")
+    launches = []
+    for V in (592 * 256, 592 * 256 + 1):
+        ws = torch.empty(U.arrol_lm_head_backward_workspace(ctx, T, d, V), dtype=torch.uint8, device="cuda")
+        W, dW = torch.zeros((V, d), dtype=torch.bfloat16, device="cuda"), torch.empty((V, d), device="cuda")
+        before = B.arrol_launch_count(ctx)
+        U.arrol_lm_head_backward(ctx, H, W, y, gl, gl, T, d, V, torch.empty((T, d), device="cuda"), dW, ws)
+        launches.append(B.arrol_launch_count(ctx) - before)
+    assert B.arrol_poll_status(ctx) == 0
+    assert launches[1] == launches[0] + 1
+
+
 def test_lm_head_backwards_in_flight_on_two_streams(ctx):
     """Each launch fills the GPU and keeps its pairs of blocks in step; two at once get a part of the SMs each, so neither can
     count on all of its pairs running."""
