@@ -162,11 +162,13 @@ column_sum_kernel(const float* partial, const double* chunk_loss, int chunks, in
     }
 }
 
-// MLP head: everything between the forward and the dW1 contraction in one launch: ds_i, the loss, du_ij, and per hidden unit
+// MLP heads whose forward does not form du itself (fp32, h not a multiple of 8, and where the tensor-core forward goes without clusters):
+// everything between the forward and the dW1 contraction in one launch: ds_i, the loss, du_ij, and per hidden unit
 // the sums dw2_j = sum_i ds_i gelu(u_ij), db1_j = sum_i du_ij.  (It was four launches: ds by one block, du, two column sums,
-// 22 us at N = 2,048, h = 256 against 9 now.)  Block (x, y): 32 hidden units, a run of rollouts.  Every block counts the labelled rollouts itself and forms the
-// ds of its own run; the last block of a column tile to arrive (a counter per tile, zero again when that block is through) adds the runs' sums in
-// index order, the one of tile 0 the loss and db2 as well.  The score is given, or the sum of the forward's tile partials + b2.
+// 22 us at N = 2,048, h = 256 against 9.)  Block (x, y): 32 hidden units, a run of rollouts.  Every block counts the labelled
+// rollouts itself and forms the ds of its own run; the last block of a column tile to arrive (a counter per tile, zero again when that
+// block is through) adds the runs' sums in index order, the one of tile 0 the loss and db2 as well.  The score is given, or the sum of
+// the forward's tile partials + b2.
 // du goes out as float (SIMT contraction) or as the sum of two bf16 planes (error 2^-17 relative: the tensor-core operand).
 constexpr int DU_THREADS = 256;
 template <typename T>
@@ -297,7 +299,8 @@ head_du_kernel(const float* u, const float* score, const float* partial, int h_t
 // shared memory and are added in rank order; and a chunk waits for its row numbers and then for its rows, so they are requested
 // two chunks and one ahead.  N = 2,000, d = 512, h = 256 (fp32): this
 // kernel 292 us under the profiler as 32 blocks that waited for every load; whole call, with the forward's K over a cluster
-// too, graph of 20: 234 -> 74 us, N = 8,000, d = 1,024, h = 256 962 -> 336, 5,000, 256, 64 488 -> 65, 283, 288, 64 55 -> 27.
+// too and the launches below, graph of 20: 235 -> 58 us, N = 8,000, d = 1,024, h = 256 957 -> 315,
+// 5,000, 256, 64 488 -> 61, 283, 288, 64 55 -> 23.
 constexpr int GT = 64, GK = 32, GPAD = 4, DW1_THREADS = 128, DW1_SPLITS = 8;
 template <typename T>
 __global__ void __launch_bounds__(DW1_THREADS)
@@ -448,10 +451,10 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
     } else {
         float* u = reinterpret_cast<float*>(ws + L.u);
         float* du = reinterpret_cast<float*>(ws + L.du);
+        const int rows_per = ((N + DU_RUNS - 1) / DU_RUNS + 7) / 8 * 8;
+        const int runs = (N + rows_per - 1) / rows_per;
         auto launch_du = [&](const float* score, const float* tile_partial, int h_tiles, float* du_f, __nv_bfloat16* hi,
                              __nv_bfloat16* lo, uint32_t* counters) -> int {
-            const int rows_per = ((N + DU_RUNS - 1) / DU_RUNS + 7) / 8 * 8;
-            const int runs = (N + rows_per - 1) / rows_per;
             ARROL_CUDA_OK(arrol_launch_pdl(head_du_kernel<T>, dim3((h + 31) / 32, runs), dim3(DU_THREADS), sizeof(float) * rows_per, s,
                                            static_cast<const float*>(u), score, tile_partial, h_tiles,
                                            score ? nullptr : static_cast<const T*>(head->b2), rewards, mask,
@@ -498,8 +501,13 @@ int run_head_grad(arrol_ctx* ctx, const void* hidden, int64_t row_stride, const 
         const int tiles = ((d + GT - 1) / GT) * ((h + GT - 1) / GT), row_chunks = (N + GK - 1) / GK;
         int splits = 1;                     // two chunks at least, and no more than about four blocks per SM
         while (splits < DW1_SPLITS && tiles * splits * 2 <= 4 * ctx->sm_count && row_chunks >= splits * 2 * 2) splits *= 2;
-        ARROL_CUDA_OK(arrol_launch_pdl_cluster(mlp_dw1_kernel<T>, dim3((d + GT - 1) / GT, (h + GT - 1) / GT, splits), dim3(DW1_THREADS),
-                                               dim3(1, 1, splits), s, static_cast<const float*>(du), hid, row_stride, row_index, N, d, h, dW1));
+        // Launched while the du kernel runs where both kernels' blocks have an SM each: more of them would pile up on the SMs that the du
+        // kernel leaves free.  When it has ended / while it runs: N = 64, d = 256, h = 64 (4 + 16 blocks) 19.9 / 18.2 us, 300, 512, 128 (64 + 76)
+        // 27.5 / 26.6, 20,000, 256, 64 (32 + 64) 188 / 187; past the line 300, 1,024, 256 (256 + 152) 36.4 / 39.9, 4,000, 512, 128 (128 + 128)
+        // 79 / 90, 7,000, 1,024, 64 (128 + 64) 131 / 167, 700, 1,024, 64 (128 + 60) 37.1 / 36.2.
+        const bool early = tiles * splits + (h + 31) / 32 * runs <= ctx->sm_count;
+        ARROL_CUDA_OK(arrol_launch_cluster(early, mlp_dw1_kernel<T>, dim3((d + GT - 1) / GT, (h + GT - 1) / GT, splits), dim3(DW1_THREADS),
+                                           dim3(1, 1, splits), s, static_cast<const float*>(du), hid, row_stride, row_index, N, d, h, dW1));
         ctx->launches += 1;
     }
     ARROL_CUDA_OK(cudaGetLastError());

@@ -87,14 +87,13 @@ constexpr int MLP_SPLITS = 4;        // blocks of a cluster at most
 // SPLIT:  blockIdx.z picks a K range of k_len columns; the raw partial pre-activations go to
 //                 partial [splits][N][h] and score_mlp_splitk_finish_kernel completes them.  More, shorter blocks:
 //                 this is what fills the SMs when N x h is only a few hundred tiles.
-// A training step's tiles are launched while the kernel before them runs (programmatic launch) and its counters are
-// zeroed by the first block here: a launch, a gap and a clearing between kernels of a few microseconds each cost more than
-// their work.  Graphs of 20 calls, with ordinary launches and a memset -> now: N = 2,000, d = 512, h = 256 74 -> 69 us, N = 283, d = 288,
-// h = 64 27 -> 24.  Scores (WHOLE, SPLIT) are not: their blocks, bound by arithmetic, would pile up on the SMs that the finishing kernel of the
-// call before leaves free.  Ordinary / programmatic launches, scores of fp32 heads: N = 500, d = 1,024, h = 256 20.3 / 30.1 us, 1,500, 1,024, 64
-// 16.2 / 24.5, 500, 256, 512 19.7 / 23.7, 12,000, 256, 64 24.3 / 26.3, 64, 256, 64 6.6 / 6.2; prune steps P = 16, G = 8, d = 1,024,
-// h = 256 22.6 / 33.2, P = 128, 512, 128 19.1 / 24.6, P = 4, 256, 64 12.1 / 12.7.  Launching the finishing kernel alone that way: 10.2 / 12.6 at N = 64,
-// d = 256, h = 256, 1,500, 256, 64 8.3 / 8.1; the trigger behind the contraction: prune step P = 64, 512, 128 17.3 / 24.2.
+// The tiles' blocks are bound by arithmetic and launched when the kernel before them has ended: launched while it runs (programmatic launch)
+// they pile up on the SMs that it leaves free.  Ordinary / programmatic launches, graphs of 20 calls, scores of fp32 heads: N = 500,
+// d = 1,024, h = 256 20.3 / 30.1 us, 1,500, 1,024, 64 16.2 / 24.5, 500, 256, 512 19.7 / 23.7, 12,000, 256, 64 24.3 / 26.3, 64, 256, 64 6.6 / 6.2; prune
+// steps P = 16, G = 8, d = 1,024, h = 256 22.6 / 33.2, P = 128, 512, 128 19.1 / 24.6, P = 4, 256, 64 12.1 / 12.7; training steps N = 700, 1,024,
+// 256 51.3 / 70.3, 20,000, 256, 64 186 / 270, 64, 256, 64 17.9 / 18.9.  Launching the finishing kernel of the scores early: 10.2 / 12.6 at N = 64,
+// d = 256, h = 256, 1,500, 256, 64 8.3 / 8.1; the trigger behind the contraction: prune step P = 64, 512, 128 17.3 / 24.2.  A training step's du
+// kernel is launched early, and its counters are zeroed by the first block here instead of a memset.
 enum MlpMode { WHOLE, CLUSTERED, SPLIT };
 template <typename T, MlpMode MODE>
 __global__ void __launch_bounds__(MLP_THREADS)
@@ -112,8 +111,6 @@ score_mlp_tile_kernel(const T* hidden, int64_t row_stride, const int64_t* row_in
 
     if constexpr (MODE == CLUSTERED) {
         pdl_launch_dependents();
-        pdl_wait();
-        hidden = pdl_acquire(hidden); row_index = pdl_acquire(row_index); W1 = pdl_acquire(W1); b1 = pdl_acquire(b1); w2 = pdl_acquire(w2);
         if (blockIdx.x + blockIdx.y + blockIdx.z == 0)       // the du kernel's, which follows
             for (int i = threadIdx.x; i < n_counters; i += MLP_THREADS) counters[i] = 0u;
     }
@@ -373,12 +370,12 @@ int arrol_internal_mlp_tiles(arrol_ctx* ctx, const void* hidden, int64_t row_str
     const int k_len = ((head->d + splits - 1) / splits + TK - 1) / TK * TK;
     const dim3 grid(m_tiles, h_tiles, splits), cluster(1, 1, splits);
     if (head->dtype == ARROL_F32)
-        ARROL_CUDA_OK(arrol_launch_pdl_cluster(score_mlp_tile_kernel<float, CLUSTERED>, grid, dim3(MLP_THREADS), cluster, s,
+        ARROL_CUDA_OK(arrol_launch_cluster(false, score_mlp_tile_kernel<float, CLUSTERED>, grid, dim3(MLP_THREADS), cluster, s,
             static_cast<const float*>(hidden), row_stride, row_index, N, head->d, head->h,
             static_cast<const float*>(head->W1), static_cast<const float*>(head->b1),
             static_cast<const float*>(head->w2), partial, u_out, k_len, ctx->source_rows, ctx->d_status, counters, n_counters));
     else
-        ARROL_CUDA_OK(arrol_launch_pdl_cluster(score_mlp_tile_kernel<__nv_bfloat16, CLUSTERED>, grid, dim3(MLP_THREADS), cluster, s,
+        ARROL_CUDA_OK(arrol_launch_cluster(false, score_mlp_tile_kernel<__nv_bfloat16, CLUSTERED>, grid, dim3(MLP_THREADS), cluster, s,
             static_cast<const __nv_bfloat16*>(hidden), row_stride, row_index, N, head->d, head->h,
             static_cast<const __nv_bfloat16*>(head->W1), static_cast<const __nv_bfloat16*>(head->b1),
             static_cast<const __nv_bfloat16*>(head->w2), partial, u_out, k_len, ctx->source_rows, ctx->d_status, counters, n_counters));

@@ -11,23 +11,24 @@
 //   score_mlp_tc_kernel   one block per (64 or 128 rollouts x 64 hidden units, or 128 x 128); shared memory is one ring of stages
 //                         (the tile's 64 columns of X and of W1 per K step of 64), filled by four TMA producer threads,
 //                         two for X and two for W1, on alternate K steps (one thread for all of W1 takes 300 cycles a step:
-//                         N = 2,048, d = 2,048, h = 256, rows in place 8.7 -> 12.6 us).  Two (tiles of 128) or four (64) issuing warps take the K steps round robin: one
-//                         warp's wait -> four MMAs -> commit round costs nearly 500 cycles, the MMAs of a 128 x 64 x 64 step
-//                         128, and a step's operands come in in about 290.  K step ks goes to accumulator ks mod 4.  The ring's
-//                         length is a multiple of the number of issuers, so that a stage always belongs to the same one: a parity
-//                         wait cannot tell a round from the one before the last.
-//                         Epilogue by all sixteen warps (with eight, two a scheduler, the chains of erff wait for themselves: 3.0 us
-//                         for 64 units): thread = rollout x a quarter of the tile's hidden units; accumulators added in index order, then sum_j w2_j gelu(u_j + b1_j) over 32 units in index order, two such sums added
+//                         N = 2,048, d = 2,048, h = 256, rows in place 8.7 -> 12.6 us).  Two (tiles of 128) or four (64) issuing
+//                         warps take the K steps round robin: one warp's wait -> four MMAs -> commit round costs nearly 500
+//                         cycles, the MMAs of a 128 x 64 x 64 step 128, and a step's operands come in in about 290.  K step ks
+//                         goes to accumulator ks mod 4.  The ring's length is a multiple of the number of issuers, so that a
+//                         stage always belongs to the same one: a parity wait cannot tell a round from the one before the last.
+//                         Epilogue by all sixteen warps (with eight, two a scheduler, the chains of erff wait for themselves:
+//                         3.0 us for 64 units): thread = rollout x a quarter of the tile's hidden units; accumulators added in
+//                         index order, then sum_j w2_j gelu(u_j + b1_j) over 32 units in index order, two such sums added
 //                         low + high -> a partial sum per 64 units and rollout, whatever the tile's width.
 //                         The blocks of a row tile are a cluster and put their partial sums into the first block's shared
-//                         memory, which adds them in index order, adds b2 and applies the probability map.  More than 1,024
-//                         hidden units are more than eight blocks of 128: there the partial sums go through global memory and
-//                         the last block to arrive (a counter per row tile) adds them.  The result does not depend on block
-//                         order, nor on which of the two it was.  Per call of 20 in a graph, partial sums through global memory ->
-//                         cluster: N = 2,048, d = 2,048, h = 256 13.5 -> 12.0 us (rows in place 10.3 -> 8.7); 4,096, 4,096, 512 29.1 ->
-//                         26.5; 394, 1,664, 256 10.8 -> 9.3; 32, 256, 64 7.1 -> 6.0.
-//   What the N = 2,048 call spends (in-kernel stamps, before): 0.7 us to the first stage, 3.7 for 32 K steps (192 KB in flight per
-//   SM and a copy's latency of 0.85 us), 1.6 of erff (45 instructions a unit and rollout), 2.2 in counting and adding up.
+//                         memory, which adds them in index order, adds b2 and applies the probability map.  Without clusters
+//                         (more than eight blocks of 128 hidden units, or where clusters would take more waves) the partial sums
+//                         go through global memory and the last block to arrive (a counter per row tile) adds them.  The result
+//                         does not depend on block order, nor on which of the two it was.  Per call of 20 in a graph, partial
+//                         sums through global memory -> cluster: N = 2,048, d = 2,048, h = 256 13.5 -> 12.0 us (rows in place
+//                         10.3 -> 8.7); 4,096, 4,096, 512 29.1 -> 26.5; 394, 1,664, 256 10.8 -> 9.3; 32, 256, 64 7.1 -> 6.0.
+//   What the N = 2,048 call spent before the clusters (in-kernel stamps): 0.7 us to the first stage, 3.7 for 32 K steps (192 KB in flight
+//   per SM and a copy's latency of 0.85 us), 1.6 of erff (45 instructions a unit and rollout), 2.2 in counting and adding up.
 //   Packing inside this kernel, each block of a cluster a share of the row tile and the contraction following chunk by chunk,
 //   was built and measured: 17.7 us, because every chunk's report waits 2 us for the stores before it.
 // Every wait is bounded; on expiry the block records ARROL_DEV_WAIT_EXPIRED, drains and returns.
@@ -42,7 +43,7 @@ namespace {
 
 constexpr int SUB_H = 64;                    // hidden units per partial sum: the same for every tile width
 constexpr int S_ACCS = 4;                    // accumulators; K step ks goes to accumulator ks % 4
-constexpr int S_PRODUCERS = 2;               // TMA producer threads (lane 0 of the first warps)
+constexpr int S_PRODUCERS = 2;               // TMA producer threads per operand (lane 0 of the first warps)
 constexpr int S_PRODUCER_WARPS = 4;          // warps before the issuers
 constexpr int S_HELPER_WARP0 = 8;            // warps without a role in the contraction fetch what the epilogue needs
 constexpr int S_HELPER_WARPS = 8;
