@@ -18,7 +18,8 @@ struct arrol_ctx {
     uint32_t* d_tile_counters; // MLP head on the tensor cores: finished blocks per row tile, zero between calls
     void* d_pack;              // MLP head on the tensor cores: the scored rows packed as bf16 [N][d], ARROL_PACK_BYTES
     uint32_t* d_head_counters; // head training step: finished runs per column tile, zero between calls
-    unsigned long long* d_chain;   // fused prune step: finished blocks (and failed index checks), per-block totals; zero between calls
+    unsigned long long* d_chain;   // fused prune step: finished blocks (and failed index checks, expired waits), then per block the tokens kept
+                                   // before it and how many blocks have added theirs; zero between calls
     void* d_runs;              // fused prune step: the survivors' runs for the kernel that writes the per-token outputs, ARROL_CHAIN_BLOCKS * 32
     bool logprob_smem_set;     // the log-prob kernels' dynamic shared-memory limit has been raised on this device
     int backward_max_pairs[3]; // pairs of the lm_head backward's kernels (dz, dH, dW) that are resident at once; 0 = not asked yet
@@ -27,7 +28,8 @@ struct arrol_ctx {
     bool calib_smem_set;       // likewise for the calibrator update
     bool backward_smem_set;    // likewise for the lm_head backward
     bool prune_smem_set;       // likewise for the fused prune step
-    int score_max_clusters[3][9]; // scoring kernel, tiles of 128 x 64, 64 x 64 and 128 x 128 rollouts x hidden units: clusters of so many blocks that are resident at once; 0 = not asked yet
+    int score_max_clusters[3][9]; // scoring kernel, tiles of 128 x 64, 64 x 64 and 128 x 128 rollouts x hidden units: clusters of so many
+                               // blocks that are resident at once; 0 = not asked yet
     bool score_tc_smem_set;    // the scoring kernel's dynamic shared-memory limit has been raised on this device
     bool gather_bulk_smem_set; // likewise for the bulk-copy gather kernel
     uint32_t test_spin_limit;  // arrol_test_hook: tries per pipeline wait of the log-prob kernel, 0 = the normal limit
@@ -43,7 +45,8 @@ struct arrol_ctx {
     cudaEvent_t copy_events[ARROL_COPY_EVENTS];
     uint8_t* h_keep;               // pinned, ARROL_MAX_HOST_N bytes: the keep mask read back by the host-buffer step
     int64_t source_rows;           // arrol_set_source_rows: rows of the caller's source buffers, 0 = indices unchecked
-    uint8_t* h_stage;              // pinned, ARROL_STAGE_BYTES: the scored rows of the host-buffer step, packed for one copy
+    uint8_t* h_stage;              // pinned, ARROL_STAGE_BYTES: the scored rows of the host-buffer step, packed for one copy; then, once the stream
+                                   // has been synchronised for the keep mask (which the reuse rests on), the survivors' token ids
 };
 
 constexpr int ARROL_MAX_MLP_N = 65536;       // rollouts per arrol_score_partial call with an MLP head

@@ -141,8 +141,10 @@ __device__ __forceinline__ int token_team(int64_t T, int S, int resident) {
 }
 // RUNS: the fused prune step has left all that a team needs to know of its survivor in one place: a round trip where there are two, from
 // the counts to the ids.  Graph of 40 prune steps on four batches in turn: 1,024 survivors of 2,660 ids 23.2 -> 22.7 us, 2,048 of 3,200
-// 64.4 -> 63.6, 1,676 of 150 11.2 -> 10.6, 16 of 2,660 9.0 -> 8.9, 320 of 85 9.8 -> 10.2.  Asking for the first run while the counts are on
-// their way gained the smallest 0.2 us and cost others as much.
+// 64.4 -> 63.6, 1,676 of 150 11.2 -> 10.6, 16 of 2,660 9.0 -> 8.9, 320 of 85 9.8 -> 10.2.  The last does not make a rule: over 2 to 120 prompts of 4 to
+// 32 rollouts of 60 to 1,500 ids the records are between 7 % faster (16 and 32 a group, 100 prompts and more) and 7 % slower (48 prompts of 16), the sign
+// changes with the grid's size from one to the next, and one size differs by 3 to 5 % from process to process.  Asking for the first run while
+// the counts are on their way gained the smallest 0.2 us and cost others as much.
 template <bool RUNS>
 __global__ void __launch_bounds__(TOKENS_THREADS, TOKENS_BLOCKS)
 gather_tokens_kernel(const int64_t* __restrict__ d_num, const int64_t* __restrict__ cu_seqlens,

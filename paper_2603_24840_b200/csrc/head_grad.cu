@@ -54,7 +54,8 @@ __device__ __forceinline__ void load_vector(const float* p, float (&o)[4]) {
 // the latency of its loads: the row numbers come with what ds is made of, and sixteen rows are in flight.  Rows without a factor are
 // not read.  Second kernel: the chunks' sums.  As three kernels, ds by one block, blocks of 2,048 columns with eight rows in flight, a thread per
 // column for the sums, a whole call took 19.6 us where it takes 9.4 now (graph of 20, N = 2,048, d = 2,048, bf16; 172, 1,464 15.2 -> 7.7; 8,192,
-// 4,096 48.6 -> 25.6; 8,192, 512, fp32 30.4 -> 11.5).
+// 4,096 48.6 -> 25.6; 8,192, 512, fp32 30.4 -> 11.5).  What every block's counting costs grows with the square of the rollouts: N = 65,536, d = 4,096
+// 215 us without a mask, 233 with one, 301 with one that is not 16-byte aligned (448 when one block counted, and formed ds for all).
 constexpr int LIN_ROWS = 32, LIN_AHEAD = 16, LIN_THREADS = 128;
 template <typename T>
 __global__ void __launch_bounds__(LIN_THREADS)

@@ -10,10 +10,11 @@
 //                        of two warps then, always 32 / G groups each).  One or
 //                        two warps run the per-group selection (select_lanes, as select_kernel) and write the keep
 //                        flags.  The first warp then scans the block's rollouts (kept, kept length), adds the block's
-//                        tokens to the sums of the blocks after it, waits until those before have added theirs to its own (a chained scan:
-//                        every block only waits for lower-numbered blocks, of at most two per SM; how many rollouts they keep is known), and writes survivor_idx, cu_seqlens and the advantages of its own
-//                        groups (group_statistics, as scan_adv_kernel); the last block writes {S, T}.  Nothing is
-//                        re-read from global memory and no block waits for the whole grid.  The second warp counts
+//                        tokens to the sums of the blocks after it, waits until those before have added theirs to its
+//                        own (a chained scan: every block only waits for lower-numbered blocks, of at most two per SM;
+//                        how many rollouts they keep is known), and writes survivor_idx, cu_seqlens and the advantages
+//                        of its own groups (group_statistics, as scan_adv_kernel); the last block writes {S, T}.
+//                        Nothing is re-read from global memory and no block waits for the whole grid.  The second warp counts
 //                        the blocks that are done with the chain; the last one clears it for the next call.
 // The device functions are the ones the three separate kernels use, so the results are bit-identical to the three
 // public calls, which remain the general path (more than SM-count blocks of 32 / G groups; group sizes above 32 are
@@ -178,10 +179,10 @@ prune_fused_kernel(const FusedParams p) {
         }
         __threadfence_block();
         named_barrier_arrive<1, 64>();
-        // The block is done with the chain when the first warp has added its total to the sums of the blocks after it and read its own.  The count's release is what
-        // the clearing rests on: every block's stores have been performed before the last one to be counted zeroes the
-        // words.  Without it what a block adds to the sum of one that has given up waiting could land after the zeros and be counted by a
-        // later call.  The release waits for
+        // The block is done with the chain when the first warp has added its total to the sums of the blocks after it and read its
+        // own.  The count's release is what the clearing rests on: every block's stores have been performed before the last one to be
+        // counted zeroes the words.  Without it what a block adds to the sum of one that has given up waiting could land after the
+        // zeros and be counted by a later call.  The release waits for
         // those stores, so it is this warp's, beside the outputs that the first one writes.  Graphs of 20 calls, this / with a fence and
         // the count in the first warp / with nothing between stores and count: 2,048 rollouts at d = 2,560 19.5 / 20.3 / 20.1 us, 4,096
         // after an MLP head 70.4 / 70.6 / 70.0, 32 rollouts 9.4 / 10.3 / 9.9.
@@ -224,7 +225,8 @@ prune_fused_kernel(const FusedParams p) {
     const int32_t block_c = __popc(kept_lanes);
     // The block adds its total to the sums of all blocks after it, and waits for its own sum to be complete: every block polls a word
     // of its own.  When each read all totals before it, 128 blocks polled the same lines, and the last total took 3.8 us to get
-    // through to them (relaxed loads, eight at a time, 5 us: the more polls the later).
+    // through to them (relaxed loads, eight at a time, 5 us: the more polls the later).  The additions grow with the square of the blocks;
+    // at two blocks an SM, 43,660 of them: 592 prompts of 16 rollouts of 60 tokens at d = 512 26.2 -> 20.1 us, of 600 39.1 -> 32.0.
     for (unsigned int b = blockIdx.x + 1 + lane; b < gridDim.x; b += 32) red_add_u64(sums + (size_t)b * SUM_WORDS, ARRIVED_ONE + (unsigned long long)block_t);
     unsigned long long sum = 0;
     bool expired = false;

@@ -116,13 +116,13 @@ struct ScoreTcParams {
     double* tile_loss;                 // [2][row tiles]: sums of the losses, divided by their number, and of ds
 };
 
-// PARTIALS: row tiles of more than eight blocks; the scores are finished through global memory.  SCORES: the blocks of a row tile
+// PARTIALS: a row tile's blocks are on their own; the scores are finished through global memory.  SCORES: the blocks of a row tile
 // (gridDim.y of them) are a cluster and finish the scores among themselves.  TRAIN: the head training step's forward and all
 // of its backward but the dW1 contraction: as SCORES, but every block gets all partial sums, forms the scores' gradients ds and
-// finishes its own hidden units: du = ds w2 gelu'(u), and the sums over the tile's rollouts that dw2 and db1 are made of, which the dW1 kernel adds up while it waits
-// for its contraction.  Both addends go to the operand ring's
-// shared memory, [unit][rollout], where the sums over rollouts are read along rows.  A kernel of its
-// own with u through global memory between took 9.4 us at N = 2,048, h = 256 (ncu).
+// finishes its own hidden units: du = ds w2 gelu'(u), and the sums over the tile's rollouts that dw2 and db1 are made of, which the
+// dW1 kernel adds up while it waits for its contraction.  Both addends go to the operand ring's shared memory, [unit][rollout], where
+// the sums over rollouts are read along rows.  A kernel of its own with u through global memory between took 9.4 us at N = 2,048,
+// h = 256 (ncu).
 enum Mode { PARTIALS, SCORES, TRAIN };
 template <int SBN, Mode MODE, int ROWS>
 __global__ void __launch_bounds__(S_THREADS, 1)
@@ -152,7 +152,8 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     float* b1_s = reinterpret_cast<float*>(tail + 512);          // [SBN]
     float* w2_s = reinterpret_cast<float*>(tail + 1024);         // [SBN]
     float* half_s = reinterpret_cast<float*>(tail + 1536);       // [2][TM] sums over 16 hidden units of a tile of 64
-    float* runs_s = reinterpret_cast<float*>(tail + 2560);       // [2 MAX_SUBS][TM] sums over 32 (of the row tile in the first block of a cluster; TRAIN: in every block)
+    float* runs_s = reinterpret_cast<float*>(tail + 2560);       // [2 MAX_SUBS][TM] sums over 32 (of the row tile in the first block of a
+                                                                 // cluster; TRAIN: in every block)
     float* ds_s = runs_s + 2 * MAX_SUBS * MAX_ROWS;                    // [TM]
     double* warp_d = reinterpret_cast<double*>(ds_s + TM);       // [2][4]
     int* warp_n = reinterpret_cast<int*>(warp_d + 8);            // [S_HELPER_WARPS]
@@ -259,9 +260,9 @@ score_mlp_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     }
     __syncwarp();
 
-    // Epilogue: all warps; thread = rollout x UNITS hidden units.  128 rollouts: accumulator row r is tensor-memory lane r, a warp reads the lanes of its
-    // number mod 4 and a quarter of the columns.  64 rollouts: row r is lane 32 (r / 16) + r mod 16, so that the upper half of a warp's
-    // lanes holds nothing; it takes over the upper half of the warp's columns.
+    // Epilogue: all warps; thread = rollout x UNITS hidden units.  128 rollouts: accumulator row r is tensor-memory lane r, a warp reads
+    // the lanes of its number mod 4 and a quarter of the columns.  64 rollouts: row r is lane 32 (r / 16) + r mod 16, so that the upper
+    // half of a warp's lanes holds nothing; it takes over the upper half of the warp's columns.
     constexpr int COLS = SBN / 4, UNITS = TM == 128 ? COLS : COLS / 2;
     const int quarter = warp & 3, cg = warp >> 2;
     const bool upper = TM == 64 && lane >= 16;
@@ -540,8 +541,8 @@ static int launch_mlp_tc(arrol_ctx* ctx, const void* hidden, int64_t row_stride,
     bool wide = m_tiles * subs > ctx->sm_count && h > SUB_H;
     const int waves = (m_tiles * (wide ? wide_tiles : subs) + ctx->sm_count - 1) / ctx->sm_count;       // without clusters
     // Tiles of 64 rollouts where all of these fit at once: half as much of the epilogue per SM, and a third fewer operand bytes.  Graph
-    // of 20 calls, tiles of 128 / 64: N = 394, d = 1,664, h = 256 9.5 / 8.8 us, 1,000, 1,000, 320 11.2 / 9.5, 283, 600, 512 8.5 / 7.4, 32, 256, 64 6.0 /
-    // 5.4; training steps N = 2,048, d = 2,048, h = 256 26.8 / 25.4, 525, 2,880, 512 27.2 / 23.5.
+    // of 20 calls, tiles of 128 / 64: N = 394, d = 1,664, h = 256 9.5 / 8.8 us, 1,000, 1,000, 320 11.2 / 9.5, 283, 600, 512 8.5 / 7.4, 32, 256,
+    // 64 6.0 / 5.4; training steps N = 2,048, d = 2,048, h = 256 26.8 / 25.4, 525, 2,880, 512 27.2 / 23.5.
     bool cluster = false, half_rows = false;
     int fit = 0;
     if (!p.u_out && subs <= 8) {        // clusters of more than eight blocks are not portable
