@@ -235,7 +235,6 @@ __device__ __forceinline__ void tcgen05_mma_bf16_pair(uint32_t d_tmem, uint64_t 
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base + i), columns c .. c+31
 __device__ __forceinline__ void tcgen05_ld_32x32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
-    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -254,7 +253,6 @@ __device__ __forceinline__ void tcgen05_ld_32x32(uint32_t taddr, float (&v)[32])
 __device__ __forceinline__ void tcgen05_ld_32(uint32_t taddr, float (&v)[32]) { tcgen05_ld_32x32(taddr, v); }
 __device__ __forceinline__ void tcgen05_ld_32(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
-    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
@@ -269,7 +267,6 @@ __device__ __forceinline__ void tcgen05_ld_32(uint32_t taddr, float (&v)[16]) {
 // the current one.  The wait takes the destination registers as read-write operands so that no use of them can be
 // scheduled before it.
 __device__ __forceinline__ void tcgen05_ld_32x32_issue(uint32_t taddr, uint32_t (&r)[32]) {
-    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
