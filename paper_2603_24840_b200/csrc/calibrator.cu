@@ -73,9 +73,9 @@ __global__ void calib_init_kernel(uint8_t* state, int B, int64_t cap, double alp
 // that one block scan ranks all of them, and the bisection is settled in two or three rounds of 31 points (see below) instead of 64
 // steps.  Per call, in a graph of 36 over changing states, mean of six (always three rounds, and a replay of all steps, before), lambda = 0.5:
 // N = 2,048, 128 bins 15.7 -> 11.3 us; N = 32, 64 bins 12.9 -> 9.1; N = 8,192, 256 bins 23.5 -> 17.2.  lambda = 0.3, whose replay takes all
-// steps: N = 2,048, 128 bins 16.6 -> 13.9; N = 64, 256 bins 19.1 -> 14.2; N = 4,000, 256 bins 20.8 -> 18.6.  Where bins meet the clip limits the root may
-// lie next to a breakpoint, which more rounds follow: lambda = 1 to 1.3 0.65 to 1.19 of the former time by the state, 0.9 of the rounds in the mean
-// of 48 states each.  More rollouts go through shared memory in pieces of CAL_STAGED,
+// steps: N = 2,048, 128 bins 16.6 -> 13.9; N = 64, 256 bins 19.1 -> 14.2; N = 4,000, 256 bins 20.8 -> 18.6.  Where bins meet the clip limits
+// the root may lie next to a breakpoint, which more rounds follow: lambda = 1 to 1.3 0.65 to 1.19 of the former time by the state, 0.9 of the
+// rounds in the mean of 48 states each.  More rollouts go through shared memory in pieces of CAL_STAGED,
 // after a pass that counts the labels, so that global memory is read in whole lines (a thread's own run read from there
 // touches a line per lane: N = 262,144 660 us a call by itself against 246 in pieces, 1,048,576 2,470 against 870; one rollout
 // per thread and scan, as it was before the runs, 460 and 1,570).  An instance each, because the pieces' code in the same one cost

@@ -90,7 +90,8 @@ constexpr int MLP_SPLITS = 4;        // blocks of a cluster at most
 // The tiles' blocks are bound by arithmetic and launched when the kernel before them has ended: launched while it runs (programmatic launch)
 // they pile up on the SMs that it leaves free.  Ordinary / programmatic launches, graphs of 20 calls, scores of fp32 heads: N = 500,
 // d = 1,024, h = 256 20.3 / 30.1 us, 1,500, 1,024, 64 16.2 / 24.5, 500, 256, 512 19.7 / 23.7, 12,000, 256, 64 24.3 / 26.3, 64, 256, 64 6.6 / 6.2; prune
-// steps P = 16, G = 8, d = 1,024, h = 256 22.6 / 33.2, P = 128, 512, 128 19.1 / 24.6, P = 4, 256, 64 12.1 / 12.7; training steps N = 700, 1,024,
+// steps P = 16, G = 8, d = 1,024, h = 256 22.6 / 33.2, P = 128, 512, 128 19.1 / 24.6, P = 4, 256, 64 12.1 / 12.7; training
+// steps N = 700, 1,024,
 // 256 51.3 / 70.3, 20,000, 256, 64 186 / 270, 64, 256, 64 17.9 / 18.9.  Launching the finishing kernel of the scores early: 10.2 / 12.6 at N = 64,
 // d = 256, h = 256, 1,500, 256, 64 8.3 / 8.1; the trigger behind the contraction: prune step P = 64, 512, 128 17.3 / 24.2.  A training step's du
 // kernel is launched early, and its counters are zeroed by the first block here instead of a memset.

@@ -67,10 +67,10 @@ constexpr size_t SM_SMEM = 228 * 1024, BLOCK_SMEM_RESERVED = 1024;      // of an
 constexpr int COMBINE_GROUP = 32, COMBINE_BLOCKS = 4;      // most tokens per block; blocks per SM
 constexpr size_t COMBINE_SMEM = 32 * 1024;
 inline size_t combine_bytes(const VocabPlan& v, int halves) { return (size_t)(v.n_sub + (v.n_mid < v.n_sub ? v.n_mid : 0)) * halves * 16; }
-// As many as give every SM a block, within the room.  While no more blocks than the kernel's four fit on every SM, that is the room beside a block of the
-// log-prob kernel (with `beside` bytes), where the first of them wait while that one runs; beyond that fewer blocks are worth more.
-// Rooms of 31,744 / 32,768 bytes, d = 256, V = 33,280 (six and seven tokens): 1,000 tokens 25.6 / 26.0 us, 1,300 30.2 / 30.6, 2,000 39.9 / 40.3, 3,000 53.8 /
-// 54.0; past the line 3,990 70.5 / 68.4, 9,000 149.4 / 146.4.
+// As many as give every SM a block, within the room.  While there are no more blocks than four an SM, which fit at once, that is the room
+// beside a block of the log-prob kernel (with `beside` bytes), where the first of them wait while that one runs; beyond that fewer blocks
+// are worth more.  Rooms of 31,744 / 32,768 bytes, d = 256, V = 33,280 (six and seven tokens): 1,000 tokens 25.6 / 26.0 us, 1,300 30.2 /
+// 30.6, 2,000 39.9 / 40.3, 3,000 53.8 / 54.0; past the line 3,990 70.5 / 68.4, 9,000 149.4 / 146.4.
 inline int combine_group(const VocabPlan& v, int halves, int64_t tail_rows, int sm_count, size_t beside) {
     const int64_t room_beside = (int64_t)((SM_SMEM - beside - 2 * BLOCK_SMEM_RESERVED) / combine_bytes(v, halves));
     const int64_t room = (int64_t)(COMBINE_SMEM / combine_bytes(v, halves));
